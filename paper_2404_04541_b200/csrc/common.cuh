@@ -81,6 +81,14 @@ struct DevCtl {
     i64 dense_warp_products, dense_warp_nnz;   // share of the dense rows the warp numeric kernel takes
 };
 
+// What a plan keeps in pinned host memory: the control block as last read back, and one slot per
+// block of the counting kernels, which write their partial sums there and the host adds up.
+constexpr int COUNT_BLOCKS = 256;
+struct HostBlock {
+    DevCtl ctl;
+    u64 partial[COUNT_BLOCKS];
+};
+
 struct ClassParams {
     int policy;             // spws_policy_t
     int reg_cap;            // CLS_ISM_REG: products <= reg_cap
@@ -179,6 +187,17 @@ __device__ __forceinline__ int block_excl_scan(int v, int* ws, int& total) {
     return ws[warp] + incl - v;
 }
 
+// Sum over the block, valid in thread 0; `ws` needs one word per warp.
+template <int THREADS>
+__device__ __forceinline__ i64 block_sum(i64 v, i64* ws) {
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < THREADS / 32; ++w) v += ws[w];
+    return v;
+}
+
 // First position in crd[lo, hi) whose coordinate is >= c (rows are sorted).
 __device__ __forceinline__ i64 lower_bound_crd(const int* __restrict__ crd, i64 lo, i64 hi, i64 c) {
     while (lo < hi) {
@@ -250,15 +269,15 @@ cudaError_t launch_hash(const LaunchCtx& c, bool numeric, int cls, int n_host, c
 cudaError_t launch_outer_counts(const LaunchCtx& c, const Csr& At, const Csr& B, int* cnt);
 size_t outer_sort_scratch_bytes(i64 n);
 cudaError_t launch_outer_ism(const LaunchCtx& c, bool numeric, const Csr& At, const Csr& B, const i64* koff, i64 P, i64 cap, i64 J,
-                             int label_bits, u64* kA, void* vA, u64* kB, void* vB, int* head, i64* at, char* sort_tmp,
-                             i64* block_sums, i64* nnz_dev, i64* nnz_host_pinned, bool* result_first);
+                             int label_bits, u64* kA, void* vA, u64* kB, void* vB, int* head, i64* at, char* sort_tmp, i64* block_sums, i64* nnz_dev, i64* nnz_host_pinned, bool* result_first);
 cudaError_t launch_coo_pos(const LaunchCtx& c, const u64* ukeys, i64 nnz, i64 m, i64 J, i64* pos);
 cudaError_t launch_coo_out(const LaunchCtx& c, const u64* ukeys, const void* uvals, i64 nnz, i64 J, int* Ccrd, void* Cval);
 cudaError_t launch_outer_dense(const LaunchCtx& c, bool numeric, const Csr& At, const Csr& B, const i64* koff, i64 P, i64 m, i64 J,
                                unsigned* dbits, void* dvals, int* cnt, const i64* pos, int* Ccrd, void* Cval);
-cudaError_t launch_outer_total(const LaunchCtx& c, const Csr& At, const Csr& B, u64* total_mapped_host);
+// number of products; partial[0 .. COUNT_BLOCKS) (pinned host memory, cleared by the caller) receives one sum per block
+cudaError_t launch_outer_total(const LaunchCtx& c, const Csr& At, const Csr& B, u64* partial);
 // higher.cu: the higher-order scatters with coordinate-form output
-cudaError_t launch_higher_total(const LaunchCtx& c, int form, const Csf3Dev& B, const Csr& C, u64* total_mapped_host);
+cudaError_t launch_higher_total(const LaunchCtx& c, int form, const Csf3Dev& B, const Csr& C, u64* partial);
 cudaError_t launch_higher_setup(const LaunchCtx& c, int form, const Csf3Dev& B, const Csr& C, int* fib_of, int* slice_of, int* cnt);
 cudaError_t launch_higher_ism(const LaunchCtx& c, bool numeric, int form, const Csf3Dev& B, const Csr& C, const Csr& D, const int* fib_of,
                               const int* slice_of, const i64* eoff, i64 P, i64 cap, u64 d1, u64 d2, int label_bits, u64* kA, void* vA,

@@ -109,8 +109,9 @@ __global__ void __launch_bounds__(OT) higher_unpack_kernel(int order, const u64*
 }
 
 // Number of numbered products, walking the tensor from its top level: a warp per stored level-0
-// coordinate, lanes over its fibres; the total is added into a word the host can read.
-__global__ void __launch_bounds__(OT) higher_total_kernel(int form, Csf3Dev B, Csr C, u64* total) {
+// coordinate, lanes over its fibres; one partial sum per block, as in outer_total_kernel.
+__global__ void __launch_bounds__(OT) higher_total_kernel(int form, Csf3Dev B, Csr C, u64* __restrict__ partial) {
+    __shared__ i64 ws[OT / 32];
     const int lane = threadIdx.x & 31;
     i64 mine = 0;
     for (i64 s = ((i64)blockIdx.x * OT + threadIdx.x) >> 5; s < B.n0; s += ((i64)gridDim.x * OT) >> 5) {
@@ -120,14 +121,15 @@ __global__ void __launch_bounds__(OT) higher_total_kernel(int form, Csf3Dev B, C
             if ((unsigned)pick < (unsigned)C.nrows) mine += (B.pos2[f + 1] - B.pos2[f]) * (C.pos[pick + 1] - C.pos[pick]);
         }
     }
-    for (int d = 16; d > 0; d >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, d);
-    if (lane == 0 && mine) atomicAdd_system(total, (u64)mine);
+    mine = block_sum<OT>(mine, ws);
+    if (threadIdx.x == 0) partial[blockIdx.x] = (u64)mine;
 }
 
 // ---- host side --------------------------------------------------------------------------------
-cudaError_t launch_higher_total(const LaunchCtx& c, int form, const Csf3Dev& B, const Csr& C, u64* total_mapped_host) {
+cudaError_t launch_higher_total(const LaunchCtx& c, int form, const Csf3Dev& B, const Csr& C, u64* partial) {
     if (B.n0 == 0) return cudaSuccess;
-    higher_total_kernel<<<grid_for(c, (i64)B.n0 * 32, OT), OT, 0, c.stream>>>(form, B, C, total_mapped_host);
+    const int grid = grid_for(c, (i64)B.n0 * 32, OT);
+    higher_total_kernel<<<grid < COUNT_BLOCKS ? grid : COUNT_BLOCKS, OT, 0, c.stream>>>(form, B, C, partial);
     return cudaGetLastError();
 }
 
@@ -158,8 +160,7 @@ cudaError_t launch_higher_ism(const LaunchCtx& c, bool numeric, int form, const 
                               u64* kB, void* vB, int* head, i64* at, char* sort_tmp, i64* block_sums, i64* nnz_dev,
                               i64* nnz_host_pinned, bool* result_first) {
     if (!numeric)
-        return higher_ism_t<double, false>(c, form, B, C, D, fib_of, slice_of, eoff, P, cap, d1, d2, label_bits, kA, nullptr, kB, nullptr, head,
-                                           at, sort_tmp, block_sums, nnz_dev, nnz_host_pinned, result_first);
+        return higher_ism_t<double, false>(c, form, B, C, D, fib_of, slice_of, eoff, P, cap, d1, d2, label_bits, kA, nullptr, kB, nullptr, head, at, sort_tmp, block_sums, nnz_dev, nnz_host_pinned, result_first);
     return c.is_f64 ? higher_ism_t<double, true>(c, form, B, C, D, fib_of, slice_of, eoff, P, cap, d1, d2, label_bits, kA, (double*)vA, kB,
                                                  (double*)vB, head, at, sort_tmp, block_sums, nnz_dev, nnz_host_pinned, result_first)
                     : higher_ism_t<float, true>(c, form, B, C, D, fib_of, slice_of, eoff, P, cap, d1, d2, label_bits, kA, (float*)vA, kB,

@@ -25,7 +25,8 @@ struct spws_plan_s {
     int is_f64 = 1;
     int policy = SPWS_AUTO;
     spws_options_t opt{};
-    DevCtl* host_ctl = nullptr; // pinned
+    HostBlock* host = nullptr;  // pinned
+    DevCtl* host_ctl = nullptr; // &host->ctl
     bool symbolic_ok = false;
     spws_stats_t stats{};
     // what the last symbolic pass saw (numeric must be called with the same shapes and scratch)
@@ -412,17 +413,24 @@ int label_bits_of(int64_t I, int64_t J) {
     return bits;
 }
 
-// products of the outer form, counted on the device into a word of the plan's pinned block
-spws_status_t outer_count_products(spws_plan_s* p, const Shapes& S, int64_t* P) {
+// adds up what a counting kernel left in the plan's pinned slots
+template <typename Launch>
+spws_status_t count_products(spws_plan_s* p, Launch launch, int64_t* P) {
     LaunchCtx c{};
     c.stream = p->h->stream;
     c.sm_count = p->h->sm_count;
-    u64* word = reinterpret_cast<u64*>(&p->host_ctl->products);
-    *word = 0;
-    CUDA_TRY(launch_outer_total(c, S.A, S.B, word));
+    memset(p->host->partial, 0, sizeof(p->host->partial));
+    CUDA_TRY(launch(c, p->host->partial));
     CUDA_TRY(cudaStreamSynchronize(c.stream));
-    *P = (int64_t)*word;
+    u64 total = 0;
+    for (int b = 0; b < COUNT_BLOCKS; ++b) total += p->host->partial[b];
+    *P = (int64_t)total;
     return SPWS_OK;
+}
+
+// products of the outer form, counted on the device
+spws_status_t outer_count_products(spws_plan_s* p, const Shapes& S, int64_t* P) {
+    return count_products(p, [&](const LaunchCtx& c, u64* partial) { return launch_outer_total(c, S.A, S.B, partial); }, P);
 }
 
 bool outer_wants_dense(const spws_plan_s* p, int64_t I, int64_t J, int64_t P, size_t scratch_bytes, const OuterLayout& L, spws_status_t* st) {
@@ -636,15 +644,7 @@ HLayout make_hlayout(const spws_plan_s* p, const HShapes& H, int64_t P) {
 }
 
 spws_status_t higher_count_products(spws_plan_s* p, const HShapes& H, int64_t* P) {
-    LaunchCtx c{};
-    c.stream = p->h->stream;
-    c.sm_count = p->h->sm_count;
-    u64* word = reinterpret_cast<u64*>(&p->host_ctl->products);
-    *word = 0;
-    CUDA_TRY(launch_higher_total(c, H.form, H.B, H.C, word));
-    CUDA_TRY(cudaStreamSynchronize(c.stream));
-    *P = (int64_t)*word;
-    return SPWS_OK;
+    return count_products(p, [&](const LaunchCtx& c, u64* partial) { return launch_higher_total(c, H.form, H.B, H.C, partial); }, P);
 }
 
 spws_status_t higher_workspace_size(spws_plan_s* plan, const spws_tensor_t* B, const spws_tensor_t* C, const spws_tensor_t* D, size_t* bytes) {
@@ -837,12 +837,13 @@ static spws_status_t plan_create_n(spws_handle_t handle, const char* expr, const
     p->is_f64 = f64 ? 1 : 0;
     p->policy = (int)policy;
     p->opt = o;
-    if (cudaMallocHost(reinterpret_cast<void**>(&p->host_ctl), sizeof(DevCtl)) != cudaSuccess) {
+    if (cudaMallocHost(reinterpret_cast<void**>(&p->host), sizeof(HostBlock)) != cudaSuccess) {
         cudaGetLastError();
         delete p;
         return SPWS_CUDA_ERROR;
     }
-    memset(p->host_ctl, 0, sizeof(DevCtl));
+    memset(p->host, 0, sizeof(HostBlock));
+    p->host_ctl = &p->host->ctl;
     *plan = p;
     return SPWS_OK;
 }
@@ -891,7 +892,7 @@ spws_status_t spws_plan_destroy(spws_plan_t plan) {
         for (int g = 0; g < SPWS_T_COUNT; ++g) cudaEventDestroy(plan->ev[g]);
         for (int g = 0; g < 3; ++g) cudaEventDestroy(plan->ev_start[g]);
     }
-    if (plan->host_ctl) cudaFreeHost(plan->host_ctl);
+    if (plan->host) cudaFreeHost(plan->host);
     delete plan;
     return SPWS_OK;
 }
