@@ -269,7 +269,8 @@ cudaError_t launch_hash(const LaunchCtx& c, bool numeric, int cls, int n_host, c
 cudaError_t launch_outer_counts(const LaunchCtx& c, const Csr& At, const Csr& B, int* cnt);
 size_t outer_sort_scratch_bytes(i64 n);
 cudaError_t launch_outer_ism(const LaunchCtx& c, bool numeric, const Csr& At, const Csr& B, const i64* koff, i64 P, i64 cap, i64 J,
-                             int label_bits, u64* kA, void* vA, u64* kB, void* vB, int* head, i64* at, char* sort_tmp, i64* block_sums, i64* nnz_dev, i64* nnz_host_pinned, bool* result_first);
+                             int label_bits, u64* kA, void* vA, u64* kB, void* vB, char* sort_tmp, i64* nnz_dev, i64* nnz_host_pinned,
+                             bool* result_first);
 cudaError_t launch_coo_pos(const LaunchCtx& c, const u64* ukeys, i64 nnz, i64 m, i64 J, i64* pos);
 cudaError_t launch_coo_out(const LaunchCtx& c, const u64* ukeys, const void* uvals, i64 nnz, i64 J, int* Ccrd, void* Cval);
 cudaError_t launch_outer_dense(const LaunchCtx& c, bool numeric, const Csr& At, const Csr& B, const i64* koff, i64 P, i64 m, i64 J,
@@ -281,8 +282,7 @@ cudaError_t launch_higher_total(const LaunchCtx& c, int form, const Csf3Dev& B, 
 cudaError_t launch_higher_setup(const LaunchCtx& c, int form, const Csf3Dev& B, const Csr& C, int* fib_of, int* slice_of, int* cnt);
 cudaError_t launch_higher_ism(const LaunchCtx& c, bool numeric, int form, const Csf3Dev& B, const Csr& C, const Csr& D, const int* fib_of,
                               const int* slice_of, const i64* eoff, i64 P, i64 cap, u64 d1, u64 d2, int label_bits, u64* kA, void* vA,
-                              u64* kB, void* vB, int* head, i64* at, char* sort_tmp, i64* block_sums, i64* nnz_dev,
-                              i64* nnz_host_pinned, bool* result_first);
+                              u64* kB, void* vB, char* sort_tmp, i64* nnz_dev, i64* nnz_host_pinned, bool* result_first);
 cudaError_t launch_higher_unpack(const LaunchCtx& c, int order, const u64* ukeys, const void* uvals, i64 nnz, u64 d1, u64 d2, int* o0,
                                  int* o1, int* o2, void* oval);
 

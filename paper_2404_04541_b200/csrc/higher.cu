@@ -144,27 +144,25 @@ cudaError_t launch_higher_setup(const LaunchCtx& c, int form, const Csf3Dev& B, 
 template <typename T, bool VALUES>
 static cudaError_t higher_ism_t(const LaunchCtx& c, int form, const Csf3Dev& B, const Csr& C, const Csr& D, const int* fib_of,
                                 const int* slice_of, const i64* eoff, i64 P, i64 cap, u64 d1, u64 d2, int label_bits, u64* kA, T* vA,
-                                u64* kB, T* vB, int* head, i64* at, char* sort_tmp, i64* block_sums, i64* nnz_dev, i64* nnz_host_pinned,
-                                bool* result_first) {
+                                u64* kB, T* vB, char* sort_tmp, i64* nnz_dev, i64* nnz_host_pinned, bool* result_first) {
     auto expand = [&](i64 t0, i64 n, u64* keys, T* vals) -> cudaError_t {
         higher_expand_kernel<T, VALUES><<<grid_for(c, n, OT * 4), OT, 0, c.stream>>>(form, B, C, D, fib_of, slice_of, eoff, t0, n, d1, d2, keys, vals);
         ++c.launches;
         return cudaGetLastError();
     };
-    return ism_rounds_t<T, VALUES>(c, expand, P, cap, label_bits, kA, vA, kB, vB, head, at, sort_tmp, block_sums, nnz_dev, nnz_host_pinned,
-                                   result_first);
+    return ism_rounds_t<T, VALUES>(c, expand, P, cap, label_bits, kA, vA, kB, vB, sort_tmp, nnz_dev, nnz_host_pinned, result_first);
 }
 
 cudaError_t launch_higher_ism(const LaunchCtx& c, bool numeric, int form, const Csf3Dev& B, const Csr& C, const Csr& D, const int* fib_of,
                               const int* slice_of, const i64* eoff, i64 P, i64 cap, u64 d1, u64 d2, int label_bits, u64* kA, void* vA,
-                              u64* kB, void* vB, int* head, i64* at, char* sort_tmp, i64* block_sums, i64* nnz_dev,
-                              i64* nnz_host_pinned, bool* result_first) {
+                              u64* kB, void* vB, char* sort_tmp, i64* nnz_dev, i64* nnz_host_pinned, bool* result_first) {
     if (!numeric)
-        return higher_ism_t<double, false>(c, form, B, C, D, fib_of, slice_of, eoff, P, cap, d1, d2, label_bits, kA, nullptr, kB, nullptr, head, at, sort_tmp, block_sums, nnz_dev, nnz_host_pinned, result_first);
+        return higher_ism_t<double, false>(c, form, B, C, D, fib_of, slice_of, eoff, P, cap, d1, d2, label_bits, kA, nullptr, kB, nullptr,
+                                           sort_tmp, nnz_dev, nnz_host_pinned, result_first);
     return c.is_f64 ? higher_ism_t<double, true>(c, form, B, C, D, fib_of, slice_of, eoff, P, cap, d1, d2, label_bits, kA, (double*)vA, kB,
-                                                 (double*)vB, head, at, sort_tmp, block_sums, nnz_dev, nnz_host_pinned, result_first)
+                                                 (double*)vB, sort_tmp, nnz_dev, nnz_host_pinned, result_first)
                     : higher_ism_t<float, true>(c, form, B, C, D, fib_of, slice_of, eoff, P, cap, d1, d2, label_bits, kA, (float*)vA, kB,
-                                                (float*)vB, head, at, sort_tmp, block_sums, nnz_dev, nnz_host_pinned, result_first);
+                                                (float*)vB, sort_tmp, nnz_dev, nnz_host_pinned, result_first);
 }
 
 cudaError_t launch_higher_unpack(const LaunchCtx& c, int order, const u64* ukeys, const void* uvals, i64 nnz, u64 d1, u64 d2, int* o0,

@@ -157,30 +157,29 @@ cudaError_t launch_outer_total(const LaunchCtx& c, const Csr& At, const Csr& B, 
     return cudaGetLastError();
 }
 
-size_t outer_sort_scratch_bytes(i64 n) {
-    const i64 nblocks = (n + RS_TILE - 1) / RS_TILE;
-    const size_t cells = (size_t)256 * (size_t)(nblocks > 0 ? nblocks : 1);
-    return ((cells * 4 + 255) & ~(size_t)255) + (((cells + 1) * 8 + 255) & ~(size_t)255) + (((cells / 2048 + 2) * 8 + 255) & ~(size_t)255);
-}
+size_t outer_sort_scratch_bytes(i64 n) { return sort_scratch_bytes(n); }
 
 template <typename T, bool VALUES>
 static cudaError_t outer_ism_t(const LaunchCtx& c, const Csr& At, const Csr& B, const i64* koff, i64 P, i64 cap, i64 J, int label_bits,
-                               u64* kA, T* vA, u64* kB, T* vB, int* head, i64* at, char* sort_tmp, i64* block_sums, i64* nnz_dev, i64* nnz_host_pinned, bool* result_first) {
+                               u64* kA, T* vA, u64* kB, T* vB, char* sort_tmp, i64* nnz_dev, i64* nnz_host_pinned, bool* result_first) {
     auto expand = [&](i64 t0, i64 n, u64* keys, T* vals) -> cudaError_t {
         outer_expand_kernel<T, VALUES, false><<<grid_for(c, n, OT * 4), OT, 0, c.stream>>>(At, B, koff, t0, n, J, keys, vals, nullptr, nullptr, 0, c.ctl);
         ++c.launches;
         return cudaGetLastError();
     };
-    return ism_rounds_t<T, VALUES>(c, expand, P, cap, label_bits, kA, vA, kB, vB, head, at, sort_tmp, block_sums, nnz_dev, nnz_host_pinned,
-                                   result_first);
+    return ism_rounds_t<T, VALUES>(c, expand, P, cap, label_bits, kA, vA, kB, vB, sort_tmp, nnz_dev, nnz_host_pinned, result_first);
 }
 
 cudaError_t launch_outer_ism(const LaunchCtx& c, bool numeric, const Csr& At, const Csr& B, const i64* koff, i64 P, i64 cap, i64 J,
-                             int label_bits, u64* kA, void* vA, u64* kB, void* vB, int* head, i64* at, char* sort_tmp, i64* block_sums, i64* nnz_dev, i64* nnz_host_pinned, bool* result_first) {
+                             int label_bits, u64* kA, void* vA, u64* kB, void* vB, char* sort_tmp, i64* nnz_dev, i64* nnz_host_pinned,
+                             bool* result_first) {
     if (!numeric)
-        return outer_ism_t<double, false>(c, At, B, koff, P, cap, J, label_bits, kA, nullptr, kB, nullptr, head, at, sort_tmp, block_sums, nnz_dev, nnz_host_pinned, result_first);
-    return c.is_f64 ? outer_ism_t<double, true>(c, At, B, koff, P, cap, J, label_bits, kA, (double*)vA, kB, (double*)vB, head, at, sort_tmp, block_sums, nnz_dev, nnz_host_pinned, result_first)
-                    : outer_ism_t<float, true>(c, At, B, koff, P, cap, J, label_bits, kA, (float*)vA, kB, (float*)vB, head, at, sort_tmp, block_sums, nnz_dev, nnz_host_pinned, result_first);
+        return outer_ism_t<double, false>(c, At, B, koff, P, cap, J, label_bits, kA, nullptr, kB, nullptr, sort_tmp, nnz_dev, nnz_host_pinned,
+                                          result_first);
+    return c.is_f64 ? outer_ism_t<double, true>(c, At, B, koff, P, cap, J, label_bits, kA, (double*)vA, kB, (double*)vB, sort_tmp, nnz_dev,
+                                                nnz_host_pinned, result_first)
+                    : outer_ism_t<float, true>(c, At, B, koff, P, cap, J, label_bits, kA, (float*)vA, kB, (float*)vB, sort_tmp, nnz_dev,
+                    nnz_host_pinned, result_first);
 }
 
 cudaError_t launch_coo_pos(const LaunchCtx& c, const u64* ukeys, i64 nnz, i64 m, i64 J, i64* pos) {

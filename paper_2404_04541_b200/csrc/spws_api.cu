@@ -370,7 +370,7 @@ inline void mark_start(spws_plan_s* p, int pass) {
 struct OuterLayout {
     size_t ctl, cnt, koff, block_sums, fixed_end;
     // sparse workspace
-    size_t kA, kB, vA, vB, head, at, sort_tmp, ism_end;
+    size_t kA, kB, vA, vB, sort_tmp, ism_end;
     // dense workspace
     size_t dbits, dvals, dcnt, dense_end;
     int64_t N;                  // entries of each (label, value) array
@@ -393,8 +393,6 @@ OuterLayout make_outer_layout(const spws_plan_s* p, int64_t I, int64_t K, int64_
     L.kB = take(8 * (size_t)L.N);
     L.vA = take(V * (size_t)L.N);
     L.vB = take(V * (size_t)L.N);
-    L.head = take(4 * (size_t)L.N);
-    L.at = take(8 * ((size_t)L.N + 1));
     L.sort_tmp = take(outer_sort_scratch_bytes(L.N));
     L.ism_end = o;
     o = L.fixed_end;
@@ -487,8 +485,7 @@ spws_status_t outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_t* 
         i64* nnz_host = reinterpret_cast<i64*>(&plan->host_ctl->nnz);
         const int64_t cap = plan->opt.outer_cap > 0 ? plan->opt.outer_cap : (P > 0 ? P : 1);
         CUDA_TRY(launch_outer_ism(c, false, S.A, S.B, koff, P, cap, J, label_bits_of(I, J), reinterpret_cast<u64*>(sc + L.kA), nullptr,
-                                  reinterpret_cast<u64*>(sc + L.kB), nullptr, reinterpret_cast<int*>(sc + L.head),
-                                  reinterpret_cast<i64*>(sc + L.at), sc + L.sort_tmp, block_sums, &c.ctl->nnz, nnz_host, &first));
+                                  reinterpret_cast<u64*>(sc + L.kB), nullptr, sc + L.sort_tmp, &c.ctl->nnz, nnz_host, &first));
         nnz = *nnz_host;
         CUDA_TRY(cudaMemcpyAsync(&c.ctl->nnz, nnz_host, sizeof(i64), cudaMemcpyHostToDevice, stream));
         CUDA_TRY(launch_coo_pos(c, reinterpret_cast<u64*>(sc + (first ? L.kA : L.kB)), nnz, I, J, pos));
@@ -547,8 +544,7 @@ spws_status_t outer_numeric(spws_plan_s* plan, const Shapes& S, spws_tensor_t* C
         i64* nnz_host = reinterpret_cast<i64*>(&plan->host_ctl->nnz);
         const int64_t cap = plan->opt.outer_cap > 0 ? plan->opt.outer_cap : (P > 0 ? P : 1);
         CUDA_TRY(launch_outer_ism(c, true, S.A, S.B, koff, P, cap, J, label_bits_of(I, J), reinterpret_cast<u64*>(sc + L.kA), sc + L.vA,
-                                  reinterpret_cast<u64*>(sc + L.kB), sc + L.vB, reinterpret_cast<int*>(sc + L.head),
-                                  reinterpret_cast<i64*>(sc + L.at), sc + L.sort_tmp, block_sums, &c.ctl->kept[0], nnz_host, &first));
+                                  reinterpret_cast<u64*>(sc + L.kB), sc + L.vB, sc + L.sort_tmp, &c.ctl->kept[0], nnz_host, &first));
         if (*nnz_host != plan->stats.nnz) return SPWS_BAD_SEQUENCE;     // operands differ from the symbolic pass's
         CUDA_TRY(launch_coo_out(c, reinterpret_cast<u64*>(sc + (first ? L.kA : L.kB)), sc + (first ? L.vA : L.vB), *nnz_host, J, C->crd[1], C->val));
         mark(plan, SPWS_T_NUM_ISM_GLOBAL);
@@ -613,7 +609,7 @@ spws_status_t check_higher(const spws_plan_s* p, const spws_tensor_t* B, const s
 }
 
 struct HLayout {
-    size_t ctl, fib_of, slice_of, cnt, eoff, block_sums, fixed_end, kA, kB, vA, vB, head, at, sort_tmp, end;
+    size_t ctl, fib_of, slice_of, cnt, eoff, block_sums, fixed_end, kA, kB, vA, vB, sort_tmp, end;
     int64_t N;
 };
 
@@ -636,8 +632,6 @@ HLayout make_hlayout(const spws_plan_s* p, const HShapes& H, int64_t P) {
     L.kB = take(8 * (size_t)L.N);
     L.vA = take(V * (size_t)L.N);
     L.vB = take(V * (size_t)L.N);
-    L.head = take(4 * (size_t)L.N);
-    L.at = take(8 * ((size_t)L.N + 1));
     L.sort_tmp = take(outer_sort_scratch_bytes(L.N));
     L.end = o;
     return L;
@@ -698,8 +692,7 @@ spws_status_t higher_symbolic(spws_plan_s* plan, const spws_tensor_t* B, const s
     const int64_t cap = plan->opt.outer_cap > 0 ? plan->opt.outer_cap : (P > 0 ? P : 1);
     CUDA_TRY(launch_higher_ism(c, false, H.form, H.B, H.C, H.D, fib_of, slice_of, eoff, P, cap, H.d1, H.d2, H.label_bits,
                                reinterpret_cast<u64*>(sc + L.kA), nullptr, reinterpret_cast<u64*>(sc + L.kB), nullptr,
-                               reinterpret_cast<int*>(sc + L.head), reinterpret_cast<i64*>(sc + L.at), sc + L.sort_tmp, block_sums,
-                               &c.ctl->nnz, nnz_host, &first));
+                               sc + L.sort_tmp, &c.ctl->nnz, nnz_host, &first));
     const int64_t nnz = *nnz_host;
     mark(plan, SPWS_T_SYM_ISM_GLOBAL);
     CUDA_TRY(cudaMemcpyAsync(&plan->host_ctl->status, &c.ctl->status, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
@@ -751,9 +744,7 @@ spws_status_t higher_numeric(spws_plan_s* plan, const spws_tensor_t* B, const sp
     const int64_t cap = plan->opt.outer_cap > 0 ? plan->opt.outer_cap : (P > 0 ? P : 1);
     CUDA_TRY(launch_higher_ism(c, true, H.form, H.B, H.C, H.D, reinterpret_cast<int*>(sc + L.fib_of), reinterpret_cast<int*>(sc + L.slice_of),
                                reinterpret_cast<i64*>(sc + L.eoff), P, cap, H.d1, H.d2, H.label_bits, reinterpret_cast<u64*>(sc + L.kA),
-                               sc + L.vA, reinterpret_cast<u64*>(sc + L.kB), sc + L.vB, reinterpret_cast<int*>(sc + L.head),
-                               reinterpret_cast<i64*>(sc + L.at), sc + L.sort_tmp, reinterpret_cast<i64*>(sc + L.block_sums),
-                               &c.ctl->kept[0], nnz_host, &first));
+                               sc + L.vA, reinterpret_cast<u64*>(sc + L.kB), sc + L.vB, sc + L.sort_tmp, &c.ctl->kept[0], nnz_host, &first));
     if (*nnz_host != nnz) return SPWS_BAD_SEQUENCE;                 // operands differ from the symbolic pass's
     CUDA_TRY(launch_higher_unpack(c, H.order, reinterpret_cast<u64*>(sc + (first ? L.kA : L.kB)), sc + (first ? L.vA : L.vB), nnz, H.d1, H.d2,
                                   Out->crd[0], Out->crd[1], Out->crd[2], Out->val));

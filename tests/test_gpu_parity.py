@@ -557,6 +557,22 @@ def test_outer_product_sparse_workspace_reproduces_algorithm1(ctx, oracle_mod, c
         assert np.allclose(val, ref.val, rtol=1e-5, atol=1e-6)
 
 
+@pytest.mark.parametrize("na,nb,wide", [(1, 1, 8), (1, 682, 1 << 20), (1, 683, 1 << 20), (3, 683, 900), (37, 111, 1 << 24), (64, 4001, 5000),
+                                        (700, 700, 701)])
+def test_sort_and_run_reduction_at_tile_edges(ctx, oracle_mod, na, nb, wide):
+    """Products just below, at and beyond a tile of the sort (2048) and of the run reduction (4096), and
+    many tiles; three live k with the same columns, so labels meet in runs that cross tiles.  Sums are
+    in loop order: equal to the oracle's restatement bit for bit."""
+    rng = np.random.default_rng(na * 1000 + nb)
+    ca, cb = np.sort(rng.choice(na + 5, na, replace=False)), np.sort(rng.choice(wide, nb, replace=False))
+    At = CSR(3, na + 5, np.arange(4) * na, np.tile(ca, 3).astype(np.int32), rng.uniform(-1, 1, 3 * na))
+    B = CSR(3, wide, np.arange(4) * nb, np.tile(cb, 3).astype(np.int32), rng.uniform(-1, 1, 3 * nb))
+    ref = oracle_mod.ism_outer(At.transpose(), B, 3 * na * nb)
+    pos, crd, val, stats = run_outer(ctx, At.transpose(), B, "ism")
+    assert stats["products"] == 3 * na * nb
+    assert np.array_equal(pos, ref.pos) and np.array_equal(crd, ref.crd) and np.array_equal(val, ref.val)
+
+
 def test_outer_product_on_a_power_law_matrix_and_wide_labels(ctx, oracle_mod):
     A = rmat_csr(11, 8, 5)
     ref = oracle_mod.spgemm(A, A, threads=4)
