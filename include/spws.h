@@ -24,8 +24,10 @@
  * result: sparse (Algorithm 1 on integer labels i*J + j, Sec. 5.2, with the accumulation array
  * and the all array in the scratch buffer) under SPWS_SPARSE_ISM, an I x J value array with
  * flags under SPWS_DENSE (SPWS_WORKSPACE_TOO_LARGE when the scratch given cannot hold it: the
- * paper's dense workspace running out of memory, Sec. 7.2), and under SPWS_AUTO the dense one
- * when it fits and either I*J <= 2^27 or the products number at least I*J/16.  The last three are
+ * paper's dense workspace running out of memory, Sec. 7.2), and under SPWS_AUTO A's
+ * entries are put in output-row order and the product is taken row by row when the columns fit
+ * dense_max_span (else the dense one when it fits and either I*J <= 2^27 or the products number at
+ * least I*J/16, else the sparse one).  The last three are
  * the higher-order scatters of Sec. 7.3 (sparse output in coordinate form): their workspace is the sparse one on
  * integer labels over all scattered output indices (third order for SpTTM); no dense workspace
  * is offered for them (SPWS_DENSE: SPWS_WORKSPACE_TOO_LARGE at plan creation).

@@ -86,7 +86,7 @@ struct DevCtl {
 constexpr int COUNT_BLOCKS = 256;
 struct HostBlock {
     DevCtl ctl;
-    u64 partial[COUNT_BLOCKS];
+    u64 partial[2 * COUNT_BLOCKS];
 };
 
 struct ClassParams {
@@ -99,6 +99,16 @@ struct ClassParams {
     float span_words_per_product;
     int unit_cap;           // entries available in the unit table
     u64 bm_arena_words;     // capacity of the bitmap arena
+};
+
+// Scratch of the forms whose first operand is put in output-row order (rowwise.cu).
+struct RowwiseBufs {
+    u64 *kA, *kB, *pA, *pB;     // labels and payloads of the entries, two buffers each for the sort
+    char* sort_tmp;
+    i64* pos;                   // the reordered operand
+    int* crd;
+    int* src;
+    u64* row_key;               // output-row labels (coordinate-form results)
 };
 
 struct Csr {
@@ -275,7 +285,7 @@ cudaError_t launch_coo_pos(const LaunchCtx& c, const u64* ukeys, i64 nnz, i64 m,
 cudaError_t launch_coo_out(const LaunchCtx& c, const u64* ukeys, const void* uvals, i64 nnz, i64 J, int* Ccrd, void* Cval);
 cudaError_t launch_outer_dense(const LaunchCtx& c, bool numeric, const Csr& At, const Csr& B, const i64* koff, i64 P, i64 m, i64 J,
                                unsigned* dbits, void* dvals, int* cnt, const i64* pos, int* Ccrd, void* Cval);
-// number of products; partial[0 .. COUNT_BLOCKS) (pinned host memory, cleared by the caller) receives one sum per block
+// number of products; partial[0 .. 2 COUNT_BLOCKS) (pinned host memory, cleared by the caller) receives one sum per block
 cudaError_t launch_outer_total(const LaunchCtx& c, const Csr& At, const Csr& B, u64* partial);
 // higher.cu: the higher-order scatters with coordinate-form output
 cudaError_t launch_higher_total(const LaunchCtx& c, int form, const Csf3Dev& B, const Csr& C, u64* partial);
@@ -285,5 +295,15 @@ cudaError_t launch_higher_ism(const LaunchCtx& c, bool numeric, int form, const 
                               u64* kB, void* vB, char* sort_tmp, i64* nnz_dev, i64* nnz_host_pinned, bool* result_first);
 cudaError_t launch_higher_unpack(const LaunchCtx& c, int order, const u64* ukeys, const void* uvals, i64 nnz, u64 d1, u64 d2, int* o0,
                                  int* o1, int* o2, void* oval);
+
+// rowwise.cu: the same forms taken row by row
+size_t rw_sort_bytes(i64 n);
+cudaError_t launch_rw_outer(const LaunchCtx& c, const Csr& At, i64 n, const Csr& B, i64 nnzB, int bits, const RowwiseBufs& b);
+cudaError_t launch_rw_csf(const LaunchCtx& c, int form, const Csf3Dev& B, u64 d, i64 m, int bits, const RowwiseBufs& b);
+cudaError_t launch_rw_values(const LaunchCtx& c, const void* val, const int* src, i64 n, void* out);
+cudaError_t launch_rw_fibre_rows(const LaunchCtx& c, bool values, const Csf3Dev& B, const Csr& C, const Csr& D, int* cnt, i64* fpos, int* fcrd,
+                                 void* fval, i64* block_sums);
+cudaError_t launch_rw_coords(const LaunchCtx& c, int order, const i64* rowptr, const u64* row_key, i64 m, i64 nnz, u64 d, const int* cols, int* o0,
+                             int* o1, int* o2);
 
 }  // namespace spws

@@ -109,20 +109,29 @@ __global__ void __launch_bounds__(OT) higher_unpack_kernel(int order, const u64*
 }
 
 // Number of numbered products, walking the tensor from its top level: a warp per stored level-0
-// coordinate, lanes over its fibres; one partial sum per block, as in outer_total_kernel.
+// coordinate, lanes over its fibres; one partial sum per block, as in outer_total_kernel, and behind
+// those COUNT_BLOCKS sums as many of the picked rows' lengths counted once per fibre.
 __global__ void __launch_bounds__(OT) higher_total_kernel(int form, Csf3Dev B, Csr C, u64* __restrict__ partial) {
-    __shared__ i64 ws[OT / 32];
+    __shared__ i64 ws[OT / 32], ws2[OT / 32];
     const int lane = threadIdx.x & 31;
-    i64 mine = 0;
+    i64 mine = 0, once = 0;
     for (i64 s = ((i64)blockIdx.x * OT + threadIdx.x) >> 5; s < B.n0; s += ((i64)gridDim.x * OT) >> 5) {
         const int c0 = B.crd0[s];
         for (i64 f = B.pos1[s] + lane; f < B.pos1[s + 1]; f += 32) {
             const int pick = form == 1 ? B.crd1[f] : c0;
-            if ((unsigned)pick < (unsigned)C.nrows) mine += (B.pos2[f + 1] - B.pos2[f]) * (C.pos[pick + 1] - C.pos[pick]);
+            if ((unsigned)pick < (unsigned)C.nrows) {
+                const i64 len = C.pos[pick + 1] - C.pos[pick];
+                mine += (B.pos2[f + 1] - B.pos2[f]) * len;
+                once += len;
+            }
         }
     }
     mine = block_sum<OT>(mine, ws);
-    if (threadIdx.x == 0) partial[blockIdx.x] = (u64)mine;
+    once = block_sum<OT>(once, ws2);
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = (u64)mine;
+        partial[COUNT_BLOCKS + blockIdx.x] = (u64)once;
+    }
 }
 
 // ---- host side --------------------------------------------------------------------------------

@@ -1,0 +1,341 @@
+// The scatters of second and third order taken row by row.
+//
+// When a form's first operand is put in the order of the output rows, the reduction variable moves
+// next to the last index and every output row owns a first-order workspace (Sec. 2.2), whose rows
+// the row-wise kernels count and fill.  Only the stored ENTRIES of the first operand are sorted
+// (label = output row, stable, so a row keeps its entries in loop order), never the products, and
+// nothing of size I x J is touched:
+//   outer      C(i,j)   = A(k,i) B(k,j)          rows i,      entry (k,i)   picks row k of B
+//   SpTTM      A(i,j,l) = B(k,i,j) C(k,l)        rows (i,j),  entry (k,i,j) picks row k of C
+//   SpTTM-I    A(k,j,l) = B(k,i,j) C(i,l)        rows (k,j),  entry (k,i,j) picks row i of C
+//   SpMTTKRP   A(i,j)   = B(k,l,i) C(k,j) D(l,j) rows i,      entry (k,l,i) picks row (k,l) of F,
+//              F((k,l),j) = C(k,j) D(l,j) formed once per stored fibre (k,l)
+// The reordered operand is a CSR matrix in scratch: pos, crd (the picked row), src (where the entry's
+// value stands in the operand as given, so that a numeric pass reads the values of its own call).
+#include <algorithm>
+
+#include "sortmerge.cuh"
+
+namespace spws {
+
+// The last r in [lo, hi) with pos[r] <= p (pos[lo] <= p < pos[hi]).
+__device__ __forceinline__ int owner_row(const i64* __restrict__ pos, int lo, int hi, i64 p) {
+    while (hi - lo > 1) {
+        const int mid = (int)(((i64)lo + hi) >> 1);
+        if (__ldg(pos + mid) <= p) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+constexpr int RK_ITEMS = 4;
+constexpr int RK_TILE = OT * RK_ITEMS;
+
+// Output-row label and payload (picked row above, entry below) of every entry; a block takes a tile of
+// consecutive entries, so the owners of its first and last entry bound every search.  B's columns
+// are checked on the way (the row kernels look at the ends of a row only).
+__global__ void __launch_bounds__(OT) rw_keys_outer_kernel(Csr At, i64 n, Csr B, i64 nnzB, u64* __restrict__ keys, u64* __restrict__ pay,
+                                                           DevCtl* ctl) {
+    __shared__ int s_lo, s_hi;
+    bool bad = false;
+    for (i64 q = (i64)blockIdx.x * OT + threadIdx.x; q < nnzB; q += (i64)gridDim.x * OT) bad |= (unsigned)__ldg(B.crd + q) >= (unsigned)B.ncols;
+    for (i64 t0 = (i64)blockIdx.x * RK_TILE; t0 < n; t0 += (i64)gridDim.x * RK_TILE) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_lo = owner_row(At.pos, 0, At.nrows, t0);
+        if (threadIdx.x == 32) s_hi = owner_row(At.pos, 0, At.nrows, min(n, t0 + RK_TILE) - 1) + 1;
+        __syncthreads();
+        for (int x = 0; x < RK_ITEMS; ++x) {
+            const i64 p = t0 + x * OT + threadIdx.x;
+            if (p >= n) break;
+            const int i = __ldg(At.crd + p);
+            bad |= (unsigned)i >= (unsigned)At.ncols;
+            keys[p] = (u64)(unsigned)i;
+            pay[p] = ((u64)(unsigned)owner_row(At.pos, s_lo, s_hi, p) << 32) | (u64)(unsigned)p;
+        }
+    }
+    if (bad) raise_status(ctl, DEV_NONCANONICAL);
+}
+
+// form: 0 SpTTM, 1 SpTTM-I, 2 SpMTTKRP.  `d` = extent of the label's inner coordinate (forms 0, 1).
+__global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u64 d, u64* __restrict__ keys, u64* __restrict__ pay) {
+    __shared__ int s_f[2], s_s[2];
+    for (i64 t0 = (i64)blockIdx.x * RK_TILE; t0 < B.nnz; t0 += (i64)gridDim.x * RK_TILE) {
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0 && threadIdx.x < 64) {
+            const int which = threadIdx.x >> 5;
+            const int f = owner_row(B.pos2, 0, B.n1, which == 0 ? t0 : min(B.nnz, t0 + RK_TILE) - 1);
+            s_f[which] = f;
+            s_s[which] = owner_row(B.pos1, 0, B.n0, f);
+        }
+        __syncthreads();
+        for (int x = 0; x < RK_ITEMS; ++x) {
+            const i64 e = t0 + x * OT + threadIdx.x;
+            if (e >= B.nnz) break;
+            const int f = owner_row(B.pos2, s_f[0], s_f[1] + 1, e);
+            const u64 c2 = (u64)(unsigned)__ldg(B.crd2 + e);
+            u64 key = c2, pick = (u64)(unsigned)f;
+            if (form != 2) {
+                const u64 c1 = (u64)(unsigned)__ldg(B.crd1 + f);
+                const u64 c0 = (u64)(unsigned)__ldg(B.crd0 + owner_row(B.pos1, s_s[0], s_s[1] + 1, f));
+                key = (form == 0 ? c1 : c0) * d + c2;
+                pick = form == 0 ? c0 : c1;
+            }
+            keys[e] = key;
+            pay[e] = (pick << 32) | (u64)(unsigned)e;
+        }
+    }
+}
+
+// CSR result: the reordered operand has one row per output row; pos by binary search in the sorted labels.
+__global__ void __launch_bounds__(OT) rw_dense_rows_kernel(const u64* __restrict__ keys, const u64* __restrict__ pay, i64 n, i64 m,
+                                                           i64* __restrict__ pos, int* __restrict__ crd, int* __restrict__ src) {
+    const i64 stride = (i64)gridDim.x * OT, t0 = (i64)blockIdx.x * OT + threadIdx.x;
+    for (i64 i = t0; i <= m; i += stride) {
+        i64 lo = 0, hi = n;
+        while (lo < hi) {
+            const i64 mid = (lo + hi) >> 1;
+            if (keys[mid] < (u64)i) lo = mid + 1; else hi = mid;
+        }
+        pos[i] = lo;
+    }
+    for (i64 p = t0; p < n; p += stride) {
+        const u64 w = pay[p];
+        crd[p] = (int)(w >> 32);
+        src[p] = (int)(unsigned)w;
+    }
+}
+
+__global__ void __launch_bounds__(OT) fill_pos_kernel(i64* __restrict__ pos, i64 m, i64 value) {
+    for (i64 i = (i64)blockIdx.x * OT + threadIdx.x; i <= m; i += (i64)gridDim.x * OT) pos[i] = value;
+}
+
+// Coordinate-form result: only the labels that occur become rows, in order (row r has label row_key[r]);
+// pos was filled with n, so the rows past the last label are empty.  Tiles hand the number of rows
+// on as in reduce_runs_kernel.  More than m labels mean a coordinate out of its range.
+__global__ void __launch_bounds__(OT) rw_sparse_rows_kernel(const u64* __restrict__ keys, const u64* __restrict__ pay, i64 n, i64 m,
+                                                            int* __restrict__ ticket, u64* __restrict__ status, DevCtl* ctl,
+                                                            u64* __restrict__ row_key, i64* __restrict__ pos, int* __restrict__ crd,
+                                                            int* __restrict__ src) {
+    __shared__ u64 s_edge[RK_ITEMS][OT / 32];
+    __shared__ int s_ws[33];
+    __shared__ int s_tile;
+    __shared__ i64 s_before;
+    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1);
+    __syncthreads();
+    const int tile = s_tile;
+    const i64 t0 = (i64)tile * RK_TILE;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    u64 key[RK_ITEMS];
+#pragma unroll
+    for (int x = 0; x < RK_ITEMS; ++x) {
+        const i64 p = t0 + x * OT + threadIdx.x;
+        key[x] = p < n ? keys[p] : ABSENT_LABEL;
+        if (p < n) {
+            const u64 w = pay[p];
+            crd[p] = (int)(w >> 32);
+            src[p] = (int)(unsigned)w;
+        }
+        if (lane == 31) s_edge[x][warp] = key[x];
+    }
+    __syncthreads();
+    // heads before this thread's in the tile = heads of the earlier rounds of OT entries + of its round
+    int rank[RK_ITEMS], total = 0;
+    bool head[RK_ITEMS];
+#pragma unroll
+    for (int x = 0; x < RK_ITEMS; ++x) {
+        u64 prev = __shfl_up_sync(0xffffffffu, key[x], 1);
+        if (lane == 0) {
+            if (warp > 0) prev = s_edge[x][warp - 1];
+            else if (x > 0) prev = s_edge[x - 1][OT / 32 - 1];
+            else prev = t0 > 0 ? keys[t0 - 1] : ABSENT_LABEL;
+        }
+        head[x] = key[x] != ABSENT_LABEL && key[x] != prev;
+        int round;
+        rank[x] = total + block_excl_scan<OT>(head[x], s_ws, round);
+        total += round;
+    }
+    if (warp == 0) {
+        if (lane == 0) look_publish(status + tile, tile == 0 ? 2 : 1, total);
+        i64 before = 0;
+        if (tile > 0) {
+            before = look_back_warp(status, tile, 0, ctl);
+            if (lane == 0) look_publish(status + tile, 2, before + total);
+        }
+        if (lane == 0) s_before = before;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < RK_ITEMS; ++x)
+        if (head[x]) {
+            const i64 r = s_before + rank[x];
+            if (r >= m) { raise_status(ctl, DEV_NONCANONICAL); continue; }
+            row_key[r] = key[x];
+            pos[r] = t0 + x * OT + threadIdx.x;
+        }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(OT) rw_values_kernel(const T* __restrict__ val, const int* __restrict__ src, i64 n, T* __restrict__ out) {
+    for (i64 p = (i64)blockIdx.x * OT + threadIdx.x; p < n; p += (i64)gridDim.x * OT) out[p] = __ldg(val + (unsigned)src[p]);
+}
+
+// Rows of F (SpMTTKRP): a warp per stored fibre (k,l) walks the shorter of C's row k and D's row l and
+// looks every column up in the longer one.  PASS 0 counts, 1 writes the columns, 2 the products.
+template <typename T, int PASS>
+__global__ void __launch_bounds__(OT) rw_fibre_rows_kernel(Csf3Dev B, Csr C, Csr D, int* __restrict__ cnt, const i64* __restrict__ fpos,
+                                                           int* __restrict__ fcrd, T* __restrict__ fval, DevCtl* ctl) {
+    const int lane = threadIdx.x & 31;
+    for (i64 f = ((i64)blockIdx.x * OT + threadIdx.x) >> 5; f < B.n1; f += ((i64)gridDim.x * OT) >> 5) {
+        const int k = __ldg(B.crd0 + owner_row(B.pos1, 0, B.n0, f)), l = __ldg(B.crd1 + f);
+        if ((unsigned)k >= (unsigned)C.nrows || (unsigned)l >= (unsigned)D.nrows) {
+            raise_status(ctl, DEV_NONCANONICAL);
+            if (PASS == 0 && lane == 0) cnt[f] = 0;
+            continue;
+        }
+        i64 s0 = __ldg(C.pos + k), s1 = __ldg(C.pos + k + 1), g0 = __ldg(D.pos + l), g1 = __ldg(D.pos + l + 1);
+        const int* __restrict__ scrd = C.crd;
+        const int* __restrict__ gcrd = D.crd;
+        const T* __restrict__ sval = (const T*)C.val;
+        const T* __restrict__ gval = (const T*)D.val;
+        if (s1 - s0 > g1 - g0) {
+            i64 t = s0; s0 = g0; g0 = t;
+            t = s1; s1 = g1; g1 = t;
+            scrd = D.crd; gcrd = C.crd;
+            sval = (const T*)D.val; gval = (const T*)C.val;
+        }
+        int found = 0;
+        i64 out = PASS > 0 ? fpos[f] : 0;
+        for (i64 q0 = s0; q0 < s1; q0 += 32) {
+            const i64 q = q0 + lane;
+            const int col = q < s1 ? __ldg(scrd + q) : -1;
+            const i64 at = q < s1 ? lower_bound_crd(gcrd, g0, g1, col) : g1;
+            const bool hit = at < g1 && __ldg(gcrd + at) == col;
+            const unsigned hits = __ballot_sync(0xffffffffu, hit);
+            if (PASS > 0 && hit) {
+                const i64 o = out + __popc(hits & ((1u << lane) - 1u));
+                if (PASS == 1) fcrd[o] = col;
+                else fval[o] = mul_rn(__ldg(sval + q), __ldg(gval + at));
+            }
+            found += __popc(hits);
+            out += __popc(hits);
+        }
+        if (PASS == 0 && lane == 0) cnt[f] = found;
+    }
+}
+
+// Coordinates of a coordinate-form result from its row pointer, row labels and columns.  A block takes a
+// tile of consecutive entries; the rows of the first and the last one bound every search.
+constexpr int RC_ITEMS = 8;
+constexpr int RC_TILE = OT * RC_ITEMS;
+
+__global__ void __launch_bounds__(OT) rw_coords_kernel(int order, const i64* __restrict__ rowptr, const u64* __restrict__ row_key, i64 m, i64 nnz,
+                                                       u64 d, const int* __restrict__ cols, int* __restrict__ o0, int* __restrict__ o1,
+                                                       int* __restrict__ o2) {
+    __shared__ int s_lo, s_hi;
+    for (i64 t0 = (i64)blockIdx.x * RC_TILE; t0 < nnz; t0 += (i64)gridDim.x * RC_TILE) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_lo = owner_row(rowptr, 0, (int)m, t0);
+        if (threadIdx.x == 32) s_hi = owner_row(rowptr, 0, (int)m, min(nnz, t0 + RC_TILE) - 1) + 1;
+        __syncthreads();
+        const int hi = s_hi;
+        int r = s_lo;                           // a thread's entries ascend, so each search starts at the last row found
+        for (int x = 0; x < RC_ITEMS; ++x) {
+            const i64 t = t0 + x * OT + threadIdx.x;
+            if (t >= nnz) break;
+            r = owner_row(rowptr, r, hi, t);
+            const u64 key = __ldg(row_key + r);
+            if (order == 3) {
+                o0[t] = (int)(key / d);
+                o1[t] = (int)(key % d);
+                o2[t] = __ldg(cols + t);
+            } else {
+                o0[t] = (int)key;
+                o1[t] = __ldg(cols + t);
+            }
+        }
+    }
+}
+
+// ---- host side --------------------------------------------------------------------------------
+size_t rw_sort_bytes(i64 n) {
+    const size_t rows_status = sort_head_bytes() + 8 * (size_t)((n + RK_TILE - 1) / RK_TILE + 1);
+    return std::max(sort_scratch_bytes(n), rows_status);
+}
+
+// Sorts the entries by output row and writes the reordered operand (all but its values).  `sparse`: a row per
+// label that occurs (at most m), labels to row_key; otherwise a row per label value.
+static cudaError_t rw_reorder(const LaunchCtx& c, i64 n, i64 m, int bits, bool sparse, const RowwiseBufs& b) {
+    cudaError_t e;
+    if (sparse) {
+        fill_pos_kernel<<<grid_for(c, m + 1, OT), OT, 0, c.stream>>>(b.pos, m, n);
+        ++c.launches;
+    }
+    bool first = true;
+    if ((e = radix_sort_t<u64, true>(c, n, bits, b.kA, b.pA, b.kB, b.pB, b.sort_tmp, &first)) != cudaSuccess) return e;
+    const u64* ks = first ? b.kA : b.kB;
+    const u64* ps = first ? b.pA : b.pB;
+    if (!sparse) {
+        rw_dense_rows_kernel<<<grid_for(c, n > m ? n : m + 1, OT), OT, 0, c.stream>>>(ks, ps, n, m, b.pos, b.crd, b.src);
+        ++c.launches;
+    } else if (n > 0) {
+        const int tiles = (int)((n + RK_TILE - 1) / RK_TILE);
+        SortHead* head = reinterpret_cast<SortHead*>(b.sort_tmp);
+        if ((e = cudaMemsetAsync(b.sort_tmp, 0, sort_head_bytes() + 8 * (size_t)tiles, c.stream)) != cudaSuccess) return e;
+        rw_sparse_rows_kernel<<<tiles, OT, 0, c.stream>>>(ks, ps, n, m, &head->ticket[0], reinterpret_cast<u64*>(b.sort_tmp + sort_head_bytes()),
+                                                         c.ctl, b.row_key, b.pos, b.crd, b.src);
+        ++c.launches;
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rw_outer(const LaunchCtx& c, const Csr& At, i64 n, const Csr& B, i64 nnzB, int bits, const RowwiseBufs& b) {
+    rw_keys_outer_kernel<<<grid_for(c, std::max(n, nnzB), RK_TILE), OT, 0, c.stream>>>(At, n, B, nnzB, b.kA, b.pA, c.ctl);
+    ++c.launches;
+    return rw_reorder(c, n, At.ncols, bits, false, b);
+}
+
+cudaError_t launch_rw_csf(const LaunchCtx& c, int form, const Csf3Dev& B, u64 d, i64 m, int bits, const RowwiseBufs& b) {
+    if (B.nnz > 0) {
+        rw_keys_csf_kernel<<<grid_for(c, B.nnz, RK_TILE), OT, 0, c.stream>>>(form, B, d, b.kA, b.pA);
+        ++c.launches;
+    }
+    return rw_reorder(c, B.nnz, m, bits, true, b);
+}
+
+cudaError_t launch_rw_values(const LaunchCtx& c, const void* val, const int* src, i64 n, void* out) {
+    if (n == 0) return cudaSuccess;
+    if (c.is_f64) rw_values_kernel<double><<<grid_for(c, n, OT), OT, 0, c.stream>>>((const double*)val, src, n, (double*)out);
+    else rw_values_kernel<float><<<grid_for(c, n, OT), OT, 0, c.stream>>>((const float*)val, src, n, (float*)out);
+    ++c.launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rw_fibre_rows(const LaunchCtx& c, bool values, const Csf3Dev& B, const Csr& C, const Csr& D, int* cnt, i64* fpos, int* fcrd,
+                                 void* fval, i64* block_sums) {
+    const int grid = grid_for(c, (i64)B.n1 * 32, OT);
+    if (values) {
+        if (B.n1 == 0) return cudaSuccess;
+        if (c.is_f64) rw_fibre_rows_kernel<double, 2><<<grid, OT, 0, c.stream>>>(B, C, D, nullptr, fpos, nullptr, (double*)fval, c.ctl);
+        else rw_fibre_rows_kernel<float, 2><<<grid, OT, 0, c.stream>>>(B, C, D, nullptr, fpos, nullptr, (float*)fval, c.ctl);
+        ++c.launches;
+        return cudaGetLastError();
+    }
+    if (B.n1 > 0) {
+        rw_fibre_rows_kernel<float, 0><<<grid, OT, 0, c.stream>>>(B, C, D, cnt, nullptr, nullptr, nullptr, c.ctl);
+        ++c.launches;
+    }
+    cudaError_t e = launch_scan_counts(c, cnt, B.n1, fpos, block_sums, nullptr);
+    if (e != cudaSuccess || B.n1 == 0) return e;
+    rw_fibre_rows_kernel<float, 1><<<grid, OT, 0, c.stream>>>(B, C, D, nullptr, fpos, fcrd, nullptr, c.ctl);
+    ++c.launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rw_coords(const LaunchCtx& c, int order, const i64* rowptr, const u64* row_key, i64 m, i64 nnz, u64 d, const int* cols, int* o0,
+                             int* o1, int* o2) {
+    if (nnz == 0) return cudaSuccess;
+    rw_coords_kernel<<<grid_for(c, nnz, RC_TILE), OT, 0, c.stream>>>(order, rowptr, row_key, m, nnz, d, cols, o0, o1, o2);
+    ++c.launches;
+    return cudaGetLastError();
+}
+
+}  // namespace spws

@@ -39,6 +39,8 @@ struct spws_plan_s {
     // outer-product form: what the last symbolic pass decided
     int64_t outer_products = 0;
     bool outer_dense = false;
+    bool rowwise = false;       // the last symbolic pass put the first operand in output-row order (rowwise.cu)
+    int64_t rw_once = 0;        // entries the fibre matrix of SpMTTKRP has at most
     // optional per-kernel timing: ev[g] is recorded after group g; ev_start[] before each pass
     bool profiling = false;
     cudaEvent_t ev[SPWS_T_COUNT] = {};
@@ -156,14 +158,15 @@ bool is_pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 // ---- scratch layout ------------------------------------------------------------------------
 struct Layout {
     size_t ctl, ub, rowptr_raw, cnt, jmin, jmax, cls, perm, bm_off, warp_rows, row_unit0, unit_row, block_sums,
-        fpos, sflags, spos, bw_long, bw, brow, rest, fixed_end;
+        fpos, sflags, spos, bw_long, bw, brow, extra, rest, fixed_end;
     bool has_brow;
     int unit_cap;
     int bw_long_cap;            // 0: no word lists for this B
     int dense_smem_words;
 };
 
-Layout make_layout(const spws_plan_s* p, int64_t m, int64_t ncols, int64_t n_i, int64_t nnzB, int64_t k, int64_t nnzA) {
+// extra_bytes: room a form of higher order keeps between the fixed tables and the arenas
+Layout make_layout(const spws_plan_s* p, int64_t m, int64_t ncols, int64_t n_i, int64_t nnzB, int64_t k, int64_t nnzA, size_t extra_bytes = 0) {
     Layout L{};
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o = align256(o + bytes); return at; };
@@ -207,6 +210,7 @@ Layout make_layout(const spws_plan_s* p, int64_t m, int64_t ncols, int64_t n_i, 
         L.has_brow = true;
         L.brow = take(16 * (size_t)k);
     }
+    L.extra = take(extra_bytes);
     L.fixed_end = o;
     L.rest = o;
     return L;
@@ -366,6 +370,146 @@ inline void mark_start(spws_plan_s* p, int pass) {
     p->ev_pass[pass] = true;
 }
 
+// ---- the row-wise passes: every output row (fibre) through the workspace of its class ------------
+// `ttmA` / `ttmC`: the 3-tensor operand and result, whose upper levels are rebuilt (null for the matrix
+// forms).  `c` is make_ctx of the layout; the control block has been cleared.  On success the plan
+// holds the statistics and what the numeric pass needs.
+spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L, LaunchCtx& c, const spws_tensor_t* ttmA, spws_tensor_t* ttmC,
+                            i64* rowptr, char* sc) {
+    cudaStream_t stream = c.stream;
+    // a1: upper bounds + classes; a2: binning
+    CUDA_TRY(launch_row_bounds(c, S.A, S.B, S.nnzA));
+    CUDA_TRY(launch_bw_build(c, S.B));
+    mark(plan, SPWS_T_SYM_BOUNDS);
+    CUDA_TRY(launch_bin_rows(c, (int)S.m));
+    mark(plan, SPWS_T_SYM_BIN);
+    // the class sizes come back now, so that only the workspaces that have rows are launched, with
+    // grids sized for them (a launch for an empty class costs as much as a small class's work)
+    int* hcount = plan->host_ctl->class_count;
+    CUDA_TRY(cudaMemcpyAsync(hcount, c.ctl->class_count, sizeof(int) * NCLASS, cudaMemcpyDeviceToHost, stream));
+    CUDA_TRY(cudaMemcpyAsync(&plan->host_ctl->max_ub_smem, &c.ctl->max_ub_smem, sizeof(i64), cudaMemcpyDeviceToHost, stream));
+    CUDA_TRY(cudaStreamSynchronize(stream));
+    plan->max_ub_smem = plan->host_ctl->max_ub_smem;
+    c.max_ub_smem = plan->max_ub_smem;
+    // a3: exact count per row through the workspace of its class
+    if (S.m > 0) {
+        for (int cls = CLS_ISM_REG8; cls <= CLS_ISM_REG; ++cls)
+            if (hcount[cls] > 0) {
+                CUDA_TRY(launch_ism_reg(c, false, cls, hcount[cls], S.A, S.B, rowptr, nullptr, nullptr));
+                mark(plan, SPWS_T_SYM_ISM_REG);
+            }
+        // under `auto` the rows of the shared-memory insert-sort-merge classes are counted through a
+        // hash set of their columns: the count needs no order
+        const bool count_by_hash = plan->policy == SPWS_AUTO;
+        if (hcount[CLS_ISM_SMEM_S] > 0) {
+            if (count_by_hash) CUDA_TRY(launch_hash(c, false, CLS_ISM_SMEM_S, hcount[CLS_ISM_SMEM_S], S.A, S.B, rowptr, nullptr, nullptr));
+            else CUDA_TRY(launch_ism_smem(c, false, CLS_ISM_SMEM_S, hcount[CLS_ISM_SMEM_S], S.A, S.B, rowptr, nullptr, nullptr));
+            mark(plan, SPWS_T_SYM_ISM_SMEM_S);
+        }
+        if (hcount[CLS_ISM_SMEM] > 0) {
+            if (count_by_hash) CUDA_TRY(launch_hash(c, false, CLS_ISM_SMEM, hcount[CLS_ISM_SMEM], S.A, S.B, rowptr, nullptr, nullptr));
+            else CUDA_TRY(launch_ism_smem(c, false, CLS_ISM_SMEM, hcount[CLS_ISM_SMEM], S.A, S.B, rowptr, nullptr, nullptr));
+            mark(plan, SPWS_T_SYM_ISM_SMEM);
+        }
+        if (hcount[CLS_DENSE_WARP] > 0) {
+            CUDA_TRY(launch_dense_sym_warp(c, S.A, S.B));
+            mark(plan, SPWS_T_SYM_DENSE_WARP);
+        }
+        if (hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0) {
+            CUDA_TRY(launch_dense_sym_cta(c, S.A, S.B));
+            mark(plan, SPWS_T_SYM_DENSE_CTA);
+        }
+        if (hcount[CLS_ISM_GLOBAL] > 0) {
+            CUDA_TRY(launch_ism_global(c, false, hcount[CLS_ISM_GLOBAL], S.A, S.B, rowptr, nullptr, nullptr));
+            mark(plan, SPWS_T_SYM_ISM_GLOBAL);
+        }
+        for (int cls = CLS_HASH_S; cls <= CLS_HASH; ++cls)
+            if (hcount[cls] > 0) {
+                CUDA_TRY(launch_hash(c, false, cls, hcount[cls], S.A, S.B, rowptr, nullptr, nullptr));
+                mark(plan, SPWS_T_SYM_HASH);
+            }
+    }
+    // a4: exclusive scan into the row pointer
+    if (ttmA) {
+        // with C's fibre and slice levels rebuilt from the fibres that produced an output
+        CUDA_TRY(launch_ttm_scan_compact(c, (int)S.n_i, (int)S.m, LL(ttmA->pos[1]), ttmA->crd[0], ttmA->crd[1], rowptr,
+                                         reinterpret_cast<i64*>(sc + L.fpos), reinterpret_cast<int*>(sc + L.sflags),
+                                         reinterpret_cast<i64*>(sc + L.spos), reinterpret_cast<i64*>(sc + L.block_sums), &c.ctl->nnz,
+                                         LL(ttmC->pos[0]), ttmC->crd[0], LL(ttmC->pos[1]), ttmC->crd[1], LL(ttmC->pos[2])));
+    } else {
+        CUDA_TRY(launch_scan_counts(c, c.tab.cnt, (int)S.m, rowptr, reinterpret_cast<i64*>(sc + L.block_sums), &c.ctl->nnz));
+    }
+    if (hcount[CLS_DENSE_WARP] + hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0) CUDA_TRY(launch_dense_rebin(c, (int)S.m, rowptr));
+    CUDA_TRY(launch_class_nnz(c, (int)S.m));
+    mark(plan, SPWS_T_SYM_SCAN);
+    CUDA_TRY(cudaMemcpyAsync(plan->host_ctl, c.ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, stream));
+    CUDA_TRY(cudaStreamSynchronize(stream));
+    const DevCtl& hc = *plan->host_ctl;
+    plan->stats = spws_stats_t{};
+    plan->stats.device_status = hc.status;
+    if (hc.status != 0) return from_dev_status(hc.status);
+    plan->stats.rows = S.m;
+    plan->stats.products = hc.products;
+    plan->stats.nnz = hc.nnz;
+    plan->stats.max_row_products = hc.max_ub;
+    for (int k = 0; k < NCLASS; ++k) {
+        plan->bin_rows[k] = hc.class_count[k];
+        plan->stats.rows_per_class[public_class(k)] += hc.class_count[k];
+        plan->stats.products_per_class[public_class(k)] += hc.class_products[k];
+        plan->stats.nnz_per_class[public_class(k)] += hc.class_nnz[k];
+    }
+    plan->stats.dense_units = hc.n_units;
+    plan->stats.dense_warp_rows = hc.n_warp_rows;
+    plan->stats.dense_warp_products = hc.dense_warp_products;
+    plan->stats.dense_warp_nnz = hc.dense_warp_nnz;
+    plan->stats.bitmap_bytes = (int64_t)hc.bm_words_used * 4;
+    plan->max_span_words = hc.max_span_words;
+    plan->max_warp_cnt = hc.max_warp_cnt;
+    plan->stats.launches_symbolic = c.launches;
+    return SPWS_OK;
+}
+
+spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, const i64* rowptr, int* crd, void* val) {
+    CUDA_TRY(cudaMemsetAsync(c.ctl->work_counter, 0, sizeof(c.ctl->work_counter), c.stream));
+    c.max_ub_smem = plan->max_ub_smem;
+    const spws_stats_t& s = plan->stats;
+    const int64_t* bins = plan->bin_rows;
+    for (int cls : {(int)CLS_COPY8, (int)CLS_ISM_REG8, (int)CLS_ISM_REG16, (int)CLS_ISM_REG})
+        if (bins[cls] > 0) {
+            CUDA_TRY(launch_ism_reg(c, true, cls, (int)bins[cls], S.A, S.B, rowptr, crd, val));
+            mark(plan, SPWS_T_NUM_ISM_REG);
+        }
+    if (bins[CLS_ISM_SMEM_S] > 0) {
+        CUDA_TRY(launch_ism_smem(c, true, CLS_ISM_SMEM_S, (int)bins[CLS_ISM_SMEM_S], S.A, S.B, rowptr, crd, val));
+        mark(plan, SPWS_T_NUM_ISM_SMEM_S);
+    }
+    if (bins[CLS_ISM_SMEM] > 0) {
+        CUDA_TRY(launch_ism_smem(c, true, CLS_ISM_SMEM, (int)bins[CLS_ISM_SMEM], S.A, S.B, rowptr, crd, val));
+        mark(plan, SPWS_T_NUM_ISM_SMEM);
+    }
+    if (s.dense_warp_rows > 0) {
+        CUDA_TRY(launch_dense_num_warp(c, (int)s.dense_warp_rows, plan->max_span_words, plan->max_warp_cnt, S.A, S.B, rowptr, crd, val));
+        mark(plan, SPWS_T_NUM_DENSE_WARP);
+    }
+    if (s.dense_units > 0) {
+        CUDA_TRY(launch_dense_num_cta(c, 0, (int)s.dense_units, plan->max_span_words, s.products, S.A, S.B, rowptr, crd, val));
+        mark(plan, SPWS_T_NUM_DENSE_EMIT);
+        CUDA_TRY(launch_dense_num_cta(c, 1, (int)s.dense_units, plan->max_span_words, s.products, S.A, S.B, rowptr, crd, val));
+        mark(plan, SPWS_T_NUM_DENSE_CTA);
+    }
+    if (bins[CLS_ISM_GLOBAL] > 0) {
+        CUDA_TRY(launch_ism_global(c, true, (int)bins[CLS_ISM_GLOBAL], S.A, S.B, rowptr, crd, val));
+        mark(plan, SPWS_T_NUM_ISM_GLOBAL);
+    }
+    for (int cls = CLS_HASH_S; cls <= CLS_HASH; ++cls)
+        if (bins[cls] > 0) {
+            CUDA_TRY(launch_hash(c, true, cls, (int)bins[cls], S.A, S.B, rowptr, crd, val));
+            mark(plan, SPWS_T_NUM_HASH);
+        }
+    plan->stats.launches_numeric = c.launches;
+    return SPWS_OK;
+}
+
 // ---- outer-product form (kind 2): scratch layout and the two passes -------------------------
 struct OuterLayout {
     size_t ctl, cnt, koff, block_sums, fixed_end;
@@ -412,23 +556,99 @@ int label_bits_of(int64_t I, int64_t J) {
 }
 
 // adds up what a counting kernel left in the plan's pinned slots
+// (*once, when given: the second set of slots)
 template <typename Launch>
-spws_status_t count_products(spws_plan_s* p, Launch launch, int64_t* P) {
+spws_status_t count_products(spws_plan_s* p, Launch launch, int64_t* P, int64_t* once = nullptr) {
     LaunchCtx c{};
     c.stream = p->h->stream;
     c.sm_count = p->h->sm_count;
     memset(p->host->partial, 0, sizeof(p->host->partial));
     CUDA_TRY(launch(c, p->host->partial));
     CUDA_TRY(cudaStreamSynchronize(c.stream));
-    u64 total = 0;
-    for (int b = 0; b < COUNT_BLOCKS; ++b) total += p->host->partial[b];
+    u64 total = 0, total2 = 0;
+    for (int b = 0; b < COUNT_BLOCKS; ++b) { total += p->host->partial[b]; total2 += p->host->partial[COUNT_BLOCKS + b]; }
     *P = (int64_t)total;
+    if (once) *once = (int64_t)total2;
     return SPWS_OK;
 }
 
 // products of the outer form, counted on the device
 spws_status_t outer_count_products(spws_plan_s* p, const Shapes& S, int64_t* P) {
     return count_products(p, [&](const LaunchCtx& c, u64* partial) { return launch_outer_total(c, S.A, S.B, partial); }, P);
+}
+
+// ---- second- and higher-order forms taken row by row (rowwise.cu) -----------------------------
+struct RwLayout {
+    size_t kA, kB, pA, pB, sort_tmp, pos, crd, src, val, row_key, rowptr, cols, fcnt, fpos, fcrd, fval, block_sums, bytes;
+};
+
+// n entries to sort, m rows (or the most there can be), coo: coordinate-form result of at most `outs` entries,
+// n_fib / f_entries: rows and at most so many entries of the fibre matrix F (SpMTTKRP)
+RwLayout make_rw_layout(const spws_plan_s* p, int64_t n, int64_t m, bool coo, int64_t outs, int64_t n_fib, int64_t f_entries) {
+    RwLayout R{};
+    const size_t V = p->is_f64 ? 8 : 4;
+    size_t o = 0;
+    auto take = [&](size_t bytes) { size_t at = o; o = align256(o + bytes); return at; };
+    R.kA = take(8 * (size_t)n);
+    R.kB = take(8 * (size_t)n);
+    R.pA = take(8 * (size_t)n);
+    R.pB = take(8 * (size_t)n);
+    R.sort_tmp = take(rw_sort_bytes(n));
+    R.pos = take(8 * ((size_t)m + 1));
+    R.crd = take(4 * (size_t)n);
+    R.src = take(4 * (size_t)n);
+    R.val = take(V * (size_t)n);
+    if (coo) {
+        R.row_key = take(8 * (size_t)m);
+        R.rowptr = take(8 * ((size_t)m + 1));
+        R.cols = take(4 * (size_t)outs);
+    }
+    if (p->kind == 5) {
+        R.fcnt = take(4 * (size_t)n_fib);
+        R.fpos = take(8 * ((size_t)n_fib + 1));
+        R.fcrd = take(4 * (size_t)f_entries);
+        R.fval = take(V * (size_t)f_entries);
+        R.block_sums = take(8 * ((size_t)n_fib / 2048 + 2));
+    }
+    R.bytes = o;
+    return R;
+}
+
+RowwiseBufs rw_bufs(char* x, const RwLayout& R) {
+    RowwiseBufs b{};
+    b.kA = reinterpret_cast<u64*>(x + R.kA);
+    b.kB = reinterpret_cast<u64*>(x + R.kB);
+    b.pA = reinterpret_cast<u64*>(x + R.pA);
+    b.pB = reinterpret_cast<u64*>(x + R.pB);
+    b.sort_tmp = x + R.sort_tmp;
+    b.pos = reinterpret_cast<i64*>(x + R.pos);
+    b.crd = reinterpret_cast<int*>(x + R.crd);
+    b.src = reinterpret_cast<int*>(x + R.src);
+    b.row_key = reinterpret_cast<u64*>(x + R.row_key);
+    return b;
+}
+
+// Whether `auto` takes the form row by row: always when a row's columns fit the first-order dense
+// workspace (beyond it, a row of more than 4096 products would fall to the global-memory
+// insert-sort-merge, which one long row serialises, while sorting all products does not), unless the
+// tables of m rows (about 80 bytes each) would outgrow both 1 GiB and what sorting the products
+// takes (about 48 bytes each).  A plan that sets outer_cap asks for Algorithm 1's rounds.
+// Measured per call on B200: outer 10^4 x 10^4, 1e8 products 5091 -> 1026 us against the dense
+// second-order workspace; 2e5 x 1.8e5, 12e6 products 2108 -> 1034 us and SpTTM with 43e6 products
+// 7997 -> 3126 us against the sorted products.
+bool rw_wanted(const spws_plan_s* p, int64_t m, int64_t ncols, int64_t n, int64_t P) {
+    if (p->policy != SPWS_AUTO || p->opt.outer_cap != 0 || ncols > p->opt.dense_max_span || n > 0x7fff0000ll) return false;
+    return 80.0 * (double)m <= std::max(1073741824.0, 48.0 * (double)P);
+}
+
+// Upper bound of the bitmap arena of `auto` rows: a dense row's bitmap has at most the matrix's words, and
+// no more than the routing rule allows for its products.
+size_t rw_arena_bound(const spws_plan_s* p, int64_t m, int64_t ncols, int64_t P) {
+    const double nw = (double)((ncols + 31) / 32 + 1);
+    const double slot = nw + (nw + 31) / 32 + 4;
+    const double per_product = std::max((double)p->opt.dense_span_words_per_product, 16384.0 / (double)(p->opt.ism_cta_cap + 1));
+    const double words = std::min((double)m * slot, 1.04 * per_product * (double)P + 8.0 * (double)m);
+    return align256((size_t)(words * 4.0) + 256);
 }
 
 bool outer_wants_dense(const spws_plan_s* p, int64_t I, int64_t J, int64_t P, size_t scratch_bytes, const OuterLayout& L, spws_status_t* st) {
@@ -444,12 +664,59 @@ bool outer_wants_dense(const spws_plan_s* p, int64_t I, int64_t J, int64_t P, si
     return fits && ((double)I * (double)J <= 134217728.0 || (double)P * 16.0 >= (double)I * (double)J);
 }
 
+// A's entries in the order of their output row i: the row-wise operand A' (I x K) and everything after it
+struct RwOuter { RwLayout R; Layout L; Shapes S; };
+
+RwOuter rw_outer_layout(const spws_plan_s* p, const Shapes& S, char* sc) {
+    RwOuter w{};
+    w.R = make_rw_layout(p, S.nnzA, S.m, false, 0, 0, 0);
+    w.L = make_layout(p, S.m, S.ncols, 0, S.nnzB, S.k, S.nnzA, w.R.bytes);
+    w.S = S;
+    if (sc) {
+        const RowwiseBufs b = rw_bufs(sc + w.L.extra, w.R);
+        w.S.A = Csr{b.pos, b.crd, sc + w.L.extra + w.R.val, (int)S.m, (int)S.k};
+    }
+    return w;
+}
+
+spws_status_t rw_outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_t* C, void* scratch, size_t scratch_bytes, int64_t* sizes_out) {
+    char* sc = static_cast<char*>(scratch);
+    const RwOuter w = rw_outer_layout(plan, S, sc);
+    if (scratch_bytes < w.L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
+    LaunchCtx c = make_ctx(plan, sc, scratch_bytes, w.L);
+    CUDA_TRY(cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream));
+    mark_start(plan, 0);
+    CUDA_TRY(launch_rw_outer(c, S.A, S.nnzA, S.B, S.nnzB, label_bits_of(S.m, 1), rw_bufs(sc + w.L.extra, w.R)));
+    const spws_status_t st = rows_symbolic(plan, w.S, w.L, c, nullptr, nullptr, LL(C->pos[1]), sc);
+    if (st != SPWS_OK) return st;
+    C->n[0] = C->dims[0];
+    C->n[1] = plan->stats.nnz;
+    C->n[2] = 0;
+    if (sizes_out) { sizes_out[0] = C->n[0]; sizes_out[1] = C->n[1]; sizes_out[2] = 0; }
+    plan->symbolic_ok = true;
+    plan->m = S.m;
+    plan->scratch = scratch;
+    return SPWS_OK;
+}
+
+spws_status_t rw_outer_numeric(spws_plan_s* plan, const Shapes& S, spws_tensor_t* C, void* scratch, size_t scratch_bytes) {
+    char* sc = static_cast<char*>(scratch);
+    const RwOuter w = rw_outer_layout(plan, S, sc);
+    if (scratch_bytes < w.L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
+    LaunchCtx c = make_ctx(plan, sc, scratch_bytes, w.L);
+    mark_start(plan, 1);
+    CUDA_TRY(launch_rw_values(c, S.A.val, rw_bufs(sc + w.L.extra, w.R).src, S.nnzA, sc + w.L.extra + w.R.val));
+    return rows_numeric(plan, w.S, c, LL(C->pos[1]), C->crd[1], C->val);
+}
+
 spws_status_t outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_t* C, void* scratch, size_t scratch_bytes, int64_t* sizes_out) {
     const int64_t I = S.m, K = S.k, J = S.ncols;
     if (I * J < 0 || (I > 0 && J > (int64_t)(0x7fffffffffffffffll / (I > 0 ? I : 1)))) return SPWS_INVALID_ARGUMENT;
     int64_t P = 0;
     spws_status_t st = outer_count_products(plan, S, &P);
     if (st != SPWS_OK) return st;
+    plan->rowwise = rw_wanted(plan, I, J, S.nnzA, P);
+    if (plan->rowwise) return rw_outer_symbolic(plan, S, C, scratch, scratch_bytes, sizes_out);
     if (P > 0x7fff0000ll) return SPWS_INTERNAL_OVERFLOW;            // product ordinals and scans are 31-bit here
     const OuterLayout L = make_outer_layout(plan, I, K, J, P);
     if (scratch_bytes < L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
@@ -520,6 +787,7 @@ spws_status_t outer_numeric(spws_plan_s* plan, const Shapes& S, spws_tensor_t* C
     const int64_t I = S.m, K = S.k, J = S.ncols, P = plan->outer_products;
     if (C->n[1] < plan->stats.nnz) return SPWS_OUTPUT_TOO_SMALL;
     if (plan->stats.nnz > 0 && (!C->crd[1] || !C->val)) return SPWS_INVALID_ARGUMENT;
+    if (plan->rowwise) return rw_outer_numeric(plan, S, C, scratch, scratch_bytes);
     const OuterLayout L = make_outer_layout(plan, I, K, J, P);
     if (scratch_bytes < (plan->outer_dense ? L.dense_end : L.ism_end)) return SPWS_SCRATCH_TOO_SMALL;
     char* sc = static_cast<char*>(scratch);
@@ -558,6 +826,7 @@ struct HShapes {
     int form;                   // 0 SpTTM, 1 SpTTM-I, 2 SpMTTKRP
     Csf3Dev B;
     Csr C, D;
+    int64_t nnzC;
     int order;                  // of the output
     int64_t odims[3];
     u64 d1, d2;                 // label = (c_a * d1 + c_b) * d2 + c_c, or c_a * d2 + c_b
@@ -576,6 +845,7 @@ spws_status_t check_higher(const spws_plan_s* p, const spws_tensor_t* B, const s
     if (C->dims[0] < 0 || C->dims[1] < 0 || C->dims[1] > 0x7ffffff0ll || C->n[1] < 0) return SPWS_INVALID_ARGUMENT;
     H.B = Csf3Dev{LL(B->pos[1]), LL(B->pos[2]), B->crd[0], B->crd[1], B->crd[2], B->val, (int)B->n[0], (int)B->n[1], B->n[2]};
     H.C = Csr{LL(C->pos[1]), C->crd[1], C->val, (int)C->dims[0], (int)C->dims[1]};
+    H.nnzC = C->n[1];
     H.D = Csr{};
     if (H.form == 0) {          // B(k,i,j), C(k,l) -> (i,j,l)
         if (C->dims[0] != B->dims[0]) return SPWS_DIM_MISMATCH;
@@ -637,16 +907,102 @@ HLayout make_hlayout(const spws_plan_s* p, const HShapes& H, int64_t P) {
     return L;
 }
 
-spws_status_t higher_count_products(spws_plan_s* p, const HShapes& H, int64_t* P) {
-    return count_products(p, [&](const LaunchCtx& c, u64* partial) { return launch_higher_total(c, H.form, H.B, H.C, partial); }, P);
+spws_status_t higher_count_products(spws_plan_s* p, const HShapes& H, int64_t* P, int64_t* once) {
+    return count_products(p, [&](const LaunchCtx& c, u64* partial) { return launch_higher_total(c, H.form, H.B, H.C, partial); }, P, once);
+}
+
+// The tensor's entries in the order of their output row: (i,j), (k,j) or i, of which at most m occur.  The matrix the
+// rows pick from is C, or F with a row per stored fibre for SpMTTKRP.
+struct RwHigher { RwLayout R; Layout L; Shapes S; int64_t m; int bits; };
+
+int64_t rw_higher_rows(const HShapes& H) {
+    const double space = H.order == 3 ? (double)H.odims[0] * (double)H.odims[1] : (double)H.odims[0];
+    return space < (double)H.B.nnz ? (int64_t)space : (int64_t)H.B.nnz;
+}
+
+RwHigher rw_higher_layout(const spws_plan_s* p, const HShapes& H, int64_t P, int64_t once, char* sc) {
+    RwHigher w{};
+    const int64_t n = H.B.nnz, ncols = H.odims[H.order - 1];
+    w.m = rw_higher_rows(H);
+    w.bits = H.order == 3 ? label_bits_of(H.odims[0], H.odims[1]) : label_bits_of(H.odims[0], 1);
+    const bool fibres = H.form == 2;
+    const int64_t k = fibres ? H.B.n1 : H.C.nrows;
+    const double most = std::min((double)P, (double)w.m * (double)ncols);
+    w.R = make_rw_layout(p, n, w.m, true, (int64_t)most, fibres ? H.B.n1 : 0, fibres ? once : 0);
+    w.S.m = w.m; w.S.k = k; w.S.ncols = ncols; w.S.nnzA = n; w.S.nnzB = fibres ? once : H.nnzC; w.S.n_i = 0;
+    w.L = make_layout(p, w.m, ncols, 0, w.S.nnzB, k, n, w.R.bytes);
+    if (sc) {
+        char* x = sc + w.L.extra;
+        const RowwiseBufs b = rw_bufs(x, w.R);
+        w.S.A = Csr{b.pos, b.crd, x + w.R.val, (int)w.m, (int)k};
+        w.S.B = fibres ? Csr{reinterpret_cast<i64*>(x + w.R.fpos), reinterpret_cast<int*>(x + w.R.fcrd), x + w.R.fval, (int)k, (int)ncols} : H.C;
+    }
+    return w;
+}
+
+bool rw_higher_wanted(const spws_plan_s* p, const HShapes& H, int64_t P) {
+    return rw_wanted(p, rw_higher_rows(H), H.odims[H.order - 1], H.B.nnz, P);
+}
+
+spws_status_t rw_higher_symbolic(spws_plan_s* plan, const HShapes& H, int64_t P, int64_t once, spws_tensor_t* Out, void* scratch,
+                                 size_t scratch_bytes, int64_t* sizes_out) {
+    char* sc = static_cast<char*>(scratch);
+    const RwHigher w = rw_higher_layout(plan, H, P, once, sc);
+    if (scratch_bytes < w.L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
+    LaunchCtx c = make_ctx(plan, sc, scratch_bytes, w.L);
+    char* x = sc + w.L.extra;
+    CUDA_TRY(cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream));
+    mark_start(plan, 0);
+    if (H.form == 2)
+        CUDA_TRY(launch_rw_fibre_rows(c, false, H.B, H.C, H.D, reinterpret_cast<int*>(x + w.R.fcnt), reinterpret_cast<i64*>(x + w.R.fpos),
+                                      reinterpret_cast<int*>(x + w.R.fcrd), nullptr, reinterpret_cast<i64*>(x + w.R.block_sums)));
+    CUDA_TRY(launch_rw_csf(c, H.form, H.B, (u64)(H.order == 3 ? H.odims[1] : 1), w.m, w.bits, rw_bufs(x, w.R)));
+    const spws_status_t st = rows_symbolic(plan, w.S, w.L, c, nullptr, nullptr, reinterpret_cast<i64*>(x + w.R.rowptr), sc);
+    if (st != SPWS_OK) return st;
+    plan->stats.rows = H.B.nnz;
+    plan->stats.products = P;
+    plan->outer_products = P;
+    plan->rw_once = once;
+    Out->n[0] = plan->stats.nnz; Out->n[1] = 0; Out->n[2] = 0;
+    if (sizes_out) { sizes_out[0] = plan->stats.nnz; sizes_out[1] = 0; sizes_out[2] = 0; }
+    plan->symbolic_ok = true;
+    plan->m = H.B.nnz;
+    plan->scratch = scratch;
+    return SPWS_OK;
+}
+
+spws_status_t rw_higher_numeric(spws_plan_s* plan, const HShapes& H, spws_tensor_t* Out, void* scratch, size_t scratch_bytes) {
+    char* sc = static_cast<char*>(scratch);
+    const RwHigher w = rw_higher_layout(plan, H, plan->outer_products, plan->rw_once, sc);
+    if (scratch_bytes < w.L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
+    LaunchCtx c = make_ctx(plan, sc, scratch_bytes, w.L);
+    char* x = sc + w.L.extra;
+    const RowwiseBufs b = rw_bufs(x, w.R);
+    const i64* rowptr = reinterpret_cast<const i64*>(x + w.R.rowptr);
+    int* cols = reinterpret_cast<int*>(x + w.R.cols);
+    mark_start(plan, 1);
+    CUDA_TRY(launch_rw_values(c, H.B.val, b.src, H.B.nnz, x + w.R.val));
+    if (H.form == 2)
+        CUDA_TRY(launch_rw_fibre_rows(c, true, H.B, H.C, H.D, nullptr, reinterpret_cast<i64*>(x + w.R.fpos), nullptr, x + w.R.fval, nullptr));
+    const spws_status_t st = rows_numeric(plan, w.S, c, rowptr, cols, Out->val);
+    if (st != SPWS_OK) return st;
+    CUDA_TRY(launch_rw_coords(c, H.order, rowptr, b.row_key, w.m, plan->stats.nnz, (u64)(H.order == 3 ? H.odims[1] : 1), cols, Out->crd[0],
+                              Out->crd[1], Out->crd[2]));
+    plan->stats.launches_numeric = c.launches;
+    return SPWS_OK;
 }
 
 spws_status_t higher_workspace_size(spws_plan_s* plan, const spws_tensor_t* B, const spws_tensor_t* C, const spws_tensor_t* D, size_t* bytes) {
     HShapes H{};
     spws_status_t st = check_higher(plan, B, C, D, H, true);
     if (st != SPWS_OK) return st;
-    int64_t P = 0;
-    if ((st = higher_count_products(plan, H, &P)) != SPWS_OK) return st;
+    int64_t P = 0, once = 0;
+    if ((st = higher_count_products(plan, H, &P, &once)) != SPWS_OK) return st;
+    if (rw_higher_wanted(plan, H, P)) {
+        const RwHigher w = rw_higher_layout(plan, H, P, once, nullptr);
+        *bytes = w.L.fixed_end + rw_arena_bound(plan, w.m, w.S.ncols, P);
+        return SPWS_OK;
+    }
     *bytes = make_hlayout(plan, H, P).end;
     return SPWS_OK;
 }
@@ -666,8 +1022,10 @@ spws_status_t higher_symbolic(spws_plan_s* plan, const spws_tensor_t* B, const s
     if (st != SPWS_OK) return st;
     if ((st = check_coo_output(H, Out)) != SPWS_OK) return st;
     if (!scratch || (reinterpret_cast<uintptr_t>(scratch) & 255)) return SPWS_INVALID_ARGUMENT;
-    int64_t P = 0;
-    if ((st = higher_count_products(plan, H, &P)) != SPWS_OK) return st;
+    int64_t P = 0, once = 0;
+    if ((st = higher_count_products(plan, H, &P, &once)) != SPWS_OK) return st;
+    plan->rowwise = rw_higher_wanted(plan, H, P);
+    if (plan->rowwise) return rw_higher_symbolic(plan, H, P, once, Out, scratch, scratch_bytes, sizes_out);
     if (P > 0x7fff0000ll || H.B.nnz > 0x7fff0000ll) return SPWS_INTERNAL_OVERFLOW;       // ordinals and scans are 31-bit here
     const HLayout L = make_hlayout(plan, H, P);
     if (scratch_bytes < L.end) return SPWS_SCRATCH_TOO_SMALL;
@@ -730,6 +1088,7 @@ spws_status_t higher_numeric(spws_plan_s* plan, const spws_tensor_t* B, const sp
         if (!Out->val) return SPWS_INVALID_ARGUMENT;
         for (int a = 0; a < H.order; ++a) if (!Out->crd[a]) return SPWS_INVALID_ARGUMENT;
     }
+    if (plan->rowwise) return rw_higher_numeric(plan, H, Out, scratch, scratch_bytes);
     const HLayout L = make_hlayout(plan, H, P);
     if (scratch_bytes < L.end) return SPWS_SCRATCH_TOO_SMALL;
     char* sc = static_cast<char*>(scratch);
@@ -898,6 +1257,10 @@ spws_status_t spws_workspace_size(spws_plan_t plan, const spws_tensor_t* A, cons
     if (plan->kind == 2) {                      // sized by the number of products, counted on the device
         int64_t P = 0;
         if ((st = outer_count_products(plan, S, &P)) != SPWS_OK) return st;
+        if (rw_wanted(plan, S.m, S.ncols, S.nnzA, P)) {
+            *bytes = rw_outer_layout(plan, S, nullptr).L.fixed_end + rw_arena_bound(plan, S.m, S.ncols, P);
+            return SPWS_OK;
+        }
         const OuterLayout OL = make_outer_layout(plan, S.m, S.k, S.ncols, P);
         const size_t dense_ok = (double)S.m * (double)S.ncols <= 2.0e9 ? OL.dense_end : 0;     // a dense workspace beyond 2^31 cells is never offered
         *bytes = (plan->policy == SPWS_SPARSE_ISM || plan->policy == SPWS_HASH) ? OL.ism_end
@@ -975,97 +1338,10 @@ spws_status_t spws_symbolic(spws_plan_t plan, const spws_tensor_t* A, const spws
         CUDA_TRY(cudaStreamSynchronize(stream));
         if (plan->host_ctl->status != 0) return from_dev_status(plan->host_ctl->status);
     }
-    // a1: upper bounds + classes; a2: binning
     mark_start(plan, 0);
-    CUDA_TRY(launch_row_bounds(c, S.A, S.B, S.nnzA));
-    CUDA_TRY(launch_bw_build(c, S.B));
-    mark(plan, SPWS_T_SYM_BOUNDS);
-    CUDA_TRY(launch_bin_rows(c, (int)S.m));
-    mark(plan, SPWS_T_SYM_BIN);
-    // the class sizes come back now, so that only the workspaces that have rows are launched, with
-    // grids sized for them (a launch for an empty class costs as much as a small class's work)
-    int* hcount = plan->host_ctl->class_count;
-    CUDA_TRY(cudaMemcpyAsync(hcount, c.ctl->class_count, sizeof(int) * NCLASS, cudaMemcpyDeviceToHost, stream));
-    CUDA_TRY(cudaMemcpyAsync(&plan->host_ctl->max_ub_smem, &c.ctl->max_ub_smem, sizeof(i64), cudaMemcpyDeviceToHost, stream));
-    CUDA_TRY(cudaStreamSynchronize(stream));
-    plan->max_ub_smem = plan->host_ctl->max_ub_smem;
-    c.max_ub_smem = plan->max_ub_smem;
-    // a3: exact count per row through the workspace of its class
     i64* rowptr = (plan->kind == 0) ? LL(C->pos[1]) : reinterpret_cast<i64*>(sc + L.rowptr_raw);
-    if (S.m > 0) {
-        for (int cls = CLS_ISM_REG8; cls <= CLS_ISM_REG; ++cls)
-            if (hcount[cls] > 0) {
-                CUDA_TRY(launch_ism_reg(c, false, cls, hcount[cls], S.A, S.B, rowptr, nullptr, nullptr));
-                mark(plan, SPWS_T_SYM_ISM_REG);
-            }
-        // under `auto` the rows of the shared-memory insert-sort-merge classes are counted through a
-        // hash set of their columns: the count needs no order
-        const bool count_by_hash = plan->policy == SPWS_AUTO;
-        if (hcount[CLS_ISM_SMEM_S] > 0) {
-            if (count_by_hash) CUDA_TRY(launch_hash(c, false, CLS_ISM_SMEM_S, hcount[CLS_ISM_SMEM_S], S.A, S.B, rowptr, nullptr, nullptr));
-            else CUDA_TRY(launch_ism_smem(c, false, CLS_ISM_SMEM_S, hcount[CLS_ISM_SMEM_S], S.A, S.B, rowptr, nullptr, nullptr));
-            mark(plan, SPWS_T_SYM_ISM_SMEM_S);
-        }
-        if (hcount[CLS_ISM_SMEM] > 0) {
-            if (count_by_hash) CUDA_TRY(launch_hash(c, false, CLS_ISM_SMEM, hcount[CLS_ISM_SMEM], S.A, S.B, rowptr, nullptr, nullptr));
-            else CUDA_TRY(launch_ism_smem(c, false, CLS_ISM_SMEM, hcount[CLS_ISM_SMEM], S.A, S.B, rowptr, nullptr, nullptr));
-            mark(plan, SPWS_T_SYM_ISM_SMEM);
-        }
-        if (hcount[CLS_DENSE_WARP] > 0) {
-            CUDA_TRY(launch_dense_sym_warp(c, S.A, S.B));
-            mark(plan, SPWS_T_SYM_DENSE_WARP);
-        }
-        if (hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0) {
-            CUDA_TRY(launch_dense_sym_cta(c, S.A, S.B));
-            mark(plan, SPWS_T_SYM_DENSE_CTA);
-        }
-        if (hcount[CLS_ISM_GLOBAL] > 0) {
-            CUDA_TRY(launch_ism_global(c, false, hcount[CLS_ISM_GLOBAL], S.A, S.B, rowptr, nullptr, nullptr));
-            mark(plan, SPWS_T_SYM_ISM_GLOBAL);
-        }
-        for (int cls = CLS_HASH_S; cls <= CLS_HASH; ++cls)
-            if (hcount[cls] > 0) {
-                CUDA_TRY(launch_hash(c, false, cls, hcount[cls], S.A, S.B, rowptr, nullptr, nullptr));
-                mark(plan, SPWS_T_SYM_HASH);
-            }
-    }
-    // a4: exclusive scan into the row pointer
-    if (plan->kind == 1) {
-        // with C's fibre and slice levels rebuilt from the fibres that produced an output
-        CUDA_TRY(launch_ttm_scan_compact(c, (int)S.n_i, (int)S.m, LL(A->pos[1]), A->crd[0], A->crd[1], rowptr,
-                                         reinterpret_cast<i64*>(sc + L.fpos), reinterpret_cast<int*>(sc + L.sflags),
-                                         reinterpret_cast<i64*>(sc + L.spos), reinterpret_cast<i64*>(sc + L.block_sums), &c.ctl->nnz,
-                                         LL(C->pos[0]), C->crd[0], LL(C->pos[1]), C->crd[1], LL(C->pos[2])));
-    } else {
-        CUDA_TRY(launch_scan_counts(c, c.tab.cnt, (int)S.m, rowptr, reinterpret_cast<i64*>(sc + L.block_sums), &c.ctl->nnz));
-    }
-    if (hcount[CLS_DENSE_WARP] + hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0) CUDA_TRY(launch_dense_rebin(c, (int)S.m, rowptr));
-    CUDA_TRY(launch_class_nnz(c, (int)S.m));
-    mark(plan, SPWS_T_SYM_SCAN);
-    CUDA_TRY(cudaMemcpyAsync(plan->host_ctl, c.ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, stream));
-    CUDA_TRY(cudaStreamSynchronize(stream));
+    if ((st = rows_symbolic(plan, S, L, c, plan->kind == 1 ? A : nullptr, C, rowptr, sc)) != SPWS_OK) return st;
     const DevCtl& hc = *plan->host_ctl;
-    plan->stats = spws_stats_t{};
-    plan->stats.device_status = hc.status;
-    if (hc.status != 0) return from_dev_status(hc.status);
-    plan->stats.rows = S.m;
-    plan->stats.products = hc.products;
-    plan->stats.nnz = hc.nnz;
-    plan->stats.max_row_products = hc.max_ub;
-    for (int k = 0; k < NCLASS; ++k) {
-        plan->bin_rows[k] = hc.class_count[k];
-        plan->stats.rows_per_class[public_class(k)] += hc.class_count[k];
-        plan->stats.products_per_class[public_class(k)] += hc.class_products[k];
-        plan->stats.nnz_per_class[public_class(k)] += hc.class_nnz[k];
-    }
-    plan->stats.dense_units = hc.n_units;
-    plan->stats.dense_warp_rows = hc.n_warp_rows;
-    plan->stats.dense_warp_products = hc.dense_warp_products;
-    plan->stats.dense_warp_nnz = hc.dense_warp_nnz;
-    plan->stats.bitmap_bytes = (int64_t)hc.bm_words_used * 4;
-    plan->max_span_words = hc.max_span_words;
-    plan->max_warp_cnt = hc.max_warp_cnt;
-    plan->stats.launches_symbolic = c.launches;
     if (plan->kind == 0) {
         C->n[0] = C->dims[0];
         C->n[1] = hc.nnz;
@@ -1102,46 +1378,8 @@ spws_status_t spws_numeric(spws_plan_t plan, const spws_tensor_t* A, const spws_
     char* sc = static_cast<char*>(scratch);
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, L);
     const i64* rowptr = (plan->kind == 0) ? LL(C->pos[1]) : reinterpret_cast<const i64*>(sc + L.rowptr_raw);
-    CUDA_TRY(cudaMemsetAsync(c.ctl->work_counter, 0, sizeof(c.ctl->work_counter), c.stream));
     mark_start(plan, 1);
-    c.max_ub_smem = plan->max_ub_smem;
-    const spws_stats_t& s = plan->stats;
-    int* crd = C->crd[last];
-    const int64_t* bins = plan->bin_rows;
-    for (int cls : {(int)CLS_COPY8, (int)CLS_ISM_REG8, (int)CLS_ISM_REG16, (int)CLS_ISM_REG})
-        if (bins[cls] > 0) {
-            CUDA_TRY(launch_ism_reg(c, true, cls, (int)bins[cls], S.A, S.B, rowptr, crd, C->val));
-            mark(plan, SPWS_T_NUM_ISM_REG);
-        }
-    if (bins[CLS_ISM_SMEM_S] > 0) {
-        CUDA_TRY(launch_ism_smem(c, true, CLS_ISM_SMEM_S, (int)bins[CLS_ISM_SMEM_S], S.A, S.B, rowptr, crd, C->val));
-        mark(plan, SPWS_T_NUM_ISM_SMEM_S);
-    }
-    if (bins[CLS_ISM_SMEM] > 0) {
-        CUDA_TRY(launch_ism_smem(c, true, CLS_ISM_SMEM, (int)bins[CLS_ISM_SMEM], S.A, S.B, rowptr, crd, C->val));
-        mark(plan, SPWS_T_NUM_ISM_SMEM);
-    }
-    if (s.dense_warp_rows > 0) {
-        CUDA_TRY(launch_dense_num_warp(c, (int)s.dense_warp_rows, plan->max_span_words, plan->max_warp_cnt, S.A, S.B, rowptr, crd, C->val));
-        mark(plan, SPWS_T_NUM_DENSE_WARP);
-    }
-    if (s.dense_units > 0) {
-        CUDA_TRY(launch_dense_num_cta(c, 0, (int)s.dense_units, plan->max_span_words, s.products, S.A, S.B, rowptr, crd, C->val));
-        mark(plan, SPWS_T_NUM_DENSE_EMIT);
-        CUDA_TRY(launch_dense_num_cta(c, 1, (int)s.dense_units, plan->max_span_words, s.products, S.A, S.B, rowptr, crd, C->val));
-        mark(plan, SPWS_T_NUM_DENSE_CTA);
-    }
-    if (bins[CLS_ISM_GLOBAL] > 0) {
-        CUDA_TRY(launch_ism_global(c, true, (int)bins[CLS_ISM_GLOBAL], S.A, S.B, rowptr, crd, C->val));
-        mark(plan, SPWS_T_NUM_ISM_GLOBAL);
-    }
-    for (int cls = CLS_HASH_S; cls <= CLS_HASH; ++cls)
-        if (bins[cls] > 0) {
-            CUDA_TRY(launch_hash(c, true, cls, (int)bins[cls], S.A, S.B, rowptr, crd, C->val));
-            mark(plan, SPWS_T_NUM_HASH);
-        }
-    plan->stats.launches_numeric = c.launches;
-    return SPWS_OK;
+    return rows_numeric(plan, S, c, rowptr, C->crd[last], C->val);
 }
 
 spws_status_t spws_gather_ceiling(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, const spws_tensor_t* C,

@@ -632,6 +632,65 @@ def test_higher_order_scatters_match_the_oracle(ctx, oracle_mod, dims, nnz, L, s
             assert ok.all(), expr
 
 
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("dims,nnz,L,density", [((1, 1, 1), 1, 1, 1.0), ((6, 7, 8), 80, 9, 0.4), ((3, 40, 50), 1023, 33, 0.3), ((40, 30, 50), 1025, 64, 0.3),
+                                                ((9, 100, 200), 8193, 4097, 0.02), ((8, 64, 2), 700, 300, 0.5)])
+def test_scatters_taken_row_by_row(ctx, oracle_mod, dims, nnz, L, density, dtype):
+    """`auto` puts the tensor's entries in output-row order and runs the row-wise passes: entries at and
+    around the tiles that number the rows (1024), rows of one to thousands of products, every label
+    present and few of them, empty rows of the matrices."""
+    from paper_2404_04541_b200 import api
+    B = uniform_csf3(dims, nnz, nnz + L, dtype=dtype)
+    dB = api.DeviceCSF3.from_host(B)
+    M0 = random_csr(dims[0], L, density, 5, empty_row_frac=0.2, dtype=dtype)
+    M1 = random_csr(dims[1], L, density, 6, empty_row_frac=0.2, dtype=dtype)
+    for expr, fn, mats in [(api.EXPR_SPTTM, oracle_mod.spttm, [M0]), (api.EXPR_SPTTM_I, oracle_mod.spttm_i, [M1]),
+                           (api.EXPR_SPMTTKRP, oracle_mod.spmttkrp, [M0, M1])]:
+        ref = fn(B, *mats)
+        crd, val, stats = ctx.scatter_coo(expr, dB, *[api.DeviceCSR.from_host(m) for m in mats])
+        assert stats["nnz"] == ref.nnz and crd.shape == (ref.nnz, 2 if expr == api.EXPR_SPMTTKRP else 3) and crd.is_contiguous(), expr
+        assert np.array_equal(crd.cpu().numpy().astype(np.int64), ref.crd), expr
+        ok, _ = values_close(val.cpu().numpy(), ref.val_ref, ref.abs, TOL[np.dtype(dtype)])
+        assert ok.all(), expr
+
+
+@pytest.mark.parametrize("m,k,n,dens", [(1, 1, 1, 1.0), (300, 20, 5000, 0.1), (2048, 33, 40, 0.02), (5, 3000, 1 << 19, 0.3), (5, 300, (1 << 19) + 1, 0.3)])
+def test_outer_product_taken_row_by_row(ctx, oracle_mod, m, k, n, dens):
+    """`auto` sorts A's entries by output row; at the widest column space the row workspace covers and just
+    beyond it (where the products are sorted instead), with value changes between two numeric passes."""
+    from paper_2404_04541_b200 import api, binding
+    A = random_csr(m, k, dens, 31, empty_row_frac=0.1)
+    B = uniform_rows_csr(k, n, 9, 32) if n > 9 else random_csr(k, n, 0.7, 32)
+    dAt, dB = api.DeviceCSR.from_host(A.transpose()), api.DeviceCSR.from_host(B)
+    plan = ctx.plan(api.EXPR_OUTER, (binding.SPWS_CSR,) * 3, np.float64)
+    c, state = ctx.outer_symbolic(plan, dAt, dB)
+    for scale in (1.0, -3.0):
+        dAt.val.mul_(scale)
+        A.val *= scale
+        ref = oracle_mod.spgemm(A, B, threads=4)
+        C = ctx.spgemm_numeric(plan, c, state)
+        plan.get_stats()
+        assert_matches((C.pos.cpu().numpy(), C.crd.cpu().numpy(), C.val.cpu().numpy()), ref, np.float64)
+    plan.close()
+
+
+def test_forms_taken_row_by_row_report_coordinates_out_of_range(ctx):
+    from paper_2404_04541_b200 import api, binding
+    At, B = random_csr(40, 30, 0.3, 1), random_csr(40, 50, 0.3, 2)
+    for where, limit in ((At, 30), (B, 50)):
+        keep = where.crd[3]
+        where.crd[3] = limit
+        with pytest.raises(binding.SpwsError) as e:
+            ctx.spgemm_outer(api.DeviceCSR.from_host(At), api.DeviceCSR.from_host(B))
+        assert e.value.status == binding.SPWS_NONCANONICAL_INPUT
+        where.crd[3] = keep
+    T = uniform_csf3((6, 7, 8), 80, 3)
+    T.crd0[2] = 6                                       # picks a row that C does not have
+    with pytest.raises(binding.SpwsError) as e:
+        ctx.scatter_coo(api.EXPR_SPTTM, api.DeviceCSF3.from_host(T), api.DeviceCSR.from_host(random_csr(6, 9, 0.5, 4)))
+    assert e.value.status == binding.SPWS_NONCANONICAL_INPUT
+
+
 def test_higher_order_scatters_refuse_a_dense_workspace(ctx):
     from paper_2404_04541_b200 import api, binding
     with pytest.raises(binding.SpwsError) as e:
