@@ -29,12 +29,15 @@ constexpr int NUM_SLOT = 16;   // work_counter[cls] in the symbolic pass, work_c
 constexpr int CEIL_SLOT = 32;  // work_counter[CEIL_SLOT + cls] in the gather-only (iteration-only) kernels
 constexpr int EMIT_SLOT = 48;  // work_counter slot of the coordinate emission of the CTA dense route
 constexpr int BW_SLOT = 49;    // work_counter slot of the word-list build
+constexpr int ISM_CTA_SLOT = 50; // work_counter slots of the CTA kernel of the shared-memory ISM, symbolic and numeric
+constexpr int ISM_CTA_NUM_SLOT = 51;
 constexpr int N_WORK_COUNTERS = 64;
 // index of a class in the public statistics (the three register classes are reported as one)
 __host__ __device__ inline int public_class(int cls) { return cls == 0 ? 0 : ((cls <= 3 || cls == 12) ? 1 : cls - 2); }
 constexpr int N_PUBLIC_CLASS = 10;
 constexpr int HASH_SMALL_CAP = 1024;       // products of a row the small / the full hash workspace takes
 constexpr int HASH_CAP = 4096;
+constexpr int ISM_WARP_MAX = 1024;         // products of a row the warp kernel of the shared-memory ISM takes
 
 // Capacities fixed at compile time.
 constexpr int DENSE_WARP_BM_WORDS = 1024;  // bitmap words a warp-per-row workspace may span (32768 columns)
@@ -215,6 +218,14 @@ __device__ __forceinline__ i64 lower_bound_crd(const int* __restrict__ crd, i64 
         if ((i64)__ldg(crd + mid) < c) lo = mid + 1; else hi = mid;
     }
     return lo;
+}
+
+// lanes per A entry: the smallest power of two >= the mean B-row segment length
+__device__ __forceinline__ int pick_group_size(i64 ub, i64 entries, int parts) {
+    const float avg = (float)ub / fmaxf(1.0f, (float)entries * (float)parts);
+    int gs = 32;
+    while (gs > 1 && (float)(gs >> 1) >= avg) gs >>= 1;
+    return gs;
 }
 
 // Products are formed as a rounded multiply followed by rounded adds (no contraction), so the

@@ -43,14 +43,6 @@ constexpr i64 BM_OFF_MASK = (1ll << BM_NZW_SHIFT) - 1;
 // the chunk's first bit (an exclusive prefix of the chunk popcounts).
 __device__ __forceinline__ int chunks_of(int nw) { return (nw + 31) >> 5; }
 
-// lanes per A entry: the smallest power of two >= the mean B-row segment length
-__device__ __forceinline__ int pick_group_size(i64 ub, i64 entries, int parts) {
-    const float avg = (float)ub / fmaxf(1.0f, (float)entries * (float)parts);
-    int gs = 32;
-    while (gs > 1 && (float)(gs >> 1) >= avg) gs >>= 1;
-    return gs;
-}
-
 // ---------------------------------------------------------------------------------------
 // symbolic, warp per row
 // ---------------------------------------------------------------------------------------

@@ -18,7 +18,7 @@ constexpr int HASH_EMPTY = -1;
 
 template <typename T, int CAP, int THREADS, bool NUMERIC>
 __global__ void __launch_bounds__(THREADS) hash_kernel(const int* __restrict__ perm, DevCtl* __restrict__ ctl, int cls, int counter_slot,
-                                                       Csr A, Csr B, const i64* __restrict__ ub, int* __restrict__ cnt,
+                                                       i64 above, Csr A, Csr B, const i64* __restrict__ ub, int* __restrict__ cnt,
                                                        const i64* __restrict__ rowptr, int* __restrict__ Ccrd, T* __restrict__ Cval) {
     constexpr int SLOTS = 2 * CAP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(THREADS) hash_kernel(const int* __restrict__ p
         const int r = s_next;
         if (r >= n) break;
         const int row = rows[r];
+        if (ub[row] <= above) continue;                 // rows another kernel takes
         const i64 ps = A.pos[row], pe = A.pos[row + 1];
         // the numeric pass knows the row's distinct columns and sizes the table from them
         // (the counting pass sizes it from the row's product count, an upper bound of them)
@@ -168,7 +169,9 @@ static size_t hash_smem_bytes(bool numeric) {
 template <typename T, int CAP, int THREADS, bool NUMERIC>
 static cudaError_t hash_launch_k(const LaunchCtx& c, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
     const size_t smem = hash_smem_bytes<T, CAP, THREADS>(NUMERIC);
-    const int slot = cls + (NUMERIC ? NUM_SLOT : 0);
+    // the counting pass also serves the shared-memory insert-sort-merge rows of more than 1024 products
+    const bool ism = cls == CLS_ISM_SMEM;
+    const int slot = ism ? ISM_CTA_SLOT : cls + (NUMERIC ? NUM_SLOT : 0);
     cudaError_t e;
     int per_sm = 0;
     auto k = hash_kernel<T, CAP, THREADS, NUMERIC>;
@@ -176,7 +179,7 @@ static cudaError_t hash_launch_k(const LaunchCtx& c, int cls, int n_host, const 
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, THREADS, smem)) != cudaSuccess) return e;
     i64 grid = (i64)c.sm_count * (per_sm > 0 ? per_sm : 1);
     if (n_host >= 0 && n_host < grid) grid = n_host > 0 ? n_host : 1;
-    k<<<(int)grid, THREADS, smem, c.stream>>>(c.tab.perm, c.ctl, cls, slot, A, B, c.tab.ub, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
+    k<<<(int)grid, THREADS, smem, c.stream>>>(c.tab.perm, c.ctl, cls, slot, ism ? (i64)ISM_WARP_MAX : 0, A, B, c.tab.ub, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
     ++c.launches;
     return cudaGetLastError();
 }
@@ -184,9 +187,7 @@ static cudaError_t hash_launch_k(const LaunchCtx& c, int cls, int n_host, const 
 template <typename T>
 static cudaError_t hash_launch_t(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr,
                                  int* Ccrd, void* Cval) {
-    // the counting pass also serves the shared-memory insert-sort-merge classes (no sort is needed to
-    // count distinct columns); their rows have at most HASH_CAP products
-    if (!numeric && cls == CLS_ISM_SMEM_S) return hash_launch_k<T, HASH_SMALL_CAP, 128, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
+    // shared-memory insert-sort-merge rows have at most HASH_CAP products
     if (!numeric && cls == CLS_ISM_SMEM) return hash_launch_k<T, HASH_CAP, 256, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
     if (cls == CLS_HASH_S)
         return numeric ? hash_launch_k<T, HASH_SMALL_CAP, 128, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)

@@ -1,6 +1,6 @@
-// Insert-sort-merge workspace in shared memory: one CTA per output row with at most CAP
-// products (Algorithm 1; the accumulation array is the CTA's shared memory and is never full
-// because the symbolic upper bound sized it; coordinate-sort policy, Sec. 5.2).
+// Insert-sort-merge workspace of mid-size rows: a warp per output row with at most 1024 products, a
+// CTA per row beyond (Algorithm 1; the accumulation array is shared memory and is never full because
+// the symbolic upper bound sized it; coordinate-sort policy, Sec. 5.2).
 //   Insert : product t of the row (loop order k, then j) is appended at slot t: its value stays
 //            there, and the packed word (j, t) enters the sort (accumulation indexing, Sec. 5.1:
 //            only integers move).  The word is 32 bits (j << log2 CAP | t) when the column count
@@ -32,8 +32,9 @@ template <int CAP> struct Pack<unsigned, CAP> {
 
 template <typename T, typename P, int CAP, int THREADS, bool NUMERIC>
 __global__ void __launch_bounds__(THREADS) ism_smem_kernel(const int* __restrict__ perm, DevCtl* __restrict__ ctl, int cls,
-                                                           int counter_slot, Csr A, Csr B, int* __restrict__ cnt,
-                                                           const i64* __restrict__ rowptr, int* __restrict__ Ccrd, T* __restrict__ Cval) {
+                                                           int counter_slot, i64 above, Csr A, Csr B, const i64* __restrict__ ub,
+                                                           int* __restrict__ cnt, const i64* __restrict__ rowptr, int* __restrict__ Ccrd,
+                                                           T* __restrict__ Cval) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     typedef Pack<P, CAP> PK;
     T* vals = reinterpret_cast<T*>(smem_raw);                             // CAP (numeric only)
@@ -59,6 +60,7 @@ __global__ void __launch_bounds__(THREADS) ism_smem_kernel(const int* __restrict
         const int r = s_next;
         if (r >= n) break;
         const int row = rows[r];
+        if (ub[row] <= above) continue;                 // the warp kernel's rows
         const i64 ps = A.pos[row], pe = A.pos[row + 1];
 
         // ---- Insert
@@ -144,6 +146,209 @@ __global__ void __launch_bounds__(THREADS) ism_smem_kernel(const int* __restrict
     }
 }
 
+// ---------------------------------------------------------------------------------------
+// A warp per row, the sort in registers.  Lane l holds E packed words; comparisons over a distance
+// below E stay inside the lane, longer ones cost one shuffle per word, and no barrier is left: a
+// network in shared memory took about 12 warp instructions per product and 55 barriers at 1024
+// products, this one about 2.7.  Bound by instruction issue.
+//   Insert : 32 A entries at a time; a group of lanes per entry (as many as the mean B row has
+//            entries) writes the products of its B row at their slots.
+//   Sort   : E = 2 .. 32 words per lane, the smallest network that holds the row.
+//   Merge  : the sorted words go back to shared memory, the places of the run heads are packed, and
+//            one lane per run sums it in slot order.
+// Stencil 41 x 37 x 53 (f32, 674 products a row): count 1714 -> 508 us, numeric 1905 -> 863 us against a CTA per
+// row; 59-product rows of the outer form (2e5 of them): 259 -> 125 us (hash set) and 439 -> 146 us.
+// ---------------------------------------------------------------------------------------
+constexpr int IW_WARPS = 4;
+
+template <typename P>
+__device__ __forceinline__ void sort_pair(P& a, P& b) {
+    const P lo = min(a, b), hi = max(a, b);
+    a = lo;
+    b = hi;
+}
+
+// Ascending bitonic sort of 32 * E words, element index = lane * E + x.  Every merge starts with the
+// mirrored comparison (i against i ^ (k - 1)), so all comparisons point the same way.
+template <typename P, int E>
+__device__ __forceinline__ void warp_sort(P (&w)[E]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 2; k <= 32 * E; k <<= 1) {
+        if (k <= E) {
+#pragma unroll
+            for (int x = 0; x < E; ++x)
+                if (!(x & (k >> 1))) sort_pair(w[x], w[x ^ (k - 1)]);
+        } else {
+            const int mask = k / E - 1;
+            const bool low = (lane & (k / (2 * E))) == 0;
+#pragma unroll
+            for (int x = 0; x < (E + 1) / 2; ++x) {
+                const int y = E - 1 - x;
+                const P ox = __shfl_xor_sync(0xffffffffu, w[y], mask);
+                if (y != x) {
+                    const P oy = __shfl_xor_sync(0xffffffffu, w[x], mask);
+                    w[y] = low ? min(w[y], oy) : max(w[y], oy);
+                }
+                w[x] = low ? min(w[x], ox) : max(w[x], ox);
+            }
+        }
+#pragma unroll
+        for (int j = k >> 2; j > 0; j >>= 1) {
+            if (j >= E) {
+                const bool low = (lane & (j / E)) == 0;
+#pragma unroll
+                for (int x = 0; x < E; ++x) {
+                    const P other = __shfl_xor_sync(0xffffffffu, w[x], j / E);
+                    w[x] = low ? min(w[x], other) : max(w[x], other);
+                }
+            } else {
+#pragma unroll
+                for (int x = 0; x < E; ++x)
+                    if (!(x & j)) sort_pair(w[x], w[x + j]);
+            }
+        }
+    }
+}
+
+// one word of padding per 32 keeps both the strided and the per-lane consecutive accesses conflict-free
+__device__ __forceinline__ int padded(int i) { return i + (i >> 5); }
+
+// Sorts the row's packed words and counts its distinct columns; numeric: leaves the sorted words in `packed`
+// and the places of the run heads in `heads`.
+template <typename PK, typename P, int E, bool NUMERIC>
+__device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int total) {
+    const int lane = threadIdx.x & 31;
+    P w[E];
+#pragma unroll
+    for (int x = 0; x < E; ++x) {
+        const int i = x * 32 + lane;
+        w[x] = i < total ? packed[padded(i)] : PK::sentinel();
+    }
+    warp_sort<P, E>(w);
+    const P before = __shfl_up_sync(0xffffffffu, w[E - 1], 1);
+    unsigned head = 0;
+#pragma unroll
+    for (int x = 0; x < E; ++x) {
+        const bool first = x == 0 ? (lane == 0 || PK::key(w[x]) != PK::key(before)) : PK::key(w[x]) != PK::key(w[x > 0 ? x - 1 : 0]);
+        if (w[x] != PK::sentinel() && first) head |= 1u << x;
+    }
+    const int mine = __popc(head);
+    const int incl = warp_incl_scan(mine);
+    const int n = __shfl_sync(0xffffffffu, incl, 31);
+    if (NUMERIC) {
+        __syncwarp();
+        int at = incl - mine;
+#pragma unroll
+        for (int x = 0; x < E; ++x) {
+            packed[padded(lane * E + x)] = w[x];
+            if ((head >> x) & 1u) heads[at++] = (unsigned short)(lane * E + x);
+        }
+        __syncwarp();
+    }
+    return n;
+}
+
+template <typename T, typename P, int CAP, bool NUMERIC>
+__global__ void __launch_bounds__(IW_WARPS * 32) ism_warp_kernel(const int* __restrict__ perm, DevCtl* __restrict__ ctl, int cls, int counter_slot,
+                                                                 Csr A, Csr B, const i64* __restrict__ ub, int* __restrict__ cnt,
+                                                                 const i64* __restrict__ rowptr, int* __restrict__ Ccrd, T* __restrict__ Cval) {
+    typedef Pack<P, CAP> PK;
+    constexpr int SLOTS = CAP + CAP / 32;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T* const vals = reinterpret_cast<T*>(smem_raw) + warp * (NUMERIC ? CAP : 0);
+    P* const packed = reinterpret_cast<P*>(smem_raw + (NUMERIC ? sizeof(T) * CAP * IW_WARPS : 0)) + warp * SLOTS;
+    unsigned short* const heads = reinterpret_cast<unsigned short*>(smem_raw + ((NUMERIC ? sizeof(T) * CAP : 0) + sizeof(P) * SLOTS) * IW_WARPS) + warp * CAP;
+    if (ctl->status != 0) return;
+    int off, n;
+    class_range(ctl, cls, off, n);
+    const T* __restrict__ Aval = (const T*)A.val;
+    const T* __restrict__ Bval = (const T*)B.val;
+    for (;;) {
+        int r = 0;
+        if (lane == 0) r = atomicAdd(&ctl->work_counter[counter_slot], 1);
+        r = __shfl_sync(0xffffffffu, r, 0);
+        if (r >= n) break;
+        const int row = __ldg(perm + off + r);
+        const i64 products = __ldg(ub + row);
+        if (products > CAP) continue;                            // the CTA kernel's rows
+        const i64 ps = __ldg(A.pos + row), pe = __ldg(A.pos + row + 1);
+        const int gs = pick_group_size(products, pe - ps, 1);
+        const int g = lane / gs, gl = lane % gs, ng = 32 / gs;
+
+        // ---- Insert
+        int total = 0;
+        for (i64 p0 = ps; p0 < pe; p0 += 32) {
+            int len = 0;
+            i64 qs = 0;
+            T a = 0;
+            if (p0 + lane < pe) {
+                const int k = __ldg(A.crd + p0 + lane);
+                if (NUMERIC) a = __ldg(Aval + p0 + lane);
+                if ((unsigned)k < (unsigned)B.nrows) {
+                    qs = __ldg(B.pos + k);
+                    len = (int)(__ldg(B.pos + k + 1) - qs);
+                }
+            }
+            const int incl = warp_incl_scan(len);
+            const int base = total + incl - len;
+            const int nE = (int)min((i64)32, pe - p0);
+            for (int i = 0; i < nE; i += 2 * ng) {
+                // two entries per group, the first element of both loaded before either is stored
+                const int e0 = i + g, e1 = min(i + ng + g, 31);
+                const i64 q0 = __shfl_sync(0xffffffffu, qs, e0), q1 = __shfl_sync(0xffffffffu, qs, e1);
+                const int l0 = __shfl_sync(0xffffffffu, len, e0), b0 = __shfl_sync(0xffffffffu, base, e0);
+                const int l1r = __shfl_sync(0xffffffffu, len, e1), b1 = __shfl_sync(0xffffffffu, base, e1);
+                const int l1 = i + ng + g < 32 ? l1r : 0;
+                T a0 = 0, a1 = 0;
+                if (NUMERIC) { a0 = __shfl_sync(0xffffffffu, a, e0); a1 = __shfl_sync(0xffffffffu, a, e1); }
+                int c0 = 0, c1 = 0;
+                T v0 = 0, v1 = 0;
+                if (gl < l0) { c0 = __ldg(B.crd + q0 + gl); if (NUMERIC) v0 = __ldg(Bval + q0 + gl); }
+                if (gl < l1) { c1 = __ldg(B.crd + q1 + gl); if (NUMERIC) v1 = __ldg(Bval + q1 + gl); }
+                auto put = [&](int slot, int col, T v) {
+                    if (slot < CAP) {                            // always so for a correctly classed row
+                        packed[padded(slot)] = PK::make(col, slot);
+                        if (NUMERIC) vals[slot] = v;
+                    }
+                };
+                if (gl < l0) put(b0 + gl, c0, mul_rn(a0, v0));
+                for (int t = gl + gs; t < l0; t += gs) put(b0 + t, __ldg(B.crd + q0 + t), NUMERIC ? mul_rn(a0, __ldg(Bval + q0 + t)) : (T)0);
+                if (gl < l1) put(b1 + gl, c1, mul_rn(a1, v1));
+                for (int t = gl + gs; t < l1; t += gs) put(b1 + t, __ldg(B.crd + q1 + t), NUMERIC ? mul_rn(a1, __ldg(Bval + q1 + t)) : (T)0);
+            }
+            total += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        total = min(total, CAP);
+        __syncwarp();
+
+        // ---- Sort
+        int distinct;
+        if (total <= 64) distinct = sort_row<PK, P, 2, NUMERIC>(packed, heads, total);
+        else if (total <= 128) distinct = sort_row<PK, P, 4, NUMERIC>(packed, heads, total);
+        else if (CAP <= 256 || total <= 256) distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total);
+        else if (total <= 512) distinct = sort_row<PK, P, (CAP > 256 ? 16 : 8), NUMERIC>(packed, heads, total);
+        else distinct = sort_row<PK, P, (CAP > 256 ? 32 : 8), NUMERIC>(packed, heads, total);
+
+        // ---- Merge
+        if (!NUMERIC) {
+            if (lane == 0) cnt[row] = distinct;
+        } else {
+            const i64 out0 = __ldg(rowptr + row);
+            for (int h = lane; h < distinct; h += 32) {
+                const int x0 = heads[h], x1 = h + 1 < distinct ? (int)heads[h + 1] : total;
+                const P w = packed[padded(x0)];
+                T sum = vals[PK::slot(w)];
+                for (int x = x0 + 1; x < x1; ++x) sum = add_rn(sum, vals[PK::slot(packed[padded(x)])]);
+                Ccrd[out0 + h] = (int)PK::key(w);
+                Cval[out0 + h] = sum;
+            }
+        }
+        __syncwarp();
+    }
+}
+
 template <typename T, typename P, int CAP, int THREADS>
 static size_t smem_bytes(bool numeric) {
     return (((numeric ? sizeof(T) * CAP : 0) + sizeof(P) * CAP + 7) & ~(size_t)7) + sizeof(i64) * THREADS + sizeof(T) * THREADS +
@@ -154,7 +359,7 @@ template <typename T, typename P, int CAP, int THREADS, bool NUMERIC>
 static cudaError_t launch_k(const LaunchCtx& c, int cls, int n_host, const Csr& A, const Csr& B,
                             const i64* rowptr, int* Ccrd, void* Cval) {
     const size_t smem = smem_bytes<T, P, CAP, THREADS>(NUMERIC);
-    const int slot = cls + (NUMERIC ? NUM_SLOT : 0);
+    const int slot = NUMERIC ? ISM_CTA_NUM_SLOT : ISM_CTA_SLOT;
     cudaError_t e;
     int per_sm = 0;
     auto k = ism_smem_kernel<T, P, CAP, THREADS, NUMERIC>;
@@ -162,34 +367,60 @@ static cudaError_t launch_k(const LaunchCtx& c, int cls, int n_host, const Csr& 
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, THREADS, smem)) != cudaSuccess) return e;
     i64 grid = (i64)c.sm_count * (per_sm > 0 ? per_sm : 1);
     if (n_host >= 0 && n_host < grid) grid = n_host > 0 ? n_host : 1;
-    k<<<(int)grid, THREADS, smem, c.stream>>>(c.tab.perm, c.ctl, cls, slot, A, B, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
+    k<<<(int)grid, THREADS, smem, c.stream>>>(c.tab.perm, c.ctl, cls, slot, (i64)ISM_WARP_MAX, A, B, c.tab.ub, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
     ++c.launches;
     return cudaGetLastError();
 }
 
-template <typename T, int CAP, int THREADS>
-static cudaError_t launch_cap(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B,
-                              const i64* rowptr, int* Ccrd, void* Cval) {
-    // 32-bit packed words when (column, slot) fits below the all-ones sentinel
-    const bool narrow = (i64)B.ncols < (1ll << (32 - Log2<CAP>::value));
-    if (narrow)
-        return numeric ? launch_k<T, unsigned, CAP, THREADS, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
-                       : launch_k<T, unsigned, CAP, THREADS, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
-    return numeric ? launch_k<T, u64, CAP, THREADS, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
-                   : launch_k<T, u64, CAP, THREADS, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
+template <typename T, typename P, int CAP, bool NUMERIC>
+static cudaError_t launch_warp_k(const LaunchCtx& c, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
+    const size_t smem = (size_t)IW_WARPS * ((NUMERIC ? (sizeof(T) + sizeof(short)) * CAP : 0) + sizeof(P) * (CAP + CAP / 32));
+    cudaError_t e;
+    int per_sm = 0;
+    auto k = ism_warp_kernel<T, P, CAP, NUMERIC>;
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, IW_WARPS * 32, smem)) != cudaSuccess) return e;
+    i64 grid = (i64)c.sm_count * (per_sm > 0 ? per_sm : 1);
+    const i64 want = n_host >= 0 ? ((i64)n_host + IW_WARPS - 1) / IW_WARPS : grid;
+    if (want < grid) grid = want > 0 ? want : 1;
+    k<<<(int)grid, IW_WARPS * 32, smem, c.stream>>>(c.tab.perm, c.ctl, cls, cls + (NUMERIC ? NUM_SLOT : 0), A, B, c.tab.ub, c.tab.cnt, rowptr, Ccrd,
+                                                    (T*)Cval);
+    ++c.launches;
+    return cudaGetLastError();
+}
+
+// Packed words are 32 bits wide when (column, slot) fits below the all-ones sentinel.
+template <int CAP>
+static bool narrow(const Csr& B) { return (i64)B.ncols < (1ll << (32 - Log2<CAP>::value)); }
+
+template <typename T, int CAP>
+static cudaError_t launch_warp(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd,
+                               void* Cval) {
+    if (narrow<CAP>(B))
+        return numeric ? launch_warp_k<T, unsigned, CAP, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
+                       : launch_warp_k<T, unsigned, CAP, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
+    return numeric ? launch_warp_k<T, u64, CAP, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
+                   : launch_warp_k<T, u64, CAP, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
 }
 
 template <typename T>
 static cudaError_t launch_t(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B,
                             const i64* rowptr, int* Ccrd, void* Cval) {
-    // the full class is launched for the largest row it actually holds when that is known: a
-    // smaller accumulation array means more CTAs per SM and cheaper barriers
-    int cap = (cls == CLS_ISM_SMEM_S) ? c.prm.smem_small_cap : c.prm.smem_cap;
-    if (cls == CLS_ISM_SMEM && c.max_ub_smem > 0 && c.max_ub_smem < cap) cap = (int)c.max_ub_smem;
-    if (cap <= 64) return launch_cap<T, 64, 64>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
-    if (cap <= 256) return launch_cap<T, 256, 64>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
-    if (cap <= 1024) return launch_cap<T, 1024, 128>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
-    return launch_cap<T, 4096, 256>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
+    // the small class, and the full one when its largest row is that small: fewer registers and less
+    // shared memory per warp
+    i64 most = (cls == CLS_ISM_SMEM_S) ? c.prm.smem_small_cap : c.prm.smem_cap;
+    if (cls == CLS_ISM_SMEM && c.max_ub_smem > 0 && c.max_ub_smem < most) most = c.max_ub_smem;
+    if (most <= 256) return launch_warp<T, 256>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
+    cudaError_t e = launch_warp<T, ISM_WARP_MAX>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
+    if (e != cudaSuccess || most <= ISM_WARP_MAX) return e;
+    // rows of 1025 .. 4096 products: a CTA each (a counter of their own: the two kernels share the class);
+    // under `auto` they are counted through a hash set of their columns, which needs no order
+    if (!numeric && c.prm.policy == 2) return launch_hash(c, false, CLS_ISM_SMEM, n_host, A, B, rowptr, Ccrd, Cval);
+    if (narrow<4096>(B))
+        return numeric ? launch_k<T, unsigned, 4096, 256, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
+                       : launch_k<T, unsigned, 4096, 256, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
+    return numeric ? launch_k<T, u64, 4096, 256, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
+                   : launch_k<T, u64, 4096, 256, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
 }
 
 cudaError_t launch_ism_smem(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B,

@@ -121,6 +121,19 @@ def test_capacity_boundaries(ctx, oracle_mod, policy):
     check_spgemm(ctx, oracle_mod, A, B, policy, **SMALL_ROUTES)
 
 
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("ncols", [2000, (1 << 22) - 1, 1 << 22, 1 << 25])
+def test_ism_warp_rows_at_every_register_width(ctx, oracle_mod, ncols, dtype):
+    """Rows one product below, at and above each size of the register sort, with 32- and 64-bit packed
+    words; the sums are in loop order, so double values equal the oracle's plain sum bit for bit."""
+    targets = [33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 2000]
+    A, B = _rows_with_products(targets, ncols, 13, dtype)
+    for opts in ({}, dict(ism_cta_cap=256), dict(ism_cta_cap=1024)):
+        stats = check_spgemm(ctx, oracle_mod, A, B, "ism", exact_values=dtype == np.float64 and not opts, **opts)
+        assert stats["rows_per_class"][2] + stats["rows_per_class"][3] > 0
+    check_spgemm(ctx, oracle_mod, A, B, "auto")
+
+
 @pytest.mark.parametrize("policy", POLICIES)
 def test_edge_cases(ctx, oracle_mod, policy):
     # all-empty A, empty B rows, one huge row among empty ones
