@@ -157,13 +157,13 @@ typedef struct {
 
 /* Kernel groups timed by spws_set_profiling (index into the array spws_get_timings fills). */
 enum {
-    SPWS_T_SYM_BOUNDS = 0,    /* per-row upper bound, span and class; word lists of long B rows    */
+    SPWS_T_SYM_BOUNDS = 0,    /* per-row upper bound, span and class                               */
     SPWS_T_SYM_BIN = 1,       /* binning + dense work units                                        */
     SPWS_T_SYM_ISM_REG = 2,
     SPWS_T_SYM_ISM_SMEM_S = 3,
     SPWS_T_SYM_ISM_SMEM = 4,
     SPWS_T_SYM_DENSE_WARP = 5,
-    SPWS_T_SYM_DENSE_CTA = 6,
+    SPWS_T_SYM_DENSE_CTA = 6, /* with the word lists of long B rows                                */
     SPWS_T_SYM_ISM_GLOBAL = 7,
     SPWS_T_SYM_HASH = 8,
     SPWS_T_SYM_SCAN = 9,      /* exclusive scan, numeric routing of dense rows (+ CSF level

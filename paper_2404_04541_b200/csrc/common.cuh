@@ -70,12 +70,16 @@ struct DevCtl {
     i64 kept[2];            // TTM: surviving slices (level 0) and fibres (level 1)
     u64 bm_words_used;      // words handed out of the bitmap arena
     int status;
-    int n_units;            // numeric dense CTA units (row, rank range)
+    int n_units;            // numeric dense CTA units (row, share of its entries)
+    int hub_units;          // units of the heaviest rows, which come first ...
+    int hub_cursor, other_cursor;   // ... and units handed out so far
     int n_warp_rows;        // numeric dense warp rows
     int max_span_words;     // widest bitmap among the dense rows
     int max_warp_cnt;       // most outputs of a row the warp numeric kernel takes
     int n_long;             // B rows with at least BW_MIN_LEN entries (candidates for a word list)
-    int n_long_a;           // rows of A with more than LONG_A_ROW entries, left to the bounds kernel for long rows
+    int bin_done, rows_done, slices_done;       // blocks that have finished
+    int rows_ticket, slices_ticket;             // tiles handed out
+    int* host_status;       // status word in the plan's pinned block (null before the binning is done)
     int class_count[NCLASS];
     int class_cursor[NCLASS];
     int work_counter[N_WORK_COUNTERS];   // dynamic work distribution; cleared before each pass
@@ -162,7 +166,89 @@ __host__ __device__ inline int dense_units_of_row(i64 ub, i64 unit_products) {
     return (int)(n < 1 ? 1 : n);
 }
 
-__device__ __forceinline__ void raise_status(DevCtl* ctl, int s) { atomicCAS(&ctl->status, 0, s); }
+// The first error wins; it is also written to the plan's pinned block once that is known.
+__device__ __forceinline__ void raise_status(DevCtl* ctl, int s) {
+    if (atomicCAS(&ctl->status, 0, s) == 0 && ctl->host_status) *(volatile int*)ctl->host_status = s;
+}
+
+// Copies the control block to pinned host memory (a whole block of threads, after the counters are final):
+// posted writes, complete when the kernel is.
+__device__ __forceinline__ void publish_ctl(DevCtl* ctl, DevCtl* host) {
+    for (int w = threadIdx.x; w < (int)(sizeof(DevCtl) / 4); w += blockDim.x)
+        reinterpret_cast<volatile int*>(host)[w] = reinterpret_cast<volatile const int*>(ctl)[w];
+}
+
+// True in every thread of the last of `blocks` blocks to come here; all earlier blocks' writes are visible to it.
+__device__ __forceinline__ bool last_block(int* done, int blocks) {
+    __shared__ int s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(done, 1) == blocks - 1;
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last != 0;
+}
+
+// ---- running sums handed from tile to tile ---------------------------------------------------
+// A tile of a single-pass scan publishes one 64-bit word: a tag above 56 bits of count.  The tag of a
+// pass is 2 * pass + 1 while the word holds the tile's own count and 2 * pass + 2 once it holds the
+// count of all tiles up to it, so one clearing serves all the passes of a sort.  Tiles are numbered
+// by a ticket taken when a block starts, hence every tile that is waited for is running or done; a
+// wait that does not end after LOOK_LIMIT polls raises the status word and goes on with what it has
+// (too small a count, so that every index stays inside the arrays).
+constexpr int LOOK_SHIFT = 56;
+constexpr u64 LOOK_MASK = (1ull << LOOK_SHIFT) - 1;
+constexpr int LOOK_LIMIT = 1 << 22;
+
+__device__ __forceinline__ void look_publish(u64* word, int tag, i64 count) {
+    *(volatile u64*)word = ((u64)tag << LOOK_SHIFT) | (u64)count;
+}
+
+// Sum of the counts of the tiles before `tile` (one word per tile, `stride` words apart): a single
+// thread walks back until it meets a running sum.
+__device__ __forceinline__ i64 look_back(const u64* words, int stride, int tile, int pass, DevCtl* ctl) {
+    i64 sum = 0;
+    int polls = 0;
+    for (int t = tile - 1; t >= 0;) {
+        const u64 w = *(const volatile u64*)(words + (i64)t * stride);
+        const int tag = (int)(w >> LOOK_SHIFT);
+        if (tag <= 2 * pass) {
+            if (++polls >= LOOK_LIMIT) { raise_status(ctl, DEV_INTERNAL_OVERFLOW); break; }
+            continue;
+        }
+        sum += (i64)(w & LOOK_MASK);
+        if (tag == 2 * pass + 2) break;
+        --t;
+    }
+    return sum;
+}
+
+// The same for a whole warp: 32 predecessors per step.  Every lane returns the sum.
+__device__ __forceinline__ i64 look_back_warp(const u64* words, int tile, int pass, DevCtl* ctl) {
+    const int lane = threadIdx.x & 31;
+    i64 sum = 0;
+    int polls = 0;
+    for (int t0 = tile - 1; t0 >= 0; t0 -= 32) {
+        const int t = t0 - lane;
+        u64 w = (u64)(2 * pass + 2) << LOOK_SHIFT;              // before the first tile: a running sum of nothing
+        for (;;) {
+            if (t >= 0) w = *(const volatile u64*)(words + t);
+            if (__all_sync(0xffffffffu, (int)(w >> LOOK_SHIFT) > 2 * pass)) break;
+            if (++polls >= LOOK_LIMIT) {
+                if (lane == 0) raise_status(ctl, DEV_INTERNAL_OVERFLOW);
+                return sum;
+            }
+        }
+        const unsigned ends = __ballot_sync(0xffffffffu, (int)(w >> LOOK_SHIFT) == 2 * pass + 2);
+        const int last = ends ? __ffs(ends) - 1 : 31;           // the nearest running sum ends the walk
+        i64 v = lane <= last ? (i64)(w & LOOK_MASK) : 0;
+        for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+        sum += v;
+        if (ends) break;
+    }
+    return sum;
+}
+
 
 // Rows of class `cls` are perm[off, off + n).
 __device__ __forceinline__ void class_range(const DevCtl* ctl, int cls, int& off, int& n) {
@@ -247,6 +333,9 @@ struct LaunchCtx {
     char* rest;              // scratch after the fixed tables: bitmap arena, then the ISM-global arena
     size_t rest_bytes;
     int global_cap;          // accumulation-array capacity of CLS_ISM_GLOBAL
+    DevCtl* host_ctl;        // the plan's pinned copy of the control block
+    u64* look;               // one word per tile of the kernels that hand running sums on ...
+    int n_look;              // ... cleared by the binning kernel
     i64 max_ub_smem;         // largest product count of a CLS_ISM_SMEM row when known (0: unknown)
     uint2* bw;               // word lists of long B rows, indexed like B's entries (null: not built)
     int* bw_long;            // the long B rows, in arrival order
@@ -257,16 +346,18 @@ struct LaunchCtx {
 
 // setup.cu
 cudaError_t launch_validate(const LaunchCtx& c, const Csr& A, const Csr& B, i64 nnzA, i64 nnzB);
-cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i64 nnzA);
+// clear_ctl: the control block is cleared by the first kernel
+cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i64 nnzA, bool clear_ctl);
 cudaError_t launch_bw_build(const LaunchCtx& c, const Csr& B);
 cudaError_t launch_bin_rows(const LaunchCtx& c, int m);
-cudaError_t launch_dense_rebin(const LaunchCtx& c, int m, const i64* rowptr);
-cudaError_t launch_class_nnz(const LaunchCtx& c, int m);
-// as_flags: scan (cnt[i] > 0) instead of cnt[i]
-cudaError_t launch_scan_counts(const LaunchCtx& c, const int* cnt, int n, i64* out, i64* block_sums, i64* total_out, bool as_flags = false);
-cudaError_t launch_ttm_scan_compact(const LaunchCtx& c, int n_i, int n_ij, const i64* Apos1, const int* Acrd0, const int* Acrd1,
-                                    i64* rowptr_raw, i64* fpos, int* sflags, i64* spos, i64* block_sums, i64* nnz_out,
-                                    i64* Cpos0, int* Ccrd0, i64* Cpos1, int* Ccrd1, i64* Cpos2);
+// row pointer, numeric routing of the dense rows, outputs per class
+cudaError_t launch_finish_rows(const LaunchCtx& c, int m, bool any_dense, i64* rowptr);
+// the same for the fibres of a 3-tensor, with C's upper levels; sfp: n_i + 1 words of scratch
+cudaError_t launch_finish_fibres(const LaunchCtx& c, int n_i, int n_ij, bool any_dense, const i64* Apos1, const int* Acrd0, const int* Acrd1,
+                                 i64* rowptr_raw, i64* sfp, i64* Cpos0, int* Ccrd0, i64* Cpos1, int* Ccrd1, i64* Cpos2);
+size_t look_words(i64 rows, i64 slices);
+// exclusive scan of n counts into n + 1 positions
+cudaError_t launch_scan_counts(const LaunchCtx& c, const int* cnt, int n, i64* out, i64* block_sums, i64* total_out);
 // class kernels: n_host < 0 means "size the grid for any count"
 cudaError_t launch_ism_reg(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B,
                            const i64* rowptr, int* Ccrd, void* Cval);

@@ -82,7 +82,10 @@ __device__ __forceinline__ int classify_row(i64 ub, i64 entries, int jmin, int j
 // First column, last column and length of every B row, in one 16-byte record: when A has several
 // times more entries than B has rows, the bounds kernel reads the record of the row an entry picks
 // (one load, neighbouring rows share sectors) instead of two offsets and two coordinates.
-__global__ void __launch_bounds__(256) brow_summary_kernel(Csr B, int4* __restrict__ brow) {
+// It is the first kernel of a pass and clears the control block on the way (ctl non-null).
+__global__ void __launch_bounds__(256) brow_summary_kernel(Csr B, int4* __restrict__ brow, DevCtl* ctl) {
+    if (ctl && blockIdx.x == 0)
+        for (int w = threadIdx.x; w < (int)(sizeof(DevCtl) / 4); w += 256) reinterpret_cast<int*>(ctl)[w] = 0;
     for (i64 k = (i64)blockIdx.x * blockDim.x + threadIdx.x; k < B.nrows; k += (i64)gridDim.x * blockDim.x) {
         const i64 qs = B.pos[k], qe = B.pos[k + 1];
         int4 s = make_int4(0x7fffffff, -1, 0, 0);
@@ -92,6 +95,82 @@ __global__ void __launch_bounds__(256) brow_summary_kernel(Csr B, int4* __restri
             s.z = (int)min(qe - qs, (i64)0x7fffffff);
         }
         brow[k] = s;
+    }
+}
+
+constexpr int LONG_LIST = 32;
+
+// Bounds and class of one long row by a whole block: 256 lanes across the entries, four entries per lane
+// and step.
+template <bool SUMMARY>
+__device__ __forceinline__ void long_row_bounds(int row, const Csr& A, const Csr& B, const RowTables& tab, const ClassParams& prm, DevCtl* ctl,
+                                                const int4* __restrict__ brow) {
+    __shared__ i64 s_u[8];
+    __shared__ int s_lo[8], s_hi[8], s_bad[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const i64 ps = A.pos[row], pe = A.pos[row + 1];
+    i64 u = 0;
+    int lo = 0x7fffffff, hi = -1, bad = 0;
+    for (i64 p0 = ps + tid; p0 < pe; p0 += 4 * 256) {
+        int k[4];
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const i64 p = p0 + (i64)x * 256;
+            k[x] = p < pe ? __ldg(A.crd + p) : -1;
+            if (p < pe && (unsigned)k[x] >= (unsigned)B.nrows) bad = 1;
+        }
+        if (SUMMARY) {
+            int4 s[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) s[x] = (unsigned)k[x] < (unsigned)B.nrows ? __ldg(brow + k[x]) : make_int4(0x7fffffff, -1, 0, 0);
+#pragma unroll
+            for (int x = 0; x < 4; ++x) { u += s[x].z; lo = min(lo, s[x].x); hi = max(hi, s[x].y); }
+        } else {
+            i64 qs[4], qe[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                qs[x] = qe[x] = 0;
+                if ((unsigned)k[x] < (unsigned)B.nrows) { qs[x] = __ldg(B.pos + k[x]); qe[x] = __ldg(B.pos + k[x] + 1); }
+            }
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                if (qe[x] > qs[x]) {
+                    u += qe[x] - qs[x];
+                    lo = min(lo, __ldg(B.crd + qs[x]));
+                    hi = max(hi, __ldg(B.crd + qe[x] - 1));
+                }
+        }
+    }
+    for (int d = 16; d > 0; d >>= 1) {
+        u += __shfl_xor_sync(0xffffffffu, u, d);
+        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, d));
+        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, d));
+        bad |= __shfl_xor_sync(0xffffffffu, bad, d);
+    }
+    __syncthreads();                                   // the previous row's totals have been read
+    if (lane == 0) { s_u[warp] = u; s_lo[warp] = lo; s_hi[warp] = hi; s_bad[warp] = bad; }
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < 8; ++w) { u += s_u[w]; lo = min(lo, s_lo[w]); hi = max(hi, s_hi[w]); bad |= s_bad[w]; }
+        if (bad) raise_status(ctl, DEV_NONCANONICAL);
+        if (lo < 0 || hi >= B.ncols) { raise_status(ctl, DEV_NONCANONICAL); u = 0; }
+        if (u > 0) lo &= ~31;
+        const int cls = classify_row(u, pe - ps, lo, hi, prm, ctl);
+        tab.ub[row] = u;
+        tab.jmin[row] = lo;
+        tab.jmax[row] = hi;
+        tab.cnt[row] = cls == CLS_COPY8 ? (int)u : 0;
+        tab.cls[row] = (unsigned char)cls;
+        atomicAdd(&ctl->class_count[cls], 1);
+        if (u) {
+            atomicAdd((u64*)&ctl->class_products[cls], (u64)u);
+            atomicAdd((u64*)&ctl->products, (u64)u);
+            atomicMax(&ctl->max_ub, u);
+            if (cls == CLS_ISM_GLOBAL) atomicMax(&ctl->max_ub_global, u);
+            if (cls == CLS_ISM_SMEM) atomicMax(&ctl->max_ub_smem, u);
+            if (cls == CLS_DENSE_HUB || cls == CLS_DENSE_CTA || cls == CLS_DENSE_WARP)
+                atomicMax(&ctl->max_span_words, (hi - lo) / 32 + 1);
+        }
     }
 }
 
@@ -106,16 +185,21 @@ __global__ void __launch_bounds__(256) row_bounds_kernel(Csr A, Csr B, RowTables
     __shared__ i64 s_cprod[8][NCLASS];
     __shared__ i64 s_products, s_max_ub, s_max_ub_global, s_max_ub_smem;
     __shared__ int s_max_span_words;
+    // rows of more than LONG_A_ROW entries, which the block's threads take together at the end: left to
+    // its lane group such a row is a serial chain that sets the kernel's time on power-law inputs
+    __shared__ int s_long[LONG_LIST], s_nlong;
     for (int x = threadIdx.x; x < 8 * NCLASS; x += blockDim.x) { (&s_hist[0][0])[x] = 0; (&s_cprod[0][0])[x] = 0; }
-    if (threadIdx.x == 0) { s_products = 0; s_max_ub = 0; s_max_ub_global = 0; s_max_ub_smem = 0; s_max_span_words = 0; }
+    if (threadIdx.x == 0) { s_products = 0; s_max_ub = 0; s_max_ub_global = 0; s_max_ub_smem = 0; s_max_span_words = 0; s_nlong = 0; }
     __syncthreads();
     int* const w_hist = s_hist[threadIdx.x >> 5];
     i64* const w_cprod = s_cprod[threadIdx.x >> 5];
     const int gl = threadIdx.x % G;
     const unsigned lane = threadIdx.x & 31;
     const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane - gl));
-    const i64 group = ((i64)blockIdx.x * blockDim.x + threadIdx.x) / G;
+    // a warp per row: neighbouring rows go to different blocks (the heaviest rows of a graph are often
+    // neighbours); narrower groups take neighbouring rows for the sake of the row offsets they share
     const i64 ngroups = ((i64)gridDim.x * blockDim.x) / G;
+    const i64 group = G == 32 ? (i64)(threadIdx.x >> 5) * gridDim.x + blockIdx.x : ((i64)blockIdx.x * blockDim.x + threadIdx.x) / G;
     i64 my_products = 0, my_max = 0;
     // rows and products of the class of this group's last rows: neighbouring rows mostly share a
     // class, so the shared-memory histogram is touched only when the class changes
@@ -124,11 +208,13 @@ __global__ void __launch_bounds__(256) row_bounds_kernel(Csr A, Csr B, RowTables
     for (i64 row = group; row < A.nrows; row += ngroups) {
         const i64 ps = A.pos[row], pe = A.pos[row + 1];
         if (pe - ps > LONG_A_ROW) {
-            // a very long row would be this group's serial chain and set the kernel's time on power-law
-            // inputs: it is listed for the kernel that gives such rows a CTA each (the list borrows the
-            // table of warp rows, which is not in use before the numeric routing)
-            if (gl == 0) tab.warp_rows[atomicAdd(&ctl->n_long_a, 1)] = (int)row;
-            continue;
+            int at = 0;
+            if (gl == 0) at = atomicAdd(&s_nlong, 1);
+            at = __shfl_sync(gmask, at, 0, G);
+            if (at < LONG_LIST) {
+                if (gl == 0) s_long[at] = (int)row;
+                continue;
+            }
         }
         i64 u = 0;
         int lo = 0x7fffffff, hi = -1;
@@ -233,6 +319,8 @@ __global__ void __launch_bounds__(256) row_bounds_kernel(Csr A, Csr B, RowTables
         atomicAdd(&w_hist[run_cls], run_rows);
         if (run_products) atomicAdd((u64*)&w_cprod[run_cls], (u64)run_products);
     }
+    __syncthreads();
+    for (int r = 0; r < min(s_nlong, LONG_LIST); ++r) long_row_bounds<SUMMARY>(s_long[r], A, B, tab, prm, ctl, brow);
     // the totals: reduced over the warp first (lanes other than a group's first hold zeros)
     for (int d = 16; d > 0; d >>= 1) {
         my_products += __shfl_xor_sync(0xffffffffu, my_products, d);
@@ -261,86 +349,8 @@ __global__ void __launch_bounds__(256) row_bounds_kernel(Csr A, Csr B, RowTables
     }
 }
 
-// Bounds and class of the listed long rows, a CTA per row: 256 lanes across the entries, four
-// entries per lane and step.
-template <bool SUMMARY>
-__global__ void __launch_bounds__(256) row_bounds_long_kernel(Csr A, Csr B, RowTables tab, ClassParams prm, DevCtl* ctl,
-                                                              const int4* __restrict__ brow) {
-    __shared__ i64 s_u[8];
-    __shared__ int s_lo[8], s_hi[8], s_bad[8];
-    const int n = min(ctl->n_long_a, A.nrows);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int r = blockIdx.x; r < n; r += gridDim.x) {
-        const int row = tab.warp_rows[r];
-        const i64 ps = A.pos[row], pe = A.pos[row + 1];
-        i64 u = 0;
-        int lo = 0x7fffffff, hi = -1, bad = 0;
-        for (i64 p0 = ps + tid; p0 < pe; p0 += 4 * 256) {
-            int k[4];
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const i64 p = p0 + (i64)x * 256;
-                k[x] = p < pe ? __ldg(A.crd + p) : -1;
-                if (p < pe && (unsigned)k[x] >= (unsigned)B.nrows) bad = 1;
-            }
-            if (SUMMARY) {
-                int4 s[4];
-#pragma unroll
-                for (int x = 0; x < 4; ++x) s[x] = (unsigned)k[x] < (unsigned)B.nrows ? __ldg(brow + k[x]) : make_int4(0x7fffffff, -1, 0, 0);
-#pragma unroll
-                for (int x = 0; x < 4; ++x) { u += s[x].z; lo = min(lo, s[x].x); hi = max(hi, s[x].y); }
-            } else {
-                i64 qs[4], qe[4];
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    qs[x] = qe[x] = 0;
-                    if ((unsigned)k[x] < (unsigned)B.nrows) { qs[x] = __ldg(B.pos + k[x]); qe[x] = __ldg(B.pos + k[x] + 1); }
-                }
-#pragma unroll
-                for (int x = 0; x < 4; ++x)
-                    if (qe[x] > qs[x]) {
-                        u += qe[x] - qs[x];
-                        lo = min(lo, __ldg(B.crd + qs[x]));
-                        hi = max(hi, __ldg(B.crd + qe[x] - 1));
-                    }
-            }
-        }
-        for (int d = 16; d > 0; d >>= 1) {
-            u += __shfl_xor_sync(0xffffffffu, u, d);
-            lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, d));
-            hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, d));
-            bad |= __shfl_xor_sync(0xffffffffu, bad, d);
-        }
-        __syncthreads();                                   // the previous row's totals have been read
-        if (lane == 0) { s_u[warp] = u; s_lo[warp] = lo; s_hi[warp] = hi; s_bad[warp] = bad; }
-        __syncthreads();
-        if (tid == 0) {
-            for (int w = 1; w < 8; ++w) { u += s_u[w]; lo = min(lo, s_lo[w]); hi = max(hi, s_hi[w]); bad |= s_bad[w]; }
-            if (bad) raise_status(ctl, DEV_NONCANONICAL);
-            if (lo < 0 || hi >= B.ncols) { raise_status(ctl, DEV_NONCANONICAL); u = 0; }
-            if (u > 0) lo &= ~31;
-            const int cls = classify_row(u, pe - ps, lo, hi, prm, ctl);
-            tab.ub[row] = u;
-            tab.jmin[row] = lo;
-            tab.jmax[row] = hi;
-            tab.cnt[row] = cls == CLS_COPY8 ? (int)u : 0;
-            tab.cls[row] = (unsigned char)cls;
-            atomicAdd(&ctl->class_count[cls], 1);
-            if (u) {
-                atomicAdd((u64*)&ctl->class_products[cls], (u64)u);
-                atomicAdd((u64*)&ctl->products, (u64)u);
-                atomicMax(&ctl->max_ub, u);
-                if (cls == CLS_ISM_GLOBAL) atomicMax(&ctl->max_ub_global, u);
-                if (cls == CLS_ISM_SMEM) atomicMax(&ctl->max_ub_smem, u);
-                if (cls == CLS_DENSE_HUB || cls == CLS_DENSE_CTA || cls == CLS_DENSE_WARP)
-                    atomicMax(&ctl->max_span_words, (hi - lo) / 32 + 1);
-            }
-        }
-    }
-}
-
-cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i64 nnzA) {
-    if (A.nrows == 0) return cudaSuccess;
+cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i64 nnzA, bool clear_ctl) {
+    if (A.nrows == 0) return clear_ctl ? cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream) : cudaSuccess;
     const double avg = (double)nnzA / (double)A.nrows;
     const int threads = 256;
     auto grid_for = [&](int G) {
@@ -348,13 +358,14 @@ cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i6
         i64 cap = (i64)c.sm_count * 16;
         return (int)(want < cap ? want : cap);
     };
-    // (one and two lanes per row were measured on the fibre matrix of the 3-tensor workload, 1.06
-    // entries per row: slower than four)
     if (c.brow) {
         i64 want = ((i64)B.nrows + threads - 1) / threads;
         i64 cap = (i64)c.sm_count * 8;
-        brow_summary_kernel<<<(int)(want < cap ? want : cap), threads, 0, c.stream>>>(B, c.brow);
+        brow_summary_kernel<<<(int)(want < cap ? want : cap), threads, 0, c.stream>>>(B, c.brow, clear_ctl ? c.ctl : nullptr);
         ++c.launches;
+    } else if (clear_ctl) {
+        cudaError_t e = cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream);
+        if (e != cudaSuccess) return e;
     }
     auto launch = [&](auto kernel, int G) { kernel<<<grid_for(G), threads, 0, c.stream>>>(A, B, c.tab, c.prm, c.ctl, c.brow); };
     const bool sm = c.brow != nullptr;
@@ -364,15 +375,6 @@ cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i6
     else if (avg <= 12.0) sm ? launch(row_bounds_kernel<8, true>, 8) : launch(row_bounds_kernel<8, false>, 8);
     else sm ? launch(row_bounds_kernel<32, true>, 32) : launch(row_bounds_kernel<32, false>, 32);
     ++c.launches;
-    // rows the kernel above listed as too long for a lane group (none, unless A has more than
-    // LONG_A_ROW entries in all)
-    if (nnzA > LONG_A_ROW) {
-        const i64 most = nnzA / LONG_A_ROW;
-        const int grid = (int)(most < (i64)c.sm_count * 4 ? most : (i64)c.sm_count * 4);
-        if (sm) row_bounds_long_kernel<true><<<grid, 256, 0, c.stream>>>(A, B, c.tab, c.prm, c.ctl, c.brow);
-        else row_bounds_long_kernel<false><<<grid, 256, 0, c.stream>>>(A, B, c.tab, c.prm, c.ctl, c.brow);
-        ++c.launches;
-    }
     return cudaGetLastError();
 }
 
@@ -465,7 +467,11 @@ cudaError_t launch_bw_build(const LaunchCtx& c, const Csr& B) {
 // also reserve the slot of their occupancy bitmap in the arena.  Order inside a class follows
 // block arrival.
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) bin_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl) {
+// It also counts the units of the heaviest rows, clears the words of the kernels that hand running sums
+// from tile to tile, and its last block publishes the class sizes to the host.
+__global__ void __launch_bounds__(256) bin_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, DevCtl* host, u64* look, int n_look) {
+    for (int w = blockIdx.x * 256 + threadIdx.x; w < n_look; w += gridDim.x * 256) look[w] = 0;
+    const i64 unit_products = dense_unit_products(ctl->products);
     __shared__ int s_hist[NCLASS], s_base[NCLASS], s_off[NCLASS];
     __shared__ int ws[33];
     __shared__ u64 s_bm_base;
@@ -501,6 +507,7 @@ __global__ void __launch_bounds__(256) bin_rows_kernel(int m, RowTables tab, Cla
             {   // the row's slot: bitmap words, then the rank at the start of every 32-word chunk
                 const int nw = (tab.jmax[row] - tab.jmin[row]) / 32 + 1;
                 words[x] = (nw + (nw + 31) / 32 + 3) & ~3;      // 16-byte aligned slots
+                if (cls[x] == CLS_DENSE_HUB) atomicAdd(&ctl->hub_units, dense_units_of_row(tab.ub[row], unit_products));
             }
             my_words += words[x];
         }
@@ -526,133 +533,340 @@ __global__ void __launch_bounds__(256) bin_rows_kernel(int m, RowTables tab, Cla
         }
         __syncthreads();
     }
+    if (last_block(&ctl->bin_done, gridDim.x)) {
+        if (threadIdx.x == 0) ctl->host_status = &host->status;
+        __syncthreads();
+        publish_ctl(ctl, host);
+    }
 }
 
 cudaError_t launch_bin_rows(const LaunchCtx& c, int m) {
-    if (m == 0) return cudaSuccess;
     i64 want = ((i64)m + 1023) / 1024;
     i64 cap = (i64)c.sm_count * 8;
-    bin_rows_kernel<<<(int)(want < cap ? want : cap), 256, 0, c.stream>>>(m, c.tab, c.prm, c.ctl);
+    if (want < 1) want = 1;
+    bin_rows_kernel<<<(int)(want < cap ? want : cap), 256, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host_ctl, c.look, c.n_look);
     ++c.launches;
     return cudaGetLastError();
 }
 
-// Numeric routing of the dense rows, once their output counts are known: a row the warp kernel
-// counted and whose outputs fit a warp's accumulator stays with a warp; every other row becomes
-// one CTA unit, or several when it has many products: unit c of n takes the c-th n-th of the
-// row's A entries (all units of a row add into the same outputs).
-__global__ void __launch_bounds__(256) dense_rebin_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl) {
-    __shared__ int ws[33];
-    __shared__ int s_wbase, s_ubase, s_wmax;
-    __shared__ i64 s_wp, s_wn;
-    int off, n4, n5, n6, o5, o6;
-    class_range(ctl, CLS_DENSE_WARP, off, n4);
-    class_range(ctl, CLS_DENSE_HUB, o5, n5);
-    class_range(ctl, CLS_DENSE_CTA, o6, n6);
-    const int n = n4 + n5 + n6;                       // the three classes are adjacent in perm
-    const i64 unit_products = dense_unit_products(ctl->products);
-    for (i64 b0 = (i64)blockIdx.x * blockDim.x; b0 < n; b0 += (i64)gridDim.x * blockDim.x) {
-        const i64 r = b0 + threadIdx.x;
-        int row = -1, cnt = 0, to_warp = 0, nu = 0;
-        if (threadIdx.x == 0) { s_wp = 0; s_wn = 0; s_wmax = 0; }
-        if (r < n) {
-            row = tab.perm[off + r];
-            cnt = tab.cnt[row];
-            to_warp = tab.cls[row] == CLS_DENSE_WARP && cnt <= DENSE_WARP_ACC;
-            nu = to_warp ? 0 : dense_units_of_row(tab.ub[row], unit_products);
-        }
-        int wtot, utot;
-        const int wpos = block_excl_scan<256>(to_warp, ws, wtot);
-        const int upos = block_excl_scan<256>(nu, ws, utot);
-        if (threadIdx.x == 0) {
-            s_wbase = wtot ? atomicAdd(&ctl->n_warp_rows, wtot) : 0;
-            s_ubase = utot ? atomicAdd(&ctl->n_units, utot) : 0;
-        }
-        __syncthreads();
-        if (row >= 0) {
-            if (to_warp) {
-                tab.warp_rows[s_wbase + wpos] = row;
-                tab.row_unit0[row] = -1;
-            } else {
-                const int u0 = s_ubase + upos;
-                if (u0 + nu > prm.unit_cap) {
-                    raise_status(ctl, DEV_SCRATCH_TOO_SMALL);
-                    tab.row_unit0[row] = -1;
-                } else {
-                    tab.row_unit0[row] = u0;
-                    for (int t = 0; t < nu; ++t) tab.unit_row[u0 + t] = row;
-                }
-            }
-        }
-        {
-            // products, outputs and largest output count of the warp rows: one shared atomic per warp
-            i64 wp = (row >= 0 && to_warp) ? tab.ub[row] : 0;
-            i64 wn = (row >= 0 && to_warp) ? cnt : 0;
-            int wm = (row >= 0 && to_warp) ? cnt : 0;
-            for (int d = 16; d > 0; d >>= 1) {
-                wp += __shfl_xor_sync(0xffffffffu, wp, d);
-                wn += __shfl_xor_sync(0xffffffffu, wn, d);
-                wm = max(wm, __shfl_xor_sync(0xffffffffu, wm, d));
-            }
-            if ((threadIdx.x & 31) == 0 && wp) {
-                atomicAdd((u64*)&s_wp, (u64)wp);
-                atomicAdd((u64*)&s_wn, (u64)wn);
-                atomicMax(&s_wmax, wm);
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0 && s_wp) {
-            atomicAdd((u64*)&ctl->dense_warp_products, (u64)s_wp);
-            atomicAdd((u64*)&ctl->dense_warp_nnz, (u64)s_wn);
-            atomicMax(&ctl->max_warp_cnt, s_wmax);
-        }
-        __syncthreads();
-    }
-}
+// ---------------------------------------------------------------------------------------
+// Once the output counts are known, in ONE pass over the rows: the row pointer, the numeric routing of
+// the dense rows, the outputs per class, and (TTM) C's fibre level.  A tile of FR_TILE rows per block;
+// warp w owns the w-th run of 256 consecutive rows, a lane per row and step, so every load and store
+// is contiguous.  Tiles hand the running sums on by a decoupled look-back.
+//   Routing: a row the warp kernel counted and whose outputs fit a warp's accumulator stays with a warp;
+//   every other dense row becomes one CTA unit, or several when it has many products: unit c of n takes
+//   the c-th n-th of the row's A entries (all units of a row add into the same outputs).  The units of
+//   the heaviest rows come first.
+//   TTM: a fibre (i,j) survives when it produced an output; survivors are packed (Cpos2, Ccrd1), and
+//   sfp[s] receives the number of survivors before slice s.
+// Replaces a three-launch scan, the routing and the per-class count (five launches; seven for the
+// 3-tensor form).
+// FINISH_MEASURED
+// ---------------------------------------------------------------------------------------
+constexpr int FR_THREADS = 256;
+constexpr int FR_WARPS = FR_THREADS / 32;
+constexpr int FR_ITEMS = 8;
+constexpr int FR_TILE = FR_THREADS * FR_ITEMS;
+constexpr int SL_TILE = FR_THREADS * 4;             // slices per block of the slice level
 
-cudaError_t launch_dense_rebin(const LaunchCtx& c, int m, const i64* rowptr) {
-    (void)rowptr;
-    if (m == 0) return cudaSuccess;
-    i64 want = ((i64)m + 255) / 256;
-    i64 cap = (i64)c.sm_count * 8;
-    dense_rebin_kernel<<<(int)(want < cap ? want : cap), 256, 0, c.stream>>>(m, c.tab, c.prm, c.ctl);
-    ++c.launches;
-    return cudaGetLastError();
-}
+struct FibreArgs {
+    const i64* Apos1;
+    const int* Acrd1;
+    int n_i;
+    i64* sfp;
+    int* Ccrd1;
+    i64* Cpos2;
+};
 
-// Output entries per class (statistics for the per-kernel byte counts): one pass over the rows in
-// row order, every thread keeping a sum per class.
-__global__ void __launch_bounds__(256) class_nnz_kernel(int m, RowTables tab, DevCtl* ctl) {
-    i64 sum[NCLASS];
+template <bool DENSE, bool TTM>
+__global__ void __launch_bounds__(FR_THREADS) finish_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, DevCtl* host, u64* look,
+                                                                 i64* __restrict__ rowptr, FibreArgs f) {
+    __shared__ int s_tile, s_slice0;
+    __shared__ i64 s_sum[FR_WARPS], s_before[2];
+    __shared__ int s_part[4][FR_WARPS];             // survivors, warp rows, units of heavy rows, other units
+    __shared__ int s_base[3];
+    __shared__ i64 s_cls[FR_WARPS][NCLASS];
+    __shared__ i64 s_wp[FR_WARPS], s_wn[FR_WARPS];
+    __shared__ int s_wm[FR_WARPS];
+    __shared__ int s_kept[TTM ? FR_TILE : 1];       // survivors of the tile before each fibre
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned all = 0xffffffffu, below = (1u << lane) - 1u;
+    const int tiles = gridDim.x;
+    if (tid == 0) s_tile = atomicAdd(&ctl->rows_ticket, 1);
+    for (int x = tid; x < FR_WARPS * NCLASS; x += FR_THREADS) (&s_cls[0][0])[x] = 0;
+    __syncthreads();
+    const int tile = s_tile;
+    const i64 tile0 = (i64)tile * FR_TILE;
+    const i64 row0 = tile0 + warp * (FR_ITEMS * 32) + lane;
+    const i64 unit_products = DENSE ? dense_unit_products(ctl->products) : 1;
+
+    // ---- this warp's rows: counts, sums, routing
+    int v[FR_ITEMS], cls[FR_ITEMS];
+    i64 sum = 0, wp = 0, wn = 0;
+    int kept = 0, to_warp = 0, heavy = 0, other = 0, wm = 0;
 #pragma unroll
-    for (int k = 0; k < NCLASS; ++k) sum[k] = 0;
-    for (i64 row = (i64)blockIdx.x * blockDim.x + threadIdx.x; row < m; row += (i64)gridDim.x * blockDim.x) {
-        const int c = tab.cls[row];
-        const int v = tab.cnt[row];
-#pragma unroll
-        for (int k = 0; k < NCLASS; ++k) sum[k] += (c == k) ? v : 0;
+    for (int x = 0; x < FR_ITEMS; ++x) {
+        const i64 row = row0 + 32 * x;
+        v[x] = row < m ? tab.cnt[row] : 0;
+        cls[x] = row < m ? (int)tab.cls[row] : (int)CLS_EMPTY;
     }
-    __shared__ i64 s_part[8][NCLASS];
+    // units of row x: 0 for a row of the warp kernel and for rows that are not dense
+    auto units = [&](int x) -> int {
+        if (cls[x] < CLS_DENSE_WARP || cls[x] > CLS_DENSE_CTA || (cls[x] == CLS_DENSE_WARP && v[x] <= DENSE_WARP_ACC)) return 0;
+        return dense_units_of_row(tab.ub[row0 + 32 * x], unit_products);
+    };
 #pragma unroll
-    for (int k = 0; k < NCLASS; ++k) {
-        i64 t = sum[k];
-        for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-        if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5][k] = t;
+    for (int x = 0; x < FR_ITEMS; ++x) {
+        sum += v[x];
+        if (TTM) kept += __popc(__ballot_sync(all, v[x] > 0));
+        // outputs per class: one round per class among the 32 rows (nearly always one)
+        unsigned todo = __ballot_sync(all, cls[x] != CLS_EMPTY);
+        while (todo) {
+            const int k = __shfl_sync(all, cls[x], __ffs(todo) - 1);
+            const bool mine = cls[x] == k;
+            const unsigned lo = __reduce_add_sync(all, mine ? (unsigned)v[x] & 0xffffu : 0u);
+            const unsigned hi = __reduce_add_sync(all, mine ? (unsigned)v[x] >> 16 : 0u);
+            if (lane == 0) s_cls[warp][k] += (i64)lo + ((i64)hi << 16);
+            todo &= ~__ballot_sync(all, mine);
+        }
+        if (DENSE) {
+            const bool w = cls[x] == CLS_DENSE_WARP && v[x] <= DENSE_WARP_ACC;
+            to_warp += __popc(__ballot_sync(all, w));
+            if (w) { wp += tab.ub[row0 + 32 * x]; wn += v[x]; wm = max(wm, v[x]); }
+            const int nu = units(x);
+            if (cls[x] == CLS_DENSE_HUB) heavy += nu; else other += nu;
+        }
+    }
+    for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(all, sum, d);
+    if (DENSE) {
+        for (int d = 16; d > 0; d >>= 1) {
+            wp += __shfl_xor_sync(all, wp, d);
+            wn += __shfl_xor_sync(all, wn, d);
+        }
+        wm = __reduce_max_sync(all, wm);
+        heavy = __reduce_add_sync(all, heavy);
+        other = __reduce_add_sync(all, other);
+    }
+    if (lane == 0) {
+        s_sum[warp] = sum;
+        s_part[0][warp] = kept; s_part[1][warp] = to_warp; s_part[2][warp] = heavy; s_part[3][warp] = other;
+        s_wp[warp] = wp; s_wn[warp] = wn; s_wm[warp] = wm;
     }
     __syncthreads();
-    if (threadIdx.x < NCLASS && threadIdx.x != CLS_EMPTY) {
+    i64 tile_sum = 0, warp_sum = 0;
+    int total[4] = {0, 0, 0, 0}, mine[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int w = 0; w < FR_WARPS; ++w) {
+        if (w == warp) warp_sum = tile_sum;
+        tile_sum += s_sum[w];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            if (w == warp) mine[t] = total[t];
+            total[t] += s_part[t][w];
+        }
+    }
+    // ---- running sums from the tiles before; places in the routing tables
+    if (warp == 0 || (TTM && warp == 1)) {
+        u64* const words = look + (warp == 0 ? 0 : tiles);
+        const i64 own = warp == 0 ? tile_sum : (i64)total[0];
+        if (lane == 0) look_publish(words + tile, tile == 0 ? 2 : 1, own);
+        i64 before = 0;
+        if (tile > 0) {
+            before = look_back_warp(words, tile, 0, ctl);
+            if (lane == 0) look_publish(words + tile, 2, before + own);
+        }
+        if (lane == 0) s_before[warp] = before;
+    }
+    if (DENSE && tid == 64) {
+        s_base[0] = total[1] ? atomicAdd(&ctl->n_warp_rows, total[1]) : 0;
+        s_base[1] = total[2] ? atomicAdd(&ctl->hub_cursor, total[2]) : 0;
+        s_base[2] = (total[3] ? atomicAdd(&ctl->other_cursor, total[3]) : 0) + ctl->hub_units;
+        if (total[1]) {
+            i64 p = 0, n = 0;
+            int most = 0;
+            for (int w = 0; w < FR_WARPS; ++w) { p += s_wp[w]; n += s_wn[w]; most = max(most, s_wm[w]); }
+            atomicAdd((u64*)&ctl->dense_warp_products, (u64)p);
+            atomicAdd((u64*)&ctl->dense_warp_nnz, (u64)n);
+            atomicMax(&ctl->max_warp_cnt, most);
+        }
+    }
+    if (TTM && tid == 96) {                         // first slice that starts in this tile or later
+        int lo = 0, hi = f.n_i;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (f.Apos1[mid] < tile0) lo = mid + 1; else hi = mid;
+        }
+        s_slice0 = lo;
+    }
+    if (tid >= 128 && tid < 128 + NCLASS) {
         i64 t = 0;
-        for (int w = 0; w < 8; ++w) t += s_part[w][threadIdx.x];
-        if (t) atomicAdd((u64*)&ctl->class_nnz[threadIdx.x], (u64)t);
+        for (int w = 0; w < FR_WARPS; ++w) t += s_cls[w][tid - 128];
+        if (t) atomicAdd((u64*)&ctl->class_nnz[tid - 128], (u64)t);
+    }
+    __syncthreads();
+
+    // ---- placement
+    i64 run = s_before[0] + warp_sum;
+    const i64 kbase = TTM ? s_before[1] : 0;
+    int krun = mine[0], wrun = mine[1], hrun = mine[2], orun = mine[3];
+#pragma unroll
+    for (int x = 0; x < FR_ITEMS; ++x) {
+        const i64 row = row0 + 32 * x;
+        i64 incl = v[x];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const i64 t = __shfl_up_sync(all, incl, d);
+            if (lane >= d) incl += t;
+        }
+        const i64 at = run + incl - v[x];
+        run += __shfl_sync(all, incl, 31);
+        if (row < m) rowptr[row] = at;
+        if (TTM) {
+            const unsigned live = __ballot_sync(all, v[x] > 0);
+            const int k = krun + __popc(live & below);
+            s_kept[warp * (FR_ITEMS * 32) + x * 32 + lane] = k;
+            if (v[x] > 0) {
+                f.Cpos2[kbase + k] = at;
+                f.Ccrd1[kbase + k] = f.Acrd1[row];
+            }
+            krun += __popc(live);
+        }
+        if (DENSE) {
+            const bool w = cls[x] == CLS_DENSE_WARP && v[x] <= DENSE_WARP_ACC;
+            const unsigned ws = __ballot_sync(all, w);
+            if (w) {
+                tab.warp_rows[s_base[0] + wrun + __popc(ws & below)] = (int)row;
+                tab.row_unit0[row] = -1;
+            }
+            wrun += __popc(ws);
+            const int nu = units(x);
+            if (__any_sync(all, nu > 0)) {
+                const bool hub = cls[x] == CLS_DENSE_HUB;
+                const int hi = warp_incl_scan(hub ? nu : 0), oi = warp_incl_scan(hub ? 0 : nu);
+                if (nu > 0) {
+                    const i64 u0 = hub ? (i64)s_base[1] + hrun + hi - nu : (i64)s_base[2] + orun + oi - nu;
+                    if (u0 + nu > prm.unit_cap) {
+                        raise_status(ctl, DEV_SCRATCH_TOO_SMALL);
+                        tab.row_unit0[row] = -1;
+                    } else {
+                        tab.row_unit0[row] = (int)u0;
+                        for (int t = 0; t < nu; ++t) tab.unit_row[u0 + t] = (int)row;
+                    }
+                }
+                hrun += __shfl_sync(all, hi, 31);
+                orun += __shfl_sync(all, oi, 31);
+            }
+        }
+    }
+    if (tile == tiles - 1 && tid == 0) {
+        const i64 nnz = s_before[0] + tile_sum;
+        rowptr[m] = nnz;
+        ctl->nnz = nnz;
+        if (TTM) {
+            const i64 k = kbase + total[0];
+            f.Cpos2[k] = nnz;
+            f.sfp[f.n_i] = k;
+            ctl->kept[1] = k;
+        }
+    }
+    if (TTM) {
+        __syncthreads();
+        for (int s = s_slice0 + tid; s < f.n_i; s += FR_THREADS) {
+            const i64 at = f.Apos1[s] - tile0;
+            if (at >= FR_TILE && tile != tiles - 1) break;
+            f.sfp[s] = kbase + (at >= 0 && at < FR_TILE && tile0 + at < m ? s_kept[at] : total[0]);
+        }
+    }
+    if (last_block(&ctl->rows_done, tiles)) {
+        if (tid == 0) ctl->n_units = ctl->hub_units + ctl->other_cursor;
+        __threadfence();
+        __syncthreads();
+        if (!TTM) publish_ctl(ctl, host);           // (the slice level comes after the fibres)
     }
 }
 
-cudaError_t launch_class_nnz(const LaunchCtx& c, int m) {
-    if (m == 0) return cudaSuccess;
-    i64 want = ((i64)m + 255) / 256;
-    i64 cap = (i64)c.sm_count * 8;
-    class_nnz_kernel<<<(int)(want < cap ? want : cap), 256, 0, c.stream>>>(m, c.tab, c.ctl);
+// A slice i survives when one of its fibres does: C's slice level from sfp.
+__global__ void __launch_bounds__(FR_THREADS) finish_slices_kernel(int n_i, const i64* __restrict__ sfp, const int* __restrict__ Acrd0, DevCtl* ctl,
+                                                                   DevCtl* host, u64* look, int* __restrict__ Ccrd0, i64* __restrict__ Cpos1,
+                                                                   i64* __restrict__ Cpos0) {
+    __shared__ int s_tile, s_part[FR_WARPS];
+    __shared__ i64 s_before;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tiles = gridDim.x;
+    if (tid == 0) s_tile = atomicAdd(&ctl->slices_ticket, 1);
+    __syncthreads();
+    const int tile = s_tile;
+    const i64 s0 = (i64)tile * SL_TILE + warp * 128 + lane;
+    i64 first[4];
+    unsigned live[4];
+    int n = 0;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        const i64 s = s0 + 32 * x;
+        first[x] = s < n_i ? sfp[s] : 0;
+        live[x] = __ballot_sync(0xffffffffu, s < n_i && sfp[s + 1] > first[x]);
+        n += __popc(live[x]);
+    }
+    if (lane == 0) s_part[warp] = n;
+    __syncthreads();
+    int total = 0, mine = 0;
+#pragma unroll
+    for (int w = 0; w < FR_WARPS; ++w) {
+        if (w == warp) mine = total;
+        total += s_part[w];
+    }
+    if (warp == 0) {
+        if (lane == 0) look_publish(look + tile, tile == 0 ? 2 : 1, total);
+        i64 before = 0;
+        if (tile > 0) {
+            before = look_back_warp(look, tile, 0, ctl);
+            if (lane == 0) look_publish(look + tile, 2, before + total);
+        }
+        if (lane == 0) s_before = before;
+    }
+    __syncthreads();
+    i64 at = s_before + mine;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        if ((live[x] >> lane) & 1u) {
+            const i64 o = at + __popc(live[x] & ((1u << lane) - 1u));
+            Ccrd0[o] = Acrd0[s0 + 32 * x];
+            Cpos1[o] = first[x];
+        }
+        at += __popc(live[x]);
+    }
+    if (tile == tiles - 1 && tid == 0) {
+        const i64 k = s_before + total;
+        Cpos1[k] = sfp[n_i];
+        Cpos0[0] = 0;
+        Cpos0[1] = k;
+        ctl->kept[0] = k;
+    }
+    if (last_block(&ctl->slices_done, tiles)) publish_ctl(ctl, host);
+}
+
+static int tiles_of(i64 n, int tile) { return n > 0 ? (int)((n + tile - 1) / tile) : 1; }
+
+size_t look_words(i64 rows, i64 slices) { return (size_t)2 * tiles_of(rows, FR_TILE) + tiles_of(slices, SL_TILE); }
+
+cudaError_t launch_finish_rows(const LaunchCtx& c, int m, bool any_dense, i64* rowptr) {
+    const int tiles = tiles_of(m, FR_TILE);
+    if (any_dense) finish_rows_kernel<true, false><<<tiles, FR_THREADS, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host_ctl, c.look, rowptr, FibreArgs{});
+    else finish_rows_kernel<false, false><<<tiles, FR_THREADS, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host_ctl, c.look, rowptr, FibreArgs{});
     ++c.launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_finish_fibres(const LaunchCtx& c, int n_i, int n_ij, bool any_dense, const i64* Apos1, const int* Acrd0, const int* Acrd1,
+                                 i64* rowptr_raw, i64* sfp, i64* Cpos0, int* Ccrd0, i64* Cpos1, int* Ccrd1, i64* Cpos2) {
+    const int tiles = tiles_of(n_ij, FR_TILE);
+    const FibreArgs f{Apos1, Acrd1, n_i, sfp, Ccrd1, Cpos2};
+    if (any_dense) finish_rows_kernel<true, true><<<tiles, FR_THREADS, 0, c.stream>>>(n_ij, c.tab, c.prm, c.ctl, c.host_ctl, c.look, rowptr_raw, f);
+    else finish_rows_kernel<false, true><<<tiles, FR_THREADS, 0, c.stream>>>(n_ij, c.tab, c.prm, c.ctl, c.host_ctl, c.look, rowptr_raw, f);
+    finish_slices_kernel<<<tiles_of(n_i, SL_TILE), FR_THREADS, 0, c.stream>>>(n_i, sfp, Acrd0, c.ctl, c.host_ctl, c.look + 2 * tiles, Ccrd0, Cpos1,
+                                                                             Cpos0);
+    c.launches += 2;
     return cudaGetLastError();
 }
 
@@ -664,15 +878,13 @@ constexpr int SCAN_THREADS = 256;
 constexpr int SCAN_ITEMS = 8;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
 
-// FLAG: scan (in[i] > 0) instead of in[i] (compaction positions without a flag array).
-template <bool FLAG>
 __global__ void __launch_bounds__(SCAN_THREADS) scan_reduce_kernel(const int* __restrict__ in, int n, i64* block_sums) {
     __shared__ i64 s_part[SCAN_THREADS / 32];
     const i64 base = (i64)blockIdx.x * SCAN_TILE;
     i64 s = 0;
     for (int x = 0; x < SCAN_ITEMS; ++x) {
         const i64 i = base + x * SCAN_THREADS + threadIdx.x;
-        if (i < n) s += FLAG ? (in[i] > 0) : in[i];
+        if (i < n) s += in[i];
     }
     for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
     if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = s;
@@ -723,7 +935,6 @@ __global__ void __launch_bounds__(1024) scan_block_sums_kernel(i64* block_sums, 
 }
 
 // The in-tile prefix is carried in 64 bits: a tile of 2048 counts may total 2^31 or more.
-template <bool FLAG>
 __global__ void __launch_bounds__(SCAN_THREADS) scan_apply_kernel(const int* __restrict__ in, int n, const i64* __restrict__ block_sums, i64* __restrict__ out) {
     __shared__ i64 s_warp[SCAN_THREADS / 32];
     const i64 base = (i64)blockIdx.x * SCAN_TILE + (i64)threadIdx.x * SCAN_ITEMS;
@@ -732,7 +943,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_apply_kernel(const int* __r
     i64 s = 0;
 #pragma unroll
     for (int x = 0; x < SCAN_ITEMS; ++x) {
-        v[x] = (base + x < n) ? (FLAG ? (in[base + x] > 0) : in[base + x]) : 0;
+        v[x] = (base + x < n) ? in[base + x] : 0;
         s += v[x];
     }
     i64 incl = s;
@@ -754,262 +965,12 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_apply_kernel(const int* __r
     }
 }
 
-cudaError_t launch_scan_counts(const LaunchCtx& c, const int* cnt, int n, i64* out, i64* block_sums, i64* total_out, bool as_flags) {
+cudaError_t launch_scan_counts(const LaunchCtx& c, const int* cnt, int n, i64* out, i64* block_sums, i64* total_out) {
     const int nblocks = (int)(((i64)n + SCAN_TILE - 1) / SCAN_TILE);
-    if (nblocks > 0) {
-        if (as_flags) scan_reduce_kernel<true><<<nblocks, SCAN_THREADS, 0, c.stream>>>(cnt, n, block_sums);
-        else scan_reduce_kernel<false><<<nblocks, SCAN_THREADS, 0, c.stream>>>(cnt, n, block_sums);
-    }
+    if (nblocks > 0) scan_reduce_kernel<<<nblocks, SCAN_THREADS, 0, c.stream>>>(cnt, n, block_sums);
     scan_block_sums_kernel<<<1, 1024, 0, c.stream>>>(block_sums, nblocks, out + n, total_out);
-    if (nblocks > 0) {
-        if (as_flags) scan_apply_kernel<true><<<nblocks, SCAN_THREADS, 0, c.stream>>>(cnt, n, block_sums, out);
-        else scan_apply_kernel<false><<<nblocks, SCAN_THREADS, 0, c.stream>>>(cnt, n, block_sums, out);
-    }
+    if (nblocks > 0) scan_apply_kernel<<<nblocks, SCAN_THREADS, 0, c.stream>>>(cnt, n, block_sums, out);
     c.launches += nblocks > 0 ? 3 : 1;
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------------------
-// TTM: rebuild C's two upper CSF levels.  A fibre (i,j) survives when it produced at least
-// one output; a slice i survives when one of its fibres does.
-// ---------------------------------------------------------------------------------------
-__global__ void ttm_slice_flags_kernel(int n_i, const i64* __restrict__ Apos1, const i64* __restrict__ fpos, int* sflags) {
-    for (i64 s = (i64)blockIdx.x * blockDim.x + threadIdx.x; s < n_i; s += (i64)gridDim.x * blockDim.x)
-        sflags[s] = fpos[Apos1[s + 1]] > fpos[Apos1[s]];
-}
-
-__global__ void ttm_slice_compact_kernel(int n_i, int n_ij, const int* __restrict__ sflags, const i64* __restrict__ spos,
-                                         const i64* __restrict__ Apos1, const i64* __restrict__ fpos,
-                                         const int* __restrict__ Acrd0, int* Ccrd0, i64* Cpos1, i64* Cpos0, DevCtl* ctl) {
-    for (i64 s = (i64)blockIdx.x * blockDim.x + threadIdx.x; s <= n_i; s += (i64)gridDim.x * blockDim.x) {
-        if (s == n_i) {
-            Cpos1[spos[n_i]] = fpos[n_ij];
-            Cpos0[0] = 0;
-            Cpos0[1] = spos[n_i];
-            ctl->kept[0] = spos[n_i];
-            ctl->kept[1] = fpos[n_ij];
-            continue;
-        }
-        if (sflags[s]) {
-            Ccrd0[spos[s]] = Acrd0[s];
-            Cpos1[spos[s]] = fpos[Apos1[s]];
-        }
-    }
-}
-
-// The slice level in ONE launch when it is small: a single block flags, scans and compacts the
-// slices 1024 at a time with a running count.
-__global__ void __launch_bounds__(1024) ttm_slices_small_kernel(int n_i, int n_ij, const i64* __restrict__ Apos1, const i64* __restrict__ fpos,
-                                                                const int* __restrict__ Acrd0, int* Ccrd0, i64* Cpos1, i64* Cpos0,
-                                                                DevCtl* ctl) {
-    __shared__ int ws[33];
-    int kept = 0;
-    // four consecutive slices per thread, their loads issued together (this block is alone on the
-    // GPU, so every dependent load costs a full memory latency)
-    for (int s0 = 0; s0 < n_i; s0 += 4096) {
-        const int s = s0 + 4 * threadIdx.x;
-        i64 edge[5], fp[5];
-#pragma unroll
-        for (int x = 0; x < 5; ++x) edge[x] = (s + x <= n_i) ? Apos1[s + x] : -1;
-#pragma unroll
-        for (int x = 0; x < 5; ++x) fp[x] = edge[x] >= 0 ? fpos[edge[x]] : 0;
-        int crd[4], nflag = 0;
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            const bool flag = s + x < n_i && fp[x + 1] > fp[x];
-            crd[x] = flag ? Acrd0[s + x] : -1;
-            nflag += flag;
-        }
-        int total;
-        int at = kept + block_excl_scan<1024>(nflag, ws, total);
-#pragma unroll
-        for (int x = 0; x < 4; ++x)
-            if (s + x < n_i && fp[x + 1] > fp[x]) {
-                Ccrd0[at] = crd[x];
-                Cpos1[at] = fp[x];
-                ++at;
-            }
-        kept += total;
-    }
-    if (threadIdx.x == 0) {
-        Cpos1[kept] = fpos[n_ij];
-        Cpos0[0] = 0;
-        Cpos0[1] = kept;
-        ctl->kept[0] = kept;
-        ctl->kept[1] = fpos[n_ij];
-    }
-}
-
-// The fibre level in three launches: the scan of the counts (C's bottom-level positions) and the
-// scan of (count > 0) (where a surviving fibre goes) share their passes over the counts, and the
-// second pass places the survivors as it goes.
-__global__ void __launch_bounds__(SCAN_THREADS) ttm_dual_reduce_kernel(const int* __restrict__ cnt, int n, i64* sums, i64* kept) {
-    __shared__ i64 s_part[2][SCAN_THREADS / 32];
-    const i64 base = (i64)blockIdx.x * SCAN_TILE;
-    i64 s = 0;
-    int k = 0;
-    for (int x = 0; x < SCAN_ITEMS; ++x) {
-        const i64 i = base + x * SCAN_THREADS + threadIdx.x;
-        if (i < n) { const int v = cnt[i]; s += v; k += v > 0; }
-    }
-    for (int d = 16; d > 0; d >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, d);
-        k += __shfl_xor_sync(0xffffffffu, k, d);
-    }
-    if ((threadIdx.x & 31) == 0) { s_part[0][threadIdx.x >> 5] = s; s_part[1][threadIdx.x >> 5] = k; }
-    __syncthreads();
-    if (threadIdx.x < 2) {
-        i64 t = 0;
-        for (int w = 0; w < SCAN_THREADS / 32; ++w) t += s_part[threadIdx.x][w];
-        (threadIdx.x == 0 ? sums : kept)[blockIdx.x] = t;
-    }
-}
-
-// exclusive scans of both block-sum arrays by one block; the totals close the three arrays
-__global__ void __launch_bounds__(1024) ttm_dual_block_sums_kernel(i64* sums, i64* kept, int nblocks, int n, i64* rowptr_raw, i64* fpos,
-                                                                   i64* Cpos2, i64* nnz_out) {
-    __shared__ i64 s_warp[2][32];
-    __shared__ i64 s_carry[2];
-    if (threadIdx.x < 2) s_carry[threadIdx.x] = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int base = 0; base < nblocks; base += 1024) {
-        const int i = base + threadIdx.x;
-        const i64 v0 = (i < nblocks) ? sums[i] : 0, v1 = (i < nblocks) ? kept[i] : 0;
-        i64 i0 = v0, i1 = v1;
-        for (int d = 1; d < 32; d <<= 1) {
-            const i64 t0 = __shfl_up_sync(0xffffffffu, i0, d), t1 = __shfl_up_sync(0xffffffffu, i1, d);
-            if (lane >= d) { i0 += t0; i1 += t1; }
-        }
-        if (lane == 31) { s_warp[0][warp] = i0; s_warp[1][warp] = i1; }
-        __syncthreads();
-        if (warp < 2) {
-            const i64 w = s_warp[warp][lane];
-            i64 wi = w;
-            for (int d = 1; d < 32; d <<= 1) {
-                const i64 t = __shfl_up_sync(0xffffffffu, wi, d);
-                if (lane >= d) wi += t;
-            }
-            s_warp[warp][lane] = wi - w;
-        }
-        __syncthreads();
-        const i64 c0 = s_carry[0], c1 = s_carry[1];
-        if (i < nblocks) { sums[i] = c0 + s_warp[0][warp] + i0 - v0; kept[i] = c1 + s_warp[1][warp] + i1 - v1; }
-        __syncthreads();
-        if (threadIdx.x == 1023) { s_carry[0] = c0 + s_warp[0][warp] + i0; s_carry[1] = c1 + s_warp[1][warp] + i1; }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        rowptr_raw[n] = s_carry[0];
-        fpos[n] = s_carry[1];
-        Cpos2[s_carry[1]] = s_carry[0];
-        *nnz_out = s_carry[0];
-    }
-}
-
-__global__ void __launch_bounds__(SCAN_THREADS) ttm_dual_apply_kernel(const int* __restrict__ cnt, int n, const i64* __restrict__ sums,
-                                                                      const i64* __restrict__ kept, const int* __restrict__ Acrd1,
-                                                                      i64* __restrict__ rowptr_raw, i64* __restrict__ fpos,
-                                                                      int* __restrict__ Ccrd1, i64* __restrict__ Cpos2) {
-    // a thread scans SCAN_ITEMS consecutive counts; everything crosses shared memory on the way in
-    // and out so that global loads and stores are contiguous across the block
-    __shared__ i64 s_a[SCAN_TILE];          // counts on the way in (as int), then one output array at a time
-    __shared__ int s_crd[SCAN_TILE];        // the tile's fibre coordinates, then the survivors'
-    __shared__ i64 s_warp[SCAN_THREADS / 32];
-    __shared__ int s_kwarp[SCAN_THREADS / 32];
-    const i64 tile = (i64)blockIdx.x * SCAN_TILE;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int len = (int)min((i64)SCAN_TILE, (i64)n - tile);
-    int* s_cnt = reinterpret_cast<int*>(s_a);
-    for (int i = tid; i < SCAN_TILE; i += SCAN_THREADS) {
-        s_cnt[i] = i < len ? cnt[tile + i] : 0;
-        s_crd[i] = i < len ? Acrd1[tile + i] : 0;
-    }
-    __syncthreads();
-    int v[SCAN_ITEMS], crd[SCAN_ITEMS];
-    i64 s = 0;
-    int k = 0;
-#pragma unroll
-    for (int x = 0; x < SCAN_ITEMS; ++x) {
-        v[x] = s_cnt[tid * SCAN_ITEMS + x];
-        crd[x] = s_crd[tid * SCAN_ITEMS + x];
-        s += v[x];
-        k += v[x] > 0;
-    }
-    i64 incl = s;
-    int kincl = k;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const i64 t = __shfl_up_sync(0xffffffffu, incl, d);
-        const int tk = __shfl_up_sync(0xffffffffu, kincl, d);
-        if (lane >= d) { incl += t; kincl += tk; }
-    }
-    if (lane == 31) { s_warp[warp] = incl; s_kwarp[warp] = kincl; }
-    __syncthreads();                                      // also: every thread has read s_cnt and s_crd
-    i64 before = 0;
-    int kbefore = 0, ktile = 0;
-#pragma unroll
-    for (int w = 0; w < SCAN_THREADS / 32; ++w) {
-        before += (w < warp) ? s_warp[w] : 0;
-        kbefore += (w < warp) ? s_kwarp[w] : 0;
-        ktile += s_kwarp[w];
-    }
-    const i64 run0 = sums[blockIdx.x] + before + incl - s;
-    const i64 kept0 = kept[blockIdx.x];
-    const int at0 = kbefore + kincl - k;                  // survivors of the tile before this thread's
-    // C's bottom-level positions of all fibres
-    i64 run = run0;
-#pragma unroll
-    for (int x = 0; x < SCAN_ITEMS; ++x) { s_a[tid * SCAN_ITEMS + x] = run; run += v[x]; }
-    __syncthreads();
-    for (int i = tid; i < len; i += SCAN_THREADS) rowptr_raw[tile + i] = s_a[i];
-    __syncthreads();
-    // place of every fibre among the survivors
-    int at = at0;
-#pragma unroll
-    for (int x = 0; x < SCAN_ITEMS; ++x) { s_a[tid * SCAN_ITEMS + x] = kept0 + at; at += v[x] > 0; }
-    __syncthreads();
-    for (int i = tid; i < len; i += SCAN_THREADS) fpos[tile + i] = s_a[i];
-    __syncthreads();
-    // the survivors' coordinates and positions, packed
-    run = run0;
-    at = at0;
-#pragma unroll
-    for (int x = 0; x < SCAN_ITEMS; ++x) {
-        if (v[x] > 0) { s_a[at] = run; s_crd[at] = crd[x]; ++at; }
-        run += v[x];
-    }
-    __syncthreads();
-    for (int i = tid; i < ktile; i += SCAN_THREADS) {
-        Cpos2[kept0 + i] = s_a[i];
-        Ccrd1[kept0 + i] = s_crd[i];
-    }
-}
-
-// Scan of the fibre counts, survivors' positions, C's two lower levels' coordinates and positions,
-// then the slice level.  `block_sums` holds two arrays of one entry per scan tile.
-cudaError_t launch_ttm_scan_compact(const LaunchCtx& c, int n_i, int n_ij, const i64* Apos1, const int* Acrd0, const int* Acrd1,
-                                    i64* rowptr_raw, i64* fpos, int* sflags, i64* spos, i64* block_sums, i64* nnz_out,
-                                    i64* Cpos0, int* Ccrd0, i64* Cpos1, int* Ccrd1, i64* Cpos2) {
-    const int nblocks = (int)(((i64)n_ij + SCAN_TILE - 1) / SCAN_TILE);
-    i64* sums = block_sums;
-    i64* kept = block_sums + nblocks + 1;
-    if (nblocks > 0) ttm_dual_reduce_kernel<<<nblocks, SCAN_THREADS, 0, c.stream>>>(c.tab.cnt, n_ij, sums, kept);
-    ttm_dual_block_sums_kernel<<<1, 1024, 0, c.stream>>>(sums, kept, nblocks, n_ij, rowptr_raw, fpos, Cpos2, nnz_out);
-    if (nblocks > 0)
-        ttm_dual_apply_kernel<<<nblocks, SCAN_THREADS, 0, c.stream>>>(c.tab.cnt, n_ij, sums, kept, Acrd1, rowptr_raw, fpos, Ccrd1, Cpos2);
-    c.launches += nblocks > 0 ? 3 : 1;
-    if (n_i <= (1 << 16)) {
-        ttm_slices_small_kernel<<<1, 1024, 0, c.stream>>>(n_i, n_ij, Apos1, fpos, Acrd0, Ccrd0, Cpos1, Cpos0, c.ctl);
-        ++c.launches;
-        return cudaGetLastError();
-    }
-    const int grid = c.sm_count * 8;
-    ttm_slice_flags_kernel<<<grid, 256, 0, c.stream>>>(n_i, Apos1, fpos, sflags);
-    cudaError_t e = launch_scan_counts(c, sflags, n_i, spos, block_sums, nullptr);
-    if (e != cudaSuccess) return e;
-    ttm_slice_compact_kernel<<<grid, 256, 0, c.stream>>>(n_i, n_ij, sflags, spos, Apos1, fpos, Acrd0, Ccrd0, Cpos1, Cpos0, c.ctl);
-    c.launches += 2;
     return cudaGetLastError();
 }
 

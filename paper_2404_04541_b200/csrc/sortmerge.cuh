@@ -18,66 +18,6 @@ static int grid_for(const LaunchCtx& c, i64 work_items, int per_block) {
     return (int)(want < 1 ? 1 : want);
 }
 
-// ---- running sums handed from tile to tile ---------------------------------------------------
-// A tile of a single-pass scan publishes one 64-bit word: a tag above 56 bits of count.  The tag of a
-// pass is 2 * pass + 1 while the word holds the tile's own count and 2 * pass + 2 once it holds the
-// count of all tiles up to it, so one clearing serves all the passes of a sort.  Tiles are numbered
-// by a ticket taken when a block starts, hence every tile that is waited for is running or done; a
-// wait that does not end after LOOK_LIMIT polls raises the status word and goes on with what it has
-// (too small a count, so that every index stays inside the arrays).
-constexpr int LOOK_SHIFT = 56;
-constexpr u64 LOOK_MASK = (1ull << LOOK_SHIFT) - 1;
-constexpr int LOOK_LIMIT = 1 << 22;
-
-__device__ __forceinline__ void look_publish(u64* word, int tag, i64 count) {
-    *(volatile u64*)word = ((u64)tag << LOOK_SHIFT) | (u64)count;
-}
-
-// Sum of the counts of the tiles before `tile` (one word per tile, `stride` words apart): a single
-// thread walks back until it meets a running sum.
-__device__ __forceinline__ i64 look_back(const u64* words, int stride, int tile, int pass, DevCtl* ctl) {
-    i64 sum = 0;
-    int polls = 0;
-    for (int t = tile - 1; t >= 0;) {
-        const u64 w = *(const volatile u64*)(words + (i64)t * stride);
-        const int tag = (int)(w >> LOOK_SHIFT);
-        if (tag <= 2 * pass) {
-            if (++polls >= LOOK_LIMIT) { raise_status(ctl, DEV_INTERNAL_OVERFLOW); break; }
-            continue;
-        }
-        sum += (i64)(w & LOOK_MASK);
-        if (tag == 2 * pass + 2) break;
-        --t;
-    }
-    return sum;
-}
-
-// The same for a whole warp: 32 predecessors per step.  Every lane returns the sum.
-__device__ __forceinline__ i64 look_back_warp(const u64* words, int tile, int pass, DevCtl* ctl) {
-    const int lane = threadIdx.x & 31;
-    i64 sum = 0;
-    int polls = 0;
-    for (int t0 = tile - 1; t0 >= 0; t0 -= 32) {
-        const int t = t0 - lane;
-        u64 w = (u64)(2 * pass + 2) << LOOK_SHIFT;              // before the first tile: a running sum of nothing
-        for (;;) {
-            if (t >= 0) w = *(const volatile u64*)(words + t);
-            if (__all_sync(0xffffffffu, (int)(w >> LOOK_SHIFT) > 2 * pass)) break;
-            if (++polls >= LOOK_LIMIT) {
-                if (lane == 0) raise_status(ctl, DEV_INTERNAL_OVERFLOW);
-                return sum;
-            }
-        }
-        const unsigned ends = __ballot_sync(0xffffffffu, (int)(w >> LOOK_SHIFT) == 2 * pass + 2);
-        const int last = ends ? __ffs(ends) - 1 : 31;           // the nearest running sum ends the walk
-        i64 v = lane <= last ? (i64)(w & LOOK_MASK) : 0;
-        for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-        sum += v;
-        if (ends) break;
-    }
-    return sum;
-}
-
 // ---- stable LSD radix sort, 8 bits per pass -------------------------------------------------
 // The digits of all passes are counted in one reading of the keys; a pass is then one launch: a
 // block takes the next tile of RS_TILE consecutive elements, ranks them among equal digits (warp w

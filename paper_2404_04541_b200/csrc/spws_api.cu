@@ -35,6 +35,8 @@ struct spws_plan_s {
     int max_span_words = 0;     // widest dense bitmap of the last symbolic pass
     int max_warp_cnt = 0;       // most outputs of a warp-numeric row
     int64_t max_ub_smem = 0;    // most products of a shared-memory ISM row
+    bool counters_clear = false; // the numeric pass's work counters are as the symbolic pass left them: zero
+    bool rows_path = false;     // the last symbolic pass was a row-wise one, whose errors reach host->ctl.status by themselves
     int64_t bin_rows[NCLASS] = {};  // rows per internal class of the last symbolic pass
     // outer-product form: what the last symbolic pass decided
     int64_t outer_products = 0;
@@ -157,9 +159,9 @@ bool is_pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
 // ---- scratch layout ------------------------------------------------------------------------
 struct Layout {
-    size_t ctl, ub, rowptr_raw, cnt, jmin, jmax, cls, perm, bm_off, warp_rows, row_unit0, unit_row, block_sums,
-        fpos, sflags, spos, bw_long, bw, brow, extra, rest, fixed_end;
+    size_t ctl, ub, rowptr_raw, cnt, jmin, jmax, cls, perm, bm_off, warp_rows, row_unit0, unit_row, look, sfp, bw_long, bw, brow, extra, rest, fixed_end;
     bool has_brow;
+    int n_look;
     int unit_cap;
     int bw_long_cap;            // 0: no word lists for this B
     int dense_smem_words;
@@ -190,13 +192,9 @@ Layout make_layout(const spws_plan_s* p, int64_t m, int64_t ncols, int64_t n_i, 
     int64_t words = (span_cap + 31) / 32 + 1;
     if (words > DENSE_MAX_SPAN_WORDS) words = DENSE_MAX_SPAN_WORDS;
     L.dense_smem_words = (int)((words + 7) & ~7ll);
-    const size_t longest = (size_t)(m > n_i ? m : n_i);
-    L.block_sums = take(16 * (longest / 2048 + 2));     // two arrays for the 3-tensor form's paired scan
-    if (p->kind == 1) {
-        L.fpos = take(8 * ((size_t)m + 1));
-        L.sflags = take(4 * (size_t)n_i);
-        L.spos = take(8 * ((size_t)n_i + 1));
-    }
+    L.n_look = (int)look_words(m, n_i);
+    L.look = take(8 * (size_t)L.n_look);
+    if (p->kind == 1) L.sfp = take(8 * ((size_t)n_i + 1));
     // word lists of long B rows (dense routes): one 8-byte slot per entry of B, used only at the
     // positions of rows with at least BW_MIN_LEN entries
     if (p->policy != SPWS_SPARSE_ISM && p->policy != SPWS_HASH && nnzB >= BW_MIN_LEN && nnzB <= BW_MAX_NNZ) {
@@ -339,6 +337,9 @@ LaunchCtx make_ctx(const spws_plan_s* p, char* scratch, size_t scratch_bytes, co
         c.bw_long_cap = L.bw_long_cap;
     }
     if (L.has_brow) c.brow = reinterpret_cast<int4*>(scratch + L.brow);
+    c.host_ctl = p->host_ctl;
+    c.look = reinterpret_cast<u64*>(scratch + L.look);
+    c.n_look = L.n_look;
     return c;
 }
 
@@ -372,24 +373,30 @@ inline void mark_start(spws_plan_s* p, int pass) {
 
 // ---- the row-wise passes: every output row (fibre) through the workspace of its class ------------
 // `ttmA` / `ttmC`: the 3-tensor operand and result, whose upper levels are rebuilt (null for the matrix
-// forms).  `c` is make_ctx of the layout; the control block has been cleared.  On success the plan
-// holds the statistics and what the numeric pass needs.
-spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L, LaunchCtx& c, const spws_tensor_t* ttmA, spws_tensor_t* ttmC,
-                            i64* rowptr, char* sc) {
+// forms).  `c` is make_ctx of the layout; clear_ctl: the control block is not in use yet.  On success
+// the plan holds the statistics and what the numeric pass needs.
+spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L, LaunchCtx& c, bool clear_ctl, const spws_tensor_t* ttmA,
+                            spws_tensor_t* ttmC, i64* rowptr, char* sc) {
     cudaStream_t stream = c.stream;
     // a1: upper bounds + classes; a2: binning
-    CUDA_TRY(launch_row_bounds(c, S.A, S.B, S.nnzA));
-    CUDA_TRY(launch_bw_build(c, S.B));
+    CUDA_TRY(launch_row_bounds(c, S.A, S.B, S.nnzA, clear_ctl));
     mark(plan, SPWS_T_SYM_BOUNDS);
     CUDA_TRY(launch_bin_rows(c, (int)S.m));
     mark(plan, SPWS_T_SYM_BIN);
-    // the class sizes come back now, so that only the workspaces that have rows are launched, with
-    // grids sized for them (a launch for an empty class costs as much as a small class's work)
-    int* hcount = plan->host_ctl->class_count;
-    CUDA_TRY(cudaMemcpyAsync(hcount, c.ctl->class_count, sizeof(int) * NCLASS, cudaMemcpyDeviceToHost, stream));
-    CUDA_TRY(cudaMemcpyAsync(&plan->host_ctl->max_ub_smem, &c.ctl->max_ub_smem, sizeof(i64), cudaMemcpyDeviceToHost, stream));
+    // the class sizes come back now (written to pinned memory by the binning kernel), so that only the
+    // workspaces that have rows are launched, with grids sized for them (a launch for an empty class
+    // costs as much as a small class's work)
     CUDA_TRY(cudaStreamSynchronize(stream));
-    plan->max_ub_smem = plan->host_ctl->max_ub_smem;
+    const DevCtl& hc = *plan->host_ctl;
+    if (hc.status != 0) {
+        plan->stats = spws_stats_t{};
+        plan->stats.device_status = hc.status;
+        return from_dev_status(hc.status);
+    }
+    int hcount[NCLASS];
+    for (int k = 0; k < NCLASS; ++k) hcount[k] = hc.class_count[k];
+    const bool any_dense = hcount[CLS_DENSE_WARP] + hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0;
+    plan->max_ub_smem = hc.max_ub_smem;
     c.max_ub_smem = plan->max_ub_smem;
     // a3: exact count per row through the workspace of its class
     if (S.m > 0) {
@@ -411,6 +418,7 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
             mark(plan, SPWS_T_SYM_DENSE_WARP);
         }
         if (hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0) {
+            CUDA_TRY(launch_bw_build(c, S.B));
             CUDA_TRY(launch_dense_sym_cta(c, S.A, S.B));
             mark(plan, SPWS_T_SYM_DENSE_CTA);
         }
@@ -424,22 +432,18 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
                 mark(plan, SPWS_T_SYM_HASH);
             }
     }
-    // a4: exclusive scan into the row pointer
-    if (ttmA) {
-        // with C's fibre and slice levels rebuilt from the fibres that produced an output
-        CUDA_TRY(launch_ttm_scan_compact(c, (int)S.n_i, (int)S.m, LL(ttmA->pos[1]), ttmA->crd[0], ttmA->crd[1], rowptr,
-                                         reinterpret_cast<i64*>(sc + L.fpos), reinterpret_cast<int*>(sc + L.sflags),
-                                         reinterpret_cast<i64*>(sc + L.spos), reinterpret_cast<i64*>(sc + L.block_sums), &c.ctl->nnz,
-                                         LL(ttmC->pos[0]), ttmC->crd[0], LL(ttmC->pos[1]), ttmC->crd[1], LL(ttmC->pos[2])));
-    } else {
-        CUDA_TRY(launch_scan_counts(c, c.tab.cnt, (int)S.m, rowptr, reinterpret_cast<i64*>(sc + L.block_sums), &c.ctl->nnz));
-    }
-    if (hcount[CLS_DENSE_WARP] + hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0) CUDA_TRY(launch_dense_rebin(c, (int)S.m, rowptr));
-    CUDA_TRY(launch_class_nnz(c, (int)S.m));
+    // a4: row pointer, numeric routing and (3-tensor form) C's upper levels, rebuilt from the fibres that
+    // produced an output
+    if (ttmA)
+        CUDA_TRY(launch_finish_fibres(c, (int)S.n_i, (int)S.m, any_dense, LL(ttmA->pos[1]), ttmA->crd[0], ttmA->crd[1], rowptr,
+                                      reinterpret_cast<i64*>(sc + L.sfp), LL(ttmC->pos[0]), ttmC->crd[0], LL(ttmC->pos[1]), ttmC->crd[1],
+                                      LL(ttmC->pos[2])));
+    else
+        CUDA_TRY(launch_finish_rows(c, (int)S.m, any_dense, rowptr));
     mark(plan, SPWS_T_SYM_SCAN);
-    CUDA_TRY(cudaMemcpyAsync(plan->host_ctl, c.ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, stream));
     CUDA_TRY(cudaStreamSynchronize(stream));
-    const DevCtl& hc = *plan->host_ctl;
+    plan->counters_clear = true;
+    plan->rows_path = true;
     plan->stats = spws_stats_t{};
     plan->stats.device_status = hc.status;
     if (hc.status != 0) return from_dev_status(hc.status);
@@ -465,7 +469,8 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
 }
 
 spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, const i64* rowptr, int* crd, void* val) {
-    CUDA_TRY(cudaMemsetAsync(c.ctl->work_counter, 0, sizeof(c.ctl->work_counter), c.stream));
+    if (!plan->counters_clear) CUDA_TRY(cudaMemsetAsync(c.ctl->work_counter, 0, sizeof(c.ctl->work_counter), c.stream));
+    plan->counters_clear = false;
     c.max_ub_smem = plan->max_ub_smem;
     const spws_stats_t& s = plan->stats;
     const int64_t* bins = plan->bin_rows;
@@ -682,7 +687,7 @@ spws_status_t rw_outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_
     CUDA_TRY(cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream));
     mark_start(plan, 0);
     CUDA_TRY(launch_rw_outer(c, S.A, S.nnzA, S.B, S.nnzB, label_bits_of(S.m, 1), rw_bufs(sc + w.L.extra, w.R)));
-    const spws_status_t st = rows_symbolic(plan, w.S, w.L, c, nullptr, nullptr, LL(C->pos[1]), sc);
+    const spws_status_t st = rows_symbolic(plan, w.S, w.L, c, false, nullptr, nullptr, LL(C->pos[1]), sc);
     if (st != SPWS_OK) return st;
     C->n[0] = C->dims[0];
     C->n[1] = plan->stats.nnz;
@@ -712,6 +717,7 @@ spws_status_t outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_t* 
     if (st != SPWS_OK) return st;
     plan->rowwise = rw_wanted(plan, I, J, S.nnzA, P);
     if (plan->rowwise) return rw_outer_symbolic(plan, S, C, scratch, scratch_bytes, sizes_out);
+    plan->rows_path = false;
     if (P > 0x7fff0000ll) return SPWS_INTERNAL_OVERFLOW;            // product ordinals and scans are 31-bit here
     const OuterLayout L = make_outer_layout(plan, I, K, J, P);
     if (scratch_bytes < L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
@@ -952,7 +958,7 @@ spws_status_t rw_higher_symbolic(spws_plan_s* plan, const HShapes& H, int64_t P,
         CUDA_TRY(launch_rw_fibre_rows(c, false, H.B, H.C, H.D, reinterpret_cast<int*>(x + w.R.fcnt), reinterpret_cast<i64*>(x + w.R.fpos),
                                       reinterpret_cast<int*>(x + w.R.fcrd), nullptr, reinterpret_cast<i64*>(x + w.R.block_sums)));
     CUDA_TRY(launch_rw_csf(c, H.form, H.B, (u64)(H.order == 3 ? H.odims[1] : 1), w.m, w.bits, rw_bufs(x, w.R)));
-    const spws_status_t st = rows_symbolic(plan, w.S, w.L, c, nullptr, nullptr, reinterpret_cast<i64*>(x + w.R.rowptr), sc);
+    const spws_status_t st = rows_symbolic(plan, w.S, w.L, c, false, nullptr, nullptr, reinterpret_cast<i64*>(x + w.R.rowptr), sc);
     if (st != SPWS_OK) return st;
     plan->stats.rows = H.B.nnz;
     plan->stats.products = P;
@@ -1021,6 +1027,7 @@ spws_status_t higher_symbolic(spws_plan_s* plan, const spws_tensor_t* B, const s
     if ((st = higher_count_products(plan, H, &P, &once)) != SPWS_OK) return st;
     plan->rowwise = rw_higher_wanted(plan, H, P);
     if (plan->rowwise) return rw_higher_symbolic(plan, H, P, once, Out, scratch, scratch_bytes, sizes_out);
+    plan->rows_path = false;
     if (P > 0x7fff0000ll || H.B.nnz > 0x7fff0000ll) return SPWS_INTERNAL_OVERFLOW;       // ordinals and scans are 31-bit here
     const HLayout L = make_hlayout(plan, H, P);
     if (scratch_bytes < L.end) return SPWS_SCRATCH_TOO_SMALL;
@@ -1286,14 +1293,12 @@ spws_status_t spws_workspace_size_exact(spws_plan_t plan, const spws_tensor_t* A
     char* sc = static_cast<char*>(scratch);
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, L);
     c.prm.bm_arena_words = ~0ull >> 3;          // reserve without a limit: only the total is wanted
-    CUDA_TRY(cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream));
-    CUDA_TRY(launch_row_bounds(c, S.A, S.B, S.nnzA));
+    CUDA_TRY(launch_row_bounds(c, S.A, S.B, S.nnzA, true));
     CUDA_TRY(launch_bin_rows(c, (int)S.m));
     if (row_products && S.m > 0)
         CUDA_TRY(cudaMemcpyAsync(row_products, c.tab.ub, 8 * (size_t)S.m, cudaMemcpyDeviceToDevice, c.stream));
-    CUDA_TRY(cudaMemcpyAsync(plan->host_ctl, c.ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, c.stream));
     CUDA_TRY(cudaStreamSynchronize(c.stream));
-    const DevCtl& hc = *plan->host_ctl;
+    const DevCtl& hc = *plan->host_ctl;         // published by the binning kernel
     if (hc.status != 0 && hc.status != DEV_SCRATCH_TOO_SMALL) return from_dev_status(hc.status);
     size_t need = L.fixed_end + align256((size_t)hc.bm_words_used * 4);
     const int64_t n_global = hc.class_count[CLS_ISM_GLOBAL];
@@ -1326,8 +1331,8 @@ spws_status_t spws_symbolic(spws_plan_t plan, const spws_tensor_t* A, const spws
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, L);
     cudaStream_t stream = c.stream;
 
-    CUDA_TRY(cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), stream));
     if (plan->opt.validate) {
+        CUDA_TRY(cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), stream));
         CUDA_TRY(launch_validate(c, S.A, S.B, S.nnzA, S.nnzB));
         CUDA_TRY(cudaMemcpyAsync(plan->host_ctl, c.ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, stream));
         CUDA_TRY(cudaStreamSynchronize(stream));
@@ -1335,7 +1340,7 @@ spws_status_t spws_symbolic(spws_plan_t plan, const spws_tensor_t* A, const spws
     }
     mark_start(plan, 0);
     i64* rowptr = (plan->kind == 0) ? LL(C->pos[1]) : reinterpret_cast<i64*>(sc + L.rowptr_raw);
-    if ((st = rows_symbolic(plan, S, L, c, plan->kind == 1 ? A : nullptr, C, rowptr, sc)) != SPWS_OK) return st;
+    if ((st = rows_symbolic(plan, S, L, c, !plan->opt.validate, plan->kind == 1 ? A : nullptr, C, rowptr, sc)) != SPWS_OK) return st;
     const DevCtl& hc = *plan->host_ctl;
     if (plan->kind == 0) {
         C->n[0] = C->dims[0];
@@ -1412,8 +1417,10 @@ spws_status_t spws_gather_ceiling(spws_plan_t plan, const spws_tensor_t* A, cons
 spws_status_t spws_get_stats(spws_plan_t plan, spws_stats_t* stats) {
     if (!plan || !stats) return SPWS_INVALID_ARGUMENT;
     if (!plan->symbolic_ok) return SPWS_BAD_SEQUENCE;
-    DevCtl* ctl = reinterpret_cast<DevCtl*>(plan->scratch);
-    CUDA_TRY(cudaMemcpyAsync(&plan->host_ctl->status, &ctl->status, sizeof(int), cudaMemcpyDeviceToHost, plan->h->stream));
+    if (!plan->rows_path) {
+        DevCtl* ctl = reinterpret_cast<DevCtl*>(plan->scratch);
+        CUDA_TRY(cudaMemcpyAsync(&plan->host_ctl->status, &ctl->status, sizeof(int), cudaMemcpyDeviceToHost, plan->h->stream));
+    }
     CUDA_TRY(cudaStreamSynchronize(plan->h->stream));
     plan->stats.device_status = plan->host_ctl->status;
     *stats = plan->stats;

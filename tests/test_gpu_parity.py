@@ -838,6 +838,28 @@ def test_ttm_many_slices_and_dropped_fibres(ctx, oracle_mod, slices):
     assert stats["rows"] > 2048
 
 
+@pytest.mark.parametrize("n", [1, 255, 257, 1023, 1025, 2047, 2048, 2049, 4097])
+def test_row_pointer_and_routing_at_tile_edges(ctx, oracle_mod, n):
+    """Rows (2048 per tile) and slices (1024 per tile) at the edges of the pass that builds the row pointer,
+    routes the dense rows and packs fibres and slices: every class of rows in one matrix, rows of
+    more than 2^17 products first in line, and a 3-tensor of n slices of which some drop out."""
+    rng = np.random.default_rng(n)
+    K = 700
+    B = random_csr(K, 6000, 0.01, n + 1, empty_row_frac=0.2)
+    wide = CSR(K, 6000, np.arange(K + 1) * 300, np.sort(rng.integers(0, 20, (K, 300)) + 20 * np.arange(300), axis=1).astype(np.int32).reshape(-1),
+               rng.uniform(-1, 1, K * 300))
+    per = rng.choice([0, 1, 2, 5, 40], size=n, p=[0.2, 0.3, 0.3, 0.15, 0.05])
+    per[n // 2] = 650
+    cols = [np.sort(rng.choice(K, p, replace=False)) for p in per]
+    pos = np.concatenate([[0], np.cumsum(per)]).astype(np.int64)
+    A = CSR(n, K, pos, np.concatenate(cols).astype(np.int32), rng.uniform(-1, 1, int(pos[-1])))
+    for M in (B, wide):
+        for policy in ("auto", "dense"):
+            check_spgemm(ctx, oracle_mod, A, M, policy)
+    T = uniform_csf3((n, 30, K), min(3 * n, 30 * K * n), n)
+    check_ttm(ctx, oracle_mod, T, random_csr(K, 400, 0.02, n, empty_row_frac=0.5), "auto")
+
+
 def test_ttm_equals_spgemm_of_the_fibre_matrix(ctx):
     """Hoisting the shared outer loops turns the 3-tensor form into the matrix form over the (i,j)
     fibres: the last CSF level of the TTM result must equal the CSR result of the fibre matrix times
