@@ -85,25 +85,29 @@ class Context:
         return B_.Plan(self.handle, expr, fmts, dtype, policy, **options)
 
     def exact_scratch_bytes(self, plan: B_.Plan, a: B_.TensorArrays, b: B_.TensorArrays, row_products: torch.Tensor | None = None) -> int:
-        """Bytes the two passes really use for these operands (one sizing pass on the device; the
-        result is remembered per plan and operand pair).  `row_products` (int64, one per row)
-        receives the per-row product counts when given."""
-        ptrs = lambda t: tuple(x.data_ptr() for x in list(t.pos) + list(t.crd) if x is not None)
-        key = (ptrs(a), ptrs(b), tuple(a.n), tuple(b.n))
-        cache = plan.__dict__.setdefault("_exact_bytes", {})
-        if key in cache and row_products is None:
-            return cache[key]
+        """Bytes the two passes really use for these operands (one sizing pass on the device).
+        `row_products` (int64, one per row) receives the per-row product counts when given."""
         own = plan.workspace_size_exact(a, b)
         sc = self.scratch(own)
-        cache[key] = plan.workspace_size_exact(a, b, self._aligned_ptr(sc), own,
-                                               row_products.data_ptr() if row_products is not None else None)
-        return cache[key]
+        return plan.workspace_size_exact(a, b, self._aligned_ptr(sc), own, row_products.data_ptr() if row_products is not None else None)
 
     def scratch(self, nbytes: int) -> torch.Tensor:
         if self._scratch is None or self._scratch.numel() < nbytes:
             self._scratch = None
             self._scratch = torch.empty(nbytes + 256, dtype=torch.uint8, device=self.device)
         return self._scratch
+
+    def _symbolic(self, plan: B_.Plan, a, b, c, d=None):
+        """The symbolic pass in the scratch at hand, which grows when the pass says so; returns
+        (scratch, bytes the passes use)."""
+        sc = self._scratch
+        while True:
+            ptr = self._aligned_ptr(sc) if sc is not None else None
+            done, nbytes = plan.symbolic_sized(a, b, c, ptr, sc.numel() - 256 if sc is not None else 0, d)
+            if done:
+                return sc, nbytes
+            sc = None
+            sc = self.scratch(nbytes)
 
     @staticmethod
     def _aligned_ptr(t: torch.Tensor) -> int:
@@ -112,11 +116,9 @@ class Context:
     # ------------------------------------------------------------------ SpGEMM
     def spgemm_symbolic(self, plan: B_.Plan, A: DeviceCSR, B: DeviceCSR):
         a, b = A.arrays(), B.arrays()
-        nbytes = self.exact_scratch_bytes(plan, a, b)
-        sc = self.scratch(nbytes)
         pos = torch.empty(A.nrows + 1, dtype=torch.int64, device=self.device)
         c = B_.csr_arrays(A.nrows, B.ncols, pos, None, None)
-        plan.symbolic(a, b, c, self._aligned_ptr(sc), nbytes)
+        sc, nbytes = self._symbolic(plan, a, b, c)
         return c, (a, b, sc, nbytes)
 
     def spgemm_numeric(self, plan: B_.Plan, c: B_.TensorArrays, state, crd=None, val=None) -> DeviceCSR:
@@ -155,11 +157,9 @@ class Context:
     def outer_symbolic(self, plan: B_.Plan, At: DeviceCSR, B: DeviceCSR):
         """Symbolic pass of C(i,j) = sum_k A(k,i) B(k,j); `At` holds A by its rows k (K x I)."""
         a, b = At.arrays(), B.arrays()
-        nbytes = plan.workspace_size(a, b)          # counts the products on the device
-        sc = self.scratch(nbytes)
         pos = torch.empty(At.ncols + 1, dtype=torch.int64, device=self.device)
         c = B_.csr_arrays(At.ncols, B.ncols, pos, None, None)
-        plan.symbolic(a, b, c, self._aligned_ptr(sc), nbytes)
+        sc, nbytes = self._symbolic(plan, a, b, c)
         return c, (a, b, sc, nbytes)
 
     def spgemm_outer(self, At: DeviceCSR, B: DeviceCSR, policy="auto", plan: B_.Plan | None = None, **options):
@@ -187,8 +187,6 @@ class Context:
         try:
             t, c = T.arrays(), C.arrays()
             d = D.arrays() if D is not None else None
-            nbytes = plan.workspace_size(t, c, d)
-            sc = self.scratch(nbytes)
             if expr == EXPR_SPMTTKRP:
                 order, dims = 2, (T.dims[2], C.ncols, 0)
             elif expr == EXPR_SPTTM:
@@ -196,7 +194,8 @@ class Context:
             else:
                 order, dims = 3, (T.dims[0], T.dims[2], C.ncols)
             out = B_.TensorArrays(order, dims, [None, None, None], [None, None, None], None, [0, 0, 0])
-            nnz = plan.symbolic(t, c, out, self._aligned_ptr(sc), nbytes, D=d)[0]
+            sc, nbytes = self._symbolic(plan, t, c, out, d)
+            nnz = out.n[0]
             crd = [torch.empty(nnz, dtype=torch.int32, device=self.device) for _ in range(order)]
             out.crd = crd + [None] * (3 - order)
             out.val = torch.empty(nnz, dtype=T.val.dtype, device=self.device)
@@ -211,8 +210,6 @@ class Context:
         """Symbolic pass of the 3-tensor form: allocates C's upper levels (bounded by A's) and returns
         (C arrays with sizes filled in, state for ttm_numeric)."""
         a, b = A.arrays(), B.arrays()
-        nbytes = self.exact_scratch_bytes(plan, a, b)
-        sc = self.scratch(nbytes)
         n_i, n_ij = a.n[0], a.n[1]
         i64, i32, dev = torch.int64, torch.int32, self.device
         pos0 = torch.empty(2, dtype=i64, device=dev)
@@ -222,8 +219,8 @@ class Context:
         pos2 = torch.empty(n_ij + 1, dtype=i64, device=dev)
         c = B_.TensorArrays(3, (A.dims[0], A.dims[1], B.ncols), [pos0, pos1, pos2], [crd0, crd1, None], None,
                             [n_i, n_ij, 0])
-        sizes = plan.symbolic(a, b, c, self._aligned_ptr(sc), nbytes)
-        return c, (a, b, sc, nbytes, sizes)
+        sc, nbytes = self._symbolic(plan, a, b, c)
+        return c, (a, b, sc, nbytes, c.n)
 
     def ttm_numeric(self, plan: B_.Plan, c: B_.TensorArrays, state, crd=None, val=None) -> DeviceCSF3:
         a, b, sc, nbytes, sizes = state

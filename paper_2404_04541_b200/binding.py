@@ -35,7 +35,7 @@ EXPORTS = ("spws_create", "spws_destroy", "spws_set_stream", "spws_plan_create",
            "spws_check_expression", "spws_workspace_size", "spws_workspace_size_exact", "spws_symbolic", "spws_numeric",
            "spws_get_stats", "spws_set_profiling", "spws_get_timings", "spws_execute_host", "spws_gather_ceiling",
            "spws_row_pointer_static", "spws_status_string", "spws_plan_create3", "spws_workspace_size3", "spws_symbolic3",
-           "spws_numeric3")
+           "spws_numeric3", "spws_symbolic_sized")
 STATIC_MAX_ROWS = 16777216
 TIMING_GROUPS = ("sym_bounds", "sym_bin", "sym_ism_reg", "sym_ism_smem_s", "sym_ism_smem", "sym_dense_warp",
                  "sym_dense_cta", "sym_ism_global", "sym_hash", "sym_scan", "num_ism_reg", "num_ism_smem_s", "num_ism_smem",
@@ -94,6 +94,7 @@ def lib():
         L.spws_plan_create3.argtypes = L.spws_plan_create.argtypes
         L.spws_workspace_size3.argtypes = [vp, T, T, T, ctypes.POINTER(sz)]
         L.spws_symbolic3.argtypes = [vp, T, T, T, T, vp, sz, ctypes.POINTER(ctypes.c_int64)]
+        L.spws_symbolic_sized.argtypes = [vp, T, T, T, T, vp, sz, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(sz)]
         L.spws_numeric3.argtypes = [vp, T, T, T, T, vp, sz]
         L.spws_plan_destroy.argtypes = [vp]
         L.spws_check_expression.argtypes = [ctypes.c_char_p, ctypes.POINTER(i32), ctypes.POINTER(i32)]
@@ -146,7 +147,7 @@ def _ptr(t):
         return None
     if isinstance(t, np.ndarray):
         return t.ctypes.data if t.size else None
-    return t.data_ptr() if t.numel() else None
+    return t.data_ptr() or None             # (a tensor without elements has no storage)
 
 
 @dataclass
@@ -161,15 +162,9 @@ class TensorArrays:
     n: list = field(default_factory=lambda: [0, 0, 0])
 
     def c_struct(self) -> spws_tensor_t:
-        t = spws_tensor_t()
-        t.order = self.order
-        for a in range(3):
-            t.dims[a] = int(self.dims[a]) if a < len(self.dims) else 0
-            t.n[a] = int(self.n[a])
-            t.pos[a] = _ptr(self.pos[a]) if a < len(self.pos) else None
-            t.crd[a] = _ptr(self.crd[a]) if a < len(self.crd) else None
-        t.val = _ptr(self.val)
-        return t
+        d, n, pos, crd = self.dims, self.n, self.pos, self.crd
+        return spws_tensor_t(self.order, 0, (int(d[0]), int(d[1]), int(d[2]) if len(d) > 2 else 0), (int(n[0]), int(n[1]), int(n[2])),
+                             (_ptr(pos[0]), _ptr(pos[1]), _ptr(pos[2])), (_ptr(crd[0]), _ptr(crd[1]), _ptr(crd[2])), _ptr(self.val))
 
 
 def csr_arrays(nrows, ncols, pos, crd, val) -> TensorArrays:
@@ -257,6 +252,21 @@ class Plan:
                                         ctypes.c_void_p(scratch_ptr), scratch_bytes, sizes), "spws_symbolic3")
         C.n = [int(sizes[0]), int(sizes[1]), int(sizes[2])]
         return C.n
+
+    def symbolic_sized(self, A, B, C, scratch_ptr, scratch_bytes: int, D=None):
+        """spws_symbolic_sized: (True, bytes the passes use) with C's sizes filled in, or (False, bytes to try
+        next) when the scratch is too small."""
+        a, b, c = A.c_struct(), B.c_struct(), C.c_struct()
+        d = ctypes.byref(D.c_struct()) if D is not None else None
+        sizes = (ctypes.c_int64 * 3)()
+        need = ctypes.c_size_t(0)
+        st = lib().spws_symbolic_sized(self._p, ctypes.byref(a), ctypes.byref(b), d, ctypes.byref(c), scratch_ptr, scratch_bytes, sizes,
+                                       ctypes.byref(need))
+        if st == SPWS_SCRATCH_TOO_SMALL and need.value > scratch_bytes:
+            return False, need.value
+        _check(st, "spws_symbolic")
+        C.n = list(sizes)
+        return True, need.value
 
     def numeric(self, A, B, C, scratch_ptr: int, scratch_bytes: int, D=None):
         a, b, c = A.c_struct(), B.c_struct(), C.c_struct()

@@ -344,6 +344,9 @@ struct LaunchCtx {
     mutable int launches;    // kernels enqueued through this context
 };
 
+// Blocks of `kernel` that fit one SM with `smem` bytes of dynamic shared memory, for which the kernel is made ready.
+cudaError_t resident_blocks(const void* kernel, int threads, size_t smem, int* per_sm);
+
 // setup.cu
 cudaError_t launch_validate(const LaunchCtx& c, const Csr& A, const Csr& B, i64 nnzA, i64 nnzB);
 // clear_ctl: the control block is cleared by the first kernel

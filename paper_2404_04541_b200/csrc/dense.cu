@@ -810,7 +810,7 @@ static int persistent_grid(const LaunchCtx& c, int per_sm, i64 work) {
 
 cudaError_t launch_dense_sym_warp(const LaunchCtx& c, const Csr& A, const Csr& B) {
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dense_sym_warp_kernel, DW_THREADS, 0);
+    cudaError_t e = resident_blocks((const void*)dense_sym_warp_kernel, DW_THREADS, 0, &per_sm);
     if (e != cudaSuccess) return e;
     dense_sym_warp_kernel<<<persistent_grid(c, per_sm, -1), DW_THREADS, 0, c.stream>>>(c.ctl, A, B, c.tab);
     ++c.launches;
@@ -821,8 +821,7 @@ cudaError_t launch_dense_sym_cta(const LaunchCtx& c, const Csr& A, const Csr& B)
     const size_t smem = (size_t)c.dense_smem_words * 4 + (size_t)(c.dense_smem_words / 32 + 1) * 4;
     cudaError_t e;
     int per_sm = 0;
-    if ((e = cudaFuncSetAttribute(dense_sym_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dense_sym_cta_kernel, DC_THREADS, smem)) != cudaSuccess) return e;
+    if ((e = resident_blocks((const void*)dense_sym_cta_kernel, DC_THREADS, smem, &per_sm)) != cudaSuccess) return e;
     dense_sym_cta_kernel<<<persistent_grid(c, per_sm, -1), DC_THREADS, smem, c.stream>>>(c.ctl, c.dense_smem_words, A, B, c.tab, c.bw);
     ++c.launches;
     return cudaGetLastError();
@@ -835,8 +834,7 @@ static cudaError_t num_warp_t(const LaunchCtx& c, int n_host, int bmw, int accw,
     const size_t smem = (size_t)DW_WARPS * (sizeof(T) * (size_t)accw + 8 * (size_t)bmw);
     cudaError_t e;
     auto k = dense_num_warp_kernel<T, CEIL>;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, DW_THREADS, smem)) != cudaSuccess) return e;
+    if ((e = resident_blocks((const void*)k, DW_THREADS, smem, &per_sm)) != cudaSuccess) return e;
     const i64 work = n_host >= 0 ? ((i64)n_host + DW_WARPS - 1) / DW_WARPS : -1;
     k<<<persistent_grid(c, per_sm, work), DW_THREADS, smem, c.stream>>>(c.ctl, bmw, accw, A, B, c.tab, rowptr, Ccrd, (T*)Cval, chk_idx, chk_val);
     ++c.launches;
@@ -867,12 +865,11 @@ static cudaError_t num_cta_t(const LaunchCtx& c, int phase, int n_units_host, in
     cudaError_t e;
     int per_sm = 0;
     auto k = dense_num_cta_kernel<T, CEIL>;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, DN_THREADS, smem)) != cudaSuccess) return e;
+    if ((e = resident_blocks((const void*)k, DN_THREADS, smem, &per_sm)) != cudaSuccess) return e;
     if (phase == 0) {
         // units are dealt out dynamically, so the grid is what is resident at once
         int emit_per_sm = 0;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&emit_per_sm, dense_emit_crd_kernel<T>, DE_THREADS, 0)) != cudaSuccess) return e;
+        if ((e = resident_blocks((const void*)dense_emit_crd_kernel<T>, DE_THREADS, 0, &emit_per_sm)) != cudaSuccess) return e;
         const i64 work = n_units_host >= 0 ? ((i64)n_units_host + DE_WARPS - 1) / DE_WARPS : -1;
         dense_emit_crd_kernel<T><<<persistent_grid(c, emit_per_sm, work), DE_THREADS, 0, c.stream>>>(c.ctl, unit_products, c.tab, rowptr, Ccrd, (T*)Cval);
     } else {

@@ -175,8 +175,7 @@ static cudaError_t hash_launch_k(const LaunchCtx& c, int cls, int n_host, const 
     cudaError_t e;
     int per_sm = 0;
     auto k = hash_kernel<T, CAP, THREADS, NUMERIC>;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, THREADS, smem)) != cudaSuccess) return e;
+    if ((e = resident_blocks((const void*)k, THREADS, smem, &per_sm)) != cudaSuccess) return e;
     i64 grid = (i64)c.sm_count * (per_sm > 0 ? per_sm : 1);
     if (n_host >= 0 && n_host < grid) grid = n_host > 0 ? n_host : 1;
     k<<<(int)grid, THREADS, smem, c.stream>>>(c.tab.perm, c.ctl, cls, slot, ism ? (i64)ISM_WARP_MAX : 0, A, B, c.tab.ub, c.tab.cnt, rowptr, Ccrd, (T*)Cval);

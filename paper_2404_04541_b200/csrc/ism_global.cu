@@ -248,16 +248,17 @@ static cudaError_t launch_t(const LaunchCtx& c, bool numeric, int n_host, const 
                         sizeof(int) * (3 * GL_CAPMAX + 1 + GL_THREADS + 1 + 33) + 16;
     const int slot = CLS_ISM_GLOBAL + (numeric ? NUM_SLOT : 0);
     cudaError_t e;
+    int per_sm = 0;
     i64 grid = (i64)c.sm_count * 2;
     if (n_host >= 0 && n_host < grid) grid = n_host > 0 ? n_host : 1;
     if (numeric) {
         auto k = ism_global_kernel<T, true>;
-        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+        if ((e = resident_blocks((const void*)k, GL_THREADS, smem, &per_sm)) != cudaSuccess) return e;
         k<<<(int)grid, GL_THREADS, smem, c.stream>>>(c.tab.perm, c.ctl, slot, c.global_cap, c.rest, c.rest_bytes,
                                                     A, B, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
     } else {
         auto k = ism_global_kernel<T, false>;
-        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+        if ((e = resident_blocks((const void*)k, GL_THREADS, smem, &per_sm)) != cudaSuccess) return e;
         k<<<(int)grid, GL_THREADS, smem, c.stream>>>(c.tab.perm, c.ctl, slot, c.global_cap, c.rest, c.rest_bytes,
                                                     A, B, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
     }

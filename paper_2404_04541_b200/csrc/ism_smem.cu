@@ -363,8 +363,7 @@ static cudaError_t launch_k(const LaunchCtx& c, int cls, int n_host, const Csr& 
     cudaError_t e;
     int per_sm = 0;
     auto k = ism_smem_kernel<T, P, CAP, THREADS, NUMERIC>;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, THREADS, smem)) != cudaSuccess) return e;
+    if ((e = resident_blocks((const void*)k, THREADS, smem, &per_sm)) != cudaSuccess) return e;
     i64 grid = (i64)c.sm_count * (per_sm > 0 ? per_sm : 1);
     if (n_host >= 0 && n_host < grid) grid = n_host > 0 ? n_host : 1;
     k<<<(int)grid, THREADS, smem, c.stream>>>(c.tab.perm, c.ctl, cls, slot, (i64)ISM_WARP_MAX, A, B, c.tab.ub, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
@@ -378,8 +377,7 @@ static cudaError_t launch_warp_k(const LaunchCtx& c, int cls, int n_host, const 
     cudaError_t e;
     int per_sm = 0;
     auto k = ism_warp_kernel<T, P, CAP, NUMERIC>;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, IW_WARPS * 32, smem)) != cudaSuccess) return e;
+    if ((e = resident_blocks((const void*)k, IW_WARPS * 32, smem, &per_sm)) != cudaSuccess) return e;
     i64 grid = (i64)c.sm_count * (per_sm > 0 ? per_sm : 1);
     const i64 want = n_host >= 0 ? ((i64)n_host + IW_WARPS - 1) / IW_WARPS : grid;
     if (want < grid) grid = want > 0 ? want : 1;

@@ -4,6 +4,8 @@
 #include <cctype>
 #include <cstdio>
 #include <cstring>
+#include <memory>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -13,7 +15,44 @@
 
 using namespace spws;
 
+// Pinned blocks of closed plans, kept for the next plan of the same handle (pinning memory costs more than a
+// small product): eight at most, given back with the last plan or handle that refers to the pool.
+struct PinnedPool {
+    std::mutex lock;
+    std::vector<HostBlock*> spare;
+    HostBlock* take() {
+        {
+            std::lock_guard<std::mutex> hold(lock);
+            if (!spare.empty()) {
+                HostBlock* b = spare.back();
+                spare.pop_back();
+                return b;
+            }
+        }
+        void* p = nullptr;
+        if (cudaMallocHost(&p, sizeof(HostBlock)) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return static_cast<HostBlock*>(p);
+    }
+    void give(HostBlock* b) {
+        {
+            std::lock_guard<std::mutex> hold(lock);
+            if (spare.size() < 8) {
+                spare.push_back(b);
+                return;
+            }
+        }
+        cudaFreeHost(b);
+    }
+    ~PinnedPool() {
+        for (HostBlock* b : spare) cudaFreeHost(b);
+    }
+};
+
 struct spws_handle_s {
+    std::shared_ptr<PinnedPool> pinned = std::make_shared<PinnedPool>();
     cudaStream_t stream = nullptr;
     int device = 0;
     int sm_count = 0;
@@ -25,7 +64,9 @@ struct spws_plan_s {
     int is_f64 = 1;
     int policy = SPWS_AUTO;
     spws_options_t opt{};
+    std::shared_ptr<PinnedPool> pool;
     HostBlock* host = nullptr;  // pinned
+    bool in_flight = false;     // kernels that may still write to the pinned block are enqueued
     DevCtl* host_ctl = nullptr; // &host->ctl
     bool symbolic_ok = false;
     spws_stats_t stats{};
@@ -50,6 +91,33 @@ struct spws_plan_s {
     bool ev_ran[SPWS_T_COUNT] = {};
     bool ev_pass[3] = {};
 };
+
+namespace spws {
+
+cudaError_t resident_blocks(const void* kernel, int threads, size_t smem, int* per_sm) {
+    struct Known { const void* kernel; size_t smem; int device, threads, per_sm; };
+    static thread_local std::vector<Known> known;
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    for (const Known& k : known)
+        if (k.kernel == kernel && k.smem == smem && k.threads == threads && k.device == device) {
+            *per_sm = k.per_sm;
+            return cudaSuccess;
+        }
+    // the limit is raised to all the device has, the same for every caller, so that no thread undoes another's
+    cudaFuncAttributes fa;
+    int most = 0;
+    if ((e = cudaFuncGetAttributes(&fa, kernel)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device)) != cudaSuccess) return e;
+    if (smem > 0 && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kernel, threads, smem)) != cudaSuccess) return e;
+    if (known.size() >= 256) known.clear();
+    known.push_back(Known{kernel, smem, device, threads, *per_sm});
+    return cudaSuccess;
+}
+
+}  // namespace spws
 
 namespace {
 
@@ -371,13 +439,35 @@ inline void mark_start(spws_plan_s* p, int pass) {
     p->ev_pass[pass] = true;
 }
 
+// What both passes use, known once the rows are binned: the fixed tables, the bitmaps of exactly the dense rows,
+// and the slots of the global-memory ISM, sized for its largest row.
+size_t rows_need(const spws_plan_s* plan, const Layout& L, const DevCtl& hc, int64_t ncols) {
+    size_t need = L.fixed_end + align256((size_t)hc.bm_words_used * 4);
+    const int64_t n_global = hc.class_count[CLS_ISM_GLOBAL];
+    if (n_global > 0) {
+        int64_t elems = hc.max_ub_global < ncols ? hc.max_ub_global : ncols;
+        elems = (elems + 63) & ~63ll;
+        const size_t comp = 4 + (plan->is_f64 ? 8 : 4);
+        const size_t slot = align256(2 * (size_t)elems * comp);
+        need += slot * global_ism_slots(plan, slot, n_global);
+    }
+    return need;
+}
+
+// A first guess for a caller that has no scratch yet: the fixed tables and some room for bitmaps
+// (the fixed tables once more, 16 MiB at least), no more than the host-side upper bound.
+size_t rows_guess(const spws_plan_s* plan, const Layout& L, int64_t m, int64_t ncols) {
+    return L.fixed_end + std::min(rest_reserve(plan, m, ncols), std::max(L.fixed_end, (size_t)16 << 20));
+}
+
 // ---- the row-wise passes: every output row (fibre) through the workspace of its class ------------
 // `ttmA` / `ttmC`: the 3-tensor operand and result, whose upper levels are rebuilt (null for the matrix
 // forms).  `c` is make_ctx of the layout; clear_ctl: the control block is not in use yet.  On success
 // the plan holds the statistics and what the numeric pass needs.
-spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L, LaunchCtx& c, bool clear_ctl, const spws_tensor_t* ttmA,
+spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L, LaunchCtx& c, size_t scratch_bytes, size_t* needed, bool clear_ctl, const spws_tensor_t* ttmA,
                             spws_tensor_t* ttmC, i64* rowptr, char* sc) {
     cudaStream_t stream = c.stream;
+    plan->in_flight = true;
     // a1: upper bounds + classes; a2: binning
     CUDA_TRY(launch_row_bounds(c, S.A, S.B, S.nnzA, clear_ctl));
     mark(plan, SPWS_T_SYM_BOUNDS);
@@ -387,12 +477,18 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     // workspaces that have rows are launched, with grids sized for them (a launch for an empty class
     // costs as much as a small class's work)
     CUDA_TRY(cudaStreamSynchronize(stream));
+    plan->in_flight = false;
     const DevCtl& hc = *plan->host_ctl;
+    if (needed && (hc.status == 0 || hc.status == DEV_SCRATCH_TOO_SMALL)) {
+        *needed = rows_need(plan, L, hc, S.ncols);
+        if (scratch_bytes < *needed) return SPWS_SCRATCH_TOO_SMALL;
+    }
     if (hc.status != 0) {
         plan->stats = spws_stats_t{};
         plan->stats.device_status = hc.status;
         return from_dev_status(hc.status);
     }
+    plan->in_flight = true;
     int hcount[NCLASS];
     for (int k = 0; k < NCLASS; ++k) hcount[k] = hc.class_count[k];
     const bool any_dense = hcount[CLS_DENSE_WARP] + hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0;
@@ -442,6 +538,7 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
         CUDA_TRY(launch_finish_rows(c, (int)S.m, any_dense, rowptr));
     mark(plan, SPWS_T_SYM_SCAN);
     CUDA_TRY(cudaStreamSynchronize(stream));
+    plan->in_flight = false;
     plan->counters_clear = true;
     plan->rows_path = true;
     plan->stats = spws_stats_t{};
@@ -469,6 +566,7 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
 }
 
 spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, const i64* rowptr, int* crd, void* val) {
+    plan->in_flight = true;
     if (!plan->counters_clear) CUDA_TRY(cudaMemsetAsync(c.ctl->work_counter, 0, sizeof(c.ctl->work_counter), c.stream));
     plan->counters_clear = false;
     c.max_ub_smem = plan->max_ub_smem;
@@ -563,8 +661,10 @@ spws_status_t count_products(spws_plan_s* p, Launch launch, int64_t* P, int64_t*
     c.stream = p->h->stream;
     c.sm_count = p->h->sm_count;
     memset(p->host->partial, 0, sizeof(p->host->partial));
+    p->in_flight = true;
     CUDA_TRY(launch(c, p->host->partial));
     CUDA_TRY(cudaStreamSynchronize(c.stream));
+    p->in_flight = false;
     u64 total = 0, total2 = 0;
     for (int b = 0; b < COUNT_BLOCKS; ++b) { total += p->host->partial[b]; total2 += p->host->partial[COUNT_BLOCKS + b]; }
     *P = (int64_t)total;
@@ -651,6 +751,14 @@ size_t rw_arena_bound(const spws_plan_s* p, int64_t m, int64_t ncols, int64_t P)
     return align256((size_t)(words * 4.0) + 256);
 }
 
+size_t outer_need(const spws_plan_s* p, const OuterLayout& L, int64_t I, int64_t J, int64_t P) {
+    const double cells = (double)I * (double)J;
+    const size_t dense_ok = cells <= 2.0e9 ? L.dense_end : 0;      // a dense workspace beyond 2^31 cells is never offered
+    if (p->policy == SPWS_SPARSE_ISM || p->policy == SPWS_HASH) return L.ism_end;
+    if (p->policy == SPWS_DENSE) return L.dense_end;
+    return std::max(L.ism_end, (cells <= 134217728.0 || (double)P * 16.0 >= cells) ? dense_ok : (size_t)0);
+}
+
 bool outer_wants_dense(const spws_plan_s* p, int64_t I, int64_t J, int64_t P, size_t scratch_bytes, const OuterLayout& L, spws_status_t* st) {
     *st = SPWS_OK;
     const bool fits = scratch_bytes >= L.dense_end;
@@ -679,15 +787,18 @@ RwOuter rw_outer_layout(const spws_plan_s* p, const Shapes& S, char* sc) {
     return w;
 }
 
-spws_status_t rw_outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_t* C, void* scratch, size_t scratch_bytes, int64_t* sizes_out) {
+spws_status_t rw_outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_t* C, void* scratch, size_t scratch_bytes, int64_t* sizes_out,
+                                size_t* needed) {
     char* sc = static_cast<char*>(scratch);
     const RwOuter w = rw_outer_layout(plan, S, sc);
+    if (needed) *needed = rows_guess(plan, w.L, S.m, S.ncols);
     if (scratch_bytes < w.L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, w.L);
+    plan->in_flight = true;
     CUDA_TRY(cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream));
     mark_start(plan, 0);
     CUDA_TRY(launch_rw_outer(c, S.A, S.nnzA, S.B, S.nnzB, label_bits_of(S.m, 1), rw_bufs(sc + w.L.extra, w.R)));
-    const spws_status_t st = rows_symbolic(plan, w.S, w.L, c, false, nullptr, nullptr, LL(C->pos[1]), sc);
+    const spws_status_t st = rows_symbolic(plan, w.S, w.L, c, scratch_bytes, needed, false, nullptr, nullptr, LL(C->pos[1]), sc);
     if (st != SPWS_OK) return st;
     C->n[0] = C->dims[0];
     C->n[1] = plan->stats.nnz;
@@ -709,22 +820,28 @@ spws_status_t rw_outer_numeric(spws_plan_s* plan, const Shapes& S, spws_tensor_t
     return rows_numeric(plan, w.S, c, LL(C->pos[1]), C->crd[1], C->val);
 }
 
-spws_status_t outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_t* C, void* scratch, size_t scratch_bytes, int64_t* sizes_out) {
+spws_status_t outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_t* C, void* scratch, size_t scratch_bytes, int64_t* sizes_out,
+                             size_t* needed) {
     const int64_t I = S.m, K = S.k, J = S.ncols;
     if (I * J < 0 || (I > 0 && J > (int64_t)(0x7fffffffffffffffll / (I > 0 ? I : 1)))) return SPWS_INVALID_ARGUMENT;
     int64_t P = 0;
     spws_status_t st = outer_count_products(plan, S, &P);
     if (st != SPWS_OK) return st;
     plan->rowwise = rw_wanted(plan, I, J, S.nnzA, P);
-    if (plan->rowwise) return rw_outer_symbolic(plan, S, C, scratch, scratch_bytes, sizes_out);
+    if (plan->rowwise) return rw_outer_symbolic(plan, S, C, scratch, scratch_bytes, sizes_out, needed);
     plan->rows_path = false;
     if (P > 0x7fff0000ll) return SPWS_INTERNAL_OVERFLOW;            // product ordinals and scans are 31-bit here
     const OuterLayout L = make_outer_layout(plan, I, K, J, P);
+    if (needed) {
+        *needed = outer_need(plan, L, I, J, P);
+        if (scratch_bytes < *needed) return SPWS_SCRATCH_TOO_SMALL;
+    }
     if (scratch_bytes < L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
     const bool dense = outer_wants_dense(plan, I, J, P, scratch_bytes, L, &st);
     if (st != SPWS_OK) return st;
     if (!dense && scratch_bytes < L.ism_end) return SPWS_SCRATCH_TOO_SMALL;
     char* sc = static_cast<char*>(scratch);
+    plan->in_flight = true;
     LaunchCtx c{};
     c.stream = plan->h->stream;
     c.sm_count = plan->h->sm_count;
@@ -791,6 +908,7 @@ spws_status_t outer_numeric(spws_plan_s* plan, const Shapes& S, spws_tensor_t* C
     if (plan->rowwise) return rw_outer_numeric(plan, S, C, scratch, scratch_bytes);
     const OuterLayout L = make_outer_layout(plan, I, K, J, P);
     if (scratch_bytes < (plan->outer_dense ? L.dense_end : L.ism_end)) return SPWS_SCRATCH_TOO_SMALL;
+    plan->in_flight = true;
     char* sc = static_cast<char*>(scratch);
     LaunchCtx c{};
     c.stream = plan->h->stream;
@@ -946,19 +1064,21 @@ bool rw_higher_wanted(const spws_plan_s* p, const HShapes& H, int64_t P) {
 }
 
 spws_status_t rw_higher_symbolic(spws_plan_s* plan, const HShapes& H, int64_t P, int64_t once, spws_tensor_t* Out, void* scratch,
-                                 size_t scratch_bytes, int64_t* sizes_out) {
+                                 size_t scratch_bytes, int64_t* sizes_out, size_t* needed) {
     char* sc = static_cast<char*>(scratch);
     const RwHigher w = rw_higher_layout(plan, H, P, once, sc);
+    if (needed) *needed = rows_guess(plan, w.L, w.m, w.S.ncols);
     if (scratch_bytes < w.L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, w.L);
     char* x = sc + w.L.extra;
+    plan->in_flight = true;
     CUDA_TRY(cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream));
     mark_start(plan, 0);
     if (H.form == 2)
         CUDA_TRY(launch_rw_fibre_rows(c, false, H.B, H.C, H.D, reinterpret_cast<int*>(x + w.R.fcnt), reinterpret_cast<i64*>(x + w.R.fpos),
                                       reinterpret_cast<int*>(x + w.R.fcrd), nullptr, reinterpret_cast<i64*>(x + w.R.block_sums)));
     CUDA_TRY(launch_rw_csf(c, H.form, H.B, (u64)(H.order == 3 ? H.odims[1] : 1), w.m, w.bits, rw_bufs(x, w.R)));
-    const spws_status_t st = rows_symbolic(plan, w.S, w.L, c, false, nullptr, nullptr, reinterpret_cast<i64*>(x + w.R.rowptr), sc);
+    const spws_status_t st = rows_symbolic(plan, w.S, w.L, c, scratch_bytes, needed, false, nullptr, nullptr, reinterpret_cast<i64*>(x + w.R.rowptr), sc);
     if (st != SPWS_OK) return st;
     plan->stats.rows = H.B.nnz;
     plan->stats.products = P;
@@ -1016,21 +1136,24 @@ spws_status_t check_coo_output(const HShapes& H, const spws_tensor_t* Out) {
 }
 
 spws_status_t higher_symbolic(spws_plan_s* plan, const spws_tensor_t* B, const spws_tensor_t* C, const spws_tensor_t* D, spws_tensor_t* Out,
-                              void* scratch, size_t scratch_bytes, int64_t* sizes_out) {
+                              void* scratch, size_t scratch_bytes, int64_t* sizes_out, size_t* needed) {
     plan->symbolic_ok = false;
     HShapes H{};
     spws_status_t st = check_higher(plan, B, C, D, H, true);
     if (st != SPWS_OK) return st;
     if ((st = check_coo_output(H, Out)) != SPWS_OK) return st;
-    if (!scratch || (reinterpret_cast<uintptr_t>(scratch) & 255)) return SPWS_INVALID_ARGUMENT;
+    if ((!scratch && !needed) || (reinterpret_cast<uintptr_t>(scratch) & 255)) return SPWS_INVALID_ARGUMENT;
+    if (!scratch) scratch_bytes = 0;
     int64_t P = 0, once = 0;
     if ((st = higher_count_products(plan, H, &P, &once)) != SPWS_OK) return st;
     plan->rowwise = rw_higher_wanted(plan, H, P);
-    if (plan->rowwise) return rw_higher_symbolic(plan, H, P, once, Out, scratch, scratch_bytes, sizes_out);
+    if (plan->rowwise) return rw_higher_symbolic(plan, H, P, once, Out, scratch, scratch_bytes, sizes_out, needed);
     plan->rows_path = false;
     if (P > 0x7fff0000ll || H.B.nnz > 0x7fff0000ll) return SPWS_INTERNAL_OVERFLOW;       // ordinals and scans are 31-bit here
     const HLayout L = make_hlayout(plan, H, P);
+    if (needed) *needed = L.end;
     if (scratch_bytes < L.end) return SPWS_SCRATCH_TOO_SMALL;
+    plan->in_flight = true;
     char* sc = static_cast<char*>(scratch);
     LaunchCtx c{};
     c.stream = plan->h->stream;
@@ -1093,6 +1216,7 @@ spws_status_t higher_numeric(spws_plan_s* plan, const spws_tensor_t* B, const sp
     if (plan->rowwise) return rw_higher_numeric(plan, H, Out, scratch, scratch_bytes);
     const HLayout L = make_hlayout(plan, H, P);
     if (scratch_bytes < L.end) return SPWS_SCRATCH_TOO_SMALL;
+    plan->in_flight = true;
     char* sc = static_cast<char*>(scratch);
     LaunchCtx c{};
     c.stream = plan->h->stream;
@@ -1189,8 +1313,9 @@ static spws_status_t plan_create_n(spws_handle_t handle, const char* expr, const
     p->is_f64 = f64 ? 1 : 0;
     p->policy = (int)policy;
     p->opt = o;
-    if (cudaMallocHost(reinterpret_cast<void**>(&p->host), sizeof(HostBlock)) != cudaSuccess) {
-        cudaGetLastError();
+    p->pool = handle->pinned;
+    p->host = p->pool->take();
+    if (!p->host) {
         delete p;
         return SPWS_CUDA_ERROR;
     }
@@ -1244,7 +1369,9 @@ spws_status_t spws_plan_destroy(spws_plan_t plan) {
         for (int g = 0; g < SPWS_T_COUNT; ++g) cudaEventDestroy(plan->ev[g]);
         for (int g = 0; g < 3; ++g) cudaEventDestroy(plan->ev_start[g]);
     }
-    if (plan->host) cudaFreeHost(plan->host);
+    // with kernels still enqueued the block is freed (which waits for them) and not handed on
+    if (plan->in_flight) cudaFreeHost(plan->host);
+    else if (plan->host) plan->pool->give(plan->host);
     delete plan;
     return SPWS_OK;
 }
@@ -1264,10 +1391,7 @@ spws_status_t spws_workspace_size(spws_plan_t plan, const spws_tensor_t* A, cons
             return SPWS_OK;
         }
         const OuterLayout OL = make_outer_layout(plan, S.m, S.k, S.ncols, P);
-        const size_t dense_ok = (double)S.m * (double)S.ncols <= 2.0e9 ? OL.dense_end : 0;     // a dense workspace beyond 2^31 cells is never offered
-        *bytes = (plan->policy == SPWS_SPARSE_ISM || plan->policy == SPWS_HASH) ? OL.ism_end
-                 : plan->policy == SPWS_DENSE ? OL.dense_end
-                 : std::max(OL.ism_end, ((double)S.m * (double)S.ncols <= 134217728.0 || (double)P * 16.0 >= (double)S.m * (double)S.ncols) ? dense_ok : (size_t)0);
+        *bytes = outer_need(plan, OL, S.m, S.ncols, P);
         return SPWS_OK;
     }
     const Layout L = make_layout(plan, S.m, S.ncols, S.n_i, S.nnzB, S.k, S.nnzA);
@@ -1293,54 +1417,53 @@ spws_status_t spws_workspace_size_exact(spws_plan_t plan, const spws_tensor_t* A
     char* sc = static_cast<char*>(scratch);
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, L);
     c.prm.bm_arena_words = ~0ull >> 3;          // reserve without a limit: only the total is wanted
+    plan->in_flight = true;
     CUDA_TRY(launch_row_bounds(c, S.A, S.B, S.nnzA, true));
     CUDA_TRY(launch_bin_rows(c, (int)S.m));
     if (row_products && S.m > 0)
         CUDA_TRY(cudaMemcpyAsync(row_products, c.tab.ub, 8 * (size_t)S.m, cudaMemcpyDeviceToDevice, c.stream));
     CUDA_TRY(cudaStreamSynchronize(c.stream));
+    plan->in_flight = false;
     const DevCtl& hc = *plan->host_ctl;         // published by the binning kernel
     if (hc.status != 0 && hc.status != DEV_SCRATCH_TOO_SMALL) return from_dev_status(hc.status);
-    size_t need = L.fixed_end + align256((size_t)hc.bm_words_used * 4);
-    const int64_t n_global = hc.class_count[CLS_ISM_GLOBAL];
-    if (n_global > 0) {                         // numeric slots of the global-memory ISM, sized for its largest row
-        int64_t elems = hc.max_ub_global < S.ncols ? hc.max_ub_global : S.ncols;
-        elems = (elems + 63) & ~63ll;
-        const size_t comp = 4 + (plan->is_f64 ? 8 : 4);
-        const size_t slot = align256(2 * (size_t)elems * comp);
-        need += slot * global_ism_slots(plan, slot, n_global);
-    }
-    *bytes = need;
+    *bytes = rows_need(plan, L, hc, S.ncols);
     return SPWS_OK;
 }
 
-spws_status_t spws_symbolic(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, spws_tensor_t* C,
-                            void* scratch, size_t scratch_bytes, int64_t* sizes_out) {
+// needed (may be null): receives the scratch bytes the passes use, or a size to try next when they could not be learnt
+static spws_status_t symbolic_any(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, const spws_tensor_t* D, spws_tensor_t* C,
+                                  void* scratch, size_t scratch_bytes, int64_t* sizes_out, size_t* needed) {
     if (!plan) return SPWS_INVALID_ARGUMENT;
-    if (plan->kind == 5) return SPWS_INVALID_ARGUMENT;
-    if (plan->kind >= 3) return higher_symbolic(plan, A, B, nullptr, C, scratch, scratch_bytes, sizes_out);
+    if (needed) *needed = 0;
+    if ((plan->kind == 5) != (D != nullptr)) return SPWS_INVALID_ARGUMENT;
+    if (plan->kind >= 3) return higher_symbolic(plan, A, B, D, C, scratch, scratch_bytes, sizes_out, needed);
     plan->symbolic_ok = false;
     Shapes S{};
     spws_status_t st = check_operands(plan, A, B, S);
     if (st != SPWS_OK) return st;
     if ((st = check_output_dims(plan, A, B, C)) != SPWS_OK) return st;
-    if (!scratch || (reinterpret_cast<uintptr_t>(scratch) & 255)) return SPWS_INVALID_ARGUMENT;
-    if (plan->kind == 2) return outer_symbolic(plan, S, C, scratch, scratch_bytes, sizes_out);
+    if ((!scratch && !needed) || (reinterpret_cast<uintptr_t>(scratch) & 255)) return SPWS_INVALID_ARGUMENT;
+    if (!scratch) scratch_bytes = 0;
+    if (plan->kind == 2) return outer_symbolic(plan, S, C, scratch, scratch_bytes, sizes_out, needed);
     const Layout L = make_layout(plan, S.m, S.ncols, S.n_i, S.nnzB, S.k, S.nnzA);
+    if (needed) *needed = rows_guess(plan, L, S.m, S.ncols);
     if (scratch_bytes < L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
     char* sc = static_cast<char*>(scratch);
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, L);
     cudaStream_t stream = c.stream;
 
     if (plan->opt.validate) {
+        plan->in_flight = true;
         CUDA_TRY(cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), stream));
         CUDA_TRY(launch_validate(c, S.A, S.B, S.nnzA, S.nnzB));
         CUDA_TRY(cudaMemcpyAsync(plan->host_ctl, c.ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, stream));
         CUDA_TRY(cudaStreamSynchronize(stream));
+        plan->in_flight = false;
         if (plan->host_ctl->status != 0) return from_dev_status(plan->host_ctl->status);
     }
     mark_start(plan, 0);
     i64* rowptr = (plan->kind == 0) ? LL(C->pos[1]) : reinterpret_cast<i64*>(sc + L.rowptr_raw);
-    if ((st = rows_symbolic(plan, S, L, c, !plan->opt.validate, plan->kind == 1 ? A : nullptr, C, rowptr, sc)) != SPWS_OK) return st;
+    if ((st = rows_symbolic(plan, S, L, c, scratch_bytes, needed, !plan->opt.validate, plan->kind == 1 ? A : nullptr, C, rowptr, sc)) != SPWS_OK) return st;
     const DevCtl& hc = *plan->host_ctl;
     if (plan->kind == 0) {
         C->n[0] = C->dims[0];
@@ -1356,6 +1479,17 @@ spws_status_t spws_symbolic(spws_plan_t plan, const spws_tensor_t* A, const spws
     plan->m = S.m;
     plan->scratch = scratch;
     return SPWS_OK;
+}
+
+spws_status_t spws_symbolic(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, spws_tensor_t* C,
+                            void* scratch, size_t scratch_bytes, int64_t* sizes_out) {
+    return symbolic_any(plan, A, B, nullptr, C, scratch, scratch_bytes, sizes_out, nullptr);
+}
+
+spws_status_t spws_symbolic_sized(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, const spws_tensor_t* D, spws_tensor_t* C,
+                                  void* scratch, size_t scratch_bytes, int64_t* sizes_out, size_t* needed) {
+    if (!needed) return SPWS_INVALID_ARGUMENT;
+    return symbolic_any(plan, A, B, D, C, scratch, scratch_bytes, sizes_out, needed);
 }
 
 spws_status_t spws_numeric(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, spws_tensor_t* C,
@@ -1422,6 +1556,7 @@ spws_status_t spws_get_stats(spws_plan_t plan, spws_stats_t* stats) {
         CUDA_TRY(cudaMemcpyAsync(&plan->host_ctl->status, &ctl->status, sizeof(int), cudaMemcpyDeviceToHost, plan->h->stream));
     }
     CUDA_TRY(cudaStreamSynchronize(plan->h->stream));
+    plan->in_flight = false;
     plan->stats.device_status = plan->host_ctl->status;
     *stats = plan->stats;
     return from_dev_status(plan->host_ctl->status);
@@ -1434,8 +1569,8 @@ spws_status_t spws_workspace_size3(spws_plan_t plan, const spws_tensor_t* A, con
 
 spws_status_t spws_symbolic3(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, const spws_tensor_t* D, spws_tensor_t* C,
                              void* scratch, size_t scratch_bytes, int64_t* sizes_out) {
-    if (!plan || plan->kind != 5) return SPWS_INVALID_ARGUMENT;
-    return higher_symbolic(plan, A, B, D, C, scratch, scratch_bytes, sizes_out);
+    if (!plan || plan->kind != 5 || !D) return SPWS_INVALID_ARGUMENT;
+    return symbolic_any(plan, A, B, D, C, scratch, scratch_bytes, sizes_out, nullptr);
 }
 
 spws_status_t spws_numeric3(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, const spws_tensor_t* D, spws_tensor_t* C,

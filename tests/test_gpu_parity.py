@@ -964,6 +964,54 @@ def test_exact_workspace_size_suffices_and_is_tight(ctx, oracle_mod, policy):
     plan.close()
 
 
+def test_symbolic_sized_grows_the_scratch_and_remembers_no_operand(ctx, oracle_mod):
+    """The sized symbolic pass starts without a scratch buffer, asks for what the operands at hand need
+    and is right when operands change in place under the same addresses (narrow rows, then rows that
+    span the matrix and need far more bitmap), for every form."""
+    import torch
+    from paper_2404_04541_b200 import api, binding
+    n, d = 3000, 12
+    fresh = api.Context("cuda")
+    band = CSR(n, n, np.arange(n + 1) * d, (np.minimum(np.arange(n)[:, None], n - d) + np.arange(d)).astype(np.int32).reshape(-1),
+               np.random.default_rng(1).uniform(-1, 1, n * d))
+    spread = uniform_rows_csr(n, n, d, 2)
+    dA = api.DeviceCSR.from_host(band)
+    plan = fresh.plan(api.EXPR_SPGEMM, (binding.SPWS_CSR,) * 3, np.float64)
+    sizes = []
+    for M in (band, spread, band):
+        dA.crd.copy_(torch.from_numpy(M.crd))
+        M.val = dA.val.cpu().numpy()
+        c, state = fresh.spgemm_symbolic(plan, dA, dA)
+        sizes.append(state[3])
+        C = fresh.spgemm_numeric(plan, c, state)
+        plan.get_stats()
+        ref = oracle_mod.spgemm(M, M, threads=4)
+        assert_matches((C.pos.cpu().numpy(), C.crd.cpu().numpy(), C.val.cpu().numpy()), ref, np.float64)
+    assert sizes[0] == sizes[2] < sizes[1]
+    # too little scratch is refused before any workspace runs, with the size that suffices
+    a = dA.arrays()
+    cc = binding.csr_arrays(n, n, torch.empty(n + 1, dtype=torch.int64, device="cuda"), None, None)
+    ok, need = plan.symbolic_sized(a, a, cc, None, 0)
+    assert not ok
+    buf = torch.empty(max(need, sizes[0]) + 256, dtype=torch.uint8, device="cuda")
+    assert plan.symbolic_sized(a, a, cc, fresh._aligned_ptr(buf), sizes[0] - 256) == (False, sizes[0])
+    assert plan.symbolic_sized(a, a, cc, fresh._aligned_ptr(buf), sizes[0]) == (True, sizes[0])
+    plan.close()
+    # the other forms, each on a context of its own
+    for policy in POLICIES:
+        small = random_csr(60, 70, 0.1, 3)
+        ref = oracle_mod.spgemm(small, random_csr(70, 80, 0.1, 4))
+        C, _ = api.Context("cuda").spgemm_outer(api.DeviceCSR.from_host(small.transpose()), api.DeviceCSR.from_host(random_csr(70, 80, 0.1, 4)), policy=policy)
+        assert np.array_equal(C.crd.cpu().numpy(), ref.crd)
+    T, M0, M1 = uniform_csf3((6, 7, 8), 80, 5), random_csr(6, 9, 0.5, 6), random_csr(7, 9, 0.5, 7)
+    for policy in ("auto", "ism"):
+        own = api.Context("cuda")
+        for _ in range(20):                              # plans closed one after another hand on their pinned block
+            crd, val, _ = own.scatter_coo(api.EXPR_SPMTTKRP, api.DeviceCSF3.from_host(T), api.DeviceCSR.from_host(M0), api.DeviceCSR.from_host(M1),
+                                          policy=policy)
+        assert np.array_equal(crd.cpu().numpy().astype(np.int64), oracle_mod.spmttkrp(T, M0, M1).crd)
+
+
 # ------------------------------------------------------------------ boundary behaviour
 def test_error_statuses(ctx):
     import torch
