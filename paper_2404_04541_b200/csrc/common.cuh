@@ -29,6 +29,8 @@ constexpr int NUM_SLOT = 16;   // work_counter[cls] in the symbolic pass, work_c
 constexpr int CEIL_SLOT = 32;  // work_counter[CEIL_SLOT + cls] in the gather-only (iteration-only) kernels
 constexpr int EMIT_SLOT = 48;  // work_counter slot of the coordinate emission of the CTA dense route
 constexpr int BW_SLOT = 49;    // work_counter slot of the word-list build
+constexpr int WARP_SLOT = 52;  // work_counter slots of the lists of the warp dense route: numeric, gather-only
+constexpr int CEIL_WARP_SLOT = 54;
 constexpr int ISM_CTA_SLOT = 50; // work_counter slots of the CTA kernel of the shared-memory ISM, symbolic and numeric
 constexpr int ISM_CTA_NUM_SLOT = 51;
 constexpr int N_WORK_COUNTERS = 64;
@@ -41,7 +43,9 @@ constexpr int ISM_WARP_MAX = 1024;         // products of a row the warp kernel 
 
 // Capacities fixed at compile time.
 constexpr int DENSE_WARP_BM_WORDS = 1024;  // bitmap words a warp-per-row workspace may span (32768 columns)
-constexpr int DENSE_WARP_ACC = 256;        // outputs a warp-per-row numeric workspace may hold
+constexpr int DENSE_WARP_ACC = 256;        // outputs a warp-per-row numeric workspace may hold ...
+constexpr int DENSE_WARP_ACC2 = 1024;      // ... and the larger one that `auto` gives rows of more outputs
+constexpr int N_WARP_LISTS = 2;            // rows of the warp numeric kernel by those capacities
 constexpr int DENSE_WARP_MAX_UB = 4096;    // products a single warp is given at most
 constexpr i64 DENSE_HUB_UB = 1ll << 17;    // rows with at least this many products are scheduled first
 constexpr int DENSE_MAX_SPAN_WORDS = 16384;// 2^19 columns: the widest bitmap (8 bytes per word with its rank) one CTA holds
@@ -71,11 +75,11 @@ struct DevCtl {
     u64 bm_words_used;      // words handed out of the bitmap arena
     int status;
     int n_units;            // numeric dense CTA units (row, share of its entries)
-    int hub_units;          // units of the heaviest rows, which come first ...
-    int hub_cursor, other_cursor;   // ... and units handed out so far
-    int n_warp_rows;        // numeric dense warp rows
+    int units_of[7];        // units per bucket of rows (counted by the binning, without the rows that outgrow a warp) ...
+    int unit_cursor[7];     // ... and units numbered so far
+    int n_warp_rows[N_WARP_LISTS];  // numeric dense warp rows by the accumulator they need
     int max_span_words;     // widest bitmap among the dense rows
-    int max_warp_cnt;       // most outputs of a row the warp numeric kernel takes
+    int max_warp_cnt[N_WARP_LISTS]; // most outputs of a row on each list
     int n_long;             // B rows with at least BW_MIN_LEN entries (candidates for a word list)
     int bin_done, rows_done, slices_done;       // blocks that have finished
     int rows_ticket, slices_ticket;             // tiles handed out
@@ -106,6 +110,7 @@ struct ClassParams {
     float span_words_per_product;
     int unit_cap;           // entries available in the unit table
     u64 bm_arena_words;     // capacity of the bitmap arena
+    int warp_outputs;       // most outputs of a row that stays with a warp
 };
 
 // Scratch of the forms whose first operand is put in output-row order (rowwise.cu).
@@ -148,7 +153,7 @@ struct RowTables {
     int* perm;
     i64* bm_off;        // word offset of the row's bitmap in the arena (dense classes)
     unsigned* bm_arena;
-    int* warp_rows;     // numeric: rows handled by the warp-per-row dense kernel
+    int* warp_rows;     // numeric: rows handled by the warp-per-row dense kernel: list 0 from the front, list 1 from the back
     int* row_unit0;     // numeric: first CTA unit of a row
     int* unit_row;      // numeric: row of a CTA unit
 };
@@ -160,6 +165,23 @@ struct RowTables {
 __host__ __device__ inline i64 dense_unit_products(i64 total_products) {
     const i64 need = (total_products + (1ll << 19) - 1) >> 19;
     return need > (1ll << 16) ? need : (1ll << 16);
+}
+// The order in which CTA units are taken.  With few of them the heaviest rows come first, by powers of two of the
+// row's products (2^17 and more, 2^16, .., 2^13, fewer, rows that outgrew a warp), so that the last units
+// taken are small: power law on 16381 vertices, 4e3 units, accumulation 362 -> 310 us.  With many, units
+// are numbered in row order and taken in runs of UNIT_RUN whose order is scattered: rows of like weight
+// tend to be neighbours (the hubs of a graph first of all), and a mixture overlaps what heavy and light
+// rows wait for: power law on 2^18 vertices, 1.4e5 units, coordinates 4200 -> 3860 us and accumulation
+// 14350 -> 14050 us against heaviest first (runs of 64 .. 1024 units within 0.3 %).
+constexpr int UNIT_BUCKETS = 7;
+static_assert(sizeof(DevCtl::units_of) == 4 * UNIT_BUCKETS, "a counter per bucket");
+constexpr int UNIT_FEW = 1 << 14;       // (about 55 units per CTA)
+constexpr int UNIT_RUN = 256;
+__device__ __forceinline__ int unit_bucket(i64 ub) { return ub >= (1ll << 17) ? 0 : ub < (1ll << 13) ? 5 : __clz((int)ub) - 14; }
+__device__ __forceinline__ int unit_at(int t, int n) {
+    const unsigned runs = (unsigned)n / UNIT_RUN, run = (unsigned)t / UNIT_RUN;
+    if (n < UNIT_FEW || run >= runs) return t;
+    return (int)((u64)run * 2654435761ull % runs) * UNIT_RUN + (int)((unsigned)t % UNIT_RUN);      // (a prime: a permutation of the runs)
 }
 __host__ __device__ inline int dense_units_of_row(i64 ub, i64 unit_products) {
     const i64 n = (ub + unit_products - 1) / unit_products;
@@ -368,8 +390,9 @@ cudaError_t launch_ism_smem(const LaunchCtx& c, bool numeric, int cls, int n_hos
                             const i64* rowptr, int* Ccrd, void* Cval);
 cudaError_t launch_dense_sym_warp(const LaunchCtx& c, const Csr& A, const Csr& B);
 cudaError_t launch_dense_sym_cta(const LaunchCtx& c, const Csr& A, const Csr& B);
-// chk_idx / chk_val non-null: the gather-only form of the same kernel (workspace stripped, checksums out)
-cudaError_t launch_dense_num_warp(const LaunchCtx& c, int n_host, int max_span_words, int max_cnt, const Csr& A, const Csr& B,
+// chk_idx / chk_val non-null: the gather-only form of the same kernel (workspace stripped, checksums out).
+// n[], max_cnt[]: rows on each list and their largest output counts
+cudaError_t launch_dense_num_warp(const LaunchCtx& c, const int* n, const int* max_cnt, int m, int max_span_words, const Csr& A, const Csr& B,
                                   const i64* rowptr, int* Ccrd, void* Cval, u64* chk_idx = nullptr, double* chk_val = nullptr);
 // phase 0: write the coordinates and clear the value segments several units add into; 1: accumulate
 cudaError_t launch_dense_num_cta(const LaunchCtx& c, int phase, int n_units_host, int max_span_words, i64 total_products,

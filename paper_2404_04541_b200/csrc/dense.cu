@@ -13,7 +13,8 @@
 //              product; acc is copied straight to the row's value segment and the set bits give
 //              the column indices.
 // Two granularities:
-//   warp per row : bitmap <= 1024 words, <= 256 outputs.  A warp walks the A entries one at a
+//   warp per row : bitmap <= 1024 words, <= 256 outputs (<= 1024 under `auto`, in a launch of their own, so
+//              that the larger accumulators do not cost the others their occupancy).  A warp walks the A entries one at a
 //              time with its lanes across the B row, so no two lanes ever hit the same slot and
 //              the accumulator needs no atomics; sums are in loop order.
 //   CTA units    : any span up to 2^19 columns.  A unit is a row, or an equal share of the A
@@ -46,7 +47,7 @@ __device__ __forceinline__ int chunks_of(int nw) { return (nw + 31) >> 5; }
 // ---------------------------------------------------------------------------------------
 // symbolic, warp per row
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __restrict__ ctl, Csr A, Csr B, RowTables tab) {
+__global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __restrict__ ctl, int warp_outputs, Csr A, Csr B, RowTables tab) {
     __shared__ unsigned s_bm[DW_WARPS][DENSE_WARP_BM_WORDS];
     // bit w of the summary = bitmap word w is non-empty, so the copy-out walks only those words
     __shared__ unsigned s_sum[DW_WARPS][DENSE_WARP_BM_WORDS / 32];
@@ -141,7 +142,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __re
         __syncwarp();
         const i64 slot = tab.bm_off[row];
         unsigned* out = tab.bm_arena + slot;
-        if (cnt <= DENSE_WARP_ACC && 2 * nzw <= nw + chunks_of(nw)) {
+        if (cnt <= warp_outputs && 2 * nzw <= nw + chunks_of(nw)) {
             // compact form for the warp numeric kernel: only the non-empty words, as (bits, word
             // index) in column order; lane l owns the words its summary word flags
             uint2* out2 = reinterpret_cast<uint2*>(out);
@@ -282,18 +283,18 @@ __global__ void __launch_bounds__(DC_THREADS) dense_sym_cta_kernel(DevCtl* __res
 // CEIL = true: the same walk over rows, entries and B rows with the workspace stripped (Sec. 7.2,
 // iteration-only lower bound); the gathered indices and products go into two checksums.
 template <typename T, bool CEIL>
-__global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __restrict__ ctl, int bmw, int accw, Csr A, Csr B, RowTables tab,
+__global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __restrict__ ctl, const int* __restrict__ rows, int step, int n, int slot_,
+                                                                    int bmw, int accw, Csr A, Csr B, RowTables tab,
                                                                     const i64* __restrict__ rowptr, int* __restrict__ Ccrd,
                                                                     T* __restrict__ Cval, u64* __restrict__ chk_idx,
                                                                     double* __restrict__ chk_val) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (ctl->status != 0) return;
-    const int n = ctl->n_warp_rows;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     // per warp: a table of bmw bitmap words, each with the number of outputs before it (one load
     // ranks a column), and accw values (sized from the widest / largest row of this launch)
     uint2* tbl = reinterpret_cast<uint2*>(smem_raw) + warp * bmw;
-    T* acc = reinterpret_cast<T*>(reinterpret_cast<uint2*>(smem_raw) + DW_WARPS * bmw) + warp * accw;
+    T* acc = reinterpret_cast<T*>(reinterpret_cast<uint2*>(smem_raw) + warps * bmw) + warp * accw;
     const T* __restrict__ Aval = (const T*)A.val;
     const T* __restrict__ Bval = (const T*)B.val;
     if (!CEIL)
@@ -303,10 +304,10 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
     double my_val = 0.0;
     for (;;) {
         int r = 0;
-        if (lane == 0) r = atomicAdd(&ctl->work_counter[(CEIL ? CEIL_SLOT : NUM_SLOT) + CLS_DENSE_WARP], 1);
+        if (lane == 0) r = atomicAdd(&ctl->work_counter[slot_], 1);
         r = __shfl_sync(0xffffffffu, r, 0);
         if (r >= n) break;
-        const int row = tab.warp_rows[r];
+        const int row = __ldg(rows + (i64)r * step);
         const int base = tab.jmin[row];
         const int nw = min((tab.jmax[row] - base) / 32 + 1, bmw);
         const unsigned span = (unsigned)nw * 32u;
@@ -351,10 +352,10 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
                 if (rel != 0xffffffffu) { my_idx += (u64)(rel + (unsigned)base); my_val += (double)prod; }
             } else if (rel < span) {
                 const uint2 t = tbl[rel >> 5];
-                const int slot_ = (int)t.y + __popc(t.x & ((1u << (rel & 31)) - 1u));
-                if (slot_ < accw) {
-                    if (shared_slot) atomicAdd(&acc[slot_], prod);
-                    else acc[slot_] = add_rn(acc[slot_], prod);
+                const int at_ = (int)t.y + __popc(t.x & ((1u << (rel & 31)) - 1u));
+                if (at_ < accw) {
+                    if (shared_slot) atomicAdd(&acc[at_], prod);
+                    else acc[at_] = add_rn(acc[at_], prod);
                 }
             }
         };
@@ -494,8 +495,8 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
         __syncthreads();
         if (tid == 0) s_next = atomicAdd(&ctl->work_counter[(CEIL ? CEIL_SLOT : NUM_SLOT) + CLS_DENSE_CTA], 1);
         __syncthreads();
-        const int u = s_next;
-        if (u >= n_units) break;
+        if (s_next >= n_units) break;
+        const int u = unit_at(s_next, n_units);
         const int row = tab.unit_row[u];
         const int uidx = u - tab.row_unit0[row];
         const int nun = dense_units_of_row(tab.ub[row], unit_products);
@@ -714,6 +715,7 @@ __global__ void __launch_bounds__(DE_THREADS) dense_emit_crd_kernel(DevCtl* __re
         if (lane == 0) u = atomicAdd(&ctl->work_counter[EMIT_SLOT], 1);
         u = __shfl_sync(0xffffffffu, u, 0);
         if (u >= n_units) break;
+        u = unit_at(u, n_units);
         const int row = tab.unit_row[u];
         const int uidx = u - tab.row_unit0[row];
         const int nun = dense_units_of_row(tab.ub[row], unit_products);
@@ -812,7 +814,7 @@ cudaError_t launch_dense_sym_warp(const LaunchCtx& c, const Csr& A, const Csr& B
     int per_sm = 0;
     cudaError_t e = resident_blocks((const void*)dense_sym_warp_kernel, DW_THREADS, 0, &per_sm);
     if (e != cudaSuccess) return e;
-    dense_sym_warp_kernel<<<persistent_grid(c, per_sm, -1), DW_THREADS, 0, c.stream>>>(c.ctl, A, B, c.tab);
+    dense_sym_warp_kernel<<<persistent_grid(c, per_sm, -1), DW_THREADS, 0, c.stream>>>(c.ctl, c.prm.warp_outputs, A, B, c.tab);
     ++c.launches;
     return cudaGetLastError();
 }
@@ -828,31 +830,37 @@ cudaError_t launch_dense_sym_cta(const LaunchCtx& c, const Csr& A, const Csr& B)
 }
 
 template <typename T, bool CEIL>
-static cudaError_t num_warp_t(const LaunchCtx& c, int n_host, int bmw, int accw, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd,
-                              void* Cval, u64* chk_idx, double* chk_val) {
-    int per_sm = 0;
-    const size_t smem = (size_t)DW_WARPS * (sizeof(T) * (size_t)accw + 8 * (size_t)bmw);
-    cudaError_t e;
+static cudaError_t num_warp_t(const LaunchCtx& c, const int* n, const int* max_cnt, int m, int bmw, const Csr& A, const Csr& B, const i64* rowptr,
+                              int* Ccrd, void* Cval, u64* chk_idx, double* chk_val) {
     auto k = dense_num_warp_kernel<T, CEIL>;
-    if ((e = resident_blocks((const void*)k, DW_THREADS, smem, &per_sm)) != cudaSuccess) return e;
-    const i64 work = n_host >= 0 ? ((i64)n_host + DW_WARPS - 1) / DW_WARPS : -1;
-    k<<<persistent_grid(c, per_sm, work), DW_THREADS, smem, c.stream>>>(c.ctl, bmw, accw, A, B, c.tab, rowptr, Ccrd, (T*)Cval, chk_idx, chk_val);
-    ++c.launches;
+    const int* const rows[N_WARP_LISTS] = {c.tab.warp_rows, c.tab.warp_rows + m - 1};
+    for (int list = N_WARP_LISTS - 1; list >= 0; --list) {          // the longest rows first
+        if (n[list] == 0) continue;
+        // values reserved per warp; smaller CTAs for larger accumulators, so that the SM's shared memory is used up
+        const int accw = (max_cnt[list] + 31) & ~31;
+        const int threads = DW_THREADS >> list, warps = threads / 32;
+        const size_t smem = (size_t)warps * (sizeof(T) * (size_t)accw + 8 * (size_t)bmw);
+        int per_sm = 0;
+        cudaError_t e;
+        if ((e = resident_blocks((const void*)k, threads, smem, &per_sm)) != cudaSuccess) return e;
+        k<<<persistent_grid(c, per_sm, ((i64)n[list] + warps - 1) / warps), threads, smem, c.stream>>>(
+            c.ctl, rows[list], list == 0 ? 1 : -1, n[list], (CEIL ? CEIL_WARP_SLOT : WARP_SLOT) + list, bmw, accw, A, B, c.tab, rowptr, Ccrd, (T*)Cval,
+            chk_idx, chk_val);
+        ++c.launches;
+    }
     return cudaGetLastError();
 }
 
-cudaError_t launch_dense_num_warp(const LaunchCtx& c, int n_host, int max_span_words, int max_cnt, const Csr& A, const Csr& B,
+cudaError_t launch_dense_num_warp(const LaunchCtx& c, const int* n, const int* max_cnt, int m, int max_span_words, const Csr& A, const Csr& B,
                                   const i64* rowptr, int* Ccrd, void* Cval, u64* chk_idx, double* chk_val) {
     // bitmap words reserved per warp: the widest dense row of this pass, at most the class limit
     int bmw = max_span_words > 0 ? ((max_span_words + 31) & ~31) : DENSE_WARP_BM_WORDS;
     if (bmw > DENSE_WARP_BM_WORDS) bmw = DENSE_WARP_BM_WORDS;
-    int accw = max_cnt > 0 ? ((max_cnt + 31) & ~31) : DENSE_WARP_ACC;     // values reserved per warp
-    if (accw > DENSE_WARP_ACC) accw = DENSE_WARP_ACC;
     if (chk_idx)      // same launch shape (shared memory reserved, hence occupancy) as the full kernel
-        return c.is_f64 ? num_warp_t<double, true>(c, n_host, bmw, accw, A, B, rowptr, Ccrd, Cval, chk_idx, chk_val)
-                        : num_warp_t<float, true>(c, n_host, bmw, accw, A, B, rowptr, Ccrd, Cval, chk_idx, chk_val);
-    return c.is_f64 ? num_warp_t<double, false>(c, n_host, bmw, accw, A, B, rowptr, Ccrd, Cval, nullptr, nullptr)
-                    : num_warp_t<float, false>(c, n_host, bmw, accw, A, B, rowptr, Ccrd, Cval, nullptr, nullptr);
+        return c.is_f64 ? num_warp_t<double, true>(c, n, max_cnt, m, bmw, A, B, rowptr, Ccrd, Cval, chk_idx, chk_val)
+                        : num_warp_t<float, true>(c, n, max_cnt, m, bmw, A, B, rowptr, Ccrd, Cval, chk_idx, chk_val);
+    return c.is_f64 ? num_warp_t<double, false>(c, n, max_cnt, m, bmw, A, B, rowptr, Ccrd, Cval, nullptr, nullptr)
+                    : num_warp_t<float, false>(c, n, max_cnt, m, bmw, A, B, rowptr, Ccrd, Cval, nullptr, nullptr);
 }
 
 template <typename T, bool CEIL>

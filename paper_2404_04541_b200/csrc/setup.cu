@@ -72,6 +72,10 @@ __device__ __forceinline__ int classify_row(i64 ub, i64 entries, int jmin, int j
     // auto: few products -> sort them in registers; a bitmap that is small next to the work ->
     // dense; mid-size rows -> shared-memory ISM; long rows -> dense; otherwise global ISM.
     if (reg_ok) return reg_cls;
+    // up to 128 products the register sort beats the bitmap whatever the span; up to 256 when the bitmap is wide
+    // (6e6 products, f64, both passes, dense against ISM: 60 products a row 263 : 172 us, 117 a row 156 : 126
+    // us, 240 a row on 94 words 119 : 113 us and on 626 words 160 : 110 us; 380 a row 98 : 168 us)
+    if (ub <= prm.smem_small_cap && (ub <= 128 || span_words > 256)) return CLS_ISM_SMEM_S;
     if (dense_ok && (float)span_words <= prm.span_words_per_product * (float)ub) return dense_class(ub, span_words);
     if (ub <= prm.smem_small_cap) return CLS_ISM_SMEM_S;
     if (ub <= prm.smem_cap) return CLS_ISM_SMEM;
@@ -177,7 +181,7 @@ __device__ __forceinline__ void long_row_bounds(int row, const Csr& A, const Csr
 // SUMMARY: brow holds the B-row summaries (the instantiation without them carries B's own arrays'
 // two-level gathers and needs more registers).
 template <int G, bool SUMMARY>
-__global__ void __launch_bounds__(256) row_bounds_kernel(Csr A, Csr B, RowTables tab, ClassParams prm, DevCtl* ctl,
+__global__ void __launch_bounds__(256, SUMMARY ? 6 : 5) row_bounds_kernel(Csr A, Csr B, RowTables tab, ClassParams prm, DevCtl* ctl,
                                                          const int4* __restrict__ brow) {
     // rows and products per class, one histogram per warp: 64-bit shared-memory adds are
     // compare-and-swap loops, which many threads on one address turn into a queue
@@ -467,53 +471,54 @@ cudaError_t launch_bw_build(const LaunchCtx& c, const Csr& B) {
 // also reserve the slot of their occupancy bitmap in the arena.  Order inside a class follows
 // block arrival.
 // ---------------------------------------------------------------------------------------
-// It also counts the units of the heaviest rows, clears the words of the kernels that hand running sums
+// It also counts the units per bucket of rows, clears the words of the kernels that hand running sums
 // from tile to tile, and its last block publishes the class sizes to the host.
-__global__ void __launch_bounds__(256) bin_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, DevCtl* host, u64* look, int n_look) {
+__global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, DevCtl* host, u64* look, int n_look) {
+    __shared__ int s_units[UNIT_BUCKETS];
+    if (threadIdx.x < UNIT_BUCKETS) s_units[threadIdx.x] = 0;
     for (int w = blockIdx.x * 256 + threadIdx.x; w < n_look; w += gridDim.x * 256) look[w] = 0;
     const i64 unit_products = dense_unit_products(ctl->products);
     __shared__ int s_hist[NCLASS], s_base[NCLASS], s_off[NCLASS];
     __shared__ int ws[33];
     __shared__ u64 s_bm_base;
     const int rows_per_block = blockDim.x * 4;
-    if (threadIdx.x == 0) {
-        int o = 0;
-        for (int c = 0; c < NCLASS; ++c) { s_off[c] = o; o += ctl->class_count[c]; }
+    if (threadIdx.x < 32) {                             // start of every class in perm
+        const int n = threadIdx.x < NCLASS ? ctl->class_count[threadIdx.x] : 0;
+        const int o = warp_incl_scan(n) - n;
+        if (threadIdx.x < NCLASS) s_off[threadIdx.x] = o;
     }
     for (i64 r0 = (i64)blockIdx.x * rows_per_block; r0 < m; r0 += (i64)gridDim.x * rows_per_block) {
         if (threadIdx.x < NCLASS) s_hist[threadIdx.x] = 0;
-        __syncthreads();
-        int cls[4], rank[4];
+        int cls[4], rank[4], words[4], my_words = 0;
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
             const i64 row = r0 + x * blockDim.x + threadIdx.x;
-            cls[x] = -1;
-            if (row < m) {
-                cls[x] = tab.cls[row];
-                rank[x] = atomicAdd(&s_hist[cls[x]], 1);
-            }
+            cls[x] = row < m ? (int)tab.cls[row] : -1;
         }
         __syncthreads();
-        if (threadIdx.x < NCLASS && s_hist[threadIdx.x])
-            s_base[threadIdx.x] = atomicAdd(&ctl->class_cursor[threadIdx.x], s_hist[threadIdx.x]);
-        __syncthreads();
-        // bitmap words of this thread's dense rows; one arena reservation per block
-        int words[4], my_words = 0;
+        // bitmap words of this thread's dense rows (the words, then the rank at the start of every 32-word chunk,
+        // 16-byte aligned)
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
             const i64 row = r0 + x * blockDim.x + threadIdx.x;
             words[x] = 0;
-            if (cls[x] == CLS_DENSE_WARP || cls[x] == CLS_DENSE_HUB || cls[x] == CLS_DENSE_CTA)
-            {   // the row's slot: bitmap words, then the rank at the start of every 32-word chunk
+            if (cls[x] >= 0) rank[x] = atomicAdd(&s_hist[cls[x]], 1);
+            if (cls[x] == CLS_DENSE_WARP || cls[x] == CLS_DENSE_HUB || cls[x] == CLS_DENSE_CTA) {
                 const int nw = (tab.jmax[row] - tab.jmin[row]) / 32 + 1;
-                words[x] = (nw + (nw + 31) / 32 + 3) & ~3;      // 16-byte aligned slots
-                if (cls[x] == CLS_DENSE_HUB) atomicAdd(&ctl->hub_units, dense_units_of_row(tab.ub[row], unit_products));
+                words[x] = (nw + (nw + 31) / 32 + 3) & ~3;
+                if (cls[x] != CLS_DENSE_WARP) {
+                    const i64 u = tab.ub[row];
+                    atomicAdd(&s_units[unit_bucket(u)], dense_units_of_row(u, unit_products));
+                }
             }
             my_words += words[x];
         }
+        // places in perm and in the arena: one reservation per class and one of the arena per block, side by side
         int block_words;
         int my_off = block_excl_scan<256>(my_words, ws, block_words);
-        if (threadIdx.x == 0 && block_words) s_bm_base = atomicAdd(&ctl->bm_words_used, (u64)block_words);
+        if (threadIdx.x < NCLASS && s_hist[threadIdx.x])
+            s_base[threadIdx.x] = atomicAdd(&ctl->class_cursor[threadIdx.x], s_hist[threadIdx.x]);
+        if (threadIdx.x == 32 && block_words) s_bm_base = atomicAdd(&ctl->bm_words_used, (u64)block_words);
         __syncthreads();
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
@@ -533,6 +538,7 @@ __global__ void __launch_bounds__(256) bin_rows_kernel(int m, RowTables tab, Cla
         }
         __syncthreads();
     }
+    if (threadIdx.x < UNIT_BUCKETS && s_units[threadIdx.x]) atomicAdd(&ctl->units_of[threadIdx.x], s_units[threadIdx.x]);
     if (last_block(&ctl->bin_done, gridDim.x)) {
         if (threadIdx.x == 0) ctl->host_status = &host->status;
         __syncthreads();
@@ -556,13 +562,13 @@ cudaError_t launch_bin_rows(const LaunchCtx& c, int m) {
 // is contiguous.  Tiles hand the running sums on by a decoupled look-back.
 //   Routing: a row the warp kernel counted and whose outputs fit a warp's accumulator stays with a warp;
 //   every other dense row becomes one CTA unit, or several when it has many products: unit c of n takes
-//   the c-th n-th of the row's A entries (all units of a row add into the same outputs).  The units of
-//   the heaviest rows come first.
+//   the c-th n-th of the row's A entries (all units of a row add into the same outputs).
 //   TTM: a fibre (i,j) survives when it produced an output; survivors are packed (Cpos2, Ccrd1), and
 //   sfp[s] receives the number of survivors before slice s.
 // Replaces a three-launch scan, the routing and the per-class count (five launches; seven for the
 // 3-tensor form).
-// FINISH_MEASURED
+// Bound by the chain of its steps below a few tiles (2048 rows: 9 us where the five launches took 13 and their gaps),
+// by HBM beyond (2e6 fibres: 43 us against 56).
 // ---------------------------------------------------------------------------------------
 constexpr int FR_THREADS = 256;
 constexpr int FR_WARPS = FR_THREADS / 32;
@@ -580,88 +586,138 @@ struct FibreArgs {
 };
 
 template <bool DENSE, bool TTM>
-__global__ void __launch_bounds__(FR_THREADS) finish_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, DevCtl* host, u64* look,
+__global__ void __launch_bounds__(FR_THREADS, 3) finish_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, DevCtl* host, u64* look,
                                                                  i64* __restrict__ rowptr, FibreArgs f) {
     __shared__ int s_tile, s_slice0;
     __shared__ i64 s_sum[FR_WARPS], s_before[2];
-    __shared__ int s_part[4][FR_WARPS];             // survivors, warp rows, units of heavy rows, other units
-    __shared__ int s_base[3];
+    __shared__ int s_part[1 + N_WARP_LISTS][FR_WARPS];     // survivors, warp rows on each list
+    __shared__ int s_wbase[N_WARP_LISTS], s_units[UNIT_BUCKETS];           // places in the routing tables; units: the tile's count, then the running place
     __shared__ i64 s_cls[FR_WARPS][NCLASS];
-    __shared__ i64 s_wp[FR_WARPS], s_wn[FR_WARPS];
-    __shared__ int s_wm[FR_WARPS];
+    __shared__ i64 s_wp[FR_WARPS];
+    __shared__ int s_wn[FR_WARPS], s_wm[N_WARP_LISTS][FR_WARPS];
     __shared__ int s_kept[TTM ? FR_TILE : 1];       // survivors of the tile before each fibre
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned all = 0xffffffffu, below = (1u << lane) - 1u;
     const int tiles = gridDim.x;
     if (tid == 0) s_tile = atomicAdd(&ctl->rows_ticket, 1);
     for (int x = tid; x < FR_WARPS * NCLASS; x += FR_THREADS) (&s_cls[0][0])[x] = 0;
+    if (tid >= 128 && tid < 128 + UNIT_BUCKETS) s_units[tid - 128] = 0;
     __syncthreads();
     const int tile = s_tile;
     const i64 tile0 = (i64)tile * FR_TILE;
     const i64 row0 = tile0 + warp * (FR_ITEMS * 32) + lane;
     const i64 unit_products = DENSE ? dense_unit_products(ctl->products) : 1;
+    int unit_count = 0;                             // units of all rows but those that outgrow a warp
+    if (DENSE)
+        for (int k = 0; k < UNIT_BUCKETS; ++k) unit_count += ctl->units_of[k];
+    const bool few = unit_count < UNIT_FEW;
 
     // ---- this warp's rows: counts, sums, routing
     int v[FR_ITEMS], cls[FR_ITEMS];
-    i64 sum = 0, wp = 0, wn = 0;
-    int kept = 0, to_warp = 0, heavy = 0, other = 0, wm = 0;
+    i64 sum = 0, wp = 0;
+    int kept = 0, wn = 0, to_warp[N_WARP_LISTS] = {}, wm[N_WARP_LISTS] = {};
+    // all loads first: what the rows below need is a few registers, a load inside the loops is a wait each
+    int q[DENSE ? FR_ITEMS : 1];                    // products of a warp-class row; bucket and units of another dense row
+    int acrd[TTM ? FR_ITEMS : 1];
+    {
+        i64 ub[DENSE ? FR_ITEMS : 1];
 #pragma unroll
-    for (int x = 0; x < FR_ITEMS; ++x) {
-        const i64 row = row0 + 32 * x;
-        v[x] = row < m ? tab.cnt[row] : 0;
-        cls[x] = row < m ? (int)tab.cls[row] : (int)CLS_EMPTY;
+        for (int x = 0; x < FR_ITEMS; ++x) {
+            const i64 row = row0 + 32 * x;
+            v[x] = row < m ? tab.cnt[row] : 0;
+            cls[x] = row < m ? (int)tab.cls[row] : (int)CLS_EMPTY;
+            if (DENSE) ub[x] = row < m ? tab.ub[row] : 0;
+            if (TTM) acrd[x] = row < m ? f.Acrd1[row] : 0;
+        }
+        if (DENSE)
+#pragma unroll
+            for (int x = 0; x < FR_ITEMS; ++x)
+                q[x] = cls[x] == CLS_DENSE_WARP ? (int)ub[x] : (unit_bucket(ub[x]) << 28) | dense_units_of_row(ub[x], unit_products);
     }
-    // units of row x: 0 for a row of the warp kernel and for rows that are not dense
-    auto units = [&](int x) -> int {
-        if (cls[x] < CLS_DENSE_WARP || cls[x] > CLS_DENSE_CTA || (cls[x] == CLS_DENSE_WARP && v[x] <= DENSE_WARP_ACC)) return 0;
-        return dense_units_of_row(tab.ub[row0 + 32 * x], unit_products);
+    // list of the warp numeric kernel a row goes to; -1: to CTA units or not dense
+    auto list_of = [&](int x) -> int {
+        if (!DENSE || cls[x] != CLS_DENSE_WARP || v[x] > prm.warp_outputs) return -1;
+        return v[x] <= DENSE_WARP_ACC ? 0 : 1;
     };
+    auto unit_row = [&](int x) { return DENSE && cls[x] >= CLS_DENSE_WARP && cls[x] <= CLS_DENSE_CTA && list_of(x) < 0; };
+    // (a row that outgrew a warp has at most DENSE_WARP_MAX_UB products: one unit)
+    auto units = [&](int x) { return cls[x] == CLS_DENSE_WARP ? 1 : q[x] & 0xfffffff; };
+    auto bucket = [&](int x) { return !few ? 0 : cls[x] == CLS_DENSE_WARP ? UNIT_BUCKETS - 1 : q[x] >> 28; };
+    bool one_class = true;
+    // the class of the warp's first row that is not empty in the first 32 rows (all empty: any)
+    const unsigned some = __ballot_sync(all, cls[0] != CLS_EMPTY);
+    const int cls0 = __shfl_sync(all, cls[0], some ? __ffs(some) - 1 : 0);
 #pragma unroll
     for (int x = 0; x < FR_ITEMS; ++x) {
         sum += v[x];
+        one_class &= cls[x] == cls0 || cls[x] == CLS_EMPTY;
         if (TTM) kept += __popc(__ballot_sync(all, v[x] > 0));
-        // outputs per class: one round per class among the 32 rows (nearly always one)
-        unsigned todo = __ballot_sync(all, cls[x] != CLS_EMPTY);
-        while (todo) {
-            const int k = __shfl_sync(all, cls[x], __ffs(todo) - 1);
-            const bool mine = cls[x] == k;
-            const unsigned lo = __reduce_add_sync(all, mine ? (unsigned)v[x] & 0xffffu : 0u);
-            const unsigned hi = __reduce_add_sync(all, mine ? (unsigned)v[x] >> 16 : 0u);
-            if (lane == 0) s_cls[warp][k] += (i64)lo + ((i64)hi << 16);
-            todo &= ~__ballot_sync(all, mine);
-        }
         if (DENSE) {
-            const bool w = cls[x] == CLS_DENSE_WARP && v[x] <= DENSE_WARP_ACC;
-            to_warp += __popc(__ballot_sync(all, w));
-            if (w) { wp += tab.ub[row0 + 32 * x]; wn += v[x]; wm = max(wm, v[x]); }
-            const int nu = units(x);
-            if (cls[x] == CLS_DENSE_HUB) heavy += nu; else other += nu;
+            const int l = list_of(x);
+#pragma unroll
+            for (int t = 0; t < N_WARP_LISTS; ++t) {
+                to_warp[t] += __popc(__ballot_sync(all, l == t));
+                if (l == t) wm[t] = max(wm[t], v[x]);
+            }
+            if (l >= 0) { wp += q[x]; wn += v[x]; }
+            if (unit_row(x)) atomicAdd(&s_units[bucket(x)], units(x));
         }
     }
     for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(all, sum, d);
-    if (DENSE) {
-        for (int d = 16; d > 0; d >>= 1) {
-            wp += __shfl_xor_sync(all, wp, d);
-            wn += __shfl_xor_sync(all, wn, d);
+    // outputs per class: this warp's sum when its 256 rows share a class, else one round per class and 32 rows
+    if (__all_sync(all, one_class)) {
+        if (lane == 0 && cls0 != CLS_EMPTY) s_cls[warp][cls0] = sum;
+    } else {
+#pragma unroll
+        for (int x = 0; x < FR_ITEMS; ++x) {
+            unsigned todo = __ballot_sync(all, cls[x] != CLS_EMPTY);
+            while (todo) {
+                const int k = __shfl_sync(all, cls[x], __ffs(todo) - 1);
+                const bool mine = cls[x] == k;
+                const unsigned lo = __reduce_add_sync(all, mine ? (unsigned)v[x] & 0xffffu : 0u);
+                const unsigned hi = __reduce_add_sync(all, mine ? (unsigned)v[x] >> 16 : 0u);
+                if (lane == 0) s_cls[warp][k] += (i64)lo + ((i64)hi << 16);
+                todo &= ~__ballot_sync(all, mine);
+            }
         }
-        wm = __reduce_max_sync(all, wm);
-        heavy = __reduce_add_sync(all, heavy);
-        other = __reduce_add_sync(all, other);
+    }
+    if (DENSE) {
+        for (int d = 16; d > 0; d >>= 1) wp += __shfl_xor_sync(all, wp, d);
+        wn = __reduce_add_sync(all, wn);                // at most 256 rows of 1024 outputs
+#pragma unroll
+        for (int t = 0; t < N_WARP_LISTS; ++t) wm[t] = __reduce_max_sync(all, wm[t]);
+    }
+    if (TTM && warp == FR_WARPS - 1) {              // first slice that starts in this tile or later: 32 probes per step
+        int lo = 0, hi = f.n_i;                     // Apos1[lo - 1] < tile0 <= Apos1[hi]
+        while (lo < hi) {
+            const int step = (hi - lo + 31) >> 5, at = lo + lane * step;
+            const int n = __popc(__ballot_sync(all, at < hi && f.Apos1[at] < tile0));     // probes that start earlier
+            const int from = n ? lo + (n - 1) * step + 1 : lo;
+            hi = min(hi, lo + n * step);
+            lo = from;
+        }
+        if (lane == 0) s_slice0 = lo;
     }
     if (lane == 0) {
         s_sum[warp] = sum;
-        s_part[0][warp] = kept; s_part[1][warp] = to_warp; s_part[2][warp] = heavy; s_part[3][warp] = other;
-        s_wp[warp] = wp; s_wn[warp] = wn; s_wm[warp] = wm;
+        s_part[0][warp] = kept;
+        s_wp[warp] = wp;
+        s_wn[warp] = wn;
+#pragma unroll
+        for (int t = 0; t < N_WARP_LISTS; ++t) {
+            s_part[1 + t][warp] = to_warp[t];
+            s_wm[t][warp] = wm[t];
+        }
     }
     __syncthreads();
     i64 tile_sum = 0, warp_sum = 0;
-    int total[4] = {0, 0, 0, 0}, mine[4] = {0, 0, 0, 0};
+    int total[1 + N_WARP_LISTS] = {}, mine[1 + N_WARP_LISTS] = {};
 #pragma unroll
     for (int w = 0; w < FR_WARPS; ++w) {
         if (w == warp) warp_sum = tile_sum;
         tile_sum += s_sum[w];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int t = 0; t < 1 + N_WARP_LISTS; ++t) {
             if (w == warp) mine[t] = total[t];
             total[t] += s_part[t][w];
         }
@@ -678,84 +734,95 @@ __global__ void __launch_bounds__(FR_THREADS) finish_rows_kernel(int m, RowTable
         }
         if (lane == 0) s_before[warp] = before;
     }
-    if (DENSE && tid == 64) {
-        s_base[0] = total[1] ? atomicAdd(&ctl->n_warp_rows, total[1]) : 0;
-        s_base[1] = total[2] ? atomicAdd(&ctl->hub_cursor, total[2]) : 0;
-        s_base[2] = (total[3] ? atomicAdd(&ctl->other_cursor, total[3]) : 0) + ctl->hub_units;
-        if (total[1]) {
-            i64 p = 0, n = 0;
-            int most = 0;
-            for (int w = 0; w < FR_WARPS; ++w) { p += s_wp[w]; n += s_wn[w]; most = max(most, s_wm[w]); }
+    if (DENSE && warp >= 2 && warp < 2 + N_WARP_LISTS && lane == 0) {
+        const int list = warp - 2;
+        int n_rows = total[1];
+#pragma unroll
+        for (int t = 1; t < N_WARP_LISTS; ++t) n_rows = list == t ? total[1 + t] : n_rows;
+        if (n_rows) s_wbase[list] = atomicAdd(&ctl->n_warp_rows[list], n_rows);
+        i64 p = 0;
+        int n = 0, most = 0;
+        for (int w = 0; w < FR_WARPS; ++w) { p += s_wp[w]; n += s_wn[w]; most = max(most, s_wm[list][w]); }
+        if (most) atomicMax(&ctl->max_warp_cnt[list], most);
+        if (list == 0 && p) {
             atomicAdd((u64*)&ctl->dense_warp_products, (u64)p);
             atomicAdd((u64*)&ctl->dense_warp_nnz, (u64)n);
-            atomicMax(&ctl->max_warp_cnt, most);
         }
     }
-    if (TTM && tid == 96) {                         // first slice that starts in this tile or later
-        int lo = 0, hi = f.n_i;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (f.Apos1[mid] < tile0) lo = mid + 1; else hi = mid;
+    if (DENSE && tid >= 160 && tid < 160 + UNIT_BUCKETS) {
+        const int k = tid - 160, n = s_units[k];
+        int at = 0;
+        if (n) {
+            if (few)
+                for (int j = 0; j < k; ++j) at += ctl->units_of[j];
+            at += atomicAdd(&ctl->unit_cursor[k], n);
         }
-        s_slice0 = lo;
+        s_units[k] = at;
     }
-    if (tid >= 128 && tid < 128 + NCLASS) {
+    if (tid >= 192 && tid < 192 + NCLASS) {
         i64 t = 0;
-        for (int w = 0; w < FR_WARPS; ++w) t += s_cls[w][tid - 128];
-        if (t) atomicAdd((u64*)&ctl->class_nnz[tid - 128], (u64)t);
+        for (int w = 0; w < FR_WARPS; ++w) t += s_cls[w][tid - 192];
+        if (t) atomicAdd((u64*)&ctl->class_nnz[tid - 192], (u64)t);
     }
     __syncthreads();
 
     // ---- placement
     i64 run = s_before[0] + warp_sum;
     const i64 kbase = TTM ? s_before[1] : 0;
-    int krun = mine[0], wrun = mine[1], hrun = mine[2], orun = mine[3];
+    int krun = mine[0];
+    const bool small = tile_sum < (1ll << 31);      // (a tile of 2048 counts may total 2^31 or more)
 #pragma unroll
     for (int x = 0; x < FR_ITEMS; ++x) {
         const i64 row = row0 + 32 * x;
-        i64 incl = v[x];
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const i64 t = __shfl_up_sync(all, incl, d);
-            if (lane >= d) incl += t;
+        i64 excl;
+        if (small) {
+            const int incl = warp_incl_scan(v[x]);
+            excl = incl - v[x];
+            if (row < m) rowptr[row] = run + excl;
+            excl += run;
+            run += __shfl_sync(all, incl, 31);
+        } else {
+            i64 incl = v[x];
+            for (int d = 1; d < 32; d <<= 1) {
+                const i64 t = __shfl_up_sync(all, incl, d);
+                if (lane >= d) incl += t;
+            }
+            excl = run + incl - v[x];
+            if (row < m) rowptr[row] = excl;
+            run += __shfl_sync(all, incl, 31);
         }
-        const i64 at = run + incl - v[x];
-        run += __shfl_sync(all, incl, 31);
-        if (row < m) rowptr[row] = at;
         if (TTM) {
             const unsigned live = __ballot_sync(all, v[x] > 0);
             const int k = krun + __popc(live & below);
             s_kept[warp * (FR_ITEMS * 32) + x * 32 + lane] = k;
             if (v[x] > 0) {
-                f.Cpos2[kbase + k] = at;
-                f.Ccrd1[kbase + k] = f.Acrd1[row];
+                f.Cpos2[kbase + k] = excl;
+                f.Ccrd1[kbase + k] = acrd[x];
             }
             krun += __popc(live);
         }
         if (DENSE) {
-            const bool w = cls[x] == CLS_DENSE_WARP && v[x] <= DENSE_WARP_ACC;
-            const unsigned ws = __ballot_sync(all, w);
-            if (w) {
-                tab.warp_rows[s_base[0] + wrun + __popc(ws & below)] = (int)row;
-                tab.row_unit0[row] = -1;
-            }
-            wrun += __popc(ws);
-            const int nu = units(x);
-            if (__any_sync(all, nu > 0)) {
-                const bool hub = cls[x] == CLS_DENSE_HUB;
-                const int hi = warp_incl_scan(hub ? nu : 0), oi = warp_incl_scan(hub ? 0 : nu);
-                if (nu > 0) {
-                    const i64 u0 = hub ? (i64)s_base[1] + hrun + hi - nu : (i64)s_base[2] + orun + oi - nu;
-                    if (u0 + nu > prm.unit_cap) {
-                        raise_status(ctl, DEV_SCRATCH_TOO_SMALL);
-                        tab.row_unit0[row] = -1;
-                    } else {
-                        tab.row_unit0[row] = (int)u0;
-                        for (int t = 0; t < nu; ++t) tab.unit_row[u0 + t] = (int)row;
-                    }
+            const int l = list_of(x);
+#pragma unroll
+            for (int t = 0; t < N_WARP_LISTS; ++t) {
+                const unsigned on = __ballot_sync(all, l == t);
+                if (l == t) {
+                    const int k = s_wbase[t] + mine[1 + t] + __popc(on & below);
+                    tab.warp_rows[t == 0 ? k : m - 1 - k] = (int)row;
+                    tab.row_unit0[row] = -1;
                 }
-                hrun += __shfl_sync(all, hi, 31);
-                orun += __shfl_sync(all, oi, 31);
+                mine[1 + t] += __popc(on);
+            }
+            if (unit_row(x)) {
+                const int nu = units(x);
+                const int u0 = atomicAdd(&s_units[bucket(x)], nu);
+                if ((i64)u0 + nu > prm.unit_cap) {
+                    raise_status(ctl, DEV_SCRATCH_TOO_SMALL);
+                    tab.row_unit0[row] = -1;
+                } else {
+                    tab.row_unit0[row] = u0;
+                    for (int t = 0; t < nu; ++t) tab.unit_row[u0 + t] = (int)row;
+                }
             }
         }
     }
@@ -779,8 +846,11 @@ __global__ void __launch_bounds__(FR_THREADS) finish_rows_kernel(int m, RowTable
         }
     }
     if (last_block(&ctl->rows_done, tiles)) {
-        if (tid == 0) ctl->n_units = ctl->hub_units + ctl->other_cursor;
-        __threadfence();
+        if (tid == 0) {
+            int n = 0;
+            for (int k = 0; k < UNIT_BUCKETS; ++k) n += ctl->unit_cursor[k];
+            ctl->n_units = n;
+        }
         __syncthreads();
         if (!TTM) publish_ctl(ctl, host);           // (the slice level comes after the fibres)
     }

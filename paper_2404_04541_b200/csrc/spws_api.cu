@@ -74,7 +74,8 @@ struct spws_plan_s {
     int64_t m = 0;
     void* scratch = nullptr;
     int max_span_words = 0;     // widest dense bitmap of the last symbolic pass
-    int max_warp_cnt = 0;       // most outputs of a warp-numeric row
+    int n_warp[N_WARP_LISTS] = {};          // rows on the warp numeric kernel's lists ...
+    int max_warp_cnt[N_WARP_LISTS] = {};    // ... and their largest output counts
     int64_t max_ub_smem = 0;    // most products of a shared-memory ISM row
     bool counters_clear = false; // the numeric pass's work counters are as the symbolic pass left them: zero
     bool rows_path = false;     // the last symbolic pass was a row-wise one, whose errors reach host->ctl.status by themselves
@@ -382,6 +383,8 @@ LaunchCtx make_ctx(const spws_plan_s* p, char* scratch, size_t scratch_bytes, co
     c.prm.max_span_words = (p->opt.dense_max_span + 31) / 32;
     c.prm.span_words_per_product = p->opt.dense_span_words_per_product;
     c.prm.unit_cap = L.unit_cap;
+    // rows of more than 256 outputs stay with a warp under `auto` only (and within the outputs a unit is given)
+    c.prm.warp_outputs = p->policy == SPWS_AUTO ? std::max(DENSE_WARP_ACC, std::min(DENSE_WARP_ACC2, p->opt.dense_unit_outputs)) : DENSE_WARP_ACC;
     c.rest = scratch + L.rest;
     c.rest_bytes = scratch_bytes > L.rest ? scratch_bytes - L.rest : 0;
     c.prm.bm_arena_words = (p->policy == SPWS_SPARSE_ISM || p->policy == SPWS_HASH) ? 0 : c.rest_bytes / 4;
@@ -555,12 +558,15 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
         plan->stats.nnz_per_class[public_class(k)] += hc.class_nnz[k];
     }
     plan->stats.dense_units = hc.n_units;
-    plan->stats.dense_warp_rows = hc.n_warp_rows;
+    plan->stats.dense_warp_rows = (int64_t)hc.n_warp_rows[0] + hc.n_warp_rows[1];
     plan->stats.dense_warp_products = hc.dense_warp_products;
     plan->stats.dense_warp_nnz = hc.dense_warp_nnz;
     plan->stats.bitmap_bytes = (int64_t)hc.bm_words_used * 4;
     plan->max_span_words = hc.max_span_words;
-    plan->max_warp_cnt = hc.max_warp_cnt;
+    for (int list = 0; list < N_WARP_LISTS; ++list) {
+        plan->n_warp[list] = hc.n_warp_rows[list];
+        plan->max_warp_cnt[list] = hc.max_warp_cnt[list];
+    }
     plan->stats.launches_symbolic = c.launches;
     return SPWS_OK;
 }
@@ -586,7 +592,7 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, con
         mark(plan, SPWS_T_NUM_ISM_SMEM);
     }
     if (s.dense_warp_rows > 0) {
-        CUDA_TRY(launch_dense_num_warp(c, (int)s.dense_warp_rows, plan->max_span_words, plan->max_warp_cnt, S.A, S.B, rowptr, crd, val));
+        CUDA_TRY(launch_dense_num_warp(c, plan->n_warp, plan->max_warp_cnt, (int)S.m, plan->max_span_words, S.A, S.B, rowptr, crd, val));
         mark(plan, SPWS_T_NUM_DENSE_WARP);
     }
     if (s.dense_units > 0) {
@@ -1531,14 +1537,14 @@ spws_status_t spws_gather_ceiling(spws_plan_t plan, const spws_tensor_t* A, cons
     char* sc = static_cast<char*>(scratch);
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, L);
     const i64* rowptr = (plan->kind == 0) ? LL(C->pos[1]) : reinterpret_cast<const i64*>(sc + L.rowptr_raw);
-    CUDA_TRY(cudaMemsetAsync(c.ctl->work_counter + CEIL_SLOT, 0, sizeof(int) * NCLASS, c.stream));
+    CUDA_TRY(cudaMemsetAsync(c.ctl->work_counter + CEIL_SLOT, 0, sizeof(int) * (CEIL_WARP_SLOT + N_WARP_LISTS - CEIL_SLOT), c.stream));
     CUDA_TRY(cudaMemsetAsync(index_sum, 0, sizeof(uint64_t), c.stream));
     CUDA_TRY(cudaMemsetAsync(value_sum, 0, sizeof(double), c.stream));
     mark_start(plan, 2);
     const spws_stats_t& s = plan->stats;
     u64* ci = reinterpret_cast<u64*>(index_sum);
     if (s.dense_warp_rows > 0) {
-        CUDA_TRY(launch_dense_num_warp(c, (int)s.dense_warp_rows, plan->max_span_words, plan->max_warp_cnt, S.A, S.B, rowptr, nullptr, nullptr, ci, value_sum));
+        CUDA_TRY(launch_dense_num_warp(c, plan->n_warp, plan->max_warp_cnt, (int)S.m, plan->max_span_words, S.A, S.B, rowptr, nullptr, nullptr, ci, value_sum));
         mark(plan, SPWS_T_CEIL_DENSE_WARP);
     }
     if (s.dense_units > 0) {

@@ -240,6 +240,41 @@ def test_warp_dense_route_compact_and_full_bitmaps(ctx, oracle_mod):
     assert 0 < stats["dense_warp_rows"] < 72 and stats["dense_units"] > 0
 
 
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("blen", [5, 40, 700])
+def test_warp_dense_rows_at_the_accumulators_edges(ctx, oracle_mod, blen, dtype):
+    """Rows whose output counts lie at the two accumulator sizes of the warp numeric kernel and just beyond, and rows at the most products a warp is given; short B rows (atomics) and long ones
+    (sums in loop order: bit for bit)."""
+    rng = np.random.default_rng(blen)
+    ncols = 30000
+    targets = [200, 255, 256, 257, 700, 1023, 1024, 1025, 2000, 4096, 9000]
+    rows, cols, brows, k = [], [], [], 0
+    for i, t in enumerate(targets):                     # row i: t distinct columns, each B row `blen` of them, all covered twice
+        own = np.sort(rng.choice(ncols, t, replace=False))
+        for rep in range(2):
+            for part in np.array_split(rng.permutation(own), max(1, t // blen)):
+                brows.append(np.sort(part)); rows.append(i); cols.append(k); k += 1
+    for i, n in ((len(targets), 4096), (len(targets) + 1, 4097)):         # rows of n products on 900 columns
+        own = np.sort(rng.choice(ncols, 900, replace=False))
+        left = n
+        while left:
+            take = min(left, blen)
+            brows.append(np.sort(rng.choice(own, take, replace=False))); rows.append(i); cols.append(k); k += 1
+            left -= take
+    pos = np.concatenate([[0], np.cumsum([len(b) for b in brows])]).astype(np.int64)
+    B = CSR(k, ncols, pos, np.concatenate(brows).astype(np.int32), rng.uniform(-1, 1, int(pos[-1])).astype(dtype))
+    A = CSR.from_coo(len(targets) + 2, k, rows, cols, rng.uniform(-1, 1, len(rows)), dtype=dtype)
+    ref = oracle_mod.spgemm(A, B, threads=4)
+    assert list(np.diff(ref.pos)[:len(targets)]) == targets
+    pos, crd, val, stats = run_spgemm(ctx, A, B, "auto")
+    assert_matches((pos, crd, val), ref, dtype)
+    assert stats["dense_units"] >= 1 and (blen == 5 or stats["dense_warp_rows"] >= 7)
+    if blen > 16 and dtype == np.float64:
+        upto = ref.pos[7]
+        assert np.array_equal(val[:upto], ref.val[:upto])
+    check_spgemm(ctx, oracle_mod, A, B, "auto", dense_unit_outputs=512)
+
+
 @pytest.mark.parametrize("summaries", [True, False])
 @pytest.mark.parametrize("per_row", [1, 2, 5, 10, 20])
 def test_bounds_kernel_widths_with_and_without_b_row_summaries(ctx, oracle_mod, per_row, summaries):
