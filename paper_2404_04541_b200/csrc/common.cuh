@@ -23,7 +23,7 @@ enum RowClass : int {
     CLS_ISM_GLOBAL = 9, // accumulation array in shared memory, all array in global memory
     CLS_HASH_S = 10,    // hash table in shared memory (reduction at insert time), small CTA
     CLS_HASH = 11,      // hash table in shared memory, full CTA
-    CLS_COPY8 = 12      // one A entry picking a B row of at most 8 entries: the result is that row, scaled
+    CLS_COPY = 12       // one A entry picking a B row of at most COPY_MAX entries: the result is that row, scaled
 };
 constexpr int NUM_SLOT = 16;   // work_counter[cls] in the symbolic pass, work_counter[NUM_SLOT + cls] in the numeric pass
 constexpr int CEIL_SLOT = 32;  // work_counter[CEIL_SLOT + cls] in the gather-only (iteration-only) kernels
@@ -52,6 +52,7 @@ constexpr int DENSE_MAX_SPAN_WORDS = 16384;// 2^19 columns: the widest bitmap (8
 // Word lists of long B rows (symbolic pass of the CTA dense route): a B row with at least
 // BW_MIN_LEN entries whose entries share bitmap words is also kept as (word index, bits) pairs,
 // so that a row that picks it sets one word per pair instead of one bit per entry.
+constexpr int COPY_MAX = 256;        // entries of the B row a copied row may pick (eight lanes copy a row)
 constexpr int LONG_A_ROW = 1024;     // entries of an A row beyond which a whole CTA computes its bounds
 constexpr int BW_MIN_LEN = 256;
 constexpr i64 BW_MAX_NNZ = 1ll << 26;      // lists are built only for a B with at most this many entries
@@ -384,8 +385,8 @@ size_t look_words(i64 rows, i64 slices);
 // exclusive scan of n counts into n + 1 positions
 cudaError_t launch_scan_counts(const LaunchCtx& c, const int* cnt, int n, i64* out, i64* block_sums, i64* total_out);
 // class kernels: n_host < 0 means "size the grid for any count"
-cudaError_t launch_ism_reg(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B,
-                           const i64* rowptr, int* Ccrd, void* Cval);
+// rows[cls] = rows of the three register classes and of the copied class, in ONE launch
+cudaError_t launch_ism_reg(const LaunchCtx& c, bool numeric, const i64* rows, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval);
 cudaError_t launch_ism_smem(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B,
                             const i64* rowptr, int* Ccrd, void* Cval);
 cudaError_t launch_dense_sym_warp(const LaunchCtx& c, const Csr& A, const Csr& B);

@@ -55,9 +55,12 @@ __device__ __forceinline__ int classify_row(i64 ub, i64 entries, int jmin, int j
         if (!dense_ok) { raise_status(ctl, DEV_WORKSPACE_TOO_LARGE); return CLS_EMPTY; }
         return dense_class(ub, span_words);
     }
-    // a single entry picking a short B row: Insert, Sort and Merge are the identity and the
-    // output count is the B row's length, known right here
-    const int reg_cls = ub <= 8 ? (entries == 1 ? CLS_COPY8 : CLS_ISM_REG8) : (ub <= 16 ? CLS_ISM_REG16 : CLS_ISM_REG);
+    // a single entry: Insert, Sort and Merge are the identity and the output count is the B row's length,
+    // known right here (up to COPY_MAX entries, which eight lanes copy; SpTTM with 41-entry rows, two
+    // thirds of them from one entry: 1421 us through the warp dense workspace, 534 us with those copied and
+    // most of the others through the register sort)
+    if (entries == 1 && ub <= COPY_MAX && prm.policy != 3) return CLS_COPY;
+    const int reg_cls = ub <= 8 ? CLS_ISM_REG8 : (ub <= 16 ? CLS_ISM_REG16 : CLS_ISM_REG);
     if (prm.policy == 1) {                       // sparse ISM forced
         if (reg_ok) return reg_cls;
         if (ub <= prm.smem_small_cap) return CLS_ISM_SMEM_S;
@@ -163,7 +166,7 @@ __device__ __forceinline__ void long_row_bounds(int row, const Csr& A, const Csr
         tab.ub[row] = u;
         tab.jmin[row] = lo;
         tab.jmax[row] = hi;
-        tab.cnt[row] = cls == CLS_COPY8 ? (int)u : 0;
+        tab.cnt[row] = cls == CLS_COPY ? (int)u : 0;
         tab.cls[row] = (unsigned char)cls;
         atomicAdd(&ctl->class_count[cls], 1);
         if (u) {
@@ -181,7 +184,7 @@ __device__ __forceinline__ void long_row_bounds(int row, const Csr& A, const Csr
 // SUMMARY: brow holds the B-row summaries (the instantiation without them carries B's own arrays'
 // two-level gathers and needs more registers).
 template <int G, bool SUMMARY>
-__global__ void __launch_bounds__(256, SUMMARY ? 6 : 5) row_bounds_kernel(Csr A, Csr B, RowTables tab, ClassParams prm, DevCtl* ctl,
+__global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A, Csr B, RowTables tab, ClassParams prm, DevCtl* ctl,
                                                          const int4* __restrict__ brow) {
     // rows and products per class, one histogram per warp: 64-bit shared-memory adds are
     // compare-and-swap loops, which many threads on one address turn into a queue
@@ -209,14 +212,30 @@ __global__ void __launch_bounds__(256, SUMMARY ? 6 : 5) row_bounds_kernel(Csr A,
     // class, so the shared-memory histogram is touched only when the class changes
     int run_cls = -1, run_rows = 0, my_span_words = 0;
     i64 run_products = 0;
+    // the next row's range and this lane's first entry of it are loaded while the current row is in hand: with
+    // a few entries per row the kernel is a chain of dependent loads otherwise
+    i64 ps_n = 0, pe_n = 0;
+    int k_n = -1;
+    if (group < A.nrows) {
+        ps_n = A.pos[group];
+        pe_n = A.pos[group + 1];
+        if (ps_n + gl < pe_n) k_n = __ldg(A.crd + ps_n + gl);
+    }
     for (i64 row = group; row < A.nrows; row += ngroups) {
-        const i64 ps = A.pos[row], pe = A.pos[row + 1];
+        const i64 ps = ps_n, pe = pe_n;
+        const int k_first = k_n;
+        const bool more = row + ngroups < A.nrows;
+        if (more) {
+            ps_n = A.pos[row + ngroups];
+            pe_n = A.pos[row + ngroups + 1];
+        }
         if (pe - ps > LONG_A_ROW) {
             int at = 0;
             if (gl == 0) at = atomicAdd(&s_nlong, 1);
             at = __shfl_sync(gmask, at, 0, G);
             if (at < LONG_LIST) {
                 if (gl == 0) s_long[at] = (int)row;
+                if (more && ps_n + gl < pe_n) k_n = __ldg(A.crd + ps_n + gl);
                 continue;
             }
         }
@@ -228,7 +247,7 @@ __global__ void __launch_bounds__(256, SUMMARY ? 6 : 5) row_bounds_kernel(Csr A,
         i64 p0 = ps + gl;
         if (pe - ps <= G) {                         // the common short row: one entry per lane
             if (p0 < pe) {
-                const int k = __ldg(A.crd + p0);
+                const int k = k_first;
                 if ((unsigned)k < (unsigned)B.nrows) {
                     if (SUMMARY) {
                         const int4 s = __ldg(brow + k);
@@ -283,6 +302,7 @@ __global__ void __launch_bounds__(256, SUMMARY ? 6 : 5) row_bounds_kernel(Csr A,
                 }
             }
         }
+        if (more && ps_n + gl < pe_n) k_n = __ldg(A.crd + ps_n + gl);
 #pragma unroll
         for (int d = G / 2; d > 0; d >>= 1) {
             u += __shfl_xor_sync(gmask, u, d, G);
@@ -295,9 +315,11 @@ __global__ void __launch_bounds__(256, SUMMARY ? 6 : 5) row_bounds_kernel(Csr A,
             if (u > 0) lo &= ~31;               // bitmap words of every row start at a multiple of 32 columns
             const int cls = classify_row(u, pe - ps, lo, hi, prm, ctl);
             tab.ub[row] = u;
-            tab.jmin[row] = lo;
-            tab.jmax[row] = hi;
-            tab.cnt[row] = cls == CLS_COPY8 ? (int)u : 0;
+            if (cls != CLS_COPY && cls != CLS_EMPTY) {      // (nothing reads the span of these)
+                tab.jmin[row] = lo;
+                tab.jmax[row] = hi;
+            }
+            tab.cnt[row] = cls == CLS_COPY ? (int)u : 0;
             tab.cls[row] = (unsigned char)cls;
             if (cls != run_cls) {
                 if (run_rows) {
@@ -502,7 +524,12 @@ __global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, 
         for (int x = 0; x < 4; ++x) {
             const i64 row = r0 + x * blockDim.x + threadIdx.x;
             words[x] = 0;
-            if (cls[x] >= 0) rank[x] = atomicAdd(&s_hist[cls[x]], 1);
+            // one addition per class among the 32 rows (a block of like rows would queue at one counter otherwise)
+            const unsigned peers = __match_any_sync(0xffffffffu, cls[x]);
+            const int first = __ffs(peers) - 1;
+            int at = 0;
+            if (cls[x] >= 0 && (int)(threadIdx.x & 31) == first) at = atomicAdd(&s_hist[cls[x]], __popc(peers));
+            rank[x] = __shfl_sync(0xffffffffu, at, first) + __popc(peers & ((1u << (threadIdx.x & 31)) - 1u));
             if (cls[x] == CLS_DENSE_WARP || cls[x] == CLS_DENSE_HUB || cls[x] == CLS_DENSE_CTA) {
                 const int nw = (tab.jmax[row] - tab.jmin[row]) / 32 + 1;
                 words[x] = (nw + (nw + 31) / 32 + 3) & ~3;

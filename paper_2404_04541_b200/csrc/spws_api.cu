@@ -492,24 +492,23 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
         return from_dev_status(hc.status);
     }
     plan->in_flight = true;
-    int hcount[NCLASS];
+    i64 hcount[NCLASS];
     for (int k = 0; k < NCLASS; ++k) hcount[k] = hc.class_count[k];
     const bool any_dense = hcount[CLS_DENSE_WARP] + hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0;
     plan->max_ub_smem = hc.max_ub_smem;
     c.max_ub_smem = plan->max_ub_smem;
     // a3: exact count per row through the workspace of its class
     if (S.m > 0) {
-        for (int cls = CLS_ISM_REG8; cls <= CLS_ISM_REG; ++cls)
-            if (hcount[cls] > 0) {
-                CUDA_TRY(launch_ism_reg(c, false, cls, hcount[cls], S.A, S.B, rowptr, nullptr, nullptr));
-                mark(plan, SPWS_T_SYM_ISM_REG);
-            }
+        if (hcount[CLS_ISM_REG8] + hcount[CLS_ISM_REG16] + hcount[CLS_ISM_REG] > 0) {
+            CUDA_TRY(launch_ism_reg(c, false, hcount, S.A, S.B, rowptr, nullptr, nullptr));
+            mark(plan, SPWS_T_SYM_ISM_REG);
+        }
         if (hcount[CLS_ISM_SMEM_S] > 0) {
-            CUDA_TRY(launch_ism_smem(c, false, CLS_ISM_SMEM_S, hcount[CLS_ISM_SMEM_S], S.A, S.B, rowptr, nullptr, nullptr));
+            CUDA_TRY(launch_ism_smem(c, false, CLS_ISM_SMEM_S, (int)hcount[CLS_ISM_SMEM_S], S.A, S.B, rowptr, nullptr, nullptr));
             mark(plan, SPWS_T_SYM_ISM_SMEM_S);
         }
         if (hcount[CLS_ISM_SMEM] > 0) {
-            CUDA_TRY(launch_ism_smem(c, false, CLS_ISM_SMEM, hcount[CLS_ISM_SMEM], S.A, S.B, rowptr, nullptr, nullptr));
+            CUDA_TRY(launch_ism_smem(c, false, CLS_ISM_SMEM, (int)hcount[CLS_ISM_SMEM], S.A, S.B, rowptr, nullptr, nullptr));
             mark(plan, SPWS_T_SYM_ISM_SMEM);
         }
         if (hcount[CLS_DENSE_WARP] > 0) {
@@ -522,12 +521,12 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
             mark(plan, SPWS_T_SYM_DENSE_CTA);
         }
         if (hcount[CLS_ISM_GLOBAL] > 0) {
-            CUDA_TRY(launch_ism_global(c, false, hcount[CLS_ISM_GLOBAL], S.A, S.B, rowptr, nullptr, nullptr));
+            CUDA_TRY(launch_ism_global(c, false, (int)hcount[CLS_ISM_GLOBAL], S.A, S.B, rowptr, nullptr, nullptr));
             mark(plan, SPWS_T_SYM_ISM_GLOBAL);
         }
         for (int cls = CLS_HASH_S; cls <= CLS_HASH; ++cls)
             if (hcount[cls] > 0) {
-                CUDA_TRY(launch_hash(c, false, cls, hcount[cls], S.A, S.B, rowptr, nullptr, nullptr));
+                CUDA_TRY(launch_hash(c, false, cls, (int)hcount[cls], S.A, S.B, rowptr, nullptr, nullptr));
                 mark(plan, SPWS_T_SYM_HASH);
             }
     }
@@ -578,11 +577,10 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, con
     c.max_ub_smem = plan->max_ub_smem;
     const spws_stats_t& s = plan->stats;
     const int64_t* bins = plan->bin_rows;
-    for (int cls : {(int)CLS_COPY8, (int)CLS_ISM_REG8, (int)CLS_ISM_REG16, (int)CLS_ISM_REG})
-        if (bins[cls] > 0) {
-            CUDA_TRY(launch_ism_reg(c, true, cls, (int)bins[cls], S.A, S.B, rowptr, crd, val));
-            mark(plan, SPWS_T_NUM_ISM_REG);
-        }
+    if (bins[CLS_COPY] + bins[CLS_ISM_REG8] + bins[CLS_ISM_REG16] + bins[CLS_ISM_REG] > 0) {
+        CUDA_TRY(launch_ism_reg(c, true, LL(bins), S.A, S.B, rowptr, crd, val));
+        mark(plan, SPWS_T_NUM_ISM_REG);
+    }
     if (bins[CLS_ISM_SMEM_S] > 0) {
         CUDA_TRY(launch_ism_smem(c, true, CLS_ISM_SMEM_S, (int)bins[CLS_ISM_SMEM_S], S.A, S.B, rowptr, crd, val));
         mark(plan, SPWS_T_NUM_ISM_SMEM_S);

@@ -241,6 +241,29 @@ def test_warp_dense_route_compact_and_full_bitmaps(ctx, oracle_mod):
 
 
 @pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("others", [0, 40, 5000])
+def test_copied_rows(ctx, oracle_mod, others, dtype):
+    """Rows with one entry are copied out, scaled: B rows at the lengths the eight copying lanes and the class
+    end at (256 entries), among few rows of other kinds (all rows walked in order) and among many (a list of
+    the copied ones).  One product per output: exact."""
+    rng = np.random.default_rng(others)
+    lens = [0, 1, 7, 8, 9, 31, 32, 33, 255, 256, 257, 300]
+    n = 1 << 16
+    brows = [np.sort(rng.choice(n, t, replace=False)) for t in lens]
+    pos = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    B = CSR(len(lens), n, pos, np.concatenate(brows).astype(np.int32), rng.uniform(-1, 1, int(pos[-1])).astype(dtype))
+    per = np.concatenate([np.ones(1500, int), rng.choice([0, 2, 3], size=others)])
+    rng.shuffle(per)
+    cols = [np.sort(rng.choice(len(lens), p, replace=False)) for p in per]
+    apos = np.concatenate([[0], np.cumsum(per)]).astype(np.int64)
+    A = CSR(len(per), len(lens), apos, np.concatenate(cols).astype(np.int32), rng.uniform(-1, 1, int(apos[-1])).astype(dtype))
+    for policy in ("auto", "ism"):
+        stats = check_spgemm(ctx, oracle_mod, A, B, policy, exact_values=others == 0)
+        copied = sum(len(c) == 1 and 0 < lens[c[0]] <= 256 for c in cols)
+        assert stats["rows_per_class"][1] >= copied
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
 @pytest.mark.parametrize("blen", [5, 40, 700])
 def test_warp_dense_rows_at_the_accumulators_edges(ctx, oracle_mod, blen, dtype):
     """Rows whose output counts lie at the two accumulator sizes of the warp numeric kernel and just beyond, and rows at the most products a warp is given; short B rows (atomics) and long ones
