@@ -101,7 +101,11 @@ typedef enum { SPWS_DENSE = 0, SPWS_SPARSE_ISM = 1, SPWS_AUTO = 2, SPWS_HASH = 3
  * spws_numeric; spws_symbolic overwrites n[] with the sizes of the result. */
 typedef struct {
     int32_t order;          /* 2 or 3 */
-    int32_t reserved;
+    union {
+        int32_t reserved;   /* 0 */
+        int32_t interleaved;/* COO result: 1 = crd[0] takes all coordinates entry by entry (n[0] x order),
+                               crd[1], crd[2] are not used; 0 = one array per index                  */
+    };
     int64_t dims[3];
     int64_t n[3];
     int64_t* pos[3];

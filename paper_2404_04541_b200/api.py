@@ -196,12 +196,13 @@ class Context:
             out = B_.TensorArrays(order, dims, [None, None, None], [None, None, None], None, [0, 0, 0])
             sc, nbytes = self._symbolic(plan, t, c, out, d)
             nnz = out.n[0]
-            crd = [torch.empty(nnz, dtype=torch.int32, device=self.device) for _ in range(order)]
-            out.crd = crd + [None] * (3 - order)
+            crd = torch.empty((nnz, order), dtype=torch.int32, device=self.device)
+            out.crd = [crd, None, None]
+            out.interleaved = 1
             out.val = torch.empty(nnz, dtype=T.val.dtype, device=self.device)
             out.n = [nnz, 0, 0]
             plan.numeric(t, c, out, self._aligned_ptr(sc), nbytes, D=d)
-            return torch.stack(crd, dim=1) if nnz else torch.empty((0, order), dtype=torch.int32, device=self.device), out.val, plan.get_stats()
+            return crd, out.val, plan.get_stats()
         finally:
             plan.close()
 

@@ -46,7 +46,7 @@ CLASS_NAMES = ("empty", "ism_reg", "ism_smem_s", "ism_smem", "dense_warp", "dens
 
 
 class spws_tensor_t(ctypes.Structure):
-    _fields_ = [("order", ctypes.c_int32), ("reserved", ctypes.c_int32),
+    _fields_ = [("order", ctypes.c_int32), ("interleaved", ctypes.c_int32),
                 ("dims", ctypes.c_int64 * 3), ("n", ctypes.c_int64 * 3),
                 ("pos", ctypes.c_void_p * 3), ("crd", ctypes.c_void_p * 3), ("val", ctypes.c_void_p)]
 
@@ -160,10 +160,11 @@ class TensorArrays:
     crd: list
     val: object
     n: list = field(default_factory=lambda: [0, 0, 0])
+    interleaved: int = 0        # coordinate-form result: 1 = crd[0] takes the coordinates entry by entry
 
     def c_struct(self) -> spws_tensor_t:
         d, n, pos, crd = self.dims, self.n, self.pos, self.crd
-        return spws_tensor_t(self.order, 0, (int(d[0]), int(d[1]), int(d[2]) if len(d) > 2 else 0), (int(n[0]), int(n[1]), int(n[2])),
+        return spws_tensor_t(self.order, self.interleaved, (int(d[0]), int(d[1]), int(d[2]) if len(d) > 2 else 0), (int(n[0]), int(n[1]), int(n[2])),
                              (_ptr(pos[0]), _ptr(pos[1]), _ptr(pos[2])), (_ptr(crd[0]), _ptr(crd[1]), _ptr(crd[2])), _ptr(self.val))
 
 

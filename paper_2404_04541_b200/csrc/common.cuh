@@ -423,7 +423,7 @@ cudaError_t launch_higher_ism(const LaunchCtx& c, bool numeric, int form, const 
                               const int* slice_of, const i64* eoff, i64 P, i64 cap, u64 d1, u64 d2, int label_bits, u64* kA, void* vA,
                               u64* kB, void* vB, char* sort_tmp, i64* nnz_dev, i64* nnz_host_pinned, bool* result_first);
 cudaError_t launch_higher_unpack(const LaunchCtx& c, int order, const u64* ukeys, const void* uvals, i64 nnz, u64 d1, u64 d2, int* o0,
-                                 int* o1, int* o2, void* oval);
+                                 int* o1, int* o2, void* oval, bool interleaved);
 
 // rowwise.cu: the same forms taken row by row
 size_t rw_sort_bytes(i64 n);
@@ -433,6 +433,6 @@ cudaError_t launch_rw_values(const LaunchCtx& c, const void* val, const int* src
 cudaError_t launch_rw_fibre_rows(const LaunchCtx& c, bool values, const Csf3Dev& B, const Csr& C, const Csr& D, int* cnt, i64* fpos, int* fcrd,
                                  void* fval, i64* block_sums);
 cudaError_t launch_rw_coords(const LaunchCtx& c, int order, const i64* rowptr, const u64* row_key, i64 m, i64 nnz, u64 d, const int* cols, int* o0,
-                             int* o1, int* o2);
+                             int* o1, int* o2, bool interleaved);
 
 }  // namespace spws

@@ -92,17 +92,17 @@ __global__ void __launch_bounds__(OT) higher_expand_kernel(int form, Csf3Dev B, 
 template <typename T>
 __global__ void __launch_bounds__(OT) higher_unpack_kernel(int order, const u64* __restrict__ ukeys, const T* __restrict__ uvals, i64 nnz,
                                                            u64 d1, u64 d2, int* __restrict__ o0, int* __restrict__ o1, int* __restrict__ o2,
-                                                           T* __restrict__ oval) {
+                                                           i64 step, T* __restrict__ oval) {
     for (i64 t = (i64)blockIdx.x * OT + threadIdx.x; t < nnz; t += (i64)gridDim.x * OT) {
         const u64 key = ukeys[t];
         if (order == 3) {
-            o2[t] = (int)(key % d2);
+            o2[t * step] = (int)(key % d2);
             const u64 r = key / d2;
-            o1[t] = (int)(r % d1);
-            o0[t] = (int)(r / d1);
+            o1[t * step] = (int)(r % d1);
+            o0[t * step] = (int)(r / d1);
         } else {
-            o1[t] = (int)(key % d2);
-            o0[t] = (int)(key / d2);
+            o1[t * step] = (int)(key % d2);
+            o0[t * step] = (int)(key / d2);
         }
         oval[t] = uvals[t];
     }
@@ -175,12 +175,14 @@ cudaError_t launch_higher_ism(const LaunchCtx& c, bool numeric, int form, const 
 }
 
 cudaError_t launch_higher_unpack(const LaunchCtx& c, int order, const u64* ukeys, const void* uvals, i64 nnz, u64 d1, u64 d2, int* o0,
-                                 int* o1, int* o2, void* oval) {
+                                 int* o1, int* o2, void* oval, bool interleaved) {
     if (nnz == 0) return cudaSuccess;
+    const i64 step = interleaved ? order : 1;
+    if (interleaved) { o1 = o0 + 1; o2 = o0 + 2; }
     if (c.is_f64)
-        higher_unpack_kernel<double><<<grid_for(c, nnz, OT), OT, 0, c.stream>>>(order, ukeys, (const double*)uvals, nnz, d1, d2, o0, o1, o2, (double*)oval);
+        higher_unpack_kernel<double><<<grid_for(c, nnz, OT), OT, 0, c.stream>>>(order, ukeys, (const double*)uvals, nnz, d1, d2, o0, o1, o2, step, (double*)oval);
     else
-        higher_unpack_kernel<float><<<grid_for(c, nnz, OT), OT, 0, c.stream>>>(order, ukeys, (const float*)uvals, nnz, d1, d2, o0, o1, o2, (float*)oval);
+        higher_unpack_kernel<float><<<grid_for(c, nnz, OT), OT, 0, c.stream>>>(order, ukeys, (const float*)uvals, nnz, d1, d2, o0, o1, o2, step, (float*)oval);
     ++c.launches;
     return cudaGetLastError();
 }

@@ -223,33 +223,81 @@ __global__ void __launch_bounds__(OT) rw_fibre_rows_kernel(Csf3Dev B, Csr C, Csr
 }
 
 // Coordinates of a coordinate-form result from its row pointer, row labels and columns.  A block takes a
-// tile of consecutive entries; the rows of the first and the last one bound every search.
+// tile of RC_TILE consecutive entries: the first entry of every row in the tile leaves the row's
+// coordinates in shared memory, a running maximum hands each entry the place of its row's first one,
+// and a thread writes the coordinates of its eight consecutive entries.  Bound by HBM.
+// 43e6 entries of three coordinates: 333 us for three arrays with a search per entry and 883 us to interleave
+// them, 274 us for the interleaved coordinates (516 MB out, 172 MB in).
 constexpr int RC_ITEMS = 8;
 constexpr int RC_TILE = OT * RC_ITEMS;
 
-__global__ void __launch_bounds__(OT) rw_coords_kernel(int order, const i64* __restrict__ rowptr, const u64* __restrict__ row_key, i64 m, i64 nnz,
-                                                       u64 d, const int* __restrict__ cols, int* __restrict__ o0, int* __restrict__ o1,
+template <int ORDER, bool INTERLEAVED>
+__global__ void __launch_bounds__(OT) rw_coords_kernel(const i64* __restrict__ rowptr, const u64* __restrict__ row_key, i64 m, i64 nnz, u64 d,
+                                                       const int* __restrict__ cols, int* __restrict__ o0, int* __restrict__ o1,
                                                        int* __restrict__ o2) {
-    __shared__ int s_lo, s_hi;
+    __shared__ int s_c0[RC_TILE], s_c1[ORDER == 3 ? RC_TILE : 1];
+    __shared__ __align__(16) int s_head[RC_TILE];       // entry i: i when a row starts there, else 0
+    __shared__ int s_lo, s_hi, s_warp[OT / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool vec = (((u64)o0 | (INTERLEAVED ? 0 : (u64)o1 | (u64)o2)) & 15) == 0;      // 16-byte stores
     for (i64 t0 = (i64)blockIdx.x * RC_TILE; t0 < nnz; t0 += (i64)gridDim.x * RC_TILE) {
         __syncthreads();
-        if (threadIdx.x == 0) s_lo = owner_row(rowptr, 0, (int)m, t0);
-        if (threadIdx.x == 32) s_hi = owner_row(rowptr, 0, (int)m, min(nnz, t0 + RC_TILE) - 1) + 1;
+        const i64 t1 = min(nnz, t0 + RC_TILE);
+        if (tid == 0) s_lo = owner_row(rowptr, 0, (int)m, t0);
+        if (tid == 32) s_hi = owner_row(rowptr, 0, (int)m, t1 - 1) + 1;
+        for (int i = tid; i < RC_TILE; i += OT) s_head[i] = 0;
         __syncthreads();
-        const int hi = s_hi;
-        int r = s_lo;                           // a thread's entries ascend, so each search starts at the last row found
-        for (int x = 0; x < RC_ITEMS; ++x) {
-            const i64 t = t0 + x * OT + threadIdx.x;
-            if (t >= nnz) break;
-            r = owner_row(rowptr, r, hi, t);
+        const int lo = s_lo, hi = s_hi;
+        for (int r = lo + tid; r < hi; r += OT) {
+            const i64 a = __ldg(rowptr + r), b = __ldg(rowptr + r + 1);
+            if (a == b) continue;
+            const int i = r == lo ? 0 : (int)(a - t0);  // (the first row may have begun before the tile)
             const u64 key = __ldg(row_key + r);
-            if (order == 3) {
-                o0[t] = (int)(key / d);
-                o1[t] = (int)(key % d);
-                o2[t] = __ldg(cols + t);
-            } else {
-                o0[t] = (int)key;
-                o1[t] = __ldg(cols + t);
+            s_c0[i] = ORDER == 3 ? (int)(key / d) : (int)key;
+            if (ORDER == 3) s_c1[i] = (int)(key % d);
+            s_head[i] = i;
+        }
+        __syncthreads();
+        int h[RC_ITEMS];
+        const int4 ha = reinterpret_cast<const int4*>(s_head)[2 * tid], hb = reinterpret_cast<const int4*>(s_head)[2 * tid + 1];
+        h[0] = ha.x; h[1] = ha.y; h[2] = ha.z; h[3] = ha.w; h[4] = hb.x; h[5] = hb.y; h[6] = hb.z; h[7] = hb.w;
+#pragma unroll
+        for (int x = 1; x < RC_ITEMS; ++x) h[x] = max(h[x], h[x - 1]);
+        int incl = h[RC_ITEMS - 1];
+#pragma unroll
+        for (int e = 1; e < 32; e <<= 1) incl = max(incl, __shfl_up_sync(0xffffffffu, incl, e));
+        if (lane == 31) s_warp[warp] = incl;
+        int before = __shfl_up_sync(0xffffffffu, incl, 1);
+        if (lane == 0) before = 0;
+        __syncthreads();
+        for (int w = 0; w < warp; ++w) before = max(before, s_warp[w]);
+        const int i0 = tid * RC_ITEMS;
+        if (vec && t0 + i0 + RC_ITEMS <= t1) {
+            int out[RC_ITEMS * ORDER], col[RC_ITEMS];       // entry by entry, or array by array
+            *reinterpret_cast<int4*>(col) = __ldg(reinterpret_cast<const int4*>(cols + t0 + i0));
+            *reinterpret_cast<int4*>(col + 4) = __ldg(reinterpret_cast<const int4*>(cols + t0 + i0) + 1);
+#pragma unroll
+            for (int x = 0; x < RC_ITEMS; ++x) {
+                const int at = max(h[x], before);
+                out[INTERLEAVED ? x * ORDER : x] = s_c0[at];
+                if (ORDER == 3) out[INTERLEAVED ? x * ORDER + 1 : x + RC_ITEMS] = s_c1[at];
+                out[INTERLEAVED ? x * ORDER + ORDER - 1 : x + (ORDER - 1) * RC_ITEMS] = col[x];
+            }
+#pragma unroll
+            for (int y = 0; y < RC_ITEMS * ORDER / 4; ++y) {
+                int* const to = INTERLEAVED ? o0 + (t0 + i0) * ORDER + 4 * y : (y < 2 ? o0 : y < 4 ? o1 : o2) + t0 + i0 + 4 * (y & 1);
+                *reinterpret_cast<int4*>(to) = make_int4(out[4 * y], out[4 * y + 1], out[4 * y + 2], out[4 * y + 3]);
+            }
+        } else {
+#pragma unroll
+            for (int x = 0; x < RC_ITEMS; ++x) {
+                const i64 t = t0 + i0 + x;
+                if (t >= t1) break;
+                const int at = max(h[x], before);
+                const i64 o = INTERLEAVED ? t * ORDER : t;
+                o0[o] = s_c0[at];
+                if (ORDER == 3) (INTERLEAVED ? o0 + 1 : o1)[o] = s_c1[at];
+                (INTERLEAVED ? o0 + ORDER - 1 : ORDER == 3 ? o2 : o1)[o] = __ldg(cols + t);
             }
         }
     }
@@ -331,9 +379,12 @@ cudaError_t launch_rw_fibre_rows(const LaunchCtx& c, bool values, const Csf3Dev&
 }
 
 cudaError_t launch_rw_coords(const LaunchCtx& c, int order, const i64* rowptr, const u64* row_key, i64 m, i64 nnz, u64 d, const int* cols, int* o0,
-                             int* o1, int* o2) {
+                             int* o1, int* o2, bool interleaved) {
     if (nnz == 0) return cudaSuccess;
-    rw_coords_kernel<<<grid_for(c, nnz, RC_TILE), OT, 0, c.stream>>>(order, rowptr, row_key, m, nnz, d, cols, o0, o1, o2);
+    const int grid = grid_for(c, nnz, RC_TILE);
+    auto k = order == 3 ? (interleaved ? rw_coords_kernel<3, true> : rw_coords_kernel<3, false>)
+                        : (interleaved ? rw_coords_kernel<2, true> : rw_coords_kernel<2, false>);
+    k<<<grid, OT, 0, c.stream>>>(rowptr, row_key, m, nnz, d, cols, o0, o1, o2);
     ++c.launches;
     return cudaGetLastError();
 }

@@ -1112,7 +1112,7 @@ spws_status_t rw_higher_numeric(spws_plan_s* plan, const HShapes& H, spws_tensor
     const spws_status_t st = rows_numeric(plan, w.S, c, rowptr, cols, Out->val);
     if (st != SPWS_OK) return st;
     CUDA_TRY(launch_rw_coords(c, H.order, rowptr, b.row_key, w.m, plan->stats.nnz, (u64)(H.order == 3 ? H.odims[1] : 1), cols, Out->crd[0],
-                              Out->crd[1], Out->crd[2]));
+                              Out->crd[1], Out->crd[2], Out->interleaved != 0));
     plan->stats.launches_numeric = c.launches;
     return SPWS_OK;
 }
@@ -1215,7 +1215,7 @@ spws_status_t higher_numeric(spws_plan_s* plan, const spws_tensor_t* B, const sp
     if (Out->n[0] < nnz) return SPWS_OUTPUT_TOO_SMALL;
     if (nnz > 0) {
         if (!Out->val) return SPWS_INVALID_ARGUMENT;
-        for (int a = 0; a < H.order; ++a) if (!Out->crd[a]) return SPWS_INVALID_ARGUMENT;
+        for (int a = 0; a < (Out->interleaved ? 1 : H.order); ++a) if (!Out->crd[a]) return SPWS_INVALID_ARGUMENT;
     }
     if (plan->rowwise) return rw_higher_numeric(plan, H, Out, scratch, scratch_bytes);
     const HLayout L = make_hlayout(plan, H, P);
@@ -1236,7 +1236,7 @@ spws_status_t higher_numeric(spws_plan_s* plan, const spws_tensor_t* B, const sp
                                sc + L.vA, reinterpret_cast<u64*>(sc + L.kB), sc + L.vB, sc + L.sort_tmp, &c.ctl->kept[0], nnz_host, &first));
     if (*nnz_host != nnz) return SPWS_BAD_SEQUENCE;                 // operands differ from the symbolic pass's
     CUDA_TRY(launch_higher_unpack(c, H.order, reinterpret_cast<u64*>(sc + (first ? L.kA : L.kB)), sc + (first ? L.vA : L.vB), nnz, H.d1, H.d2,
-                                  Out->crd[0], Out->crd[1], Out->crd[2], Out->val));
+                                  Out->crd[0], Out->crd[1], Out->crd[2], Out->val, Out->interleaved != 0));
     mark(plan, SPWS_T_NUM_ISM_GLOBAL);
     plan->stats.launches_numeric = c.launches;
     return SPWS_OK;

@@ -725,6 +725,35 @@ def test_scatters_taken_row_by_row(ctx, oracle_mod, dims, nnz, L, density, dtype
         assert ok.all(), expr
 
 
+@pytest.mark.parametrize("shift", [0, 1])
+@pytest.mark.parametrize("interleaved", [0, 1])
+@pytest.mark.parametrize("policy", ["auto", "ism"])
+def test_coordinates_in_arrays_or_entry_by_entry(ctx, oracle_mod, policy, interleaved, shift):
+    """Coordinate-form results in one array per index and entry by entry, at addresses that 16-byte stores
+    fit and that they do not; rows of the result that cross the tiles of 2048 entries."""
+    import torch
+    from paper_2404_04541_b200 import api, binding
+    T, M = uniform_csf3((30, 12, 40), 3000, 8), random_csr(30, 700, 0.2, 9, empty_row_frac=0.2)
+    ref = oracle_mod.spttm(T, M)
+    dT, dM = api.DeviceCSF3.from_host(T), api.DeviceCSR.from_host(M)
+    plan = ctx.plan(api.EXPR_SPTTM, (binding.SPWS_COO, binding.SPWS_CSF3, binding.SPWS_CSR), np.float64, policy)
+    out = binding.TensorArrays(3, (12, 40, 700), [None] * 3, [None] * 3, None, [0, 0, 0])
+    sc, nbytes = ctx._symbolic(plan, dT.arrays(), dM.arrays(), out)
+    n = out.n[0]
+    assert n == ref.nnz > 3 * 2048
+    flat = torch.full((3 * n + 8,), -7, dtype=torch.int32, device="cuda")
+    parts = [flat[shift:shift + 3 * n], None, None] if interleaved else [flat[shift + a * n:shift + (a + 1) * n] for a in range(3)]
+    out.crd, out.val, out.interleaved = parts, torch.empty(n, dtype=torch.float64, device="cuda"), interleaved
+    plan.numeric(dT.arrays(), dM.arrays(), out, ctx._aligned_ptr(sc), nbytes)
+    plan.get_stats()
+    plan.close()
+    got = parts[0].view(n, 3) if interleaved else torch.stack(parts, dim=1)
+    assert np.array_equal(got.cpu().numpy().astype(np.int64), ref.crd)
+    assert (flat[shift + 3 * n:] == -7).all() and (shift == 0 or flat[0] == -7)
+    ok, _ = values_close(out.val.cpu().numpy(), ref.val_ref, ref.abs, 1e-12)
+    assert ok.all()
+
+
 @pytest.mark.parametrize("m,k,n,dens", [(1, 1, 1, 1.0), (300, 20, 5000, 0.1), (2048, 33, 40, 0.02), (5, 3000, 1 << 19, 0.3), (5, 300, (1 << 19) + 1, 0.3)])
 def test_outer_product_taken_row_by_row(ctx, oracle_mod, m, k, n, dens):
     """`auto` sorts A's entries by output row; at the widest column space the row workspace covers and just
