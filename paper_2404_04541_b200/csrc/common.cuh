@@ -389,7 +389,8 @@ cudaError_t launch_scan_counts(const LaunchCtx& c, const int* cnt, int n, i64* o
 cudaError_t launch_ism_reg(const LaunchCtx& c, bool numeric, const i64* rows, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval);
 cudaError_t launch_ism_smem(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B,
                             const i64* rowptr, int* Ccrd, void* Cval);
-cudaError_t launch_dense_sym_warp(const LaunchCtx& c, const Csr& A, const Csr& B);
+// max_span_words: widest dense row of the pass
+cudaError_t launch_dense_sym_warp(const LaunchCtx& c, int max_span_words, const Csr& A, const Csr& B);
 cudaError_t launch_dense_sym_cta(const LaunchCtx& c, const Csr& A, const Csr& B);
 // chk_idx / chk_val non-null: the gather-only form of the same kernel (workspace stripped, checksums out).
 // n[], max_cnt[]: rows on each list and their largest output counts

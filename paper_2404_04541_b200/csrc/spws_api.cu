@@ -512,7 +512,7 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
             mark(plan, SPWS_T_SYM_ISM_SMEM);
         }
         if (hcount[CLS_DENSE_WARP] > 0) {
-            CUDA_TRY(launch_dense_sym_warp(c, S.A, S.B));
+            CUDA_TRY(launch_dense_sym_warp(c, hc.max_span_words, S.A, S.B));
             mark(plan, SPWS_T_SYM_DENSE_WARP);
         }
         if (hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0) {

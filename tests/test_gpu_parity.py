@@ -435,6 +435,26 @@ def test_wide_columns_with_many_products(ctx, oracle_mod, policy):
     check_spgemm(ctx, oracle_mod, Abig, B, policy)
 
 
+@pytest.mark.parametrize("words", [1, 31, 33, 255, 256, 257, 1024])
+@pytest.mark.parametrize("per_row", [2, 30, 70])
+def test_dense_warp_rows_at_the_span_that_chooses_the_counting(ctx, oracle_mod, words, per_row):
+    """Warp dense rows whose span is exactly the first / last column of `words` bitmap words: below and
+    above the width up to which the symbolic kernel counts by a scan of the bitmap, B rows shorter and
+    longer than a warp, and A rows of fewer and more entries than one batch of descriptors holds."""
+    n = 32 * words
+    per_row = min(per_row, n)
+    rng = np.random.default_rng(words)
+    crd = np.sort(np.argsort(rng.random((90, n)), axis=1)[:, :per_row], axis=1).astype(np.int32)
+    crd[:, 0], crd[:, -1] = 0, n - 1
+    crd = [np.unique(c) for c in crd]
+    B = CSR(90, n, np.concatenate([[0], np.cumsum([c.size for c in crd])]), np.concatenate(crd), rng.uniform(-1, 1, sum(c.size for c in crd)))
+    lengths = [1, 2, 31, 32, 33, 50]
+    A = CSR.from_coo(len(lengths), 90, np.repeat(np.arange(len(lengths)), lengths),
+                     np.concatenate([np.sort(rng.choice(90, x, replace=False)) for x in lengths]), rng.uniform(-1, 1, sum(lengths)))
+    stats = check_spgemm(ctx, oracle_mod, A, B, "dense")
+    assert stats["rows_per_class"][4] == len(lengths)
+
+
 def test_dense_cta_widest_span_and_just_beyond(ctx, oracle_mod):
     """Rows whose outputs cover almost 2^19 columns (the widest dense workspace one CTA holds, with
     the whole bitmap and its ranks in shared memory) and rows a little wider, which must fall back
