@@ -106,23 +106,20 @@ __global__ void __launch_bounds__(256) brow_summary_kernel(Csr B, int4* __restri
 }
 
 constexpr int LONG_LIST = 32;
+constexpr int MID_LIST = 64;
 
-// Bounds and class of one long row by a whole block: 256 lanes across the entries, four entries per lane
-// and step.
-template <bool SUMMARY>
-__device__ __forceinline__ void long_row_bounds(int row, const Csr& A, const Csr& B, const RowTables& tab, const ClassParams& prm, DevCtl* ctl,
-                                                const int4* __restrict__ brow) {
-    __shared__ i64 s_u[8];
-    __shared__ int s_lo[8], s_hi[8], s_bad[8];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const i64 ps = A.pos[row], pe = A.pos[row + 1];
-    i64 u = 0;
-    int lo = 0x7fffffff, hi = -1, bad = 0;
-    for (i64 p0 = ps + tid; p0 < pe; p0 += 4 * 256) {
+// Products and first / last column of the entries ps + at, ps + at + LANES, ..: four entries per step; the totals of
+// a warp's lanes are returned in every lane.
+template <bool SUMMARY, int LANES>
+__device__ __forceinline__ void entry_totals(i64 ps, i64 pe, int at, const Csr& A, const Csr& B, const int4* __restrict__ brow, i64& u, int& lo,
+                                             int& hi, int& bad) {
+    u = 0;
+    lo = 0x7fffffff, hi = -1, bad = 0;
+    for (i64 p0 = ps + at; p0 < pe; p0 += 4 * LANES) {
         int k[4];
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
-            const i64 p = p0 + (i64)x * 256;
+            const i64 p = p0 + (i64)x * LANES;
             k[x] = p < pe ? __ldg(A.crd + p) : -1;
             if (p < pe && (unsigned)k[x] >= (unsigned)B.nrows) bad = 1;
         }
@@ -154,6 +151,19 @@ __device__ __forceinline__ void long_row_bounds(int row, const Csr& A, const Csr
         hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, d));
         bad |= __shfl_xor_sync(0xffffffffu, bad, d);
     }
+}
+
+// Bounds and class of one long row by a whole block.
+template <bool SUMMARY>
+__device__ __forceinline__ void long_row_bounds(int row, const Csr& A, const Csr& B, const RowTables& tab, const ClassParams& prm, DevCtl* ctl,
+                                                const int4* __restrict__ brow) {
+    __shared__ i64 s_u[8];
+    __shared__ int s_lo[8], s_hi[8], s_bad[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const i64 ps = A.pos[row], pe = A.pos[row + 1];
+    i64 u;
+    int lo, hi, bad;
+    entry_totals<SUMMARY, 256>(ps, pe, tid, A, B, brow, u, lo, hi, bad);
     __syncthreads();                                   // the previous row's totals have been read
     if (lane == 0) { s_u[warp] = u; s_lo[warp] = lo; s_hi[warp] = hi; s_bad[warp] = bad; }
     __syncthreads();
@@ -186,32 +196,75 @@ __device__ __forceinline__ void long_row_bounds(int row, const Csr& A, const Csr
 template <int G, bool SUMMARY>
 __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A, Csr B, RowTables tab, ClassParams prm, DevCtl* ctl,
                                                          const int4* __restrict__ brow) {
-    // rows and products per class, one histogram per warp: 64-bit shared-memory adds are
-    // compare-and-swap loops, which many threads on one address turn into a queue
+    // rows and products per class, one histogram per warp: 64-bit shared-memory adds are compare-and-swap loops,
+    // which many threads on one address turn into a queue, so what fits is added in 32 bits (a thread's run of
+    // products below 2^16; a warp adds fewer than 2^16 of those)
     __shared__ int s_hist[8][NCLASS];
+    __shared__ unsigned s_clow[8][NCLASS];
     __shared__ i64 s_cprod[8][NCLASS];
     __shared__ i64 s_products, s_max_ub, s_max_ub_global, s_max_ub_smem;
     __shared__ int s_max_span_words;
     // rows of more than LONG_A_ROW entries, which the block's threads take together at the end: left to
     // its lane group such a row is a serial chain that sets the kernel's time on power-law inputs
     __shared__ int s_long[LONG_LIST], s_nlong;
-    for (int x = threadIdx.x; x < 8 * NCLASS; x += blockDim.x) { (&s_hist[0][0])[x] = 0; (&s_cprod[0][0])[x] = 0; }
-    if (threadIdx.x == 0) { s_products = 0; s_max_ub = 0; s_max_ub_global = 0; s_max_ub_smem = 0; s_max_span_words = 0; s_nlong = 0; }
+    // rows of more than two steps of a narrow lane group, which the block's warps take at the end
+    __shared__ int s_mid[MID_LIST], s_nmid;
+    for (int x = threadIdx.x; x < 8 * NCLASS; x += blockDim.x) { (&s_hist[0][0])[x] = 0; (&s_clow[0][0])[x] = 0; (&s_cprod[0][0])[x] = 0; }
+    if (threadIdx.x == 0) { s_products = 0; s_max_ub = 0; s_max_ub_global = 0; s_max_ub_smem = 0; s_max_span_words = 0; s_nlong = s_nmid = 0; }
     __syncthreads();
     int* const w_hist = s_hist[threadIdx.x >> 5];
     i64* const w_cprod = s_cprod[threadIdx.x >> 5];
+    unsigned* const w_clow = s_clow[threadIdx.x >> 5];
+    int low_adds = 0;                               // 32-bit additions of this thread
+    auto flush = [&](int cls, int rows, i64 products) {
+        if (rows) atomicAdd(&w_hist[cls], rows);
+        if (products == 0) return;
+        if (products < 65536 && low_adds < 2047) {  // 32 threads x 2047 additions x 65535 < 2^32
+            atomicAdd(&w_clow[cls], (unsigned)products);
+            ++low_adds;
+        } else {
+            atomicAdd((u64*)&w_cprod[cls], (u64)products);
+        }
+    };
     const int gl = threadIdx.x % G;
     const unsigned lane = threadIdx.x & 31;
     const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane - gl));
-    // a warp per row: neighbouring rows go to different blocks (the heaviest rows of a graph are often
+    // eight lanes or more per row: neighbouring rows go to different blocks (the heaviest rows of a graph are often
     // neighbours); narrower groups take neighbouring rows for the sake of the row offsets they share
     const i64 ngroups = ((i64)gridDim.x * blockDim.x) / G;
-    const i64 group = G == 32 ? (i64)(threadIdx.x >> 5) * gridDim.x + blockIdx.x : ((i64)blockIdx.x * blockDim.x + threadIdx.x) / G;
+    const i64 group = G >= 8 ? (i64)(threadIdx.x / G) * gridDim.x + blockIdx.x : ((i64)blockIdx.x * blockDim.x + threadIdx.x) / G;
     i64 my_products = 0, my_max = 0;
     // rows and products of the class of this group's last rows: neighbouring rows mostly share a
     // class, so the shared-memory histogram is touched only when the class changes
     int run_cls = -1, run_rows = 0, my_span_words = 0;
     i64 run_products = 0;
+    auto classify = [&](int row, i64 entries, i64 u, int lo, int hi) {
+        if (lo < 0 || hi >= B.ncols) { raise_status(ctl, DEV_NONCANONICAL); u = 0; }
+        if (u > 0) lo &= ~31;               // bitmap words of every row start at a multiple of 32 columns
+        const int cls = classify_row(u, entries, lo, hi, prm, ctl);
+        tab.ub[row] = u;
+        if (cls != CLS_COPY && cls != CLS_EMPTY) {      // (nothing reads the span of these)
+            tab.jmin[row] = lo;
+            tab.jmax[row] = hi;
+        }
+        tab.cnt[row] = cls == CLS_COPY ? (int)u : 0;
+        tab.cls[row] = (unsigned char)cls;
+        if (cls != run_cls) {
+            if (run_rows) flush(run_cls, run_rows, run_products);
+            run_cls = cls;
+            run_rows = 0;
+            run_products = 0;
+        }
+        ++run_rows;
+        run_products += u;
+        my_products += u;
+        my_max = max(my_max, u);
+        // (rare classes: straight to shared memory, and only when the maximum would move)
+        if (cls == CLS_ISM_GLOBAL && u > s_max_ub_global) atomicMax(&s_max_ub_global, u);
+        if (cls == CLS_ISM_SMEM && u > s_max_ub_smem) atomicMax(&s_max_ub_smem, u);
+        if (cls == CLS_DENSE_HUB || cls == CLS_DENSE_CTA || cls == CLS_DENSE_WARP)
+            my_span_words = max(my_span_words, (hi - lo) / 32 + 1);
+    };
     // the next row's range and this lane's first entry of it are loaded while the current row is in hand: with
     // a few entries per row the kernel is a chain of dependent loads otherwise
     i64 ps_n = 0, pe_n = 0;
@@ -229,12 +282,13 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
             ps_n = A.pos[row + ngroups];
             pe_n = A.pos[row + ngroups + 1];
         }
-        if (pe - ps > LONG_A_ROW) {
+        if (pe - ps > (G < 32 ? 8 * G : LONG_A_ROW)) {
+            const bool mid = G < 32 && pe - ps <= LONG_A_ROW;
             int at = 0;
-            if (gl == 0) at = atomicAdd(&s_nlong, 1);
+            if (gl == 0) at = atomicAdd(mid ? &s_nmid : &s_nlong, 1);
             at = __shfl_sync(gmask, at, 0, G);
-            if (at < LONG_LIST) {
-                if (gl == 0) s_long[at] = (int)row;
+            if (at < (mid ? MID_LIST : LONG_LIST)) {
+                if (gl == 0) (mid ? s_mid : s_long)[at] = (int)row;
                 if (more && ps_n + gl < pe_n) k_n = __ldg(A.crd + ps_n + gl);
                 continue;
             }
@@ -310,41 +364,23 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
             hi = max(hi, __shfl_xor_sync(gmask, hi, d, G));
         }
         if (bad) raise_status(ctl, DEV_NONCANONICAL);
-        if (gl == 0) {
-            if (lo < 0 || hi >= B.ncols) { raise_status(ctl, DEV_NONCANONICAL); u = 0; }
-            if (u > 0) lo &= ~31;               // bitmap words of every row start at a multiple of 32 columns
-            const int cls = classify_row(u, pe - ps, lo, hi, prm, ctl);
-            tab.ub[row] = u;
-            if (cls != CLS_COPY && cls != CLS_EMPTY) {      // (nothing reads the span of these)
-                tab.jmin[row] = lo;
-                tab.jmax[row] = hi;
+        if (gl == 0) classify((int)row, pe - ps, u, lo, hi);
+    }
+    if (G < 32) {
+        __syncthreads();
+        for (int r = threadIdx.x >> 5; r < min(s_nmid, MID_LIST); r += 8) {
+            const int row = s_mid[r];
+            const i64 ps = A.pos[row], pe = A.pos[row + 1];
+            i64 u;
+            int lo, hi, bad;
+            entry_totals<SUMMARY, 32>(ps, pe, (int)lane, A, B, brow, u, lo, hi, bad);
+            if (lane == 0) {
+                if (bad) raise_status(ctl, DEV_NONCANONICAL);
+                classify(row, pe - ps, u, lo, hi);
             }
-            tab.cnt[row] = cls == CLS_COPY ? (int)u : 0;
-            tab.cls[row] = (unsigned char)cls;
-            if (cls != run_cls) {
-                if (run_rows) {
-                    atomicAdd(&w_hist[run_cls], run_rows);
-                    if (run_products) atomicAdd((u64*)&w_cprod[run_cls], (u64)run_products);
-                }
-                run_cls = cls;
-                run_rows = 0;
-                run_products = 0;
-            }
-            ++run_rows;
-            run_products += u;
-            my_products += u;
-            my_max = max(my_max, u);
-            // (rare classes: straight to shared memory, and only when the maximum would move)
-            if (cls == CLS_ISM_GLOBAL && u > s_max_ub_global) atomicMax(&s_max_ub_global, u);
-            if (cls == CLS_ISM_SMEM && u > s_max_ub_smem) atomicMax(&s_max_ub_smem, u);
-            if (cls == CLS_DENSE_HUB || cls == CLS_DENSE_CTA || cls == CLS_DENSE_WARP)
-                my_span_words = max(my_span_words, (hi - lo) / 32 + 1);
         }
     }
-    if (gl == 0 && run_rows) {
-        atomicAdd(&w_hist[run_cls], run_rows);
-        if (run_products) atomicAdd((u64*)&w_cprod[run_cls], (u64)run_products);
-    }
+    if (gl == 0 && run_rows) flush(run_cls, run_rows, run_products);
     __syncthreads();
     for (int r = 0; r < min(s_nlong, LONG_LIST); ++r) long_row_bounds<SUMMARY>(s_long[r], A, B, tab, prm, ctl, brow);
     // the totals: reduced over the warp first (lanes other than a group's first hold zeros)
@@ -362,7 +398,7 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
     if (threadIdx.x < NCLASS) {
         int rows = 0;
         i64 prods = 0;
-        for (int w = 0; w < 8; ++w) { rows += s_hist[w][threadIdx.x]; prods += s_cprod[w][threadIdx.x]; }
+        for (int w = 0; w < 8; ++w) { rows += s_hist[w][threadIdx.x]; prods += s_cprod[w][threadIdx.x] + s_clow[w][threadIdx.x]; }
         if (rows) atomicAdd(&ctl->class_count[threadIdx.x], rows);
         if (prods) atomicAdd((u64*)&ctl->class_products[threadIdx.x], (u64)prods);
     }
@@ -398,7 +434,10 @@ cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i6
     if (avg <= 1.5) sm ? launch(row_bounds_kernel<1, true>, 1) : launch(row_bounds_kernel<1, false>, 1);
     else if (avg <= 3.0) sm ? launch(row_bounds_kernel<2, true>, 2) : launch(row_bounds_kernel<2, false>, 2);
     else if (avg <= 6.0) sm ? launch(row_bounds_kernel<4, true>, 4) : launch(row_bounds_kernel<4, false>, 4);
-    else if (avg <= 12.0) sm ? launch(row_bounds_kernel<8, true>, 8) : launch(row_bounds_kernel<8, false>, 8);
+    // (eight lanes take 32 entries in one step, four loads each, and the warps of a block take its longer rows at the
+    // end: a 27-point stencil of 2^18 rows 90 -> 47 us, a power law of 2^18 rows 122 -> 89 us against a warp
+    // per row; with so few rows that the longest sets the time a warp per row: power law of 16381 rows 28 -> 18 us)
+    else if (avg <= (A.nrows >= (1 << 16) ? 32.0 : 12.0)) sm ? launch(row_bounds_kernel<8, true>, 8) : launch(row_bounds_kernel<8, false>, 8);
     else sm ? launch(row_bounds_kernel<32, true>, 32) : launch(row_bounds_kernel<32, false>, 32);
     ++c.launches;
     return cudaGetLastError();
@@ -495,7 +534,7 @@ cudaError_t launch_bw_build(const LaunchCtx& c, const Csr& B) {
 // ---------------------------------------------------------------------------------------
 // It also counts the units per bucket of rows, clears the words of the kernels that hand running sums
 // from tile to tile, and its last block publishes the class sizes to the host.
-__global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, DevCtl* host, u64* look, int n_look) {
+__global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, HostBlock* host, u64* look, int n_look) {
     __shared__ int s_units[UNIT_BUCKETS];
     if (threadIdx.x < UNIT_BUCKETS) s_units[threadIdx.x] = 0;
     for (int w = blockIdx.x * 256 + threadIdx.x; w < n_look; w += gridDim.x * 256) look[w] = 0;
@@ -556,7 +595,9 @@ __global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, 
                 const u64 at = s_bm_base + (u64)my_off;
                 my_off += words[x];
                 if (at + (u64)words[x] > prm.bm_arena_words) {
-                    raise_status(ctl, DEV_SCRATCH_TOO_SMALL);
+                    // the reservations follow one another, so one row crosses the end: it alone reports (262144
+                    // rows queueing at the status word cost a first pass that guessed too small a scratch 190 us)
+                    if (at <= prm.bm_arena_words) raise_status(ctl, DEV_SCRATCH_TOO_SMALL);
                     tab.bm_off[row] = -1;
                 } else {
                     tab.bm_off[row] = (i64)at;
@@ -567,7 +608,7 @@ __global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, 
     }
     if (threadIdx.x < UNIT_BUCKETS && s_units[threadIdx.x]) atomicAdd(&ctl->units_of[threadIdx.x], s_units[threadIdx.x]);
     if (last_block(&ctl->bin_done, gridDim.x)) {
-        if (threadIdx.x == 0) ctl->host_status = &host->status;
+        if (threadIdx.x == 0) ctl->host_status = &host->ctl.status;
         __syncthreads();
         publish_ctl(ctl, host);
     }
@@ -577,7 +618,7 @@ cudaError_t launch_bin_rows(const LaunchCtx& c, int m) {
     i64 want = ((i64)m + 1023) / 1024;
     i64 cap = (i64)c.sm_count * 8;
     if (want < 1) want = 1;
-    bin_rows_kernel<<<(int)(want < cap ? want : cap), 256, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host_ctl, c.look, c.n_look);
+    bin_rows_kernel<<<(int)(want < cap ? want : cap), 256, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.look, c.n_look);
     ++c.launches;
     return cudaGetLastError();
 }
@@ -613,7 +654,7 @@ struct FibreArgs {
 };
 
 template <bool DENSE, bool TTM>
-__global__ void __launch_bounds__(FR_THREADS, 3) finish_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, DevCtl* host, u64* look,
+__global__ void __launch_bounds__(FR_THREADS, DENSE ? 3 : 5) finish_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, HostBlock* host, u64* look,
                                                                  i64* __restrict__ rowptr, FibreArgs f) {
     __shared__ int s_tile, s_slice0;
     __shared__ i64 s_sum[FR_WARPS], s_before[2];
@@ -885,7 +926,7 @@ __global__ void __launch_bounds__(FR_THREADS, 3) finish_rows_kernel(int m, RowTa
 
 // A slice i survives when one of its fibres does: C's slice level from sfp.
 __global__ void __launch_bounds__(FR_THREADS) finish_slices_kernel(int n_i, const i64* __restrict__ sfp, const int* __restrict__ Acrd0, DevCtl* ctl,
-                                                                   DevCtl* host, u64* look, int* __restrict__ Ccrd0, i64* __restrict__ Cpos1,
+                                                                   HostBlock* host, u64* look, int* __restrict__ Ccrd0, i64* __restrict__ Cpos1,
                                                                    i64* __restrict__ Cpos0) {
     __shared__ int s_tile, s_part[FR_WARPS];
     __shared__ i64 s_before;
@@ -949,8 +990,8 @@ size_t look_words(i64 rows, i64 slices) { return (size_t)2 * tiles_of(rows, FR_T
 
 cudaError_t launch_finish_rows(const LaunchCtx& c, int m, bool any_dense, i64* rowptr) {
     const int tiles = tiles_of(m, FR_TILE);
-    if (any_dense) finish_rows_kernel<true, false><<<tiles, FR_THREADS, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host_ctl, c.look, rowptr, FibreArgs{});
-    else finish_rows_kernel<false, false><<<tiles, FR_THREADS, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host_ctl, c.look, rowptr, FibreArgs{});
+    if (any_dense) finish_rows_kernel<true, false><<<tiles, FR_THREADS, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.look, rowptr, FibreArgs{});
+    else finish_rows_kernel<false, false><<<tiles, FR_THREADS, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.look, rowptr, FibreArgs{});
     ++c.launches;
     return cudaGetLastError();
 }
@@ -959,9 +1000,9 @@ cudaError_t launch_finish_fibres(const LaunchCtx& c, int n_i, int n_ij, bool any
                                  i64* rowptr_raw, i64* sfp, i64* Cpos0, int* Ccrd0, i64* Cpos1, int* Ccrd1, i64* Cpos2) {
     const int tiles = tiles_of(n_ij, FR_TILE);
     const FibreArgs f{Apos1, Acrd1, n_i, sfp, Ccrd1, Cpos2};
-    if (any_dense) finish_rows_kernel<true, true><<<tiles, FR_THREADS, 0, c.stream>>>(n_ij, c.tab, c.prm, c.ctl, c.host_ctl, c.look, rowptr_raw, f);
-    else finish_rows_kernel<false, true><<<tiles, FR_THREADS, 0, c.stream>>>(n_ij, c.tab, c.prm, c.ctl, c.host_ctl, c.look, rowptr_raw, f);
-    finish_slices_kernel<<<tiles_of(n_i, SL_TILE), FR_THREADS, 0, c.stream>>>(n_i, sfp, Acrd0, c.ctl, c.host_ctl, c.look + 2 * tiles, Ccrd0, Cpos1,
+    if (any_dense) finish_rows_kernel<true, true><<<tiles, FR_THREADS, 0, c.stream>>>(n_ij, c.tab, c.prm, c.ctl, c.host, c.look, rowptr_raw, f);
+    else finish_rows_kernel<false, true><<<tiles, FR_THREADS, 0, c.stream>>>(n_ij, c.tab, c.prm, c.ctl, c.host, c.look, rowptr_raw, f);
+    finish_slices_kernel<<<tiles_of(n_i, SL_TILE), FR_THREADS, 0, c.stream>>>(n_i, sfp, Acrd0, c.ctl, c.host, c.look + 2 * tiles, Ccrd0, Cpos1,
                                                                              Cpos0);
     c.launches += 2;
     return cudaGetLastError();

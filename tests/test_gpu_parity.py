@@ -314,6 +314,30 @@ def test_bounds_kernel_widths_with_and_without_b_row_summaries(ctx, oracle_mod, 
 
 
 @pytest.mark.parametrize("summaries", [True, False])
+@pytest.mark.parametrize("short", [1, 14, 30, 34])
+def test_bounds_of_long_rows_next_to_narrow_lane_groups(ctx, oracle_mod, short, summaries):
+    """Mean row lengths on both sides of each width of the bounds kernel, with rows at the lengths from
+    which a warp takes them (eight entries per lane of the group) or a block does (1025), first and
+    last ones among them."""
+    k = 2000
+    reps = 700 if short < 14 else 260
+    lengths = [257] + [short] * reps + [8, 9, 64, 65, 1024, 1025] + [short] * reps + [1500]
+    if summaries:
+        lengths = lengths * (4 * k // sum(lengths) + 1)
+    rng = np.random.default_rng(short)
+    rows = np.repeat(np.arange(len(lengths)), lengths)
+    cols = np.concatenate([np.sort(rng.choice(k, x, replace=False)) for x in lengths])
+    A = CSR.from_coo(len(lengths), k, rows, cols, rng.uniform(-1, 1, rows.size))
+    if not summaries:
+        k *= 40
+        A = CSR(A.nrows, k, A.pos, (A.crd * 40).astype(np.int32), A.val)
+    assert (A.nnz >= 4 * k) == summaries
+    B = random_csr(k, 3000, 0.002, 7, empty_row_frac=0.3)
+    for policy in ("auto", "dense"):
+        check_spgemm(ctx, oracle_mod, A, B, policy)
+
+
+@pytest.mark.parametrize("summaries", [True, False])
 def test_bounds_of_rows_with_thousands_of_entries(ctx, oracle_mod, summaries):
     """Rows of A with more than 1024 entries get a CTA each in the bounds pass (listed by the lane-group
     kernel, which skips them): a few such rows of different lengths among short and empty ones, at the
