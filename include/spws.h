@@ -258,9 +258,9 @@ spws_status_t spws_workspace_size_exact(spws_plan_t plan, const spws_tensor_t* A
  * C->pos[] must be allocated by the caller: CSR: pos[1] with dims[0]+1 entries;
  * CSF3: pos[0] (2), crd[0] (A->n[0]), pos[1] (A->n[0]+1), crd[1] (A->n[1]), pos[2] (A->n[1]+1),
  * i.e. the sizes of A's upper levels, which bound C's.  On return C->n[] holds the result sizes
- * and `sizes_out` (host, 3 entries, may be NULL) a copy.  Synchronises the stream twice: after
+ * and `sizes_out` (host, 3 entries, may be NULL) a copy.  Waits for the device twice: after
  * binning, to learn which workspaces have rows (only those are launched), and at the end, to read
- * the sizes back. */
+ * the sizes back; C->pos[] is complete when the call returns. */
 spws_status_t spws_symbolic(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B,
                             spws_tensor_t* C, void* scratch, size_t scratch_bytes,
                             int64_t* sizes_out);

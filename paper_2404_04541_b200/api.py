@@ -115,7 +115,8 @@ class Context:
 
     # ------------------------------------------------------------------ SpGEMM
     def spgemm_symbolic(self, plan: B_.Plan, A: DeviceCSR, B: DeviceCSR):
-        a, b = A.arrays(), B.arrays()
+        a = B_.fixed(A.arrays())
+        b = a if B is A else B_.fixed(B.arrays())
         pos = torch.empty(A.nrows + 1, dtype=torch.int64, device=self.device)
         c = B_.csr_arrays(A.nrows, B.ncols, pos, None, None)
         sc, nbytes = self._symbolic(plan, a, b, c)
@@ -156,7 +157,7 @@ class Context:
     # ------------------------------------------------------------------ outer-product SpGEMM
     def outer_symbolic(self, plan: B_.Plan, At: DeviceCSR, B: DeviceCSR):
         """Symbolic pass of C(i,j) = sum_k A(k,i) B(k,j); `At` holds A by its rows k (K x I)."""
-        a, b = At.arrays(), B.arrays()
+        a, b = B_.fixed(At.arrays()), B_.fixed(B.arrays())
         pos = torch.empty(At.ncols + 1, dtype=torch.int64, device=self.device)
         c = B_.csr_arrays(At.ncols, B.ncols, pos, None, None)
         sc, nbytes = self._symbolic(plan, a, b, c)
@@ -185,8 +186,8 @@ class Context:
         fmts = (B_.SPWS_COO, B_.SPWS_CSF3, B_.SPWS_CSR) + ((B_.SPWS_CSR,) if D is not None else ())
         plan = self.plan(expr, fmts, dt, policy, **options)
         try:
-            t, c = T.arrays(), C.arrays()
-            d = D.arrays() if D is not None else None
+            t, c = B_.fixed(T.arrays()), B_.fixed(C.arrays())
+            d = B_.fixed(D.arrays()) if D is not None else None
             if expr == EXPR_SPMTTKRP:
                 order, dims = 2, (T.dims[2], C.ncols, 0)
             elif expr == EXPR_SPTTM:
@@ -210,7 +211,7 @@ class Context:
     def ttm_symbolic(self, plan: B_.Plan, A: DeviceCSF3, B: DeviceCSR):
         """Symbolic pass of the 3-tensor form: allocates C's upper levels (bounded by A's) and returns
         (C arrays with sizes filled in, state for ttm_numeric)."""
-        a, b = A.arrays(), B.arrays()
+        a, b = B_.fixed(A.arrays()), B_.fixed(B.arrays())
         n_i, n_ij = a.n[0], a.n[1]
         i64, i32, dev = torch.int64, torch.int32, self.device
         pos0 = torch.empty(2, dtype=i64, device=dev)

@@ -6,6 +6,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from dataclasses import dataclass, field
 
 import numpy as np
@@ -51,6 +52,9 @@ class spws_tensor_t(ctypes.Structure):
                 ("pos", ctypes.c_void_p * 3), ("crd", ctypes.c_void_p * 3), ("val", ctypes.c_void_p)]
 
 
+_TENSOR = struct.Struct("=2i6q7Q")          # the fields of spws_tensor_t, packed in one go
+
+
 class spws_options_t(ctypes.Structure):
     _fields_ = [("validate", ctypes.c_int32), ("ism_warp_cap", ctypes.c_int32), ("ism_cta_cap", ctypes.c_int32),
                 ("dense_unit_outputs", ctypes.c_int32), ("dense_max_span", ctypes.c_int32),
@@ -66,6 +70,9 @@ class spws_stats_t(ctypes.Structure):
                 ("launches_symbolic", ctypes.c_int32), ("launches_numeric", ctypes.c_int32),
                 ("dense_warp_rows", ctypes.c_int64), ("dense_warp_products", ctypes.c_int64),
                 ("dense_warp_nnz", ctypes.c_int64), ("bitmap_bytes", ctypes.c_int64)]
+
+
+_STATS = struct.Struct("=4q10qq2i10q10q2i4q")     # the fields of spws_stats_t
 
 
 class SpwsError(RuntimeError):
@@ -142,12 +149,12 @@ def row_pointer_static(counts_ptr: int, n: int, pos_ptr: int, stream_ptr: int | 
 
 # ---------------------------------------------------------------------------- tensors
 def _ptr(t):
-    """Address of a torch tensor's (or numpy array's) storage, or None."""
+    """Address of a torch tensor's (or numpy array's) storage, or 0."""
     if t is None:
-        return None
+        return 0
     if isinstance(t, np.ndarray):
-        return t.ctypes.data if t.size else None
-    return t.data_ptr() or None             # (a tensor without elements has no storage)
+        return t.ctypes.data if t.size else 0
+    return t.data_ptr()                     # (0 for a tensor without storage)
 
 
 @dataclass
@@ -161,11 +168,22 @@ class TensorArrays:
     val: object
     n: list = field(default_factory=lambda: [0, 0, 0])
     interleaved: int = 0        # coordinate-form result: 1 = crd[0] takes the coordinates entry by entry
+    fixed: object = None        # the C struct, for arrays that will not change any more
 
     def c_struct(self) -> spws_tensor_t:
+        if self.fixed is not None:
+            return self.fixed
         d, n, pos, crd = self.dims, self.n, self.pos, self.crd
-        return spws_tensor_t(self.order, self.interleaved, (int(d[0]), int(d[1]), int(d[2]) if len(d) > 2 else 0), (int(n[0]), int(n[1]), int(n[2])),
-                             (_ptr(pos[0]), _ptr(pos[1]), _ptr(pos[2])), (_ptr(crd[0]), _ptr(crd[1]), _ptr(crd[2])), _ptr(self.val))
+        t = spws_tensor_t()
+        _TENSOR.pack_into(t, 0, self.order, self.interleaved, int(d[0]), int(d[1]), int(d[2]) if len(d) > 2 else 0, n[0], n[1], n[2],
+                          _ptr(pos[0]), _ptr(pos[1]), _ptr(pos[2]), _ptr(crd[0]), _ptr(crd[1]), _ptr(crd[2]), _ptr(self.val))
+        return t
+
+
+def fixed(arrays: TensorArrays) -> TensorArrays:
+    """`arrays` with its C struct made once and kept (operands that several calls of a pass take)."""
+    arrays.fixed = arrays.c_struct()
+    return arrays
 
 
 def csr_arrays(nrows, ncols, pos, crd, val) -> TensorArrays:
@@ -290,14 +308,11 @@ class Plan:
     def get_stats(self) -> dict:
         s = spws_stats_t()
         st = lib().spws_get_stats(self._p, ctypes.byref(s))
-        d = dict(rows=s.rows, products=s.products, nnz=s.nnz, max_row_products=s.max_row_products,
-                 rows_per_class=list(s.rows_per_class), dense_units=s.dense_units, device_status=s.device_status,
-                 products_per_class=list(s.products_per_class), nnz_per_class=list(s.nnz_per_class),
-                 launches_symbolic=s.launches_symbolic, launches_numeric=s.launches_numeric,
-                 dense_warp_rows=s.dense_warp_rows, dense_warp_products=s.dense_warp_products,
-                 dense_warp_nnz=s.dense_warp_nnz, bitmap_bytes=s.bitmap_bytes)
+        v = _STATS.unpack_from(s)
         _check(st, "spws_get_stats")
-        return d
+        return dict(rows=v[0], products=v[1], nnz=v[2], max_row_products=v[3], rows_per_class=list(v[4:14]), dense_units=v[14],
+                    device_status=v[15], products_per_class=list(v[17:27]), nnz_per_class=list(v[27:37]), launches_symbolic=v[37],
+                    launches_numeric=v[38], dense_warp_rows=v[39], dense_warp_products=v[40], dense_warp_nnz=v[41], bitmap_bytes=v[42])
 
     def set_profiling(self, enabled: bool):
         _check(lib().spws_set_profiling(self._p, int(bool(enabled))), "spws_set_profiling")

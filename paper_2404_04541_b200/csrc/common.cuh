@@ -93,14 +93,6 @@ struct DevCtl {
     i64 dense_warp_products, dense_warp_nnz;   // share of the dense rows the warp numeric kernel takes
 };
 
-// What a plan keeps in pinned host memory: the control block as last read back, and one slot per
-// block of the counting kernels, which write their partial sums there and the host adds up.
-constexpr int COUNT_BLOCKS = 256;
-struct HostBlock {
-    DevCtl ctl;
-    u64 partial[2 * COUNT_BLOCKS];
-};
-
 struct ClassParams {
     int policy;             // spws_policy_t
     int reg_cap;            // CLS_ISM_REG: products <= reg_cap
@@ -189,16 +181,30 @@ __host__ __device__ inline int dense_units_of_row(i64 ub, i64 unit_products) {
     return (int)(n < 1 ? 1 : n);
 }
 
+// What a plan keeps in pinned host memory: the control block as last read back, and one slot per
+// block of the counting kernels, which write their partial sums there and the host adds up.
+constexpr int COUNT_BLOCKS = 256;
+struct HostBlock {
+    DevCtl ctl;
+    int seq;                // number of the publication `ctl` holds, written last
+    int pad[31];
+    u64 partial[2 * COUNT_BLOCKS];
+};
+
 // The first error wins; it is also written to the plan's pinned block once that is known.
 __device__ __forceinline__ void raise_status(DevCtl* ctl, int s) {
     if (atomicCAS(&ctl->status, 0, s) == 0 && ctl->host_status) *(volatile int*)ctl->host_status = s;
 }
 
-// Copies the control block to pinned host memory (a whole block of threads, after the counters are final):
-// posted writes, complete when the kernel is.
-__device__ __forceinline__ void publish_ctl(DevCtl* ctl, DevCtl* host) {
+// Copies the control block to pinned host memory (a whole block of threads, after the counters are final), and
+// then the number of the publication, which the host polls: it goes on about 5 us before a stream
+// synchronisation would let it.
+__device__ __forceinline__ void publish_ctl(DevCtl* ctl, HostBlock* host, int seq) {
     for (int w = threadIdx.x; w < (int)(sizeof(DevCtl) / 4); w += blockDim.x)
-        reinterpret_cast<volatile int*>(host)[w] = reinterpret_cast<volatile const int*>(ctl)[w];
+        reinterpret_cast<volatile int*>(&host->ctl)[w] = reinterpret_cast<volatile const int*>(ctl)[w];
+    __threadfence_system();
+    __syncthreads();
+    if (threadIdx.x == 0) *(volatile int*)&host->seq = seq;
 }
 
 // True in every thread of the last of `blocks` blocks to come here; all earlier blocks' writes are visible to it.
@@ -356,7 +362,8 @@ struct LaunchCtx {
     char* rest;              // scratch after the fixed tables: bitmap arena, then the ISM-global arena
     size_t rest_bytes;
     int global_cap;          // accumulation-array capacity of CLS_ISM_GLOBAL
-    DevCtl* host_ctl;        // the plan's pinned copy of the control block
+    HostBlock* host;         // the plan's pinned block: receives the control block ...
+    int seq;                 // ... as publication `seq` (binning) and `seq` + 1 (row pointer)
     u64* look;               // one word per tile of the kernels that hand running sums on ...
     int n_look;              // ... cleared by the binning kernel
     i64 max_ub_smem;         // largest product count of a CLS_ISM_SMEM row when known (0: unknown)

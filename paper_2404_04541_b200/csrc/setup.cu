@@ -534,7 +534,7 @@ cudaError_t launch_bw_build(const LaunchCtx& c, const Csr& B) {
 // ---------------------------------------------------------------------------------------
 // It also counts the units per bucket of rows, clears the words of the kernels that hand running sums
 // from tile to tile, and its last block publishes the class sizes to the host.
-__global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, HostBlock* host, u64* look, int n_look) {
+__global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, HostBlock* host, int seq, u64* look, int n_look) {
     __shared__ int s_units[UNIT_BUCKETS];
     if (threadIdx.x < UNIT_BUCKETS) s_units[threadIdx.x] = 0;
     for (int w = blockIdx.x * 256 + threadIdx.x; w < n_look; w += gridDim.x * 256) look[w] = 0;
@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, 
     if (last_block(&ctl->bin_done, gridDim.x)) {
         if (threadIdx.x == 0) ctl->host_status = &host->ctl.status;
         __syncthreads();
-        publish_ctl(ctl, host);
+        publish_ctl(ctl, host, seq);
     }
 }
 
@@ -618,7 +618,7 @@ cudaError_t launch_bin_rows(const LaunchCtx& c, int m) {
     i64 want = ((i64)m + 1023) / 1024;
     i64 cap = (i64)c.sm_count * 8;
     if (want < 1) want = 1;
-    bin_rows_kernel<<<(int)(want < cap ? want : cap), 256, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.look, c.n_look);
+    bin_rows_kernel<<<(int)(want < cap ? want : cap), 256, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.seq, c.look, c.n_look);
     ++c.launches;
     return cudaGetLastError();
 }
@@ -654,7 +654,7 @@ struct FibreArgs {
 };
 
 template <bool DENSE, bool TTM>
-__global__ void __launch_bounds__(FR_THREADS, DENSE ? 3 : 5) finish_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, HostBlock* host, u64* look,
+__global__ void __launch_bounds__(FR_THREADS, DENSE ? 3 : 5) finish_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, HostBlock* host, int seq, u64* look,
                                                                  i64* __restrict__ rowptr, FibreArgs f) {
     __shared__ int s_tile, s_slice0;
     __shared__ i64 s_sum[FR_WARPS], s_before[2];
@@ -920,13 +920,13 @@ __global__ void __launch_bounds__(FR_THREADS, DENSE ? 3 : 5) finish_rows_kernel(
             ctl->n_units = n;
         }
         __syncthreads();
-        if (!TTM) publish_ctl(ctl, host);           // (the slice level comes after the fibres)
+        if (!TTM) publish_ctl(ctl, host, seq);           // (the slice level comes after the fibres)
     }
 }
 
 // A slice i survives when one of its fibres does: C's slice level from sfp.
 __global__ void __launch_bounds__(FR_THREADS) finish_slices_kernel(int n_i, const i64* __restrict__ sfp, const int* __restrict__ Acrd0, DevCtl* ctl,
-                                                                   HostBlock* host, u64* look, int* __restrict__ Ccrd0, i64* __restrict__ Cpos1,
+                                                                   HostBlock* host, int seq, u64* look, int* __restrict__ Ccrd0, i64* __restrict__ Cpos1,
                                                                    i64* __restrict__ Cpos0) {
     __shared__ int s_tile, s_part[FR_WARPS];
     __shared__ i64 s_before;
@@ -981,7 +981,7 @@ __global__ void __launch_bounds__(FR_THREADS) finish_slices_kernel(int n_i, cons
         Cpos0[1] = k;
         ctl->kept[0] = k;
     }
-    if (last_block(&ctl->slices_done, tiles)) publish_ctl(ctl, host);
+    if (last_block(&ctl->slices_done, tiles)) publish_ctl(ctl, host, seq);
 }
 
 static int tiles_of(i64 n, int tile) { return n > 0 ? (int)((n + tile - 1) / tile) : 1; }
@@ -990,8 +990,8 @@ size_t look_words(i64 rows, i64 slices) { return (size_t)2 * tiles_of(rows, FR_T
 
 cudaError_t launch_finish_rows(const LaunchCtx& c, int m, bool any_dense, i64* rowptr) {
     const int tiles = tiles_of(m, FR_TILE);
-    if (any_dense) finish_rows_kernel<true, false><<<tiles, FR_THREADS, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.look, rowptr, FibreArgs{});
-    else finish_rows_kernel<false, false><<<tiles, FR_THREADS, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.look, rowptr, FibreArgs{});
+    if (any_dense) finish_rows_kernel<true, false><<<tiles, FR_THREADS, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.seq + 1, c.look, rowptr, FibreArgs{});
+    else finish_rows_kernel<false, false><<<tiles, FR_THREADS, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.seq + 1, c.look, rowptr, FibreArgs{});
     ++c.launches;
     return cudaGetLastError();
 }
@@ -1000,9 +1000,9 @@ cudaError_t launch_finish_fibres(const LaunchCtx& c, int n_i, int n_ij, bool any
                                  i64* rowptr_raw, i64* sfp, i64* Cpos0, int* Ccrd0, i64* Cpos1, int* Ccrd1, i64* Cpos2) {
     const int tiles = tiles_of(n_ij, FR_TILE);
     const FibreArgs f{Apos1, Acrd1, n_i, sfp, Ccrd1, Cpos2};
-    if (any_dense) finish_rows_kernel<true, true><<<tiles, FR_THREADS, 0, c.stream>>>(n_ij, c.tab, c.prm, c.ctl, c.host, c.look, rowptr_raw, f);
-    else finish_rows_kernel<false, true><<<tiles, FR_THREADS, 0, c.stream>>>(n_ij, c.tab, c.prm, c.ctl, c.host, c.look, rowptr_raw, f);
-    finish_slices_kernel<<<tiles_of(n_i, SL_TILE), FR_THREADS, 0, c.stream>>>(n_i, sfp, Acrd0, c.ctl, c.host, c.look + 2 * tiles, Ccrd0, Cpos1,
+    if (any_dense) finish_rows_kernel<true, true><<<tiles, FR_THREADS, 0, c.stream>>>(n_ij, c.tab, c.prm, c.ctl, c.host, c.seq + 1, c.look, rowptr_raw, f);
+    else finish_rows_kernel<false, true><<<tiles, FR_THREADS, 0, c.stream>>>(n_ij, c.tab, c.prm, c.ctl, c.host, c.seq + 1, c.look, rowptr_raw, f);
+    finish_slices_kernel<<<tiles_of(n_i, SL_TILE), FR_THREADS, 0, c.stream>>>(n_i, sfp, Acrd0, c.ctl, c.host, c.seq + 1, c.look + 2 * tiles, Ccrd0, Cpos1,
                                                                              Cpos0);
     c.launches += 2;
     return cudaGetLastError();

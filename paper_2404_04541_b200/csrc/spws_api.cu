@@ -1,7 +1,9 @@
 // C ABI of the spws library: handles, plans, expression check, scratch layout and the launch
 // sequences of the symbolic and numeric passes.  Host code only.
 #include <algorithm>
+#include <atomic>
 #include <cctype>
+#include <chrono>
 #include <cstdio>
 #include <cstring>
 #include <memory>
@@ -66,6 +68,7 @@ struct spws_plan_s {
     spws_options_t opt{};
     std::shared_ptr<PinnedPool> pool;
     HostBlock* host = nullptr;  // pinned
+    int seq = 0;                // publications asked for so far
     bool in_flight = false;     // kernels that may still write to the pinned block are enqueued
     DevCtl* host_ctl = nullptr; // &host->ctl
     bool symbolic_ok = false;
@@ -408,7 +411,7 @@ LaunchCtx make_ctx(const spws_plan_s* p, char* scratch, size_t scratch_bytes, co
         c.bw_long_cap = L.bw_long_cap;
     }
     if (L.has_brow) c.brow = reinterpret_cast<int4*>(scratch + L.brow);
-    c.host_ctl = p->host_ctl;
+    c.host = p->host;
     c.look = reinterpret_cast<u64*>(scratch + L.look);
     c.n_look = L.n_look;
     return c;
@@ -442,6 +445,22 @@ inline void mark_start(spws_plan_s* p, int pass) {
     p->ev_pass[pass] = true;
 }
 
+// Waits for publication `seq` of the control block: polled for a fifth of a millisecond, then by synchronising
+// the stream (which also reports a failed kernel).
+spws_status_t wait_published(spws_plan_s* p, int seq) {
+    const volatile int* at = &p->host->seq;
+    const auto end = std::chrono::steady_clock::now() + std::chrono::microseconds(200);
+    do {
+        for (int k = 0; k < 64; ++k)
+            if (*at == seq) {
+                std::atomic_thread_fence(std::memory_order_acquire);
+                return SPWS_OK;
+            }
+    } while (std::chrono::steady_clock::now() < end);
+    CUDA_TRY(cudaStreamSynchronize(p->h->stream));
+    return *at == seq ? SPWS_OK : SPWS_CUDA_ERROR;
+}
+
 // What both passes use, known once the rows are binned: the fixed tables, the bitmaps of exactly the dense rows,
 // and the slots of the global-memory ISM, sized for its largest row.
 size_t rows_need(const spws_plan_s* plan, const Layout& L, const DevCtl& hc, int64_t ncols) {
@@ -469,8 +488,9 @@ size_t rows_guess(const spws_plan_s* plan, const Layout& L, int64_t m, int64_t n
 // the plan holds the statistics and what the numeric pass needs.
 spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L, LaunchCtx& c, size_t scratch_bytes, size_t* needed, bool clear_ctl, const spws_tensor_t* ttmA,
                             spws_tensor_t* ttmC, i64* rowptr, char* sc) {
-    cudaStream_t stream = c.stream;
     plan->in_flight = true;
+    c.seq = plan->seq + 1;
+    plan->seq += 2;
     // a1: upper bounds + classes; a2: binning
     CUDA_TRY(launch_row_bounds(c, S.A, S.B, S.nnzA, clear_ctl));
     mark(plan, SPWS_T_SYM_BOUNDS);
@@ -479,7 +499,8 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     // the class sizes come back now (written to pinned memory by the binning kernel), so that only the
     // workspaces that have rows are launched, with grids sized for them (a launch for an empty class
     // costs as much as a small class's work)
-    CUDA_TRY(cudaStreamSynchronize(stream));
+    spws_status_t st = wait_published(plan, c.seq);
+    if (st != SPWS_OK) return st;
     plan->in_flight = false;
     const DevCtl& hc = *plan->host_ctl;
     if (needed && (hc.status == 0 || hc.status == DEV_SCRATCH_TOO_SMALL)) {
@@ -539,7 +560,7 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     else
         CUDA_TRY(launch_finish_rows(c, (int)S.m, any_dense, rowptr));
     mark(plan, SPWS_T_SYM_SCAN);
-    CUDA_TRY(cudaStreamSynchronize(stream));
+    if ((st = wait_published(plan, c.seq + 1)) != SPWS_OK) return st;
     plan->in_flight = false;
     plan->counters_clear = true;
     plan->rows_path = true;
@@ -1422,6 +1443,7 @@ spws_status_t spws_workspace_size_exact(spws_plan_t plan, const spws_tensor_t* A
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, L);
     c.prm.bm_arena_words = ~0ull >> 3;          // reserve without a limit: only the total is wanted
     plan->in_flight = true;
+    c.seq = ++plan->seq;
     CUDA_TRY(launch_row_bounds(c, S.A, S.B, S.nnzA, true));
     CUDA_TRY(launch_bin_rows(c, (int)S.m));
     if (row_products && S.m > 0)
