@@ -268,8 +268,9 @@ spws_status_t spws_symbolic(spws_plan_t plan, const spws_tensor_t* A, const spws
 /* The symbolic pass for a caller that does not know the scratch size: as spws_symbolic (D = NULL) or
  * spws_symbolic3, but `scratch` may be NULL and the call returns SPWS_SCRATCH_TOO_SMALL, before any
  * workspace has run, when `scratch_bytes` is less than what the passes use for these operands.
- * *needed receives that size (as spws_workspace_size_exact would report it), or a size to try next
- * while it cannot be known.  A caller that keeps its scratch buffer from call to call runs the sizing
+ * *needed receives that size (what spws_workspace_size_exact would report, and room to keep the sorted
+ * order of rows of 257 .. 1024 products for the numeric pass, which sorts again without it), or a size to
+ * try next while it cannot be known.  A caller that keeps its scratch buffer from call to call runs the sizing
  * steps once instead of twice. */
 spws_status_t spws_symbolic_sized(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B,
                                   const spws_tensor_t* D, spws_tensor_t* C, void* scratch, size_t scratch_bytes,

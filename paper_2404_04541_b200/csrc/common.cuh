@@ -74,6 +74,7 @@ struct DevCtl {
     i64 max_ub_smem;        // largest product count among CLS_ISM_SMEM rows (sizes that kernel's launch)
     i64 kept[2];            // TTM: surviving slices (level 0) and fibres (level 1)
     u64 bm_words_used;      // words handed out of the bitmap arena
+    u64 order_used;         // bytes handed out of the arena of sorted words
     int status;
     int n_units;            // numeric dense CTA units (row, share of its entries)
     int units_of[7];        // units per bucket of rows (counted by the binning, without the rows that outgrow a warp) ...
@@ -144,7 +145,7 @@ struct RowTables {
     int* jmax;
     unsigned char* cls;
     int* perm;
-    i64* bm_off;        // word offset of the row's bitmap in the arena (dense classes)
+    i64* bm_off;        // word offset of the row's bitmap in the arena (dense classes); byte offset of its sorted words (CLS_ISM_SMEM)
     unsigned* bm_arena;
     int* warp_rows;     // numeric: rows handled by the warp-per-row dense kernel: list 0 from the front, list 1 from the back
     int* row_unit0;     // numeric: first CTA unit of a row
@@ -361,6 +362,8 @@ struct LaunchCtx {
     int dense_smem_words;    // bitmap words the CTA dense kernels reserve (from ncols)
     char* rest;              // scratch after the fixed tables: bitmap arena, then the ISM-global arena
     size_t rest_bytes;
+    char* order;             // arena of sorted words (null: every pass sorts)
+    size_t order_bytes;
     int global_cap;          // accumulation-array capacity of CLS_ISM_GLOBAL
     HostBlock* host;         // the plan's pinned block: receives the control block ...
     int seq;                 // ... as publication `seq` (binning) and `seq` + 1 (row pointer)
@@ -394,6 +397,8 @@ cudaError_t launch_scan_counts(const LaunchCtx& c, const int* cnt, int n, i64* o
 // class kernels: n_host < 0 means "size the grid for any count"
 // rows[cls] = rows of the three register classes and of the copied class, in ONE launch
 cudaError_t launch_ism_reg(const LaunchCtx& c, bool numeric, const i64* rows, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval);
+// scratch that keeps the sorted words of the rows of the warp-per-row ISM from the counting pass to the numeric one
+size_t order_bytes_of(i64 rows, i64 products, i64 max_products, i64 ncols);
 cudaError_t launch_ism_smem(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B,
                             const i64* rowptr, int* Ccrd, void* Cval);
 // max_span_words: widest dense row of the pass

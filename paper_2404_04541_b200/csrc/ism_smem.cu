@@ -156,6 +156,11 @@ __global__ void __launch_bounds__(THREADS) ism_smem_kernel(const int* __restrict
 //   Sort   : E = 2 .. 32 words per lane, the smallest network that holds the row.
 //   Merge  : the sorted words go back to shared memory, the places of the run heads are packed, and
 //            one lane per run sums it in slot order.
+//   Of rows of more than 256 products the counting pass leaves the sorted words in scratch when there is room
+// (coalesced: word x of lane l at x * lanes + l, lanes past the last word left out), and the numeric pass then only
+// fetches the values: 8e4 rows of 674 products, f32: count 507 -> 578 us, numeric 871 -> 400 us; 2e5 rows
+// of 470, f64: 154 -> 210 and 494 -> 225 us.  Shorter rows gain nothing (fibres of about 110 products: numeric 104 us with
+// and without, count 82 -> 100 us), their sort is a small part of the work.
 // Stencil 41 x 37 x 53 (f32, 674 products a row): count 1714 -> 508 us, numeric 1905 -> 863 us against a CTA per
 // row; 59-product rows of the outer form (2e5 of them): 259 -> 125 us (hash set) and 439 -> 146 us.
 // ---------------------------------------------------------------------------------------
@@ -214,18 +219,33 @@ __device__ __forceinline__ void warp_sort(P (&w)[E]) {
 // one word of padding per 32 keeps both the strided and the per-lane consecutive accesses conflict-free
 __device__ __forceinline__ int padded(int i) { return i + (i >> 5); }
 
+// words each lane holds for a row of `total` words, and the lanes whose words are kept in scratch
+__device__ __forceinline__ int words_per_lane(int total) { return total <= 64 ? 2 : total <= 128 ? 4 : total <= 256 ? 8 : total <= 512 ? 16 : 32; }
+__device__ __forceinline__ int order_lanes(int total, int e) { return ((total + e - 1) / e + 7) & ~7; }
+
 // Sorts the row's packed words and counts its distinct columns; numeric: leaves the sorted words in `packed`
-// and the places of the run heads in `heads`.
+// and the places of the run heads in `heads`.  `order` (may be null): numeric: the words as sorted before;
+// else receives them.
 template <typename PK, typename P, int E, bool NUMERIC>
-__device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int total) {
+__device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int total, P* order) {
     const int lane = threadIdx.x & 31;
     P w[E];
+    const int lanes = order_lanes(total, E);
+    if (NUMERIC && order) {
 #pragma unroll
-    for (int x = 0; x < E; ++x) {
-        const int i = x * 32 + lane;
-        w[x] = i < total ? packed[padded(i)] : PK::sentinel();
+        for (int x = 0; x < E; ++x) w[x] = lane < lanes ? order[x * lanes + lane] : PK::sentinel();
+    } else {
+#pragma unroll
+        for (int x = 0; x < E; ++x) {
+            const int i = x * 32 + lane;
+            w[x] = i < total ? packed[padded(i)] : PK::sentinel();
+        }
+        warp_sort<P, E>(w);
+        if (!NUMERIC && order && lane < lanes) {
+#pragma unroll
+            for (int x = 0; x < E; ++x) order[x * lanes + lane] = w[x];
+        }
     }
-    warp_sort<P, E>(w);
     const P before = __shfl_up_sync(0xffffffffu, w[E - 1], 1);
     unsigned head = 0;
 #pragma unroll
@@ -251,7 +271,8 @@ __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int to
 
 template <typename T, typename P, int CAP, bool NUMERIC>
 __global__ void __launch_bounds__(IW_WARPS * 32) ism_warp_kernel(const int* __restrict__ perm, DevCtl* __restrict__ ctl, int cls, int counter_slot,
-                                                                 Csr A, Csr B, const i64* __restrict__ ub, int* __restrict__ cnt,
+                                                                 Csr A, Csr B, const i64* __restrict__ ub, i64* __restrict__ order_off, char* order_arena,
+                                                                 size_t order_bytes, int* __restrict__ cnt,
                                                                  const i64* __restrict__ rowptr, int* __restrict__ Ccrd, T* __restrict__ Cval) {
     typedef Pack<P, CAP> PK;
     constexpr int SLOTS = CAP + CAP / 32;
@@ -273,6 +294,21 @@ __global__ void __launch_bounds__(IW_WARPS * 32) ism_warp_kernel(const int* __re
         const int row = __ldg(perm + off + r);
         const i64 products = __ldg(ub + row);
         if (products > CAP) continue;                            // the CTA kernel's rows
+        P* order = nullptr;
+        if (CAP > 256 && order_arena) {
+            i64 at = -1;
+            if (NUMERIC) {
+                at = order_off[row];
+            } else if (lane == 0) {
+                const int e = words_per_lane((int)products);
+                const u64 bytes = (u64)e * order_lanes((int)products, e) * sizeof(P);
+                at = (i64)atomicAdd(&ctl->order_used, bytes);
+                if ((u64)at + bytes > order_bytes) at = -1;
+            }
+            if (!NUMERIC) at = __shfl_sync(0xffffffffu, at, 0);
+            if (at >= 0) order = reinterpret_cast<P*>(order_arena + at);
+        }
+        const bool sorted = CAP > 256 && NUMERIC && order;
         const i64 ps = __ldg(A.pos + row), pe = __ldg(A.pos + row + 1);
         const int gs = pick_group_size(products, pe - ps, 1);
         const int g = lane / gs, gl = lane % gs, ng = 32 / gs;
@@ -305,18 +341,18 @@ __global__ void __launch_bounds__(IW_WARPS * 32) ism_warp_kernel(const int* __re
                 if (NUMERIC) { a0 = __shfl_sync(0xffffffffu, a, e0); a1 = __shfl_sync(0xffffffffu, a, e1); }
                 int c0 = 0, c1 = 0;
                 T v0 = 0, v1 = 0;
-                if (gl < l0) { c0 = __ldg(B.crd + q0 + gl); if (NUMERIC) v0 = __ldg(Bval + q0 + gl); }
-                if (gl < l1) { c1 = __ldg(B.crd + q1 + gl); if (NUMERIC) v1 = __ldg(Bval + q1 + gl); }
+                if (gl < l0) { if (!sorted) c0 = __ldg(B.crd + q0 + gl); if (NUMERIC) v0 = __ldg(Bval + q0 + gl); }
+                if (gl < l1) { if (!sorted) c1 = __ldg(B.crd + q1 + gl); if (NUMERIC) v1 = __ldg(Bval + q1 + gl); }
                 auto put = [&](int slot, int col, T v) {
                     if (slot < CAP) {                            // always so for a correctly classed row
-                        packed[padded(slot)] = PK::make(col, slot);
+                        if (!sorted) packed[padded(slot)] = PK::make(col, slot);
                         if (NUMERIC) vals[slot] = v;
                     }
                 };
                 if (gl < l0) put(b0 + gl, c0, mul_rn(a0, v0));
-                for (int t = gl + gs; t < l0; t += gs) put(b0 + t, __ldg(B.crd + q0 + t), NUMERIC ? mul_rn(a0, __ldg(Bval + q0 + t)) : (T)0);
+                for (int t = gl + gs; t < l0; t += gs) put(b0 + t, sorted ? 0 : __ldg(B.crd + q0 + t), NUMERIC ? mul_rn(a0, __ldg(Bval + q0 + t)) : (T)0);
                 if (gl < l1) put(b1 + gl, c1, mul_rn(a1, v1));
-                for (int t = gl + gs; t < l1; t += gs) put(b1 + t, __ldg(B.crd + q1 + t), NUMERIC ? mul_rn(a1, __ldg(Bval + q1 + t)) : (T)0);
+                for (int t = gl + gs; t < l1; t += gs) put(b1 + t, sorted ? 0 : __ldg(B.crd + q1 + t), NUMERIC ? mul_rn(a1, __ldg(Bval + q1 + t)) : (T)0);
             }
             total += __shfl_sync(0xffffffffu, incl, 31);
         }
@@ -325,11 +361,15 @@ __global__ void __launch_bounds__(IW_WARPS * 32) ism_warp_kernel(const int* __re
 
         // ---- Sort
         int distinct;
-        if (total <= 64) distinct = sort_row<PK, P, 2, NUMERIC>(packed, heads, total);
-        else if (total <= 128) distinct = sort_row<PK, P, 4, NUMERIC>(packed, heads, total);
-        else if (CAP <= 256 || total <= 256) distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total);
-        else if (total <= 512) distinct = sort_row<PK, P, (CAP > 256 ? 16 : 8), NUMERIC>(packed, heads, total);
-        else distinct = sort_row<PK, P, (CAP > 256 ? 32 : 8), NUMERIC>(packed, heads, total);
+        const int e = words_per_lane(total);
+        if (total != (int)products) order = nullptr;             // (a malformed B row)
+        P* const keep = CAP > 256 ? order : nullptr;
+        if (CAP > 256 && !NUMERIC && order_arena && lane == 0) order_off[row] = order ? (i64)(reinterpret_cast<char*>(order) - order_arena) : -1;
+        if (e == 2) distinct = sort_row<PK, P, 2, NUMERIC>(packed, heads, total, keep);
+        else if (e == 4) distinct = sort_row<PK, P, 4, NUMERIC>(packed, heads, total, keep);
+        else if (CAP <= 256 || e == 8) distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total, keep);
+        else if (e == 16) distinct = sort_row<PK, P, (CAP > 256 ? 16 : 8), NUMERIC>(packed, heads, total, keep);
+        else distinct = sort_row<PK, P, (CAP > 256 ? 32 : 8), NUMERIC>(packed, heads, total, keep);
 
         // ---- Merge
         if (!NUMERIC) {
@@ -381,8 +421,8 @@ static cudaError_t launch_warp_k(const LaunchCtx& c, int cls, int n_host, const 
     i64 grid = (i64)c.sm_count * (per_sm > 0 ? per_sm : 1);
     const i64 want = n_host >= 0 ? ((i64)n_host + IW_WARPS - 1) / IW_WARPS : grid;
     if (want < grid) grid = want > 0 ? want : 1;
-    k<<<(int)grid, IW_WARPS * 32, smem, c.stream>>>(c.tab.perm, c.ctl, cls, cls + (NUMERIC ? NUM_SLOT : 0), A, B, c.tab.ub, c.tab.cnt, rowptr, Ccrd,
-                                                    (T*)Cval);
+    k<<<(int)grid, IW_WARPS * 32, smem, c.stream>>>(c.tab.perm, c.ctl, cls, cls + (NUMERIC ? NUM_SLOT : 0), A, B, c.tab.ub, c.tab.bm_off, c.order,
+                                                    c.order_bytes, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
     ++c.launches;
     return cudaGetLastError();
 }
@@ -390,6 +430,13 @@ static cudaError_t launch_warp_k(const LaunchCtx& c, int cls, int n_host, const 
 // Packed words are 32 bits wide when (column, slot) fits below the all-ones sentinel.
 template <int CAP>
 static bool narrow(const Csr& B) { return (i64)B.ncols < (1ll << (32 - Log2<CAP>::value)); }
+
+size_t order_bytes_of(i64 rows, i64 products, i64 max_products, i64 ncols) {
+    if (rows == 0 || max_products <= 256) return 0;
+    // (up to eight lanes hold fewer words than they have room for: half a row, 16 words at least; wide words from
+    // 2^22 columns on)
+    return (size_t)(products + products / 2 + 16 * rows) * (ncols < (1ll << (32 - Log2<ISM_WARP_MAX>::value)) ? 4 : 8);
+}
 
 template <typename T, int CAP>
 static cudaError_t launch_warp(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd,

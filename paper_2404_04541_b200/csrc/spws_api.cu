@@ -77,6 +77,7 @@ struct spws_plan_s {
     int64_t m = 0;
     void* scratch = nullptr;
     int max_span_words = 0;     // widest dense bitmap of the last symbolic pass
+    size_t order_off = 0, order_bytes = 0;      // where it left the sorted words of mid-size rows in the scratch (0 bytes: nowhere)
     int n_warp[N_WARP_LISTS] = {};          // rows on the warp numeric kernel's lists ...
     int max_warp_cnt[N_WARP_LISTS] = {};    // ... and their largest output counts
     int64_t max_ub_smem = 0;    // most products of a shared-memory ISM row
@@ -482,6 +483,14 @@ size_t rows_guess(const spws_plan_s* plan, const Layout& L, int64_t m, int64_t n
     return L.fixed_end + std::min(rest_reserve(plan, m, ncols), std::max(L.fixed_end, (size_t)16 << 20));
 }
 
+// Hands the arena of sorted words to the kernels and takes it from what follows the bitmaps.
+void use_order(const spws_plan_s* plan, LaunchCtx& c, char* sc, size_t scratch_bytes) {
+    if (plan->order_bytes == 0 || plan->order_off + plan->order_bytes > scratch_bytes) return;
+    c.order = sc + plan->order_off;
+    c.order_bytes = plan->order_bytes;
+    c.rest_bytes = (size_t)(c.order - c.rest);
+}
+
 // ---- the row-wise passes: every output row (fibre) through the workspace of its class ------------
 // `ttmA` / `ttmC`: the 3-tensor operand and result, whose upper levels are rebuilt (null for the matrix
 // forms).  `c` is make_ctx of the layout; clear_ctl: the control block is not in use yet.  On success
@@ -503,10 +512,16 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     if (st != SPWS_OK) return st;
     plan->in_flight = false;
     const DevCtl& hc = *plan->host_ctl;
+    // the sorted words of the mid-size rows are kept for the numeric pass at the end of the scratch when it has room
+    const size_t need = rows_need(plan, L, hc, S.ncols);
+    const size_t order = align256(order_bytes_of(hc.class_count[CLS_ISM_SMEM], hc.class_products[CLS_ISM_SMEM], hc.max_ub_smem, S.ncols));
     if (needed && (hc.status == 0 || hc.status == DEV_SCRATCH_TOO_SMALL)) {
-        *needed = rows_need(plan, L, hc, S.ncols);
+        *needed = need + order;
         if (scratch_bytes < *needed) return SPWS_SCRATCH_TOO_SMALL;
     }
+    plan->order_bytes = order > 0 && scratch_bytes >= need + order ? order : 0;
+    plan->order_off = (scratch_bytes & ~(size_t)255) - plan->order_bytes;
+    use_order(plan, c, sc, scratch_bytes);
     if (hc.status != 0) {
         plan->stats = spws_stats_t{};
         plan->stats.device_status = hc.status;
@@ -591,8 +606,9 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     return SPWS_OK;
 }
 
-spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, const i64* rowptr, int* crd, void* val) {
+spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, char* sc, size_t scratch_bytes, const i64* rowptr, int* crd, void* val) {
     plan->in_flight = true;
+    use_order(plan, c, sc, scratch_bytes);
     if (!plan->counters_clear) CUDA_TRY(cudaMemsetAsync(c.ctl->work_counter, 0, sizeof(c.ctl->work_counter), c.stream));
     plan->counters_clear = false;
     c.max_ub_smem = plan->max_ub_smem;
@@ -842,7 +858,7 @@ spws_status_t rw_outer_numeric(spws_plan_s* plan, const Shapes& S, spws_tensor_t
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, w.L);
     mark_start(plan, 1);
     CUDA_TRY(launch_rw_values(c, S.A.val, rw_bufs(sc + w.L.extra, w.R).src, S.nnzA, sc + w.L.extra + w.R.val));
-    return rows_numeric(plan, w.S, c, LL(C->pos[1]), C->crd[1], C->val);
+    return rows_numeric(plan, w.S, c, sc, scratch_bytes, LL(C->pos[1]), C->crd[1], C->val);
 }
 
 spws_status_t outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_t* C, void* scratch, size_t scratch_bytes, int64_t* sizes_out,
@@ -1130,7 +1146,7 @@ spws_status_t rw_higher_numeric(spws_plan_s* plan, const HShapes& H, spws_tensor
     CUDA_TRY(launch_rw_values(c, H.B.val, b.src, H.B.nnz, x + w.R.val));
     if (H.form == 2)
         CUDA_TRY(launch_rw_fibre_rows(c, true, H.B, H.C, H.D, nullptr, reinterpret_cast<i64*>(x + w.R.fpos), nullptr, x + w.R.fval, nullptr));
-    const spws_status_t st = rows_numeric(plan, w.S, c, rowptr, cols, Out->val);
+    const spws_status_t st = rows_numeric(plan, w.S, c, sc, scratch_bytes, rowptr, cols, Out->val);
     if (st != SPWS_OK) return st;
     CUDA_TRY(launch_rw_coords(c, H.order, rowptr, b.row_key, w.m, plan->stats.nnz, (u64)(H.order == 3 ? H.odims[1] : 1), cols, Out->crd[0],
                               Out->crd[1], Out->crd[2], Out->interleaved != 0));
@@ -1539,7 +1555,7 @@ spws_status_t spws_numeric(spws_plan_t plan, const spws_tensor_t* A, const spws_
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, L);
     const i64* rowptr = (plan->kind == 0) ? LL(C->pos[1]) : reinterpret_cast<const i64*>(sc + L.rowptr_raw);
     mark_start(plan, 1);
-    return rows_numeric(plan, S, c, rowptr, C->crd[last], C->val);
+    return rows_numeric(plan, S, c, sc, scratch_bytes, rowptr, C->crd[last], C->val);
 }
 
 spws_status_t spws_gather_ceiling(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, const spws_tensor_t* C,

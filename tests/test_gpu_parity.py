@@ -134,6 +134,44 @@ def test_ism_warp_rows_at_every_register_width(ctx, oracle_mod, ncols, dtype):
     check_spgemm(ctx, oracle_mod, A, B, "auto")
 
 
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("ncols", [2000, 1 << 22])
+def test_sorted_words_kept_for_the_numeric_pass(ctx, oracle_mod, ncols, dtype):
+    """Rows of 257 .. 1024 products with scratch of exactly the passes' need (both sort) and with the room the
+    sized symbolic pass asks for (the numeric pass takes the order the counting pass left): the same
+    results bit for bit, and again after the values change in place."""
+    import torch
+    from paper_2404_04541_b200 import api, binding
+    targets = [200, 256, 257, 383, 384, 385, 511, 512, 513, 767, 769, 1000, 1023, 1024, 1025] * 3
+    A, B = _rows_with_products(targets, ncols, 21, dtype)
+    dA, dB = api.DeviceCSR.from_host(A), api.DeviceCSR.from_host(B)
+    plan = ctx.plan(api.EXPR_SPGEMM, (binding.SPWS_CSR,) * 3, dtype, "ism")
+    a, b = dA.arrays(), dB.arrays()
+    own = plan.workspace_size_exact(a, b)
+    exact = plan.workspace_size_exact(a, b, ctx._aligned_ptr(torch.empty(own + 256, dtype=torch.uint8, device="cuda")), own)
+    pos = torch.empty(A.nrows + 1, dtype=torch.int64, device="cuda")
+    c = binding.csr_arrays(A.nrows, B.ncols, pos, None, None)
+    _, sized = plan.symbolic_sized(a, b, c, None, 0)
+    buf = torch.empty(max(sized, exact) + (8 << 20), dtype=torch.uint8, device="cuda")
+    _, sized = plan.symbolic_sized(a, b, c, ctx._aligned_ptr(buf), buf.numel() - 256)
+    assert sized > exact
+    for vals in (A.val, A.val[::-1].copy()):
+        dA.val.copy_(torch.from_numpy(vals))
+        ref = oracle_mod.spgemm(CSR(A.nrows, A.ncols, A.pos, A.crd, vals), B, threads=4)
+        got = []
+        for room in (exact, sized):
+            plan.symbolic(a, b, c, ctx._aligned_ptr(buf), room)
+            crd = torch.empty(c.n[1], dtype=torch.int32, device="cuda")
+            val = torch.empty(c.n[1], dtype=dA.val.dtype, device="cuda")
+            c.crd[1], c.val = crd, val
+            plan.numeric(a, b, c, ctx._aligned_ptr(buf), room)
+            plan.get_stats()
+            got.append((pos.cpu().numpy(), crd.cpu().numpy(), val.cpu().numpy()))
+            assert_matches(got[-1], ref, dtype)
+        assert all(np.array_equal(x, y) for x, y in zip(*got))
+    plan.close()
+
+
 @pytest.mark.parametrize("policy", POLICIES)
 def test_edge_cases(ctx, oracle_mod, policy):
     # all-empty A, empty B rows, one huge row among empty ones
