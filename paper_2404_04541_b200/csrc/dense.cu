@@ -486,9 +486,20 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
 // many products.  Every unit streams its B rows once, whole.  Outputs with rank < CAP accumulate
 // in shared memory; outputs beyond accumulate straight into the row's value segment in global
 // memory (zeroed beforehand), which keeps any row to a single pass whatever its output count.
+// Bound by latency: the ranks and the compare-and-swap loops of the shared-memory additions form chains, at 32 warps
+// per SM (64 registers, 111 KB).  Power law on 2^18 / 16381 vertices, f64 / f32: with nine barriers per unit,
+// metadata fetched between them and loads one step ahead 14050 / 309 us; without the prefetch (its register copies
+// cost more than the other warps' work hides) and with two steps to find a tile's entry 13590 / 287 us; with three barriers and the next unit
+// fetched meanwhile 12770 / 252 us.  Every output in shared memory, by segments of a row's ranks: 28000 / 339 us.
 // ---------------------------------------------------------------------------------------
 constexpr int DN_ENTRIES = 768;      // A entries whose descriptors are staged per round
 constexpr int DN_TILE = 256;         // products a warp takes per fetch
+
+// What a block needs to know of a unit, fetched by one thread while the block is busy with the unit before.
+struct CtaUnit {
+    i64 e_lo, e_hi, out0, bm;           // A entries, first output, bitmap
+    int base, nw, cnt, nun, mean, valid;    // mean: products per entry
+};
 
 // CEIL = true is the same traversal with the workspace stripped (the iteration-only lower bound of
 // Sec. 7.2): units, descriptor rounds, product tiles and gathers as below, but no bitmap, no rank
@@ -500,14 +511,14 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
                                                                    u64* __restrict__ chk_idx, double* __restrict__ chk_val) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* acc = reinterpret_cast<T*>(smem_raw);                                        // CAP
-    // per bitmap word: .x = the word, .y = outputs of the row before it (one load gives a rank)
+    // per bitmap word: .x = the word, .y = outputs of the row before it, less one (one load gives a rank)
     uint2* bmr = reinterpret_cast<uint2*>(acc + CAP);                                // smem_words
     // staged descriptors of up to DN_ENTRIES A entries: B-row start, A value, running product count
     i64* d_qs = reinterpret_cast<i64*>(smem_raw + ((sizeof(T) * (size_t)CAP + 8 * (size_t)smem_words + 15) & ~(size_t)15));
     T* d_a = reinterpret_cast<T*>(d_qs + DN_ENTRIES);
     int* d_pre = reinterpret_cast<int*>(d_a + DN_ENTRIES);                           // DN_ENTRIES + 1
-    __shared__ int s_next, s_tile;
-    __shared__ int ws[33];
+    __shared__ CtaUnit s_unit[2];
+    __shared__ int s_tile, ws[DN_WARPS];
     if (ctl->status != 0) return;
     const int n_units = ctl->n_units;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -518,185 +529,185 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
     u64 my_idx = 0;
     double my_val = 0.0;
 
-    for (;;) {
-        __syncthreads();
-        if (tid == 0) s_next = atomicAdd(&ctl->work_counter[(CEIL ? CEIL_SLOT : NUM_SLOT) + CLS_DENSE_CTA], 1);
-        __syncthreads();
-        if (s_next >= n_units) break;
-        const int u = unit_at(s_next, n_units);
+    auto fetch_unit = [&](CtaUnit& U) {                 // one thread
+        const int t = atomicAdd(&ctl->work_counter[(CEIL ? CEIL_SLOT : NUM_SLOT) + CLS_DENSE_CTA], 1);
+        U.valid = t < n_units;
+        if (t >= n_units) return;
+        const int u = unit_at(t, n_units);
         const int row = tab.unit_row[u];
         const int uidx = u - tab.row_unit0[row];
-        const int nun = dense_units_of_row(tab.ub[row], unit_products);
-        const int base = tab.jmin[row], last = tab.jmax[row];
-        const int nw = min((last - base) / 32 + 1, smem_words);
-        const int nch = chunks_of(nw);
-        const unsigned span_bits = (unsigned)nw * 32u;
-        const i64 out0 = rowptr[row];
-        const int cnt = (int)(rowptr[row + 1] - out0);
-        const i64 ps = A.pos[row], pe = A.pos[row + 1];
-        const i64 e_lo = ps + (pe - ps) * uidx / nun, e_hi = ps + (pe - ps) * (uidx + 1) / nun;
-        T* const gacc = Cval + out0;
-        if (!CEIL && nun == 1)                          // outputs beyond the shared-memory part start at zero
-            for (int x = CAP + tid; x < cnt; x += DN_THREADS) gacc[x] = 0;
+        const i64 ub = tab.ub[row], ps = A.pos[row], n = A.pos[row + 1] - ps, out0 = rowptr[row];
+        const int nun = dense_units_of_row(ub, unit_products), base = tab.jmin[row];
+        U.nw = min((tab.jmax[row] - base) / 32 + 1, smem_words);
+        U.bm = tab.bm_off[row];
+        U.cnt = (int)(rowptr[row + 1] - out0);
+        U.e_lo = ps + n * uidx / nun;
+        U.e_hi = ps + n * (uidx + 1) / nun;
+        U.mean = (int)min(ub / max(n, (i64)1), (i64)0x7fffffff);
+        U.out0 = out0;
+        U.base = base;
+        U.nun = nun;
+    };
+    if (tid == 0) fetch_unit(s_unit[0]);
+    __syncthreads();
 
-        // the row's bitmap with the rank of every word's first bit (the symbolic pass saved the
-        // rank at every chunk start).  A warp takes eight chunks at a time, all loads first.
-        const unsigned* src = tab.bm_arena + tab.bm_off[row];
-        for (int c0 = warp; !CEIL && c0 < nch; c0 += DN_WARPS * 8) {
-            unsigned word[8], rank_c[8];
+    // Three barriers per round of descriptors and none besides: whatever a unit writes before its first tile is
+    // next read behind two of them, and the unit before has left its tiles behind one.
+    for (int cur = 0;; cur ^= 1) {
+        const CtaUnit& U = s_unit[cur];
+        if (!U.valid) break;
+        const int base = U.base, cnt = U.cnt;
+        const unsigned span_bits = (unsigned)U.nw * 32u;
+        T* const gacc = Cval + U.out0;
+        if (!CEIL) {
+            if (U.nun == 1)                             // outputs beyond the shared-memory part start at zero
+                for (int x = CAP + tid; x < cnt; x += DN_THREADS) gacc[x] = 0;
+            // the row's bitmap with the rank of every word's first bit (the symbolic pass saved the
+            // rank at every chunk start).  A warp takes eight chunks at a time, all loads first.
+            const unsigned* src = tab.bm_arena + U.bm;
+            const int nw = U.nw, nch = chunks_of(nw);
+            for (int c0 = warp; c0 < nch; c0 += DN_WARPS * 8) {
+                unsigned word[8], rank_c[8];
 #pragma unroll
-            for (int x = 0; x < 8; ++x) {
-                const int c = c0 + x * DN_WARPS, w = (c << 5) + lane;
-                word[x] = (w < nw) ? src[w] : 0u;
-                rank_c[x] = (c < nch) ? src[nw + c] : 0u;
-            }
-#pragma unroll
-            for (int x = 0; x < 8; ++x) {
-                const int c = c0 + x * DN_WARPS, w = (c << 5) + lane;
-                const int pc = __popc(word[x]);
-                const int incl = warp_incl_scan(pc);
-                if (w < nw) bmr[w] = make_uint2(word[x], rank_c[x] + (unsigned)(incl - pc));
-            }
-        }
-        __syncthreads();
-
-#define SPWS_DENSE_ADD(REL, VAL)                                                                          \
-        if (CEIL) {                                                                                       \
-            if ((REL) != 0xffffffffu) { my_idx += (u64)((REL) + (unsigned)base); my_val += (double)(VAL); } \
-        } else if ((REL) < span_bits) {                                                                   \
-            const uint2 br_ = bmr[(REL) >> 5];                                                            \
-            const int r_ = (int)br_.y + __popc(br_.x & ((1u << ((REL) & 31)) - 1u));                      \
-            if (r_ < CAP) atomicAdd(&acc[r_], (VAL));                                                     \
-            else if (r_ < cnt) atomicAdd(gacc + r_, (VAL));                                               \
-        }
-
-        const float avg_len = (float)tab.ub[row] / fmaxf(1.0f, (float)(pe - ps));
-        const bool long_rows = avg_len >= 64.0f;
-        {
-            // Rounds of up to DN_ENTRIES A entries.  Step 1: every thread fetches the descriptors
-            // of two entries; a block scan turns the B-row lengths into a running product count.
-            // Step 2: warps pull tiles of DN_TILE consecutive products of that stream, so the
-            // work is shared evenly however long the individual B rows are.
-            for (i64 e0 = e_lo; e0 < e_hi; e0 += DN_ENTRIES) {
-                const int nE = (int)min((i64)DN_ENTRIES, e_hi - e0);
-                int len2[2] = {0, 0};
-#pragma unroll
-                for (int x = 0; x < 2; ++x) {
-                    const int i = 2 * tid + x;
-                    if (i < nE) {
-                        const int k = __ldg(A.crd + e0 + i);
-                        i64 qs = 0;
-                        if ((unsigned)k < (unsigned)B.nrows) {
-                            qs = __ldg(B.pos + k);
-                            len2[x] = (int)(__ldg(B.pos + k + 1) - qs);
-                        }
-                        d_qs[i] = qs;
-                        d_a[i] = __ldg(Aval + e0 + i);
-                    }
+                for (int x = 0; x < 8; ++x) {
+                    const int c = c0 + x * DN_WARPS, w = (c << 5) + lane;
+                    word[x] = (w < nw) ? src[w] : 0u;
+                    rank_c[x] = (c < nch) ? src[nw + c] : 0u;
                 }
-                int total;
-                const int excl = block_excl_scan<DN_THREADS>(len2[0] + len2[1], ws, total);
-                if (2 * tid < nE) d_pre[2 * tid] = excl;
-                if (2 * tid + 1 < nE) d_pre[2 * tid + 1] = excl + len2[0];
-                if (tid == 0) { d_pre[nE] = total; s_tile = 0; }
-                __syncthreads();
-                // Every warp walks the product stream tile by tile.  The loads of a step are
-                // issued before the previous step is ranked and added, so gather latency and
-                // accumulation overlap inside a warp as well as across warps.
-                int t0 = 0, t1 = 0, e = 0;              // stream position, end of the tile in hand, entry at t0
-                auto next_tile = [&]() -> bool {
-                    int s = 0;
-                    if (lane == 0) s = atomicAdd(&s_tile, DN_TILE);
-                    t0 = __shfl_sync(0xffffffffu, s, 0);
-                    if (t0 >= total) return false;
-                    t1 = min(total, t0 + DN_TILE);
-                    int lo = 0, hi = nE;                // the last entry whose running count is <= t0
-                    while (hi - lo > 1) {
-                        const int mid = (lo + hi) >> 1;
-                        if (d_pre[mid] <= t0) lo = mid; else hi = mid;
+#pragma unroll
+                for (int x = 0; x < 8; ++x) {
+                    const int c = c0 + x * DN_WARPS, w = (c << 5) + lane;
+                    const int pc = __popc(word[x]);
+                    const int incl = warp_incl_scan(pc);
+                    if (w < nw) bmr[w] = make_uint2(word[x], rank_c[x] + (unsigned)(incl - pc) - 1u);
+                }
+            }
+        }
+
+        auto add = [&](unsigned rel, T v) {
+            if (CEIL) {
+                if (rel != 0xffffffffu) { my_idx += (u64)(rel + (unsigned)base); my_val += (double)v; }
+            } else if (rel < span_bits) {
+                const uint2 br = bmr[rel >> 5];
+                // the column's bit is set: bits up to and including it, one less in the table
+                const unsigned r = br.y + (unsigned)__popc(__funnelshift_l(0u, br.x, ~rel));
+                if (r < (unsigned)CAP) atomicAdd(&acc[r], v);
+                else if (r < (unsigned)cnt) atomicAdd(gacc + r, v);
+            }
+        };
+
+        bool next_known = false;
+        // Rounds of up to DN_ENTRIES A entries.  Step 1: every thread fetches the descriptors
+        // of two entries; a block scan turns the B-row lengths into a running product count.
+        // Step 2: warps pull tiles of DN_TILE consecutive products of that stream, so the
+        // work is shared evenly however long the individual B rows are.
+        const i64 e_hi = U.e_hi;
+        for (i64 e0 = U.e_lo; e0 < e_hi; e0 += DN_ENTRIES) {
+            const int nE = (int)min((i64)DN_ENTRIES, e_hi - e0);
+            int len2[2] = {0, 0};
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                const int i = 2 * tid + x;
+                if (i < nE) {
+                    const int k = __ldg(A.crd + e0 + i);
+                    i64 qs = 0;
+                    if ((unsigned)k < (unsigned)B.nrows) {
+                        qs = __ldg(B.pos + k);
+                        len2[x] = (int)(__ldg(B.pos + k + 1) - qs);
                     }
-                    e = lo;
-                    return true;
-                };
-                if (long_rows) {
-                    // a step = up to 128 consecutive products of one B row, four per lane
-                    auto fetch = [&](unsigned (&rel)[4], T (&b)[4], T& a) -> bool {
-                        if (t0 >= t1 && !next_tile()) return false;
-                        while (d_pre[e + 1] <= t0) ++e;
-                        const int off = t0 - d_pre[e];
-                        const int n = min(min(t1, d_pre[e + 1]) - t0, 128);
-                        const int* __restrict__ ck = B.crd + d_qs[e] + off;
-                        const T* __restrict__ vk = Bval + d_qs[e] + off;
-                        a = d_a[e];
+                    d_qs[i] = qs;
+                    d_a[i] = __ldg(Aval + e0 + i);
+                }
+            }
+            const int incl = warp_incl_scan(len2[0] + len2[1]);
+            if (lane == 31) ws[warp] = incl;
+            if (tid == 0) s_tile = 0;
+            __syncthreads();
+            const int wt = lane < DN_WARPS ? ws[lane] : 0;
+            const int wi = warp_incl_scan(wt);
+            const int total = __shfl_sync(0xffffffffu, wi, 31);
+            const int excl = __shfl_sync(0xffffffffu, wi - wt, warp) + incl - len2[0] - len2[1];
+            if (2 * tid < nE) d_pre[2 * tid] = excl;
+            if (2 * tid + 1 < nE) d_pre[2 * tid + 1] = excl + len2[0];
+            if (tid == 0) d_pre[nE] = total;
+            __syncthreads();
+            if (!next_known && tid == DN_THREADS - 1) fetch_unit(s_unit[cur ^ 1]);
+            next_known = true;
+            __syncwarp();
+
+            int t0 = 0, t1 = 0, e = 0;              // stream position, end of the tile in hand, entry at t0
+            auto next_tile = [&]() -> bool {
+                int s = 0;
+                if (lane == 0) s = atomicAdd(&s_tile, DN_TILE);
+                t0 = __shfl_sync(0xffffffffu, s, 0);
+                if (t0 >= total) return false;
+                t1 = min(total, t0 + DN_TILE);
+                // the last entry whose running count is <= t0: among 32 spread entries, then among those in between
+                constexpr int STRIDE = DN_ENTRIES / 32;
+                static_assert(STRIDE <= 32, "two steps");
+                const int i1 = lane * STRIDE;
+                const int lo = (__popc(__ballot_sync(0xffffffffu, i1 < nE && d_pre[i1] <= t0)) - 1) * STRIDE;
+                const int i2 = lo + lane;
+                e = lo + __popc(__ballot_sync(0xffffffffu, lane < STRIDE && i2 < nE && d_pre[i2] <= t0)) - 1;
+                return true;
+            };
+            if (U.mean >= 64) {
+                // a step = up to 128 consecutive products of one B row, four per lane, all loads first
+                while (t0 < t1 || next_tile()) {
+                    int next = d_pre[e + 1];
+                    while (next <= t0) next = d_pre[++e + 1];
+                    const int n = min(min(t1, next) - t0, 128);
+                    const i64 q = d_qs[e] + (t0 - d_pre[e]) + lane;
+                    const int* __restrict__ ck = B.crd + q;
+                    const T* __restrict__ vk = Bval + q;
+                    const T a = d_a[e];
+                    unsigned rel[4];
+                    T b[4];
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        rel[x] = 0xffffffffu;
+                        if (lane + 32 * x < n) { rel[x] = (unsigned)(__ldg(ck + 32 * x) - base); b[x] = __ldg(vk + 32 * x); }
+                    }
+                    t0 += n;
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) add(rel[x], a * b[x]);
+                }
+            } else {
+                // short B rows: a step = 128 consecutive products of the stream, four per lane; every lane advances
+                // its own entry index across row boundaries
+                while (next_tile()) {
+                    int my_e = e;
+                    for (; t0 < t1; t0 += 128) {
+                        unsigned rel[4];
+                        T b[4];
 #pragma unroll
                         for (int x = 0; x < 4; ++x) {
-                            const int idx = lane + 32 * x;
-                            rel[x] = idx < n ? (unsigned)(__ldg(ck + idx) - base) : 0xffffffffu;
-                            b[x] = idx < n ? __ldg(vk + idx) : (T)0;
-                        }
-                        t0 += n;
-                        return true;
-                    };
-                    unsigned relc[4] = {0, 0, 0, 0}, reln[4] = {0, 0, 0, 0};
-                    T bc[4] = {0, 0, 0, 0}, bn[4] = {0, 0, 0, 0};
-                    T ac = 0, an = 0;
-                    bool have = fetch(relc, bc, ac);
-                    while (have) {
-                        const bool more = fetch(reln, bn, an);
-#pragma unroll
-                        for (int x = 0; x < 4; ++x) { SPWS_DENSE_ADD(relc[x], ac * bc[x]) }
-#pragma unroll
-                        for (int x = 0; x < 4; ++x) { relc[x] = reln[x]; bc[x] = bn[x]; }
-                        ac = an;
-                        have = more;
-                    }
-                } else {
-                    // short B rows: a step = 64 consecutive products of the stream, two per lane;
-                    // every lane advances its own entry index across row boundaries
-                    int my_e = 0;
-                    auto fetch = [&](unsigned (&rel)[2], T (&b)[2], T (&a)[2]) -> bool {
-                        if (t0 >= t1) {
-                            if (!next_tile()) return false;
-                            my_e = e;
-                        }
-#pragma unroll
-                        for (int x = 0; x < 2; ++x) {
                             const int t = t0 + lane + 32 * x;
                             rel[x] = 0xffffffffu;
-                            b[x] = 0;
-                            a[x] = 0;
                             if (t < t1) {
                                 while (d_pre[my_e + 1] <= t) ++my_e;
                                 const i64 q = d_qs[my_e] + (t - d_pre[my_e]);
-                                a[x] = d_a[my_e];
                                 rel[x] = (unsigned)(__ldg(B.crd + q) - base);
-                                b[x] = __ldg(Bval + q);
+                                b[x] = d_a[my_e] * __ldg(Bval + q);
                             }
                         }
-                        t0 = min(t1, t0 + 64);
-                        return true;
-                    };
-                    unsigned relc[2] = {0, 0}, reln[2] = {0, 0};
-                    T bc[2] = {0, 0}, bn[2] = {0, 0}, ac[2] = {0, 0}, an[2] = {0, 0};
-                    bool have = fetch(relc, bc, ac);
-                    while (have) {
-                        const bool more = fetch(reln, bn, an);
 #pragma unroll
-                        for (int x = 0; x < 2; ++x) { SPWS_DENSE_ADD(relc[x], ac[x] * bc[x]) }
-#pragma unroll
-                        for (int x = 0; x < 2; ++x) { relc[x] = reln[x]; bc[x] = bn[x]; ac[x] = an[x]; }
-                        have = more;
+                        for (int x = 0; x < 4; ++x) add(rel[x], b[x]);
                     }
                 }
-                __syncthreads();
             }
+            __syncthreads();
         }
-#undef SPWS_DENSE_ADD
+        if (!next_known) {                              // a share without entries
+            __syncthreads();
+            if (tid == 0) fetch_unit(s_unit[cur ^ 1]);
+            __syncthreads();
+        }
 
         // copy out the shared-memory part of the values (the coordinates are written by
         // dense_emit_crd_kernel)
         const int n_smem = CEIL ? 0 : min(cnt, CAP);
-        if (nun == 1) {
+        if (U.nun == 1) {
             for (int x = tid; x < n_smem; x += DN_THREADS) { gacc[x] = acc[x]; acc[x] = 0; }
         } else {
             for (int x = tid; x < n_smem; x += DN_THREADS) {
