@@ -199,63 +199,79 @@ __global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __re
 
 // ---------------------------------------------------------------------------------------
 // symbolic, CTA per row (hub rows first: classes HUB and CTA are adjacent in perm)
+// Bound by latency: chains of loads and the barriers of short rows.  With entries dealt out in turn, eight barriers per row
+// and a chain of four loads per entry, power law on 2^18 / 60000 / 16381 vertices: 3149 / 726 / 193 us; now 2915 /
+// 622 / 183 us.
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(DC_THREADS) dense_sym_cta_kernel(DevCtl* __restrict__ ctl, int smem_words, Csr A, Csr B, RowTables tab,
+// What a block needs to know of a row, fetched by one thread while the block is busy with the row before.
+struct SymRow {
+    i64 ps, pe, bm;
+    int row, base, nw, gs, batch;       // row < 0: no more rows
+};
+
+__global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __restrict__ ctl, int smem_words, Csr A, Csr B, RowTables tab,
                                                                    const uint2* __restrict__ bw) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    unsigned* bm = reinterpret_cast<unsigned*>(smem_raw);                 // smem_words
+    unsigned* bm = reinterpret_cast<unsigned*>(smem_raw);                 // smem_words, clear between rows
     int* chunk = reinterpret_cast<int*>(bm + smem_words);                  // smem_words / 32
-    __shared__ int s_next;
-    __shared__ int ws[33];
+    __shared__ SymRow s_row[2];
+    __shared__ int s_entry[2];                                              // A entries handed out
     if (ctl->status != 0) return;
     int off, n_hub, o6, n_cta;
     class_range(ctl, CLS_DENSE_HUB, off, n_hub);
     class_range(ctl, CLS_DENSE_CTA, o6, n_cta);
     const int n = n_hub + n_cta;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (;;) {
-        __syncthreads();
-        if (tid == 0) s_next = atomicAdd(&ctl->work_counter[CLS_DENSE_CTA], 1);
-        __syncthreads();
-        const int r = s_next;
-        if (r >= n) break;
-        const int row = tab.perm[off + r];
-        const int base = tab.jmin[row];
-        const int nw = min((tab.jmax[row] - base) / 32 + 1, smem_words);
+    auto fetch_row = [&](int to) {                      // one thread
+        SymRow& R = s_row[to];
+        const int r = atomicAdd(&ctl->work_counter[CLS_DENSE_CTA], 1);
+        s_entry[to] = 0;
+        R.row = -1;
+        if (r >= n) return;
+        const int row = tab.perm[off + r], base = tab.jmin[row];
+        R.ps = A.pos[row];
+        R.pe = A.pos[row + 1];
+        R.bm = tab.bm_off[row];
+        R.nw = min((tab.jmax[row] - base) / 32 + 1, smem_words);
+        const i64 ub = tab.ub[row], entries = R.pe - R.ps;
+        R.gs = pick_group_size(ub, entries, 1);
+        R.batch = ub < 512 * entries ? 8 : 4;
+        R.base = base;
+        R.row = row;
+    };
+    if (tid == 0) fetch_row(0);
+    for (int w = tid; w < smem_words; w += DC_THREADS) bm[w] = 0;
+    __syncthreads();
+    // two barriers per row: before the bitmap is saved (and cleared), and after
+    for (int cur = 0;; cur ^= 1) {
+        const SymRow& R = s_row[cur];
+        if (R.row < 0) break;
+        const int base = R.base, nw = R.nw, gs = R.gs;
         const unsigned span = (unsigned)nw * 32u;
         const unsigned base_w = (unsigned)base >> 5;                     // base is a multiple of 32
-        const i64 ps = A.pos[row], pe = A.pos[row + 1];
-        for (int w = tid; w < nw; w += DC_THREADS) bm[w] = 0;
-        __syncthreads();
-        const int gs = pick_group_size(tab.ub[row], pe - ps, 1);
-        const int g = tid / gs, gl = tid % gs, ng = DC_THREADS / gs;
-        for (i64 p = ps + g; p < pe; p += ng) {
-            const int k = __ldg(A.crd + p);
-            if ((unsigned)k >= (unsigned)B.nrows) continue;
-            const i64 qs = __ldg(B.pos + k);
-            const int len = (int)(__ldg(B.pos + k + 1) - qs);
-            if (bw && len >= BW_MIN_LEN) {
-                // a long B row with a word list: one atomic per (word, bits) pair, and the lanes
-                // of a warp hold distinct words
-                const int np = (int)__ldg(&bw[qs].x);
-                if (np > 0) {
-                    const uint2* __restrict__ pk = bw + qs + 1;
-                    int t = gl;
-                    for (; t + 3 * gs < np; t += 4 * gs) {
-                        const uint2 e0 = __ldg(pk + t), e1 = __ldg(pk + t + gs), e2 = __ldg(pk + t + 2 * gs), e3 = __ldg(pk + t + 3 * gs);
-                        const unsigned w0 = e0.x - base_w, w1 = e1.x - base_w, w2 = e2.x - base_w, w3 = e3.x - base_w;
-                        if (w0 < (unsigned)nw) atomicOr(&bm[w0], e0.y);
-                        if (w1 < (unsigned)nw) atomicOr(&bm[w1], e1.y);
-                        if (w2 < (unsigned)nw) atomicOr(&bm[w2], e2.y);
-                        if (w3 < (unsigned)nw) atomicOr(&bm[w3], e3.y);
-                    }
-                    for (; t < np; t += gs) {
-                        const uint2 e0 = __ldg(pk + t);
-                        const unsigned w0 = e0.x - base_w;
-                        if (w0 < (unsigned)nw) atomicOr(&bm[w0], e0.y);
-                    }
-                    continue;
+        const i64 ps = R.ps, pe = R.pe;
+        if (tid == DC_THREADS - 1) fetch_row(cur ^ 1);
+        __syncwarp();
+        // one B row by `gs` lanes, of which this is lane gl
+        auto take = [&](i64 qs, int len, int np, int gl, int gs) {
+            if (np > 0) {
+                // a long B row with a word list: one atomic per (word, bits) pair, and the lanes hold distinct words
+                const uint2* __restrict__ pk = bw + qs + 1;
+                int t = gl;
+                for (; t + 3 * gs < np; t += 4 * gs) {
+                    const uint2 e0 = __ldg(pk + t), e1 = __ldg(pk + t + gs), e2 = __ldg(pk + t + 2 * gs), e3 = __ldg(pk + t + 3 * gs);
+                    const unsigned w0 = e0.x - base_w, w1 = e1.x - base_w, w2 = e2.x - base_w, w3 = e3.x - base_w;
+                    if (w0 < (unsigned)nw) atomicOr(&bm[w0], e0.y);
+                    if (w1 < (unsigned)nw) atomicOr(&bm[w1], e1.y);
+                    if (w2 < (unsigned)nw) atomicOr(&bm[w2], e2.y);
+                    if (w3 < (unsigned)nw) atomicOr(&bm[w3], e3.y);
                 }
+                for (; t < np; t += gs) {
+                    const uint2 e0 = __ldg(pk + t);
+                    const unsigned w0 = e0.x - base_w;
+                    if (w0 < (unsigned)nw) atomicOr(&bm[w0], e0.y);
+                }
+                return;
             }
             const int* __restrict__ ck = B.crd + qs;
             int t = gl;
@@ -273,28 +289,67 @@ __global__ void __launch_bounds__(DC_THREADS) dense_sym_cta_kernel(DevCtl* __res
                 const unsigned r0 = (unsigned)(__ldg(ck + t) - base);
                 if (r0 < span) atomicOr(&bm[r0 >> 5], 1u << (r0 & 31));
             }
+        };
+        if (gs == 32) {
+            const int batch = R.batch;
+            // warps pull a batch of entries at a time: the chain of loads that leads to a B row is walked for all of
+            // them side by side, and no warp waits for one that met the longest B rows.  Eight entries, four
+            // when their B rows are long (whole batches weigh more than the chain then): power law on 2^18
+            // vertices 3350 us with eight, 2870 with four, 2900 with two; on 60000 620, 670 and 750 us
+            for (;;) {
+                int at = 0;
+                if (lane == 0) at = atomicAdd(&s_entry[cur], batch);
+                at = __shfl_sync(0xffffffffu, at, 0);
+                if (at >= pe - ps) break;
+                i64 my_qs = 0;
+                int my_len = 0, my_np = 0;
+                if (lane < batch && ps + at + lane < pe) {
+                    const int k = __ldg(A.crd + ps + at + lane);
+                    if ((unsigned)k < (unsigned)B.nrows) {
+                        my_qs = __ldg(B.pos + k);
+                        my_len = (int)(__ldg(B.pos + k + 1) - my_qs);
+                        if (bw && my_len >= BW_MIN_LEN) my_np = (int)__ldg(&bw[my_qs].x);
+                    }
+                }
+                const int nE = (int)min((i64)batch, pe - ps - at);
+                for (int i = 0; i < nE; ++i) {
+                    const i64 qs = __shfl_sync(0xffffffffu, my_qs, i);
+                    const int len = __shfl_sync(0xffffffffu, my_len, i), np = __shfl_sync(0xffffffffu, my_np, i);
+                    take(qs, len, np, lane, 32);
+                }
+            }
+        } else {
+            const int g = tid / gs, gl = tid % gs, ng = DC_THREADS / gs;
+            for (i64 p = ps + g; p < pe; p += ng) {
+                const int k = __ldg(A.crd + p);
+                if ((unsigned)k >= (unsigned)B.nrows) continue;
+                const i64 qs = __ldg(B.pos + k);
+                const int len = (int)(__ldg(B.pos + k + 1) - qs);
+                take(qs, len, bw && len >= BW_MIN_LEN ? (int)__ldg(&bw[qs].x) : 0, gl, gs);
+            }
         }
         __syncthreads();
         // save the bitmap, then the rank at every chunk start
-        unsigned* out = tab.bm_arena + tab.bm_off[row];
-        const int nch = chunks_of(nw);
+        unsigned* out = tab.bm_arena + R.bm;
+        const int nch = chunks_of(nw), row = R.row;
         for (int c = warp; c < nch; c += DC_WARPS) {
             const int w = (c << 5) + lane;
             const unsigned word = (w < nw) ? bm[w] : 0u;
-            if (w < nw) out[w] = word;
-            int pc = __popc(word);
-            for (int d = 16; d > 0; d >>= 1) pc += __shfl_xor_sync(0xffffffffu, pc, d);
+            if (w < nw) { out[w] = word; bm[w] = 0; }
+            const int pc = (int)__reduce_add_sync(0xffffffffu, (unsigned)__popc(word));
             if (lane == 0) chunk[c] = pc;
         }
         __syncthreads();
-        const int cpt = (nch + DC_THREADS - 1) / DC_THREADS;
-        const int c_lo = min(nch, tid * cpt), c_hi = min(nch, c_lo + cpt);
-        int local = 0;
-        for (int c = c_lo; c < c_hi; ++c) local += chunk[c];
-        int total;
-        int run = block_excl_scan<DC_THREADS>(local, ws, total);
-        for (int c = c_lo; c < c_hi; ++c) { out[nw + c] = (unsigned)run; run += chunk[c]; }
-        if (tid == 0) tab.cnt[row] = total;
+        if (warp == 0) {                                // the others go on with the next row
+            int carry = 0;
+            for (int c0 = 0; c0 < nch; c0 += 32) {
+                const int v = c0 + lane < nch ? chunk[c0 + lane] : 0;
+                const int incl = warp_incl_scan(v);
+                if (c0 + lane < nch) out[nw + c0 + lane] = (unsigned)(carry + incl - v);
+                carry += __shfl_sync(0xffffffffu, incl, 31);
+            }
+            if (lane == 0) tab.cnt[row] = carry;
+        }
     }
 }
 
