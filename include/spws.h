@@ -276,6 +276,18 @@ spws_status_t spws_symbolic_sized(spws_plan_t plan, const spws_tensor_t* A, cons
                                   const spws_tensor_t* D, spws_tensor_t* C, void* scratch, size_t scratch_bytes,
                                   int64_t* sizes_out, size_t* needed);
 
+/* spws_symbolic_sized (CSR and CSF results) in two halves, for a numeric pass that follows on the device without
+ * the host in between: that is possible when it needs nothing the symbolic pass finds out (no row goes to
+ * the dense workspace).  If it is, and the result's bound (one entry per product) is at most `most`, _begin
+ * returns once the pass is enqueued, with the bound in *upper; spws_numeric may then be called with room
+ * for *upper entries in C's last crd and val (C->n[] says so), and _end waits for the symbolic pass, fills
+ * in the sizes and returns its status (after a failure nothing of C is to be relied on).  Otherwise
+ * _begin is spws_symbolic_sized, *upper is 0 and there is no _end. */
+spws_status_t spws_symbolic_begin(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, spws_tensor_t* C,
+                                  void* scratch, size_t scratch_bytes, int64_t most, int64_t* sizes_out,
+                                  size_t* needed, int64_t* upper);
+spws_status_t spws_symbolic_end(spws_plan_t plan, spws_tensor_t* C, int64_t* sizes_out);
+
 /* Numeric pass.  C->crd[last] and C->val must now hold C->n[last] entries.  Asynchronous: returns
  * after enqueueing; a device-side failure is reported by the next spws_get_stats.  (The sparse
  * workspace of the outer-product form synchronises once per round of its accumulation array.) */

@@ -11,6 +11,10 @@ import torch
 
 from . import binding as B_
 
+# A result whose bound (one entry per product) fits in this many bytes may be given arrays of that size and cut to
+# its own: the numeric pass then follows the symbolic one on the device (2048 rows of 64 products, f64: 82 -> 71 us a call).
+BOUND_BYTES = 64 << 20
+
 EXPR_SPGEMM = "C(i,j) = A(i,k) * B(k,j)"
 EXPR_TTM = "C(i,j,l) = A(i,j,k) * B(k,l)"
 EXPR_OUTER = "C(i,j) = A(k,i) * B(k,j)"
@@ -109,6 +113,31 @@ class Context:
             sc = None
             sc = self.scratch(nbytes)
 
+    def _begin(self, plan: B_.Plan, a, b, c):
+        """The symbolic pass of a whole call.  When the numeric pass does not wait for its outcome and a bound
+        on the result fits BOUND_BYTES, the numeric pass is enqueued behind it into arrays of that size, so
+        that the device does not idle while the host learns the sizes: returns (state, (crd, val)), the
+        arrays to be cut to the sizes now in `c`.  Else returns (state, None) for the numeric call."""
+        sc = self._scratch
+        f64 = plan.np_dtype == np.float64
+        while True:
+            ptr = self._aligned_ptr(sc) if sc is not None else None
+            done, nbytes, upper = plan.symbolic_begin(a, b, c, ptr, sc.numel() - 256 if sc is not None else 0, BOUND_BYTES // (12 if f64 else 8))
+            if done:
+                break
+            sc = None
+            sc = self.scratch(nbytes)
+        room = None
+        if upper:
+            last = c.order - 1
+            c.crd[last] = torch.empty(upper, dtype=torch.int32, device=self.device)
+            c.val = torch.empty(upper, dtype=torch.float64 if f64 else torch.float32, device=self.device)
+            c.n[last] = upper
+            plan.numeric(a, b, c, ptr, nbytes)
+            plan.symbolic_end(c)
+            room = c.crd[last], c.val
+        return (a, b, sc, nbytes, c.n), room
+
     @staticmethod
     def _aligned_ptr(t: torch.Tensor) -> int:
         return (t.data_ptr() + 255) & ~255
@@ -123,7 +152,7 @@ class Context:
         return c, (a, b, sc, nbytes)
 
     def spgemm_numeric(self, plan: B_.Plan, c: B_.TensorArrays, state, crd=None, val=None) -> DeviceCSR:
-        a, b, sc, nbytes = state
+        a, b, sc, nbytes = state[:4]
         nnz = c.n[1]
         vt = torch.float64 if plan.np_dtype == np.float64 else torch.float32
         c.crd[1] = crd if crd is not None else torch.empty(nnz, dtype=torch.int32, device=self.device)
@@ -147,8 +176,15 @@ class Context:
             dt = np.float64 if A.val.dtype == torch.float64 else np.float32
             plan = self.plan(EXPR_SPGEMM, (B_.SPWS_CSR,) * 3, dt, policy, **options)
         try:
-            c, state = self.spgemm_symbolic(plan, A, B)
-            C = self.spgemm_numeric(plan, c, state)
+            a = B_.fixed(A.arrays())
+            b = a if B is A else B_.fixed(B.arrays())
+            c = B_.csr_arrays(A.nrows, B.ncols, torch.empty(A.nrows + 1, dtype=torch.int64, device=self.device), None, None)
+            state, room = self._begin(plan, a, b, c)
+            if room is None:
+                C = self.spgemm_numeric(plan, c, state)
+            else:
+                nnz = c.n[1]
+                C = DeviceCSR(A.nrows, B.ncols, c.pos[1], room[0][:nnz], room[1][:nnz])
             return C, plan.get_stats()
         finally:
             if own:
@@ -211,6 +247,11 @@ class Context:
     def ttm_symbolic(self, plan: B_.Plan, A: DeviceCSF3, B: DeviceCSR):
         """Symbolic pass of the 3-tensor form: allocates C's upper levels (bounded by A's) and returns
         (C arrays with sizes filled in, state for ttm_numeric)."""
+        a, b, c = self._ttm_arrays(A, B)
+        sc, nbytes = self._symbolic(plan, a, b, c)
+        return c, (a, b, sc, nbytes, c.n)
+
+    def _ttm_arrays(self, A: DeviceCSF3, B: DeviceCSR):
         a, b = B_.fixed(A.arrays()), B_.fixed(B.arrays())
         n_i, n_ij = a.n[0], a.n[1]
         i64, i32, dev = torch.int64, torch.int32, self.device
@@ -221,8 +262,12 @@ class Context:
         pos2 = torch.empty(n_ij + 1, dtype=i64, device=dev)
         c = B_.TensorArrays(3, (A.dims[0], A.dims[1], B.ncols), [pos0, pos1, pos2], [crd0, crd1, None], None,
                             [n_i, n_ij, 0])
-        sc, nbytes = self._symbolic(plan, a, b, c)
-        return c, (a, b, sc, nbytes, c.n)
+        return a, b, c
+
+    @staticmethod
+    def _ttm_result(c: B_.TensorArrays, sizes, crd, val) -> DeviceCSF3:
+        return DeviceCSF3(c.dims, c.pos[0], c.crd[0][:sizes[0]], c.pos[1][:sizes[0] + 1], c.crd[1][:sizes[1]],
+                          c.pos[2][:sizes[1] + 1], crd[:sizes[2]], val[:sizes[2]])
 
     def ttm_numeric(self, plan: B_.Plan, c: B_.TensorArrays, state, crd=None, val=None) -> DeviceCSF3:
         a, b, sc, nbytes, sizes = state
@@ -231,8 +276,7 @@ class Context:
         c.crd[2] = crd if crd is not None else torch.empty(nnz, dtype=torch.int32, device=self.device)
         c.val = val if val is not None else torch.empty(nnz, dtype=vt, device=self.device)
         plan.numeric(a, b, c, self._aligned_ptr(sc), nbytes)
-        return DeviceCSF3(c.dims, c.pos[0], c.crd[0][:sizes[0]], c.pos[1][:sizes[0] + 1], c.crd[1][:sizes[1]],
-                          c.pos[2][:sizes[1] + 1], c.crd[2][:nnz], c.val[:nnz])
+        return self._ttm_result(c, sizes, c.crd[2], c.val)
 
     def ttm(self, A: DeviceCSF3, B: DeviceCSR, policy="auto", plan: B_.Plan | None = None, **options):
         """C(i,j,l) = sum_k A(i,j,k) B(k,l) with A, C in CSF; returns (C, stats)."""
@@ -241,8 +285,12 @@ class Context:
             dt = np.float64 if A.val.dtype == torch.float64 else np.float32
             plan = self.plan(EXPR_TTM, (B_.SPWS_CSF3, B_.SPWS_CSF3, B_.SPWS_CSR), dt, policy, **options)
         try:
-            c, state = self.ttm_symbolic(plan, A, B)
-            C = self.ttm_numeric(plan, c, state)
+            a, b, c = self._ttm_arrays(A, B)
+            state, room = self._begin(plan, a, b, c)
+            if room is None:
+                C = self.ttm_numeric(plan, c, state)
+            else:
+                C = self._ttm_result(c, c.n, room[0], room[1])
             return C, plan.get_stats()
         finally:
             if own:

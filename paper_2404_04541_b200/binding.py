@@ -36,7 +36,7 @@ EXPORTS = ("spws_create", "spws_destroy", "spws_set_stream", "spws_plan_create",
            "spws_check_expression", "spws_workspace_size", "spws_workspace_size_exact", "spws_symbolic", "spws_numeric",
            "spws_get_stats", "spws_set_profiling", "spws_get_timings", "spws_execute_host", "spws_gather_ceiling",
            "spws_row_pointer_static", "spws_status_string", "spws_plan_create3", "spws_workspace_size3", "spws_symbolic3",
-           "spws_numeric3", "spws_symbolic_sized")
+           "spws_numeric3", "spws_symbolic_sized", "spws_symbolic_begin", "spws_symbolic_end")
 STATIC_MAX_ROWS = 16777216
 TIMING_GROUPS = ("sym_bounds", "sym_bin", "sym_ism_reg", "sym_ism_smem_s", "sym_ism_smem", "sym_dense_warp",
                  "sym_dense_cta", "sym_ism_global", "sym_hash", "sym_scan", "num_ism_reg", "num_ism_smem_s", "num_ism_smem",
@@ -102,6 +102,9 @@ def lib():
         L.spws_workspace_size3.argtypes = [vp, T, T, T, ctypes.POINTER(sz)]
         L.spws_symbolic3.argtypes = [vp, T, T, T, T, vp, sz, ctypes.POINTER(ctypes.c_int64)]
         L.spws_symbolic_sized.argtypes = [vp, T, T, T, T, vp, sz, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(sz)]
+        L.spws_symbolic_begin.argtypes = [vp, T, T, T, vp, sz, ctypes.c_int64, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(sz),
+                                          ctypes.POINTER(ctypes.c_int64)]
+        L.spws_symbolic_end.argtypes = [vp, T, ctypes.POINTER(ctypes.c_int64)]
         L.spws_numeric3.argtypes = [vp, T, T, T, T, vp, sz]
         L.spws_plan_destroy.argtypes = [vp]
         L.spws_check_expression.argtypes = [ctypes.c_char_p, ctypes.POINTER(i32), ctypes.POINTER(i32)]
@@ -286,6 +289,29 @@ class Plan:
         _check(st, "spws_symbolic")
         C.n = list(sizes)
         return True, need.value
+
+    def symbolic_begin(self, A, B, C, scratch_ptr, scratch_bytes: int, most: int):
+        """spws_symbolic_begin: (True, bytes the passes use, bound on the result's entries) with the pass enqueued,
+        (True, bytes, 0) with C's sizes filled in, or (False, bytes to try next, 0) when the scratch is
+        too small."""
+        a, b, c = A.c_struct(), B.c_struct(), C.c_struct()
+        sizes = (ctypes.c_int64 * 3)()
+        need, upper = ctypes.c_size_t(0), ctypes.c_int64(0)
+        st = lib().spws_symbolic_begin(self._p, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c), scratch_ptr, scratch_bytes, most, sizes,
+                                       ctypes.byref(need), ctypes.byref(upper))
+        if st == SPWS_SCRATCH_TOO_SMALL and need.value > scratch_bytes:
+            return False, need.value, 0
+        _check(st, "spws_symbolic")
+        if upper.value == 0:
+            C.n = list(sizes)
+        return True, need.value, upper.value
+
+    def symbolic_end(self, C):
+        """spws_symbolic_end: waits for the pass and fills in C's sizes."""
+        c = C.c_struct()
+        sizes = (ctypes.c_int64 * 3)()
+        _check(lib().spws_symbolic_end(self._p, ctypes.byref(c), sizes), "spws_symbolic")
+        C.n = list(sizes)
 
     def numeric(self, A, B, C, scratch_ptr: int, scratch_bytes: int, D=None):
         a, b, c = A.c_struct(), B.c_struct(), C.c_struct()

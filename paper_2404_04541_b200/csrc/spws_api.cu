@@ -72,6 +72,9 @@ struct spws_plan_s {
     bool in_flight = false;     // kernels that may still write to the pinned block are enqueued
     DevCtl* host_ctl = nullptr; // &host->ctl
     bool symbolic_ok = false;
+    bool pending = false;       // a symbolic pass is enqueued and not yet waited for (spws_symbolic_begin)
+    bool numeric_behind = false;                // .. and the numeric pass behind it
+    int64_t upper = 0;          // .. a bound on its result's entries when the numeric pass may be enqueued behind it, else 0
     spws_stats_t stats{};
     // what the last symbolic pass saw (numeric must be called with the same shapes and scratch)
     int64_t m = 0;
@@ -494,10 +497,12 @@ void use_order(const spws_plan_s* plan, LaunchCtx& c, char* sc, size_t scratch_b
 // ---- the row-wise passes: every output row (fibre) through the workspace of its class ------------
 // `ttmA` / `ttmC`: the 3-tensor operand and result, whose upper levels are rebuilt (null for the matrix
 // forms).  `c` is make_ctx of the layout; clear_ctl: the control block is not in use yet.  On success
-// the plan holds the statistics and what the numeric pass needs.
+// the pass is enqueued; rows_collect waits for it, and then the plan holds the statistics and what the numeric
+// pass needs.
 spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L, LaunchCtx& c, size_t scratch_bytes, size_t* needed, bool clear_ctl, const spws_tensor_t* ttmA,
                             spws_tensor_t* ttmC, i64* rowptr, char* sc) {
     plan->in_flight = true;
+    plan->pending = false;
     c.seq = plan->seq + 1;
     plan->seq += 2;
     // a1: upper bounds + classes; a2: binning
@@ -530,6 +535,7 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     plan->in_flight = true;
     i64 hcount[NCLASS];
     for (int k = 0; k < NCLASS; ++k) hcount[k] = hc.class_count[k];
+    const i64 products = hc.products;
     const bool any_dense = hcount[CLS_DENSE_WARP] + hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0;
     plan->max_ub_smem = hc.max_ub_smem;
     c.max_ub_smem = plan->max_ub_smem;
@@ -575,19 +581,35 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     else
         CUDA_TRY(launch_finish_rows(c, (int)S.m, any_dense, rowptr));
     mark(plan, SPWS_T_SYM_SCAN);
-    if ((st = wait_published(plan, c.seq + 1)) != SPWS_OK) return st;
-    plan->in_flight = false;
     plan->counters_clear = true;
     plan->rows_path = true;
+    // without dense rows the numeric pass needs nothing that the kernels above find out: it may follow them at once
+    for (int k = 0; k < NCLASS; ++k) plan->bin_rows[k] = hcount[k];
     plan->stats = spws_stats_t{};
+    plan->stats.launches_symbolic = c.launches;
+    plan->m = S.m;
+    plan->upper = any_dense ? 0 : products;
+    return SPWS_OK;
+}
+
+// Waits for the symbolic pass that rows_symbolic enqueued and takes over what it found out.
+spws_status_t rows_collect(spws_plan_s* plan) {
+    plan->pending = false;
+    const spws_status_t st = wait_published(plan, plan->seq);
+    if (st != SPWS_OK) return st;
+    if (!plan->numeric_behind) plan->in_flight = false;
+    const DevCtl& hc = *plan->host_ctl;
+    const spws_stats_t enqueued = plan->stats;
+    plan->stats = spws_stats_t{};
+    plan->stats.launches_symbolic = enqueued.launches_symbolic;
+    plan->stats.launches_numeric = enqueued.launches_numeric;
     plan->stats.device_status = hc.status;
     if (hc.status != 0) return from_dev_status(hc.status);
-    plan->stats.rows = S.m;
+    plan->stats.rows = plan->m;
     plan->stats.products = hc.products;
     plan->stats.nnz = hc.nnz;
     plan->stats.max_row_products = hc.max_ub;
     for (int k = 0; k < NCLASS; ++k) {
-        plan->bin_rows[k] = hc.class_count[k];
         plan->stats.rows_per_class[public_class(k)] += hc.class_count[k];
         plan->stats.products_per_class[public_class(k)] += hc.class_products[k];
         plan->stats.nnz_per_class[public_class(k)] += hc.class_nnz[k];
@@ -602,7 +624,6 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
         plan->n_warp[list] = hc.n_warp_rows[list];
         plan->max_warp_cnt[list] = hc.max_warp_cnt[list];
     }
-    plan->stats.launches_symbolic = c.launches;
     return SPWS_OK;
 }
 
@@ -839,8 +860,8 @@ spws_status_t rw_outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_
     CUDA_TRY(cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream));
     mark_start(plan, 0);
     CUDA_TRY(launch_rw_outer(c, S.A, S.nnzA, S.B, S.nnzB, label_bits_of(S.m, 1), rw_bufs(sc + w.L.extra, w.R)));
-    const spws_status_t st = rows_symbolic(plan, w.S, w.L, c, scratch_bytes, needed, false, nullptr, nullptr, LL(C->pos[1]), sc);
-    if (st != SPWS_OK) return st;
+    spws_status_t st = rows_symbolic(plan, w.S, w.L, c, scratch_bytes, needed, false, nullptr, nullptr, LL(C->pos[1]), sc);
+    if (st != SPWS_OK || (st = rows_collect(plan)) != SPWS_OK) return st;
     C->n[0] = C->dims[0];
     C->n[1] = plan->stats.nnz;
     C->n[2] = 0;
@@ -1119,8 +1140,8 @@ spws_status_t rw_higher_symbolic(spws_plan_s* plan, const HShapes& H, int64_t P,
         CUDA_TRY(launch_rw_fibre_rows(c, false, H.B, H.C, H.D, reinterpret_cast<int*>(x + w.R.fcnt), reinterpret_cast<i64*>(x + w.R.fpos),
                                       reinterpret_cast<int*>(x + w.R.fcrd), nullptr, reinterpret_cast<i64*>(x + w.R.block_sums)));
     CUDA_TRY(launch_rw_csf(c, H.form, H.B, (u64)(H.order == 3 ? H.odims[1] : 1), w.m, w.bits, rw_bufs(x, w.R)));
-    const spws_status_t st = rows_symbolic(plan, w.S, w.L, c, scratch_bytes, needed, false, nullptr, nullptr, reinterpret_cast<i64*>(x + w.R.rowptr), sc);
-    if (st != SPWS_OK) return st;
+    spws_status_t st = rows_symbolic(plan, w.S, w.L, c, scratch_bytes, needed, false, nullptr, nullptr, reinterpret_cast<i64*>(x + w.R.rowptr), sc);
+    if (st != SPWS_OK || (st = rows_collect(plan)) != SPWS_OK) return st;
     plan->stats.rows = H.B.nnz;
     plan->stats.products = P;
     plan->outer_products = P;
@@ -1454,7 +1475,7 @@ spws_status_t spws_workspace_size_exact(spws_plan_t plan, const spws_tensor_t* A
     }
     if (reinterpret_cast<uintptr_t>(scratch) & 255) return SPWS_INVALID_ARGUMENT;
     if (scratch_bytes < L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
-    plan->symbolic_ok = false;                  // the tables of an earlier symbolic pass are overwritten
+    plan->symbolic_ok = plan->pending = false;  // the tables of an earlier symbolic pass are overwritten
     char* sc = static_cast<char*>(scratch);
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, L);
     c.prm.bm_arena_words = ~0ull >> 3;          // reserve without a limit: only the total is wanted
@@ -1472,10 +1493,31 @@ spws_status_t spws_workspace_size_exact(spws_plan_t plan, const spws_tensor_t* A
     return SPWS_OK;
 }
 
-// needed (may be null): receives the scratch bytes the passes use, or a size to try next when they could not be learnt
+// The second half of a symbolic pass over rows: waits for it and fills in the sizes.
+static spws_status_t symbolic_collect(spws_plan_t plan, spws_tensor_t* C, int64_t* sizes_out) {
+    const spws_status_t st = rows_collect(plan);
+    if (st != SPWS_OK) return st;
+    const DevCtl& hc = *plan->host_ctl;
+    if (plan->kind == 0) {
+        C->n[0] = C->dims[0];
+        C->n[1] = hc.nnz;
+        C->n[2] = 0;
+    } else {
+        C->n[0] = hc.kept[0];
+        C->n[1] = hc.kept[1];
+        C->n[2] = hc.nnz;
+    }
+    if (sizes_out) { sizes_out[0] = C->n[0]; sizes_out[1] = C->n[1]; sizes_out[2] = C->n[2]; }
+    plan->symbolic_ok = true;
+    return SPWS_OK;
+}
+
+// needed (may be null): receives the scratch bytes the passes use, or a size to try next when they could not be learnt;
+// begin_only (matrix and 3-tensor forms): return once the pass is enqueued
 static spws_status_t symbolic_any(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, const spws_tensor_t* D, spws_tensor_t* C,
-                                  void* scratch, size_t scratch_bytes, int64_t* sizes_out, size_t* needed) {
+                                  void* scratch, size_t scratch_bytes, int64_t* sizes_out, size_t* needed, bool begin_only = false) {
     if (!plan) return SPWS_INVALID_ARGUMENT;
+    plan->pending = false;
     if (needed) *needed = 0;
     if ((plan->kind == 5) != (D != nullptr)) return SPWS_INVALID_ARGUMENT;
     if (plan->kind >= 3) return higher_symbolic(plan, A, B, D, C, scratch, scratch_bytes, sizes_out, needed);
@@ -1506,21 +1548,10 @@ static spws_status_t symbolic_any(spws_plan_t plan, const spws_tensor_t* A, cons
     mark_start(plan, 0);
     i64* rowptr = (plan->kind == 0) ? LL(C->pos[1]) : reinterpret_cast<i64*>(sc + L.rowptr_raw);
     if ((st = rows_symbolic(plan, S, L, c, scratch_bytes, needed, !plan->opt.validate, plan->kind == 1 ? A : nullptr, C, rowptr, sc)) != SPWS_OK) return st;
-    const DevCtl& hc = *plan->host_ctl;
-    if (plan->kind == 0) {
-        C->n[0] = C->dims[0];
-        C->n[1] = hc.nnz;
-        C->n[2] = 0;
-    } else {
-        C->n[0] = hc.kept[0];
-        C->n[1] = hc.kept[1];
-        C->n[2] = hc.nnz;
-    }
-    if (sizes_out) { sizes_out[0] = C->n[0]; sizes_out[1] = C->n[1]; sizes_out[2] = C->n[2]; }
-    plan->symbolic_ok = true;
-    plan->m = S.m;
     plan->scratch = scratch;
-    return SPWS_OK;
+    plan->pending = true;
+    plan->numeric_behind = false;
+    return begin_only ? SPWS_OK : symbolic_collect(plan, C, sizes_out);
 }
 
 spws_status_t spws_symbolic(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, spws_tensor_t* C,
@@ -1534,12 +1565,30 @@ spws_status_t spws_symbolic_sized(spws_plan_t plan, const spws_tensor_t* A, cons
     return symbolic_any(plan, A, B, D, C, scratch, scratch_bytes, sizes_out, needed);
 }
 
+spws_status_t spws_symbolic_begin(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, spws_tensor_t* C, void* scratch,
+                                  size_t scratch_bytes, int64_t most, int64_t* sizes_out, size_t* needed, int64_t* upper) {
+    if (!plan || !needed || !upper || plan->kind > 1) return SPWS_INVALID_ARGUMENT;
+    *upper = 0;
+    const spws_status_t st = symbolic_any(plan, A, B, nullptr, C, scratch, scratch_bytes, nullptr, needed, true);
+    if (st != SPWS_OK) return st;
+    if (plan->upper == 0 || plan->upper > most) return symbolic_collect(plan, C, sizes_out);
+    *upper = plan->upper;
+    return SPWS_OK;
+}
+
+spws_status_t spws_symbolic_end(spws_plan_t plan, spws_tensor_t* C, int64_t* sizes_out) {
+    if (!plan || !C) return SPWS_INVALID_ARGUMENT;
+    if (!plan->pending) return SPWS_BAD_SEQUENCE;
+    return symbolic_collect(plan, C, sizes_out);
+}
+
 spws_status_t spws_numeric(spws_plan_t plan, const spws_tensor_t* A, const spws_tensor_t* B, spws_tensor_t* C,
                            void* scratch, size_t scratch_bytes) {
     if (!plan) return SPWS_INVALID_ARGUMENT;
     if (plan->kind == 5) return SPWS_INVALID_ARGUMENT;
     if (plan->kind >= 3) return higher_numeric(plan, A, B, nullptr, C, scratch, scratch_bytes);
-    if (!plan->symbolic_ok) return SPWS_BAD_SEQUENCE;
+    const bool behind = plan->pending && plan->upper > 0;        // enqueued behind a symbolic pass that is not waited for
+    if (!plan->symbolic_ok && !behind) return SPWS_BAD_SEQUENCE;
     Shapes S{};
     spws_status_t st = check_operands(plan, A, B, S);
     if (st != SPWS_OK) return st;
@@ -1547,8 +1596,10 @@ spws_status_t spws_numeric(spws_plan_t plan, const spws_tensor_t* A, const spws_
     if (scratch != plan->scratch || S.m != plan->m) return SPWS_BAD_SEQUENCE;
     if (plan->kind == 2) return outer_numeric(plan, S, C, scratch, scratch_bytes);
     const int last = plan->kind == 0 ? 1 : 2;
-    if (C->n[last] < plan->stats.nnz) return SPWS_OUTPUT_TOO_SMALL;
-    if (plan->stats.nnz > 0 && (!C->crd[last] || !C->val)) return SPWS_INVALID_ARGUMENT;
+    const int64_t entries = behind ? plan->upper : plan->stats.nnz;
+    if (C->n[last] < entries) return SPWS_OUTPUT_TOO_SMALL;
+    if (entries > 0 && (!C->crd[last] || !C->val)) return SPWS_INVALID_ARGUMENT;
+    plan->numeric_behind = behind;
     const Layout L = make_layout(plan, S.m, S.ncols, S.n_i, S.nnzB, S.k, S.nnzA);
     if (scratch_bytes < L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
     char* sc = static_cast<char*>(scratch);

@@ -1181,6 +1181,68 @@ def test_symbolic_sized_grows_the_scratch_and_remembers_no_operand(ctx, oracle_m
         assert np.array_equal(crd.cpu().numpy().astype(np.int64), oracle_mod.spmttkrp(T, M0, M1).crd)
 
 
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_numeric_pass_enqueued_behind_the_symbolic_one(ctx, oracle_mod, monkeypatch, dtype):
+    """A call whose rows need no dense workspace enqueues the numeric pass before the sizes are known, into arrays
+    as large as the product count: the same results as with the host in between, for both forms, and
+    with dense rows (no bound, hence no such call); the halves refuse a wrong order."""
+    import torch
+    from paper_2404_04541_b200 import api, binding
+    A, B = random_csr(300, 200, 0.01, 31, empty_row_frac=0.2), random_csr(200, 5000, 0.002, 32, empty_row_frac=0.2)
+    T, M = uniform_csf3((20, 30, 40), 900, 33), random_csr(40, 600, 0.02, 34)
+    for m in (A, B, T, M):
+        m.val = m.val.astype(dtype)
+    dA, dB, dT, dM = api.DeviceCSR.from_host(A), api.DeviceCSR.from_host(B), api.DeviceCSF3.from_host(T), api.DeviceCSR.from_host(M)
+    results = []
+    for limit in (api.BOUND_BYTES, 0):
+        monkeypatch.setattr(api, "BOUND_BYTES", limit)
+        C, stats = ctx.spgemm(dA, dB)
+        D, tstats = ctx.ttm(dT, dM)
+        assert stats["launches_symbolic"] > 0 and stats["launches_numeric"] > 0
+        assert stats["nnz"] == C.crd.numel() == C.val.numel() and tstats["nnz"] == D.val.numel()
+        results.append([x.cpu().numpy() for x in (C.pos, C.crd, C.val, D.pos0, D.crd0, D.pos1, D.crd1, D.pos2, D.crd2, D.val)])
+    assert all(np.array_equal(x, y) for x, y in zip(*results))
+    ref = oracle_mod.spgemm(A, B, threads=2)
+    assert_matches(results[0][:3], ref, dtype)
+    # the two halves by hand
+    plan = ctx.plan(api.EXPR_SPGEMM, (binding.SPWS_CSR,) * 3, dtype)
+    a, b = dA.arrays(), dB.arrays()
+    buf = torch.empty(64 << 20, dtype=torch.uint8, device="cuda")
+    ptr, room = ctx._aligned_ptr(buf), buf.numel() - 256
+    pos = torch.empty(A.nrows + 1, dtype=torch.int64, device="cuda")
+    c = binding.csr_arrays(A.nrows, B.ncols, pos, None, None)
+    with pytest.raises(binding.SpwsError) as e:
+        plan.symbolic_end(c)
+    assert e.value.status == binding.SPWS_BAD_SEQUENCE
+    assert not plan.symbolic_begin(a, b, c, ptr, 256, 1 << 30)[0]
+    products = int(ref.products.sum())
+    ok, need, upper = plan.symbolic_begin(a, b, c, ptr, room, products - 1)
+    assert ok and upper == 0 and c.n[1] == ref.nnz
+    with pytest.raises(binding.SpwsError) as e:
+        plan.symbolic_end(c)
+    assert e.value.status == binding.SPWS_BAD_SEQUENCE
+    ok, need, upper = plan.symbolic_begin(a, b, c, ptr, room, products)
+    assert ok and upper == products
+    c.crd[1] = torch.empty(upper, dtype=torch.int32, device="cuda")
+    c.val = torch.empty(upper, dtype=dA.val.dtype, device="cuda")
+    c.n[1] = upper - 1
+    with pytest.raises(binding.SpwsError) as e:
+        plan.numeric(a, b, c, ptr, room)
+    assert e.value.status == binding.SPWS_OUTPUT_TOO_SMALL
+    plan.symbolic_end(c)
+    assert c.n[1] == ref.nnz
+    plan.numeric(a, b, c, ptr, room)
+    plan.get_stats()
+    assert np.array_equal(c.crd[1][:ref.nnz].cpu().numpy(), ref.crd)
+    plan.close()
+    # rows of the dense workspace: the numeric pass has to wait for their counts
+    plan = ctx.plan(api.EXPR_SPGEMM, (binding.SPWS_CSR,) * 3, dtype, "dense")
+    c = binding.csr_arrays(A.nrows, B.ncols, pos, None, None)
+    ok, need, upper = plan.symbolic_begin(a, b, c, ptr, room, 1 << 30)
+    assert ok and upper == 0 and c.n[1] == ref.nnz
+    plan.close()
+
+
 # ------------------------------------------------------------------ boundary behaviour
 def test_error_statuses(ctx):
     import torch
