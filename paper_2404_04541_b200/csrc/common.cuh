@@ -337,11 +337,8 @@ __device__ __forceinline__ i64 lower_bound_crd(const int* __restrict__ crd, i64 
 }
 
 // lanes per A entry: the smallest power of two >= the mean B-row segment length
-__device__ __forceinline__ int pick_group_size(i64 ub, i64 entries, int parts) {
-    const float avg = (float)ub / fmaxf(1.0f, (float)entries * (float)parts);
-    int gs = 32;
-    while (gs > 1 && (float)(gs >> 1) >= avg) gs >>= 1;
-    return gs;
+__device__ __forceinline__ int pick_group_log(i64 ub, i64 entries) {
+    return (ub > entries) + (ub > 2 * entries) + (ub > 4 * entries) + (ub > 8 * entries) + (ub > 16 * entries);
 }
 
 // Products are formed as a rounded multiply followed by rounded adds (no contraction), so the

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __re
         const int nw = min((tab.jmax[row] - base) / 32 + 1, SCAN ? DW_SCAN_WORDS : DENSE_WARP_BM_WORDS);
         const unsigned span = (unsigned)nw * 32u;
         const i64 ps = A.pos[row], pe = A.pos[row + 1];
-        const int gs = pick_group_size(tab.ub[row], pe - ps, 1);
+        const int lg = pick_group_log(tab.ub[row], pe - ps), gs = 1 << lg;
         // the lane that sets a bit first counts the output; the lane that touches a word first
         // counts the word and flags it in the summary
         int cnt = 0, nzw = 0;
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __re
                 }
             }
         } else {
-            const int g = lane / gs, gl = lane % gs, ng = 32 / gs;
+            const int g = lane >> lg, gl = lane & (gs - 1), ng = 32 >> lg;
             for (i64 p = ps + g; p < pe; p += ng) {
                 const int k = __ldg(A.crd + p);
                 if ((unsigned)k >= (unsigned)B.nrows) continue;
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __re
 // What a block needs to know of a row, fetched by one thread while the block is busy with the row before.
 struct SymRow {
     i64 ps, pe, bm;
-    int row, base, nw, gs, batch;       // row < 0: no more rows
+    int row, base, nw, lg, batch;       // row < 0: no more rows
 };
 
 __global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __restrict__ ctl, int smem_words, Csr A, Csr B, RowTables tab,
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __
         R.bm = tab.bm_off[row];
         R.nw = min((tab.jmax[row] - base) / 32 + 1, smem_words);
         const i64 ub = tab.ub[row], entries = R.pe - R.ps;
-        R.gs = pick_group_size(ub, entries, 1);
+        R.lg = pick_group_log(ub, entries);
         R.batch = ub < 512 * entries ? 8 : 4;
         R.base = base;
         R.row = row;
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __
     for (int cur = 0;; cur ^= 1) {
         const SymRow& R = s_row[cur];
         if (R.row < 0) break;
-        const int base = R.base, nw = R.nw, gs = R.gs;
+        const int base = R.base, nw = R.nw, lg = R.lg, gs = 1 << lg;
         const unsigned span = (unsigned)nw * 32u;
         const unsigned base_w = (unsigned)base >> 5;                     // base is a multiple of 32
         const i64 ps = R.ps, pe = R.pe;
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __
                 }
             }
         } else {
-            const int g = tid / gs, gl = tid % gs, ng = DC_THREADS / gs;
+            const int g = tid >> lg, gl = tid & (gs - 1), ng = DC_THREADS >> lg;
             for (i64 p = ps + g; p < pe; p += ng) {
                 const int k = __ldg(A.crd + p);
                 if ((unsigned)k >= (unsigned)B.nrows) continue;
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
                 }
             }
         };
-        const int gs = pick_group_size(tab.ub[row], pe - ps, 1);
+        const int lg = pick_group_log(tab.ub[row], pe - ps), gs = 1 << lg;
         if (gs == 32) {
             // one A entry at a time, lanes across its B row: distinct columns, no atomics,
             // every output summed in loop order
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
             }
         } else {
             // short B rows: several A entries in flight, so slots can collide -> atomics
-            const int g = lane / gs, gl = lane % gs, ng = 32 / gs;
+            const int g = lane >> lg, gl = lane & (gs - 1), ng = 32 >> lg;
             for (i64 p = ps + g; p < pe; p += ng) {
                 const int k = __ldg(A.crd + p);
                 if ((unsigned)k >= (unsigned)B.nrows) continue;

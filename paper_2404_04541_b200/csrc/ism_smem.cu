@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(THREADS) ism_smem_kernel(const int* __restrict
 // products, this one about 2.7.  Bound by instruction issue.
 //   Insert : 32 A entries at a time; a group of lanes per entry (as many as the mean B row has
 //            entries) writes the products of its B row at their slots.
-//   Sort   : E = 2 .. 32 words per lane, the smallest network that holds the row.
+//   Sort   : E = 2, 3, 4, 6, 8, 12, 16, 24 or 32 words per lane, the smallest network that holds the row.
 //   Merge  : the sorted words go back to shared memory, the places of the run heads are packed, and
 //            one lane per run sums it in slot order.
 //   Of rows of more than 256 products the counting pass leaves the sorted words in scratch when there is room
@@ -162,7 +162,9 @@ __global__ void __launch_bounds__(THREADS) ism_smem_kernel(const int* __restrict
 // of 470, f64: 154 -> 210 and 494 -> 225 us.  Shorter rows gain nothing (fibres of about 110 products: numeric 104 us with
 // and without, count 82 -> 100 us), their sort is a small part of the work.
 // Stencil 41 x 37 x 53 (f32, 674 products a row): count 1714 -> 508 us, numeric 1905 -> 863 us against a CTA per
-// row; 59-product rows of the outer form (2e5 of them): 259 -> 125 us (hash set) and 439 -> 146 us.
+// row; 59-product rows of the outer form (2e5 of them): 259 -> 125 us (hash set) and 439 -> 146 us.  With sizes of
+// three times a power of two, long merges as loops and lane groups found by shifts: count 578 -> 384 us on
+// the stencil (now 370 us numeric), 210 -> 172 us on the rows of 470; 143-product rows (3e4): 44 -> 37 and 55 -> 50 us.
 // ---------------------------------------------------------------------------------------
 constexpr int IW_WARPS = 4;
 
@@ -173,46 +175,67 @@ __device__ __forceinline__ void sort_pair(P& a, P& b) {
     b = hi;
 }
 
-// Ascending bitonic sort of 32 * E words, element index = lane * E + x.  Every merge starts with the
-// mirrored comparison (i against i ^ (k - 1)), so all comparisons point the same way.
+// Ascending bitonic sort of 32 * E words, element index = lane * E + x, E = 2^a or 3 * 2^a.  Every merge starts with
+// the mirrored comparison (i against i ^ (k - 1) within its k), so all comparisons point the same way; with
+// a factor of three the merges end at triples, which three comparisons sort.
 template <typename P, int E>
 __device__ __forceinline__ void warp_sort(P (&w)[E]) {
+    constexpr int BASE = E % 3 == 0 ? 3 : 1;
     const int lane = threadIdx.x & 31;
+    auto triples = [&]() {
+        if (BASE == 3) {
 #pragma unroll
-    for (int k = 2; k <= 32 * E; k <<= 1) {
-        if (k <= E) {
+            for (int x = 0; x + 2 < E; x += 3) {
+                sort_pair(w[x], w[x + 1]);
+                sort_pair(w[x + 1], w[x + 2]);
+                sort_pair(w[x], w[x + 1]);
+            }
+        }
+    };
+    // the last stages of a merge: bitonic runs of up to E words inside a lane
+    auto lane_merge = [&](int k) {
+#pragma unroll
+        for (int j = k >> 1; j >= BASE; j >>= 1)
 #pragma unroll
             for (int x = 0; x < E; ++x)
-                if (!(x & (k >> 1))) sort_pair(w[x], w[x ^ (k - 1)]);
-        } else {
-            const int mask = k / E - 1;
-            const bool low = (lane & (k / (2 * E))) == 0;
+                if (x % (2 * j) < j) sort_pair(w[x], w[x + j]);
+        triples();
+    };
+    triples();
 #pragma unroll
-            for (int x = 0; x < (E + 1) / 2; ++x) {
-                const int y = E - 1 - x;
-                const P ox = __shfl_xor_sync(0xffffffffu, w[y], mask);
-                if (y != x) {
-                    const P oy = __shfl_xor_sync(0xffffffffu, w[x], mask);
-                    w[y] = low ? min(w[y], oy) : max(w[y], oy);
-                }
-                w[x] = low ? min(w[x], ox) : max(w[x], ox);
+    for (int k = 2 * BASE; k <= E; k <<= 1) {
+#pragma unroll
+        for (int x = 0; x < E; ++x)
+            if (x % k < k / 2) sort_pair(w[x], w[x / k * k + k - 1 - x % k]);
+        lane_merge(k / 2);
+    }
+    // merges across m lanes; the long ones stay loops: a kernel whose warps run several unrolled networks of
+    // 16 .. 32 words outgrows the instruction cache (counting 2e5 rows of 257 .. 1024 products: 300 us against 172; 8e4
+    // rows of 674: 456 against 384; of up to 8 words the unrolled ones are faster, 50 against 55 us)
+    constexpr int U = E > 8 ? 1 : 5;
+#pragma unroll U
+    for (int m = 2; m <= 32; m <<= 1) {
+        const bool low_half = (lane & (m >> 1)) == 0;
+#pragma unroll
+        for (int x = 0; x < (E + 1) / 2; ++x) {
+            const int y = E - 1 - x;
+            const P ox = __shfl_xor_sync(0xffffffffu, w[y], m - 1);
+            if (y != x) {
+                const P oy = __shfl_xor_sync(0xffffffffu, w[x], m - 1);
+                w[y] = low_half ? min(w[y], oy) : max(w[y], oy);
+            }
+            w[x] = low_half ? min(w[x], ox) : max(w[x], ox);
+        }
+#pragma unroll U
+        for (int d = m >> 2; d > 0; d >>= 1) {
+            const bool low = (lane & d) == 0;
+#pragma unroll
+            for (int x = 0; x < E; ++x) {
+                const P other = __shfl_xor_sync(0xffffffffu, w[x], d);
+                w[x] = low ? min(w[x], other) : max(w[x], other);
             }
         }
-#pragma unroll
-        for (int j = k >> 2; j > 0; j >>= 1) {
-            if (j >= E) {
-                const bool low = (lane & (j / E)) == 0;
-#pragma unroll
-                for (int x = 0; x < E; ++x) {
-                    const P other = __shfl_xor_sync(0xffffffffu, w[x], j / E);
-                    w[x] = low ? min(w[x], other) : max(w[x], other);
-                }
-            } else {
-#pragma unroll
-                for (int x = 0; x < E; ++x)
-                    if (!(x & j)) sort_pair(w[x], w[x + j]);
-            }
-        }
+        lane_merge(E);
     }
 }
 
@@ -220,7 +243,11 @@ __device__ __forceinline__ void warp_sort(P (&w)[E]) {
 __device__ __forceinline__ int padded(int i) { return i + (i >> 5); }
 
 // words each lane holds for a row of `total` words, and the lanes whose words are kept in scratch
-__device__ __forceinline__ int words_per_lane(int total) { return total <= 64 ? 2 : total <= 128 ? 4 : total <= 256 ? 8 : total <= 512 ? 16 : 32; }
+template <int CAP>
+__device__ __forceinline__ int words_per_lane(int total) {
+    if (CAP <= 256) return total <= 128 ? (total <= 64 ? 2 : total <= 96 ? 3 : 4) : total <= 192 ? 6 : 8;
+    return total <= 384 ? (total <= 256 ? 8 : 12) : total <= 512 ? 16 : total <= 768 ? 24 : 32;
+}
 __device__ __forceinline__ int order_lanes(int total, int e) { return ((total + e - 1) / e + 7) & ~7; }
 
 // Sorts the row's packed words and counts its distinct columns; numeric: leaves the sorted words in `packed`
@@ -269,8 +296,15 @@ __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int to
     return n;
 }
 
+// blocks an SM is to hold (the compiler would keep several of the networks below in registers at once)
 template <typename T, typename P, int CAP, bool NUMERIC>
-__global__ void __launch_bounds__(IW_WARPS * 32) ism_warp_kernel(const int* __restrict__ perm, DevCtl* __restrict__ ctl, int cls, int counter_slot,
+constexpr int iw_blocks() {
+    if (CAP <= 256) return sizeof(P) == 8 || (NUMERIC && sizeof(T) == 8) ? 9 : 12;
+    return sizeof(P) == 8 || (NUMERIC && sizeof(T) == 8) ? 3 : NUMERIC ? 5 : 6;
+}
+
+template <typename T, typename P, int CAP, bool NUMERIC>
+__global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>())) ism_warp_kernel(const int* __restrict__ perm, DevCtl* __restrict__ ctl, int cls, int counter_slot,
                                                                  Csr A, Csr B, const i64* __restrict__ ub, i64* __restrict__ order_off, char* order_arena,
                                                                  size_t order_bytes, int* __restrict__ cnt,
                                                                  const i64* __restrict__ rowptr, int* __restrict__ Ccrd, T* __restrict__ Cval) {
@@ -300,7 +334,7 @@ __global__ void __launch_bounds__(IW_WARPS * 32) ism_warp_kernel(const int* __re
             if (NUMERIC) {
                 at = order_off[row];
             } else if (lane == 0) {
-                const int e = words_per_lane((int)products);
+                const int e = words_per_lane<CAP>((int)products);
                 const u64 bytes = (u64)e * order_lanes((int)products, e) * sizeof(P);
                 at = (i64)atomicAdd(&ctl->order_used, bytes);
                 if ((u64)at + bytes > order_bytes) at = -1;
@@ -310,8 +344,8 @@ __global__ void __launch_bounds__(IW_WARPS * 32) ism_warp_kernel(const int* __re
         }
         const bool sorted = CAP > 256 && NUMERIC && order;
         const i64 ps = __ldg(A.pos + row), pe = __ldg(A.pos + row + 1);
-        const int gs = pick_group_size(products, pe - ps, 1);
-        const int g = lane / gs, gl = lane % gs, ng = 32 / gs;
+        const int lg = pick_group_log(products, pe - ps), gs = 1 << lg;
+        const int g = lane >> lg, gl = lane & (gs - 1), ng = 32 >> lg;
 
         // ---- Insert
         int total = 0;
@@ -361,15 +395,27 @@ __global__ void __launch_bounds__(IW_WARPS * 32) ism_warp_kernel(const int* __re
 
         // ---- Sort
         int distinct;
-        const int e = words_per_lane(total);
+        const int e = words_per_lane<CAP>(total);
         if (total != (int)products) order = nullptr;             // (a malformed B row)
         P* const keep = CAP > 256 ? order : nullptr;
         if (CAP > 256 && !NUMERIC && order_arena && lane == 0) order_off[row] = order ? (i64)(reinterpret_cast<char*>(order) - order_arena) : -1;
-        if (e == 2) distinct = sort_row<PK, P, 2, NUMERIC>(packed, heads, total, keep);
-        else if (e == 4) distinct = sort_row<PK, P, 4, NUMERIC>(packed, heads, total, keep);
-        else if (CAP <= 256 || e == 8) distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total, keep);
-        else if (e == 16) distinct = sort_row<PK, P, (CAP > 256 ? 16 : 8), NUMERIC>(packed, heads, total, keep);
-        else distinct = sort_row<PK, P, (CAP > 256 ? 32 : 8), NUMERIC>(packed, heads, total, keep);
+        if constexpr (CAP <= 256) {
+            switch (e) {
+                case 2: distinct = sort_row<PK, P, 2, NUMERIC>(packed, heads, total, keep); break;
+                case 3: distinct = sort_row<PK, P, 3, NUMERIC>(packed, heads, total, keep); break;
+                case 4: distinct = sort_row<PK, P, 4, NUMERIC>(packed, heads, total, keep); break;
+                case 6: distinct = sort_row<PK, P, 6, NUMERIC>(packed, heads, total, keep); break;
+                default: distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total, keep); break;
+            }
+        } else {
+            switch (e) {
+                case 8: distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total, keep); break;
+                case 12: distinct = sort_row<PK, P, 12, NUMERIC>(packed, heads, total, keep); break;
+                case 16: distinct = sort_row<PK, P, 16, NUMERIC>(packed, heads, total, keep); break;
+                case 24: distinct = sort_row<PK, P, 24, NUMERIC>(packed, heads, total, keep); break;
+                default: distinct = sort_row<PK, P, 32, NUMERIC>(packed, heads, total, keep); break;
+            }
+        }
 
         // ---- Merge
         if (!NUMERIC) {

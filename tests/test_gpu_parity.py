@@ -134,6 +134,16 @@ def test_ism_warp_rows_at_every_register_width(ctx, oracle_mod, ncols, dtype):
     check_spgemm(ctx, oracle_mod, A, B, "auto")
 
 
+@pytest.mark.parametrize("policy", ["ism", "auto"])
+@pytest.mark.parametrize("ncols", [2000, 1 << 25])
+def test_ism_warp_rows_of_three_times_a_power_of_two_words(ctx, oracle_mod, ncols, policy):
+    """Rows one product below, at and above the sizes where a lane holds 3, 6, 12 or 24 words, with 32- and
+    64-bit packed words, bit for bit the oracle's plain sum."""
+    targets = [65, 95, 96, 97, 129, 191, 192, 193, 257, 383, 384, 385, 513, 767, 768, 769, 1024]
+    A, B = _rows_with_products(targets, ncols, 14, np.float64)
+    check_spgemm(ctx, oracle_mod, A, B, policy, exact_values=policy == "ism")
+
+
 @pytest.mark.parametrize("dtype", [np.float64, np.float32])
 @pytest.mark.parametrize("ncols", [2000, 1 << 22])
 def test_sorted_words_kept_for_the_numeric_pass(ctx, oracle_mod, ncols, dtype):
