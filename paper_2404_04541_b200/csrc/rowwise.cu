@@ -222,12 +222,14 @@ __global__ void __launch_bounds__(OT) rw_fibre_rows_kernel(Csf3Dev B, Csr C, Csr
     }
 }
 
-// Coordinates of a coordinate-form result from its row pointer, row labels and columns.  A block takes a
-// tile of RC_TILE consecutive entries: the first entry of every row in the tile leaves the row's
+// Coordinates of a coordinate-form result from its row pointer, row labels and columns.  A block takes a run of
+// tiles of RC_TILE consecutive entries: the first entry of every row in the tile leaves the row's
 // coordinates in shared memory, a running maximum hands each entry the place of its row's first one,
-// and a thread writes the coordinates of its eight consecutive entries.  Bound by HBM.
+// and a thread writes the coordinates of its eight consecutive entries.  The rows of a tile are read 256 at a time from where
+// the tile before ended.  Bound by HBM and the four barriers of a tile.
 // 43e6 entries of three coordinates: 333 us for three arrays with a search per entry and 883 us to interleave
-// them, 274 us for the interleaved coordinates (516 MB out, 172 MB in).
+// them; interleaved 276 us with two searches per tile, 198 us without them and 165 us with whole lines per store
+// (516 MB out, 172 MB in).
 constexpr int RC_ITEMS = 8;
 constexpr int RC_TILE = OT * RC_ITEMS;
 
@@ -236,31 +238,49 @@ __global__ void __launch_bounds__(OT) rw_coords_kernel(const i64* __restrict__ r
                                                        const int* __restrict__ cols, int* __restrict__ o0, int* __restrict__ o1,
                                                        int* __restrict__ o2) {
     __shared__ int s_c0[RC_TILE], s_c1[ORDER == 3 ? RC_TILE : 1];
-    __shared__ __align__(16) int s_head[RC_TILE];       // entry i: i when a row starts there, else 0
-    __shared__ int s_lo, s_hi, s_warp[OT / 32];
+    __shared__ __align__(16) unsigned short s_head[RC_TILE];    // entry i: i when a row starts there, else 0; zero between tiles
+    __shared__ __align__(16) int s_out[INTERLEAVED ? ORDER * RC_TILE : 4];
+    __shared__ int s_lo, s_warp[OT / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool vec = (((u64)o0 | (INTERLEAVED ? 0 : (u64)o1 | (u64)o2)) & 15) == 0;      // 16-byte stores
-    for (i64 t0 = (i64)blockIdx.x * RC_TILE; t0 < nnz; t0 += (i64)gridDim.x * RC_TILE) {
-        __syncthreads();
-        const i64 t1 = min(nnz, t0 + RC_TILE);
-        if (tid == 0) s_lo = owner_row(rowptr, 0, (int)m, t0);
-        if (tid == 32) s_hi = owner_row(rowptr, 0, (int)m, t1 - 1) + 1;
-        for (int i = tid; i < RC_TILE; i += OT) s_head[i] = 0;
-        __syncthreads();
-        const int lo = s_lo, hi = s_hi;
-        for (int r = lo + tid; r < hi; r += OT) {
-            const i64 a = __ldg(rowptr + r), b = __ldg(rowptr + r + 1);
-            if (a == b) continue;
-            const int i = r == lo ? 0 : (int)(a - t0);  // (the first row may have begun before the tile)
-            const u64 key = __ldg(row_key + r);
-            s_c0[i] = ORDER == 3 ? (int)(key / d) : (int)key;
-            if (ORDER == 3) s_c1[i] = (int)(key % d);
-            s_head[i] = i;
+    const i64 tiles = (nnz + RC_TILE - 1) / RC_TILE;
+    const i64 first = tiles * blockIdx.x / gridDim.x, last = tiles * (blockIdx.x + 1) / gridDim.x;
+    for (int i = tid; i < RC_TILE; i += OT) s_head[i] = 0;
+    if (tid == 0 && first < last) s_lo = owner_row(rowptr, 0, (int)m, first * RC_TILE);
+    for (i64 tile = first; tile < last; ++tile) {
+        const i64 t0 = tile * RC_TILE, t1 = min(nnz, t0 + RC_TILE);
+        const int i0 = tid * RC_ITEMS;
+        const bool whole = vec && t0 + RC_TILE <= nnz;
+        int col[RC_ITEMS];
+        if (whole) {
+            *reinterpret_cast<int4*>(col) = __ldg(reinterpret_cast<const int4*>(cols + t0 + i0));
+            *reinterpret_cast<int4*>(col + 4) = __ldg(reinterpret_cast<const int4*>(cols + t0 + i0) + 1);
         }
         __syncthreads();
+        const int lo = s_lo;                            // a row that starts at or before t0, none but empty ones between
+        __syncthreads();
+        for (i64 r0 = lo;; r0 += OT) {
+            const i64 r = r0 + tid;
+            bool inside = false;
+            if (r < m) {
+                const i64 a = __ldg(rowptr + r), b = __ldg(rowptr + r + 1);
+                inside = a < t1;
+                if (inside && b > t0 && b > a) {
+                    const int i = (int)max(a - t0, (i64)0);     // (the first row may have begun before the tile)
+                    const u64 key = __ldg(row_key + r);
+                    s_c0[i] = ORDER == 3 ? (int)(key / d) : (int)key;
+                    if (ORDER == 3) s_c1[i] = (int)(key % d);
+                    s_head[i] = (unsigned short)i;
+                }
+                if (inside && b >= t1) s_lo = (int)r;           // the next tile starts here
+            }
+            if (!__syncthreads_or(tid == OT - 1 && inside)) break;
+        }
         int h[RC_ITEMS];
-        const int4 ha = reinterpret_cast<const int4*>(s_head)[2 * tid], hb = reinterpret_cast<const int4*>(s_head)[2 * tid + 1];
-        h[0] = ha.x; h[1] = ha.y; h[2] = ha.z; h[3] = ha.w; h[4] = hb.x; h[5] = hb.y; h[6] = hb.z; h[7] = hb.w;
+        const uint4 hv = reinterpret_cast<const uint4*>(s_head)[tid];
+        reinterpret_cast<uint4*>(s_head)[tid] = make_uint4(0, 0, 0, 0);
+        h[0] = hv.x & 0xffff; h[1] = hv.x >> 16; h[2] = hv.y & 0xffff; h[3] = hv.y >> 16;
+        h[4] = hv.z & 0xffff; h[5] = hv.z >> 16; h[6] = hv.w & 0xffff; h[7] = hv.w >> 16;
 #pragma unroll
         for (int x = 1; x < RC_ITEMS; ++x) h[x] = max(h[x], h[x - 1]);
         int incl = h[RC_ITEMS - 1];
@@ -271,11 +291,8 @@ __global__ void __launch_bounds__(OT) rw_coords_kernel(const i64* __restrict__ r
         if (lane == 0) before = 0;
         __syncthreads();
         for (int w = 0; w < warp; ++w) before = max(before, s_warp[w]);
-        const int i0 = tid * RC_ITEMS;
-        if (vec && t0 + i0 + RC_ITEMS <= t1) {
-            int out[RC_ITEMS * ORDER], col[RC_ITEMS];       // entry by entry, or array by array
-            *reinterpret_cast<int4*>(col) = __ldg(reinterpret_cast<const int4*>(cols + t0 + i0));
-            *reinterpret_cast<int4*>(col + 4) = __ldg(reinterpret_cast<const int4*>(cols + t0 + i0) + 1);
+        if (whole) {
+            int out[RC_ITEMS * ORDER];                      // entry by entry, or array by array
 #pragma unroll
             for (int x = 0; x < RC_ITEMS; ++x) {
                 const int at = max(h[x], before);
@@ -283,10 +300,20 @@ __global__ void __launch_bounds__(OT) rw_coords_kernel(const i64* __restrict__ r
                 if (ORDER == 3) out[INTERLEAVED ? x * ORDER + 1 : x + RC_ITEMS] = s_c1[at];
                 out[INTERLEAVED ? x * ORDER + ORDER - 1 : x + (ORDER - 1) * RC_ITEMS] = col[x];
             }
+            constexpr int QUADS = RC_ITEMS * ORDER / 4;
+            if (INTERLEAVED) {                              // through shared memory, so that a warp stores whole lines
 #pragma unroll
-            for (int y = 0; y < RC_ITEMS * ORDER / 4; ++y) {
-                int* const to = INTERLEAVED ? o0 + (t0 + i0) * ORDER + 4 * y : (y < 2 ? o0 : y < 4 ? o1 : o2) + t0 + i0 + 4 * (y & 1);
-                *reinterpret_cast<int4*>(to) = make_int4(out[4 * y], out[4 * y + 1], out[4 * y + 2], out[4 * y + 3]);
+                for (int y = 0; y < QUADS; ++y)
+                    reinterpret_cast<int4*>(s_out)[tid * QUADS + y] = make_int4(out[4 * y], out[4 * y + 1], out[4 * y + 2], out[4 * y + 3]);
+                __syncwarp();
+                int4* const to = reinterpret_cast<int4*>(o0 + t0 * ORDER) + warp * (32 * QUADS);
+#pragma unroll
+                for (int y = 0; y < QUADS; ++y) to[y * 32 + lane] = reinterpret_cast<const int4*>(s_out)[warp * (32 * QUADS) + y * 32 + lane];
+                __syncwarp();
+            } else {
+#pragma unroll
+                for (int y = 0; y < QUADS; ++y)
+                    *reinterpret_cast<int4*>((y < 2 ? o0 : y < 4 ? o1 : o2) + t0 + i0 + 4 * (y & 1)) = make_int4(out[4 * y], out[4 * y + 1], out[4 * y + 2], out[4 * y + 3]);
             }
         } else {
 #pragma unroll
