@@ -58,6 +58,21 @@ struct spws_handle_s {
     cudaStream_t stream = nullptr;
     int device = 0;
     int sm_count = 0;
+    // streams on which independent workspaces run beside the caller's (all or nothing: joined[1] is made last)
+    cudaStream_t side[2] = {};
+    cudaEvent_t forked = nullptr, joined[2] = {};
+    void make_sides() {
+        for (cudaStream_t& t : side)
+            if (cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); t = nullptr; return; }
+        for (cudaEvent_t* e : {&forked, &joined[0], &joined[1]})
+            if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); *e = nullptr; return; }
+    }
+    ~spws_handle_s() {
+        for (cudaEvent_t e : {forked, joined[0], joined[1]})
+            if (e) cudaEventDestroy(e);
+        for (cudaStream_t t : side)
+            if (t) cudaStreamDestroy(t);
+    }
 };
 
 struct spws_plan_s {
@@ -80,6 +95,7 @@ struct spws_plan_s {
     int64_t m = 0;
     void* scratch = nullptr;
     int max_span_words = 0;     // widest dense bitmap of the last symbolic pass
+    int64_t sparse_products = 0;                // products of the rows its sparse workspaces take
     size_t order_off = 0, order_bytes = 0;      // where it left the sorted words of mid-size rows in the scratch (0 bytes: nowhere)
     int n_warp[N_WARP_LISTS] = {};          // rows on the warp numeric kernel's lists ...
     int max_warp_cnt[N_WARP_LISTS] = {};    // ... and their largest output counts
@@ -486,6 +502,49 @@ size_t rows_guess(const spws_plan_s* plan, const Layout& L, int64_t m, int64_t n
     return L.fixed_end + std::min(rest_reserve(plan, m, ncols), std::max(L.fixed_end, (size_t)16 << 20));
 }
 
+// The workspaces of a pass are independent of one another: the sparse ones (from FORK_PRODUCTS products on, with the
+// dense rows otherwise), the dense one by warps and the rest go to a stream each, forked from the caller's and
+// joined to it, when at least two of the three have work.  Kernels that do not fill the device then run side by side,
+// and the last rows of one beside the first of the next: power law on 2484 / 16381 vertices 353 -> 265 / 795 -> 676 us a
+// call, fibres of 110 products 503 -> 481 us.  The events cost the host about 5 us a pass, which a handful of
+// sparse rows does not repay (7 x 7 x 8 stencil 121 us without, 131 us with).  Not while kernel groups are being timed.
+constexpr int64_t FORK_PRODUCTS = 1 << 15;
+class Fork {
+    LaunchCtx& c_;
+    spws_handle_s* h_;
+    cudaStream_t main_;
+    bool on_ = false, used_[2] = {};
+    int sparse_ = 2;
+
+public:
+    Fork(spws_plan_s* p, LaunchCtx& c, bool warp, bool rest) : c_(c), h_(p->h), main_(c.stream) {
+        const bool sparse = p->sparse_products >= FORK_PRODUCTS;
+        sparse_ = sparse ? 0 : warp ? 1 : 2;
+        on_ = (int)sparse + (int)warp + (int)rest >= 2 && !p->profiling && h_->joined[1] && cudaEventRecord(h_->forked, main_) == cudaSuccess;
+    }
+    ~Fork() { join(); }
+    // the kernels launched next belong to this group: 0 sparse, 1 dense by warps, 2 the rest (on the caller's stream)
+    void group(int g) {
+        c_.stream = main_;
+        if (g == 0) g = sparse_;
+        if (!on_ || g == 2) return;
+        if (!used_[g] && cudaStreamWaitEvent(h_->side[g], h_->forked, 0) != cudaSuccess) return;
+        used_[g] = true;
+        c_.stream = h_->side[g];
+    }
+    cudaError_t join() {
+        c_.stream = main_;
+        cudaError_t e = cudaSuccess;
+        for (int g = 0; g < 2; ++g)
+            if (used_[g]) {
+                used_[g] = false;
+                if (e == cudaSuccess) e = cudaEventRecord(h_->joined[g], h_->side[g]);
+                if (e == cudaSuccess) e = cudaStreamWaitEvent(main_, h_->joined[g], 0);
+            }
+        return e;
+    }
+};
+
 // Hands the arena of sorted words to the kernels and takes it from what follows the bitmaps.
 void use_order(const spws_plan_s* plan, LaunchCtx& c, char* sc, size_t scratch_bytes) {
     if (plan->order_bytes == 0 || plan->order_off + plan->order_bytes > scratch_bytes) return;
@@ -536,11 +595,16 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     i64 hcount[NCLASS];
     for (int k = 0; k < NCLASS; ++k) hcount[k] = hc.class_count[k];
     const i64 products = hc.products;
+    plan->sparse_products = 0;
+    for (int k : {CLS_COPY, CLS_ISM_REG8, CLS_ISM_REG16, CLS_ISM_REG, CLS_ISM_SMEM_S, CLS_ISM_SMEM}) plan->sparse_products += hc.class_products[k];
     const bool any_dense = hcount[CLS_DENSE_WARP] + hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0;
     plan->max_ub_smem = hc.max_ub_smem;
     c.max_ub_smem = plan->max_ub_smem;
     // a3: exact count per row through the workspace of its class
     if (S.m > 0) {
+        const bool dense_cta = hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0;
+        Fork fork(plan, c, hcount[CLS_DENSE_WARP] > 0, dense_cta || hcount[CLS_ISM_GLOBAL] > 0);
+        fork.group(0);
         if (hcount[CLS_ISM_REG8] + hcount[CLS_ISM_REG16] + hcount[CLS_ISM_REG] > 0) {
             CUDA_TRY(launch_ism_reg(c, false, hcount, S.A, S.B, rowptr, nullptr, nullptr));
             mark(plan, SPWS_T_SYM_ISM_REG);
@@ -553,11 +617,13 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
             CUDA_TRY(launch_ism_smem(c, false, CLS_ISM_SMEM, (int)hcount[CLS_ISM_SMEM], S.A, S.B, rowptr, nullptr, nullptr));
             mark(plan, SPWS_T_SYM_ISM_SMEM);
         }
+        fork.group(1);
         if (hcount[CLS_DENSE_WARP] > 0) {
             CUDA_TRY(launch_dense_sym_warp(c, hc.max_span_words, S.A, S.B));
             mark(plan, SPWS_T_SYM_DENSE_WARP);
         }
-        if (hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0) {
+        fork.group(2);
+        if (dense_cta) {
             CUDA_TRY(launch_bw_build(c, S.B));
             CUDA_TRY(launch_dense_sym_cta(c, S.A, S.B));
             mark(plan, SPWS_T_SYM_DENSE_CTA);
@@ -571,6 +637,7 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
                 CUDA_TRY(launch_hash(c, false, cls, (int)hcount[cls], S.A, S.B, rowptr, nullptr, nullptr));
                 mark(plan, SPWS_T_SYM_HASH);
             }
+        CUDA_TRY(fork.join());
     }
     // a4: row pointer, numeric routing and (3-tensor form) C's upper levels, rebuilt from the fibres that
     // produced an output
@@ -635,6 +702,8 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, cha
     c.max_ub_smem = plan->max_ub_smem;
     const spws_stats_t& s = plan->stats;
     const int64_t* bins = plan->bin_rows;
+    Fork fork(plan, c, s.dense_warp_rows > 0, s.dense_units > 0 || bins[CLS_ISM_GLOBAL] > 0);
+    fork.group(0);
     if (bins[CLS_COPY] + bins[CLS_ISM_REG8] + bins[CLS_ISM_REG16] + bins[CLS_ISM_REG] > 0) {
         CUDA_TRY(launch_ism_reg(c, true, LL(bins), S.A, S.B, rowptr, crd, val));
         mark(plan, SPWS_T_NUM_ISM_REG);
@@ -647,10 +716,12 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, cha
         CUDA_TRY(launch_ism_smem(c, true, CLS_ISM_SMEM, (int)bins[CLS_ISM_SMEM], S.A, S.B, rowptr, crd, val));
         mark(plan, SPWS_T_NUM_ISM_SMEM);
     }
+    fork.group(1);
     if (s.dense_warp_rows > 0) {
         CUDA_TRY(launch_dense_num_warp(c, plan->n_warp, plan->max_warp_cnt, (int)S.m, plan->max_span_words, S.A, S.B, rowptr, crd, val));
         mark(plan, SPWS_T_NUM_DENSE_WARP);
     }
+    fork.group(2);
     if (s.dense_units > 0) {
         CUDA_TRY(launch_dense_num_cta(c, 0, (int)s.dense_units, plan->max_span_words, s.products, S.A, S.B, rowptr, crd, val));
         mark(plan, SPWS_T_NUM_DENSE_EMIT);
@@ -666,6 +737,7 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, cha
             CUDA_TRY(launch_hash(c, true, cls, (int)bins[cls], S.A, S.B, rowptr, crd, val));
             mark(plan, SPWS_T_NUM_HASH);
         }
+    CUDA_TRY(fork.join());
     plan->stats.launches_numeric = c.launches;
     return SPWS_OK;
 }
@@ -1324,6 +1396,7 @@ spws_status_t spws_create(spws_handle_t* handle) {
         delete h;
         return SPWS_CUDA_ERROR;
     }
+    h->make_sides();
     *handle = h;
     return SPWS_OK;
 }
