@@ -174,8 +174,10 @@ __device__ __forceinline__ void copy_rows(const int* __restrict__ rows, const un
 // classes run side by side and no class waits for the last rows of another (four launches before).
 struct RegBlocks { int end[4]; };       // blocks of the copied rows, of 8, 16 and 32 lanes per row: ends of the ranges
 
+// (six blocks per SM, but five for double values, which spill at 40 registers: 2e6 fibres, count 25.5 -> 22.6 us; 65536
+// rows of 16 products, f32, 19.3 + 27.2 -> 17.7 + 25.4 us)
 template <typename T, bool NUMERIC>
-__global__ void __launch_bounds__(256, 5) ism_reg_kernel(const int* __restrict__ perm, const unsigned char* __restrict__ cls, const DevCtl* __restrict__ ctl,
+__global__ void __launch_bounds__(256, NUMERIC && sizeof(T) == 8 ? 5 : 6) ism_reg_kernel(const int* __restrict__ perm, const unsigned char* __restrict__ cls, const DevCtl* __restrict__ ctl,
                                                       RegBlocks g, Csr A, Csr B,
                                                       const int* __restrict__ jmin, int* __restrict__ cnt, const i64* __restrict__ rowptr,
                                                       int* __restrict__ Ccrd, T* __restrict__ Cval) {
