@@ -200,13 +200,13 @@ __global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __re
 // ---------------------------------------------------------------------------------------
 // symbolic, CTA per row (hub rows first: classes HUB and CTA are adjacent in perm)
 // Bound by latency: chains of loads and the barriers of short rows.  With entries dealt out in turn, eight barriers per row
-// and a chain of four loads per entry, power law on 2^18 / 60000 / 16381 vertices: 3149 / 726 / 193 us; now 2915 /
+// and a chain of four loads per entry, power law on 2^18 / 60000 / 16381 vertices: 3149 / 726 / 193 us; now 2815 /
 // 622 / 183 us.
 // ---------------------------------------------------------------------------------------
 // What a block needs to know of a row, fetched by one thread while the block is busy with the row before.
 struct SymRow {
     i64 ps, pe, bm;
-    int row, base, nw, lg, batch;       // row < 0: no more rows
+    int row, base, nw, lg, batch, whole;       // row < 0: no more rows
 };
 
 __global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __restrict__ ctl, int smem_words, Csr A, Csr B, RowTables tab,
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __
     unsigned* bm = reinterpret_cast<unsigned*>(smem_raw);                 // smem_words, clear between rows
     int* chunk = reinterpret_cast<int*>(bm + smem_words);                  // smem_words / 32
     __shared__ SymRow s_row[2];
-    __shared__ int s_entry[2];                                              // A entries handed out
+    __shared__ int s_entry[2];                                              // batches of A entries handed out
     if (ctl->status != 0) return;
     int off, n_hub, o6, n_cta;
     class_range(ctl, CLS_DENSE_HUB, off, n_hub);
@@ -236,6 +236,8 @@ __global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __
         const i64 ub = tab.ub[row], entries = R.pe - R.ps;
         R.lg = pick_group_log(ub, entries);
         R.batch = ub < 512 * entries ? 8 : 4;
+        R.whole = (int)(entries * 3 / 4) / R.batch;         // batches of that size; pairs for the last quarter, so that
+                                                            // the warps finish together (2915 -> 2815 us on 2^18 vertices)
         R.base = base;
         R.row = row;
     };
@@ -291,15 +293,17 @@ __global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __
             }
         };
         if (gs == 32) {
-            const int batch = R.batch;
+            const int full = R.batch, whole = R.whole;
             // warps pull a batch of entries at a time: the chain of loads that leads to a B row is walked for all of
             // them side by side, and no warp waits for one that met the longest B rows.  Eight entries, four
             // when their B rows are long (whole batches weigh more than the chain then): power law on 2^18
             // vertices 3350 us with eight, 2870 with four, 2900 with two; on 60000 620, 670 and 750 us
             for (;;) {
                 int at = 0;
-                if (lane == 0) at = atomicAdd(&s_entry[cur], batch);
+                if (lane == 0) at = atomicAdd(&s_entry[cur], 1);
                 at = __shfl_sync(0xffffffffu, at, 0);
+                const int batch = at < whole ? full : 2;
+                at = at < whole ? at * full : whole * full + (at - whole) * 2;
                 if (at >= pe - ps) break;
                 i64 my_qs = 0;
                 int my_len = 0, my_np = 0;
