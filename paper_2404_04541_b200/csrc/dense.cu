@@ -937,13 +937,21 @@ static cudaError_t num_warp_t(const LaunchCtx& c, const int* n, const int* max_c
     const int* const rows[N_WARP_LISTS] = {c.tab.warp_rows, c.tab.warp_rows + m - 1};
     for (int list = N_WARP_LISTS - 1; list >= 0; --list) {          // the longest rows first
         if (n[list] == 0) continue;
-        // values reserved per warp; smaller CTAs for larger accumulators, so that the SM's shared memory is used up
+        // values reserved per warp; of 256, 128 and 64 threads the CTA size that keeps most warps on an SM, since
+        // whole CTAs must fit its shared memory (64^3 stencil, f64, 6 KB a warp: 32 warps in CTAs of 256, 36 in CTAs
+        // of 128: 690 -> 643 us)
         const int accw = (max_cnt[list] + 31) & ~31;
-        const int threads = DW_THREADS >> list, warps = threads / 32;
-        const size_t smem = (size_t)warps * (sizeof(T) * (size_t)accw + 8 * (size_t)bmw + 16 * 32);
-        int per_sm = 0;
-        cudaError_t e;
-        if ((e = resident_blocks((const void*)k, threads, smem, &per_sm)) != cudaSuccess) return e;
+        const size_t per_warp = sizeof(T) * (size_t)accw + 8 * (size_t)bmw + 16 * 32;
+        int threads = 0, per_sm = 0;
+        for (int t = DW_THREADS; t >= 64; t >>= 1) {
+            int fit = 0;
+            const cudaError_t e = resident_blocks((const void*)k, t, per_warp * (t / 32), &fit);
+            if (e != cudaSuccess) return e;
+            if (fit * t > per_sm * threads) { threads = t; per_sm = fit; }
+        }
+        if (threads == 0) return cudaErrorInvalidConfiguration;
+        const int warps = threads / 32;
+        const size_t smem = per_warp * warps;
         k<<<persistent_grid(c, per_sm, ((i64)n[list] + warps - 1) / warps), threads, smem, c.stream>>>(
             c.ctl, rows[list], list == 0 ? 1 : -1, n[list], (CEIL ? CEIL_WARP_SLOT : WARP_SLOT) + list, bmw, accw, A, B, c.tab, rowptr, Ccrd, (T*)Cval,
             chk_idx, chk_val);
