@@ -371,18 +371,19 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (ctl->status != 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-    // per warp: a table of bmw bitmap words, each with the number of outputs before it (one load
-    // ranks a column), and accw values (sized from the widest / largest row of this launch)
-    uint2* tbl = reinterpret_cast<uint2*>(smem_raw) + warp * bmw;
-    T* acc = reinterpret_cast<T*>(reinterpret_cast<uint2*>(smem_raw) + warps * bmw) + warp * accw;
+    // per warp: bmw bitmap words, the number of outputs before each (16 bits: 629 us against 643 with both in
+    // eight bytes, which keep fewer warps on an SM), and accw values (sized from the widest / largest row of this launch)
+    unsigned* bits = reinterpret_cast<unsigned*>(smem_raw) + warp * bmw;
+    unsigned short* rank = reinterpret_cast<unsigned short*>(reinterpret_cast<unsigned*>(smem_raw) + warps * bmw) + warp * bmw;
+    T* acc = reinterpret_cast<T*>(smem_raw + 6 * warps * bmw) + warp * accw;
     // descriptors of 32 A entries: (start of the B row << 16) | its length, and the A value; one broadcast load
     // per entry where shuffles took five slots of the same pipe (bmw and accw are multiples of 32: aligned)
     struct __align__(16) Desc { u64 row; T a; };
-    Desc* desc = reinterpret_cast<Desc*>(reinterpret_cast<T*>(reinterpret_cast<uint2*>(smem_raw) + warps * bmw) + warps * accw) + warp * 32;
+    Desc* desc = reinterpret_cast<Desc*>(reinterpret_cast<T*>(smem_raw + 6 * warps * bmw) + warps * accw) + warp * 32;
     const T* __restrict__ Aval = (const T*)A.val;
     const T* __restrict__ Bval = (const T*)B.val;
     if (!CEIL)
-        for (int w = lane; w < bmw; w += 32) tbl[w] = make_uint2(0u, 0u);   // every row leaves its table clear
+        for (int w = lane; w < bmw; w += 32) bits[w] = 0u;              // every row leaves its bitmap clear
     __syncwarp();
     u64 my_idx = 0;
     double my_val = 0.0;
@@ -413,7 +414,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
                 const uint2 e = (i < nzw) ? src2[i] : make_uint2(0u, 0u);
                 const int c = __popc(e.x);
                 const int incl = warp_incl_scan(c);
-                if (i < nzw && e.y < (unsigned)nw) tbl[e.y] = make_uint2(e.x, (unsigned)(carry + incl - c));
+                if (i < nzw && e.y < (unsigned)nw) { bits[e.y] = e.x; rank[e.y] = (unsigned short)(carry + incl - c); }
                 carry += __shfl_sync(0xffffffffu, incl, 31);
             }
         } else {
@@ -423,7 +424,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
                 const unsigned word = (w < nw) ? src[w] : 0u;
                 const int c = __popc(word);
                 const int incl = warp_incl_scan(c);
-                if (w < nw) tbl[w] = make_uint2(word, src[nw + (w0 >> 5)] + (unsigned)(incl - c));
+                if (w < nw) { bits[w] = word; rank[w] = (unsigned short)(src[nw + (w0 >> 5)] + (unsigned)(incl - c)); }
             }
         }
         if (!CEIL)
@@ -435,8 +436,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
             if (CEIL) {
                 if (rel != 0xffffffffu) { my_idx += (u64)(rel + (unsigned)base); my_val += (double)prod; }
             } else if (rel < span) {
-                const uint2 t = tbl[rel >> 5];
-                const int at_ = (int)t.y + __popc(t.x & ((1u << (rel & 31)) - 1u));
+                const int at_ = (int)rank[rel >> 5] + __popc(bits[rel >> 5] & ((1u << (rel & 31)) - 1u));
                 if (at_ < accw) {
                     if (shared_slot) atomicAdd(&acc[at_], prod);
                     else acc[at_] = add_rn(acc[at_], prod);
@@ -508,8 +508,8 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
                 const uint2 e = src2[i];
                 if (e.y >= (unsigned)nw) continue;
                 unsigned word = e.x;
-                i64 o = out0 + tbl[e.y].y;
-                tbl[e.y] = make_uint2(0u, 0u);
+                i64 o = out0 + rank[e.y];
+                bits[e.y] = 0u;
                 while (word) {
                     const int b = __ffs(word) - 1;
                     word &= word - 1;
@@ -518,10 +518,9 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
             }
         } else {
             for (int w = lane; w < nw; w += 32) {
-                const uint2 t = tbl[w];
-                unsigned word = t.x;
-                i64 o = out0 + t.y;
-                tbl[w] = make_uint2(0u, 0u);
+                unsigned word = bits[w];
+                i64 o = out0 + rank[w];
+                bits[w] = 0u;
                 while (word) {
                     const int b = __ffs(word) - 1;
                     word &= word - 1;
@@ -941,7 +940,7 @@ static cudaError_t num_warp_t(const LaunchCtx& c, const int* n, const int* max_c
         // whole CTAs must fit its shared memory (64^3 stencil, f64, 6 KB a warp: 32 warps in CTAs of 256, 36 in CTAs
         // of 128: 690 -> 643 us)
         const int accw = (max_cnt[list] + 31) & ~31;
-        const size_t per_warp = sizeof(T) * (size_t)accw + 8 * (size_t)bmw + 16 * 32;
+        const size_t per_warp = sizeof(T) * (size_t)accw + 6 * (size_t)bmw + 16 * 32;
         int threads = 0, per_sm = 0;
         for (int t = DW_THREADS; t >= 64; t >>= 1) {
             int fit = 0;
