@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(THREADS) ism_smem_kernel(const int* __restrict
 // Stencil 41 x 37 x 53 (f32, 674 products a row): count 1714 -> 508 us, numeric 1905 -> 863 us against a CTA per
 // row; 59-product rows of the outer form (2e5 of them): 259 -> 125 us (hash set) and 439 -> 146 us.  With sizes of
 // three times a power of two, long merges as loops and lane groups found by shifts: count 578 -> 384 us on
-// the stencil (now 370 us numeric), 210 -> 172 us on the rows of 470; 143-product rows (3e4): 44 -> 37 and 55 -> 50 us.
+// the stencil (370 us numeric, 312 since), 210 -> 172 us on the rows of 470; 143-product rows (3e4): 44 -> 37 and 55 -> 50 us.
 // ---------------------------------------------------------------------------------------
 constexpr int IW_WARPS = 4;
 
@@ -244,7 +244,7 @@ __device__ __forceinline__ int padded(int i) { return i + (i >> 5); }
 
 // words each lane holds for a row of `total` words, and the lanes whose words are kept in scratch
 template <int CAP>
-__device__ __forceinline__ int words_per_lane(int total) {
+__host__ __device__ __forceinline__ int words_per_lane(int total) {
     if (CAP <= 256) return total <= 128 ? (total <= 64 ? 2 : total <= 96 ? 3 : 4) : total <= 192 ? 6 : 8;
     return total <= 384 ? (total <= 256 ? 8 : 12) : total <= 512 ? 16 : total <= 768 ? 24 : 32;
 }
@@ -300,21 +300,23 @@ __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int to
 template <typename T, typename P, int CAP, bool NUMERIC>
 constexpr int iw_blocks() {
     if (CAP <= 256) return sizeof(P) == 8 || (NUMERIC && sizeof(T) == 8) ? 9 : 12;
-    return sizeof(P) == 8 || (NUMERIC && sizeof(T) == 8) ? 3 : NUMERIC ? 5 : 6;
+    return sizeof(P) == 8 ? 3 : NUMERIC && sizeof(T) == 8 ? 5 : 7;
 }
 
 template <typename T, typename P, int CAP, bool NUMERIC>
 __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>())) ism_warp_kernel(const int* __restrict__ perm, DevCtl* __restrict__ ctl, int cls, int counter_slot,
                                                                  Csr A, Csr B, const i64* __restrict__ ub, i64* __restrict__ order_off, char* order_arena,
                                                                  size_t order_bytes, int* __restrict__ cnt,
-                                                                 const i64* __restrict__ rowptr, int* __restrict__ Ccrd, T* __restrict__ Cval) {
+                                                                 const i64* __restrict__ rowptr, int* __restrict__ Ccrd, T* __restrict__ Cval, int launch_slots) {
     typedef Pack<P, CAP> PK;
-    constexpr int SLOTS = CAP + CAP / 32;
+    const int slots = CAP > 256 ? launch_slots : CAP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    T* const vals = reinterpret_cast<T*>(smem_raw) + warp * (NUMERIC ? CAP : 0);
-    P* const packed = reinterpret_cast<P*>(smem_raw + (NUMERIC ? sizeof(T) * CAP * IW_WARPS : 0)) + warp * SLOTS;
-    unsigned short* const heads = reinterpret_cast<unsigned short*>(smem_raw + ((NUMERIC ? sizeof(T) * CAP : 0) + sizeof(P) * SLOTS) * IW_WARPS) + warp * CAP;
+    // per warp, `slots` products: values, packed words (one of padding per 32), places of the run heads
+    const int padded_slots = slots + slots / 32;
+    T* const vals = reinterpret_cast<T*>(smem_raw) + warp * (NUMERIC ? slots : 0);
+    P* const packed = reinterpret_cast<P*>(smem_raw + (NUMERIC ? (int)sizeof(T) * slots * IW_WARPS : 0)) + warp * padded_slots;
+    unsigned short* const heads = reinterpret_cast<unsigned short*>(smem_raw + ((NUMERIC ? (int)sizeof(T) * slots : 0) + (int)sizeof(P) * padded_slots) * IW_WARPS) + warp * slots;
     if (ctl->status != 0) return;
     int off, n;
     class_range(ctl, cls, off, n);
@@ -322,7 +324,7 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
     const T* __restrict__ Bval = (const T*)B.val;
     // The way to a row is a chain of loads (its number, its place in perm, its fields, its A entries, their B rows).  AHEAD:
     // the first links of the next row are fetched between the steps of the current one, where few warps per SM are
-    // bound by that chain: numeric, 8e4 rows of 674 products, f32, 369 -> 345 us, 8e5 rows of 60, f64, 199 -> 178 us.
+    // bound by that chain: numeric, 8e4 rows of 674 products, f32, 369 -> 345 us (20 warps on an SM), 8e5 rows of 60, f64, 199 -> 178 us.
     // Elsewhere the registers cost more than the chain (59-product rows, f32: numeric 148 -> 191 us, count 123 -> 126 us).
     constexpr bool AHEAD = NUMERIC && (CAP > 256 || sizeof(T) == 8);
     int row, row_n = -1, products, products_n = 0;
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
         products = products_n;
         ps = ps_n;
         pe = pe_n;
-        if (products > CAP) {                                    // the CTA kernel's rows
+        if (products > slots) {                                    // the CTA kernel's rows
             if (AHEAD) next();
             continue;
         }
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
                 if (gl < l0) { if (!sorted) c0 = __ldg(B.crd + q0 + gl); if (NUMERIC) v0 = __ldg(Bval + q0 + gl); }
                 if (gl < l1) { if (!sorted) c1 = __ldg(B.crd + q1 + gl); if (NUMERIC) v1 = __ldg(Bval + q1 + gl); }
                 auto put = [&](int slot, int col, T v) {
-                    if (slot < CAP) {                            // always so for a correctly classed row
+                    if (slot < slots) {                          // always so for a correctly classed row
                         if (!sorted) packed[padded(slot)] = PK::make(col, slot);
                         if (NUMERIC) vals[slot] = v;
                     }
@@ -415,7 +417,7 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
             }
             total += __shfl_sync(0xffffffffu, incl, 31);
         }
-        total = min(total, CAP);
+        total = min(total, slots);
         __syncwarp();
         if (AHEAD) take(__shfl_sync(0xffffffffu, r_n, 0));
 
@@ -487,7 +489,10 @@ static cudaError_t launch_k(const LaunchCtx& c, int cls, int n_host, const Csr& 
 
 template <typename T, typename P, int CAP, bool NUMERIC>
 static cudaError_t launch_warp_k(const LaunchCtx& c, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
-    const size_t smem = (size_t)IW_WARPS * ((NUMERIC ? (sizeof(T) + sizeof(short)) * CAP : 0) + sizeof(P) * (CAP + CAP / 32));
+    // room for the largest row of the launch, where it is known: more warps fit (numeric, 8e4 rows of up to 729 products,
+    // f32: 345 us at 1024 slots, 312 us at 768 and seven blocks per SM; f64 435 -> 299 us)
+    const int slots = CAP > 256 && c.max_ub_smem > 0 && c.max_ub_smem < CAP ? 32 * words_per_lane<CAP>((int)c.max_ub_smem) : CAP;
+    const size_t smem = (size_t)IW_WARPS * ((NUMERIC ? (sizeof(T) + sizeof(short)) * slots : 0) + sizeof(P) * (slots + slots / 32));
     cudaError_t e;
     int per_sm = 0;
     auto k = ism_warp_kernel<T, P, CAP, NUMERIC>;
@@ -496,7 +501,7 @@ static cudaError_t launch_warp_k(const LaunchCtx& c, int cls, int n_host, const 
     const i64 want = n_host >= 0 ? ((i64)n_host + IW_WARPS - 1) / IW_WARPS : grid;
     if (want < grid) grid = want > 0 ? want : 1;
     k<<<(int)grid, IW_WARPS * 32, smem, c.stream>>>(c.tab.perm, c.ctl, cls, cls + (NUMERIC ? NUM_SLOT : 0), A, B, c.tab.ub, c.tab.bm_off, c.order,
-                                                    c.order_bytes, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
+                                                    c.order_bytes, c.tab.cnt, rowptr, Ccrd, (T*)Cval, slots);
     ++c.launches;
     return cudaGetLastError();
 }
