@@ -1253,6 +1253,43 @@ def test_numeric_pass_enqueued_behind_the_symbolic_one(ctx, oracle_mod, monkeypa
     plan.close()
 
 
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_workspaces_on_forked_streams(oracle_mod, dtype):
+    """A power-law product, whose pass forks (rows for the sparse workspaces, the dense one by warps and by CTAs), on a
+    stream that is not the default one, the operands made and the result read on that stream; then two
+    threads with a context and a stream each."""
+    import threading
+    import torch
+    from paper_2404_04541_b200 import api
+    A = rmat_csr(13, 16, 9)
+    A.val = A.val.astype(dtype)
+    ref = oracle_mod.spgemm(A, A, threads=4)
+    errors = []
+
+    def work(ctx, rounds):
+        try:
+            for _ in range(rounds):
+                dA = api.DeviceCSR.from_host(A)
+                C, stats = ctx.spgemm(dA, dA)
+                got = C.pos.cpu().numpy(), C.crd.cpu().numpy(), C.val.cpu().numpy()
+                assert sum(stats["rows_per_class"][1:4]) > 0 and stats["rows_per_class"][4] > 0 and stats["dense_units"] > 0
+                assert_matches(got, ref, dtype)
+        except BaseException as e:                      # noqa: BLE001 (handed to the test's own thread)
+            errors.append(e)
+
+    def on_own_stream():
+        with torch.cuda.stream(torch.cuda.Stream()):
+            work(api.Context("cuda"), 4)
+
+    on_own_stream()
+    threads = [threading.Thread(target=on_own_stream) for _ in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
+
+
 # ------------------------------------------------------------------ boundary behaviour
 def test_error_statuses(ctx):
     import torch
