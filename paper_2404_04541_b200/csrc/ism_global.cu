@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(GL_THREADS) ism_global_kernel(const int* __res
     const int tid = threadIdx.x;
 
     // the arena follows the bitmap arena and the sorted words of other rows in the rest of the scratch buffer
-    const size_t before = (((size_t)ctl->bm_words_used * 4 + 255) & ~(size_t)255) + order_bytes;
+    const size_t before = (((size_t)ctl->bm_words * 4 + 255) & ~(size_t)255) + order_bytes;
     char* arena = rest + before;
     const size_t arena_bytes = rest_bytes > before ? rest_bytes - before : 0;
     // one slot per CTA: two all-array buffers of slot_elems components

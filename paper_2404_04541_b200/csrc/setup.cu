@@ -105,6 +105,13 @@ __global__ void __launch_bounds__(256) brow_summary_kernel(Csr B, int4* __restri
     }
 }
 
+// Arena words of a dense row: its bitmap, then the rank at the start of every 32-word chunk, 16-byte aligned.
+__device__ __forceinline__ int slot_words(int lo, int hi) {
+    const int nw = (hi - lo) / 32 + 1;
+    return (nw + (nw + 31) / 32 + 3) & ~3;
+}
+__device__ __forceinline__ bool dense_cls(int cls) { return cls == CLS_DENSE_WARP || cls == CLS_DENSE_HUB || cls == CLS_DENSE_CTA; }
+
 constexpr int LONG_LIST = 32;
 constexpr int MID_LIST = 64;
 
@@ -188,8 +195,10 @@ __device__ __forceinline__ void long_row_bounds(int row, const Csr& A, const Csr
                 atomicMax(&ctl->max_ub_smem, u);
                 if (u <= ISM_WARP_MAX) atomicAdd(&ctl->order_words, (u64)order_words_of((int)u));
             }
-            if (cls == CLS_DENSE_HUB || cls == CLS_DENSE_CTA || cls == CLS_DENSE_WARP)
+            if (dense_cls(cls)) {
                 atomicMax(&ctl->max_span_words, (hi - lo) / 32 + 1);
+                atomicAdd(&ctl->bm_words, (u64)slot_words(lo, hi));
+            }
         }
     }
 }
@@ -205,7 +214,7 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
     __shared__ int s_hist[8][NCLASS];
     __shared__ unsigned s_clow[8][NCLASS];
     __shared__ i64 s_cprod[8][NCLASS];
-    __shared__ i64 s_products, s_max_ub, s_max_ub_global, s_max_ub_smem;
+    __shared__ i64 s_max_ub, s_max_ub_global, s_max_ub_smem, s_bm_words;
     __shared__ int s_max_span_words;
     __shared__ unsigned s_order_words;              // (at most 1024 a row: no block sees 2^22 rows)
     // rows of more than LONG_A_ROW entries, which the block's threads take together at the end: left to
@@ -214,7 +223,7 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
     // rows of more than two steps of a narrow lane group, which the block's warps take at the end
     __shared__ int s_mid[MID_LIST], s_nmid;
     for (int x = threadIdx.x; x < 8 * NCLASS; x += blockDim.x) { (&s_hist[0][0])[x] = 0; (&s_clow[0][0])[x] = 0; (&s_cprod[0][0])[x] = 0; }
-    if (threadIdx.x == 0) { s_products = 0; s_max_ub = 0; s_max_ub_global = 0; s_max_ub_smem = 0; s_max_span_words = 0; s_order_words = 0; s_nlong = s_nmid = 0; }
+    if (threadIdx.x == 0) { s_max_ub = 0; s_max_ub_global = 0; s_max_ub_smem = 0; s_max_span_words = 0; s_bm_words = 0; s_order_words = 0; s_nlong = s_nmid = 0; }
     __syncthreads();
     int* const w_hist = s_hist[threadIdx.x >> 5];
     i64* const w_cprod = s_cprod[threadIdx.x >> 5];
@@ -237,10 +246,11 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
     // neighbours); narrower groups take neighbouring rows for the sake of the row offsets they share
     const i64 ngroups = ((i64)gridDim.x * blockDim.x) / G;
     const i64 group = G >= 8 ? (i64)(threadIdx.x / G) * gridDim.x + blockIdx.x : ((i64)blockIdx.x * blockDim.x + threadIdx.x) / G;
-    i64 my_products = 0, my_max = 0;
+    i64 my_max = 0;
     // rows and products of the class of this group's last rows: neighbouring rows mostly share a
     // class, so the shared-memory histogram is touched only when the class changes
     int run_cls = -1, run_rows = 0, my_span_words = 0;
+    unsigned my_bm_words = 0;                       // (2^31 rows over the groups of a full grid stay below 2^32 words a group)
     i64 run_products = 0;
     auto classify = [&](int row, i64 entries, i64 u, int lo, int hi) {
         if (lo < 0 || hi >= B.ncols) { raise_status(ctl, DEV_NONCANONICAL); u = 0; }
@@ -261,7 +271,6 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
         }
         ++run_rows;
         run_products += u;
-        my_products += u;
         my_max = max(my_max, u);
         // (rare classes: straight to shared memory, and only when the maximum would move)
         if (cls == CLS_ISM_GLOBAL && u > s_max_ub_global) atomicMax(&s_max_ub_global, u);
@@ -269,8 +278,10 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
             if (u > s_max_ub_smem) atomicMax(&s_max_ub_smem, u);
             if (u <= ISM_WARP_MAX) atomicAdd(&s_order_words, (unsigned)order_words_of((int)u));
         }
-        if (cls == CLS_DENSE_HUB || cls == CLS_DENSE_CTA || cls == CLS_DENSE_WARP)
+        if (dense_cls(cls)) {
             my_span_words = max(my_span_words, (hi - lo) / 32 + 1);
+            my_bm_words += (unsigned)slot_words(lo, hi);
+        }
     };
     // the next row's range and this lane's first entry of it are loaded while the current row is in hand: with
     // a few entries per row the kernel is a chain of dependent loads otherwise
@@ -392,30 +403,34 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
     for (int r = 0; r < min(s_nlong, LONG_LIST); ++r) long_row_bounds<SUMMARY>(s_long[r], A, B, tab, prm, ctl, brow);
     // the totals: reduced over the warp first (lanes other than a group's first hold zeros)
     for (int d = 16; d > 0; d >>= 1) {
-        my_products += __shfl_xor_sync(0xffffffffu, my_products, d);
         my_max = max(my_max, __shfl_xor_sync(0xffffffffu, my_max, d));
         my_span_words = max(my_span_words, __shfl_xor_sync(0xffffffffu, my_span_words, d));
     }
+    const unsigned bm_lo = __reduce_add_sync(0xffffffffu, my_bm_words & 0xffffu), bm_hi = __reduce_add_sync(0xffffffffu, my_bm_words >> 16);
     if (lane == 0) {
+        if (bm_lo | bm_hi) atomicAdd((u64*)&s_bm_words, (u64)bm_lo + ((u64)bm_hi << 16));
         if (my_span_words) atomicMax(&s_max_span_words, my_span_words);
-        if (my_products) atomicAdd((u64*)&s_products, (u64)my_products);
         if (my_max) atomicMax(&s_max_ub, my_max);
     }
     __syncthreads();
-    if (threadIdx.x < NCLASS) {
+    if (threadIdx.x < 32) {
         int rows = 0;
         i64 prods = 0;
-        for (int w = 0; w < 8; ++w) { rows += s_hist[w][threadIdx.x]; prods += s_cprod[w][threadIdx.x] + s_clow[w][threadIdx.x]; }
-        if (rows) atomicAdd(&ctl->class_count[threadIdx.x], rows);
-        if (prods) atomicAdd((u64*)&ctl->class_products[threadIdx.x], (u64)prods);
+        if (threadIdx.x < NCLASS) {
+            for (int w = 0; w < 8; ++w) { rows += s_hist[w][threadIdx.x]; prods += s_cprod[w][threadIdx.x] + s_clow[w][threadIdx.x]; }
+            if (rows) atomicAdd(&ctl->class_count[threadIdx.x], rows);
+            if (prods) atomicAdd((u64*)&ctl->class_products[threadIdx.x], (u64)prods);
+        }
+        for (int d = 8; d > 0; d >>= 1) prods += __shfl_xor_sync(0xffffffffu, prods, d);
+        if (threadIdx.x == 0 && prods) atomicAdd((u64*)&ctl->products, (u64)prods);
     }
     if (threadIdx.x == 0) {
-        if (s_products) atomicAdd((u64*)&ctl->products, (u64)s_products);
         if (s_max_ub) atomicMax(&ctl->max_ub, s_max_ub);
         if (s_max_ub_global) atomicMax(&ctl->max_ub_global, s_max_ub_global);
         if (s_max_ub_smem) atomicMax(&ctl->max_ub_smem, s_max_ub_smem);
         if (s_order_words) atomicAdd(&ctl->order_words, (u64)s_order_words);
         if (s_max_span_words) atomicMax(&ctl->max_span_words, s_max_span_words);
+        if (s_bm_words) atomicAdd(&ctl->bm_words, (u64)s_bm_words);
     }
 }
 
@@ -543,12 +558,26 @@ cudaError_t launch_bw_build(const LaunchCtx& c, const Csr& B) {
 // also reserve the slot of their occupancy bitmap in the arena.  Order inside a class follows
 // block arrival.
 // ---------------------------------------------------------------------------------------
-// It also counts the units per bucket of rows, clears the words of the kernels that hand running sums
-// from tile to tile, and its last block publishes the class sizes to the host.
+// It also counts the units per bucket of rows and clears the words of the kernels that hand running sums
+// from tile to tile.  A block of its own publishes the class sizes meanwhile, so that the host's next launch does not wait
+// for the rows (2048 rows: 10 us and a gap of 10 us behind it when the last block published, 4 us without a gap now; published by
+// the bounds kernel instead, the fences of its blocks cost 6 .. 14 us).
 __global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, HostBlock* host, int seq, u64* look, int n_look) {
     __shared__ int s_units[UNIT_BUCKETS];
+    const bool too_small = ctl->bm_words > prm.bm_arena_words;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) {
+            if (too_small) raise_status(ctl, DEV_SCRATCH_TOO_SMALL);
+            ctl->host_status = &host->late;
+        }
+        __syncthreads();
+        publish_ctl(ctl, host, seq);
+        return;
+    }
+    if (too_small) return;
+    const int block = blockIdx.x - 1, blocks = gridDim.x - 1;
     if (threadIdx.x < UNIT_BUCKETS) s_units[threadIdx.x] = 0;
-    for (int w = blockIdx.x * 256 + threadIdx.x; w < n_look; w += gridDim.x * 256) look[w] = 0;
+    for (int w = block * 256 + threadIdx.x; w < n_look; w += blocks * 256) look[w] = 0;
     const i64 unit_products = dense_unit_products(ctl->products, prm.unit_products);
     __shared__ int s_hist[NCLASS], s_base[NCLASS], s_off[NCLASS];
     __shared__ int ws[33];
@@ -559,7 +588,7 @@ __global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, 
         const int o = warp_incl_scan(n) - n;
         if (threadIdx.x < NCLASS) s_off[threadIdx.x] = o;
     }
-    for (i64 r0 = (i64)blockIdx.x * rows_per_block; r0 < m; r0 += (i64)gridDim.x * rows_per_block) {
+    for (i64 r0 = (i64)block * rows_per_block; r0 < m; r0 += (i64)blocks * rows_per_block) {
         if (threadIdx.x < NCLASS) s_hist[threadIdx.x] = 0;
         int cls[4], rank[4], words[4], my_words = 0;
 #pragma unroll
@@ -568,8 +597,7 @@ __global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, 
             cls[x] = row < m ? (int)tab.cls[row] : -1;
         }
         __syncthreads();
-        // bitmap words of this thread's dense rows (the words, then the rank at the start of every 32-word chunk,
-        // 16-byte aligned)
+        // bitmap words of this thread's dense rows
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
             const i64 row = r0 + x * blockDim.x + threadIdx.x;
@@ -580,9 +608,8 @@ __global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, 
             int at = 0;
             if (cls[x] >= 0 && (int)(threadIdx.x & 31) == first) at = atomicAdd(&s_hist[cls[x]], __popc(peers));
             rank[x] = __shfl_sync(0xffffffffu, at, first) + __popc(peers & ((1u << (threadIdx.x & 31)) - 1u));
-            if (cls[x] == CLS_DENSE_WARP || cls[x] == CLS_DENSE_HUB || cls[x] == CLS_DENSE_CTA) {
-                const int nw = (tab.jmax[row] - tab.jmin[row]) / 32 + 1;
-                words[x] = (nw + (nw + 31) / 32 + 3) & ~3;
+            if (dense_cls(cls[x])) {
+                words[x] = slot_words(tab.jmin[row], tab.jmax[row]);
                 if (cls[x] != CLS_DENSE_WARP) {
                     const i64 u = tab.ub[row];
                     atomicAdd(&s_units[unit_bucket(u)], dense_units_of_row(u, unit_products));
@@ -605,31 +632,19 @@ __global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, 
             if (words[x]) {
                 const u64 at = s_bm_base + (u64)my_off;
                 my_off += words[x];
-                if (at + (u64)words[x] > prm.bm_arena_words) {
-                    // the reservations follow one another, so one row crosses the end: it alone reports (262144
-                    // rows queueing at the status word cost a first pass that guessed too small a scratch 190 us)
-                    if (at <= prm.bm_arena_words) raise_status(ctl, DEV_SCRATCH_TOO_SMALL);
-                    tab.bm_off[row] = -1;
-                } else {
-                    tab.bm_off[row] = (i64)at;
-                }
+                tab.bm_off[row] = (i64)at;              // (inside the arena: the bounds kernel compared the total)
             }
         }
         __syncthreads();
     }
     if (threadIdx.x < UNIT_BUCKETS && s_units[threadIdx.x]) atomicAdd(&ctl->units_of[threadIdx.x], s_units[threadIdx.x]);
-    if (last_block(&ctl->bin_done, gridDim.x)) {
-        if (threadIdx.x == 0) ctl->host_status = &host->ctl.status;
-        __syncthreads();
-        publish_ctl(ctl, host, seq);
-    }
 }
 
 cudaError_t launch_bin_rows(const LaunchCtx& c, int m) {
     i64 want = ((i64)m + 1023) / 1024;
     i64 cap = (i64)c.sm_count * 8;
     if (want < 1) want = 1;
-    bin_rows_kernel<<<(int)(want < cap ? want : cap), 256, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.seq, c.look, c.n_look);
+    bin_rows_kernel<<<1 + (int)(want < cap ? want : cap), 256, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.seq, c.look, c.n_look);
     ++c.launches;
     return cudaGetLastError();
 }

@@ -184,7 +184,7 @@ struct spws_plan_s {
     int max_warp_cnt[N_WARP_LISTS] = {};    // ... and their largest output counts
     int64_t max_ub_smem = 0;    // most products of a shared-memory ISM row
     bool counters_clear = false; // the numeric pass's work counters are as the symbolic pass left them: zero
-    bool rows_path = false;     // the last symbolic pass was a row-wise one, whose errors reach host->ctl.status by themselves
+    bool rows_path = false;     // the last symbolic pass was a row-wise one, whose errors reach host->late by themselves
     int64_t bin_rows[NCLASS] = {};  // rows per internal class of the last symbolic pass
     // outer-product form: what the last symbolic pass decided
     int64_t outer_products = 0;
@@ -553,26 +553,33 @@ inline void mark_start(spws_plan_s* p, int pass) {
     p->ev_pass[pass] = true;
 }
 
-// Waits for publication `seq` of the control block: polled for a fifth of a millisecond, then by synchronising
-// the stream (which also reports a failed kernel).
+// Takes over publication `seq` of the control block: its words are polled for a fifth of a millisecond, then the stream is
+// synchronised (which also reports a failed kernel).
 spws_status_t wait_published(spws_plan_s* p, int seq) {
-    const volatile int* at = &p->host->seq;
+    const volatile u64* words = p->host->words;
+    int* const ctl = reinterpret_cast<int*>(&p->host->ctl);
+    int got = 0;
+    auto take = [&]() {
+        for (; got < CTL_WORDS; ++got) {
+            const u64 w = words[got];
+            if ((int)(w >> 32) != seq) return false;
+            ctl[got] = (int)(unsigned)w;
+        }
+        return true;
+    };
     const auto end = std::chrono::steady_clock::now() + std::chrono::microseconds(200);
     do {
         for (int k = 0; k < 64; ++k)
-            if (*at == seq) {
-                std::atomic_thread_fence(std::memory_order_acquire);
-                return SPWS_OK;
-            }
+            if (take()) return SPWS_OK;
     } while (std::chrono::steady_clock::now() < end);
     CUDA_TRY(cudaStreamSynchronize(p->h->stream));
-    return *at == seq ? SPWS_OK : SPWS_CUDA_ERROR;
+    return take() ? SPWS_OK : SPWS_CUDA_ERROR;
 }
 
-// What both passes use, known once the rows are binned: the fixed tables, the bitmaps of exactly the dense rows,
+// What both passes use, known with the class sizes: the fixed tables, the bitmaps of exactly the dense rows,
 // and the slots of the global-memory ISM, sized for its largest row.
 size_t rows_need(const spws_plan_s* plan, const Layout& L, const DevCtl& hc, int64_t ncols) {
-    size_t need = L.fixed_end + align256((size_t)hc.bm_words_used * 4);
+    size_t need = L.fixed_end + align256((size_t)hc.bm_words * 4);
     const int64_t n_global = hc.class_count[CLS_ISM_GLOBAL];
     if (n_global > 0) {
         int64_t elems = hc.max_ub_global < ncols ? hc.max_ub_global : ncols;
@@ -650,6 +657,7 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
                             spws_tensor_t* ttmC, i64* rowptr, char* sc) {
     plan->in_flight = true;
     plan->pending = false;
+    plan->host->late = 0;
     c.seq = plan->seq + 1;
     plan->seq += 2;
     // a1: upper bounds + classes; a2: binning
@@ -657,13 +665,18 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     mark(plan, SPWS_T_SYM_BOUNDS);
     CUDA_TRY(launch_bin_rows(c, (int)S.m));
     mark(plan, SPWS_T_SYM_BIN);
-    // the class sizes come back now (written to pinned memory by the binning kernel), so that only the
-    // workspaces that have rows are launched, with grids sized for them (a launch for an empty class
+    // the class sizes come back now (written to pinned memory while the binning runs), so that
+    // only the workspaces that have rows are launched, with grids sized for them (a launch for an empty class
     // costs as much as a small class's work)
     spws_status_t st = wait_published(plan, c.seq);
     if (st != SPWS_OK) return st;
-    plan->in_flight = false;
     const DevCtl& hc = *plan->host_ctl;
+    // a pass that ends here leaves nothing behind that still runs
+    auto give_up = [&](spws_status_t why) -> spws_status_t {
+        if (cudaStreamSynchronize(c.stream) != cudaSuccess) { cudaGetLastError(); return SPWS_CUDA_ERROR; }
+        plan->in_flight = false;
+        return why;
+    };
     // the sorted words of the mid-size rows are kept for the numeric pass behind the bitmaps when the scratch has room:
     // within the bytes that *needed tells, which are all that a caller need give the numeric pass
     const size_t need = rows_need(plan, L, hc, S.ncols);
@@ -671,18 +684,17 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     if (needed && (hc.status == 0 || hc.status == DEV_SCRATCH_TOO_SMALL)) {
         *needed = need + order;
         plan->least = need;
-        if (scratch_bytes < *needed) return SPWS_SCRATCH_TOO_SMALL;
+        if (scratch_bytes < *needed) return give_up(SPWS_SCRATCH_TOO_SMALL);
     }
     plan->order_bytes = order > 0 && scratch_bytes >= need + order ? order : 0;
-    plan->order_off = L.fixed_end + align256((size_t)hc.bm_words_used * 4);
+    plan->order_off = L.fixed_end + align256((size_t)hc.bm_words * 4);
     plan->order_need = need + order;
     use_order(plan, c, sc, scratch_bytes);
     if (hc.status != 0) {
         plan->stats = spws_stats_t{};
         plan->stats.device_status = hc.status;
-        return from_dev_status(hc.status);
+        return give_up(from_dev_status(hc.status));
     }
-    plan->in_flight = true;
     i64 hcount[NCLASS];
     for (int k = 0; k < NCLASS; ++k) hcount[k] = hc.class_count[k];
     const i64 products = hc.products;
@@ -776,7 +788,7 @@ spws_status_t rows_collect(spws_plan_s* plan) {
     plan->stats.dense_warp_rows = (int64_t)hc.n_warp_rows[0] + hc.n_warp_rows[1];
     plan->stats.dense_warp_products = hc.dense_warp_products;
     plan->stats.dense_warp_nnz = hc.dense_warp_nnz;
-    plan->stats.bitmap_bytes = (int64_t)hc.bm_words_used * 4;
+    plan->stats.bitmap_bytes = (int64_t)hc.bm_words * 4;
     plan->max_span_words = hc.max_span_words;
     for (int list = 0; list < N_WARP_LISTS; ++list) {
         plan->n_warp[list] = hc.n_warp_rows[list];
@@ -1676,7 +1688,8 @@ spws_status_t spws_workspace_size_exact(spws_plan_t plan, const spws_tensor_t* A
         CUDA_TRY(cudaMemcpyAsync(row_products, c.tab.ub, 8 * (size_t)S.m, cudaMemcpyDeviceToDevice, c.stream));
     CUDA_TRY(cudaStreamSynchronize(c.stream));
     plan->in_flight = false;
-    const DevCtl& hc = *plan->host_ctl;         // published by the binning kernel
+    if ((st = wait_published(plan, c.seq)) != SPWS_OK) return st;
+    const DevCtl& hc = *plan->host_ctl;
     if (hc.status != 0 && hc.status != DEV_SCRATCH_TOO_SMALL) return from_dev_status(hc.status);
     *bytes = rows_need(plan, L, hc, S.ncols);
     return SPWS_OK;
@@ -1846,6 +1859,7 @@ spws_status_t spws_get_stats(spws_plan_t plan, spws_stats_t* stats) {
     }
     CUDA_TRY(cudaStreamSynchronize(plan->h->stream));
     plan->in_flight = false;
+    if (plan->rows_path && plan->host->late != 0) plan->host_ctl->status = plan->host->late;
     plan->stats.device_status = plan->host_ctl->status;
     *stats = plan->stats;
     return from_dev_status(plan->host_ctl->status);
