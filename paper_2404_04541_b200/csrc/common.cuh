@@ -8,14 +8,14 @@ namespace spws {
 typedef long long i64;
 typedef unsigned long long u64;
 
-constexpr int NCLASS = 13;
+constexpr int NCLASS = 15;
 // Row classes = the workspace a row (or (i,j) fibre) is routed to in the symbolic pass.
 enum RowClass : int {
     CLS_EMPTY = 0,      // no intermediate product
     CLS_ISM_REG8 = 1,   // insert-sort-merge in registers, 8 lanes per row (<= 8 products)
     CLS_ISM_REG16 = 2,  // ... 16 lanes per row (<= 16 products)
     CLS_ISM_REG = 3,    // ... one warp per row (<= 32 products)
-    CLS_ISM_SMEM_S = 4, // insert-sort-merge in shared memory, small CTA
+    CLS_ISM_SMEM_S = 4, // insert-sort-merge of 129 .. 256 products, one warp per row
     CLS_ISM_SMEM = 5,   // insert-sort-merge in shared memory, full CTA
     CLS_DENSE_WARP = 6, // dense workspace (occupancy bitmap), one warp per row
     CLS_DENSE_HUB = 7,  // dense workspace, one CTA per row, heaviest rows (scheduled first)
@@ -23,7 +23,9 @@ enum RowClass : int {
     CLS_ISM_GLOBAL = 9, // accumulation array in shared memory, all array in global memory
     CLS_HASH_S = 10,    // hash table in shared memory (reduction at insert time), small CTA
     CLS_HASH = 11,      // hash table in shared memory, full CTA
-    CLS_COPY = 12       // one A entry picking a B row of at most COPY_MAX entries: the result is that row, scaled
+    CLS_COPY = 12,      // one A entry picking a B row of at most COPY_MAX entries: the result is that row, scaled
+    CLS_ISM_GROUP8 = 13,    // insert-sort-merge of at most 64 products by 8 lanes per row
+    CLS_ISM_GROUP16 = 14    // ... of 65 .. 128 products by 16 lanes
 };
 constexpr int NUM_SLOT = 16;   // work_counter[cls] in the symbolic pass, work_counter[NUM_SLOT + cls] in the numeric pass
 constexpr int CEIL_SLOT = 32;  // work_counter[CEIL_SLOT + cls] in the gather-only (iteration-only) kernels
@@ -34,8 +36,8 @@ constexpr int CEIL_WARP_SLOT = 54;
 constexpr int ISM_CTA_SLOT = 50; // work_counter slots of the CTA kernel of the shared-memory ISM, symbolic and numeric
 constexpr int ISM_CTA_NUM_SLOT = 51;
 constexpr int N_WORK_COUNTERS = 64;
-// index of a class in the public statistics (the three register classes are reported as one)
-__host__ __device__ inline int public_class(int cls) { return cls == 0 ? 0 : ((cls <= 3 || cls == 12) ? 1 : cls - 2); }
+// index of a class in the public statistics (the register classes are reported as one, and so are the small ISM ones)
+__host__ __device__ inline int public_class(int cls) { return cls == 0 ? 0 : (cls <= 3 || cls == 12) ? 1 : cls > 12 ? 2 : cls - 2; }
 constexpr int N_PUBLIC_CLASS = 10;
 constexpr int HASH_SMALL_CAP = 1024;       // products of a row the small / the full hash workspace takes
 constexpr int HASH_CAP = 4096;
@@ -92,14 +94,14 @@ struct DevCtl {
     int class_cursor[NCLASS];
     int work_counter[N_WORK_COUNTERS];   // dynamic work distribution; cleared before each pass
     i64 class_products[NCLASS];
-    i64 class_nnz[NCLASS];
+    i64 class_nnz[N_PUBLIC_CLASS];
     i64 dense_warp_products, dense_warp_nnz;   // share of the dense rows the warp numeric kernel takes
 };
 
 struct ClassParams {
     int policy;             // spws_policy_t
     int reg_cap;            // CLS_ISM_REG: products <= reg_cap
-    int smem_small_cap;     // CLS_ISM_SMEM_S
+    int smem_small_cap;     // CLS_ISM_GROUP8, CLS_ISM_GROUP16 and CLS_ISM_SMEM_S (at most 256)
     int smem_cap;           // CLS_ISM_SMEM
     int unit_outputs;       // accumulator capacity of a dense CTA unit
     int max_span_words;     // dense allowed up to this many bitmap words
@@ -290,7 +292,7 @@ __device__ __forceinline__ i64 look_back_warp(const u64* words, int tile, int pa
 // kept in scratch, and the words kept of a row that the kernel for up to ISM_WARP_MAX products sorts
 template <int CAP>
 __host__ __device__ __forceinline__ int words_per_lane(int total) {
-    if (CAP <= 256) return total <= 128 ? (total <= 64 ? 2 : total <= 96 ? 3 : 4) : total <= 192 ? 6 : 8;
+    if (CAP <= 256) return total <= 128 ? 4 : total <= 192 ? 6 : 8;
     return total <= 384 ? (total <= 256 ? 8 : 12) : total <= 512 ? 16 : total <= 768 ? 24 : 32;
 }
 __host__ __device__ __forceinline__ int order_lanes(int total, int e) { return ((total + e - 1) / e + 7) & ~7; }
@@ -386,6 +388,7 @@ struct LaunchCtx {
     u64* look;               // one word per tile of the kernels that hand running sums on ...
     int n_look;              // ... cleared by the binning kernel
     i64 max_ub_smem;         // largest product count of a CLS_ISM_SMEM row when known (0: unknown)
+    const i64* class_rows;   // rows per class, once they are binned
     uint2* bw;               // word lists of long B rows, indexed like B's entries (null: not built)
     int* bw_long;            // the long B rows, in arrival order
     int bw_long_cap;

@@ -1,5 +1,5 @@
-// Insert-sort-merge workspace of mid-size rows: a warp per output row with at most 1024 products, a
-// CTA per row beyond (Algorithm 1; the accumulation array is shared memory and is never full because
+// Insert-sort-merge workspace of mid-size rows: 8 or 16 lanes per output row of at most 64 or 128 products, a warp per row of
+// at most 1024, a CTA per row beyond (Algorithm 1; the accumulation array is shared memory and is never full because
 // the symbolic upper bound sized it; coordinate-sort policy, Sec. 5.2).
 //   Insert : product t of the row (loop order k, then j) is appended at slot t: its value stays
 //            there, and the packed word (j, t) enters the sort (accumulation indexing, Sec. 5.1:
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(THREADS) ism_smem_kernel(const int* __restrict
 // products, this one about 2.7.  Bound by instruction issue.
 //   Insert : 32 A entries at a time; a group of lanes per entry (as many as the mean B row has
 //            entries) writes the products of its B row at their slots.
-//   Sort   : E = 2, 3, 4, 6, 8, 12, 16, 24 or 32 words per lane, the smallest network that holds the row.
+//   Sort   : E = 4, 6, 8, 12, 16, 24 or 32 words per lane, the smallest network that holds the row.
 //   Merge  : the sorted words go back to shared memory, the places of the run heads are packed, and
 //            one lane per run sums it in slot order.
 //   Of rows of more than 256 products the counting pass leaves the sorted words in scratch when there is room
@@ -175,10 +175,10 @@ __device__ __forceinline__ void sort_pair(P& a, P& b) {
     b = hi;
 }
 
-// Ascending bitonic sort of 32 * E words, element index = lane * E + x, E = 2^a or 3 * 2^a.  Every merge starts with
-// the mirrored comparison (i against i ^ (k - 1) within its k), so all comparisons point the same way; with
+// Ascending bitonic sort of G * E words by each group of G lanes, element index = lane of the group * E + x, E = 2^a or
+// 3 * 2^a.  Every merge starts with the mirrored comparison (i against i ^ (k - 1) within its k), so all comparisons point the same way; with
 // a factor of three the merges end at triples, which three comparisons sort.
-template <typename P, int E>
+template <typename P, int E, int G = 32>
 __device__ __forceinline__ void warp_sort(P (&w)[E]) {
     constexpr int BASE = E % 3 == 0 ? 3 : 1;
     const int lane = threadIdx.x & 31;
@@ -214,7 +214,7 @@ __device__ __forceinline__ void warp_sort(P (&w)[E]) {
     // rows of 674: 456 against 384; of up to 8 words the unrolled ones are faster, 50 against 55 us)
     constexpr int U = E > 8 ? 1 : 5;
 #pragma unroll U
-    for (int m = 2; m <= 32; m <<= 1) {
+    for (int m = 2; m <= G; m <<= 1) {
         const bool low_half = (lane & (m >> 1)) == 0;
 #pragma unroll
         for (int x = 0; x < (E + 1) / 2; ++x) {
@@ -286,6 +286,175 @@ __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int to
         __syncwarp();
     }
     return n;
+}
+
+// ---------------------------------------------------------------------------------------
+// Rows of at most 64 or 128 products: G = 8 or 16 lanes per row, eight products per lane at most, so that a warp works on four
+// or two of them at a time.
+//   Insert : G entries at a time; lane l takes the products l, l + G, .. of those entries, whose owners it finds by a search
+//            among the running counts.
+//   Sort   : six or eight words per lane in registers; the narrower the group, the more of the network stays inside the lanes.
+//   Merge  : as below: the sorted words and the places of the run heads go to shared memory, a lane per run.
+// Every step of the way to a row's products is a load that waits for the one before: several rows per warp and some 40 warps
+// keep enough of them in flight, and a block for every 128 lanes' rows spares fetching ahead (persistent blocks: numeric 80 us
+// where these take 75).  Bound by the integer pipe (half of the instructions, a warp every two cycles).  A warp per row
+// against this, count + numeric: 2e5 rows of 59 products, f32, 123 + 148 and 92 + 128 us; 1.6e5 fibres of 110, 95 + 108 and 64 + 93
+// us; 1.9e5 rows of 82, f64, 137 + 178 and 99 + 144 us.
+// ---------------------------------------------------------------------------------------
+constexpr int IG_THREADS = 128;
+
+template <typename T, bool NUMERIC> struct GroupEntry { i64 q; T a; };          // start of the B row less the products before it
+template <typename T> struct GroupEntry<T, false> { i64 q; };
+
+template <int G> __host__ __device__ constexpr int group_words() { return 8 * G + G / 4 + G; }     // packed words of a row, with room against bank conflicts
+template <typename T, typename P, int G, bool NUMERIC>
+__host__ __device__ constexpr int group_row_bytes() {
+    return (int)sizeof(GroupEntry<T, NUMERIC>) * G + (NUMERIC ? (int)sizeof(T) * 9 * G : 0) + (int)sizeof(P) * group_words<G>() + (NUMERIC ? 8 * G : 0);
+}
+template <typename T, typename P, bool NUMERIC> constexpr int group_blocks() { return sizeof(P) == 8 ? 8 : NUMERIC && sizeof(T) == 8 ? 10 : 12; }
+
+// Sorts a row's packed words and counts its distinct columns; numeric: leaves the sorted words in `packed` and the places of the
+// run heads in `heads`.  For all lanes of a warp together.
+template <typename PK, typename P, int E, int G, bool NUMERIC>
+__device__ __forceinline__ int sort_group(P* packed, unsigned char* heads, int total, int gl) {
+    P w[E];
+#pragma unroll
+    for (int x = 0; x < E; ++x) {
+        const int i = x * G + gl;
+        w[x] = i < total ? packed[padded(i)] : PK::sentinel();
+    }
+    warp_sort<P, E, G>(w);
+    const P before = __shfl_up_sync(0xffffffffu, w[E - 1], 1, G);
+    unsigned head = 0;
+#pragma unroll
+    for (int x = 0; x < E; ++x) {
+        const bool first = x == 0 ? (gl == 0 || PK::key(w[x]) != PK::key(before)) : PK::key(w[x]) != PK::key(w[x > 0 ? x - 1 : 0]);
+        if (w[x] != PK::sentinel() && first) head |= 1u << x;
+    }
+    const int mine = __popc(head);
+    int incl = mine;
+#pragma unroll
+    for (int d = 1; d < G; d <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, d, G);
+        if (gl >= d) incl += t;
+    }
+    if (NUMERIC) {
+        __syncwarp();
+        int at = incl - mine;
+#pragma unroll
+        for (int x = 0; x < E; ++x) {
+            packed[padded(gl * E + x)] = w[x];
+            if ((head >> x) & 1u) heads[at++] = (unsigned char)(gl * E + x);
+        }
+        __syncwarp();
+    }
+    return __shfl_sync(0xffffffffu, incl, G - 1, G);
+}
+
+template <typename T, typename P, int G, bool NUMERIC>
+__global__ void __launch_bounds__(IG_THREADS, (group_blocks<T, P, NUMERIC>())) ism_group_kernel(const int* __restrict__ rows, int n, const DevCtl* __restrict__ ctl,
+                                                                                               Csr A, Csr B, int* __restrict__ cnt,
+                                                                                               const i64* __restrict__ rowptr, int* __restrict__ Ccrd,
+                                                                                               T* __restrict__ Cval) {
+    constexpr int CAP = 8 * G, ROWS = IG_THREADS / G;
+    typedef Pack<P, CAP> PK;
+    typedef GroupEntry<T, NUMERIC> Entry;
+    __shared__ __align__(16) unsigned char smem[ROWS * group_row_bytes<T, P, G, NUMERIC>()];
+    const int gl = threadIdx.x % G, group = threadIdx.x / G;
+    Entry* const entry = reinterpret_cast<Entry*>(smem) + group * G;
+    T* const vals = reinterpret_cast<T*>(smem + ROWS * G * sizeof(Entry)) + group * (NUMERIC ? 9 * G : 0);
+    P* const packed = reinterpret_cast<P*>(smem + ROWS * G * (sizeof(Entry) + (NUMERIC ? 9 * sizeof(T) : 0))) + group * group_words<G>();
+    unsigned char* const heads = smem + ROWS * (G * (sizeof(Entry) + (NUMERIC ? 9 * sizeof(T) : 0)) + sizeof(P) * group_words<G>()) + group * (NUMERIC ? CAP : 0);
+    const T* __restrict__ Aval = (const T*)A.val;
+    const T* __restrict__ Bval = (const T*)B.val;
+    if (ctl->status != 0) return;
+    const int r = blockIdx.x * ROWS + group;
+    if ((r & ~(32 / G - 1)) >= n) return;           // (whole warps)
+    int row = 0;
+    i64 ps = 0, pe = 0;
+    if (r < n) {
+        row = __ldg(rows + r);
+        ps = __ldg(A.pos + row);
+        pe = __ldg(A.pos + row + 1);
+    }
+    // ---- Insert
+    int total = 0;
+    for (i64 p0 = ps; __any_sync(0xffffffffu, p0 < pe); p0 += G) {
+        const i64 p = p0 + gl;
+        i64 qs = 0;
+        int len = 0;
+        T a = 0;
+        if (p < pe) {
+            const int k = __ldg(A.crd + p);
+            if (NUMERIC) a = __ldg(Aval + p);
+            if ((unsigned)k < (unsigned)B.nrows) {
+                qs = __ldg(B.pos + k);
+                len = max((int)(__ldg(B.pos + k + 1) - qs), 0);
+            }
+        }
+        int incl = len;
+#pragma unroll
+        for (int d = 1; d < G; d <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, d, G);
+            if (gl >= d) incl += t;
+        }
+        const int excl = incl - len;
+        const int chunk = min(__shfl_sync(0xffffffffu, incl, G - 1, G), CAP - total);      // (a correctly classed row fits)
+        entry[gl].q = qs - excl;
+        if constexpr (NUMERIC) entry[gl].a = a;
+        __syncwarp();
+        const int most = __reduce_max_sync(0xffffffffu, max(chunk, 0));
+        for (int u0 = 0; u0 < most; u0 += 4 * G) {
+            int col[4];
+            T v[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                // the last entry whose running count is <= u
+                const int u = u0 + x * G + gl;
+                int e = 0;
+#pragma unroll
+                for (int s = G / 2; s >= 1; s >>= 1) {
+                    const int before = __shfl_sync(0xffffffffu, excl, e + s, G);
+                    if (before <= u) e += s;
+                }
+                if (u < chunk) {
+                    const Entry d = entry[e];
+                    col[x] = __ldg(B.crd + d.q + u);
+                    if constexpr (NUMERIC) v[x] = mul_rn(d.a, __ldg(Bval + d.q + u));
+                }
+            }
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const int u = u0 + x * G + gl, slot = total + u;
+                if (u < chunk) {
+                    packed[padded(slot)] = PK::make(col[x], slot);
+                    if (NUMERIC) vals[slot] = v[x];
+                }
+            }
+        }
+        total += max(chunk, 0);
+        __syncwarp();
+    }
+    // ---- Sort
+    int distinct;
+    if (__any_sync(0xffffffffu, total > 6 * G)) distinct = sort_group<PK, P, 8, G, NUMERIC>(packed, heads, total, gl);
+    else distinct = sort_group<PK, P, 6, G, NUMERIC>(packed, heads, total, gl);
+    // ---- Merge
+    if (r < n) {
+        if (!NUMERIC) {
+            if (gl == 0) cnt[row] = distinct;
+        } else {
+            const i64 out0 = __ldg(rowptr + row);
+            for (int h = gl; h < distinct; h += G) {
+                const int x0 = heads[h], x1 = h + 1 < distinct ? (int)heads[h + 1] : total;
+                const P w = packed[padded(x0)];
+                T sum = vals[PK::slot(w)];
+                for (int x = x0 + 1; x < x1; ++x) sum = add_rn(sum, vals[PK::slot(packed[padded(x)])]);
+                Ccrd[out0 + h] = (int)PK::key(w);
+                Cval[out0 + h] = sum;
+            }
+        }
+    }
 }
 
 // blocks an SM is to hold (the compiler would keep several of the networks below in registers at once)
@@ -420,8 +589,6 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
         if (CAP > 256 && !NUMERIC && order_arena && lane == 0) order_off[row] = order ? (i64)(reinterpret_cast<char*>(order) - order_arena) : -1;
         if constexpr (CAP <= 256) {
             switch (e) {
-                case 2: distinct = sort_row<PK, P, 2, NUMERIC>(packed, heads, total, keep); break;
-                case 3: distinct = sort_row<PK, P, 3, NUMERIC>(packed, heads, total, keep); break;
                 case 4: distinct = sort_row<PK, P, 4, NUMERIC>(packed, heads, total, keep); break;
                 case 6: distinct = sort_row<PK, P, 6, NUMERIC>(packed, heads, total, keep); break;
                 default: distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total, keep); break;
@@ -506,6 +673,28 @@ size_t order_bytes_of(i64 words, i64 max_products, i64 ncols) {
     return (size_t)words * (ncols < (1ll << (32 - Log2<ISM_WARP_MAX>::value)) ? 4 : 8);     // wide words from 2^22 columns on
 }
 
+template <typename T, typename P, int G, bool NUMERIC>
+static cudaError_t launch_group_k(const LaunchCtx& c, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
+    constexpr int ROWS = IG_THREADS / G;
+    i64 off = 0;
+    for (int x = 0; x < cls; ++x) off += c.class_rows[x];
+    ism_group_kernel<T, P, G, NUMERIC><<<(n_host + ROWS - 1) / ROWS, IG_THREADS, 0, c.stream>>>(c.tab.perm + off, n_host, c.ctl, A, B, c.tab.cnt, rowptr, Ccrd,
+                                                                                             (T*)Cval);
+    ++c.launches;
+    return cudaGetLastError();
+}
+
+template <typename T, int G>
+static cudaError_t launch_group(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd,
+                                void* Cval) {
+    // (the count does not depend on the value type)
+    if (narrow<8 * G>(B))
+        return numeric ? launch_group_k<T, unsigned, G, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
+                       : launch_group_k<float, unsigned, G, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
+    return numeric ? launch_group_k<T, u64, G, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
+                   : launch_group_k<float, u64, G, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
+}
+
 template <typename T, int CAP>
 static cudaError_t launch_warp(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd,
                                void* Cval) {
@@ -519,9 +708,10 @@ static cudaError_t launch_warp(const LaunchCtx& c, bool numeric, int cls, int n_
 template <typename T>
 static cudaError_t launch_t(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B,
                             const i64* rowptr, int* Ccrd, void* Cval) {
-    // the small class, and the full one when its largest row is that small: fewer registers and less
-    // shared memory per warp
-    i64 most = (cls == CLS_ISM_SMEM_S) ? c.prm.smem_small_cap : c.prm.smem_cap;
+    if (cls == CLS_ISM_GROUP8) return launch_group<T, 8>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
+    if (cls == CLS_ISM_GROUP16) return launch_group<T, 16>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
+    // (the full class when its largest row is that small: fewer registers and less shared memory per warp)
+    i64 most = cls == CLS_ISM_SMEM_S ? 256 : c.prm.smem_cap;
     if (cls == CLS_ISM_SMEM && c.max_ub_smem > 0 && c.max_ub_smem < most) most = c.max_ub_smem;
     if (most <= 256) return launch_warp<T, 256>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
     cudaError_t e = launch_warp<T, ISM_WARP_MAX>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);

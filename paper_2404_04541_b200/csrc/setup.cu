@@ -45,6 +45,9 @@ __device__ __forceinline__ int dense_class(i64 ub, i64 span_words) {
     return ub >= DENSE_HUB_UB ? CLS_DENSE_HUB : CLS_DENSE_CTA;
 }
 
+// (a warp per row from 129 products on: 32 lanes of the group kernel took 41 + 51 us on 3e4 rows of 143 products, a warp 36 + 49)
+__device__ __forceinline__ int small_ism_class(i64 ub) { return ub <= 64 ? CLS_ISM_GROUP8 : ub <= 128 ? CLS_ISM_GROUP16 : CLS_ISM_SMEM_S; }
+
 __device__ __forceinline__ int classify_row(i64 ub, i64 entries, int jmin, int jmax, const ClassParams& prm, DevCtl* ctl) {
     if (ub == 0) return CLS_EMPTY;
     const i64 span = (i64)jmax - jmin + 1;
@@ -63,7 +66,7 @@ __device__ __forceinline__ int classify_row(i64 ub, i64 entries, int jmin, int j
     const int reg_cls = ub <= 8 ? CLS_ISM_REG8 : (ub <= 16 ? CLS_ISM_REG16 : CLS_ISM_REG);
     if (prm.policy == 1) {                       // sparse ISM forced
         if (reg_ok) return reg_cls;
-        if (ub <= prm.smem_small_cap) return CLS_ISM_SMEM_S;
+        if (ub <= prm.smem_small_cap) return small_ism_class(ub);
         if (ub <= prm.smem_cap) return CLS_ISM_SMEM;
         return CLS_ISM_GLOBAL;
     }
@@ -78,9 +81,9 @@ __device__ __forceinline__ int classify_row(i64 ub, i64 entries, int jmin, int j
     // up to 128 products the register sort beats the bitmap whatever the span; up to 256 when the bitmap is wide
     // (6e6 products, f64, both passes, dense against ISM: 60 products a row 263 : 172 us, 117 a row 156 : 126
     // us, 240 a row on 94 words 119 : 113 us and on 626 words 160 : 110 us; 380 a row 98 : 168 us)
-    if (ub <= prm.smem_small_cap && (ub <= 128 || span_words > 256)) return CLS_ISM_SMEM_S;
+    if (ub <= prm.smem_small_cap && (ub <= 128 || span_words > 256)) return small_ism_class(ub);
     if (dense_ok && (float)span_words <= prm.span_words_per_product * (float)ub) return dense_class(ub, span_words);
-    if (ub <= prm.smem_small_cap) return CLS_ISM_SMEM_S;
+    if (ub <= prm.smem_small_cap) return small_ism_class(ub);
     if (ub <= prm.smem_cap) return CLS_ISM_SMEM;
     if (dense_ok) return dense_class(ub, span_words);
     return CLS_ISM_GLOBAL;
@@ -686,7 +689,7 @@ __global__ void __launch_bounds__(FR_THREADS, DENSE ? 3 : 5) finish_rows_kernel(
     __shared__ i64 s_sum[FR_WARPS], s_before[2];
     __shared__ int s_part[1 + N_WARP_LISTS][FR_WARPS];     // survivors, warp rows on each list
     __shared__ int s_wbase[N_WARP_LISTS], s_units[UNIT_BUCKETS];           // places in the routing tables; units: the tile's count, then the running place
-    __shared__ i64 s_cls[FR_WARPS][NCLASS];
+    __shared__ i64 s_cls[FR_WARPS][N_PUBLIC_CLASS];
     __shared__ i64 s_wp[FR_WARPS];
     __shared__ int s_wn[FR_WARPS], s_wm[N_WARP_LISTS][FR_WARPS];
     __shared__ int s_kept[TTM ? FR_TILE : 1];       // survivors of the tile before each fibre
@@ -694,7 +697,7 @@ __global__ void __launch_bounds__(FR_THREADS, DENSE ? 3 : 5) finish_rows_kernel(
     const unsigned all = 0xffffffffu, below = (1u << lane) - 1u;
     const int tiles = gridDim.x;
     if (tid == 0) s_tile = atomicAdd(&ctl->rows_ticket, 1);
-    for (int x = tid; x < FR_WARPS * NCLASS; x += FR_THREADS) (&s_cls[0][0])[x] = 0;
+    for (int x = tid; x < FR_WARPS * N_PUBLIC_CLASS; x += FR_THREADS) (&s_cls[0][0])[x] = 0;
     if (tid >= 128 && tid < 128 + UNIT_BUCKETS) s_units[tid - 128] = 0;
     __syncthreads();
     const int tile = s_tile;
@@ -738,13 +741,13 @@ __global__ void __launch_bounds__(FR_THREADS, DENSE ? 3 : 5) finish_rows_kernel(
     auto units = [&](int x) { return cls[x] == CLS_DENSE_WARP ? 1 : q[x] & 0xfffffff; };
     auto bucket = [&](int x) { return !few ? 0 : cls[x] == CLS_DENSE_WARP ? UNIT_BUCKETS - 1 : q[x] >> 28; };
     bool one_class = true;
-    // the class of the warp's first row that is not empty in the first 32 rows (all empty: any)
+    // the (public) class of the warp's first row that is not empty in the first 32 rows (all empty: any)
     const unsigned some = __ballot_sync(all, cls[0] != CLS_EMPTY);
-    const int cls0 = __shfl_sync(all, cls[0], some ? __ffs(some) - 1 : 0);
+    const int cls0 = public_class(__shfl_sync(all, cls[0], some ? __ffs(some) - 1 : 0));
 #pragma unroll
     for (int x = 0; x < FR_ITEMS; ++x) {
         sum += v[x];
-        one_class &= cls[x] == cls0 || cls[x] == CLS_EMPTY;
+        one_class &= public_class(cls[x]) == cls0 || cls[x] == CLS_EMPTY;
         if (TTM) kept += __popc(__ballot_sync(all, v[x] > 0));
         if (DENSE) {
             const int l = list_of(x);
@@ -766,8 +769,8 @@ __global__ void __launch_bounds__(FR_THREADS, DENSE ? 3 : 5) finish_rows_kernel(
         for (int x = 0; x < FR_ITEMS; ++x) {
             unsigned todo = __ballot_sync(all, cls[x] != CLS_EMPTY);
             while (todo) {
-                const int k = __shfl_sync(all, cls[x], __ffs(todo) - 1);
-                const bool mine = cls[x] == k;
+                const int k = public_class(__shfl_sync(all, cls[x], __ffs(todo) - 1));
+                const bool mine = public_class(cls[x]) == k;
                 const unsigned lo = __reduce_add_sync(all, mine ? (unsigned)v[x] & 0xffffu : 0u);
                 const unsigned hi = __reduce_add_sync(all, mine ? (unsigned)v[x] >> 16 : 0u);
                 if (lane == 0) s_cls[warp][k] += (i64)lo + ((i64)hi << 16);
@@ -853,7 +856,7 @@ __global__ void __launch_bounds__(FR_THREADS, DENSE ? 3 : 5) finish_rows_kernel(
         }
         s_units[k] = at;
     }
-    if (tid >= 192 && tid < 192 + NCLASS) {
+    if (tid >= 192 && tid < 192 + N_PUBLIC_CLASS) {
         i64 t = 0;
         for (int w = 0; w < FR_WARPS; ++w) t += s_cls[w][tid - 192];
         if (t) atomicAdd((u64*)&ctl->class_nnz[tid - 192], (u64)t);

@@ -697,9 +697,10 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     }
     i64 hcount[NCLASS];
     for (int k = 0; k < NCLASS; ++k) hcount[k] = hc.class_count[k];
+    c.class_rows = hcount;
     const i64 products = hc.products;
     plan->sparse_products = 0;
-    for (int k : {CLS_COPY, CLS_ISM_REG8, CLS_ISM_REG16, CLS_ISM_REG, CLS_ISM_SMEM_S, CLS_ISM_SMEM}) plan->sparse_products += hc.class_products[k];
+    for (int k : {CLS_COPY, CLS_ISM_REG8, CLS_ISM_REG16, CLS_ISM_REG, CLS_ISM_GROUP8, CLS_ISM_GROUP16, CLS_ISM_SMEM_S, CLS_ISM_SMEM}) plan->sparse_products += hc.class_products[k];
     const bool any_dense = hcount[CLS_DENSE_WARP] + hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0;
     plan->max_ub_smem = hc.max_ub_smem;
     c.max_ub_smem = plan->max_ub_smem;
@@ -712,10 +713,11 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
             CUDA_TRY(launch_ism_reg(c, false, hcount, S.A, S.B, rowptr, nullptr, nullptr));
             mark(plan, SPWS_T_SYM_ISM_REG);
         }
-        if (hcount[CLS_ISM_SMEM_S] > 0) {
-            CUDA_TRY(launch_ism_smem(c, false, CLS_ISM_SMEM_S, (int)hcount[CLS_ISM_SMEM_S], S.A, S.B, rowptr, nullptr, nullptr));
-            mark(plan, SPWS_T_SYM_ISM_SMEM_S);
-        }
+        for (int cls : {CLS_ISM_GROUP8, CLS_ISM_GROUP16, CLS_ISM_SMEM_S})
+            if (hcount[cls] > 0) {
+                CUDA_TRY(launch_ism_smem(c, false, cls, (int)hcount[cls], S.A, S.B, rowptr, nullptr, nullptr));
+                mark(plan, SPWS_T_SYM_ISM_SMEM_S);
+            }
         if (hcount[CLS_ISM_SMEM] > 0) {
             CUDA_TRY(launch_ism_smem(c, false, CLS_ISM_SMEM, (int)hcount[CLS_ISM_SMEM], S.A, S.B, rowptr, nullptr, nullptr));
             mark(plan, SPWS_T_SYM_ISM_SMEM);
@@ -782,8 +784,8 @@ spws_status_t rows_collect(spws_plan_s* plan) {
     for (int k = 0; k < NCLASS; ++k) {
         plan->stats.rows_per_class[public_class(k)] += hc.class_count[k];
         plan->stats.products_per_class[public_class(k)] += hc.class_products[k];
-        plan->stats.nnz_per_class[public_class(k)] += hc.class_nnz[k];
     }
+    for (int k = 0; k < N_PUBLIC_CLASS; ++k) plan->stats.nnz_per_class[k] = hc.class_nnz[k];
     plan->stats.dense_units = hc.n_units;
     plan->stats.dense_warp_rows = (int64_t)hc.n_warp_rows[0] + hc.n_warp_rows[1];
     plan->stats.dense_warp_products = hc.dense_warp_products;
@@ -809,16 +811,18 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, cha
     c.max_ub_smem = plan->max_ub_smem;
     const spws_stats_t& s = plan->stats;
     const int64_t* bins = plan->bin_rows;
+    c.class_rows = LL(bins);
     Fork fork(plan, c, s.dense_warp_rows > 0, s.dense_units > 0 || bins[CLS_ISM_GLOBAL] > 0);
     fork.group(0);
     if (bins[CLS_COPY] + bins[CLS_ISM_REG8] + bins[CLS_ISM_REG16] + bins[CLS_ISM_REG] > 0) {
         CUDA_TRY(launch_ism_reg(c, true, LL(bins), S.A, S.B, rowptr, crd, val));
         mark(plan, SPWS_T_NUM_ISM_REG);
     }
-    if (bins[CLS_ISM_SMEM_S] > 0) {
-        CUDA_TRY(launch_ism_smem(c, true, CLS_ISM_SMEM_S, (int)bins[CLS_ISM_SMEM_S], S.A, S.B, rowptr, crd, val));
-        mark(plan, SPWS_T_NUM_ISM_SMEM_S);
-    }
+    for (int cls : {CLS_ISM_GROUP8, CLS_ISM_GROUP16, CLS_ISM_SMEM_S})
+        if (bins[cls] > 0) {
+            CUDA_TRY(launch_ism_smem(c, true, cls, (int)bins[cls], S.A, S.B, rowptr, crd, val));
+            mark(plan, SPWS_T_NUM_ISM_SMEM_S);
+        }
     if (bins[CLS_ISM_SMEM] > 0) {
         CUDA_TRY(launch_ism_smem(c, true, CLS_ISM_SMEM, (int)bins[CLS_ISM_SMEM], S.A, S.B, rowptr, crd, val));
         mark(plan, SPWS_T_NUM_ISM_SMEM);
