@@ -53,6 +53,13 @@ __device__ __forceinline__ int chunks_of(int nw) { return (nw + 31) >> 5; }
 // 60 us without, 49 us with the scan; 729 products on 521 words: 408 us without, 457 us with it.
 constexpr int DW_SCAN_WORDS = 256;
 
+// Place of bitmap word w in shared memory.  The planes of a grid lie some multiple of 32 words apart when its sides are powers
+// of two, its lines one or two words: bits 5 .. 8 of w move the words (and the two-byte ranks) of different planes to different
+// banks.  For spans beyond DW_SCAN_WORDS only, where such planes fit and the two instructions pay: 64^3 stencil, f64, symbolic 410 ->
+// 378 us, numeric 632 -> 611 us.
+template <bool SPREAD>
+__device__ __forceinline__ unsigned bank_spread(unsigned w) { return SPREAD ? w ^ ((w >> 4) & 30u) : w; }
+
 template <bool SCAN>
 __global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __restrict__ ctl, int warp_outputs, Csr A, Csr B, RowTables tab) {
     __shared__ unsigned s_bm[DW_WARPS][SCAN ? DW_SCAN_WORDS : DENSE_WARP_BM_WORDS];
@@ -91,7 +98,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __re
                     atomicOr(&bm[w], bit);
                     return;
                 }
-                const unsigned old = atomicOr(&bm[w], bit);
+                const unsigned old = atomicOr(&bm[bank_spread<!SCAN>(w)], bit);
                 if (!(old & bit)) {
                     ++cnt;
                     if (old == 0u) { ++nzw; atomicOr(&sum[w >> 5], 1u << (w & 31)); }
@@ -174,8 +181,8 @@ __global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __re
             while (s) {
                 const int w = (lane << 5) + __ffs(s) - 1;
                 s &= s - 1;
-                out2[at++] = make_uint2(bm[w], (unsigned)w);
-                bm[w] = 0;
+                out2[at++] = make_uint2(bm[bank_spread<!SCAN>(w)], (unsigned)w);
+                bm[bank_spread<!SCAN>(w)] = 0;
             }
             if (lane == 0) tab.bm_off[row] = slot | ((i64)nzw << BM_NZW_SHIFT) | BM_COMPACT;
         } else {
@@ -184,8 +191,8 @@ __global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __re
             int carry = 0;
             for (int w0 = 0; w0 < nw; w0 += 32) {
                 const int w = w0 + lane;
-                const unsigned word = (w < nw) ? bm[w] : 0u;
-                if (w < nw) { out[w] = word; bm[w] = 0; }
+                const unsigned word = (w < nw) ? bm[bank_spread<!SCAN>(w)] : 0u;
+                if (w < nw) { out[w] = word; bm[bank_spread<!SCAN>(w)] = 0; }
                 int c = __popc(word);
                 for (int d = 16; d > 0; d >>= 1) c += __shfl_xor_sync(0xffffffffu, c, d);
                 if (lane == 0) out[nw + (w0 >> 5)] = (unsigned)carry;
@@ -362,7 +369,7 @@ __global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __
 // ---------------------------------------------------------------------------------------
 // CEIL = true: the same walk over rows, entries and B rows with the workspace stripped (Sec. 7.2,
 // iteration-only lower bound); the gathered indices and products go into two checksums.
-template <typename T, bool CEIL>
+template <typename T, bool CEIL, bool SPREAD>
 __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __restrict__ ctl, const int* __restrict__ rows, int step, int n, int slot_,
                                                                     int bmw, int accw, Csr A, Csr B, RowTables tab,
                                                                     const i64* __restrict__ rowptr, int* __restrict__ Ccrd,
@@ -414,7 +421,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
                 const uint2 e = (i < nzw) ? src2[i] : make_uint2(0u, 0u);
                 const int c = __popc(e.x);
                 const int incl = warp_incl_scan(c);
-                if (i < nzw && e.y < (unsigned)nw) { bits[e.y] = e.x; rank[e.y] = (unsigned short)(carry + incl - c); }
+                if (i < nzw && e.y < (unsigned)nw) { const unsigned at = bank_spread<SPREAD>(e.y); bits[at] = e.x; rank[at] = (unsigned short)(carry + incl - c); }
                 carry += __shfl_sync(0xffffffffu, incl, 31);
             }
         } else {
@@ -424,7 +431,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
                 const unsigned word = (w < nw) ? src[w] : 0u;
                 const int c = __popc(word);
                 const int incl = warp_incl_scan(c);
-                if (w < nw) { bits[w] = word; rank[w] = (unsigned short)(src[nw + (w0 >> 5)] + (unsigned)(incl - c)); }
+                if (w < nw) { const unsigned at = bank_spread<SPREAD>(w); bits[at] = word; rank[at] = (unsigned short)(src[nw + (w0 >> 5)] + (unsigned)(incl - c)); }
             }
         }
         if (!CEIL)
@@ -436,7 +443,8 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
             if (CEIL) {
                 if (rel != 0xffffffffu) { my_idx += (u64)(rel + (unsigned)base); my_val += (double)prod; }
             } else if (rel < span) {
-                const int at_ = (int)rank[rel >> 5] + __popc(bits[rel >> 5] & ((1u << (rel & 31)) - 1u));
+                const unsigned w = bank_spread<SPREAD>(rel >> 5);
+                const int at_ = (int)rank[w] + __popc(bits[w] & ((1u << (rel & 31)) - 1u));
                 if (at_ < accw) {
                     if (shared_slot) atomicAdd(&acc[at_], prod);
                     else acc[at_] = add_rn(acc[at_], prod);
@@ -508,8 +516,9 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
                 const uint2 e = src2[i];
                 if (e.y >= (unsigned)nw) continue;
                 unsigned word = e.x;
-                i64 o = out0 + rank[e.y];
-                bits[e.y] = 0u;
+                const unsigned at = bank_spread<SPREAD>(e.y);
+                i64 o = out0 + rank[at];
+                bits[at] = 0u;
                 while (word) {
                     const int b = __ffs(word) - 1;
                     word &= word - 1;
@@ -518,9 +527,10 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
             }
         } else {
             for (int w = lane; w < nw; w += 32) {
-                unsigned word = bits[w];
-                i64 o = out0 + rank[w];
-                bits[w] = 0u;
+                const unsigned at = bank_spread<SPREAD>(w);
+                unsigned word = bits[at];
+                i64 o = out0 + rank[at];
+                bits[at] = 0u;
                 while (word) {
                     const int b = __ffs(word) - 1;
                     word &= word - 1;
@@ -621,23 +631,40 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
             if (U.nun == 1)                             // outputs beyond the shared-memory part start at zero
                 for (int x = CAP + tid; x < cnt; x += DN_THREADS) gacc[x] = 0;
             // the row's bitmap with the rank of every word's first bit (the symbolic pass saved the
-            // rank at every chunk start).  A warp takes eight chunks at a time, all loads first.
+            // rank at every chunk start).  A warp takes four groups of 128 words at a time, all loads first: one scan
+            // per group (a scan per chunk of 32 words: power law on 2^18 / 16381 vertices 12850 / 249 us, now 12650 / 239).
             const unsigned* src = tab.bm_arena + U.bm;
-            const int nw = U.nw, nch = chunks_of(nw);
-            for (int c0 = warp; c0 < nch; c0 += DN_WARPS * 8) {
-                unsigned word[8], rank_c[8];
+            const int nw = U.nw, nch = chunks_of(nw), ng = (nch + 3) >> 2;
+            const uint4* src4 = reinterpret_cast<const uint4*>(src);         // slots are 16-byte aligned
+            for (int g0 = warp; g0 < ng; g0 += DN_WARPS * 4) {
+                uint4 word[4];
+                unsigned rank_g[4];
 #pragma unroll
-                for (int x = 0; x < 8; ++x) {
-                    const int c = c0 + x * DN_WARPS, w = (c << 5) + lane;
-                    word[x] = (w < nw) ? src[w] : 0u;
-                    rank_c[x] = (c < nch) ? src[nw + c] : 0u;
+                for (int x = 0; x < 4; ++x) {
+                    const int g = g0 + x * DN_WARPS, w0 = (g << 7) + (lane << 2);
+                    word[x] = make_uint4(0u, 0u, 0u, 0u);
+                    if (w0 < nw) {
+                        word[x] = src4[(g << 5) + lane];
+                        if (w0 + 1 >= nw) word[x].y = 0u;
+                        if (w0 + 2 >= nw) word[x].z = 0u;
+                        if (w0 + 3 >= nw) word[x].w = 0u;
+                    }
+                    rank_g[x] = (g < ng) ? src[nw + (g << 2)] : 0u;
                 }
 #pragma unroll
-                for (int x = 0; x < 8; ++x) {
-                    const int c = c0 + x * DN_WARPS, w = (c << 5) + lane;
-                    const int pc = __popc(word[x]);
-                    const int incl = warp_incl_scan(pc);
-                    if (w < nw) bmr[w] = make_uint2(word[x], rank_c[x] + (unsigned)(incl - pc) - 1u);
+                for (int x = 0; x < 4; ++x) {
+                    const int g = g0 + x * DN_WARPS, w0 = (g << 7) + (lane << 2);
+                    const int p0 = __popc(word[x].x), p1 = p0 + __popc(word[x].y), p2 = p1 + __popc(word[x].z), p3 = p2 + __popc(word[x].w);
+                    const unsigned r = rank_g[x] + (unsigned)(warp_incl_scan(p3) - p3) - 1u;
+                    const uint4 lo = make_uint4(word[x].x, r, word[x].y, r + (unsigned)p0);
+                    const uint4 hi = make_uint4(word[x].z, r + (unsigned)p1, word[x].w, r + (unsigned)p2);
+                    // (lanes 4 .. 7 of eight store their second half first: no bank conflict)
+                    if (w0 < smem_words) {
+                        uint4* to = reinterpret_cast<uint4*>(bmr + w0);
+                        const bool second = lane & 4;
+                        to[second] = second ? hi : lo;
+                        to[!second] = second ? lo : hi;
+                    }
                 }
             }
         }
@@ -793,7 +820,8 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
 // are half full on average, every lane expands its own words into a small shared-memory stage at
 // their ranks and the stage goes out with contiguous stores; otherwise the warp takes one word
 // per step with a lane per bit.  Bound by instruction issue, most of it the expansion: 1.25e9 coordinates, 2.3
-// to a word, 3760 us taking a word's bits from the lowest, 3600 us from the highest.
+// to a word, 3760 us taking a word's bits from the lowest, 3640 us from the highest, 3510 us with one reduction for the four
+// ballots (a lane per output, which finds its word among flagged first outputs, 3656 us).
 constexpr int DE_THREADS = 256;
 constexpr int DE_WARPS = DE_THREADS / 32;
 constexpr int DE_STAGE = 2048;       // coordinates a warp stages at once (128 words, 16 bits each on average)
@@ -802,11 +830,12 @@ template <typename T>
 __global__ void __launch_bounds__(DE_THREADS) dense_emit_crd_kernel(DevCtl* __restrict__ ctl, i64 unit_products, RowTables tab,
                                                                     const i64* __restrict__ rowptr, int* __restrict__ Ccrd,
                                                                     T* __restrict__ Cval) {
-    __shared__ unsigned short s_stage[DE_WARPS][DE_STAGE];
+    __shared__ __align__(16) unsigned short s_stage[DE_WARPS][DE_STAGE];
     if (ctl->status != 0) return;
     const int n_units = ctl->n_units;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned short* stage = s_stage[warp];
+    unsigned short* const stage = s_stage[warp];
+    uint2* const list = reinterpret_cast<uint2*>(stage);                 // (a group uses one or the other)
     for (;;) {
         int u = 0;
         if (lane == 0) u = atomicAdd(&ctl->work_counter[EMIT_SLOT], 1);
@@ -852,9 +881,7 @@ __global__ void __launch_bounds__(DE_THREADS) dense_emit_crd_kernel(DevCtl* __re
                 const int p = __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
                 const int e = warp_incl_scan(p) - p;
                 const i64 o = out0 + r0;
-                const unsigned m0 = __ballot_sync(0xffffffffu, w.x != 0u), m1 = __ballot_sync(0xffffffffu, w.y != 0u);
-                const unsigned m2 = __ballot_sync(0xffffffffu, w.z != 0u), m3 = __ballot_sync(0xffffffffu, w.w != 0u);
-                const int nzw = __popc(m0) + __popc(m1) + __popc(m2) + __popc(m3);
+                const int nzw = (int)__reduce_add_sync(0xffffffffu, (unsigned)((w.x != 0u) + (w.y != 0u) + (w.z != 0u) + (w.w != 0u)));
                 if (n <= DE_STAGE && n < 16 * nzw) {
                     // every lane expands its own four words into the stage at their ranks (as 16-bit
                     // offsets from the group's first column), then the stage goes out with
@@ -876,21 +903,24 @@ __global__ void __launch_bounds__(DE_THREADS) dense_emit_crd_kernel(DevCtl* __re
                     for (int y = lane; y < n; y += 32) Ccrd[o + y] = gcol0 + (int)stage[y];
                     __syncwarp();
                 } else {
-                    // half-full words or fuller: the warp expands one non-empty word per step, lane
-                    // b testing bit b, so the word's outputs leave as one contiguous store
+                    // half-full words or fuller: the warp expands a word per step, lane b testing bit b, so the
+                    // word's outputs leave as one contiguous store.  The words and their ranks go through shared memory: one
+                    // broadcast load a word, empty ones among them, where taking turns among the lanes with words cost two
+                    // shuffles and a search (10^4 rows of 6500 outputs on 313 words: 162 -> 74 us).
+                    const unsigned e1 = (unsigned)(e + __popc(w.x)), e2 = e1 + (unsigned)__popc(w.y), e3 = e2 + (unsigned)__popc(w.z);
+                    uint4* const mine = reinterpret_cast<uint4*>(list + (lane << 2));
+                    mine[0] = make_uint4(w.x, (unsigned)e, w.y, e1);
+                    mine[1] = make_uint4(w.z, e2, w.w, e3);
+                    __syncwarp();
                     const unsigned below = (1u << lane) - 1u;
-                    const int gcol = base + (g << 12) + lane;
-                    auto spread = [&](unsigned mine, int rank_mine, unsigned m, int x) {
-                        while (m) {
-                            const int L = __ffs(m) - 1;
-                            m &= m - 1;
-                            const unsigned word = __shfl_sync(0xffffffffu, mine, L);
-                            const int at = __shfl_sync(0xffffffffu, rank_mine, L);
-                            if ((word >> lane) & 1u) Ccrd[o + at + __popc(word & below)] = gcol + (((L << 2) + x) << 5);
-                        }
-                    };
-                    const int e1 = e + __popc(w.x), e2 = e1 + __popc(w.y), e3 = e2 + __popc(w.z);
-                    spread(w.x, e, m0, 0); spread(w.y, e1, m1, 1); spread(w.z, e2, m2, 2); spread(w.w, e3, m3, 3);
+                    const int words = min(128, nw - (g << 7));
+                    int col = base + (g << 12) + lane;
+#pragma unroll 4
+                    for (int x = 0; x < words; ++x, col += 32) {
+                        const uint2 d = list[x];
+                        if ((d.x >> lane) & 1u) Ccrd[o + d.y + __popc(d.x & below)] = col;
+                    }
+                    __syncwarp();
                 }
                 if (clear)
                     for (int y = lane; y < n; y += 32) Cval[o + y] = (T)0;
@@ -929,10 +959,10 @@ cudaError_t launch_dense_sym_cta(const LaunchCtx& c, const Csr& A, const Csr& B)
     return cudaGetLastError();
 }
 
-template <typename T, bool CEIL>
+template <typename T, bool CEIL, bool SPREAD>
 static cudaError_t num_warp_t(const LaunchCtx& c, const int* n, const int* max_cnt, int m, int bmw, const Csr& A, const Csr& B, const i64* rowptr,
                               int* Ccrd, void* Cval, u64* chk_idx, double* chk_val) {
-    auto k = dense_num_warp_kernel<T, CEIL>;
+    auto k = dense_num_warp_kernel<T, CEIL, SPREAD>;
     const int* const rows[N_WARP_LISTS] = {c.tab.warp_rows, c.tab.warp_rows + m - 1};
     for (int list = N_WARP_LISTS - 1; list >= 0; --list) {          // the longest rows first
         if (n[list] == 0) continue;
@@ -965,10 +995,12 @@ cudaError_t launch_dense_num_warp(const LaunchCtx& c, const int* n, const int* m
     int bmw = max_span_words > 0 ? ((max_span_words + 31) & ~31) : DENSE_WARP_BM_WORDS;
     if (bmw > DENSE_WARP_BM_WORDS) bmw = DENSE_WARP_BM_WORDS;
     if (chk_idx)      // same launch shape (shared memory reserved, hence occupancy) as the full kernel
-        return c.is_f64 ? num_warp_t<double, true>(c, n, max_cnt, m, bmw, A, B, rowptr, Ccrd, Cval, chk_idx, chk_val)
-                        : num_warp_t<float, true>(c, n, max_cnt, m, bmw, A, B, rowptr, Ccrd, Cval, chk_idx, chk_val);
-    return c.is_f64 ? num_warp_t<double, false>(c, n, max_cnt, m, bmw, A, B, rowptr, Ccrd, Cval, nullptr, nullptr)
-                    : num_warp_t<float, false>(c, n, max_cnt, m, bmw, A, B, rowptr, Ccrd, Cval, nullptr, nullptr);
+        return c.is_f64 ? num_warp_t<double, true, false>(c, n, max_cnt, m, bmw, A, B, rowptr, Ccrd, Cval, chk_idx, chk_val)
+                        : num_warp_t<float, true, false>(c, n, max_cnt, m, bmw, A, B, rowptr, Ccrd, Cval, chk_idx, chk_val);
+    const bool spread = bmw > DW_SCAN_WORDS;
+    auto go = c.is_f64 ? (spread ? num_warp_t<double, false, true> : num_warp_t<double, false, false>)
+                       : (spread ? num_warp_t<float, false, true> : num_warp_t<float, false, false>);
+    return go(c, n, max_cnt, m, bmw, A, B, rowptr, Ccrd, Cval, nullptr, nullptr);
 }
 
 template <typename T, bool CEIL>
