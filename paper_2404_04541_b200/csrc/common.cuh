@@ -12,9 +12,9 @@ constexpr int NCLASS = 15;
 // Row classes = the workspace a row (or (i,j) fibre) is routed to in the symbolic pass.
 enum RowClass : int {
     CLS_EMPTY = 0,      // no intermediate product
-    CLS_ISM_REG8 = 1,   // insert-sort-merge in registers, 8 lanes per row (<= 8 products)
-    CLS_ISM_REG16 = 2,  // ... 16 lanes per row (<= 16 products)
-    CLS_ISM_REG = 3,    // ... one warp per row (<= 32 products)
+    CLS_ISM_REG8 = 1,   // insert-sort-merge by 4 lanes per row, two words per lane (<= 8 products)
+    CLS_ISM_REG16 = 2,  // ... four words per lane (<= 16 products)
+    CLS_ISM_REG = 3,    // ... six or eight words per lane (<= 32 products)
     CLS_ISM_SMEM_S = 4, // insert-sort-merge of 129 .. 256 products, one warp per row
     CLS_ISM_SMEM = 5,   // insert-sort-merge in shared memory, full CTA
     CLS_DENSE_WARP = 6, // dense workspace (occupancy bitmap), one warp per row
@@ -415,13 +415,25 @@ size_t look_words(i64 rows, i64 slices);
 // exclusive scan of n counts into n + 1 positions
 cudaError_t launch_scan_counts(const LaunchCtx& c, const int* cnt, int n, i64* out, i64* block_sums, i64* total_out);
 // class kernels: n_host < 0 means "size the grid for any count"
-// rows[cls] = rows of the three register classes and of the copied class, in ONE launch
-cudaError_t launch_ism_reg(const LaunchCtx& c, bool numeric, const i64* rows, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval);
+cudaError_t launch_copy_rows(const LaunchCtx& c, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval);
+// The insert-sort-merge rows of up to smem_cap products by the kernels that take them: 4, 8 or 16 lanes per row (at most 32, 64 or
+// 128 products), a warp per row (256), the kernels of the full class.
+constexpr int ISM_LEVELS = 5;
+struct RowRanges { const int* rows[ISM_LEVELS]; int end[ISM_LEVELS]; };       // rows of several classes one after the other
+__device__ __forceinline__ int row_at(const RowRanges& g, int r) {
+    int row = r < g.end[0] ? __ldg(g.rows[0] + r) : -1;
+#pragma unroll
+    for (int k = 1; k < ISM_LEVELS; ++k)
+        if (r >= g.end[k - 1] && r < g.end[k]) row = __ldg(g.rows[k] + (r - g.end[k - 1]));
+    return row;
+}
+struct IsmLaunch { int level; RowRanges g; };
+// the launches for the rows as binned (at most ISM_LEVELS); returns their number
+int ism_launches(const LaunchCtx& c, IsmLaunch* out);
+cudaError_t launch_ism(const LaunchCtx& c, bool numeric, const IsmLaunch& l, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval);
 // scratch that keeps the sorted words of the rows of the warp-per-row ISM from the counting pass to the numeric one;
 // words: DevCtl::order_words, max_products: of a CLS_ISM_SMEM row
 size_t order_bytes_of(i64 words, i64 max_products, i64 ncols);
-cudaError_t launch_ism_smem(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B,
-                            const i64* rowptr, int* Ccrd, void* Cval);
 // max_span_words: widest dense row of the pass
 cudaError_t launch_dense_sym_warp(const LaunchCtx& c, int max_span_words, const Csr& A, const Csr& B);
 cudaError_t launch_dense_sym_cta(const LaunchCtx& c, const Csr& A, const Csr& B);

@@ -1,4 +1,4 @@
-// Insert-sort-merge workspace of mid-size rows: 8 or 16 lanes per output row of at most 64 or 128 products, a warp per row of
+// Insert-sort-merge workspace: 4, 8 or 16 lanes per output row of at most 32, 64 or 128 products, a warp per row of
 // at most 1024, a CTA per row beyond (Algorithm 1; the accumulation array is shared memory and is never full because
 // the symbolic upper bound sized it; coordinate-sort policy, Sec. 5.2).
 //   Insert : product t of the row (loop order k, then j) is appended at slot t: its value stays
@@ -289,17 +289,18 @@ __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int to
 }
 
 // ---------------------------------------------------------------------------------------
-// Rows of at most 64 or 128 products: G = 8 or 16 lanes per row, eight products per lane at most, so that a warp works on four
-// or two of them at a time.
+// Rows of at most 32, 64 or 128 products: G = 4, 8 or 16 lanes per row, eight products per lane at most, so that a warp works
+// on eight, four or two of them at a time.
 //   Insert : G entries at a time; lane l takes the products l, l + G, .. of those entries, whose owners it finds by a search
 //            among the running counts.
-//   Sort   : six or eight words per lane in registers; the narrower the group, the more of the network stays inside the lanes.
+//   Sort   : six or eight words per lane in registers (two or four where no row of a warp of four-lane groups has more); the narrower the group, the more of the network stays inside the lanes.
 //   Merge  : as below: the sorted words and the places of the run heads go to shared memory, a lane per run.
 // Every step of the way to a row's products is a load that waits for the one before: several rows per warp and some 40 warps
 // keep enough of them in flight, and a block for every 128 lanes' rows spares fetching ahead (persistent blocks: numeric 80 us
 // where these take 75).  Bound by the integer pipe (half of the instructions, a warp every two cycles).  A warp per row
 // against this, count + numeric: 2e5 rows of 59 products, f32, 123 + 148 and 92 + 128 us; 1.6e5 fibres of 110, 95 + 108 and 64 + 93
-// us; 1.9e5 rows of 82, f64, 137 + 178 and 99 + 144 us.
+// us; 1.9e5 rows of 82, f64, 137 + 178 and 99 + 144 us.  Rows of at most 32 products had as many lanes as products before: 1.2e5
+// rows of 16 .. 24, f64, 22 + 45 and 12 + 40 us; 65536 rows of 16 whose B rows come from memory, 18 + 25 and 16 + 26 us.
 // ---------------------------------------------------------------------------------------
 constexpr int IG_THREADS = 128;
 
@@ -352,7 +353,7 @@ __device__ __forceinline__ int sort_group(P* packed, unsigned char* heads, int t
 }
 
 template <typename T, typename P, int G, bool NUMERIC>
-__global__ void __launch_bounds__(IG_THREADS, (group_blocks<T, P, NUMERIC>())) ism_group_kernel(const int* __restrict__ rows, int n, const DevCtl* __restrict__ ctl,
+__global__ void __launch_bounds__(IG_THREADS, (group_blocks<T, P, NUMERIC>())) ism_group_kernel(RowRanges g, int n, const DevCtl* __restrict__ ctl,
                                                                                                Csr A, Csr B, int* __restrict__ cnt,
                                                                                                const i64* __restrict__ rowptr, int* __restrict__ Ccrd,
                                                                                                T* __restrict__ Cval) {
@@ -373,7 +374,7 @@ __global__ void __launch_bounds__(IG_THREADS, (group_blocks<T, P, NUMERIC>())) i
     int row = 0;
     i64 ps = 0, pe = 0;
     if (r < n) {
-        row = __ldg(rows + r);
+        row = row_at(g, r);
         ps = __ldg(A.pos + row);
         pe = __ldg(A.pos + row + 1);
     }
@@ -437,7 +438,10 @@ __global__ void __launch_bounds__(IG_THREADS, (group_blocks<T, P, NUMERIC>())) i
     }
     // ---- Sort
     int distinct;
-    if (__any_sync(0xffffffffu, total > 6 * G)) distinct = sort_group<PK, P, 8, G, NUMERIC>(packed, heads, total, gl);
+    const int longest = __reduce_max_sync(0xffffffffu, total);
+    if (G == 4 && longest <= 2 * G) distinct = sort_group<PK, P, 2, G, NUMERIC>(packed, heads, total, gl);
+    else if (G == 4 && longest <= 4 * G) distinct = sort_group<PK, P, 4, G, NUMERIC>(packed, heads, total, gl);
+    else if (longest > 6 * G) distinct = sort_group<PK, P, 8, G, NUMERIC>(packed, heads, total, gl);
     else distinct = sort_group<PK, P, 6, G, NUMERIC>(packed, heads, total, gl);
     // ---- Merge
     if (r < n) {
@@ -465,7 +469,7 @@ constexpr int iw_blocks() {
 }
 
 template <typename T, typename P, int CAP, bool NUMERIC>
-__global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>())) ism_warp_kernel(const int* __restrict__ perm, DevCtl* __restrict__ ctl, int cls, int counter_slot,
+__global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>())) ism_warp_kernel(RowRanges rows, int n, int n_kept, DevCtl* __restrict__ ctl, int counter_slot,
                                                                  Csr A, Csr B, const i64* __restrict__ ub, i64* __restrict__ order_off, char* order_arena,
                                                                  size_t order_bytes, int* __restrict__ cnt,
                                                                  const i64* __restrict__ rowptr, int* __restrict__ Ccrd, T* __restrict__ Cval, int launch_slots) {
@@ -479,8 +483,6 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
     P* const packed = reinterpret_cast<P*>(smem_raw + (NUMERIC ? (int)sizeof(T) * slots * IW_WARPS : 0)) + warp * padded_slots;
     unsigned short* const heads = reinterpret_cast<unsigned short*>(smem_raw + ((NUMERIC ? (int)sizeof(T) * slots : 0) + (int)sizeof(P) * padded_slots) * IW_WARPS) + warp * slots;
     if (ctl->status != 0) return;
-    int off, n;
-    class_range(ctl, cls, off, n);
     const T* __restrict__ Aval = (const T*)A.val;
     const T* __restrict__ Bval = (const T*)B.val;
     // The way to a row is a chain of loads (its number, its place in perm, its fields, its A entries, their B rows).  AHEAD:
@@ -490,7 +492,8 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
     constexpr bool AHEAD = NUMERIC && (CAP > 256 || sizeof(T) == 8);
     int row, row_n = -1, products, products_n = 0;
     i64 ps, pe, ps_n = 0, pe_n = 0;
-    auto take = [&](int r) { row_n = r < n ? __ldg(perm + off + r) : -1; };
+    bool kept = false, kept_n = false;              // a row of the class that leaves its order (they come first)
+    auto take = [&](int r) { row_n = r < n ? row_at(rows, r) : -1; kept_n = r < n_kept; };
     auto fields = [&]() {
         if (row_n < 0) return;
         products_n = (int)min(__ldg(ub + row_n), (i64)0x7fffffff);
@@ -508,6 +511,7 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
         if (!AHEAD) next();
         if (row_n < 0) break;
         row = row_n;
+        kept = kept_n;
         products = products_n;
         ps = ps_n;
         pe = pe_n;
@@ -518,7 +522,7 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
         int r_n = 0;
         if (AHEAD && lane == 0) r_n = atomicAdd(&ctl->work_counter[counter_slot], 1);
         P* order = nullptr;
-        if (CAP > 256 && order_arena) {
+        if (CAP > 256 && order_arena && kept) {
             i64 at = -1;
             if (NUMERIC) {
                 at = order_off[row];
@@ -586,7 +590,7 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
         const int e = words_per_lane<CAP>(total);
         if (total != products) order = nullptr;             // (a malformed B row)
         P* const keep = CAP > 256 ? order : nullptr;
-        if (CAP > 256 && !NUMERIC && order_arena && lane == 0) order_off[row] = order ? (i64)(reinterpret_cast<char*>(order) - order_arena) : -1;
+        if (CAP > 256 && !NUMERIC && order_arena && kept && lane == 0) order_off[row] = order ? (i64)(reinterpret_cast<char*>(order) - order_arena) : -1;
         if constexpr (CAP <= 256) {
             switch (e) {
                 case 4: distinct = sort_row<PK, P, 4, NUMERIC>(packed, heads, total, keep); break;
@@ -646,7 +650,7 @@ static cudaError_t launch_k(const LaunchCtx& c, int cls, int n_host, const Csr& 
 }
 
 template <typename T, typename P, int CAP, bool NUMERIC>
-static cudaError_t launch_warp_k(const LaunchCtx& c, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
+static cudaError_t launch_warp_k(const LaunchCtx& c, const IsmLaunch& l, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
     // room for the largest row of the launch, where it is known: more warps fit (numeric, 8e4 rows of up to 729 products,
     // f32: 345 us at 1024 slots, 312 us at 768 and seven blocks per SM; f64 435 -> 299 us)
     const int slots = CAP > 256 && c.max_ub_smem > 0 && c.max_ub_smem < CAP ? 32 * words_per_lane<CAP>((int)c.max_ub_smem) : CAP;
@@ -656,9 +660,10 @@ static cudaError_t launch_warp_k(const LaunchCtx& c, int cls, int n_host, const 
     auto k = ism_warp_kernel<T, P, CAP, NUMERIC>;
     if ((e = resident_blocks((const void*)k, IW_WARPS * 32, smem, &per_sm)) != cudaSuccess) return e;
     i64 grid = (i64)c.sm_count * (per_sm > 0 ? per_sm : 1);
-    const i64 want = n_host >= 0 ? ((i64)n_host + IW_WARPS - 1) / IW_WARPS : grid;
+    const int n = l.g.end[ISM_LEVELS - 1], cls = l.level == 4 ? CLS_ISM_SMEM : CLS_ISM_SMEM_S;
+    const i64 want = ((i64)n + IW_WARPS - 1) / IW_WARPS;
     if (want < grid) grid = want > 0 ? want : 1;
-    k<<<(int)grid, IW_WARPS * 32, smem, c.stream>>>(c.tab.perm, c.ctl, cls, cls + (NUMERIC ? NUM_SLOT : 0), A, B, c.tab.ub, c.tab.bm_off, c.order,
+    k<<<(int)grid, IW_WARPS * 32, smem, c.stream>>>(l.g, n, l.g.end[0], c.ctl, cls + (NUMERIC ? NUM_SLOT : 0), A, B, c.tab.ub, c.tab.bm_off, c.order,
                                                     c.order_bytes, c.tab.cnt, rowptr, Ccrd, (T*)Cval, slots);
     ++c.launches;
     return cudaGetLastError();
@@ -674,62 +679,87 @@ size_t order_bytes_of(i64 words, i64 max_products, i64 ncols) {
 }
 
 template <typename T, typename P, int G, bool NUMERIC>
-static cudaError_t launch_group_k(const LaunchCtx& c, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
+static cudaError_t launch_group_k(const LaunchCtx& c, const IsmLaunch& l, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
     constexpr int ROWS = IG_THREADS / G;
-    i64 off = 0;
-    for (int x = 0; x < cls; ++x) off += c.class_rows[x];
-    ism_group_kernel<T, P, G, NUMERIC><<<(n_host + ROWS - 1) / ROWS, IG_THREADS, 0, c.stream>>>(c.tab.perm + off, n_host, c.ctl, A, B, c.tab.cnt, rowptr, Ccrd,
-                                                                                             (T*)Cval);
+    const int n = l.g.end[ISM_LEVELS - 1];
+    ism_group_kernel<T, P, G, NUMERIC><<<(int)(((i64)n + ROWS - 1) / ROWS), IG_THREADS, 0, c.stream>>>(l.g, n, c.ctl, A, B, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
     ++c.launches;
     return cudaGetLastError();
 }
 
 template <typename T, int G>
-static cudaError_t launch_group(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd,
-                                void* Cval) {
+static cudaError_t launch_group(const LaunchCtx& c, bool numeric, const IsmLaunch& l, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
     // (the count does not depend on the value type)
     if (narrow<8 * G>(B))
-        return numeric ? launch_group_k<T, unsigned, G, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
-                       : launch_group_k<float, unsigned, G, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
-    return numeric ? launch_group_k<T, u64, G, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
-                   : launch_group_k<float, u64, G, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
+        return numeric ? launch_group_k<T, unsigned, G, true>(c, l, A, B, rowptr, Ccrd, Cval)
+                       : launch_group_k<float, unsigned, G, false>(c, l, A, B, rowptr, Ccrd, Cval);
+    return numeric ? launch_group_k<T, u64, G, true>(c, l, A, B, rowptr, Ccrd, Cval)
+                   : launch_group_k<float, u64, G, false>(c, l, A, B, rowptr, Ccrd, Cval);
 }
 
 template <typename T, int CAP>
-static cudaError_t launch_warp(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd,
-                               void* Cval) {
+static cudaError_t launch_warp(const LaunchCtx& c, bool numeric, const IsmLaunch& l, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
     if (narrow<CAP>(B))
-        return numeric ? launch_warp_k<T, unsigned, CAP, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
-                       : launch_warp_k<T, unsigned, CAP, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
-    return numeric ? launch_warp_k<T, u64, CAP, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
-                   : launch_warp_k<T, u64, CAP, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
+        return numeric ? launch_warp_k<T, unsigned, CAP, true>(c, l, A, B, rowptr, Ccrd, Cval)
+                       : launch_warp_k<T, unsigned, CAP, false>(c, l, A, B, rowptr, Ccrd, Cval);
+    return numeric ? launch_warp_k<T, u64, CAP, true>(c, l, A, B, rowptr, Ccrd, Cval)
+                   : launch_warp_k<T, u64, CAP, false>(c, l, A, B, rowptr, Ccrd, Cval);
 }
 
 template <typename T>
-static cudaError_t launch_t(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B,
-                            const i64* rowptr, int* Ccrd, void* Cval) {
-    if (cls == CLS_ISM_GROUP8) return launch_group<T, 8>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
-    if (cls == CLS_ISM_GROUP16) return launch_group<T, 16>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
+static cudaError_t launch_t(const LaunchCtx& c, bool numeric, const IsmLaunch& l, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
+    if (l.level == 0) return launch_group<T, 4>(c, numeric, l, A, B, rowptr, Ccrd, Cval);
+    if (l.level == 1) return launch_group<T, 8>(c, numeric, l, A, B, rowptr, Ccrd, Cval);
+    if (l.level == 2) return launch_group<T, 16>(c, numeric, l, A, B, rowptr, Ccrd, Cval);
     // (the full class when its largest row is that small: fewer registers and less shared memory per warp)
-    i64 most = cls == CLS_ISM_SMEM_S ? 256 : c.prm.smem_cap;
-    if (cls == CLS_ISM_SMEM && c.max_ub_smem > 0 && c.max_ub_smem < most) most = c.max_ub_smem;
-    if (most <= 256) return launch_warp<T, 256>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
-    cudaError_t e = launch_warp<T, ISM_WARP_MAX>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
+    i64 most = l.level == 3 ? 256 : c.prm.smem_cap;
+    if (l.level == 4 && c.max_ub_smem > 0 && c.max_ub_smem < most) most = c.max_ub_smem;
+    if (most <= 256) return launch_warp<T, 256>(c, numeric, l, A, B, rowptr, Ccrd, Cval);
+    cudaError_t e = launch_warp<T, ISM_WARP_MAX>(c, numeric, l, A, B, rowptr, Ccrd, Cval);
     if (e != cudaSuccess || most <= ISM_WARP_MAX) return e;
     // rows of 1025 .. 4096 products: a CTA each (a counter of their own: the two kernels share the class);
     // under `auto` they are counted through a hash set of their columns, which needs no order
-    if (!numeric && c.prm.policy == 2) return launch_hash(c, false, CLS_ISM_SMEM, n_host, A, B, rowptr, Ccrd, Cval);
+    const int n = l.g.end[0];
+    if (!numeric && c.prm.policy == 2) return launch_hash(c, false, CLS_ISM_SMEM, n, A, B, rowptr, Ccrd, Cval);
     if (narrow<4096>(B))
-        return numeric ? launch_k<T, unsigned, 4096, 256, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
-                       : launch_k<T, unsigned, 4096, 256, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
-    return numeric ? launch_k<T, u64, 4096, 256, true>(c, cls, n_host, A, B, rowptr, Ccrd, Cval)
-                   : launch_k<T, u64, 4096, 256, false>(c, cls, n_host, A, B, rowptr, Ccrd, Cval);
+        return numeric ? launch_k<T, unsigned, 4096, 256, true>(c, CLS_ISM_SMEM, n, A, B, rowptr, Ccrd, Cval)
+                       : launch_k<T, unsigned, 4096, 256, false>(c, CLS_ISM_SMEM, n, A, B, rowptr, Ccrd, Cval);
+    return numeric ? launch_k<T, u64, 4096, 256, true>(c, CLS_ISM_SMEM, n, A, B, rowptr, Ccrd, Cval)
+                   : launch_k<T, u64, 4096, 256, false>(c, CLS_ISM_SMEM, n, A, B, rowptr, Ccrd, Cval);
 }
 
-cudaError_t launch_ism_smem(const LaunchCtx& c, bool numeric, int cls, int n_host, const Csr& A, const Csr& B,
-                            const i64* rowptr, int* Ccrd, void* Cval) {
-    return c.is_f64 ? launch_t<double>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval)
-                    : launch_t<float>(c, numeric, cls, n_host, A, B, rowptr, Ccrd, Cval);
+cudaError_t launch_ism(const LaunchCtx& c, bool numeric, const IsmLaunch& l, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
+    return c.is_f64 ? launch_t<double>(c, numeric, l, A, B, rowptr, Ccrd, Cval) : launch_t<float>(c, numeric, l, A, B, rowptr, Ccrd, Cval);
+}
+
+// A kernel takes any row with fewer products than its own as well, at more instructions a row, and a launch for a handful of rows
+// costs 4 .. 10 us: no more than ISM_FEW rows go along with those of the next larger kernel that has rows of its own (stencil
+// 41 x 37 x 53, 3e3 rows at its edges: a call 824 us with a launch for each class, 796 us).
+constexpr i64 ISM_FEW = 2048;
+int ism_launches(const LaunchCtx& c, IsmLaunch* out) {
+    const i64* const rows = c.class_rows;
+    auto first = [&](int cls) { i64 off = 0; for (int k = 0; k < cls; ++k) off += rows[k]; return c.tab.perm + off; };
+    const i64 n[ISM_LEVELS] = {rows[CLS_ISM_REG8] + rows[CLS_ISM_REG16] + rows[CLS_ISM_REG], rows[CLS_ISM_GROUP8], rows[CLS_ISM_GROUP16], rows[CLS_ISM_SMEM_S],
+                               rows[CLS_ISM_SMEM]};
+    const int cls[ISM_LEVELS] = {CLS_ISM_REG8, CLS_ISM_GROUP8, CLS_ISM_GROUP16, CLS_ISM_SMEM_S, CLS_ISM_SMEM};
+    int made = 0;
+    bool taken[ISM_LEVELS] = {};
+    for (int at = ISM_LEVELS - 1; at >= 0; --at) {
+        if (n[at] == 0 || taken[at]) continue;
+        // this level's own rows first, then those of lower levels that are few
+        IsmLaunch& l = out[made++];
+        l.level = at;
+        int k = 0;
+        i64 end = 0;
+        for (int from = at; from >= 0 && (from == at || n[from] <= ISM_FEW); --from) {
+            if (n[from] == 0) continue;
+            taken[from] = true;
+            l.g.rows[k] = first(cls[from]);
+            l.g.end[k++] = (int)(end += n[from]);
+        }
+        for (; k < ISM_LEVELS; ++k) { l.g.rows[k] = l.g.rows[0]; l.g.end[k] = (int)end; }
+    }
+    return made;
 }
 
 }  // namespace spws

@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
         if (u > 0) lo &= ~31;               // bitmap words of every row start at a multiple of 32 columns
         const int cls = classify_row(u, entries, lo, hi, prm, ctl);
         tab.ub[row] = u;
-        if (cls != CLS_COPY && cls != CLS_EMPTY) {      // (nothing reads the span of these)
+        if (dense_cls(cls)) {                           // (nothing reads the span of the others)
             tab.jmin[row] = lo;
             tab.jmax[row] = hi;
         }

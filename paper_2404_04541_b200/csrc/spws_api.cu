@@ -176,7 +176,8 @@ struct spws_plan_s {
     void* scratch = nullptr;
     int max_span_words = 0;     // widest dense bitmap of the last symbolic pass
     int64_t row_products = 0;   // products of all its rows as the device counted them (stats.products may count a form's own way)
-    int64_t sparse_products = 0;                // products of the rows its sparse workspaces take
+    int64_t sparse_products = 0;                // products of the rows its sparse workspaces take ...
+    int64_t copy_products = 0;                  // ... and of the rows it copies
     size_t order_off = 0, order_bytes = 0;      // where it left the sorted words of mid-size rows in the scratch (0 bytes: nowhere) ...
     size_t order_need = 0;      // ... and the scratch that holds them and all else the passes use
     size_t least = 0;           // scratch the last symbolic call could not do without, as far as it came (0: not known)
@@ -545,6 +546,9 @@ inline void mark(spws_plan_s* p, int group) {
 // timing groups of pass 0 (symbolic), 1 (numeric), 2 (gather-only ceiling)
 const int PASS_GROUPS[4] = {0, SPWS_T_NUM_ISM_REG, SPWS_T_CEIL_DENSE_WARP, SPWS_T_COUNT};
 
+// group of a level of the insert-sort-merge kernels
+const int ISM_GROUPS[ISM_LEVELS] = {SPWS_T_SYM_ISM_REG, SPWS_T_SYM_ISM_SMEM_S, SPWS_T_SYM_ISM_SMEM_S, SPWS_T_SYM_ISM_SMEM_S, SPWS_T_SYM_ISM_SMEM};
+
 inline void mark_start(spws_plan_s* p, int pass) {
     if (!p->profiling) return;
     const int g0 = PASS_GROUPS[pass], g1 = PASS_GROUPS[pass + 1];
@@ -700,7 +704,8 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     c.class_rows = hcount;
     const i64 products = hc.products;
     plan->sparse_products = 0;
-    for (int k : {CLS_COPY, CLS_ISM_REG8, CLS_ISM_REG16, CLS_ISM_REG, CLS_ISM_GROUP8, CLS_ISM_GROUP16, CLS_ISM_SMEM_S, CLS_ISM_SMEM}) plan->sparse_products += hc.class_products[k];
+    plan->copy_products = hc.class_products[CLS_COPY];
+    for (int k : {CLS_ISM_REG8, CLS_ISM_REG16, CLS_ISM_REG, CLS_ISM_GROUP8, CLS_ISM_GROUP16, CLS_ISM_SMEM_S, CLS_ISM_SMEM}) plan->sparse_products += hc.class_products[k];
     const bool any_dense = hcount[CLS_DENSE_WARP] + hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0;
     plan->max_ub_smem = hc.max_ub_smem;
     c.max_ub_smem = plan->max_ub_smem;
@@ -709,18 +714,11 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
         const bool dense_cta = hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0;
         Fork fork(plan, c, hcount[CLS_DENSE_WARP] > 0, dense_cta || hcount[CLS_ISM_GLOBAL] > 0);
         fork.group(0);
-        if (hcount[CLS_ISM_REG8] + hcount[CLS_ISM_REG16] + hcount[CLS_ISM_REG] > 0) {
-            CUDA_TRY(launch_ism_reg(c, false, hcount, S.A, S.B, rowptr, nullptr, nullptr));
-            mark(plan, SPWS_T_SYM_ISM_REG);
-        }
-        for (int cls : {CLS_ISM_GROUP8, CLS_ISM_GROUP16, CLS_ISM_SMEM_S})
-            if (hcount[cls] > 0) {
-                CUDA_TRY(launch_ism_smem(c, false, cls, (int)hcount[cls], S.A, S.B, rowptr, nullptr, nullptr));
-                mark(plan, SPWS_T_SYM_ISM_SMEM_S);
-            }
-        if (hcount[CLS_ISM_SMEM] > 0) {
-            CUDA_TRY(launch_ism_smem(c, false, CLS_ISM_SMEM, (int)hcount[CLS_ISM_SMEM], S.A, S.B, rowptr, nullptr, nullptr));
-            mark(plan, SPWS_T_SYM_ISM_SMEM);
+        IsmLaunch ism[ISM_LEVELS];
+        const int n_ism = ism_launches(c, ism);
+        for (int k = 0; k < n_ism; ++k) {
+            CUDA_TRY(launch_ism(c, false, ism[k], S.A, S.B, rowptr, nullptr, nullptr));
+            mark(plan, ISM_GROUPS[ism[k].level]);
         }
         fork.group(1);
         if (hcount[CLS_DENSE_WARP] > 0) {
@@ -812,20 +810,14 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, cha
     const spws_stats_t& s = plan->stats;
     const int64_t* bins = plan->bin_rows;
     c.class_rows = LL(bins);
-    Fork fork(plan, c, s.dense_warp_rows > 0, s.dense_units > 0 || bins[CLS_ISM_GLOBAL] > 0);
+    const bool copies = plan->copy_products >= FORK_PRODUCTS;
+    Fork fork(plan, c, s.dense_warp_rows > 0, copies || s.dense_units > 0 || bins[CLS_ISM_GLOBAL] > 0);
     fork.group(0);
-    if (bins[CLS_COPY] + bins[CLS_ISM_REG8] + bins[CLS_ISM_REG16] + bins[CLS_ISM_REG] > 0) {
-        CUDA_TRY(launch_ism_reg(c, true, LL(bins), S.A, S.B, rowptr, crd, val));
-        mark(plan, SPWS_T_NUM_ISM_REG);
-    }
-    for (int cls : {CLS_ISM_GROUP8, CLS_ISM_GROUP16, CLS_ISM_SMEM_S})
-        if (bins[cls] > 0) {
-            CUDA_TRY(launch_ism_smem(c, true, cls, (int)bins[cls], S.A, S.B, rowptr, crd, val));
-            mark(plan, SPWS_T_NUM_ISM_SMEM_S);
-        }
-    if (bins[CLS_ISM_SMEM] > 0) {
-        CUDA_TRY(launch_ism_smem(c, true, CLS_ISM_SMEM, (int)bins[CLS_ISM_SMEM], S.A, S.B, rowptr, crd, val));
-        mark(plan, SPWS_T_NUM_ISM_SMEM);
+    IsmLaunch ism[ISM_LEVELS];
+    const int n_ism = ism_launches(c, ism);
+    for (int k = 0; k < n_ism; ++k) {
+        CUDA_TRY(launch_ism(c, true, ism[k], S.A, S.B, rowptr, crd, val));
+        mark(plan, ISM_GROUPS[ism[k].level] + SPWS_T_NUM_ISM_REG - SPWS_T_SYM_ISM_REG);
     }
     fork.group(1);
     if (s.dense_warp_rows > 0) {
@@ -833,6 +825,10 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, cha
         mark(plan, SPWS_T_NUM_DENSE_WARP);
     }
     fork.group(2);
+    if (bins[CLS_COPY] > 0) {
+        CUDA_TRY(launch_copy_rows(c, S.A, S.B, rowptr, crd, val));
+        mark(plan, SPWS_T_NUM_ISM_REG);
+    }
     if (s.dense_units > 0) {
         CUDA_TRY(launch_dense_num_cta(c, 0, (int)s.dense_units, plan->max_span_words, plan->row_products, S.A, S.B, rowptr, crd, val));
         mark(plan, SPWS_T_NUM_DENSE_EMIT);
