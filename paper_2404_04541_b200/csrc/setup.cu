@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(256) bw_find_long_kernel(Csr B, int* __restric
     }
 }
 
-constexpr int BWB_THREADS = 256;
+constexpr int BWB_THREADS = 1024;     // (the longest row sets the time: power law on 2^18 vertices 86 us with 256, 56 with 1024)
 constexpr int BWB_ITEMS = 4;
 
 __global__ void __launch_bounds__(BWB_THREADS) bw_build_kernel(Csr B, const int* __restrict__ bw_long, int cap,
@@ -551,7 +551,7 @@ cudaError_t launch_bw_build(const LaunchCtx& c, const Csr& B) {
     i64 want = ((i64)B.nrows + 255) / 256;
     i64 cap = (i64)c.sm_count * 8;
     bw_find_long_kernel<<<(int)(want < cap ? want : cap), 256, 0, c.stream>>>(B, c.bw_long, c.bw_long_cap, c.ctl);
-    bw_build_kernel<<<c.sm_count * 8, BWB_THREADS, 0, c.stream>>>(B, c.bw_long, c.bw_long_cap, c.bw, c.ctl);
+    bw_build_kernel<<<c.sm_count * 2, BWB_THREADS, 0, c.stream>>>(B, c.bw_long, c.bw_long_cap, c.bw, c.ctl);
     c.launches += 2;
     return cudaGetLastError();
 }
