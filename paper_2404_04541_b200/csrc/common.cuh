@@ -461,10 +461,11 @@ cudaError_t launch_coo_pos(const LaunchCtx& c, const u64* ukeys, i64 nnz, i64 m,
 cudaError_t launch_coo_out(const LaunchCtx& c, const u64* ukeys, const void* uvals, i64 nnz, i64 J, int* Ccrd, void* Cval);
 cudaError_t launch_outer_dense(const LaunchCtx& c, bool numeric, const Csr& At, const Csr& B, const i64* koff, i64 P, i64 m, i64 J,
                                unsigned* dbits, void* dvals, int* cnt, const i64* pos, int* Ccrd, void* Cval);
-// number of products; partial[0 .. 2 COUNT_BLOCKS) (pinned host memory, cleared by the caller) receives one sum per block
-cudaError_t launch_outer_total(const LaunchCtx& c, const Csr& At, const Csr& B, u64* partial);
+// number of products; partial[0 .. *blocks) (pinned host memory, cleared by the caller) receives one sum per block, plus one
+cudaError_t launch_outer_total(const LaunchCtx& c, const Csr& At, const Csr& B, u64* partial, int* blocks);
 // higher.cu: the higher-order scatters with coordinate-form output
-cudaError_t launch_higher_total(const LaunchCtx& c, int form, const Csf3Dev& B, const Csr& C, u64* partial);
+// (and partial[COUNT_BLOCKS ..] another)
+cudaError_t launch_higher_total(const LaunchCtx& c, int form, const Csf3Dev& B, const Csr& C, u64* partial, int* blocks);
 cudaError_t launch_higher_setup(const LaunchCtx& c, int form, const Csf3Dev& B, const Csr& C, int* fib_of, int* slice_of, int* cnt);
 cudaError_t launch_higher_ism(const LaunchCtx& c, bool numeric, int form, const Csf3Dev& B, const Csr& C, const Csr& D, const int* fib_of,
                               const int* slice_of, const i64* eoff, i64 P, i64 cap, u64 d1, u64 d2, int label_bits, u64* kA, void* vA,

@@ -146,13 +146,14 @@ __global__ void __launch_bounds__(OT) outer_total_kernel(Csr At, Csr B, u64* __r
     for (i64 k = (i64)blockIdx.x * OT + threadIdx.x; k < At.nrows; k += (i64)gridDim.x * OT)
         mine += (At.pos[k + 1] - At.pos[k]) * (B.pos[k + 1] - B.pos[k]);
     mine = block_sum<OT>(mine, ws);
-    if (threadIdx.x == 0) partial[blockIdx.x] = (u64)mine;
+    if (threadIdx.x == 0) *(volatile u64*)&partial[blockIdx.x] = (u64)mine + 1;
 }
 
-cudaError_t launch_outer_total(const LaunchCtx& c, const Csr& At, const Csr& B, u64* partial) {
+cudaError_t launch_outer_total(const LaunchCtx& c, const Csr& At, const Csr& B, u64* partial, int* blocks) {
+    *blocks = 0;
     if (At.nrows == 0) return cudaSuccess;
-    const int grid = grid_for(c, At.nrows, OT);
-    outer_total_kernel<<<grid < COUNT_BLOCKS ? grid : COUNT_BLOCKS, OT, 0, c.stream>>>(At, B, partial);
+    *blocks = std::min(grid_for(c, At.nrows, OT), COUNT_BLOCKS);
+    outer_total_kernel<<<*blocks, OT, 0, c.stream>>>(At, B, partial);
     return cudaGetLastError();
 }
 

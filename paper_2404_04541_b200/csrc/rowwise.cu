@@ -34,9 +34,11 @@ constexpr int RK_TILE = OT * RK_ITEMS;
 // consecutive entries, so the owners of its first and last entry bound every search.  B's columns
 // are checked on the way (the row kernels look at the ends of a row only).
 __global__ void __launch_bounds__(OT) rw_keys_outer_kernel(Csr At, i64 n, Csr B, i64 nnzB, u64* __restrict__ keys, u64* __restrict__ pay,
-                                                           DevCtl* ctl) {
+                                                           int passes, SortHead* head, DevCtl* ctl) {
     __shared__ int s_lo, s_hi;
+    __shared__ DigitCounts s_digits;
     bool bad = false;
+    s_digits.start(passes);
     for (i64 q = (i64)blockIdx.x * OT + threadIdx.x; q < nnzB; q += (i64)gridDim.x * OT) bad |= (unsigned)__ldg(B.crd + q) >= (unsigned)B.ncols;
     for (i64 t0 = (i64)blockIdx.x * RK_TILE; t0 < n; t0 += (i64)gridDim.x * RK_TILE) {
         __syncthreads();
@@ -49,15 +51,21 @@ __global__ void __launch_bounds__(OT) rw_keys_outer_kernel(Csr At, i64 n, Csr B,
             const int i = __ldg(At.crd + p);
             bad |= (unsigned)i >= (unsigned)At.ncols;
             keys[p] = (u64)(unsigned)i;
+            s_digits.add((u64)(unsigned)i, passes);
             pay[p] = ((u64)(unsigned)owner_row(At.pos, s_lo, s_hi, p) << 32) | (u64)(unsigned)p;
         }
     }
+    s_digits.flush(passes, head);
     if (bad) raise_status(ctl, DEV_NONCANONICAL);
 }
 
-// form: 0 SpTTM, 1 SpTTM-I, 2 SpMTTKRP.  `d` = extent of the label's inner coordinate (forms 0, 1).
-__global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u64 d, u64* __restrict__ keys, u64* __restrict__ pay) {
+// pos[0 .. m] := nnz on the way (rw_sparse_rows_kernel writes the rows there are).  form: 0 SpTTM, 1 SpTTM-I, 2 SpMTTKRP.  `d` = extent of the label's inner coordinate (forms 0, 1).
+__global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u64 d, u64* __restrict__ keys, u64* __restrict__ pay, int passes,
+                                                         SortHead* head, i64* __restrict__ pos, i64 m) {
     __shared__ int s_f[2], s_s[2];
+    __shared__ DigitCounts s_digits;
+    s_digits.start(passes);
+    for (i64 i = (i64)blockIdx.x * OT + threadIdx.x; i <= m; i += (i64)gridDim.x * OT) pos[i] = B.nnz;
     for (i64 t0 = (i64)blockIdx.x * RK_TILE; t0 < B.nnz; t0 += (i64)gridDim.x * RK_TILE) {
         __syncthreads();
         if ((threadIdx.x & 31) == 0 && threadIdx.x < 64) {
@@ -80,9 +88,11 @@ __global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u6
                 pick = form == 0 ? c0 : c1;
             }
             keys[e] = key;
+            s_digits.add(key, passes);
             pay[e] = (pick << 32) | (u64)(unsigned)e;
         }
     }
+    s_digits.flush(passes, head);
 }
 
 // CSR result: the reordered operand has one row per output row; pos by binary search in the sorted labels.
@@ -102,10 +112,6 @@ __global__ void __launch_bounds__(OT) rw_dense_rows_kernel(const u64* __restrict
         crd[p] = (int)(w >> 32);
         src[p] = (int)(unsigned)w;
     }
-}
-
-__global__ void __launch_bounds__(OT) fill_pos_kernel(i64* __restrict__ pos, i64 m, i64 value) {
-    for (i64 i = (i64)blockIdx.x * OT + threadIdx.x; i <= m; i += (i64)gridDim.x * OT) pos[i] = value;
 }
 
 // Coordinate-form result: only the labels that occur become rows, in order (row r has label row_key[r]);
@@ -331,21 +337,18 @@ __global__ void __launch_bounds__(OT) rw_coords_kernel(const i64* __restrict__ r
 }
 
 // ---- host side --------------------------------------------------------------------------------
-size_t rw_sort_bytes(i64 n) {
-    const size_t rows_status = sort_head_bytes() + 8 * (size_t)((n + RK_TILE - 1) / RK_TILE + 1);
-    return std::max(sort_scratch_bytes(n), rows_status);
-}
+// (what the sort needs, then the ticket and the words of rw_sparse_rows_kernel: cleared together)
+size_t rw_sort_bytes(i64 n) { return sort_scratch_bytes(n) + 8 * (size_t)((n + RK_TILE - 1) / RK_TILE + 1); }
+
+static int passes_of(int bits) { return (bits + 7) / 8; }
 
 // Sorts the entries by output row and writes the reordered operand (all but its values).  `sparse`: a row per
-// label that occurs (at most m), labels to row_key; otherwise a row per label value.
+// label that occurs (at most m), labels to row_key; otherwise a row per label value.  The kernel that wrote the labels has
+// counted their digits (a kernel of its own for that, one for `pos` and their clearing took 10 .. 18 us a call).
 static cudaError_t rw_reorder(const LaunchCtx& c, i64 n, i64 m, int bits, bool sparse, const RowwiseBufs& b) {
     cudaError_t e;
-    if (sparse) {
-        fill_pos_kernel<<<grid_for(c, m + 1, OT), OT, 0, c.stream>>>(b.pos, m, n);
-        ++c.launches;
-    }
     bool first = true;
-    if ((e = radix_sort_t<u64, true>(c, n, bits, b.kA, b.pA, b.kB, b.pB, b.sort_tmp, &first)) != cudaSuccess) return e;
+    if ((e = radix_sort_t<u64, true>(c, n, bits, b.kA, b.pA, b.kB, b.pB, b.sort_tmp, &first, true)) != cudaSuccess) return e;
     const u64* ks = first ? b.kA : b.kB;
     const u64* ps = first ? b.pA : b.pB;
     if (!sparse) {
@@ -353,26 +356,28 @@ static cudaError_t rw_reorder(const LaunchCtx& c, i64 n, i64 m, int bits, bool s
         ++c.launches;
     } else if (n > 0) {
         const int tiles = (int)((n + RK_TILE - 1) / RK_TILE);
-        SortHead* head = reinterpret_cast<SortHead*>(b.sort_tmp);
-        if ((e = cudaMemsetAsync(b.sort_tmp, 0, sort_head_bytes() + 8 * (size_t)tiles, c.stream)) != cudaSuccess) return e;
-        rw_sparse_rows_kernel<<<tiles, OT, 0, c.stream>>>(ks, ps, n, m, &head->ticket[0], reinterpret_cast<u64*>(b.sort_tmp + sort_head_bytes()),
-                                                         c.ctl, b.row_key, b.pos, b.crd, b.src);
+        u64* const words = reinterpret_cast<u64*>(b.sort_tmp + sort_scratch_bytes(n));
+        rw_sparse_rows_kernel<<<tiles, OT, 0, c.stream>>>(ks, ps, n, m, reinterpret_cast<int*>(words), words + 1, c.ctl, b.row_key, b.pos, b.crd, b.src);
         ++c.launches;
     }
     return cudaGetLastError();
 }
 
 cudaError_t launch_rw_outer(const LaunchCtx& c, const Csr& At, i64 n, const Csr& B, i64 nnzB, int bits, const RowwiseBufs& b) {
-    rw_keys_outer_kernel<<<grid_for(c, std::max(n, nnzB), RK_TILE), OT, 0, c.stream>>>(At, n, B, nnzB, b.kA, b.pA, c.ctl);
+    const cudaError_t e = cudaMemsetAsync(b.sort_tmp, 0, rw_sort_bytes(n), c.stream);
+    if (e != cudaSuccess) return e;
+    rw_keys_outer_kernel<<<grid_for(c, std::max(n, nnzB), RK_TILE), OT, 0, c.stream>>>(At, n, B, nnzB, b.kA, b.pA, passes_of(bits),
+                                                                                     reinterpret_cast<SortHead*>(b.sort_tmp), c.ctl);
     ++c.launches;
     return rw_reorder(c, n, At.ncols, bits, false, b);
 }
 
 cudaError_t launch_rw_csf(const LaunchCtx& c, int form, const Csf3Dev& B, u64 d, i64 m, int bits, const RowwiseBufs& b) {
-    if (B.nnz > 0) {
-        rw_keys_csf_kernel<<<grid_for(c, B.nnz, RK_TILE), OT, 0, c.stream>>>(form, B, d, b.kA, b.pA);
-        ++c.launches;
-    }
+    const cudaError_t e = cudaMemsetAsync(b.sort_tmp, 0, rw_sort_bytes(B.nnz), c.stream);
+    if (e != cudaSuccess) return e;
+    rw_keys_csf_kernel<<<grid_for(c, std::max(B.nnz, (i64)1), RK_TILE), OT, 0, c.stream>>>(form, B, d, b.kA, b.pA, passes_of(bits),
+                                                                                         reinterpret_cast<SortHead*>(b.sort_tmp), b.pos, m);
+    ++c.launches;
     return rw_reorder(c, B.nnz, m, bits, true, b);
 }
 

@@ -41,6 +41,23 @@ struct SortHead {
 };
 static size_t sort_head_bytes() { return (sizeof(SortHead) + 255) & ~(size_t)255; }
 
+// Digits of the labels a block writes, for a kernel of 256 threads: start, add for every label, flush.
+struct DigitCounts {
+    int h[RS_PASSES][256];
+    __device__ __forceinline__ void start(int passes) {
+        for (int p = 0; p < passes; ++p) h[p][threadIdx.x] = 0;
+        __syncthreads();
+    }
+    __device__ __forceinline__ void add(u64 key, int passes) {
+        for (int p = 0; p < passes; ++p, key >>= 8) atomicAdd(&h[p][(unsigned)key & 255u], 1);
+    }
+    __device__ __forceinline__ void flush(int passes, SortHead* head) {
+        __syncthreads();
+        for (int p = 0; p < passes; ++p)
+            if (h[p][threadIdx.x]) atomicAdd(&head->hist[p][threadIdx.x], h[p][threadIdx.x]);
+    }
+};
+
 static __global__ void __launch_bounds__(RS_THREADS) radix_hist_kernel(const u64* __restrict__ keys, i64 n, int passes, SortHead* __restrict__ head) {
     __shared__ int s_h[RS_PASSES][256];
     for (int p = 0; p < passes; ++p) s_h[p][threadIdx.x] = 0;
@@ -141,20 +158,23 @@ static size_t sort_scratch_bytes(i64 n) {
 }
 
 // Sorts n (label, value) pairs by label; `bits` = number of significant label bits.  Input in
-// (k0, v0), the other buffer in (k1, v1); *in_first tells which pair holds the result.
+// (k0, v0), the other buffer in (k1, v1); *in_first tells which pair holds the result.  `counted`: the caller has cleared
+// `tmp`, and its kernel that wrote the labels has counted their digits (DigitCounts).
 template <typename T, bool VALUES>
-static cudaError_t radix_sort_t(const LaunchCtx& c, i64 n, int bits, u64* k0, T* v0, u64* k1, T* v1, char* tmp, bool* in_first) {
+static cudaError_t radix_sort_t(const LaunchCtx& c, i64 n, int bits, u64* k0, T* v0, u64* k1, T* v1, char* tmp, bool* in_first, bool counted = false) {
     *in_first = true;
     if (n <= 1) return cudaSuccess;
     const int nblocks = (int)((n + RS_TILE - 1) / RS_TILE);
     const int passes = (bits + 7) / 8;
     SortHead* head = reinterpret_cast<SortHead*>(tmp);
     u64* status = reinterpret_cast<u64*>(tmp + sort_head_bytes());
-    cudaError_t e = cudaMemsetAsync(tmp, 0, sort_scratch_bytes(n), c.stream);
-    if (e != cudaSuccess) return e;
-    const int hist_blocks = 4 * c.sm_count;
-    radix_hist_kernel<<<nblocks < hist_blocks ? nblocks : hist_blocks, RS_THREADS, 0, c.stream>>>(k0, n, passes, head);
-    ++c.launches;
+    if (!counted) {
+        const cudaError_t e = cudaMemsetAsync(tmp, 0, sort_scratch_bytes(n), c.stream);
+        if (e != cudaSuccess) return e;
+        const int hist_blocks = 4 * c.sm_count;
+        radix_hist_kernel<<<nblocks < hist_blocks ? nblocks : hist_blocks, RS_THREADS, 0, c.stream>>>(k0, n, passes, head);
+        ++c.launches;
+    }
     u64 *ki = k0, *ko = k1;
     T *vi = v0, *vo = v1;
     for (int pass = 0; pass < passes; ++pass) {

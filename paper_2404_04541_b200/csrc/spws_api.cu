@@ -896,8 +896,8 @@ int label_bits_of(int64_t I, int64_t J) {
     return bits;
 }
 
-// adds up what a counting kernel left in the plan's pinned slots
-// (*once, when given: the second set of slots)
+// Adds up what a counting kernel leaves in the plan's pinned slots: polled for a fifth of a millisecond, then the stream is
+// synchronised.  (*once, when given: the second set of slots)
 template <typename Launch>
 spws_status_t count_products(spws_plan_s* p, Launch launch, int64_t* P, int64_t* once = nullptr) {
     LaunchCtx c{};
@@ -905,19 +905,37 @@ spws_status_t count_products(spws_plan_s* p, Launch launch, int64_t* P, int64_t*
     c.sm_count = p->h->sm_count;
     memset(p->host->partial, 0, sizeof(p->host->partial));
     p->in_flight = true;
-    CUDA_TRY(launch(c, p->host->partial));
-    CUDA_TRY(cudaStreamSynchronize(c.stream));
+    int blocks = 0;
+    CUDA_TRY(launch(c, p->host->partial, &blocks));
+    const volatile u64* sums = p->host->partial;
+    const int sets = once ? 2 : 1;
+    u64 total[2] = {0, 0};
+    int got = 0;
+    auto take = [&]() {
+        for (; got < sets * blocks; ++got) {
+            const int set = got / blocks;
+            const u64 v = sums[set * COUNT_BLOCKS + got % blocks];
+            if (v == 0) return false;
+            total[set] += v - 1;
+        }
+        return true;
+    };
+    const auto end = std::chrono::steady_clock::now() + std::chrono::microseconds(200);
+    while (!take())
+        if (std::chrono::steady_clock::now() >= end) {
+            CUDA_TRY(cudaStreamSynchronize(c.stream));
+            if (!take()) return SPWS_CUDA_ERROR;
+            break;
+        }
     p->in_flight = false;
-    u64 total = 0, total2 = 0;
-    for (int b = 0; b < COUNT_BLOCKS; ++b) { total += p->host->partial[b]; total2 += p->host->partial[COUNT_BLOCKS + b]; }
-    *P = (int64_t)total;
-    if (once) *once = (int64_t)total2;
+    *P = (int64_t)total[0];
+    if (once) *once = (int64_t)total[1];
     return SPWS_OK;
 }
 
 // products of the outer form, counted on the device
 spws_status_t outer_count_products(spws_plan_s* p, const Shapes& S, int64_t* P) {
-    return count_products(p, [&](const LaunchCtx& c, u64* partial) { return launch_outer_total(c, S.A, S.B, partial); }, P);
+    return count_products(p, [&](const LaunchCtx& c, u64* partial, int* blocks) { return launch_outer_total(c, S.A, S.B, partial, blocks); }, P);
 }
 
 // ---- second- and higher-order forms taken row by row (rowwise.cu) -----------------------------
@@ -1069,16 +1087,30 @@ spws_status_t outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_t* 
                              size_t* needed) {
     const int64_t I = S.m, K = S.k, J = S.ncols;
     if (I * J < 0 || (I > 0 && J > (int64_t)(0x7fffffffffffffffll / (I > 0 ? I : 1)))) return SPWS_INVALID_ARGUMENT;
+    // the products are counted only where something depends on their number: not when the tables of the rows are small (the count
+    // and the wait for it took 17 us a call)
     int64_t P = 0;
-    spws_status_t st = outer_count_products(plan, S, &P);
-    if (st != SPWS_OK) return st;
-    const OuterLayout L = make_outer_layout(plan, I, K, J, P);
-    plan->rowwise = rw_wanted(plan, I, J, S.nnzA, P);
+    spws_status_t st = SPWS_OK;
+    bool counted = false;
+    auto count = [&]() {
+        if (!counted) st = outer_count_products(plan, S, &P);
+        counted = true;
+        return st == SPWS_OK;
+    };
+    plan->rowwise = rw_wanted(plan, I, J, S.nnzA, 0);
+    if (!plan->rowwise) {
+        if (!count()) return st;
+        plan->rowwise = rw_wanted(plan, I, J, S.nnzA, P);
+    }
     if (plan->rowwise) {
-        st = rw_outer_symbolic(plan, S, C, scratch, scratch_bytes, sizes_out, needed);
-        if (st != SPWS_SCRATCH_TOO_SMALL || needed || P > ORDINAL_MAX || scratch_bytes < std::min(L.ism_end, L.dense_end)) return st;
+        const spws_status_t done = rw_outer_symbolic(plan, S, C, scratch, scratch_bytes, sizes_out, needed);
+        if (done != SPWS_SCRATCH_TOO_SMALL || needed) return done;
+        if (!count()) return st;
+        const OuterLayout L = make_outer_layout(plan, I, K, J, P);
+        if (P > ORDINAL_MAX || scratch_bytes < std::min(L.ism_end, L.dense_end)) return done;
         plan->rowwise = false;              // a buffer too small for the tables of the rows that holds the products
     }
+    const OuterLayout L = make_outer_layout(plan, I, K, J, P);
     plan->rows_path = false;
     if (P > ORDINAL_MAX) return SPWS_INTERNAL_OVERFLOW;
     if (needed) {
@@ -1276,7 +1308,8 @@ HLayout make_hlayout(const spws_plan_s* p, const HShapes& H, int64_t P) {
 }
 
 spws_status_t higher_count_products(spws_plan_s* p, const HShapes& H, int64_t* P, int64_t* once) {
-    return count_products(p, [&](const LaunchCtx& c, u64* partial) { return launch_higher_total(c, H.form, H.B, H.C, partial); }, P, once);
+    return count_products(
+        p, [&](const LaunchCtx& c, u64* partial, int* blocks) { return launch_higher_total(c, H.form, H.B, H.C, partial, blocks); }, P, once);
 }
 
 // The tensor's entries in the order of their output row: (i,j), (k,j) or i, of which at most m occur.  The matrix the
