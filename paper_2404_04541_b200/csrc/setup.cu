@@ -664,8 +664,8 @@ cudaError_t launch_bin_rows(const LaunchCtx& c, int m) {
 //   sfp[s] receives the number of survivors before slice s.
 // Replaces a three-launch scan, the routing and the per-class count (five launches; seven for the
 // 3-tensor form).
-// Bound by the chain of its steps below a few tiles (2048 rows: 9 us where the five launches took 13 and their gaps),
-// by HBM beyond (2e6 fibres: 43 us against 56).
+// Bound by the chain of its steps below a few tiles (2048 rows: 6 us where the five launches took 13 and their gaps),
+// by HBM beyond (2e6 fibres: 33 us against 56).
 // ---------------------------------------------------------------------------------------
 constexpr int FR_THREADS = 256;
 constexpr int FR_WARPS = FR_THREADS / 32;

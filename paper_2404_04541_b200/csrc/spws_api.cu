@@ -994,9 +994,9 @@ RowwiseBufs rw_bufs(char* x, const RwLayout& R) {
 // insert-sort-merge, which one long row serialises, while sorting all products does not), unless the
 // tables of m rows (about 80 bytes each) would outgrow both 1 GiB and what sorting the products
 // takes (about 48 bytes each).  A plan that sets outer_cap asks for Algorithm 1's rounds.
-// Measured per call on B200: outer 10^4 x 10^4, 1e8 products 869 us, 5070 us by the dense
-// second-order workspace; 2e5 x 1.8e5, 12e6 products 529 us, 2110 us by sorting the products; SpTTM with 43e6
-// products 973 us, 8000 us by sorting them.  Just beyond the widest columns, where rows of up to 4096 products
+// Measured per call on B200: outer 10^4 x 10^4, 1e8 products 736 us, 5070 us by the dense
+// second-order workspace; 2e5 x 1.8e5, 12e6 products 435 us, 2110 us by sorting the products; SpTTM with 43e6
+// products 864 us, 8000 us by sorting them.  Just beyond the widest columns, where rows of up to 4096 products
 // would not need the fallback either, 7e6 products in rows of 17 take 1700 us, 430 us within them.
 bool rw_wanted(const spws_plan_s* p, int64_t m, int64_t ncols, int64_t n, int64_t P) {
     if (p->policy != SPWS_AUTO || p->opt.outer_cap != 0 || ncols > p->opt.dense_max_span || n > 0x7fff0000ll) return false;
