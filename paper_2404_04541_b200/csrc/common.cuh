@@ -428,7 +428,7 @@ __device__ __forceinline__ int row_at(const RowRanges& g, int r) {
     return row;
 }
 struct IsmLaunch { int level; RowRanges g; };
-// the launches for the rows as binned (at most ISM_LEVELS); returns their number
+// the launches for the rows as binned (at most ISM_LEVELS, lowest level first); returns their number
 int ism_launches(const LaunchCtx& c, IsmLaunch* out);
 cudaError_t launch_ism(const LaunchCtx& c, bool numeric, const IsmLaunch& l, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval);
 // scratch that keeps the sorted words of the rows of the warp-per-row ISM from the counting pass to the numeric one;

@@ -743,11 +743,12 @@ int ism_launches(const LaunchCtx& c, IsmLaunch* out) {
                                rows[CLS_ISM_SMEM]};
     const int cls[ISM_LEVELS] = {CLS_ISM_REG8, CLS_ISM_GROUP8, CLS_ISM_GROUP16, CLS_ISM_SMEM_S, CLS_ISM_SMEM};
     int made = 0;
+    IsmLaunch from_above[ISM_LEVELS];
     bool taken[ISM_LEVELS] = {};
     for (int at = ISM_LEVELS - 1; at >= 0; --at) {
         if (n[at] == 0 || taken[at]) continue;
         // this level's own rows first, then those of lower levels that are few
-        IsmLaunch& l = out[made++];
+        IsmLaunch& l = from_above[made++];
         l.level = at;
         int k = 0;
         i64 end = 0;
@@ -759,6 +760,7 @@ int ism_launches(const LaunchCtx& c, IsmLaunch* out) {
         }
         for (; k < ISM_LEVELS; ++k) { l.g.rows[k] = l.g.rows[0]; l.g.end[k] = (int)end; }
     }
+    for (int k = 0; k < made; ++k) out[k] = from_above[made - 1 - k];
     return made;
 }
 

@@ -812,6 +812,12 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, cha
     c.class_rows = LL(bins);
     const bool copies = plan->copy_products >= FORK_PRODUCTS;
     Fork fork(plan, c, s.dense_warp_rows > 0, copies || s.dense_units > 0 || bins[CLS_ISM_GLOBAL] > 0);
+    // (in the order of the timing groups: a group is timed from the end of the one before)
+    fork.group(2);
+    if (bins[CLS_COPY] > 0) {
+        CUDA_TRY(launch_copy_rows(c, S.A, S.B, rowptr, crd, val));
+        mark(plan, SPWS_T_NUM_ISM_REG);
+    }
     fork.group(0);
     IsmLaunch ism[ISM_LEVELS];
     const int n_ism = ism_launches(c, ism);
@@ -825,10 +831,6 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, cha
         mark(plan, SPWS_T_NUM_DENSE_WARP);
     }
     fork.group(2);
-    if (bins[CLS_COPY] > 0) {
-        CUDA_TRY(launch_copy_rows(c, S.A, S.B, rowptr, crd, val));
-        mark(plan, SPWS_T_NUM_ISM_REG);
-    }
     if (s.dense_units > 0) {
         CUDA_TRY(launch_dense_num_cta(c, 0, (int)s.dense_units, plan->max_span_words, plan->row_products, S.A, S.B, rowptr, crd, val));
         mark(plan, SPWS_T_NUM_DENSE_EMIT);
