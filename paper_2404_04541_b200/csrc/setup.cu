@@ -40,7 +40,10 @@ cudaError_t launch_validate(const LaunchCtx& c, const Csr& A, const Csr& B, i64 
 // [jmin, jmax] of the candidate columns (first / last coordinate of the picked B rows, which
 // are sorted), and the workspace class of the row.
 // ---------------------------------------------------------------------------------------
-__device__ __forceinline__ int dense_class(i64 ub, i64 span_words) {
+// A span that ends before it begins comes from B rows that are not ascending: such a row has no bitmap whose words could be
+// counted (the slots of all rows must lie inside the arena once their sum does).  The sparse workspaces read no span.
+__device__ __forceinline__ int dense_class(i64 ub, i64 span_words, DevCtl* ctl) {
+    if (span_words <= 0) { raise_status(ctl, DEV_NONCANONICAL); return CLS_EMPTY; }
     if (span_words <= DENSE_WARP_BM_WORDS && ub <= DENSE_WARP_MAX_UB) return CLS_DENSE_WARP;
     return ub >= DENSE_HUB_UB ? CLS_DENSE_HUB : CLS_DENSE_CTA;
 }
@@ -56,7 +59,7 @@ __device__ __forceinline__ int classify_row(i64 ub, i64 entries, int jmin, int j
     const bool reg_ok = ub <= prm.reg_cap && span <= (1ll << 26);
     if (prm.policy == 0) {                       // dense forced
         if (!dense_ok) { raise_status(ctl, DEV_WORKSPACE_TOO_LARGE); return CLS_EMPTY; }
-        return dense_class(ub, span_words);
+        return dense_class(ub, span_words, ctl);
     }
     // a single entry: Insert, Sort and Merge are the identity and the output count is the B row's length,
     // known right here (up to COPY_MAX entries, which eight lanes copy; SpTTM with 41-entry rows, two
@@ -82,10 +85,10 @@ __device__ __forceinline__ int classify_row(i64 ub, i64 entries, int jmin, int j
     // (6e6 products, f64, both passes, dense against ISM: 60 products a row 263 : 172 us, 117 a row 156 : 126
     // us, 240 a row on 94 words 119 : 113 us and on 626 words 160 : 110 us; 380 a row 98 : 168 us)
     if (ub <= prm.smem_small_cap && (ub <= 128 || span_words > 256)) return small_ism_class(ub);
-    if (dense_ok && (float)span_words <= prm.span_words_per_product * (float)ub) return dense_class(ub, span_words);
+    if (dense_ok && (float)span_words <= prm.span_words_per_product * (float)ub) return dense_class(ub, span_words, ctl);
     if (ub <= prm.smem_small_cap) return small_ism_class(ub);
     if (ub <= prm.smem_cap) return CLS_ISM_SMEM;
-    if (dense_ok) return dense_class(ub, span_words);
+    if (dense_ok) return dense_class(ub, span_words, ctl);
     return CLS_ISM_GLOBAL;
 }
 
@@ -635,7 +638,7 @@ __global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, 
             if (words[x]) {
                 const u64 at = s_bm_base + (u64)my_off;
                 my_off += words[x];
-                tab.bm_off[row] = (i64)at;              // (inside the arena: the bounds kernel compared the total)
+                tab.bm_off[row] = (i64)at;              // (inside the arena: the slots add up to the total compared above)
             }
         }
         __syncthreads();
