@@ -197,7 +197,7 @@ constexpr int COUNT_BLOCKS = 256;
 constexpr int CTL_WORDS = sizeof(DevCtl) / 4;
 struct HostBlock {
     DevCtl ctl;             // as the host last received it
-    int late;               // status raised after the first publication of a pass
+    int late;               // status raised after the first publication of a pass, which clears it
     int pad[31];
     u64 words[CTL_WORDS];   // number of the publication above a word of the control block
     u64 partial[2 * COUNT_BLOCKS];

@@ -574,6 +574,7 @@ __global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, 
     if (blockIdx.x == 0) {
         if (threadIdx.x == 0) {
             if (too_small) raise_status(ctl, DEV_SCRATCH_TOO_SMALL);
+            *(volatile int*)&host->late = 0;            // (here and not by the host: the pass before may still raise one)
             ctl->host_status = &host->late;
         }
         __syncthreads();

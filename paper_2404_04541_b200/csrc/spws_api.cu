@@ -661,7 +661,6 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
                             spws_tensor_t* ttmC, i64* rowptr, char* sc) {
     plan->in_flight = true;
     plan->pending = false;
-    plan->host->late = 0;
     c.seq = plan->seq + 1;
     plan->seq += 2;
     // a1: upper bounds + classes; a2: binning
