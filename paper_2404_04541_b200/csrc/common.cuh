@@ -33,6 +33,7 @@ constexpr int EMIT_SLOT = 48;  // work_counter slot of the coordinate emission o
 constexpr int BW_SLOT = 49;    // work_counter slot of the word-list build
 constexpr int WARP_SLOT = 52;  // work_counter slots of the lists of the warp dense route: numeric, gather-only
 constexpr int CEIL_WARP_SLOT = 54;
+constexpr int BW_WARP_SLOT = 56; // as BW_SLOT, for the rows a warp takes
 constexpr int ISM_CTA_SLOT = 50; // work_counter slots of the CTA kernel of the shared-memory ISM, symbolic and numeric
 constexpr int ISM_CTA_NUM_SLOT = 51;
 constexpr int N_WORK_COUNTERS = 64;
@@ -86,7 +87,7 @@ struct DevCtl {
     int n_warp_rows[N_WARP_LISTS];  // numeric dense warp rows by the accumulator they need
     int max_span_words;     // widest bitmap among the dense rows
     int max_warp_cnt[N_WARP_LISTS]; // most outputs of a row on each list
-    int n_long;             // B rows with at least BW_MIN_LEN entries (candidates for a word list)
+    int n_long, n_longest;  // B rows with at least BW_MIN_LEN / BW_BLOCK_ROW entries (candidates for a word list, by a warp / a block)
     int rows_done, slices_done;                 // blocks that have finished
     int rows_ticket, slices_ticket;             // tiles handed out
     int* host_status;       // HostBlock::late (null before the first publication)

@@ -481,71 +481,104 @@ cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i6
 // .y = the bits of the row's entries in that word) follow.  A list is kept only when it has at
 // most three quarters as many pairs as the row has entries.
 // ---------------------------------------------------------------------------------------
+// Rows of at least BW_BLOCK_ROW entries are listed from the end of bw_long and take a block each, the others from its start.
+// Those take a warp each when they are more than BW_FEW, else a block each too: a block of 1024 threads spends 3.1 us on a row
+// of 300 entries, a warp 13.5 us, of which 9472 run at once, and 27 us on one of 1000.  A block of 1024 for
+// every row / a warp for all but those of 1024 entries / by the count, us: power law on 8000 vertices 9 / 25 / 9, 16381
+// 24 / 33 / 24, 2^18 56 / 30 / 30; 2e4 rows of 256 207 / 31 / 31; 1e5 rows of 300 1078 / 142 / 140.  (256 threads for every row: 12,
+// 20, 80, 54, 281; 3000 rows of 4000 60, with 1024 69, by a warp 150.)
+constexpr int BW_BLOCK_ROW = 1024;
+constexpr int BW_FEW = 2048;
 __global__ void __launch_bounds__(256) bw_find_long_kernel(Csr B, int* __restrict__ bw_long, int cap, DevCtl* ctl) {
     for (i64 k = (i64)blockIdx.x * blockDim.x + threadIdx.x; k < B.nrows; k += (i64)gridDim.x * blockDim.x) {
-        if (B.pos[k + 1] - B.pos[k] >= BW_MIN_LEN) {
+        const i64 len = B.pos[k + 1] - B.pos[k];
+        if (len >= BW_BLOCK_ROW) {
+            const int at = atomicAdd(&ctl->n_longest, 1);
+            if (at < cap) bw_long[cap - 1 - at] = (int)k;
+        } else if (len >= BW_MIN_LEN) {
             const int at = atomicAdd(&ctl->n_long, 1);
             if (at < cap) bw_long[at] = (int)k;
         }
     }
 }
 
-constexpr int BWB_THREADS = 1024;     // (the longest row sets the time: power law on 2^18 vertices 86 us with 256, 56 with 1024)
+constexpr int BWB_THREADS = 1024;
 constexpr int BWB_ITEMS = 4;
 
-__global__ void __launch_bounds__(BWB_THREADS) bw_build_kernel(Csr B, const int* __restrict__ bw_long, int cap,
-                                                              uint2* __restrict__ bw, DevCtl* ctl) {
+// The list of row k by `THREADS` threads, of which this is thread `tid`.
+template <int THREADS>
+__device__ __forceinline__ void bw_build_row(int k, int tid, const Csr& B, uint2* __restrict__ bw, int* ws) {
+    const i64 qs = B.pos[k], qe = B.pos[k + 1];
+    const i64 len = qe - qs;
+    const int* __restrict__ crd = B.crd;
+    int carry = 0;                                       // pairs of the row before this tile
+    for (i64 t0 = qs; t0 < qe; t0 += THREADS * BWB_ITEMS) {
+        const i64 q0 = t0 + (i64)tid * BWB_ITEMS;
+        unsigned word[BWB_ITEMS], bits[BWB_ITEMS];
+        int nfirst = 0;
+        unsigned prev = (q0 > qs && q0 < qe) ? ((unsigned)__ldg(crd + q0 - 1) >> 5) : 0xffffffffu;
+#pragma unroll
+        for (int x = 0; x < BWB_ITEMS; ++x) {
+            const i64 q = q0 + x;
+            word[x] = 0xffffffffu;                       // not the first entry of a word
+            bits[x] = 0u;
+            if (q < qe) {
+                const unsigned c = (unsigned)__ldg(crd + q);
+                if ((c >> 5) != prev) {
+                    word[x] = c >> 5;
+                    unsigned b = 1u << (c & 31);
+                    for (i64 q2 = q + 1; q2 < qe; ++q2) {              // at most 31 more entries share the word
+                        const unsigned c2 = (unsigned)__ldg(crd + q2);
+                        if ((c2 >> 5) != word[x]) break;
+                        b |= 1u << (c2 & 31);
+                    }
+                    bits[x] = b;
+                    ++nfirst;
+                }
+                prev = c >> 5;
+            }
+        }
+        int at = carry;
+        if constexpr (THREADS == 32) {
+            const int incl = warp_incl_scan(nfirst);
+            at += incl - nfirst;
+            carry += __shfl_sync(0xffffffffu, incl, 31);
+        } else {
+            int total;
+            at += block_excl_scan<THREADS>(nfirst, ws, total);
+            carry += total;
+        }
+#pragma unroll
+        for (int x = 0; x < BWB_ITEMS; ++x)
+            if (word[x] != 0xffffffffu) {
+                if (at + 1 < len) bw[qs + 1 + at] = make_uint2(word[x], bits[x]);
+                ++at;
+            }
+    }
+    if (tid == 0) bw[qs] = make_uint2(4 * (i64)carry <= 3 * len ? (unsigned)carry : 0u, 0u);
+}
+
+__global__ void __launch_bounds__(BWB_THREADS, 2) bw_build_kernel(Csr B, const int* __restrict__ bw_long, int cap,
+                                                                 uint2* __restrict__ bw, DevCtl* ctl) {
     __shared__ int ws[33];
     __shared__ int s_next;
-    const int n_long = min(ctl->n_long, cap);
     const int tid = threadIdx.x;
+    const int n_longest = min(ctl->n_longest, cap), n_long = min(ctl->n_long, cap);
+    const bool few = n_long <= BW_FEW;
     for (;;) {
         __syncthreads();
         if (tid == 0) s_next = atomicAdd(&ctl->work_counter[BW_SLOT], 1);
         __syncthreads();
-        if (s_next >= n_long) break;
-        const int k = bw_long[s_next];
-        const i64 qs = B.pos[k], qe = B.pos[k + 1];
-        const i64 len = qe - qs;
-        const int* __restrict__ crd = B.crd;
-        int carry = 0;                                   // pairs of the row before this tile
-        for (i64 t0 = qs; t0 < qe; t0 += BWB_THREADS * BWB_ITEMS) {
-            const i64 q0 = t0 + (i64)tid * BWB_ITEMS;
-            unsigned word[BWB_ITEMS], bits[BWB_ITEMS];
-            int nfirst = 0;
-            unsigned prev = (q0 > qs && q0 < qe) ? ((unsigned)__ldg(crd + q0 - 1) >> 5) : 0xffffffffu;
-#pragma unroll
-            for (int x = 0; x < BWB_ITEMS; ++x) {
-                const i64 q = q0 + x;
-                word[x] = 0xffffffffu;                   // not the first entry of a word
-                bits[x] = 0u;
-                if (q < qe) {
-                    const unsigned c = (unsigned)__ldg(crd + q);
-                    if ((c >> 5) != prev) {
-                        word[x] = c >> 5;
-                        unsigned b = 1u << (c & 31);
-                        for (i64 q2 = q + 1; q2 < qe; ++q2) {          // at most 31 more entries share the word
-                            const unsigned c2 = (unsigned)__ldg(crd + q2);
-                            if ((c2 >> 5) != word[x]) break;
-                            b |= 1u << (c2 & 31);
-                        }
-                        bits[x] = b;
-                        ++nfirst;
-                    }
-                    prev = c >> 5;
-                }
-            }
-            int total;
-            int at = carry + block_excl_scan<BWB_THREADS>(nfirst, ws, total);
-#pragma unroll
-            for (int x = 0; x < BWB_ITEMS; ++x)
-                if (word[x] != 0xffffffffu) {
-                    if (at + 1 < len) bw[qs + 1 + at] = make_uint2(word[x], bits[x]);
-                    ++at;
-                }
-            carry += total;
-        }
-        if (tid == 0) bw[qs] = make_uint2(4 * (i64)carry <= 3 * len ? (unsigned)carry : 0u, 0u);
+        const int r = s_next;
+        if (r >= n_longest + (few ? n_long : 0)) break;
+        bw_build_row<BWB_THREADS>(r < n_longest ? bw_long[cap - 1 - r] : bw_long[r - n_longest], tid, B, bw, ws);
+    }
+    while (!few) {
+        int r = 0;
+        if ((tid & 31) == 0) r = atomicAdd(&ctl->work_counter[BW_WARP_SLOT], 1);
+        r = __shfl_sync(0xffffffffu, r, 0);
+        if (r >= n_long) break;
+        bw_build_row<32>(bw_long[r], tid & 31, B, bw, nullptr);
     }
 }
 
