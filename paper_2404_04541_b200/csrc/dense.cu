@@ -916,20 +916,26 @@ __global__ void __launch_bounds__(DE_THREADS) dense_emit_crd_kernel(DevCtl* __re
                 } else {
                     // half-full words or fuller: the warp expands a word per step, lane b testing bit b, so the
                     // word's outputs leave as one contiguous store.  The words and their ranks go through shared memory: one
-                    // broadcast load a word, empty ones among them, where taking turns among the lanes with words cost two
-                    // shuffles and a search (10^4 rows of 6500 outputs on 313 words: 162 -> 74 us).
+                    // broadcast load a word, where taking turns among the lanes with words cost two shuffles and a search.
+                    // Lanes without words are passed over: a step for every word costs a group of one full word 128 of them.
+                    // 10^4 rows, us by turns / every word / this: 6500 outputs on 313 words 162 / 70 / 71; 128 blocks of 64 columns
+                    // on 16384 words 292 / 888 / 289.  (A list of the non-empty words alone: 78 and 291 us, and more
+                    // registers or spills, for which the rows of few bits a word pay: power law on 2^18 vertices 3590 us.)
                     const unsigned e1 = (unsigned)(e + __popc(w.x)), e2 = e1 + (unsigned)__popc(w.y), e3 = e2 + (unsigned)__popc(w.z);
                     uint4* const mine = reinterpret_cast<uint4*>(list + (lane << 2));
                     mine[0] = make_uint4(w.x, (unsigned)e, w.y, e1);
                     mine[1] = make_uint4(w.z, e2, w.w, e3);
+                    const unsigned some = __ballot_sync(0xffffffffu, p != 0);
                     __syncwarp();
                     const unsigned below = (1u << lane) - 1u;
-                    const int words = min(128, nw - (g << 7));
-                    int col = base + (g << 12) + lane;
-#pragma unroll 4
-                    for (int x = 0; x < words; ++x, col += 32) {
-                        const uint2 d = list[x];
-                        if ((d.x >> lane) & 1u) Ccrd[o + d.y + __popc(d.x & below)] = col;
+                    const int col = base + (g << 12) + lane;
+                    for (unsigned m = some; m; m &= m - 1) {
+                        const int at = (__ffs(m) - 1) << 2;
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) {
+                            const uint2 d = list[at + x];
+                            if ((d.x >> lane) & 1u) Ccrd[o + d.y + __popc(d.x & below)] = col + ((at + x) << 5);
+                        }
                     }
                     __syncwarp();
                 }
