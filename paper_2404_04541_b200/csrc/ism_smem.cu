@@ -486,10 +486,11 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
     const T* __restrict__ Aval = (const T*)A.val;
     const T* __restrict__ Bval = (const T*)B.val;
     // The way to a row is a chain of loads (its number, its place in perm, its fields, its A entries, their B rows).  AHEAD:
-    // the first links of the next row are fetched between the steps of the current one, where few warps per SM are
-    // bound by that chain: numeric, 8e4 rows of 674 products, f32, 369 -> 345 us (20 warps on an SM), 8e5 rows of 60, f64, 199 -> 178 us.
-    // Elsewhere the registers cost more than the chain (59-product rows, f32: numeric 148 -> 191 us, count 123 -> 126 us).
-    constexpr bool AHEAD = NUMERIC && (CAP > 256 || sizeof(T) == 8);
+    // the number and the fields of the next row are fetched between the steps of this one.  Worth its registers in the numeric
+    // pass of rows beyond 256 products, where few warps are resident (8e4 rows of 674, f32, 20 warps on an SM, 369 -> 345 us).
+    // Not below: numeric, f64, 6e4 rows of 200 products on 2^16 columns 123 us with it and 116 without, on 2^25 267 and 253,
+    // 1e5 rows of 250 222 and 213.
+    constexpr bool AHEAD = NUMERIC && CAP > 256;
     int row, row_n = -1, products, products_n = 0;
     i64 ps, pe, ps_n = 0, pe_n = 0;
     bool kept = false, kept_n = false;              // a row of the class that leaves its order (they come first)
