@@ -15,17 +15,18 @@ enum RowClass : int {
     CLS_ISM_REG8 = 1,   // insert-sort-merge by 4 lanes per row, two words per lane (<= 8 products)
     CLS_ISM_REG16 = 2,  // ... four words per lane (<= 16 products)
     CLS_ISM_REG = 3,    // ... six or eight words per lane (<= 32 products)
-    CLS_ISM_SMEM_S = 4, // insert-sort-merge of 129 .. 256 products, one warp per row
-    CLS_ISM_SMEM = 5,   // insert-sort-merge in shared memory, full CTA
-    CLS_DENSE_WARP = 6, // dense workspace (occupancy bitmap), one warp per row
-    CLS_DENSE_HUB = 7,  // dense workspace, one CTA per row, heaviest rows (scheduled first)
-    CLS_DENSE_CTA = 8,  // dense workspace, one CTA per row
-    CLS_ISM_GLOBAL = 9, // accumulation array in shared memory, all array in global memory
-    CLS_HASH_S = 10,    // hash table in shared memory (reduction at insert time), small CTA
-    CLS_HASH = 11,      // hash table in shared memory, full CTA
-    CLS_COPY = 12,      // one A entry picking a B row of at most COPY_MAX entries: the result is that row, scaled
-    CLS_ISM_GROUP8 = 13,    // insert-sort-merge of at most 64 products by 8 lanes per row
-    CLS_ISM_GROUP16 = 14    // ... of 65 .. 128 products by 16 lanes
+    // (the sparse classes in the order of their products: rows of several go to one launch as one range of perm)
+    CLS_ISM_GROUP8 = 4, // insert-sort-merge of at most 64 products by 8 lanes per row
+    CLS_ISM_GROUP16 = 5,    // ... of 65 .. 128 products by 16 lanes
+    CLS_ISM_SMEM_S = 6, // insert-sort-merge of 129 .. 256 products, one warp per row
+    CLS_ISM_SMEM = 7,   // insert-sort-merge in shared memory, full CTA
+    CLS_DENSE_WARP = 8, // dense workspace (occupancy bitmap), one warp per row
+    CLS_DENSE_HUB = 9,  // dense workspace, one CTA per row, heaviest rows (scheduled first)
+    CLS_DENSE_CTA = 10, // dense workspace, one CTA per row
+    CLS_ISM_GLOBAL = 11,    // accumulation array in shared memory, all array in global memory
+    CLS_HASH_S = 12,    // hash table in shared memory (reduction at insert time), small CTA
+    CLS_HASH = 13,      // hash table in shared memory, full CTA
+    CLS_COPY = 14       // one A entry picking a B row of at most COPY_MAX entries: the result is that row, scaled
 };
 constexpr int NUM_SLOT = 16;   // work_counter[cls] in the symbolic pass, work_counter[NUM_SLOT + cls] in the numeric pass
 constexpr int CEIL_SLOT = 32;  // work_counter[CEIL_SLOT + cls] in the gather-only (iteration-only) kernels
@@ -38,7 +39,7 @@ constexpr int ISM_CTA_SLOT = 50; // work_counter slots of the CTA kernel of the 
 constexpr int ISM_CTA_NUM_SLOT = 51;
 constexpr int N_WORK_COUNTERS = 64;
 // index of a class in the public statistics (the register classes are reported as one, and so are the small ISM ones)
-__host__ __device__ inline int public_class(int cls) { return cls == 0 ? 0 : (cls <= 3 || cls == 12) ? 1 : cls > 12 ? 2 : cls - 2; }
+__host__ __device__ inline int public_class(int cls) { return cls == CLS_EMPTY ? 0 : (cls <= CLS_ISM_REG || cls == CLS_COPY) ? 1 : cls <= CLS_ISM_SMEM_S ? 2 : cls - 4; }
 constexpr int N_PUBLIC_CLASS = 10;
 constexpr int HASH_SMALL_CAP = 1024;       // products of a row the small / the full hash workspace takes
 constexpr int HASH_CAP = 4096;
@@ -420,15 +421,12 @@ cudaError_t launch_copy_rows(const LaunchCtx& c, const Csr& A, const Csr& B, con
 // The insert-sort-merge rows of up to smem_cap products by the kernels that take them: 4, 8 or 16 lanes per row (at most 32, 64 or
 // 128 products), a warp per row (256), the kernels of the full class.
 constexpr int ISM_LEVELS = 5;
-struct RowRanges { const int* rows[ISM_LEVELS]; int end[ISM_LEVELS]; };       // rows of several classes one after the other
-__device__ __forceinline__ int row_at(const RowRanges& g, int r) {
-    int row = r < g.end[0] ? __ldg(g.rows[0] + r) : -1;
-#pragma unroll
-    for (int k = 1; k < ISM_LEVELS; ++k)
-        if (r >= g.end[k - 1] && r < g.end[k]) row = __ldg(g.rows[k] + (r - g.end[k - 1]));
-    return row;
-}
-struct IsmLaunch { int level; RowRanges g; };
+// One launch: its rows lie one after the other in perm, the `own` rows of its level behind those of lower levels.
+struct IsmLaunch {
+    int level, first_cls;
+    const int* rows;
+    int n, own;
+};
 // the launches for the rows as binned (at most ISM_LEVELS, lowest level first); returns their number
 int ism_launches(const LaunchCtx& c, IsmLaunch* out);
 cudaError_t launch_ism(const LaunchCtx& c, bool numeric, const IsmLaunch& l, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval);

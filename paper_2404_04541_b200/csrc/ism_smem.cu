@@ -7,6 +7,7 @@
 //            leaves room for it, else 64 bits (j << 32 | t).
 //   Sort   : bitonic sort of the packed words (lexicographic on (j, t), hence stable).
 //   Merge  : runs of equal j are reduced in slot order and written at row_ptr[i] + rank.
+#include <algorithm>
 #include "common.cuh"
 
 namespace spws {
@@ -353,7 +354,7 @@ __device__ __forceinline__ int sort_group(P* packed, unsigned char* heads, int t
 }
 
 template <typename T, typename P, int G, bool NUMERIC>
-__global__ void __launch_bounds__(IG_THREADS, (group_blocks<T, P, NUMERIC>())) ism_group_kernel(RowRanges g, int n, const DevCtl* __restrict__ ctl,
+__global__ void __launch_bounds__(IG_THREADS, (group_blocks<T, P, NUMERIC>())) ism_group_kernel(const int* __restrict__ rows, int n, const DevCtl* __restrict__ ctl,
                                                                                                Csr A, Csr B, int* __restrict__ cnt,
                                                                                                const i64* __restrict__ rowptr, int* __restrict__ Ccrd,
                                                                                                T* __restrict__ Cval) {
@@ -374,7 +375,7 @@ __global__ void __launch_bounds__(IG_THREADS, (group_blocks<T, P, NUMERIC>())) i
     int row = 0;
     i64 ps = 0, pe = 0;
     if (r < n) {
-        row = row_at(g, r);
+        row = __ldg(rows + r);
         ps = __ldg(A.pos + row);
         pe = __ldg(A.pos + row + 1);
     }
@@ -469,7 +470,7 @@ constexpr int iw_blocks() {
 }
 
 template <typename T, typename P, int CAP, bool NUMERIC>
-__global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>())) ism_warp_kernel(RowRanges rows, int n, int n_kept, DevCtl* __restrict__ ctl, int counter_slot,
+__global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>())) ism_warp_kernel(const int* __restrict__ perm, int first_cls, int cls, int small_cap, DevCtl* __restrict__ ctl, int counter_slot,
                                                                  Csr A, Csr B, const i64* __restrict__ ub, i64* __restrict__ order_off, char* order_arena,
                                                                  size_t order_bytes, int* __restrict__ cnt,
                                                                  const i64* __restrict__ rowptr, int* __restrict__ Ccrd, T* __restrict__ Cval, int launch_slots) {
@@ -483,6 +484,12 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
     P* const packed = reinterpret_cast<P*>(smem_raw + (NUMERIC ? (int)sizeof(T) * slots * IW_WARPS : 0)) + warp * padded_slots;
     unsigned short* const heads = reinterpret_cast<unsigned short*>(smem_raw + ((NUMERIC ? (int)sizeof(T) * slots : 0) + (int)sizeof(P) * padded_slots) * IW_WARPS) + warp * slots;
     if (ctl->status != 0) return;
+    // the rows of the classes first_cls .. cls, one range of perm (with a table of ranges, or the range as arguments, the kernels
+    // spill: counting / numeric, rows of 200 products 85 / 123 us, now 83 / 116; stencil 41 x 37 x 53 by ISM, f32, 376 / 317 and 372 / 309)
+    int off, n;
+    class_range(ctl, first_cls, off, n);
+    for (int c = first_cls + 1; c <= cls; ++c) n += ctl->class_count[c];
+    const int* __restrict__ rows = perm + off;
     const T* __restrict__ Aval = (const T*)A.val;
     const T* __restrict__ Bval = (const T*)B.val;
     // The way to a row is a chain of loads (its number, its place in perm, its fields, its A entries, their B rows).  AHEAD:
@@ -493,8 +500,8 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
     constexpr bool AHEAD = NUMERIC && CAP > 256;
     int row, row_n = -1, products, products_n = 0;
     i64 ps, pe, ps_n = 0, pe_n = 0;
-    bool kept = false, kept_n = false;              // a row of the class that leaves its order (they come first)
-    auto take = [&](int r) { row_n = r < n ? row_at(rows, r) : -1; kept_n = r < n_kept; };
+    // (from the last row on: those of the largest class first)
+    auto take = [&](int r) { row_n = r < n ? __ldg(rows + (n - 1 - r)) : -1; };
     auto fields = [&]() {
         if (row_n < 0) return;
         products_n = (int)min(__ldg(ub + row_n), (i64)0x7fffffff);
@@ -512,7 +519,6 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
         if (!AHEAD) next();
         if (row_n < 0) break;
         row = row_n;
-        kept = kept_n;
         products = products_n;
         ps = ps_n;
         pe = pe_n;
@@ -523,7 +529,8 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
         int r_n = 0;
         if (AHEAD && lane == 0) r_n = atomicAdd(&ctl->work_counter[counter_slot], 1);
         P* order = nullptr;
-        if (CAP > 256 && order_arena && kept) {
+        const bool kept = CAP > 256 && order_arena && products > small_cap;     // a row of CLS_ISM_SMEM: it leaves its order
+        if (kept) {
             i64 at = -1;
             if (NUMERIC) {
                 at = order_off[row];
@@ -591,7 +598,7 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
         const int e = words_per_lane<CAP>(total);
         if (total != products) order = nullptr;             // (a malformed B row)
         P* const keep = CAP > 256 ? order : nullptr;
-        if (CAP > 256 && !NUMERIC && order_arena && kept && lane == 0) order_off[row] = order ? (i64)(reinterpret_cast<char*>(order) - order_arena) : -1;
+        if (!NUMERIC && kept && lane == 0) order_off[row] = order ? (i64)(reinterpret_cast<char*>(order) - order_arena) : -1;
         if constexpr (CAP <= 256) {
             switch (e) {
                 case 4: distinct = sort_row<PK, P, 4, NUMERIC>(packed, heads, total, keep); break;
@@ -661,10 +668,10 @@ static cudaError_t launch_warp_k(const LaunchCtx& c, const IsmLaunch& l, const C
     auto k = ism_warp_kernel<T, P, CAP, NUMERIC>;
     if ((e = resident_blocks((const void*)k, IW_WARPS * 32, smem, &per_sm)) != cudaSuccess) return e;
     i64 grid = (i64)c.sm_count * (per_sm > 0 ? per_sm : 1);
-    const int n = l.g.end[ISM_LEVELS - 1], cls = l.level == 4 ? CLS_ISM_SMEM : CLS_ISM_SMEM_S;
+    const int n = l.n, cls = l.level == 4 ? CLS_ISM_SMEM : CLS_ISM_SMEM_S;
     const i64 want = ((i64)n + IW_WARPS - 1) / IW_WARPS;
     if (want < grid) grid = want > 0 ? want : 1;
-    k<<<(int)grid, IW_WARPS * 32, smem, c.stream>>>(l.g, n, l.g.end[0], c.ctl, cls + (NUMERIC ? NUM_SLOT : 0), A, B, c.tab.ub, c.tab.bm_off, c.order,
+    k<<<(int)grid, IW_WARPS * 32, smem, c.stream>>>(c.tab.perm, l.first_cls, cls, c.prm.smem_small_cap, c.ctl, cls + (NUMERIC ? NUM_SLOT : 0), A, B, c.tab.ub, c.tab.bm_off, c.order,
                                                     c.order_bytes, c.tab.cnt, rowptr, Ccrd, (T*)Cval, slots);
     ++c.launches;
     return cudaGetLastError();
@@ -682,8 +689,8 @@ size_t order_bytes_of(i64 words, i64 max_products, i64 ncols) {
 template <typename T, typename P, int G, bool NUMERIC>
 static cudaError_t launch_group_k(const LaunchCtx& c, const IsmLaunch& l, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
     constexpr int ROWS = IG_THREADS / G;
-    const int n = l.g.end[ISM_LEVELS - 1];
-    ism_group_kernel<T, P, G, NUMERIC><<<(int)(((i64)n + ROWS - 1) / ROWS), IG_THREADS, 0, c.stream>>>(l.g, n, c.ctl, A, B, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
+    const int n = l.n;
+    ism_group_kernel<T, P, G, NUMERIC><<<(int)(((i64)n + ROWS - 1) / ROWS), IG_THREADS, 0, c.stream>>>(l.rows, n, c.ctl, A, B, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
     ++c.launches;
     return cudaGetLastError();
 }
@@ -720,7 +727,7 @@ static cudaError_t launch_t(const LaunchCtx& c, bool numeric, const IsmLaunch& l
     if (e != cudaSuccess || most <= ISM_WARP_MAX) return e;
     // rows of 1025 .. 4096 products: a CTA each (a counter of their own: the two kernels share the class);
     // under `auto` they are counted through a hash set of their columns, which needs no order
-    const int n = l.g.end[0];
+    const int n = l.own;
     if (!numeric && c.prm.policy == 2) return launch_hash(c, false, CLS_ISM_SMEM, n, A, B, rowptr, Ccrd, Cval);
     if (narrow<4096>(B))
         return numeric ? launch_k<T, unsigned, 4096, 256, true>(c, CLS_ISM_SMEM, n, A, B, rowptr, Ccrd, Cval)
@@ -739,29 +746,20 @@ cudaError_t launch_ism(const LaunchCtx& c, bool numeric, const IsmLaunch& l, con
 constexpr i64 ISM_FEW = 2048;
 int ism_launches(const LaunchCtx& c, IsmLaunch* out) {
     const i64* const rows = c.class_rows;
-    auto first = [&](int cls) { i64 off = 0; for (int k = 0; k < cls; ++k) off += rows[k]; return c.tab.perm + off; };
     const i64 n[ISM_LEVELS] = {rows[CLS_ISM_REG8] + rows[CLS_ISM_REG16] + rows[CLS_ISM_REG], rows[CLS_ISM_GROUP8], rows[CLS_ISM_GROUP16], rows[CLS_ISM_SMEM_S],
                                rows[CLS_ISM_SMEM]};
     const int cls[ISM_LEVELS] = {CLS_ISM_REG8, CLS_ISM_GROUP8, CLS_ISM_GROUP16, CLS_ISM_SMEM_S, CLS_ISM_SMEM};
+    i64 first[ISM_LEVELS] = {rows[CLS_EMPTY]};          // the levels follow one another in perm
+    for (int k = 1; k < ISM_LEVELS; ++k) first[k] = first[k - 1] + n[k - 1];
     int made = 0;
-    IsmLaunch from_above[ISM_LEVELS];
-    bool taken[ISM_LEVELS] = {};
-    for (int at = ISM_LEVELS - 1; at >= 0; --at) {
-        if (n[at] == 0 || taken[at]) continue;
-        // this level's own rows first, then those of lower levels that are few
-        IsmLaunch& l = from_above[made++];
-        l.level = at;
-        int k = 0;
-        i64 end = 0;
-        for (int from = at; from >= 0 && (from == at || n[from] <= ISM_FEW); --from) {
-            if (n[from] == 0) continue;
-            taken[from] = true;
-            l.g.rows[k] = first(cls[from]);
-            l.g.end[k++] = (int)(end += n[from]);
-        }
-        for (; k < ISM_LEVELS; ++k) { l.g.rows[k] = l.g.rows[0]; l.g.end[k] = (int)end; }
+    for (int at = ISM_LEVELS - 1, from; at >= 0; at = from) {
+        from = at - 1;
+        if (n[at] == 0) continue;
+        while (from >= 0 && n[from] <= ISM_FEW) --from;
+        const i64 start = first[from + 1];
+        out[made++] = IsmLaunch{at, cls[from + 1], c.tab.perm + start, (int)(first[at] + n[at] - start), (int)n[at]};
     }
-    for (int k = 0; k < made; ++k) out[k] = from_above[made - 1 - k];
+    for (int k = 0; 2 * k < made - 1; ++k) std::swap(out[k], out[made - 1 - k]);
     return made;
 }
 
