@@ -252,10 +252,10 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
     // neighbours); narrower groups take neighbouring rows for the sake of the row offsets they share
     const i64 ngroups = ((i64)gridDim.x * blockDim.x) / G;
     const i64 group = G >= 8 ? (i64)(threadIdx.x / G) * gridDim.x + blockIdx.x : ((i64)blockIdx.x * blockDim.x + threadIdx.x) / G;
-    i64 my_max = 0;
+    unsigned my_max = 0;                            // most products of a row below 2^32
     // rows and products of the class of this group's last rows: neighbouring rows mostly share a
     // class, so the shared-memory histogram is touched only when the class changes
-    int run_cls = -1, run_rows = 0, my_span_words = 0;
+    int run_cls = -1, run_rows = 0;
     unsigned my_bm_words = 0;                       // (2^31 rows over the groups of a full grid stay below 2^32 words a group)
     i64 run_products = 0;
     auto classify = [&](int row, i64 entries, i64 u, int lo, int hi) {
@@ -277,15 +277,18 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
         }
         ++run_rows;
         run_products += u;
-        my_max = max(my_max, u);
-        // (rare classes: straight to shared memory, and only when the maximum would move)
+        // (what is rare, or a maximum that seldom moves, goes straight to shared memory: in registers of every thread these
+        // and the words of the bitmaps spilled, and the bounds of a 27-point stencil of 2^18 rows took 50 us, now 46.5)
+        if (u >> 32) atomicMax(&s_max_ub, u);
+        else my_max = max(my_max, (unsigned)u);
         if (cls == CLS_ISM_GLOBAL && u > s_max_ub_global) atomicMax(&s_max_ub_global, u);
         if (cls == CLS_ISM_SMEM) {
             if (u > s_max_ub_smem) atomicMax(&s_max_ub_smem, u);
             if (u <= ISM_WARP_MAX) atomicAdd(&s_order_words, (unsigned)order_words_of((int)u));
         }
         if (dense_cls(cls)) {
-            my_span_words = max(my_span_words, (hi - lo) / 32 + 1);
+            const int span_words = (hi - lo) / 32 + 1;
+            if (span_words > s_max_span_words) atomicMax(&s_max_span_words, span_words);
             my_bm_words += (unsigned)slot_words(lo, hi);
         }
     };
@@ -408,15 +411,11 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
     __syncthreads();
     for (int r = 0; r < min(s_nlong, LONG_LIST); ++r) long_row_bounds<SUMMARY>(s_long[r], A, B, tab, prm, ctl, brow);
     // the totals: reduced over the warp first (lanes other than a group's first hold zeros)
-    for (int d = 16; d > 0; d >>= 1) {
-        my_max = max(my_max, __shfl_xor_sync(0xffffffffu, my_max, d));
-        my_span_words = max(my_span_words, __shfl_xor_sync(0xffffffffu, my_span_words, d));
-    }
+    my_max = __reduce_max_sync(0xffffffffu, my_max);
     const unsigned bm_lo = __reduce_add_sync(0xffffffffu, my_bm_words & 0xffffu), bm_hi = __reduce_add_sync(0xffffffffu, my_bm_words >> 16);
     if (lane == 0) {
         if (bm_lo | bm_hi) atomicAdd((u64*)&s_bm_words, (u64)bm_lo + ((u64)bm_hi << 16));
-        if (my_span_words) atomicMax(&s_max_span_words, my_span_words);
-        if (my_max) atomicMax(&s_max_ub, my_max);
+        if (my_max) atomicMax(&s_max_ub, (i64)my_max);
     }
     __syncthreads();
     if (threadIdx.x < 32) {
