@@ -139,7 +139,13 @@ __global__ void __launch_bounds__(OT) higher_total_kernel(int form, int threads,
 cudaError_t launch_higher_total(const LaunchCtx& c, int form, const Csf3Dev& B, const Csr& C, u64* partial, int* blocks) {
     *blocks = 0;
     if (B.n0 == 0) return cudaSuccess;
-    const int threads = (i64)B.n1 >= 256 * (i64)B.n0 ? OT : 32;      // (512 slices of 1000 fibres: a warp each 23 us, a block 12 us)
+    // A block per slice where that takes less than half as many steps as a warp per slice (COUNT_BLOCKS blocks at once; each
+    // slice begins with a chain of loads of its own).  Slices x fibres of each, warps : blocks, us: 512 x 885 23 : 12, 100 x 930 23 : 9, 50 x 2000
+    // 35 : 11, 300 x 300 12 : 9.5, 4000 x 300 14 : 15, 2000 x 420 14 : 17.
+    const i64 fibres = (i64)B.n1 / B.n0 + 1, per_block = OT / 32;
+    auto up = [](i64 x, i64 y) { return (x + y - 1) / y; };
+    const bool by_block = 2 * up(B.n0, COUNT_BLOCKS) * up(fibres, OT) < up(B.n0, COUNT_BLOCKS * per_block) * up(fibres, 32);
+    const int threads = by_block ? OT : 32;
     *blocks = std::min(grid_for(c, (i64)B.n0 * threads, OT), COUNT_BLOCKS);
     higher_total_kernel<<<*blocks, OT, 0, c.stream>>>(form, threads, B, C, partial);
     return cudaGetLastError();
