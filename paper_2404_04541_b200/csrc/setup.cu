@@ -56,7 +56,7 @@ __device__ __forceinline__ int classify_row(i64 ub, i64 entries, int jmin, int j
     const i64 span = (i64)jmax - jmin + 1;
     const i64 span_words = (span + 31) >> 5;
     const bool dense_ok = span_words <= prm.max_span_words;
-    const bool reg_ok = ub <= prm.reg_cap && span <= (1ll << 26);
+    const bool reg_ok = ub <= prm.reg_cap;      // (any span: 2.6e5 rows of 16 products over 2^28 columns, f32, by 8 lanes a row 100 + 111 us, by 4 28 + 41)
     if (prm.policy == 0) {                       // dense forced
         if (!dense_ok) { raise_status(ctl, DEV_WORKSPACE_TOO_LARGE); return CLS_EMPTY; }
         return dense_class(ub, span_words, ctl);
