@@ -635,23 +635,22 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
     for (int cur = 0;; cur ^= 1) {
         const CtaUnit& U = s_unit[cur];
         if (!U.valid) break;
-        const int base = U.base, cnt = U.cnt;
-        const unsigned span_bits = (unsigned)U.nw * 32u;
-        T* const gacc = Cval + U.out0;
         if (!CEIL) {
             if (U.nun == 1)                             // outputs beyond the shared-memory part start at zero
-                for (int x = CAP + tid; x < cnt; x += DN_THREADS) gacc[x] = 0;
+                for (int x = CAP + tid; x < U.cnt; x += DN_THREADS) Cval[U.out0 + x] = 0;
             // the row's bitmap with the rank of every word's first bit (the symbolic pass saved the
-            // rank at every chunk start).  A warp takes four groups of 128 words at a time, all loads first: one scan
-            // per group (a scan per chunk of 32 words: power law on 2^18 / 16381 vertices 12850 / 249 us, now 12650 / 239).
+            // rank at every chunk start).  A warp takes two groups of 128 words at a time, all loads first: one scan
+            // per group.  Power law on 2^18 / 16381 vertices: a scan per chunk of 32 words 12850 / 249 us; four groups at a
+            // time, which spill registers that the accumulation needs, 12650 / 238; two 12380 / 230 (spans of 16384 words and
+            // few outputs pay for the more steps: 10^4 rows of 8192 products 1041, 886, 932 us).
             const unsigned* src = tab.bm_arena + U.bm;
             const int nw = U.nw, nch = chunks_of(nw), ng = (nch + 3) >> 2;
             const uint4* src4 = reinterpret_cast<const uint4*>(src);         // slots are 16-byte aligned
-            for (int g0 = warp; g0 < ng; g0 += DN_WARPS * 4) {
-                uint4 word[4];
-                unsigned rank_g[4];
+            for (int g0 = warp; g0 < ng; g0 += DN_WARPS * 2) {
+                uint4 word[2];
+                unsigned rank_g[2];
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
+                for (int x = 0; x < 2; ++x) {
                     const int g = g0 + x * DN_WARPS, w0 = (g << 7) + (lane << 2);
                     word[x] = make_uint4(0u, 0u, 0u, 0u);
                     if (w0 < nw) {
@@ -663,7 +662,7 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
                     rank_g[x] = (g < ng) ? src[nw + (g << 2)] : 0u;
                 }
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
+                for (int x = 0; x < 2; ++x) {
                     const int g = g0 + x * DN_WARPS, w0 = (g << 7) + (lane << 2);
                     const int p0 = __popc(word[x].x), p1 = p0 + __popc(word[x].y), p2 = p1 + __popc(word[x].z), p3 = p2 + __popc(word[x].w);
                     const unsigned r = rank_g[x] + (unsigned)(warp_incl_scan(p3) - p3) - 1u;
@@ -680,6 +679,9 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
             }
         }
 
+        const int base = U.base, cnt = U.cnt;
+        const unsigned span_bits = (unsigned)U.nw * 32u;
+        T* const gacc = Cval + U.out0;
         auto add = [&](unsigned rel, T v) {
             if (CEIL) {
                 if (rel != 0xffffffffu) { my_idx += (u64)(rel + (unsigned)base); my_val += (double)v; }
