@@ -169,7 +169,11 @@ typedef struct {
     int64_t bitmap_bytes;     /* bytes of the bitmap arena in use                                 */
 } spws_stats_t;
 
-/* Kernel groups timed by spws_set_profiling (index into the array spws_get_timings fills). */
+/* Kernel groups timed by spws_set_profiling (index into the array spws_get_timings fills).  A group is a kernel's time,
+ * and the few rows of a sparse class that go along with the next larger kernel are timed with it: the group of such a
+ * class can read 0 although rows_per_class counts rows.  Those kernels are, with the products a row has at most: four lanes
+ * a row (32: ISM_REG), eight and sixteen lanes and a warp (64, 128, 256: ISM_SMEM_S), a warp and a CTA (1024,
+ * ism_cta_cap: ISM_SMEM).  SPWS_T_NUM_ISM_REG also holds the rows that are copied. */
 enum {
     SPWS_T_SYM_BOUNDS = 0,    /* per-row upper bound, span and class                               */
     SPWS_T_SYM_BIN = 1,       /* binning + dense work units                                        */
