@@ -154,18 +154,18 @@ __global__ void __launch_bounds__(THREADS) ism_smem_kernel(const int* __restrict
 // products, this one about 2.7.  Bound by instruction issue.
 //   Insert : 32 A entries at a time; a group of lanes per entry (as many as the mean B row has
 //            entries) writes the products of its B row at their slots.
-//   Sort   : E = 4, 6, 8, 12, 16, 24 or 32 words per lane, the smallest network that holds the row.
+//   Sort   : E = 6, 8, 12, 16, 24 or 32 words per lane, the smallest network that holds the row (four for the few rows of up to
+//            128 products that go along with longer ones).
 //   Merge  : the sorted words go back to shared memory, the places of the run heads are packed, and
 //            one lane per run sums it in slot order.
 //   Of rows of more than 256 products the counting pass leaves the sorted words in scratch when there is room
 // (coalesced: word x of lane l at x * lanes + l, lanes past the last word left out), and the numeric pass then only
 // fetches the values: 8e4 rows of 674 products, f32: count 507 -> 578 us, numeric 871 -> 400 us; 2e5 rows
-// of 470, f64: 154 -> 210 and 494 -> 225 us.  Shorter rows gain nothing (fibres of about 110 products: numeric 104 us with
-// and without, count 82 -> 100 us), their sort is a small part of the work.
+// of 470, f64: 154 -> 210 and 494 -> 225 us.  Shorter rows gain nothing, their sort is a small part of the work.
 // Stencil 41 x 37 x 53 (f32, 674 products a row): count 1714 -> 508 us, numeric 1905 -> 863 us against a CTA per
-// row; 59-product rows of the outer form (2e5 of them): 259 -> 125 us (hash set) and 439 -> 146 us.  With sizes of
-// three times a power of two, long merges as loops and lane groups found by shifts: count 578 -> 384 us on
-// the stencil (370 us numeric, 312 since), 210 -> 172 us on the rows of 470; 143-product rows (3e4): 44 -> 37 and 55 -> 50 us.
+// row.  With sizes of three times a power of two, long merges as loops and lane groups found by shifts: count 578 -> 384 us
+// on the stencil (372 since; numeric 370, 309 since), 210 -> 172 us on the rows of 470; 143-product rows (3e4): 44 -> 36
+// and 55 -> 49 us.
 // ---------------------------------------------------------------------------------------
 constexpr int IW_WARPS = 4;
 
@@ -294,7 +294,8 @@ __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int to
 // on eight, four or two of them at a time.
 //   Insert : G entries at a time; lane l takes the products l, l + G, .. of those entries, whose owners it finds by a search
 //            among the running counts.
-//   Sort   : six or eight words per lane in registers (two or four where no row of a warp of four-lane groups has more); the narrower the group, the more of the network stays inside the lanes.
+//   Sort   : six or eight words per lane in registers; with four lanes a row two or four where no row of the warp has more.
+//            The narrower the group, the more of the network stays inside the lanes.
 //   Merge  : as below: the sorted words and the places of the run heads go to shared memory, a lane per run.
 // Every step of the way to a row's products is a load that waits for the one before: several rows per warp and some 40 warps
 // keep enough of them in flight, and a block for every 128 lanes' rows spares fetching ahead (persistent blocks: numeric 80 us
@@ -302,6 +303,8 @@ __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int to
 // against this, count + numeric: 2e5 rows of 59 products, f32, 123 + 148 and 92 + 128 us; 1.6e5 fibres of 110, 95 + 108 and 64 + 93
 // us; 1.9e5 rows of 82, f64, 137 + 178 and 99 + 144 us.  Rows of at most 32 products had as many lanes as products before: 1.2e5
 // rows of 16 .. 24, f64, 22 + 45 and 12 + 40 us; 65536 rows of 16 whose B rows come from memory, 18 + 25 and 16 + 26 us.
+// Words of 64 bits (four lanes: from 2^27 columns on): 2.6e5 rows of 16 products, f32, 28 + 38 us, where the register kernel with
+// columns relative to the row's first took 40 + 48; words of 32 bits 18 + 30.
 // ---------------------------------------------------------------------------------------
 constexpr int IG_THREADS = 128;
 
@@ -741,8 +744,10 @@ cudaError_t launch_ism(const LaunchCtx& c, bool numeric, const IsmLaunch& l, con
 }
 
 // A kernel takes any row with fewer products than its own as well, at more instructions a row, and a launch for a handful of rows
-// costs 4 .. 10 us: no more than ISM_FEW rows go along with those of the next larger kernel that has rows of its own (stencil
-// 41 x 37 x 53, 3e3 rows at its edges: a call 824 us with a launch for each class, 796 us).
+// costs 4 .. 10 us: a kernel with no more than ISM_FEW rows leaves them to the next larger one that has rows of its own.  Stencil
+// 41 x 37 x 53, 3e3 rows at its edges: a call 824 us with a launch for each class, 796 us.  2000 rows each of 16, 60, 100 and
+// 200 products go along with 2100 rows of 400 in 23 + 29 us, and with 50 such rows in 16 + 23, where a kernel each (no lane
+// groups then) took 29 + 39 and 24 + 30; 2000 rows of 16 beside 3e4 of 900: 207 + 268 us, 211 + 274.
 constexpr i64 ISM_FEW = 2048;
 int ism_launches(const LaunchCtx& c, IsmLaunch* out) {
     const i64* const rows = c.class_rows;

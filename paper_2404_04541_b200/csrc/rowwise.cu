@@ -59,7 +59,8 @@ __global__ void __launch_bounds__(OT) rw_keys_outer_kernel(Csr At, i64 n, Csr B,
     if (bad) raise_status(ctl, DEV_NONCANONICAL);
 }
 
-// pos[0 .. m] := nnz on the way (rw_sparse_rows_kernel writes the rows there are).  form: 0 SpTTM, 1 SpTTM-I, 2 SpMTTKRP.  `d` = extent of the label's inner coordinate (forms 0, 1).
+// form: 0 SpTTM, 1 SpTTM-I, 2 SpMTTKRP.  `d` = extent of the label's inner coordinate (forms 0, 1).
+// pos[0 .. m] := nnz on the way (rw_sparse_rows_kernel writes the rows there are).
 __global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u64 d, u64* __restrict__ keys, u64* __restrict__ pay, int passes,
                                                          SortHead* head, i64* __restrict__ pos, i64 m) {
     __shared__ int s_f[2], s_s[2];
