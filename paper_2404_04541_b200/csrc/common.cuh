@@ -85,6 +85,7 @@ struct DevCtl {
     int n_units;            // numeric dense CTA units (row, share of its entries)
     int units_of[7];        // units per bucket of rows (counted by the binning, without the rows that outgrow a warp) ...
     int unit_cursor[7];     // ... and units numbered so far
+    int sym_units[2];       // symbolic dense CTA units: shares of split rows, whole rows
     int n_warp_rows[N_WARP_LISTS];  // numeric dense warp rows by the accumulator they need
     int max_span_words;     // widest bitmap among the dense rows
     int max_warp_cnt[N_WARP_LISTS]; // most outputs of a row on each list
@@ -155,8 +156,8 @@ struct RowTables {
     i64* bm_off;        // word offset of the row's bitmap in the arena (dense classes); byte offset of its sorted words (CLS_ISM_SMEM)
     unsigned* bm_arena;
     int* warp_rows;     // numeric: rows handled by the warp-per-row dense kernel: list 0 from the front, list 1 from the back
-    int* row_unit0;     // numeric: first CTA unit of a row
-    int* unit_row;      // numeric: row of a CTA unit
+    int* row_unit0;     // first CTA unit of a row: symbolic (split rows), then numeric
+    int* unit_row;      // row of a CTA unit: symbolic (shares of split rows from the front, whole rows from the back), then numeric
 };
 
 // Products one dense CTA unit should take: `least`, by default 2^16 (measured on the power-law workload: units
@@ -190,6 +191,14 @@ __host__ __device__ inline int dense_units_of_row(i64 ub, i64 unit_products) {
     const i64 n = (ub + unit_products - 1) / unit_products;
     return (int)(n < 1 ? 1 : n);
 }
+
+// Symbolic CTA units: a row with more than a 4096th of the products of its kind (about a quarter of what a block of a full grid
+// takes in all) is shared by several blocks, which otherwise wait for the one that has it (a 2048th / 16384th: power law on 2^18
+// vertices 2806 / 2644 us, 2621 like this), but not below 4096 products (8192 / 2048: 4001 vertices 31 / 25 us, 21 like this;
+// 1500 vertices 27 / 16, 20).
+constexpr i64 SYM_PART_LEAST = 4096;
+inline i64 sym_part_products(i64 cta_products) { return cta_products >> 12 > SYM_PART_LEAST ? cta_products >> 12 : SYM_PART_LEAST; }
+__device__ __forceinline__ int sym_parts_of_row(i64 ub, i64 part_products) { return (int)((ub + part_products - 1) / part_products); }
 
 // What a plan keeps in pinned host memory: the control block as last read back, and one slot per
 // block of the counting kernels, which write their partial sums there and the host adds up.
@@ -405,7 +414,9 @@ cudaError_t resident_blocks(const void* kernel, int threads, size_t smem, int* p
 cudaError_t launch_validate(const LaunchCtx& c, const Csr& A, const Csr& B, i64 nnzA, i64 nnzB);
 // clear_ctl: the control block is cleared by the first kernel
 cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i64 nnzA, bool clear_ctl);
-cudaError_t launch_bw_build(const LaunchCtx& c, const Csr& B);
+// symbolic units of the CTA rows; word lists of long B rows
+// (products: of the CTA rows)
+cudaError_t launch_cta_prepare(const LaunchCtx& c, i64 products, const Csr& B);
 // (also publishes the class sizes to the host)
 cudaError_t launch_bin_rows(const LaunchCtx& c, int m);
 // row pointer, numeric routing of the dense rows, outputs per class
@@ -435,7 +446,7 @@ cudaError_t launch_ism(const LaunchCtx& c, bool numeric, const IsmLaunch& l, con
 size_t order_bytes_of(i64 words, i64 max_products, i64 ncols);
 // max_span_words: widest dense row of the pass
 cudaError_t launch_dense_sym_warp(const LaunchCtx& c, int max_span_words, const Csr& A, const Csr& B);
-cudaError_t launch_dense_sym_cta(const LaunchCtx& c, const Csr& A, const Csr& B);
+cudaError_t launch_dense_sym_cta(const LaunchCtx& c, i64 products, const Csr& A, const Csr& B);
 // chk_idx / chk_val non-null: the gather-only form of the same kernel (workspace stripped, checksums out).
 // n[], max_cnt[]: rows on each list and their largest output counts
 cudaError_t launch_dense_num_warp(const LaunchCtx& c, const int* n, const int* max_cnt, int m, int max_span_words, const Csr& A, const Csr& B,

@@ -205,155 +205,231 @@ __global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __re
 }
 
 // ---------------------------------------------------------------------------------------
-// symbolic, CTA per row (hub rows first: classes HUB and CTA are adjacent in perm)
-// Bound by latency: chains of loads and the barriers of short rows.  With entries dealt out in turn, eight barriers per row
-// and a chain of four loads per entry, power law on 2^18 / 60000 / 16381 vertices: 3149 / 726 / 193 us; now 2815 /
-// 622 / 183 us.
+// symbolic, CTA units.  A unit is a row, or an equal share of the A entries of a row with a large part of all products,
+// whose blocks unite their bitmaps in the arena; the last of them counts.
+// Bound by latency at few vertices, by the shared-memory atomics and instruction issue at many.  Warps that pulled batches of A
+// entries of a row walked a chain of four loads per batch and had one B row's loads in flight; the entries of a round are
+// now looked up by all threads at once and the warps pull tiles of the stream of their elements, each with 128 loads in flight
+// whatever the length of the B rows.  Power law on 16381 / 60000 / 2^18 vertices: 201 / 622 / 2681 us by batches, one block a
+// row, 78 / 415 / 2621 us now.
 // ---------------------------------------------------------------------------------------
-// What a block needs to know of a row, fetched by one thread while the block is busy with the row before.
-struct SymRow {
-    i64 ps, pe, bm;
-    int row, base, nw, lg, batch, whole;       // row < 0: no more rows
+constexpr int DS_ENTRIES = DC_THREADS;      // A entries whose descriptors are staged per round
+// elements a warp takes per fetch: a 64th of the round's, so that the warps finish together (at most 1024 / 2048 / 4096: power law on
+// 2^18 vertices 2648 / 2621 / 2624 us)
+constexpr int DS_TILE = 256, DS_TILE_MOST = 2048;
+
+// What a block needs to know of a unit, fetched by one thread while the block is busy with the unit before.
+struct SymUnit {
+    i64 e_lo, e_hi, bm;
+    int row, base, nw, parts;                  // row < 0: no more units
 };
 
-__global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __restrict__ ctl, int smem_words, Csr A, Csr B, RowTables tab,
+__global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __restrict__ ctl, int smem_words, int unit_cap, i64 part_products, Csr A, Csr B, RowTables tab,
                                                                    const uint2* __restrict__ bw) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    unsigned* bm = reinterpret_cast<unsigned*>(smem_raw);                 // smem_words, clear between rows
-    int* chunk = reinterpret_cast<int*>(bm + smem_words);                  // smem_words / 32
-    __shared__ SymRow s_row[2];
-    __shared__ int s_entry[2];                                              // batches of A entries handed out
+    unsigned* bm = reinterpret_cast<unsigned*>(smem_raw);                 // smem_words, clear between units
+    int* chunk = reinterpret_cast<int*>(bm + smem_words);                  // smem_words / 32 + 1
+    // staged descriptors: twice the start of the B row, or of its word list and one; elements of the entries before
+    __shared__ i64 d_q[DS_ENTRIES];
+    __shared__ int d_pre[DS_ENTRIES + 1], ws[DC_WARPS];
+    __shared__ SymUnit s_unit[2];
+    __shared__ int s_tile, s_last;
     if (ctl->status != 0) return;
-    int off, n_hub, o6, n_cta;
-    class_range(ctl, CLS_DENSE_HUB, off, n_hub);
-    class_range(ctl, CLS_DENSE_CTA, o6, n_cta);
-    const int n = n_hub + n_cta;
+    const int n_split = ctl->sym_units[0], n = n_split + ctl->sym_units[1];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    auto fetch_row = [&](int to) {                      // one thread
-        SymRow& R = s_row[to];
-        const int r = atomicAdd(&ctl->work_counter[CLS_DENSE_CTA], 1);
-        s_entry[to] = 0;
-        R.row = -1;
-        if (r >= n) return;
-        const int row = tab.perm[off + r], base = tab.jmin[row];
-        R.ps = A.pos[row];
-        R.pe = A.pos[row + 1];
-        R.bm = tab.bm_off[row];
-        R.nw = min((tab.jmax[row] - base) / 32 + 1, smem_words);
-        const i64 ub = tab.ub[row], entries = R.pe - R.ps;
-        R.lg = pick_group_log(ub, entries);
-        R.batch = ub < 512 * entries ? 8 : 4;
-        R.whole = (int)(entries * 3 / 4) / R.batch;         // batches of that size; pairs for the last quarter, so that
-                                                            // the warps finish together (2915 -> 2815 us on 2^18 vertices)
-        R.base = base;
-        R.row = row;
+    auto fetch_unit = [&](SymUnit& U) {                 // one thread
+        const int t = atomicAdd(&ctl->work_counter[CLS_DENSE_CTA], 1);
+        U.row = -1;
+        if (t >= n) return;
+        const int u = t < n_split ? t : unit_cap - 1 - (t - n_split);
+        const int row = tab.unit_row[u], base = tab.jmin[row];
+        const i64 ps = A.pos[row], entries = A.pos[row + 1] - ps;
+        int part = 0, parts = 1;
+        if (t < n_split) {
+            part = u - tab.row_unit0[row];
+            parts = sym_parts_of_row(tab.ub[row], part_products);
+        }
+        U.bm = tab.bm_off[row];
+        U.nw = min((tab.jmax[row] - base) / 32 + 1, smem_words);
+        U.e_lo = ps + entries * part / parts;
+        U.e_hi = ps + entries * (part + 1) / parts;
+        U.parts = parts;
+        U.base = base;
+        U.row = row;
     };
-    if (tid == 0) fetch_row(0);
+    if (tid == 0) fetch_unit(s_unit[0]);
     for (int w = tid; w < smem_words; w += DC_THREADS) bm[w] = 0;
     __syncthreads();
-    // two barriers per row: before the bitmap is saved (and cleared), and after
     for (int cur = 0;; cur ^= 1) {
-        const SymRow& R = s_row[cur];
-        if (R.row < 0) break;
-        const int base = R.base, nw = R.nw, lg = R.lg, gs = 1 << lg;
-        const unsigned span = (unsigned)nw * 32u;
+        const SymUnit& U = s_unit[cur];
+        if (U.row < 0) break;
+        const int base = U.base, nw = U.nw;
         const unsigned base_w = (unsigned)base >> 5;                     // base is a multiple of 32
-        const i64 ps = R.ps, pe = R.pe;
-        if (tid == DC_THREADS - 1) fetch_row(cur ^ 1);
-        __syncwarp();
-        // one B row by `gs` lanes, of which this is lane gl
-        auto take = [&](i64 qs, int len, int np, int gl, int gs) {
-            if (np > 0) {
-                // a long B row with a word list: one atomic per (word, bits) pair, and the lanes hold distinct words
-                const uint2* __restrict__ pk = bw + qs + 1;
-                int t = gl;
-                for (; t + 3 * gs < np; t += 4 * gs) {
-                    const uint2 e0 = __ldg(pk + t), e1 = __ldg(pk + t + gs), e2 = __ldg(pk + t + 2 * gs), e3 = __ldg(pk + t + 3 * gs);
-                    const unsigned w0 = e0.x - base_w, w1 = e1.x - base_w, w2 = e2.x - base_w, w3 = e3.x - base_w;
-                    if (w0 < (unsigned)nw) atomicOr(&bm[w0], e0.y);
-                    if (w1 < (unsigned)nw) atomicOr(&bm[w1], e1.y);
-                    if (w2 < (unsigned)nw) atomicOr(&bm[w2], e2.y);
-                    if (w3 < (unsigned)nw) atomicOr(&bm[w3], e3.y);
-                }
-                for (; t < np; t += gs) {
-                    const uint2 e0 = __ldg(pk + t);
-                    const unsigned w0 = e0.x - base_w;
-                    if (w0 < (unsigned)nw) atomicOr(&bm[w0], e0.y);
-                }
-                return;
-            }
-            const int* __restrict__ ck = B.crd + qs;
-            int t = gl;
-            for (; t + 3 * gs < len; t += 4 * gs) {     // four loads in flight per lane
-                const unsigned r0 = (unsigned)(__ldg(ck + t) - base);
-                const unsigned r1 = (unsigned)(__ldg(ck + t + gs) - base);
-                const unsigned r2 = (unsigned)(__ldg(ck + t + 2 * gs) - base);
-                const unsigned r3 = (unsigned)(__ldg(ck + t + 3 * gs) - base);
-                if (r0 < span) atomicOr(&bm[r0 >> 5], 1u << (r0 & 31));
-                if (r1 < span) atomicOr(&bm[r1 >> 5], 1u << (r1 & 31));
-                if (r2 < span) atomicOr(&bm[r2 >> 5], 1u << (r2 & 31));
-                if (r3 < span) atomicOr(&bm[r3 >> 5], 1u << (r3 & 31));
-            }
-            for (; t < len; t += gs) {
-                const unsigned r0 = (unsigned)(__ldg(ck + t) - base);
-                if (r0 < span) atomicOr(&bm[r0 >> 5], 1u << (r0 & 31));
-            }
-        };
-        if (gs == 32) {
-            const int full = R.batch, whole = R.whole;
-            // warps pull a batch of entries at a time: the chain of loads that leads to a B row is walked for all of
-            // them side by side, and no warp waits for one that met the longest B rows.  Eight entries, four
-            // when their B rows are long (whole batches weigh more than the chain then): power law on 2^18
-            // vertices 3350 us with eight, 2870 with four, 2900 with two; on 60000 620, 670 and 750 us
-            for (;;) {
-                int at = 0;
-                if (lane == 0) at = atomicAdd(&s_entry[cur], 1);
-                at = __shfl_sync(0xffffffffu, at, 0);
-                const int batch = at < whole ? full : 2;
-                at = at < whole ? at * full : whole * full + (at - whole) * 2;
-                if (at >= pe - ps) break;
-                i64 my_qs = 0;
-                int my_len = 0, my_np = 0;
-                if (lane < batch && ps + at + lane < pe) {
-                    const int k = __ldg(A.crd + ps + at + lane);
-                    if ((unsigned)k < (unsigned)B.nrows) {
-                        my_qs = __ldg(B.pos + k);
-                        my_len = (int)(__ldg(B.pos + k + 1) - my_qs);
-                        if (bw && my_len >= BW_MIN_LEN) my_np = (int)__ldg(&bw[my_qs].x);
+        const i64 e_hi = U.e_hi;
+        bool next_known = false;
+        // Rounds of DS_ENTRIES A entries, one per thread: a block scan turns the lengths of the B rows (or of their word
+        // lists) into a running count, and warps pull tiles of that stream.
+        for (i64 e0 = U.e_lo; e0 < e_hi; e0 += DS_ENTRIES) {
+            const int nE = (int)min((i64)DS_ENTRIES, e_hi - e0);
+            int len = 0;
+            if (tid < nE) {
+                const int k = __ldg(A.crd + e0 + tid);
+                i64 q = 0;
+                if ((unsigned)k < (unsigned)B.nrows) {
+                    const i64 qs = __ldg(B.pos + k);
+                    len = (int)(__ldg(B.pos + k + 1) - qs);
+                    q = 2 * qs;
+                    if (bw && len >= BW_MIN_LEN) {
+                        const int np = (int)__ldg(&bw[qs].x);
+                        if (np > 0) { len = np; q = 2 * (qs + 1) + 1; }
                     }
                 }
-                const int nE = (int)min((i64)batch, pe - ps - at);
-                for (int i = 0; i < nE; ++i) {
-                    const i64 qs = __shfl_sync(0xffffffffu, my_qs, i);
-                    const int len = __shfl_sync(0xffffffffu, my_len, i), np = __shfl_sync(0xffffffffu, my_np, i);
-                    take(qs, len, np, lane, 32);
+                d_q[tid] = q;
+            }
+            const int incl = warp_incl_scan(len);
+            if (lane == 31) ws[warp] = incl;
+            __syncthreads();
+            const int wt = lane < DC_WARPS ? ws[lane] : 0;
+            const int wi = warp_incl_scan(wt);
+            const int total = __shfl_sync(0xffffffffu, wi, 31);
+            const int excl = __shfl_sync(0xffffffffu, wi - wt, warp) + incl - len;
+            if (tid < nE) d_pre[tid] = excl;
+            if (tid == 0) { d_pre[nE] = total; s_tile = 0; }
+            __syncthreads();
+            if (!next_known && tid == DC_THREADS - 1) fetch_unit(s_unit[cur ^ 1]);
+            next_known = true;
+            __syncwarp();
+            const bool long_rows = total >= 64 * nE;
+            const int tile = min(max((total >> 6) & ~127, DS_TILE), DS_TILE_MOST);
+            for (;;) {
+                int t0 = 0;
+                if (lane == 0) t0 = atomicAdd(&s_tile, tile);
+                t0 = __shfl_sync(0xffffffffu, t0, 0);
+                if (t0 >= total) break;
+                const int t1 = min(total, t0 + tile);
+                // the last entry whose running count is <= t0: among 32 spread entries, then among those in between
+                constexpr int STRIDE = DS_ENTRIES / 32;
+                const int i1 = lane * STRIDE;
+                const int lo = (__popc(__ballot_sync(0xffffffffu, i1 < nE && d_pre[i1] <= t0)) - 1) * STRIDE;
+                const int i2 = lo + lane;
+                int e = lo + __popc(__ballot_sync(0xffffffffu, lane < STRIDE && i2 < nE && d_pre[i2] <= t0)) - 1;
+                if (long_rows) {
+                    // the tile's part of one B row after the other, 128 elements a step, four per lane, all loads first
+                    while (t0 < t1) {
+                        int next = d_pre[e + 1];
+                        while (next <= t0) next = d_pre[++e + 1];
+                        int m = min(t1, next) - t0;
+                        const i64 d = d_q[e];
+                        const i64 q = (d >> 1) + (t0 - d_pre[e]) + lane;
+                        t0 += m;
+                        if (d & 1) {
+                            auto set = [&](uint2 v) {
+                                const unsigned w = v.x - base_w;
+                                if (w < (unsigned)nw) atomicOr(&bm[w], v.y);
+                            };
+                            const uint2* __restrict__ pk = bw + q;
+                            for (; m >= 128; m -= 128, pk += 128) {
+                                const uint2 v0 = __ldg(pk), v1 = __ldg(pk + 32), v2 = __ldg(pk + 64), v3 = __ldg(pk + 96);
+                                set(v0); set(v1); set(v2); set(v3);
+                            }
+                            if (m > 0) {
+                                uint2 v[4];
+#pragma unroll
+                                for (int x = 0; x < 4; ++x) v[x] = lane + 32 * x < m ? __ldg(pk + 32 * x) : make_uint2(base_w - 1u, 0u);
+#pragma unroll
+                                for (int x = 0; x < 4; ++x) set(v[x]);
+                            }
+                        } else {
+                            auto set = [&](int c) {
+                                const unsigned rel = (unsigned)(c - base);
+                                if (rel < (unsigned)nw * 32u) atomicOr(&bm[rel >> 5], 1u << (rel & 31));
+                            };
+                            const int* __restrict__ ck = B.crd + q;
+                            for (; m >= 128; m -= 128, ck += 128) {
+                                const int c0 = __ldg(ck), c1 = __ldg(ck + 32), c2 = __ldg(ck + 64), c3 = __ldg(ck + 96);
+                                set(c0); set(c1); set(c2); set(c3);
+                            }
+                            if (m > 0) {
+                                int c[4];
+#pragma unroll
+                                for (int x = 0; x < 4; ++x) c[x] = lane + 32 * x < m ? __ldg(ck + 32 * x) : base - 1;
+#pragma unroll
+                                for (int x = 0; x < 4; ++x) set(c[x]);
+                            }
+                        }
+                    }
+                } else {
+                    // short B rows: a step = 128 consecutive elements of the stream, four per lane; every lane advances its
+                    // own entry index across row boundaries
+                    for (; t0 < t1; t0 += 128) {
+                        unsigned w[4], bits[4];
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) {
+                            const int t = t0 + lane + 32 * x;
+                            w[x] = 0xffffffffu;
+                            bits[x] = 0u;
+                            if (t < t1) {
+                                while (d_pre[e + 1] <= t) ++e;
+                                const i64 d = d_q[e];
+                                const i64 q = (d >> 1) + (t - d_pre[e]);
+                                if (d & 1) {
+                                    const uint2 v = __ldg(bw + q);
+                                    w[x] = v.x - base_w;
+                                    bits[x] = v.y;
+                                } else {
+                                    const unsigned rel = (unsigned)(__ldg(B.crd + q) - base);
+                                    w[x] = rel >> 5;
+                                    bits[x] = 1u << (rel & 31);
+                                }
+                            }
+                        }
+#pragma unroll
+                        for (int x = 0; x < 4; ++x)
+                            if (w[x] < (unsigned)nw) atomicOr(&bm[w[x]], bits[x]);
+                    }
                 }
             }
-        } else {
-            const int g = tid >> lg, gl = tid & (gs - 1), ng = DC_THREADS >> lg;
-            for (i64 p = ps + g; p < pe; p += ng) {
-                const int k = __ldg(A.crd + p);
-                if ((unsigned)k >= (unsigned)B.nrows) continue;
-                const i64 qs = __ldg(B.pos + k);
-                const int len = (int)(__ldg(B.pos + k + 1) - qs);
-                take(qs, len, bw && len >= BW_MIN_LEN ? (int)__ldg(&bw[qs].x) : 0, gl, gs);
-            }
+            __syncthreads();
         }
-        __syncthreads();
+        if (!next_known) {                              // a share without entries
+            __syncthreads();
+            if (tid == 0) fetch_unit(s_unit[cur ^ 1]);
+            __syncthreads();
+        }
         // save the bitmap, then the rank at every chunk start
-        unsigned* out = tab.bm_arena + R.bm;
-        const int nch = chunks_of(nw), row = R.row;
-        // four words a lane, eight lanes a chunk (words past the span are clear; a slot holds a multiple of four words); a word a
-        // lane: power law on 2^18 vertices 2820 us, now 2740
+        unsigned* out = tab.bm_arena + U.bm;
+        const int nch = chunks_of(nw), row = U.row, parts = U.parts;
         uint4* const bm4 = reinterpret_cast<uint4*>(bm);
         uint4* const out4 = reinterpret_cast<uint4*>(out);
+        if (parts > 1) {
+            for (int q = tid; 4 * q < nw; q += DC_THREADS) {
+                const uint4 v = bm4[q];
+                if (v.x) atomicOr(out + 4 * q, v.x);
+                if (v.y) atomicOr(out + 4 * q + 1, v.y);
+                if (v.z) atomicOr(out + 4 * q + 2, v.z);
+                if (v.w) atomicOr(out + 4 * q + 3, v.w);
+                bm4[q] = make_uint4(0u, 0u, 0u, 0u);
+            }
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) s_last = atomicAdd(&tab.cnt[row], 1) == parts - 1;       // (the bounds kernel left a zero)
+            __syncthreads();
+            if (!s_last) continue;
+            __threadfence();
+        }
+        // four words a lane, eight lanes a chunk (words past the span are clear; a slot holds a multiple of four words); a word a
+        // lane: power law on 2^18 vertices 2820 us, 2740 like this
         for (int q0 = warp * 32; q0 < nch * 8; q0 += DC_WARPS * 32) {
             const int q = q0 + lane;
             uint4 v = make_uint4(0u, 0u, 0u, 0u);
             if (4 * q < nw) {
-                v = bm4[q];
-                out4[q] = v;
-                bm4[q] = make_uint4(0u, 0u, 0u, 0u);
+                if (parts > 1) {
+                    v = __ldcg(out4 + q);
+                } else {
+                    v = bm4[q];
+                    out4[q] = v;
+                    bm4[q] = make_uint4(0u, 0u, 0u, 0u);
+                }
             }
             int pc = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
             pc += __shfl_xor_sync(0xffffffffu, pc, 1);
@@ -362,7 +438,7 @@ __global__ void __launch_bounds__(DC_THREADS, 6) dense_sym_cta_kernel(DevCtl* __
             if ((lane & 7) == 0 && (q >> 3) < nch) chunk[q >> 3] = pc;
         }
         __syncthreads();
-        if (warp == 0) {                                // the others go on with the next row
+        if (warp == 0) {                                // the others go on with the next unit
             int carry = 0;
             for (int c0 = 0; c0 < nch; c0 += 32) {
                 const int v = c0 + lane < nch ? chunk[c0 + lane] : 0;
@@ -968,12 +1044,13 @@ cudaError_t launch_dense_sym_warp(const LaunchCtx& c, int max_span_words, const 
     return cudaGetLastError();
 }
 
-cudaError_t launch_dense_sym_cta(const LaunchCtx& c, const Csr& A, const Csr& B) {
+cudaError_t launch_dense_sym_cta(const LaunchCtx& c, i64 products, const Csr& A, const Csr& B) {
     const size_t smem = (size_t)c.dense_smem_words * 4 + (size_t)(c.dense_smem_words / 32 + 1) * 4;
     cudaError_t e;
     int per_sm = 0;
     if ((e = resident_blocks((const void*)dense_sym_cta_kernel, DC_THREADS, smem, &per_sm)) != cudaSuccess) return e;
-    dense_sym_cta_kernel<<<persistent_grid(c, per_sm, -1), DC_THREADS, smem, c.stream>>>(c.ctl, c.dense_smem_words, A, B, c.tab, c.bw);
+    dense_sym_cta_kernel<<<persistent_grid(c, per_sm, -1), DC_THREADS, smem, c.stream>>>(c.ctl, c.dense_smem_words, c.prm.unit_cap, sym_part_products(products), A, B,
+                                                                                                c.tab, c.bw);
     ++c.launches;
     return cudaGetLastError();
 }

@@ -1,5 +1,6 @@
 // Symbolic-pass set-up kernels: input validation, per-row product upper bound and column
 // span, routing of rows to workspaces (binning), exclusive scans, CSF level rebuild.
+#include <algorithm>
 #include "common.cuh"
 
 namespace spws {
@@ -488,8 +489,52 @@ cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i6
 // 20, 80, 54, 281; 3000 rows of 4000 60, with 1024 69, by a warp 150.)
 constexpr int BW_BLOCK_ROW = 1024;
 constexpr int BW_FEW = 2048;
-__global__ void __launch_bounds__(256) bw_find_long_kernel(Csr B, int* __restrict__ bw_long, int cap, DevCtl* ctl) {
-    for (i64 k = (i64)blockIdx.x * blockDim.x + threadIdx.x; k < B.nrows; k += (i64)gridDim.x * blockDim.x) {
+// Also numbers the symbolic units of the CTA rows (`rows`, n of them), and clears the slots of those that are split, in which their
+// blocks will unite their bitmaps.
+constexpr int CP_THREADS = 256;
+__global__ void __launch_bounds__(CP_THREADS) cta_prepare_kernel(Csr B, int* __restrict__ bw_long, int cap, const int* __restrict__ rows, int n, i64 part_products,
+                                                                int unit_cap, RowTables tab, DevCtl* ctl) {
+    __shared__ i64 s_slot[CP_THREADS];
+    __shared__ int s_quads[CP_THREADS], s_n[3], s_base[2];          // shares of split rows, whole rows, split rows of the block
+    if (ctl->status != 0) return;
+    const int tid = threadIdx.x, lane = tid & 31;
+    // (neighbours in perm go to different blocks: the rows to be split are often neighbours)
+    for (i64 r0 = 0; r0 + blockIdx.x < n; r0 += (i64)gridDim.x * CP_THREADS) {
+        const i64 r = r0 + (i64)tid * gridDim.x + blockIdx.x;
+        const int row = r < n ? rows[r] : -1;
+        const int parts = row >= 0 ? sym_parts_of_row(tab.ub[row], part_products) : 0;
+        __syncthreads();
+        if (tid < 3) s_n[tid] = 0;
+        __syncthreads();
+        // units reserved per block; whole rows: one addition a warp
+        const unsigned whole = __ballot_sync(0xffffffffu, parts == 1);
+        int at = 0;
+        if (lane == 0 && whole) at = atomicAdd(&s_n[1], __popc(whole));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(whole & ((1u << lane) - 1u));
+        if (parts > 1) {
+            at = atomicAdd(&s_n[0], parts);
+            const int x = atomicAdd(&s_n[2], 1);
+            s_slot[x] = tab.bm_off[row];
+            s_quads[x] = ((tab.jmax[row] - tab.jmin[row]) / 32 + 4) >> 2;
+        }
+        __syncthreads();
+        if (tid < 2 && s_n[tid]) s_base[tid] = atomicAdd(&ctl->sym_units[tid], s_n[tid]);
+        for (int x = tid >> 5; x < s_n[2]; x += CP_THREADS / 32) {
+            uint4* const slot = reinterpret_cast<uint4*>(tab.bm_arena + s_slot[x]);
+            for (int q = lane; q < s_quads[x]; q += 32) slot[q] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        __syncthreads();
+        // (the table holds a unit per row and 2^19 more; the shares of split rows are some 4096 and a share per such row)
+        if (parts == 1) {
+            tab.unit_row[unit_cap - 1 - (s_base[1] + at)] = row;
+        } else if (parts > 1) {
+            const int u0 = s_base[0] + at;
+            tab.row_unit0[row] = u0;
+            for (int t = 0; t < parts; ++t) tab.unit_row[u0 + t] = row;
+        }
+    }
+    if (cap == 0) return;
+    for (i64 k = (i64)blockIdx.x * CP_THREADS + tid; k < B.nrows; k += (i64)gridDim.x * CP_THREADS) {
         const i64 len = B.pos[k + 1] - B.pos[k];
         if (len >= BW_BLOCK_ROW) {
             const int at = atomicAdd(&ctl->n_longest, 1);
@@ -581,13 +626,17 @@ __global__ void __launch_bounds__(BWB_THREADS, 2) bw_build_kernel(Csr B, const i
     }
 }
 
-cudaError_t launch_bw_build(const LaunchCtx& c, const Csr& B) {
-    if (!c.bw || B.nrows == 0) return cudaSuccess;
-    i64 want = ((i64)B.nrows + 255) / 256;
-    i64 cap = (i64)c.sm_count * 8;
-    bw_find_long_kernel<<<(int)(want < cap ? want : cap), 256, 0, c.stream>>>(B, c.bw_long, c.bw_long_cap, c.ctl);
+cudaError_t launch_cta_prepare(const LaunchCtx& c, i64 products, const Csr& B) {
+    const i64 rows = c.class_rows[CLS_DENSE_HUB] + c.class_rows[CLS_DENSE_CTA];
+    const i64 want = std::max(((i64)B.nrows + CP_THREADS - 1) / CP_THREADS, std::min(rows, (i64)c.sm_count)), cap = (i64)c.sm_count * 8;
+    i64 off = 0;
+    for (int k = 0; k < CLS_DENSE_HUB; ++k) off += c.class_rows[k];
+    cta_prepare_kernel<<<(int)(want < cap ? want : cap), CP_THREADS, 0, c.stream>>>(B, c.bw_long, c.bw ? c.bw_long_cap : 0, c.tab.perm + off, (int)rows,
+                                                                                  sym_part_products(products), c.prm.unit_cap, c.tab, c.ctl);
+    ++c.launches;
+    if (!c.bw) return cudaGetLastError();
     bw_build_kernel<<<c.sm_count * 2, BWB_THREADS, 0, c.stream>>>(B, c.bw_long, c.bw_long_cap, c.bw, c.ctl);
-    c.launches += 2;
+    ++c.launches;
     return cudaGetLastError();
 }
 

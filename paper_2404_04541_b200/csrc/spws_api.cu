@@ -726,8 +726,9 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
         }
         fork.group(2);
         if (dense_cta) {
-            CUDA_TRY(launch_bw_build(c, S.B));
-            CUDA_TRY(launch_dense_sym_cta(c, S.A, S.B));
+            const i64 cta_products = hc.class_products[CLS_DENSE_HUB] + hc.class_products[CLS_DENSE_CTA];
+            CUDA_TRY(launch_cta_prepare(c, cta_products, S.B));
+            CUDA_TRY(launch_dense_sym_cta(c, cta_products, S.A, S.B));
             mark(plan, SPWS_T_SYM_DENSE_CTA);
         }
         if (hcount[CLS_ISM_GLOBAL] > 0) {
