@@ -129,7 +129,7 @@ typedef struct {
     int32_t ism_cta_cap;      /* accumulation-array capacity of the shared-memory ISM, power of
                                  two in [64, 4096]; default 4096                                  */
     int32_t dense_unit_outputs;/* outputs of a row the CTA dense workspace accumulates in shared
-                                 memory (outputs beyond them accumulate in the row's own value
+                                 memory at most (outputs beyond them accumulate in the row's own value
                                  segment in global memory), power of two in [64, 8192];
                                  default 4096                                                      */
     int32_t dense_max_span;   /* widest column span (jmax - jmin + 1) a dense workspace may cover,
@@ -144,7 +144,8 @@ typedef struct {
                                  full it is sorted, reduced and united with the all array.
                                  0 (default): all products in one round                           */
     int32_t dense_unit_products;/* products from which a row of the CTA dense workspace is split over
-                                 several CTAs, positive; default 2^16                             */
+                                 several CTAs, positive; default (0) 2^16, in jobs of fewer than
+                                 2^27 products a 2048th of them, 2^13 at least                     */
     int32_t reserved[3];
 } spws_options_t;
 

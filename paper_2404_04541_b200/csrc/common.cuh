@@ -110,7 +110,7 @@ struct ClassParams {
     int max_span_words;     // dense allowed up to this many bitmap words
     float span_words_per_product;
     int unit_cap;           // entries available in the unit table
-    int unit_products;      // products a dense CTA unit takes at least
+    int unit_products;      // products a dense CTA unit takes at least; 0: by the job's size
     u64 bm_arena_words;     // capacity of the bitmap arena
     int warp_outputs;       // most outputs of a row that stays with a warp
 };
@@ -160,14 +160,22 @@ struct RowTables {
     int* unit_row;      // row of a CTA unit: symbolic (shares of split rows from the front, whole rows from the back), then numeric
 };
 
-// Products one dense CTA unit should take: `least`, by default 2^16 (measured on the power-law workload: units
-// of 2^17 products cost the accumulation kernel 10 % more, of 2^18 products 35 % more), or more
-// when the whole job is so large that the unit table (rows + 2^19 entries) would not hold that
-// many units.  `total_products` is the sum over the rows that the binning saw: the table and the kernels that
+// Products one dense CTA unit should take: `least`, or more when the whole job is so large that the unit table (rows + 2^19
+// entries) would not hold that many units.  By default (least = 0) 2^16 (power law on 2^18 vertices: units of 2^17 products
+// cost the accumulation kernel 10 % more, of 2^18 products 35 %, of 2^15 8 %), less in small jobs, so that no block is left alone with the
+// last units: a 2048th of the products, 2^13 at least (accumulation in units of 2^16 / 2^15 / 2^14 / 2^13, us: power law on 1500
+// vertices 26 / 25 / 21 / 18, 4001 52 / 51 / 38 / 34, 8001 (f64) 142 / 124 / 100 / 93, 16381 191 / 182 / 188 / 208, 60000 1580 / 1562 / 1582 / 1725).
+// `total_products` is the sum over the rows that the binning saw: the table and the kernels that
 // walk it must divide by the same number.
 __host__ __device__ inline i64 dense_unit_products(i64 total_products, int least) {
     const i64 need = (total_products + (1ll << 19) - 1) >> 19;
-    return need > least ? need : least;
+    i64 unit = least;
+    if (least == 0) {
+        unit = total_products >> 11;
+        if (unit < (1ll << 13)) unit = 1ll << 13;
+        if (unit > (1ll << 16)) unit = 1ll << 16;
+    }
+    return need > unit ? need : unit;
 }
 // The order in which CTA units are taken.  With few of them the heaviest rows come first, by powers of two of the
 // row's products (2^17 and more, 2^16, .., 2^13, fewer, rows that outgrew a warp), so that the last units

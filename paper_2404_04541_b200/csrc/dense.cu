@@ -23,6 +23,7 @@
 //              (atomics combine the CTA's warps), the rest in the row's value segment.  The
 //              coordinates of these rows are written by a kernel of their own, which also clears
 //              the value segments that several units add into.
+#include <algorithm>
 #include "common.cuh"
 
 namespace spws {
@@ -31,8 +32,8 @@ constexpr int DW_THREADS = 256;            // warp-per-row kernels: 8 warps per 
 constexpr int DW_WARPS = DW_THREADS / 32;
 constexpr int DC_THREADS = 256;            // symbolic CTA kernel
 constexpr int DC_WARPS = DC_THREADS / 32;
-constexpr int DN_THREADS = 512;            // numeric CTA kernel
-constexpr int DN_WARPS = DN_THREADS / 32;
+constexpr int DN_THREADS = 512;            // numeric CTA kernel: at most, and where four blocks of half of them fit an SM
+constexpr int DN_THREADS_4 = 256;
 
 // A warp-route row whose bitmap is mostly empty words saves only the non-empty ones; bm_off then
 // carries a flag and the number of saved words above the slot offset.
@@ -647,8 +648,9 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
 // cost more than the other warps' work hides) and with two steps to find a tile's entry 13590 / 287 us; with three barriers and the next unit
 // fetched meanwhile 12770 / 252 us.  Every output in shared memory, by segments of a row's ranks: 28000 / 339 us.
 // ---------------------------------------------------------------------------------------
-constexpr int DN_ENTRIES = 768;      // A entries whose descriptors are staged per round
+template <int THREADS> __host__ __device__ constexpr int dn_entries() { return THREADS * 3 / 2; }      // A entries whose descriptors are staged per round
 constexpr int DN_TILE = 256;         // products a warp takes per fetch
+constexpr int DN_CAP_LEAST = 1024;   // outputs in shared memory at least, for the sake of more blocks
 
 // What a block needs to know of a unit, fetched by one thread while the block is busy with the unit before.
 struct CtaUnit {
@@ -659,28 +661,29 @@ struct CtaUnit {
 // CEIL = true is the same traversal with the workspace stripped (the iteration-only lower bound of
 // Sec. 7.2): units, descriptor rounds, product tiles and gathers as below, but no bitmap, no rank
 // and no accumulation; every gathered column index and product is folded into two checksums.
-template <typename T, bool CEIL>
-__global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __restrict__ ctl, int smem_words, int CAP, i64 unit_products,
+template <typename T, bool CEIL, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) dense_num_cta_kernel(DevCtl* __restrict__ ctl, int smem_words, int CAP, i64 unit_products,
                                                                    Csr A, Csr B, RowTables tab, const i64* __restrict__ rowptr,
                                                                    int* __restrict__ Ccrd, T* __restrict__ Cval,
                                                                    u64* __restrict__ chk_idx, double* __restrict__ chk_val) {
+    constexpr int WARPS = THREADS / 32, ENTRIES = dn_entries<THREADS>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* acc = reinterpret_cast<T*>(smem_raw);                                        // CAP
     // per bitmap word: .x = the word, .y = outputs of the row before it, less one (one load gives a rank)
     uint2* bmr = reinterpret_cast<uint2*>(acc + CAP);                                // smem_words
-    // staged descriptors of up to DN_ENTRIES A entries: B-row start, A value, running product count
+    // staged descriptors of up to ENTRIES A entries: B-row start, A value, running product count
     i64* d_qs = reinterpret_cast<i64*>(smem_raw + ((sizeof(T) * (size_t)CAP + 8 * (size_t)smem_words + 15) & ~(size_t)15));
-    T* d_a = reinterpret_cast<T*>(d_qs + DN_ENTRIES);
-    int* d_pre = reinterpret_cast<int*>(d_a + DN_ENTRIES);                           // DN_ENTRIES + 1
+    T* d_a = reinterpret_cast<T*>(d_qs + ENTRIES);
+    int* d_pre = reinterpret_cast<int*>(d_a + ENTRIES);                           // ENTRIES + 1
     __shared__ CtaUnit s_unit[2];
-    __shared__ int s_tile, ws[DN_WARPS];
+    __shared__ int s_tile, ws[WARPS];
     if (ctl->status != 0) return;
     const int n_units = ctl->n_units;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const T* __restrict__ Aval = (const T*)A.val;
     const T* __restrict__ Bval = (const T*)B.val;
     if (!CEIL)
-        for (int x = tid; x < CAP; x += DN_THREADS) acc[x] = 0;
+        for (int x = tid; x < CAP; x += THREADS) acc[x] = 0;
     u64 my_idx = 0;
     double my_val = 0.0;
 
@@ -713,7 +716,7 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
         if (!U.valid) break;
         if (!CEIL) {
             if (U.nun == 1)                             // outputs beyond the shared-memory part start at zero
-                for (int x = CAP + tid; x < U.cnt; x += DN_THREADS) Cval[U.out0 + x] = 0;
+                for (int x = CAP + tid; x < U.cnt; x += THREADS) Cval[U.out0 + x] = 0;
             // the row's bitmap with the rank of every word's first bit (the symbolic pass saved the
             // rank at every chunk start).  A warp takes two groups of 128 words at a time, all loads first: one scan
             // per group.  Power law on 2^18 / 16381 vertices: a scan per chunk of 32 words 12850 / 249 us; four groups at a
@@ -722,12 +725,12 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
             const unsigned* src = tab.bm_arena + U.bm;
             const int nw = U.nw, nch = chunks_of(nw), ng = (nch + 3) >> 2;
             const uint4* src4 = reinterpret_cast<const uint4*>(src);         // slots are 16-byte aligned
-            for (int g0 = warp; g0 < ng; g0 += DN_WARPS * 2) {
+            for (int g0 = warp; g0 < ng; g0 += WARPS * 2) {
                 uint4 word[2];
                 unsigned rank_g[2];
 #pragma unroll
                 for (int x = 0; x < 2; ++x) {
-                    const int g = g0 + x * DN_WARPS, w0 = (g << 7) + (lane << 2);
+                    const int g = g0 + x * WARPS, w0 = (g << 7) + (lane << 2);
                     word[x] = make_uint4(0u, 0u, 0u, 0u);
                     if (w0 < nw) {
                         word[x] = src4[(g << 5) + lane];
@@ -739,7 +742,7 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
                 }
 #pragma unroll
                 for (int x = 0; x < 2; ++x) {
-                    const int g = g0 + x * DN_WARPS, w0 = (g << 7) + (lane << 2);
+                    const int g = g0 + x * WARPS, w0 = (g << 7) + (lane << 2);
                     const int p0 = __popc(word[x].x), p1 = p0 + __popc(word[x].y), p2 = p1 + __popc(word[x].z), p3 = p2 + __popc(word[x].w);
                     const unsigned r = rank_g[x] + (unsigned)(warp_incl_scan(p3) - p3) - 1u;
                     const uint4 lo = make_uint4(word[x].x, r, word[x].y, r + (unsigned)p0);
@@ -771,13 +774,13 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
         };
 
         bool next_known = false;
-        // Rounds of up to DN_ENTRIES A entries.  Step 1: every thread fetches the descriptors
+        // Rounds of up to ENTRIES A entries.  Step 1: every thread fetches the descriptors
         // of two entries; a block scan turns the B-row lengths into a running product count.
         // Step 2: warps pull tiles of DN_TILE consecutive products of that stream, so the
         // work is shared evenly however long the individual B rows are.
         const i64 e_hi = U.e_hi;
-        for (i64 e0 = U.e_lo; e0 < e_hi; e0 += DN_ENTRIES) {
-            const int nE = (int)min((i64)DN_ENTRIES, e_hi - e0);
+        for (i64 e0 = U.e_lo; e0 < e_hi; e0 += ENTRIES) {
+            const int nE = (int)min((i64)ENTRIES, e_hi - e0);
             int len2[2] = {0, 0};
 #pragma unroll
             for (int x = 0; x < 2; ++x) {
@@ -797,7 +800,7 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
             if (lane == 31) ws[warp] = incl;
             if (tid == 0) s_tile = 0;
             __syncthreads();
-            const int wt = lane < DN_WARPS ? ws[lane] : 0;
+            const int wt = lane < WARPS ? ws[lane] : 0;
             const int wi = warp_incl_scan(wt);
             const int total = __shfl_sync(0xffffffffu, wi, 31);
             const int excl = __shfl_sync(0xffffffffu, wi - wt, warp) + incl - len2[0] - len2[1];
@@ -805,7 +808,7 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
             if (2 * tid + 1 < nE) d_pre[2 * tid + 1] = excl + len2[0];
             if (tid == 0) d_pre[nE] = total;
             __syncthreads();
-            if (!next_known && tid == DN_THREADS - 1) fetch_unit(s_unit[cur ^ 1]);
+            if (!next_known && tid == THREADS - 1) fetch_unit(s_unit[cur ^ 1]);
             next_known = true;
             __syncwarp();
 
@@ -817,7 +820,7 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
                 if (t0 >= total) return false;
                 t1 = min(total, t0 + DN_TILE);
                 // the last entry whose running count is <= t0: among 32 spread entries, then among those in between
-                constexpr int STRIDE = DN_ENTRIES / 32;
+                constexpr int STRIDE = ENTRIES / 32;
                 static_assert(STRIDE <= 32, "two steps");
                 const int i1 = lane * STRIDE;
                 const int lo = (__popc(__ballot_sync(0xffffffffu, i1 < nE && d_pre[i1] <= t0)) - 1) * STRIDE;
@@ -882,9 +885,9 @@ __global__ void __launch_bounds__(DN_THREADS, 2) dense_num_cta_kernel(DevCtl* __
         // dense_emit_crd_kernel)
         const int n_smem = CEIL ? 0 : min(cnt, CAP);
         if (U.nun == 1) {
-            for (int x = tid; x < n_smem; x += DN_THREADS) { gacc[x] = acc[x]; acc[x] = 0; }
+            for (int x = tid; x < n_smem; x += THREADS) { gacc[x] = acc[x]; acc[x] = 0; }
         } else {
-            for (int x = tid; x < n_smem; x += DN_THREADS) {
+            for (int x = tid; x < n_smem; x += THREADS) {
                 const T v = acc[x];
                 acc[x] = 0;
                 if (v != (T)0) atomicAdd(gacc + x, v);
@@ -1102,24 +1105,43 @@ cudaError_t launch_dense_num_warp(const LaunchCtx& c, const int* n, const int* m
 template <typename T, bool CEIL>
 static cudaError_t num_cta_t(const LaunchCtx& c, int phase, int n_units_host, int words, i64 total_products, const Csr& A,
                              const Csr& B, const i64* rowptr, int* Ccrd, void* Cval, u64* chk_idx, double* chk_val) {
-    const int CAP = c.prm.unit_outputs;
     const i64 unit_products = dense_unit_products(total_products, c.prm.unit_products);
-    const size_t smem = ((sizeof(T) * (size_t)CAP + (size_t)words * 8 + 15) & ~(size_t)15) +
-                        (size_t)DN_ENTRIES * (8 + sizeof(T)) + (size_t)(DN_ENTRIES + 1) * 4 + 16;
     cudaError_t e;
-    int per_sm = 0;
-    auto k = dense_num_cta_kernel<T, CEIL>;
-    if ((e = resident_blocks((const void*)k, DN_THREADS, smem, &per_sm)) != cudaSuccess) return e;
     if (phase == 0) {
         // units are dealt out dynamically, so the grid is what is resident at once
         int emit_per_sm = 0;
         if ((e = resident_blocks((const void*)dense_emit_crd_kernel<T>, DE_THREADS, 0, &emit_per_sm)) != cudaSuccess) return e;
         const i64 work = n_units_host >= 0 ? ((i64)n_units_host + DE_WARPS - 1) / DE_WARPS : -1;
         dense_emit_crd_kernel<T><<<persistent_grid(c, emit_per_sm, work), DE_THREADS, 0, c.stream>>>(c.ctl, unit_products, c.tab, rowptr, Ccrd, (T*)Cval);
-    } else {
-        k<<<persistent_grid(c, per_sm, n_units_host), DN_THREADS, smem, c.stream>>>(c.ctl, words, CAP, unit_products, A, B, c.tab,
-                                                                                 rowptr, Ccrd, (T*)Cval, chk_idx, chk_val);
+        ++c.launches;
+        return cudaGetLastError();
     }
+    auto smem_of = [&](int cap, int entries) {
+        return ((sizeof(T) * (size_t)cap + (size_t)words * 8 + 15) & ~(size_t)15) + (size_t)entries * (8 + sizeof(T)) + (size_t)(entries + 1) * 4 + 16;
+    };
+    // A block waits at its barriers for its slowest warp and, between units, for chains of loads: four blocks of 256 threads do
+    // so less than two of 512, where four find room (with fewer outputs in shared memory if need be: a reduction in global memory
+    // costs about the same) and the units are enough for all of them.  Accumulation, 512 / 256 threads: power law on 16381
+    // (f32) / 60000 (f64) / 100003 (f32) vertices 229 / 191, 1780 / 1580, 1795 / 1540 us; 10^4 rows of 10^4 products, f64, 419 / 356.
+    // With few units 512: power law on 1500 / 4001 vertices, f32, units of 2^13, 18 / 23 and 33 / 38.
+    int CAP = c.prm.unit_outputs, per_sm = 0;
+    auto quarter = dense_num_cta_kernel<T, CEIL, DN_THREADS_4>;
+    if (n_units_host < 0 || n_units_host > 8 * c.sm_count)
+        for (int cap = CAP; cap >= std::min(CAP, DN_CAP_LEAST); cap >>= 1) {
+            const size_t smem = smem_of(cap, dn_entries<DN_THREADS_4>());
+            if (4 * (smem + 2048) > 228 * 1024) continue;
+            if ((e = resident_blocks((const void*)quarter, DN_THREADS_4, smem, &per_sm)) != cudaSuccess) return e;
+            if (per_sm < 4) continue;
+            quarter<<<persistent_grid(c, per_sm, n_units_host), DN_THREADS_4, smem, c.stream>>>(c.ctl, words, cap, unit_products, A, B, c.tab, rowptr, Ccrd,
+                                                                                           (T*)Cval, chk_idx, chk_val);
+            ++c.launches;
+            return cudaGetLastError();
+        }
+    auto half = dense_num_cta_kernel<T, CEIL, DN_THREADS>;
+    const size_t smem = smem_of(CAP, dn_entries<DN_THREADS>());
+    if ((e = resident_blocks((const void*)half, DN_THREADS, smem, &per_sm)) != cudaSuccess) return e;
+    half<<<persistent_grid(c, per_sm, n_units_host), DN_THREADS, smem, c.stream>>>(c.ctl, words, CAP, unit_products, A, B, c.tab, rowptr, Ccrd, (T*)Cval, chk_idx,
+                                                                               chk_val);
     ++c.launches;
     return cudaGetLastError();
 }

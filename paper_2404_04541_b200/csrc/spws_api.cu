@@ -1589,7 +1589,6 @@ static spws_status_t plan_create_n(spws_handle_t handle, const char* expr, const
     if (o.ism_warp_cap == 0) o.ism_warp_cap = 32;
     if (o.ism_cta_cap == 0) o.ism_cta_cap = 4096;
     if (o.dense_unit_outputs == 0) o.dense_unit_outputs = 4096;
-    if (o.dense_unit_products == 0) o.dense_unit_products = 1 << 16;
     if (o.dense_max_span == 0) o.dense_max_span = 1 << 19;
     if (o.fallback_cap == 0) o.fallback_cap = 2048;
     if (o.dense_span_words_per_product == 0.0f) o.dense_span_words_per_product = 8.0f;
@@ -1597,7 +1596,7 @@ static spws_status_t plan_create_n(spws_handle_t handle, const char* expr, const
     if (o.ism_warp_cap < 1 || o.ism_warp_cap > 32) return SPWS_INVALID_ARGUMENT;
     if (!is_pow2(o.ism_cta_cap) || o.ism_cta_cap < 64 || o.ism_cta_cap > 4096) return SPWS_INVALID_ARGUMENT;
     if (!is_pow2(o.dense_unit_outputs) || o.dense_unit_outputs < 64 || o.dense_unit_outputs > 8192) return SPWS_INVALID_ARGUMENT;
-    if (o.dense_unit_products < 1) return SPWS_INVALID_ARGUMENT;
+    if (o.dense_unit_products < 0) return SPWS_INVALID_ARGUMENT;
     if (o.dense_max_span < 32 || o.dense_max_span > (1 << 19)) return SPWS_INVALID_ARGUMENT;
     if (!is_pow2(o.fallback_cap) || o.fallback_cap < 2 || o.fallback_cap > 2048) return SPWS_INVALID_ARGUMENT;
     if (!(o.dense_span_words_per_product > 0.0f)) return SPWS_INVALID_ARGUMENT;
