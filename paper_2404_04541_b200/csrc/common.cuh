@@ -81,6 +81,7 @@ struct DevCtl {
     u64 bm_words_used;      // words handed out so far
     u64 order_words;        // words the sorted CLS_ISM_SMEM rows of up to ISM_WARP_MAX products have (counted by the bounds kernel)
     u64 order_used;         // bytes handed out of their arena
+    int n_ranked;           // rows that left their products' places instead of their sorted words
     int status;
     int n_units;            // numeric dense CTA units (row, share of its entries)
     int units_of[7];        // units per bucket of rows (counted by the binning, without the rows that outgrow a warp) ...
@@ -401,6 +402,8 @@ struct LaunchCtx {
     size_t rest_bytes;
     char* order;             // arena of sorted words (null: every pass sorts)
     size_t order_bytes;
+    int may_rank;            // counting: rows may leave their products' places; n_ranked: numeric, such rows of the pass
+    int n_ranked;
     int global_cap;          // accumulation-array capacity of CLS_ISM_GLOBAL
     HostBlock* host;         // the plan's pinned block: receives the control block ...
     int seq;                 // ... as publication `seq` (class sizes) and `seq` + 1 (row pointer)

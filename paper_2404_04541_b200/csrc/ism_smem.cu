@@ -166,6 +166,11 @@ __global__ void __launch_bounds__(THREADS) ism_smem_kernel(const int* __restrict
 // row.  With sizes of three times a power of two, long merges as loops and lane groups found by shifts: count 578 -> 384 us
 // on the stencil (372 since; numeric 370, 309 since), 210 -> 172 us on the rows of 470; 143-product rows (3e4): 44 -> 36
 // and 55 -> 49 us.
+//   Where outputs are at most half of the products and B rows fill a warp, the counting pass leaves the places of the products
+// among the outputs and ism_rank_kernel adds: stencil 41 x 37 x 53, f32, count 374 -> 400 us, numeric 309 -> 147 (of it 11 for
+// the rows at its edges); 40^3, f64, 300 -> 321 and 296 -> 148.  Not with words of 64 bits, whose counting kernel would slow
+// down (60000 rows of 600 products, f64: 881 -> 895 us).  A hash set of the columns before the sort instead: 348 us, and 786 for
+// a numeric pass that looks its products up in it.
 // ---------------------------------------------------------------------------------------
 constexpr int IW_WARPS = 4;
 
@@ -243,11 +248,16 @@ __device__ __forceinline__ void warp_sort(P (&w)[E]) {
 // one word of padding per 32 keeps both the strided and the per-lane consecutive accesses conflict-free
 __device__ __forceinline__ int padded(int i) { return i + (i >> 5); }
 
+// What the counting pass keeps of a row whose outputs are at most half of its products and whose B rows fill a warp, instead of the
+// sorted words: the distinct columns, then every product's place among them (16 bits, loop order).  The numeric pass adds one
+// B row after the other, whose products go to different outputs, and reads no columns.
+constexpr i64 ORDER_RANKS = 1ll << 62;                  // flag above the offset of such a row
+
 // Sorts the row's packed words and counts its distinct columns; numeric: leaves the sorted words in `packed`
 // and the places of the run heads in `heads`.  `order` (may be null): numeric: the words as sorted before;
-// else receives them.
+// else receives them, or (*ranks, when the row is of that kind and may_rank) the columns and places.
 template <typename PK, typename P, int E, bool NUMERIC>
-__device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int total, P* order) {
+__device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int total, P* order, bool may_rank, bool* ranks) {
     const int lane = threadIdx.x & 31;
     P w[E];
     const int lanes = order_lanes(total, E);
@@ -261,10 +271,6 @@ __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int to
             w[x] = i < total ? packed[padded(i)] : PK::sentinel();
         }
         warp_sort<P, E>(w);
-        if (!NUMERIC && order && lane < lanes) {
-#pragma unroll
-            for (int x = 0; x < E; ++x) order[x * lanes + lane] = w[x];
-        }
     }
     const P before = __shfl_up_sync(0xffffffffu, w[E - 1], 1);
     unsigned head = 0;
@@ -285,6 +291,27 @@ __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int to
             if ((head >> x) & 1u) heads[at++] = (unsigned short)(lane * E + x);
         }
         __syncwarp();
+    } else if (order) {
+        if (may_rank && 2 * n <= total) {
+            __syncwarp();
+            unsigned* const cols = reinterpret_cast<unsigned*>(packed);
+            unsigned short* const place = reinterpret_cast<unsigned short*>(cols + n);
+            int at = incl - mine - 1;
+#pragma unroll
+            for (int x = 0; x < E; ++x)
+                if (w[x] != PK::sentinel()) {
+                    if ((head >> x) & 1u) cols[++at] = PK::key(w[x]);
+                    place[PK::slot(w[x])] = (unsigned short)at;
+                }
+            __syncwarp();
+            // (whole quads: the room of a row, like that of its packed words, is a multiple of 16 bytes)
+            for (int i = lane; 4 * i < n + (total + 1) / 2; i += 32) reinterpret_cast<uint4*>(order)[i] = reinterpret_cast<const uint4*>(packed)[i];
+            __syncwarp();
+            *ranks = true;
+        } else if (lane < lanes) {
+#pragma unroll
+            for (int x = 0; x < E; ++x) order[x * lanes + lane] = w[x];
+        }
     }
     return n;
 }
@@ -472,7 +499,8 @@ constexpr int iw_blocks() {
     return sizeof(P) == 8 ? 3 : NUMERIC && sizeof(T) == 8 ? 5 : 7;
 }
 
-template <typename T, typename P, int CAP, bool NUMERIC>
+// RANKS: counting: rows may leave their products' places; numeric: some have, and are passed over.
+template <typename T, typename P, int CAP, bool NUMERIC, bool RANKS>
 __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>())) ism_warp_kernel(const int* __restrict__ perm, int first_cls, int cls, int small_cap, DevCtl* __restrict__ ctl, int counter_slot,
                                                                  Csr A, Csr B, const i64* __restrict__ ub, i64* __restrict__ order_off, char* order_arena,
                                                                  size_t order_bytes, int* __restrict__ cnt,
@@ -537,6 +565,11 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
             i64 at = -1;
             if (NUMERIC) {
                 at = order_off[row];
+                if (RANKS && at >= 0 && (at & ORDER_RANKS)) {      // ism_rank_kernel's row
+                    take(__shfl_sync(0xffffffffu, r_n, 0));
+                    fields();
+                    continue;
+                }
             } else if (lane == 0) {
                 const u64 bytes = (u64)order_words_of(products) * sizeof(P);
                 at = (i64)atomicAdd(&ctl->order_used, bytes);
@@ -601,22 +634,24 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
         const int e = words_per_lane<CAP>(total);
         if (total != products) order = nullptr;             // (a malformed B row)
         P* const keep = CAP > 256 ? order : nullptr;
-        if (!NUMERIC && kept && lane == 0) order_off[row] = order ? (i64)(reinterpret_cast<char*>(order) - order_arena) : -1;
+        bool ranks = false;
         if constexpr (CAP <= 256) {
             switch (e) {
-                case 4: distinct = sort_row<PK, P, 4, NUMERIC>(packed, heads, total, keep); break;
-                case 6: distinct = sort_row<PK, P, 6, NUMERIC>(packed, heads, total, keep); break;
-                default: distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total, keep); break;
+                case 4: distinct = sort_row<PK, P, 4, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
+                case 6: distinct = sort_row<PK, P, 6, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
+                default: distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
             }
         } else {
             switch (e) {
-                case 8: distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total, keep); break;
-                case 12: distinct = sort_row<PK, P, 12, NUMERIC>(packed, heads, total, keep); break;
-                case 16: distinct = sort_row<PK, P, 16, NUMERIC>(packed, heads, total, keep); break;
-                case 24: distinct = sort_row<PK, P, 24, NUMERIC>(packed, heads, total, keep); break;
-                default: distinct = sort_row<PK, P, 32, NUMERIC>(packed, heads, total, keep); break;
+                case 8: distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
+                case 12: distinct = sort_row<PK, P, 12, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
+                case 16: distinct = sort_row<PK, P, 16, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
+                case 24: distinct = sort_row<PK, P, 24, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
+                default: distinct = sort_row<PK, P, 32, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
             }
         }
+        if (!NUMERIC && kept && lane == 0) order_off[row] = order ? (i64)(reinterpret_cast<char*>(order) - order_arena) | (ranks ? ORDER_RANKS : 0) : -1;
+        if (!NUMERIC && RANKS && ranks && lane == 0) atomicAdd(&ctl->n_ranked, 1);
 
         if (AHEAD) fields();
 
@@ -636,6 +671,89 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
         }
         __syncwarp();
     }
+}
+
+// ---------------------------------------------------------------------------------------
+// Numeric pass of the rows whose products' places the counting pass has kept: a warp per row, its lanes across one B row after the
+// other, so that no two lanes add into one output and every output is summed in loop order.  Bound by the chains of loads that lead
+// to a row's B rows: a block for every four rows, four B rows in flight, and shared memory for the outputs alone, so that 40 .. 48
+// warps are on an SM (as a path of ism_warp_kernel, at 28 warps, two B rows in flight 246 us, four 211).
+// ---------------------------------------------------------------------------------------
+// start of the B row and its length, place of the entry's first product, A value
+template <typename T> struct __align__(16) RankEntry { u64 row; T a; int at; };
+
+template <typename T>
+__global__ void __launch_bounds__(IW_WARPS * 32, sizeof(T) == 8 ? 10 : 12) ism_rank_kernel(const int* __restrict__ rows, int n_rows, const DevCtl* __restrict__ ctl, Csr A, Csr B,
+                                                                                          const i64* __restrict__ ub, const i64* __restrict__ order_off,
+                                                                                          const char* __restrict__ order_arena, const i64* __restrict__ rowptr,
+                                                                                          int* __restrict__ Ccrd, T* __restrict__ Cval, int most) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (ctl->status != 0) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    RankEntry<T>* const entry = reinterpret_cast<RankEntry<T>*>(smem_raw) + warp * 32;
+    T* const vals = reinterpret_cast<T*>(smem_raw + sizeof(RankEntry<T>) * 32 * IW_WARPS) + warp * most;
+    const T* __restrict__ Aval = (const T*)A.val;
+    const T* __restrict__ Bval = (const T*)B.val;
+    const int r = blockIdx.x * IW_WARPS + warp;
+    if (r >= n_rows) return;
+    const int row = __ldg(rows + r);
+    const i64 off = __ldg(order_off + row);
+    if (off < 0 || !(off & ORDER_RANKS)) return;        // ism_warp_kernel's row
+    const int products = (int)__ldg(ub + row);
+    const i64 ps = __ldg(A.pos + row), pe = __ldg(A.pos + row + 1), out0 = __ldg(rowptr + row);
+    const int n = min((int)(__ldg(rowptr + row + 1) - out0), most);
+    const unsigned* __restrict__ cols = reinterpret_cast<const unsigned*>(order_arena + (off & ~ORDER_RANKS));
+    const unsigned short* __restrict__ place = reinterpret_cast<const unsigned short*>(cols + n);
+    for (int x = lane; x < n; x += 32) {
+        Ccrd[out0 + x] = (int)__ldg(cols + x);
+        vals[x] = (T)-0.0;                              // (the sum of nothing that leaves the sign of a first zero)
+    }
+    int total = 0;
+    for (i64 p0 = ps; p0 < pe; p0 += 32) {
+        RankEntry<T> mine;
+        mine.row = 0;
+        mine.a = 0;
+        if (p0 + lane < pe) {
+            const int k = __ldg(A.crd + p0 + lane);
+            mine.a = __ldg(Aval + p0 + lane);
+            if ((unsigned)k < (unsigned)B.nrows) {
+                const i64 qs = __ldg(B.pos + k);
+                mine.row = (u64)qs << 16 | (u64)min(__ldg(B.pos + k + 1) - qs, (i64)products);
+            }
+        }
+        const int len = (int)(mine.row & 0xffffu), incl = warp_incl_scan(len);
+        mine.at = min(total + incl - len, products - len);          // (the lengths add up to the products)
+        __syncwarp();
+        entry[lane] = mine;
+        __syncwarp();
+        const bool longer = __any_sync(0xffffffffu, len > 32);
+        const int nE = (int)min((i64)32, pe - p0);
+        for (int e = 0; e < nE; e += 4) {               // (length 0 past the last entry)
+            T v[4];
+            int x[4];
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                const RankEntry<T> d = entry[e + y];
+                x[y] = -1;
+                v[y] = 0;
+                if (lane < (int)(d.row & 0xffffu)) { x[y] = __ldg(place + d.at + lane); v[y] = mul_rn(d.a, __ldg(Bval + (d.row >> 16) + lane)); }
+            }
+#pragma unroll
+            for (int y = 0; y < 4; ++y) {
+                if (x[y] >= 0) vals[x[y]] = add_rn(vals[x[y]], v[y]);
+                if (longer) {
+                    const RankEntry<T> d = entry[e + y];
+                    for (int t = 32 + lane; t < (int)(d.row & 0xffffu); t += 32) {
+                        const int z = __ldg(place + d.at + t);
+                        vals[z] = add_rn(vals[z], mul_rn(d.a, __ldg(Bval + (d.row >> 16) + t)));
+                    }
+                }
+                __syncwarp();
+            }
+        }
+        total += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    for (int x = lane; x < n; x += 32) Cval[out0 + x] = vals[x];
 }
 
 template <typename T, typename P, int CAP, int THREADS>
@@ -668,7 +786,10 @@ static cudaError_t launch_warp_k(const LaunchCtx& c, const IsmLaunch& l, const C
     const size_t smem = (size_t)IW_WARPS * ((NUMERIC ? (sizeof(T) + sizeof(short)) * slots : 0) + sizeof(P) * (slots + slots / 32));
     cudaError_t e;
     int per_sm = 0;
-    auto k = ism_warp_kernel<T, P, CAP, NUMERIC>;
+    // (words of 64 bits: as before, for the sake of their registers)
+    constexpr bool MAY = CAP > 256 && sizeof(P) == 4;
+    const bool ranks = MAY && (NUMERIC ? c.order && c.n_ranked > 0 : c.may_rank);
+    auto k = ranks ? ism_warp_kernel<T, P, CAP, NUMERIC, MAY> : ism_warp_kernel<T, P, CAP, NUMERIC, false>;
     if ((e = resident_blocks((const void*)k, IW_WARPS * 32, smem, &per_sm)) != cudaSuccess) return e;
     i64 grid = (i64)c.sm_count * (per_sm > 0 ? per_sm : 1);
     const int n = l.n, cls = l.level == 4 ? CLS_ISM_SMEM : CLS_ISM_SMEM_S;
@@ -726,8 +847,22 @@ static cudaError_t launch_t(const LaunchCtx& c, bool numeric, const IsmLaunch& l
     i64 most = l.level == 3 ? 256 : c.prm.smem_cap;
     if (l.level == 4 && c.max_ub_smem > 0 && c.max_ub_smem < most) most = c.max_ub_smem;
     if (most <= 256) return launch_warp<T, 256>(c, numeric, l, A, B, rowptr, Ccrd, Cval);
-    cudaError_t e = launch_warp<T, ISM_WARP_MAX>(c, numeric, l, A, B, rowptr, Ccrd, Cval);
-    if (e != cudaSuccess || most <= ISM_WARP_MAX) return e;
+    cudaError_t e = cudaSuccess;
+    bool rest = true;
+    if (numeric && c.order && c.n_ranked > 0) {
+        const int outputs = (int)std::min(most, (i64)ISM_WARP_MAX) / 2;             // (at most half of the products)
+        const size_t smem = IW_WARPS * (sizeof(T) * outputs + 32 * sizeof(RankEntry<T>));
+        int per_sm = 0;
+        if ((e = resident_blocks((const void*)ism_rank_kernel<T>, IW_WARPS * 32, smem, &per_sm)) != cudaSuccess) return e;
+        ism_rank_kernel<T><<<(l.own + IW_WARPS - 1) / IW_WARPS, IW_WARPS * 32, smem, c.stream>>>(l.rows + (l.n - l.own), l.own, c.ctl, A, B, c.tab.ub, c.tab.bm_off, c.order, rowptr,
+                                                                                                Ccrd, (T*)Cval, outputs);
+        ++c.launches;
+        rest = c.n_ranked < l.own;
+        // the rows of smaller classes that go along with these
+        if (!rest && l.n > l.own) e = launch_warp<T, 256>(c, numeric, IsmLaunch{3, l.first_cls, l.rows, l.n - l.own, l.n - l.own}, A, B, rowptr, Ccrd, Cval);
+    }
+    if (e == cudaSuccess && rest) e = launch_warp<T, ISM_WARP_MAX>(c, numeric, l, A, B, rowptr, Ccrd, Cval);
+    if (e != cudaSuccess || most <= ISM_WARP_MAX || !rest) return e;
     // rows of 1025 .. 4096 products: a CTA each (a counter of their own: the two kernels share the class);
     // under `auto` they are counted through a hash set of their columns, which needs no order
     const int n = l.own;

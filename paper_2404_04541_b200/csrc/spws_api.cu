@@ -169,6 +169,8 @@ struct spws_plan_s {
     bool symbolic_ok = false;
     bool pending = false;       // a symbolic pass is enqueued and not yet waited for (spws_symbolic_begin)
     bool numeric_behind = false;                // .. and the numeric pass behind it
+    int64_t behind_most = -1;   // most entries of a bound for which the caller of a symbolic pass enqueues the numeric one behind it
+    int n_ranked = 0;           // rows that left their products' places
     int64_t upper = 0;          // .. a bound on its result's entries when the numeric pass may be enqueued behind it, else 0
     spws_stats_t stats{};
     // what the last symbolic pass saw (numeric must be called with the same shapes and scratch)
@@ -708,6 +710,8 @@ spws_status_t rows_symbolic(spws_plan_s* plan, const Shapes& S, const Layout& L,
     const bool any_dense = hcount[CLS_DENSE_WARP] + hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0;
     plan->max_ub_smem = hc.max_ub_smem;
     c.max_ub_smem = plan->max_ub_smem;
+    // (a numeric pass enqueued before the outcome is known could not tell which of two kernels has rows)
+    c.may_rank = any_dense || products > plan->behind_most;
     // a3: exact count per row through the workspace of its class
     if (S.m > 0) {
         const bool dense_cta = hcount[CLS_DENSE_HUB] + hcount[CLS_DENSE_CTA] > 0;
@@ -790,6 +794,7 @@ spws_status_t rows_collect(spws_plan_s* plan) {
     plan->stats.dense_warp_nnz = hc.dense_warp_nnz;
     plan->stats.bitmap_bytes = (int64_t)hc.bm_words * 4;
     plan->max_span_words = hc.max_span_words;
+    plan->n_ranked = hc.n_ranked;
     for (int list = 0; list < N_WARP_LISTS; ++list) {
         plan->n_warp[list] = hc.n_warp_rows[list];
         plan->max_warp_cnt[list] = hc.max_warp_cnt[list];
@@ -807,6 +812,7 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, cha
         CUDA_TRY(cudaMemsetAsync(c.ctl->work_counter, 0, sizeof(c.ctl->work_counter), c.stream));
     plan->counters_clear = false;
     c.max_ub_smem = plan->max_ub_smem;
+    c.n_ranked = plan->numeric_behind ? 0 : plan->n_ranked;
     const spws_stats_t& s = plan->stats;
     const int64_t* bins = plan->bin_rows;
     c.class_rows = LL(bins);
@@ -1812,7 +1818,9 @@ spws_status_t spws_symbolic_begin(spws_plan_t plan, const spws_tensor_t* A, cons
                                   size_t scratch_bytes, int64_t most, int64_t* sizes_out, size_t* needed, int64_t* upper) {
     if (!plan || !needed || !upper || plan->kind > 1) return SPWS_INVALID_ARGUMENT;
     *upper = 0;
+    plan->behind_most = most;
     const spws_status_t st = symbolic_any(plan, A, B, nullptr, C, scratch, scratch_bytes, nullptr, needed, true);
+    plan->behind_most = -1;
     if (st != SPWS_OK) return st;
     if (plan->upper == 0 || plan->upper > most) return symbolic_collect(plan, C, sizes_out);
     *upper = plan->upper;
