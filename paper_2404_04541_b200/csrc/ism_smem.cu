@@ -399,8 +399,9 @@ __global__ void __launch_bounds__(IG_THREADS, (group_blocks<T, P, NUMERIC>())) i
     unsigned char* const heads = smem + ROWS * (G * (sizeof(Entry) + (NUMERIC ? 9 * sizeof(T) : 0)) + sizeof(P) * group_words<G>()) + group * (NUMERIC ? CAP : 0);
     const T* __restrict__ Aval = (const T*)A.val;
     const T* __restrict__ Bval = (const T*)B.val;
+    const int r = chained_start(blockIdx.x * ROWS + group);
+    not_before(ctl);
     if (ctl->status != 0) return;
-    const int r = blockIdx.x * ROWS + group;
     if ((r & ~(32 / G - 1)) >= n) return;           // (whole warps)
     int row = 0;
     i64 ps = 0, pe = 0;
@@ -514,6 +515,7 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
     T* const vals = reinterpret_cast<T*>(smem_raw) + warp * (NUMERIC ? slots : 0);
     P* const packed = reinterpret_cast<P*>(smem_raw + (NUMERIC ? (int)sizeof(T) * slots * IW_WARPS : 0)) + warp * padded_slots;
     unsigned short* const heads = reinterpret_cast<unsigned short*>(smem_raw + ((NUMERIC ? (int)sizeof(T) * slots : 0) + (int)sizeof(P) * padded_slots) * IW_WARPS) + warp * slots;
+    chained_start();
     if (ctl->status != 0) return;
     // the rows of the classes first_cls .. cls, one range of perm (with a table of ranges, or the range as arguments, the kernels
     // spill: counting / numeric, rows of 200 products 85 / 123 us, now 83 / 116; stencil 41 x 37 x 53 by ISM, f32, 376 / 317 and 372 / 309)
@@ -795,10 +797,8 @@ static cudaError_t launch_warp_k(const LaunchCtx& c, const IsmLaunch& l, const C
     const int n = l.n, cls = l.level == 4 ? CLS_ISM_SMEM : CLS_ISM_SMEM_S;
     const i64 want = ((i64)n + IW_WARPS - 1) / IW_WARPS;
     if (want < grid) grid = want > 0 ? want : 1;
-    k<<<(int)grid, IW_WARPS * 32, smem, c.stream>>>(c.tab.perm, l.first_cls, cls, c.prm.smem_small_cap, c.ctl, cls + (NUMERIC ? NUM_SLOT : 0), A, B, c.tab.ub, c.tab.bm_off, c.order,
-                                                    c.order_bytes, c.tab.cnt, rowptr, Ccrd, (T*)Cval, slots);
-    ++c.launches;
-    return cudaGetLastError();
+    return launch_chained(c, k, grid, IW_WARPS * 32, smem, c.tab.perm, l.first_cls, cls, c.prm.smem_small_cap, c.ctl, cls + (NUMERIC ? NUM_SLOT : 0), A, B, c.tab.ub,
+                          c.tab.bm_off, c.order, c.order_bytes, c.tab.cnt, rowptr, Ccrd, (T*)Cval, slots);
 }
 
 // Packed words are 32 bits wide when (column, slot) fits below the all-ones sentinel.
@@ -814,9 +814,7 @@ template <typename T, typename P, int G, bool NUMERIC>
 static cudaError_t launch_group_k(const LaunchCtx& c, const IsmLaunch& l, const Csr& A, const Csr& B, const i64* rowptr, int* Ccrd, void* Cval) {
     constexpr int ROWS = IG_THREADS / G;
     const int n = l.n;
-    ism_group_kernel<T, P, G, NUMERIC><<<(int)(((i64)n + ROWS - 1) / ROWS), IG_THREADS, 0, c.stream>>>(l.rows, n, c.ctl, A, B, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
-    ++c.launches;
-    return cudaGetLastError();
+    return launch_chained(c, ism_group_kernel<T, P, G, NUMERIC>, ((i64)n + ROWS - 1) / ROWS, IG_THREADS, 0, l.rows, n, c.ctl, A, B, c.tab.cnt, rowptr, Ccrd, (T*)Cval);
 }
 
 template <typename T, int G>

@@ -38,6 +38,9 @@ __global__ void __launch_bounds__(OT) rw_keys_outer_kernel(Csr At, i64 n, Csr B,
     __shared__ int s_lo, s_hi;
     __shared__ DigitCounts s_digits;
     bool bad = false;
+    chained_start();
+    not_before(At);
+    not_before(B);
     s_digits.start(passes);
     for (i64 q = (i64)blockIdx.x * OT + threadIdx.x; q < nnzB; q += (i64)gridDim.x * OT) bad |= (unsigned)__ldg(B.crd + q) >= (unsigned)B.ncols;
     for (i64 t0 = (i64)blockIdx.x * RK_TILE; t0 < n; t0 += (i64)gridDim.x * RK_TILE) {
@@ -65,6 +68,12 @@ __global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u6
                                                          SortHead* head, i64* __restrict__ pos, i64 m) {
     __shared__ int s_f[2], s_s[2];
     __shared__ DigitCounts s_digits;
+    chained_start();
+    not_before(B.pos1);
+    not_before(B.pos2);
+    not_before(B.crd0);
+    not_before(B.crd1);
+    not_before(B.crd2);
     s_digits.start(passes);
     for (i64 i = (i64)blockIdx.x * OT + threadIdx.x; i <= m; i += (i64)gridDim.x * OT) pos[i] = B.nnz;
     for (i64 t0 = (i64)blockIdx.x * RK_TILE; t0 < B.nnz; t0 += (i64)gridDim.x * RK_TILE) {
@@ -100,6 +109,9 @@ __global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u6
 __global__ void __launch_bounds__(OT) rw_dense_rows_kernel(const u64* __restrict__ keys, const u64* __restrict__ pay, i64 n, i64 m,
                                                            i64* __restrict__ pos, int* __restrict__ crd, int* __restrict__ src) {
     const i64 stride = (i64)gridDim.x * OT, t0 = (i64)blockIdx.x * OT + threadIdx.x;
+    chained_start();
+    not_before(keys);
+    not_before(pay);
     for (i64 i = t0; i <= m; i += stride) {
         i64 lo = 0, hi = n;
         while (lo < hi) {
@@ -126,6 +138,7 @@ __global__ void __launch_bounds__(OT) rw_sparse_rows_kernel(const u64* __restric
     __shared__ int s_ws[33];
     __shared__ int s_tile;
     __shared__ i64 s_before;
+    chained_start();
     if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1);
     __syncthreads();
     const int tile = s_tile;
@@ -353,13 +366,11 @@ static cudaError_t rw_reorder(const LaunchCtx& c, i64 n, i64 m, int bits, bool s
     const u64* ks = first ? b.kA : b.kB;
     const u64* ps = first ? b.pA : b.pB;
     if (!sparse) {
-        rw_dense_rows_kernel<<<grid_for(c, n > m ? n : m + 1, OT), OT, 0, c.stream>>>(ks, ps, n, m, b.pos, b.crd, b.src);
-        ++c.launches;
+        return launch_chained(c, rw_dense_rows_kernel, grid_for(c, n > m ? n : m + 1, OT), OT, 0, ks, ps, n, m, b.pos, b.crd, b.src);
     } else if (n > 0) {
         const int tiles = (int)((n + RK_TILE - 1) / RK_TILE);
         u64* const words = reinterpret_cast<u64*>(b.sort_tmp + sort_scratch_bytes(n));
-        rw_sparse_rows_kernel<<<tiles, OT, 0, c.stream>>>(ks, ps, n, m, reinterpret_cast<int*>(words), words + 1, c.ctl, b.row_key, b.pos, b.crd, b.src);
-        ++c.launches;
+        return launch_chained(c, rw_sparse_rows_kernel, tiles, OT, 0, ks, ps, n, m, reinterpret_cast<int*>(words), words + 1, c.ctl, b.row_key, b.pos, b.crd, b.src);
     }
     return cudaGetLastError();
 }
@@ -367,19 +378,17 @@ static cudaError_t rw_reorder(const LaunchCtx& c, i64 n, i64 m, int bits, bool s
 cudaError_t launch_rw_outer(const LaunchCtx& c, const Csr& At, i64 n, const Csr& B, i64 nnzB, int bits, const RowwiseBufs& b) {
     const cudaError_t e = cudaMemsetAsync(b.sort_tmp, 0, rw_sort_bytes(n), c.stream);
     if (e != cudaSuccess) return e;
-    rw_keys_outer_kernel<<<grid_for(c, std::max(n, nnzB), RK_TILE), OT, 0, c.stream>>>(At, n, B, nnzB, b.kA, b.pA, passes_of(bits),
-                                                                                     reinterpret_cast<SortHead*>(b.sort_tmp), c.ctl);
-    ++c.launches;
-    return rw_reorder(c, n, At.ncols, bits, false, b);
+    const cudaError_t k = launch_chained(c, rw_keys_outer_kernel, grid_for(c, std::max(n, nnzB), RK_TILE), OT, 0, At, n, B, nnzB, b.kA, b.pA, passes_of(bits),
+                                         reinterpret_cast<SortHead*>(b.sort_tmp), c.ctl);
+    return k != cudaSuccess ? k : rw_reorder(c, n, At.ncols, bits, false, b);
 }
 
 cudaError_t launch_rw_csf(const LaunchCtx& c, int form, const Csf3Dev& B, u64 d, i64 m, int bits, const RowwiseBufs& b) {
     const cudaError_t e = cudaMemsetAsync(b.sort_tmp, 0, rw_sort_bytes(B.nnz), c.stream);
     if (e != cudaSuccess) return e;
-    rw_keys_csf_kernel<<<grid_for(c, std::max(B.nnz, (i64)1), RK_TILE), OT, 0, c.stream>>>(form, B, d, b.kA, b.pA, passes_of(bits),
-                                                                                         reinterpret_cast<SortHead*>(b.sort_tmp), b.pos, m);
-    ++c.launches;
-    return rw_reorder(c, B.nnz, m, bits, true, b);
+    const cudaError_t k = launch_chained(c, rw_keys_csf_kernel, grid_for(c, std::max(B.nnz, (i64)1), RK_TILE), OT, 0, form, B, d, b.kA, b.pA, passes_of(bits),
+                                         reinterpret_cast<SortHead*>(b.sort_tmp), b.pos, m);
+    return k != cudaSuccess ? k : rw_reorder(c, B.nnz, m, bits, true, b);
 }
 
 cudaError_t launch_rw_values(const LaunchCtx& c, const void* val, const int* src, i64 n, void* out) {

@@ -98,9 +98,10 @@ __device__ __forceinline__ int classify_row(i64 ub, i64 entries, int jmin, int j
 // (one load, neighbouring rows share sectors) instead of two offsets and two coordinates.
 // It is the first kernel of a pass and clears the control block on the way (ctl non-null).
 __global__ void __launch_bounds__(256) brow_summary_kernel(Csr B, int4* __restrict__ brow, DevCtl* ctl) {
+    const int tid = chained_start(threadIdx.x);
     if (ctl && blockIdx.x == 0)
         for (int w = threadIdx.x; w < (int)(sizeof(DevCtl) / 4); w += 256) reinterpret_cast<int*>(ctl)[w] = 0;
-    for (i64 k = (i64)blockIdx.x * blockDim.x + threadIdx.x; k < B.nrows; k += (i64)gridDim.x * blockDim.x) {
+    for (i64 k = (i64)blockIdx.x * blockDim.x + tid; k < B.nrows; k += (i64)gridDim.x * blockDim.x) {
         const i64 qs = B.pos[k], qe = B.pos[k + 1];
         int4 s = make_int4(0x7fffffff, -1, 0, 0);
         if (qe > qs) {
@@ -229,6 +230,7 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
     __shared__ int s_long[LONG_LIST], s_nlong;
     // rows of more than two steps of a narrow lane group, which the block's warps take at the end
     __shared__ int s_mid[MID_LIST], s_nmid;
+    chained_start();
     for (int x = threadIdx.x; x < 8 * NCLASS; x += blockDim.x) { (&s_hist[0][0])[x] = 0; (&s_clow[0][0])[x] = 0; (&s_cprod[0][0])[x] = 0; }
     if (threadIdx.x == 0) { s_max_ub = 0; s_max_ub_global = 0; s_max_ub_smem = 0; s_max_span_words = 0; s_bm_words = 0; s_order_words = 0; s_nlong = s_nmid = 0; }
     __syncthreads();
@@ -252,7 +254,8 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
     // eight lanes or more per row: neighbouring rows go to different blocks (the heaviest rows of a graph are often
     // neighbours); narrower groups take neighbouring rows for the sake of the row offsets they share
     const i64 ngroups = ((i64)gridDim.x * blockDim.x) / G;
-    const i64 group = G >= 8 ? (i64)(threadIdx.x / G) * gridDim.x + blockIdx.x : ((i64)blockIdx.x * blockDim.x + threadIdx.x) / G;
+    i64 group = G >= 8 ? (i64)(threadIdx.x / G) * gridDim.x + blockIdx.x : ((i64)blockIdx.x * blockDim.x + threadIdx.x) / G;
+    not_before(group);
     unsigned my_max = 0;                            // most products of a row below 2^32
     // rows and products of the class of this group's last rows: neighbouring rows mostly share a
     // class, so the shared-memory histogram is touched only when the class changes
@@ -452,13 +455,14 @@ cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i6
     if (c.brow) {
         i64 want = ((i64)B.nrows + threads - 1) / threads;
         i64 cap = (i64)c.sm_count * 8;
-        brow_summary_kernel<<<(int)(want < cap ? want : cap), threads, 0, c.stream>>>(B, c.brow, clear_ctl ? c.ctl : nullptr);
-        ++c.launches;
+        const cudaError_t e = launch_chained(c, brow_summary_kernel, want < cap ? want : cap, threads, 0, B, c.brow, clear_ctl ? c.ctl : nullptr);
+        if (e != cudaSuccess) return e;
     } else if (clear_ctl) {
         cudaError_t e = cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream);
         if (e != cudaSuccess) return e;
     }
-    auto launch = [&](auto kernel, int G) { kernel<<<grid_for(G), threads, 0, c.stream>>>(A, B, c.tab, c.prm, c.ctl, c.brow); };
+    cudaError_t e = cudaSuccess;
+    auto launch = [&](auto kernel, int G) { e = launch_chained(c, kernel, grid_for(G), threads, 0, A, B, c.tab, c.prm, c.ctl, c.brow); };
     const bool sm = c.brow != nullptr;
     if (avg <= 1.5) sm ? launch(row_bounds_kernel<1, true>, 1) : launch(row_bounds_kernel<1, false>, 1);
     else if (avg <= 3.0) sm ? launch(row_bounds_kernel<2, true>, 2) : launch(row_bounds_kernel<2, false>, 2);
@@ -471,8 +475,7 @@ cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i6
     // the line, well on the side of many rows, gives up 6 us between 2^15 and 2^16)
     else if (avg <= (A.nrows >= (1 << 16) ? 32.0 : 12.0)) sm ? launch(row_bounds_kernel<8, true>, 8) : launch(row_bounds_kernel<8, false>, 8);
     else sm ? launch(row_bounds_kernel<32, true>, 32) : launch(row_bounds_kernel<32, false>, 32);
-    ++c.launches;
-    return cudaGetLastError();
+    return e;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -651,6 +654,7 @@ cudaError_t launch_cta_prepare(const LaunchCtx& c, i64 products, const Csr& B) {
 // the bounds kernel instead, the fences of its blocks cost 6 .. 14 us).
 __global__ void __launch_bounds__(256, 4) bin_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, HostBlock* host, int seq, u64* look, int n_look) {
     __shared__ int s_units[UNIT_BUCKETS];
+    chained_start();
     const bool too_small = ctl->bm_words > prm.bm_arena_words;
     if (blockIdx.x == 0) {
         if (threadIdx.x == 0) {
@@ -732,9 +736,7 @@ cudaError_t launch_bin_rows(const LaunchCtx& c, int m) {
     i64 want = ((i64)m + 1023) / 1024;
     i64 cap = (i64)c.sm_count * 8;
     if (want < 1) want = 1;
-    bin_rows_kernel<<<1 + (int)(want < cap ? want : cap), 256, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.seq, c.look, c.n_look);
-    ++c.launches;
-    return cudaGetLastError();
+    return launch_chained(c, bin_rows_kernel, 1 + (want < cap ? want : cap), 256, 0, m, c.tab, c.prm, c.ctl, c.host, c.seq, c.look, c.n_look);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -781,6 +783,7 @@ __global__ void __launch_bounds__(FR_THREADS, DENSE ? 3 : 5) finish_rows_kernel(
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned all = 0xffffffffu, below = (1u << lane) - 1u;
     const int tiles = gridDim.x;
+    chained_start();
     if (tid == 0) s_tile = atomicAdd(&ctl->rows_ticket, 1);
     for (int x = tid; x < FR_WARPS * N_PUBLIC_CLASS; x += FR_THREADS) (&s_cls[0][0])[x] = 0;
     if (tid >= 128 && tid < 128 + UNIT_BUCKETS) s_units[tid - 128] = 0;
@@ -1046,6 +1049,7 @@ __global__ void __launch_bounds__(FR_THREADS) finish_slices_kernel(int n_i, cons
     __shared__ i64 s_before;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tiles = gridDim.x;
+    chained_start();
     if (tid == 0) s_tile = atomicAdd(&ctl->slices_ticket, 1);
     __syncthreads();
     const int tile = s_tile;
@@ -1104,22 +1108,19 @@ size_t look_words(i64 rows, i64 slices) { return (size_t)2 * tiles_of(rows, FR_T
 
 cudaError_t launch_finish_rows(const LaunchCtx& c, int m, bool any_dense, i64* rowptr) {
     const int tiles = tiles_of(m, FR_TILE);
-    if (any_dense) finish_rows_kernel<true, false><<<tiles, FR_THREADS, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.seq + 1, c.look, rowptr, FibreArgs{});
-    else finish_rows_kernel<false, false><<<tiles, FR_THREADS, 0, c.stream>>>(m, c.tab, c.prm, c.ctl, c.host, c.seq + 1, c.look, rowptr, FibreArgs{});
-    ++c.launches;
-    return cudaGetLastError();
+    return launch_chained(c, any_dense ? finish_rows_kernel<true, false> : finish_rows_kernel<false, false>, tiles, FR_THREADS, 0, m, c.tab, c.prm, c.ctl,
+                          c.host, c.seq + 1, c.look, rowptr, FibreArgs{});
 }
 
 cudaError_t launch_finish_fibres(const LaunchCtx& c, int n_i, int n_ij, bool any_dense, const i64* Apos1, const int* Acrd0, const int* Acrd1,
                                  i64* rowptr_raw, i64* sfp, i64* Cpos0, int* Ccrd0, i64* Cpos1, int* Ccrd1, i64* Cpos2) {
     const int tiles = tiles_of(n_ij, FR_TILE);
     const FibreArgs f{Apos1, Acrd1, n_i, sfp, Ccrd1, Cpos2};
-    if (any_dense) finish_rows_kernel<true, true><<<tiles, FR_THREADS, 0, c.stream>>>(n_ij, c.tab, c.prm, c.ctl, c.host, c.seq + 1, c.look, rowptr_raw, f);
-    else finish_rows_kernel<false, true><<<tiles, FR_THREADS, 0, c.stream>>>(n_ij, c.tab, c.prm, c.ctl, c.host, c.seq + 1, c.look, rowptr_raw, f);
-    finish_slices_kernel<<<tiles_of(n_i, SL_TILE), FR_THREADS, 0, c.stream>>>(n_i, sfp, Acrd0, c.ctl, c.host, c.seq + 1, c.look + 2 * tiles, Ccrd0, Cpos1,
-                                                                             Cpos0);
-    c.launches += 2;
-    return cudaGetLastError();
+    const cudaError_t e = launch_chained(c, any_dense ? finish_rows_kernel<true, true> : finish_rows_kernel<false, true>, tiles, FR_THREADS, 0, n_ij, c.tab,
+                                         c.prm, c.ctl, c.host, c.seq + 1, c.look, rowptr_raw, f);
+    if (e != cudaSuccess) return e;
+    return launch_chained(c, finish_slices_kernel, tiles_of(n_i, SL_TILE), FR_THREADS, 0, n_i, sfp, Acrd0, c.ctl, c.host, c.seq + 1, c.look + 2 * tiles, Ccrd0,
+                          Cpos1, Cpos0);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -83,8 +83,9 @@ __global__ void __launch_bounds__(RS_THREADS) radix_pass_kernel(const u64* __res
     __shared__ u64 s_key[RS_TILE];
     __shared__ T s_val[VALUES ? RS_TILE : 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, shift = 8 * pass;
-    if (threadIdx.x == 0) s_tile = atomicAdd(&head->ticket[pass], 1);
     for (int d = lane; d < 256; d += 32) s_cnt[warp][d] = 0;
+    chained_start();
+    if (threadIdx.x == 0) s_tile = atomicAdd(&head->ticket[pass], 1);
     __syncthreads();
     const int tile = s_tile;
     const i64 base = (i64)tile * RS_TILE + (i64)warp * (RS_STEPS * 32);
@@ -178,8 +179,8 @@ static cudaError_t radix_sort_t(const LaunchCtx& c, i64 n, int bits, u64* k0, T*
     u64 *ki = k0, *ko = k1;
     T *vi = v0, *vo = v1;
     for (int pass = 0; pass < passes; ++pass) {
-        radix_pass_kernel<T, VALUES><<<nblocks, RS_THREADS, 0, c.stream>>>(ki, vi, n, pass, head, status, c.ctl, ko, vo);
-        ++c.launches;
+        const cudaError_t e = launch_chained(c, radix_pass_kernel<T, VALUES>, nblocks, RS_THREADS, 0, ki, vi, n, pass, head, status, c.ctl, ko, vo);
+        if (e != cudaSuccess) return e;
         u64* tk = ki; ki = ko; ko = tk;
         T* tv = vi; vi = vo; vo = tv;
         *in_first = !*in_first;

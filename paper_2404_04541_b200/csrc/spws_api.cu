@@ -523,6 +523,7 @@ LaunchCtx make_ctx(const spws_plan_s* p, char* scratch, size_t scratch_bytes, co
     }
     if (L.has_brow) c.brow = reinterpret_cast<int4*>(scratch + L.brow);
     c.host = p->host;
+    c.chain = !p->profiling;
     c.look = reinterpret_cast<u64*>(scratch + L.look);
     c.n_look = L.n_look;
     return c;
@@ -622,7 +623,8 @@ public:
         const bool sparse = p->sparse_products >= FORK_PRODUCTS;
         sparse_ = sparse ? 0 : warp ? 1 : 2;
         if ((int)sparse + (int)warp + (int)rest >= 2 && !p->profiling) h_ = p->h->fork_on();
-        on_ = h_ && cudaEventRecord(h_->forked, main_) == cudaSuccess;
+    on_ = h_ && cudaEventRecord(h_->forked, main_) == cudaSuccess;
+        if (on_) c_.chain = 0;
     }
     ~Fork() { join(); }
     // the kernels launched next belong to this group: 0 sparse, 1 dense by warps, 2 the rest (on the caller's stream)
@@ -808,6 +810,7 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, cha
     // (a pass that is being captured clears the counters itself: it may run any number of times)
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     CUDA_TRY(cudaStreamIsCapturing(c.stream, &capture));
+    if (capture != cudaStreamCaptureStatusNone) c.chain = 0;
     if (!plan->counters_clear || capture != cudaStreamCaptureStatusNone)
         CUDA_TRY(cudaMemsetAsync(c.ctl->work_counter, 0, sizeof(c.ctl->work_counter), c.stream));
     plan->counters_clear = false;
