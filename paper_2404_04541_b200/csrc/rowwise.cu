@@ -27,13 +27,28 @@ __device__ __forceinline__ int owner_row(const i64* __restrict__ pos, int lo, in
     return lo;
 }
 
+// The same by a whole warp, 32 probes a step: a block looks for the owners of its tile among all rows first (the keys of 1e6 entries
+// in 5e5 fibres 31 us by halves, 27 us like this; of 7e5 in 5e4 rows 23 and 18).
+__device__ __forceinline__ int owner_row_warp(const i64* __restrict__ pos, int lo, int hi, i64 p) {
+    const int lane = threadIdx.x & 31;
+    while (hi - lo > 1) {
+        const int step = (int)(((unsigned)(hi - lo) + 31u) >> 5);
+        const i64 at = lo + (i64)lane * step;
+        const int n = __popc(__ballot_sync(0xffffffffu, at < hi && __ldg(pos + at) <= p));       // (one at least)
+        hi = (int)min((i64)hi, lo + (i64)n * step);
+        lo += (n - 1) * step;
+    }
+    return lo;
+}
+
 constexpr int RK_ITEMS = 4;
 constexpr int RK_TILE = OT * RK_ITEMS;
 
-// Output-row label and payload (picked row above, entry below) of every entry; a block takes a tile of
+// Output-row label (K: 32 bits where they hold it) and picked row of every entry; a block takes a tile of
 // consecutive entries, so the owners of its first and last entry bound every search.  B's columns
 // are checked on the way (the row kernels look at the ends of a row only).
-__global__ void __launch_bounds__(OT) rw_keys_outer_kernel(Csr At, i64 n, Csr B, i64 nnzB, u64* __restrict__ keys, u64* __restrict__ pay,
+template <typename K>
+__global__ void __launch_bounds__(OT) rw_keys_outer_kernel(Csr At, i64 n, Csr B, i64 nnzB, K* __restrict__ keys, int* __restrict__ pick,
                                                            int passes, SortHead* head, DevCtl* ctl) {
     __shared__ int s_lo, s_hi;
     __shared__ DigitCounts s_digits;
@@ -45,17 +60,22 @@ __global__ void __launch_bounds__(OT) rw_keys_outer_kernel(Csr At, i64 n, Csr B,
     for (i64 q = (i64)blockIdx.x * OT + threadIdx.x; q < nnzB; q += (i64)gridDim.x * OT) bad |= (unsigned)__ldg(B.crd + q) >= (unsigned)B.ncols;
     for (i64 t0 = (i64)blockIdx.x * RK_TILE; t0 < n; t0 += (i64)gridDim.x * RK_TILE) {
         __syncthreads();
-        if (threadIdx.x == 0) s_lo = owner_row(At.pos, 0, At.nrows, t0);
-        if (threadIdx.x == 32) s_hi = owner_row(At.pos, 0, At.nrows, min(n, t0 + RK_TILE) - 1) + 1;
+        if (threadIdx.x < 32) {
+            const int r = owner_row_warp(At.pos, 0, At.nrows, t0);
+            if (threadIdx.x == 0) s_lo = r;
+        } else if (threadIdx.x < 64) {
+            const int r = owner_row_warp(At.pos, 0, At.nrows, min(n, t0 + RK_TILE) - 1);
+            if (threadIdx.x == 32) s_hi = r + 1;
+        }
         __syncthreads();
         for (int x = 0; x < RK_ITEMS; ++x) {
             const i64 p = t0 + x * OT + threadIdx.x;
             if (p >= n) break;
             const int i = __ldg(At.crd + p);
             bad |= (unsigned)i >= (unsigned)At.ncols;
-            keys[p] = (u64)(unsigned)i;
+            keys[p] = (K)(unsigned)i;
             s_digits.add((u64)(unsigned)i, passes);
-            pay[p] = ((u64)(unsigned)owner_row(At.pos, s_lo, s_hi, p) << 32) | (u64)(unsigned)p;
+            pick[p] = owner_row(At.pos, s_lo, s_hi, p);
         }
     }
     s_digits.flush(passes, head);
@@ -64,7 +84,8 @@ __global__ void __launch_bounds__(OT) rw_keys_outer_kernel(Csr At, i64 n, Csr B,
 
 // form: 0 SpTTM, 1 SpTTM-I, 2 SpMTTKRP.  `d` = extent of the label's inner coordinate (forms 0, 1).
 // pos[0 .. m] := nnz on the way (rw_sparse_rows_kernel writes the rows there are).
-__global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u64 d, u64* __restrict__ keys, u64* __restrict__ pay, int passes,
+template <typename K>
+__global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u64 d, K* __restrict__ keys, int* __restrict__ picks, int passes,
                                                          SortHead* head, i64* __restrict__ pos, i64 m) {
     __shared__ int s_f[2], s_s[2];
     __shared__ DigitCounts s_digits;
@@ -78,11 +99,11 @@ __global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u6
     for (i64 i = (i64)blockIdx.x * OT + threadIdx.x; i <= m; i += (i64)gridDim.x * OT) pos[i] = B.nnz;
     for (i64 t0 = (i64)blockIdx.x * RK_TILE; t0 < B.nnz; t0 += (i64)gridDim.x * RK_TILE) {
         __syncthreads();
-        if ((threadIdx.x & 31) == 0 && threadIdx.x < 64) {
+        if (threadIdx.x < 64) {
             const int which = threadIdx.x >> 5;
-            const int f = owner_row(B.pos2, 0, B.n1, which == 0 ? t0 : min(B.nnz, t0 + RK_TILE) - 1);
-            s_f[which] = f;
-            s_s[which] = owner_row(B.pos1, 0, B.n0, f);
+            const int f = owner_row_warp(B.pos2, 0, B.n1, which == 0 ? t0 : min(B.nnz, t0 + RK_TILE) - 1);
+            const int s = owner_row_warp(B.pos1, 0, B.n0, f);
+            if ((threadIdx.x & 31) == 0) { s_f[which] = f; s_s[which] = s; }
         }
         __syncthreads();
         for (int x = 0; x < RK_ITEMS; ++x) {
@@ -97,40 +118,43 @@ __global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u6
                 key = (form == 0 ? c1 : c0) * d + c2;
                 pick = form == 0 ? c0 : c1;
             }
-            keys[e] = key;
+            keys[e] = (K)key;
             s_digits.add(key, passes);
-            pay[e] = (pick << 32) | (u64)(unsigned)e;
+            picks[e] = (int)pick;
         }
     }
     s_digits.flush(passes, head);
 }
 
 // CSR result: the reordered operand has one row per output row; pos by binary search in the sorted labels.
-__global__ void __launch_bounds__(OT) rw_dense_rows_kernel(const u64* __restrict__ keys, const u64* __restrict__ pay, i64 n, i64 m,
+template <typename K>
+__global__ void __launch_bounds__(OT) rw_dense_rows_kernel(const K* __restrict__ keys, const int* __restrict__ entry, const int* __restrict__ pick, i64 n, i64 m,
                                                            i64* __restrict__ pos, int* __restrict__ crd, int* __restrict__ src) {
     const i64 stride = (i64)gridDim.x * OT, t0 = (i64)blockIdx.x * OT + threadIdx.x;
     chained_start();
     not_before(keys);
-    not_before(pay);
+    not_before(entry);
+    not_before(pick);
     for (i64 i = t0; i <= m; i += stride) {
         i64 lo = 0, hi = n;
         while (lo < hi) {
             const i64 mid = (lo + hi) >> 1;
-            if (keys[mid] < (u64)i) lo = mid + 1; else hi = mid;
+            if ((u64)keys[mid] < (u64)i) lo = mid + 1; else hi = mid;
         }
         pos[i] = lo;
     }
     for (i64 p = t0; p < n; p += stride) {
-        const u64 w = pay[p];
-        crd[p] = (int)(w >> 32);
-        src[p] = (int)(unsigned)w;
+        const int e = entry[p];
+        crd[p] = pick[(unsigned)e];
+        src[p] = e;
     }
 }
 
 // Coordinate-form result: only the labels that occur become rows, in order (row r has label row_key[r]);
 // pos was filled with n, so the rows past the last label are empty.  Tiles hand the number of rows
 // on as in reduce_runs_kernel.  More than m labels mean a coordinate out of its range.
-__global__ void __launch_bounds__(OT) rw_sparse_rows_kernel(const u64* __restrict__ keys, const u64* __restrict__ pay, i64 n, i64 m,
+template <typename K>
+__global__ void __launch_bounds__(OT) rw_sparse_rows_kernel(const K* __restrict__ keys, const int* __restrict__ entry, const int* __restrict__ pick, i64 n, i64 m,
                                                             int* __restrict__ ticket, u64* __restrict__ status, DevCtl* ctl,
                                                             u64* __restrict__ row_key, i64* __restrict__ pos, int* __restrict__ crd,
                                                             int* __restrict__ src) {
@@ -148,11 +172,11 @@ __global__ void __launch_bounds__(OT) rw_sparse_rows_kernel(const u64* __restric
 #pragma unroll
     for (int x = 0; x < RK_ITEMS; ++x) {
         const i64 p = t0 + x * OT + threadIdx.x;
-        key[x] = p < n ? keys[p] : ABSENT_LABEL;
+        key[x] = p < n ? (u64)keys[p] : ABSENT_LABEL;
         if (p < n) {
-            const u64 w = pay[p];
-            crd[p] = (int)(w >> 32);
-            src[p] = (int)(unsigned)w;
+            const int e = entry[p];
+            crd[p] = pick[(unsigned)e];
+            src[p] = e;
         }
         if (lane == 31) s_edge[x][warp] = key[x];
     }
@@ -166,7 +190,7 @@ __global__ void __launch_bounds__(OT) rw_sparse_rows_kernel(const u64* __restric
         if (lane == 0) {
             if (warp > 0) prev = s_edge[x][warp - 1];
             else if (x > 0) prev = s_edge[x - 1][OT / 32 - 1];
-            else prev = t0 > 0 ? keys[t0 - 1] : ABSENT_LABEL;
+            else prev = t0 > 0 ? (u64)keys[t0 - 1] : ABSENT_LABEL;
         }
         head[x] = key[x] != ABSENT_LABEL && key[x] != prev;
         int round;
@@ -359,36 +383,57 @@ static int passes_of(int bits) { return (bits + 7) / 8; }
 // Sorts the entries by output row and writes the reordered operand (all but its values).  `sparse`: a row per
 // label that occurs (at most m), labels to row_key; otherwise a row per label value.  The kernel that wrote the labels has
 // counted their digits (a kernel of its own for that, one for `pos` and their clearing took 10 .. 18 us a call).
+// Only the labels and 32-bit entry numbers move (the picked row is fetched at the end), labels of 32 bits where they fit: 1e6 entries
+// of 22 bits in three passes 79 us with labels, picked rows and entries in 16 bytes, 57 us like this; 7e5 of 18 bits 62 and 46.
+template <typename K>
 static cudaError_t rw_reorder(const LaunchCtx& c, i64 n, i64 m, int bits, bool sparse, const RowwiseBufs& b) {
     cudaError_t e;
     bool first = true;
-    if ((e = radix_sort_t<u64, true>(c, n, bits, b.kA, b.pA, b.kB, b.pB, b.sort_tmp, &first, true)) != cudaSuccess) return e;
-    const u64* ks = first ? b.kA : b.kB;
-    const u64* ps = first ? b.pA : b.pB;
-    if (!sparse) {
-        return launch_chained(c, rw_dense_rows_kernel, grid_for(c, n > m ? n : m + 1, OT), OT, 0, ks, ps, n, m, b.pos, b.crd, b.src);
-    } else if (n > 0) {
-        const int tiles = (int)((n + RK_TILE - 1) / RK_TILE);
-        u64* const words = reinterpret_cast<u64*>(b.sort_tmp + sort_scratch_bytes(n));
-        return launch_chained(c, rw_sparse_rows_kernel, tiles, OT, 0, ks, ps, n, m, reinterpret_cast<int*>(words), words + 1, c.ctl, b.row_key, b.pos, b.crd, b.src);
-    }
-    return cudaGetLastError();
+    K *const k0 = reinterpret_cast<K*>(b.kA), *const k1 = reinterpret_cast<K*>(b.kB);
+    if (n == 1 && (e = cudaMemsetAsync(b.entry[0], 0, sizeof(int), c.stream)) != cudaSuccess) return e;      // (nothing to sort)
+    if ((e = radix_sort_t<K, int, true>(c, n, bits, k0, b.entry[0], k1, b.entry[1], b.sort_tmp, &first, true, true)) != cudaSuccess) return e;
+    const K* ks = first ? k0 : k1;
+    const int* es = first ? b.entry[0] : b.entry[1];
+    if (!sparse) return launch_chained(c, rw_dense_rows_kernel<K>, grid_for(c, n > m ? n : m + 1, OT), OT, 0, ks, es, b.pick, n, m, b.pos, b.crd, b.src);
+    if (n == 0) return cudaSuccess;
+    const int tiles = (int)((n + RK_TILE - 1) / RK_TILE);
+    u64* const words = reinterpret_cast<u64*>(b.sort_tmp + sort_scratch_bytes(n));
+    return launch_chained(c, rw_sparse_rows_kernel<K>, tiles, OT, 0, ks, es, b.pick, n, m, reinterpret_cast<int*>(words), words + 1, c.ctl, b.row_key, b.pos, b.crd, b.src);
+}
+
+template <typename K>
+static cudaError_t rw_outer_t(const LaunchCtx& c, const Csr& At, i64 n, const Csr& B, i64 nnzB, int bits, const RowwiseBufs& b) {
+    const cudaError_t e = launch_chained(c, rw_keys_outer_kernel<K>, grid_for(c, std::max(n, nnzB), RK_TILE), OT, 0, At, n, B, nnzB, reinterpret_cast<K*>(b.kA), b.pick,
+                                         passes_of(bits), reinterpret_cast<SortHead*>(b.sort_tmp), c.ctl);
+    return e != cudaSuccess ? e : rw_reorder<K>(c, n, At.ncols, bits, false, b);
+}
+
+// Clears the control block and the sort's temporaries (a memset each took the host 3 .. 4 us more).
+__global__ void __launch_bounds__(OT) rw_clear_kernel(int* __restrict__ ctl, int n_ctl, int4* __restrict__ tmp, i64 n_tmp) {
+    chained_start();
+    const i64 t0 = (i64)blockIdx.x * OT + threadIdx.x, stride = (i64)gridDim.x * OT;
+    for (i64 i = t0; i < n_ctl; i += stride) ctl[i] = 0;
+    for (i64 i = t0; i < n_tmp; i += stride) tmp[i] = make_int4(0, 0, 0, 0);
+}
+
+cudaError_t launch_rw_clear(const LaunchCtx& c, i64 n, char* tmp) {
+    const i64 quads = (i64)(rw_sort_bytes(n) + 15) / 16;           // (its room is a multiple of 256 bytes)
+    return launch_chained(c, rw_clear_kernel, grid_for(c, quads, OT), OT, 0, reinterpret_cast<int*>(c.ctl), (int)(sizeof(DevCtl) / 4), reinterpret_cast<int4*>(tmp), quads);
 }
 
 cudaError_t launch_rw_outer(const LaunchCtx& c, const Csr& At, i64 n, const Csr& B, i64 nnzB, int bits, const RowwiseBufs& b) {
-    const cudaError_t e = cudaMemsetAsync(b.sort_tmp, 0, rw_sort_bytes(n), c.stream);
-    if (e != cudaSuccess) return e;
-    const cudaError_t k = launch_chained(c, rw_keys_outer_kernel, grid_for(c, std::max(n, nnzB), RK_TILE), OT, 0, At, n, B, nnzB, b.kA, b.pA, passes_of(bits),
-                                         reinterpret_cast<SortHead*>(b.sort_tmp), c.ctl);
-    return k != cudaSuccess ? k : rw_reorder(c, n, At.ncols, bits, false, b);
+    return rw_outer_t<unsigned>(c, At, n, B, nnzB, bits, b);        // (a row number)
+}
+
+template <typename K>
+static cudaError_t rw_csf_t(const LaunchCtx& c, int form, const Csf3Dev& B, u64 d, i64 m, int bits, const RowwiseBufs& b) {
+    const cudaError_t e = launch_chained(c, rw_keys_csf_kernel<K>, grid_for(c, std::max(B.nnz, (i64)1), RK_TILE), OT, 0, form, B, d, reinterpret_cast<K*>(b.kA), b.pick,
+                                         passes_of(bits), reinterpret_cast<SortHead*>(b.sort_tmp), b.pos, m);
+    return e != cudaSuccess ? e : rw_reorder<K>(c, B.nnz, m, bits, true, b);
 }
 
 cudaError_t launch_rw_csf(const LaunchCtx& c, int form, const Csf3Dev& B, u64 d, i64 m, int bits, const RowwiseBufs& b) {
-    const cudaError_t e = cudaMemsetAsync(b.sort_tmp, 0, rw_sort_bytes(B.nnz), c.stream);
-    if (e != cudaSuccess) return e;
-    const cudaError_t k = launch_chained(c, rw_keys_csf_kernel, grid_for(c, std::max(B.nnz, (i64)1), RK_TILE), OT, 0, form, B, d, b.kA, b.pA, passes_of(bits),
-                                         reinterpret_cast<SortHead*>(b.sort_tmp), b.pos, m);
-    return k != cudaSuccess ? k : rw_reorder(c, B.nnz, m, bits, true, b);
+    return bits <= 32 ? rw_csf_t<unsigned>(c, form, B, d, m, bits, b) : rw_csf_t<u64>(c, form, B, d, m, bits, b);
 }
 
 cudaError_t launch_rw_values(const LaunchCtx& c, const void* val, const int* src, i64 n, void* out) {

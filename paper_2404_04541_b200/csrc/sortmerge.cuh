@@ -4,6 +4,8 @@
 // order, and the driver that feeds the products in rounds of the accumulation array's capacity.
 // Included by the translation units that instantiate it.
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace spws {
@@ -71,30 +73,32 @@ static __global__ void __launch_bounds__(RS_THREADS) radix_hist_kernel(const u64
         if (s_h[p][threadIdx.x]) atomicAdd(&head->hist[p][threadIdx.x], s_h[p][threadIdx.x]);
 }
 
-template <typename T, bool VALUES>
-__global__ void __launch_bounds__(RS_THREADS) radix_pass_kernel(const u64* __restrict__ keys, const T* __restrict__ vals, i64 n, int pass,
+// K: labels of 32 or 64 bits.  `numbered`: the first pass over elements whose values are their places.
+template <typename K, typename T, bool VALUES>
+__global__ void __launch_bounds__(RS_THREADS) radix_pass_kernel(const K* __restrict__ keys, const T* __restrict__ vals, bool numbered, i64 n, int pass,
                                                                 SortHead* __restrict__ head, u64* __restrict__ status, DevCtl* ctl,
-                                                                u64* __restrict__ keys_out, T* __restrict__ vals_out) {
+                                                                K* __restrict__ keys_out, T* __restrict__ vals_out) {
     __shared__ int s_cnt[RS_WARPS][256];        // elements with the digit in this warp's slice, then their start inside the digit's part
     __shared__ int s_start[256];                // start of the digit's part inside the tile
     __shared__ i64 s_goff[256];
     __shared__ int s_ws[33];
     __shared__ int s_tile;
-    __shared__ u64 s_key[RS_TILE];
+    __shared__ K s_key[RS_TILE];
     __shared__ T s_val[VALUES ? RS_TILE : 1];
+    constexpr bool numbers = std::is_same<T, int>::value;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, shift = 8 * pass;
-    for (int d = lane; d < 256; d += 32) s_cnt[warp][d] = 0;
-    chained_start();
+    if constexpr (sizeof(K) == 4) chained_start();        // (not for long sorts, which are none the faster for it)
     if (threadIdx.x == 0) s_tile = atomicAdd(&head->ticket[pass], 1);
+    for (int d = lane; d < 256; d += 32) s_cnt[warp][d] = 0;
     __syncthreads();
     const int tile = s_tile;
     const i64 base = (i64)tile * RS_TILE + (i64)warp * (RS_STEPS * 32);
-    u64 key[RS_STEPS];
+    K key[RS_STEPS];
     int rank[RS_STEPS];
 #pragma unroll
     for (int st = 0; st < RS_STEPS; ++st) {
         const i64 t = base + st * 32 + lane;
-        key[st] = t < n ? keys[t] : ~0ull;
+        key[st] = t < n ? keys[t] : (K)~0ull;
     }
 #pragma unroll
     for (int st = 0; st < RS_STEPS; ++st) {
@@ -127,7 +131,7 @@ __global__ void __launch_bounds__(RS_THREADS) radix_pass_kernel(const u64* __res
         const int digit0 = block_excl_scan<RS_THREADS>(head->hist[pass][d], s_ws, all);
         i64 before = 0;
         if (tile > 0) {
-            before = look_back(status + d, 256, tile, pass, ctl);
+            before = look_back<sizeof(K) == 4 ? 4 : 1>(status + d, 256, tile, pass, ctl);      // (four cost the other registers)
             look_publish(mine, 2 * pass + 2, before + run);
         }
         s_start[d] = start;
@@ -141,12 +145,12 @@ __global__ void __launch_bounds__(RS_THREADS) radix_pass_kernel(const u64* __res
             const unsigned d = (unsigned)(key[st] >> shift) & 255u;
             const int at = s_start[d] + s_cnt[warp][d] + rank[st];
             s_key[at] = key[st];
-            if (VALUES) s_val[at] = vals[t];
+            if (VALUES) s_val[at] = numbers && numbered ? (T)t : vals[t];
         }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < tile_total; i += RS_THREADS) {
-        const u64 k = s_key[i];
+        const K k = s_key[i];
         const i64 at = s_goff[(unsigned)(k >> shift) & 255u] + i;
         keys_out[at] = k;
         if (VALUES) vals_out[at] = s_val[i];
@@ -161,27 +165,33 @@ static size_t sort_scratch_bytes(i64 n) {
 // Sorts n (label, value) pairs by label; `bits` = number of significant label bits.  Input in
 // (k0, v0), the other buffer in (k1, v1); *in_first tells which pair holds the result.  `counted`: the caller has cleared
 // `tmp`, and its kernel that wrote the labels has counted their digits (DigitCounts).
-template <typename T, bool VALUES>
-static cudaError_t radix_sort_t(const LaunchCtx& c, i64 n, int bits, u64* k0, T* v0, u64* k1, T* v1, char* tmp, bool* in_first, bool counted = false) {
+// `numbered`: the values are the elements' places, and v0 is not read.
+template <typename K, typename T, bool VALUES>
+static cudaError_t radix_sort_t(const LaunchCtx& c, i64 n, int bits, K* k0, T* v0, K* k1, T* v1, char* tmp, bool* in_first, bool counted = false, bool numbered = false) {
     *in_first = true;
     if (n <= 1) return cudaSuccess;
     const int nblocks = (int)((n + RS_TILE - 1) / RS_TILE);
     const int passes = (bits + 7) / 8;
     SortHead* head = reinterpret_cast<SortHead*>(tmp);
     u64* status = reinterpret_cast<u64*>(tmp + sort_head_bytes());
-    if (!counted) {
+    if constexpr (sizeof(K) == 8) if (!counted) {
         const cudaError_t e = cudaMemsetAsync(tmp, 0, sort_scratch_bytes(n), c.stream);
         if (e != cudaSuccess) return e;
         const int hist_blocks = 4 * c.sm_count;
         radix_hist_kernel<<<nblocks < hist_blocks ? nblocks : hist_blocks, RS_THREADS, 0, c.stream>>>(k0, n, passes, head);
         ++c.launches;
     }
-    u64 *ki = k0, *ko = k1;
+    K *ki = k0, *ko = k1;
     T *vi = v0, *vo = v1;
     for (int pass = 0; pass < passes; ++pass) {
-        const cudaError_t e = launch_chained(c, radix_pass_kernel<T, VALUES>, nblocks, RS_THREADS, 0, ki, vi, n, pass, head, status, c.ctl, ko, vo);
-        if (e != cudaSuccess) return e;
-        u64* tk = ki; ki = ko; ko = tk;
+        if constexpr (sizeof(K) == 4) {
+            const cudaError_t e = launch_chained(c, radix_pass_kernel<K, T, VALUES>, nblocks, RS_THREADS, 0, ki, vi, numbered && pass == 0, n, pass, head, status, c.ctl, ko, vo);
+            if (e != cudaSuccess) return e;
+        } else {
+            radix_pass_kernel<K, T, VALUES><<<nblocks, RS_THREADS, 0, c.stream>>>(ki, vi, numbered && pass == 0, n, pass, head, status, c.ctl, ko, vo);
+            ++c.launches;
+        }
+        K* tk = ki; ki = ko; ko = tk;
         T* tv = vi; vi = vo; vo = tv;
         *in_first = !*in_first;
     }
@@ -270,7 +280,7 @@ template <typename T, bool VALUES>
 static cudaError_t sort_reduce_t(const LaunchCtx& c, i64 n, int label_bits, u64* k, T* v, u64* k2, T* v2, char* sort_tmp, i64* cnt_dev,
                                  i64* cnt_host_pinned, bool* result_in_first) {
     bool first = true;
-    cudaError_t e = radix_sort_t<T, VALUES>(c, n, label_bits, k, v, k2, v2, sort_tmp, &first);
+    cudaError_t e = radix_sort_t<u64, T, VALUES>(c, n, label_bits, k, v, k2, v2, sort_tmp, &first);
     if (e != cudaSuccess) return e;
     u64* ks = first ? k : k2;
     T* vs = first ? v : v2;

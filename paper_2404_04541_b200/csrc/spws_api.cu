@@ -951,7 +951,7 @@ spws_status_t outer_count_products(spws_plan_s* p, const Shapes& S, int64_t* P) 
 
 // ---- second- and higher-order forms taken row by row (rowwise.cu) -----------------------------
 struct RwLayout {
-    size_t kA, kB, pA, pB, sort_tmp, pos, crd, src, val, row_key, rowptr, cols, fcnt, fpos, fcrd, fval, block_sums, bytes;
+    size_t kA, kB, entry[2], pick, sort_tmp, pos, crd, src, val, row_key, rowptr, cols, fcnt, fpos, fcrd, fval, block_sums, bytes;
 };
 
 // n entries to sort, m rows (or the most there can be), coo: coordinate-form result of at most `outs` entries,
@@ -963,8 +963,9 @@ RwLayout make_rw_layout(const spws_plan_s* p, int64_t n, int64_t m, bool coo, in
     auto take = [&](size_t bytes) { size_t at = o; o = align256(o + bytes); return at; };
     R.kA = take(8 * (size_t)n);
     R.kB = take(8 * (size_t)n);
-    R.pA = take(8 * (size_t)n);
-    R.pB = take(8 * (size_t)n);
+    R.entry[0] = take(4 * (size_t)n);
+    R.entry[1] = take(4 * (size_t)n);
+    R.pick = take(4 * (size_t)n);
     R.sort_tmp = take(rw_sort_bytes(n));
     R.pos = take(8 * ((size_t)m + 1));
     R.crd = take(4 * (size_t)n);
@@ -990,8 +991,9 @@ RowwiseBufs rw_bufs(char* x, const RwLayout& R) {
     RowwiseBufs b{};
     b.kA = reinterpret_cast<u64*>(x + R.kA);
     b.kB = reinterpret_cast<u64*>(x + R.kB);
-    b.pA = reinterpret_cast<u64*>(x + R.pA);
-    b.pB = reinterpret_cast<u64*>(x + R.pB);
+    b.entry[0] = reinterpret_cast<int*>(x + R.entry[0]);
+    b.entry[1] = reinterpret_cast<int*>(x + R.entry[1]);
+    b.pick = reinterpret_cast<int*>(x + R.pick);
     b.sort_tmp = x + R.sort_tmp;
     b.pos = reinterpret_cast<i64*>(x + R.pos);
     b.crd = reinterpret_cast<int*>(x + R.crd);
@@ -1069,8 +1071,8 @@ spws_status_t rw_outer_symbolic(spws_plan_s* plan, const Shapes& S, spws_tensor_
     if (scratch_bytes < w.L.fixed_end) return SPWS_SCRATCH_TOO_SMALL;
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, w.L);
     plan->in_flight = true;
-    CUDA_TRY(cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream));
     mark_start(plan, 0);
+    CUDA_TRY(launch_rw_clear(c, S.nnzA, sc + w.L.extra + w.R.sort_tmp));
     CUDA_TRY(launch_rw_outer(c, S.A, S.nnzA, S.B, S.nnzB, label_bits_of(S.m, 1), rw_bufs(sc + w.L.extra, w.R)));
     spws_status_t st = rows_symbolic(plan, w.S, w.L, c, scratch_bytes, needed, false, nullptr, nullptr, LL(C->pos[1]), sc);
     if (st != SPWS_OK || (st = rows_collect(plan)) != SPWS_OK) return st;
@@ -1366,8 +1368,8 @@ spws_status_t rw_higher_symbolic(spws_plan_s* plan, const HShapes& H, int64_t P,
     LaunchCtx c = make_ctx(plan, sc, scratch_bytes, w.L);
     char* x = sc + w.L.extra;
     plan->in_flight = true;
-    CUDA_TRY(cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream));
     mark_start(plan, 0);
+    CUDA_TRY(launch_rw_clear(c, H.B.nnz, x + w.R.sort_tmp));
     if (H.form == 2)
         CUDA_TRY(launch_rw_fibre_rows(c, false, H.B, H.C, H.D, reinterpret_cast<int*>(x + w.R.fcnt), reinterpret_cast<i64*>(x + w.R.fpos),
                                       reinterpret_cast<int*>(x + w.R.fcrd), nullptr, reinterpret_cast<i64*>(x + w.R.block_sums)));
