@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(OT) rw_fibre_rows_kernel(Csf3Dev B, Csr C, Csr
 // the tile before ended.  Bound by HBM and the four barriers of a tile.
 // 43e6 entries of three coordinates: 333 us for three arrays with a search per entry and 883 us to interleave
 // them; interleaved 276 us with two searches per tile, 198 us without them and 165 us with whole lines per store
-// (516 MB out, 172 MB in).
+// (516 MB out, 172 MB in).  As many blocks as are resident, a run of tiles each: 139 us, with 16 an SM 164.
 constexpr int RC_ITEMS = 8;
 constexpr int RC_TILE = OT * RC_ITEMS;
 
@@ -468,10 +468,13 @@ cudaError_t launch_rw_fibre_rows(const LaunchCtx& c, bool values, const Csf3Dev&
 cudaError_t launch_rw_coords(const LaunchCtx& c, int order, const i64* rowptr, const u64* row_key, i64 m, i64 nnz, u64 d, const int* cols, int* o0,
                              int* o1, int* o2, bool interleaved) {
     if (nnz == 0) return cudaSuccess;
-    const int grid = grid_for(c, nnz, RC_TILE);
     auto k = order == 3 ? (interleaved ? rw_coords_kernel<3, true> : rw_coords_kernel<3, false>)
                         : (interleaved ? rw_coords_kernel<2, true> : rw_coords_kernel<2, false>);
-    k<<<grid, OT, 0, c.stream>>>(rowptr, row_key, m, nnz, d, cols, o0, o1, o2);
+    int per_sm = 0;
+    const cudaError_t e = resident_blocks((const void*)k, OT, 0, &per_sm);
+    if (e != cudaSuccess) return e;
+    const i64 grid = std::min((nnz + RC_TILE - 1) / RC_TILE, (i64)c.sm_count * std::max(per_sm, 1));
+    k<<<(int)grid, OT, 0, c.stream>>>(rowptr, row_key, m, nnz, d, cols, o0, o1, o2);
     ++c.launches;
     return cudaGetLastError();
 }

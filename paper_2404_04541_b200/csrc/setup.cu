@@ -447,11 +447,6 @@ cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i6
     if (A.nrows == 0) return clear_ctl ? cudaMemsetAsync(c.ctl, 0, sizeof(DevCtl), c.stream) : cudaSuccess;
     const double avg = (double)nnzA / (double)A.nrows;
     const int threads = 256;
-    auto grid_for = [&](int G) {
-        i64 want = ((i64)A.nrows * G + threads - 1) / threads;
-        i64 cap = (i64)c.sm_count * 16;
-        return (int)(want < cap ? want : cap);
-    };
     if (c.brow) {
         i64 want = ((i64)B.nrows + threads - 1) / threads;
         i64 cap = (i64)c.sm_count * 8;
@@ -462,7 +457,15 @@ cudaError_t launch_row_bounds(const LaunchCtx& c, const Csr& A, const Csr& B, i6
         if (e != cudaSuccess) return e;
     }
     cudaError_t e = cudaSuccess;
-    auto launch = [&](auto kernel, int G) { e = launch_chained(c, kernel, grid_for(G), threads, 0, A, B, c.tab, c.prm, c.ctl, c.brow); };
+    // as many blocks as are resident at once: a block's start and its totals cost as much as several of its rows (with 16 blocks an
+    // SM, of which five are resident: 2e6 rows of one entry 35 -> 28 us, 1.6e5 of 9 33 -> 25, a stencil of 2^18 rows 48 -> 37,
+    // of 8e4 25 -> 15, power law on 2^18 vertices 87 -> 72)
+    auto launch = [&](auto kernel, int G) {
+        int per_sm = 0;
+        if ((e = resident_blocks((const void*)kernel, threads, 0, &per_sm)) != cudaSuccess) return;
+        const i64 want = ((i64)A.nrows * G + threads - 1) / threads, cap = (i64)c.sm_count * std::max(per_sm, 1);
+        e = launch_chained(c, kernel, std::min(want, cap), threads, 0, A, B, c.tab, c.prm, c.ctl, c.brow);
+    };
     const bool sm = c.brow != nullptr;
     if (avg <= 1.5) sm ? launch(row_bounds_kernel<1, true>, 1) : launch(row_bounds_kernel<1, false>, 1);
     else if (avg <= 3.0) sm ? launch(row_bounds_kernel<2, true>, 2) : launch(row_bounds_kernel<2, false>, 2);
