@@ -754,8 +754,8 @@ cudaError_t launch_bin_rows(const LaunchCtx& c, int m) {
 //   sfp[s] receives the number of survivors before slice s.
 // Replaces a three-launch scan, the routing and the per-class count (five launches; seven for the
 // 3-tensor form).
-// Bound by the chain of its steps below a few tiles (2048 rows: 6 us where the five launches took 13 and their gaps),
-// by HBM beyond (2e6 fibres: 33 us against 56).
+// Bound by the chain of its steps (2048 rows: 6 us where the five launches took 13 and their gaps; 2e6 fibres: 27 us with five
+// blocks an SM, 21 with seven, which hold all 963 tiles at once).
 // ---------------------------------------------------------------------------------------
 constexpr int FR_THREADS = 256;
 constexpr int FR_WARPS = FR_THREADS / 32;
@@ -773,7 +773,7 @@ struct FibreArgs {
 };
 
 template <bool DENSE, bool TTM>
-__global__ void __launch_bounds__(FR_THREADS, DENSE ? 3 : 5) finish_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, HostBlock* host, int seq, u64* look,
+__global__ void __launch_bounds__(FR_THREADS, DENSE ? 3 : 7) finish_rows_kernel(int m, RowTables tab, ClassParams prm, DevCtl* ctl, HostBlock* host, int seq, u64* look,
                                                                  i64* __restrict__ rowptr, FibreArgs f) {
     __shared__ int s_tile, s_slice0;
     __shared__ i64 s_sum[FR_WARPS], s_before[2];
