@@ -21,8 +21,8 @@ enum RowClass : int {
     CLS_ISM_SMEM_S = 6, // insert-sort-merge of 129 .. 256 products, one warp per row
     CLS_ISM_SMEM = 7,   // insert-sort-merge in shared memory, full CTA
     CLS_DENSE_WARP = 8, // dense workspace (occupancy bitmap), one warp per row
-    CLS_DENSE_HUB = 9,  // dense workspace, one CTA per row, heaviest rows (scheduled first)
-    CLS_DENSE_CTA = 10, // dense workspace, one CTA per row
+    CLS_DENSE_HUB = 9,  // dense workspace, CTA units, rows of at least DENSE_HUB_UB products (told apart in the statistics)
+    CLS_DENSE_CTA = 10, // dense workspace, CTA units
     CLS_ISM_GLOBAL = 11,    // accumulation array in shared memory, all array in global memory
     CLS_HASH_S = 12,    // hash table in shared memory (reduction at insert time), small CTA
     CLS_HASH = 13,      // hash table in shared memory, full CTA
@@ -51,7 +51,7 @@ constexpr int DENSE_WARP_ACC = 256;        // outputs a warp-per-row numeric wor
 constexpr int DENSE_WARP_ACC2 = 1024;      // ... and the larger one that `auto` gives rows of more outputs
 constexpr int N_WARP_LISTS = 2;            // rows of the warp numeric kernel by those capacities
 constexpr int DENSE_WARP_MAX_UB = 4096;    // products a single warp is given at most
-constexpr i64 DENSE_HUB_UB = 1ll << 17;    // rows with at least this many products are scheduled first
+constexpr i64 DENSE_HUB_UB = 1ll << 17;    // products from which a row counts as a hub
 constexpr int DENSE_MAX_SPAN_WORDS = 16384;// 2^19 columns: the widest bitmap (8 bytes per word with its rank) one CTA holds
 // Word lists of long B rows (symbolic pass of the CTA dense route): a B row with at least
 // BW_MIN_LEN entries whose entries share bitmap words is also kept as (word index, bits) pairs,
@@ -430,6 +430,8 @@ struct LaunchCtx {
     int seq;                 // ... as publication `seq` (class sizes) and `seq` + 1 (row pointer)
     u64* look;               // one word per tile of the kernels that hand running sums on ...
     int n_look;              // ... cleared by the binning kernel
+    i64 unit_nnz;            // numeric: outputs of a dense CTA unit's row on average, shared out among its units ...
+    i64 b_bytes;             // ... and coordinates and values of B
     i64 max_ub_smem;         // largest product count of a CLS_ISM_SMEM row when known (0: unknown)
     const i64* class_rows;   // rows per class, once they are binned
     uint2* bw;               // word lists of long B rows, indexed like B's entries (null: not built)

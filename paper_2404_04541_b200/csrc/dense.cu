@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_sym_warp_kernel(DevCtl* __re
 // entries of a row walked a chain of four loads per batch and had one B row's loads in flight; the entries of a round are
 // now looked up by all threads at once and the warps pull tiles of the stream of their elements, each with 128 loads in flight
 // whatever the length of the B rows.  Power law on 16381 / 60000 / 2^18 vertices: 201 / 622 / 2681 us by batches, one block a
-// row, 78 / 415 / 2621 us now.
+// row, 80 / 418 / 2600 us now.
 // ---------------------------------------------------------------------------------------
 constexpr int DS_ENTRIES = DC_THREADS;      // A entries whose descriptors are staged per round
 // elements a warp takes per fetch: a 64th of the round's, so that the warps finish together (at most 1024 / 2048 / 4096: power law on
@@ -643,7 +643,7 @@ __global__ void __launch_bounds__(DW_THREADS) dense_num_warp_kernel(DevCtl* __re
 // in shared memory; outputs beyond accumulate straight into the row's value segment in global
 // memory (zeroed beforehand), which keeps any row to a single pass whatever its output count.
 // Bound by latency: the ranks and the compare-and-swap loops of the shared-memory additions form chains, at 32 warps
-// per SM (64 registers, 111 KB).  Power law on 2^18 / 16381 vertices, f64 / f32: with nine barriers per unit,
+// per SM (64 registers; two blocks of 512 threads, or four of 256, see the launch).  By blocks of 512, power law on 2^18 / 16381 vertices, f64 / f32: with nine barriers per unit,
 // metadata fetched between them and loads one step ahead 14050 / 309 us; without the prefetch (its register copies
 // cost more than the other warps' work hides) and with two steps to find a tile's entry 13590 / 287 us; with three barriers and the next unit
 // fetched meanwhile 12770 / 252 us.  Every output in shared memory, by segments of a row's ranks: 28000 / 339 us.
@@ -1123,10 +1123,15 @@ static cudaError_t num_cta_t(const LaunchCtx& c, int phase, int n_units_host, in
     // so less than two of 512, where four find room (with fewer outputs in shared memory if need be: a reduction in global memory
     // costs about the same) and the units are enough for all of them.  Accumulation, 512 / 256 threads: power law on 16381
     // (f32) / 60000 (f64) / 100003 (f32) vertices 229 / 191, 1780 / 1580, 1795 / 1540 us; 10^4 rows of 10^4 products, f64, 419 / 356.
-    // With few units 512: power law on 1500 / 4001 vertices, f32, units of 2^13, 18 / 23 and 33 / 38.
+    // With few units 512: power law on 1500 / 4001 vertices, f32, units of 2^13, 18 / 23 and 33 / 38.  Nor where the values that the
+    // blocks of a full grid add into and B together outgrow what a half of L2 keeps, which they read and write back from memory
+    // then (the second column: MB of both): f64, degree 16, 8e4 vertices 46: 3270 / 3145 us, 1e5 52: 4001 / 4211, 131072 55: 4589 / 5761 (DRAM
+    // traffic 6.4 / 13.7 GB); 150000, degree 8, 47: 3187 / 3034, degree 12 63: 5564 / 7548; f32, 180000 48: 8074 / 7715.
+    constexpr i64 LIVE_BYTES = 49ll << 20;
+    const i64 live = 4ll * c.sm_count * c.unit_nnz * (i64)sizeof(T) + c.b_bytes;
     int CAP = c.prm.unit_outputs, per_sm = 0;
     auto quarter = dense_num_cta_kernel<T, CEIL, DN_THREADS_4>;
-    if (n_units_host < 0 || n_units_host > 8 * c.sm_count)
+    if (n_units_host > 8 * c.sm_count && live <= LIVE_BYTES)
         for (int cap = CAP; cap >= std::min(CAP, DN_CAP_LEAST); cap >>= 1) {
             const size_t smem = smem_of(cap, dn_entries<DN_THREADS_4>());
             if (4 * (smem + 2048) > 228 * 1024) continue;

@@ -804,6 +804,11 @@ spws_status_t rows_collect(spws_plan_s* plan) {
     return SPWS_OK;
 }
 
+// Outputs of the dense rows that CTA units take.
+int64_t dense_cta_nnz(const spws_stats_t& s) {
+    return s.nnz_per_class[public_class(CLS_DENSE_WARP)] + s.nnz_per_class[public_class(CLS_DENSE_HUB)] + s.nnz_per_class[public_class(CLS_DENSE_CTA)] - s.dense_warp_nnz;
+}
+
 spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, char* sc, size_t scratch_bytes, const i64* rowptr, int* crd, void* val) {
     plan->in_flight = true;
     use_order(plan, c, sc, scratch_bytes);
@@ -815,6 +820,8 @@ spws_status_t rows_numeric(spws_plan_s* plan, const Shapes& S, LaunchCtx& c, cha
         CUDA_TRY(cudaMemsetAsync(c.ctl->work_counter, 0, sizeof(c.ctl->work_counter), c.stream));
     plan->counters_clear = false;
     c.max_ub_smem = plan->max_ub_smem;
+    c.unit_nnz = plan->stats.dense_units > 0 ? dense_cta_nnz(plan->stats) / plan->stats.dense_units : 0;
+    c.b_bytes = S.nnzB * (4 + (plan->is_f64 ? 8 : 4));
     c.n_ranked = plan->numeric_behind ? 0 : plan->n_ranked;
     const spws_stats_t& s = plan->stats;
     const int64_t* bins = plan->bin_rows;
@@ -1885,6 +1892,8 @@ spws_status_t spws_gather_ceiling(spws_plan_t plan, const spws_tensor_t* A, cons
     CUDA_TRY(cudaMemsetAsync(value_sum, 0, sizeof(double), c.stream));
     mark_start(plan, 2);
     const spws_stats_t& s = plan->stats;
+    c.unit_nnz = s.dense_units > 0 ? dense_cta_nnz(s) / s.dense_units : 0;
+    c.b_bytes = S.nnzB * (4 + (plan->is_f64 ? 8 : 4));
     u64* ci = reinterpret_cast<u64*>(index_sum);
     if (s.dense_warp_rows > 0) {
         CUDA_TRY(launch_dense_num_warp(c, plan->n_warp, plan->max_warp_cnt, (int)S.m, plan->max_span_words, S.A, S.B, rowptr, nullptr, nullptr, ci, value_sum));
