@@ -251,7 +251,7 @@ __device__ __forceinline__ int padded(int i) { return i + (i >> 5); }
 // What the counting pass keeps of a row whose outputs are at most half of its products and whose B rows fill a warp, instead of the
 // sorted words: the distinct columns, then every product's place among them (16 bits, loop order).  The numeric pass adds one
 // B row after the other, whose products go to different outputs, and reads no columns.
-constexpr i64 ORDER_RANKS = 1ll << 62;                  // flag above the offset of such a row
+constexpr i64 ORDER_RANKS = 1ll << 61;                  // flag above the offset of such a row (no flag of a dense row's)
 
 // Sorts the row's packed words and counts its distinct columns; numeric: leaves the sorted words in `packed`
 // and the places of the run heads in `heads`.  `order` (may be null): numeric: the words as sorted before;
@@ -700,8 +700,9 @@ __global__ void __launch_bounds__(IW_WARPS * 32, sizeof(T) == 8 ? 10 : 12) ism_r
     if (r >= n_rows) return;
     const int row = __ldg(rows + r);
     const i64 off = __ldg(order_off + row);
-    if (off < 0 || !(off & ORDER_RANKS)) return;        // ism_warp_kernel's row
     const int products = (int)__ldg(ub + row);
+    // (ism_warp_kernel's row; a CTA's, of which nothing has written order_off: at most a class's 4096 products)
+    if (products > ISM_WARP_MAX || off < 0 || !(off & ORDER_RANKS)) return;
     const i64 ps = __ldg(A.pos + row), pe = __ldg(A.pos + row + 1), out0 = __ldg(rowptr + row);
     const int n = min((int)(__ldg(rowptr + row + 1) - out0), most);
     const unsigned* __restrict__ cols = reinterpret_cast<const unsigned*>(order_arena + (off & ~ORDER_RANKS));
