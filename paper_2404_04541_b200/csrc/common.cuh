@@ -543,7 +543,8 @@ size_t rw_sort_bytes(i64 n);
 // (first of all: clears the control block and the temporaries of a sort of n entries)
 cudaError_t launch_rw_clear(const LaunchCtx& c, i64 n, char* sort_tmp);
 cudaError_t launch_rw_outer(const LaunchCtx& c, const Csr& At, i64 n, const Csr& B, i64 nnzB, int bits, const RowwiseBufs& b);
-cudaError_t launch_rw_csf(const LaunchCtx& c, int form, const Csf3Dev& B, u64 d, i64 m, int bits, const RowwiseBufs& b);
+// d0, d1: extents of the coordinates of a label
+cudaError_t launch_rw_csf(const LaunchCtx& c, int form, const Csf3Dev& B, u64 d0, u64 d1, i64 m, int bits, const RowwiseBufs& b);
 cudaError_t launch_rw_values(const LaunchCtx& c, const void* val, const int* src, i64 n, void* out);
 cudaError_t launch_rw_fibre_rows(const LaunchCtx& c, bool values, const Csf3Dev& B, const Csr& C, const Csr& D, int* cnt, i64* fpos, int* fcrd,
                                  void* fval, i64* block_sums);

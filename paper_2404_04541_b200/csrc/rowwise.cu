@@ -82,13 +82,15 @@ __global__ void __launch_bounds__(OT) rw_keys_outer_kernel(Csr At, i64 n, Csr B,
     if (bad) raise_status(ctl, DEV_NONCANONICAL);
 }
 
-// form: 0 SpTTM, 1 SpTTM-I, 2 SpMTTKRP.  `d` = extent of the label's inner coordinate (forms 0, 1).
+// form: 0 SpTTM, 1 SpTTM-I, 2 SpMTTKRP.  Label: a * d1 + b of coordinates below d0 and d1 (forms 0, 1), a alone (form 2), which are
+// checked on the way: a label cut to 32 bits would be another row's.
 // pos[0 .. m] := nnz on the way (rw_sparse_rows_kernel writes the rows there are).
 template <typename K>
-__global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u64 d, K* __restrict__ keys, int* __restrict__ picks, int passes,
-                                                         SortHead* head, i64* __restrict__ pos, i64 m) {
+__global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u64 d0, u64 d1, K* __restrict__ keys, int* __restrict__ picks, int passes,
+                                                         SortHead* head, i64* __restrict__ pos, i64 m, DevCtl* ctl) {
     __shared__ int s_f[2], s_s[2];
     __shared__ DigitCounts s_digits;
+    bool bad = false;
     chained_start();
     not_before(B.pos1);
     not_before(B.pos2);
@@ -115,8 +117,12 @@ __global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u6
             if (form != 2) {
                 const u64 c1 = (u64)(unsigned)__ldg(B.crd1 + f);
                 const u64 c0 = (u64)(unsigned)__ldg(B.crd0 + owner_row(B.pos1, s_s[0], s_s[1] + 1, f));
-                key = (form == 0 ? c1 : c0) * d + c2;
+                const u64 a = form == 0 ? c1 : c0;
+                key = a * d1 + c2;
                 pick = form == 0 ? c0 : c1;
+                bad |= a >= d0 || c2 >= d1;
+            } else {
+                bad |= c2 >= d0;
             }
             keys[e] = (K)key;
             s_digits.add(key, passes);
@@ -124,6 +130,7 @@ __global__ void __launch_bounds__(OT) rw_keys_csf_kernel(int form, Csf3Dev B, u6
         }
     }
     s_digits.flush(passes, head);
+    if (bad) raise_status(ctl, DEV_NONCANONICAL);
 }
 
 // CSR result: the reordered operand has one row per output row; pos by binary search in the sorted labels.
@@ -427,14 +434,14 @@ cudaError_t launch_rw_outer(const LaunchCtx& c, const Csr& At, i64 n, const Csr&
 }
 
 template <typename K>
-static cudaError_t rw_csf_t(const LaunchCtx& c, int form, const Csf3Dev& B, u64 d, i64 m, int bits, const RowwiseBufs& b) {
-    const cudaError_t e = launch_chained(c, rw_keys_csf_kernel<K>, grid_for(c, std::max(B.nnz, (i64)1), RK_TILE), OT, 0, form, B, d, reinterpret_cast<K*>(b.kA), b.pick,
-                                         passes_of(bits), reinterpret_cast<SortHead*>(b.sort_tmp), b.pos, m);
+static cudaError_t rw_csf_t(const LaunchCtx& c, int form, const Csf3Dev& B, u64 d0, u64 d1, i64 m, int bits, const RowwiseBufs& b) {
+    const cudaError_t e = launch_chained(c, rw_keys_csf_kernel<K>, grid_for(c, std::max(B.nnz, (i64)1), RK_TILE), OT, 0, form, B, d0, d1, reinterpret_cast<K*>(b.kA), b.pick,
+                                         passes_of(bits), reinterpret_cast<SortHead*>(b.sort_tmp), b.pos, m, c.ctl);
     return e != cudaSuccess ? e : rw_reorder<K>(c, B.nnz, m, bits, true, b);
 }
 
-cudaError_t launch_rw_csf(const LaunchCtx& c, int form, const Csf3Dev& B, u64 d, i64 m, int bits, const RowwiseBufs& b) {
-    return bits <= 32 ? rw_csf_t<unsigned>(c, form, B, d, m, bits, b) : rw_csf_t<u64>(c, form, B, d, m, bits, b);
+cudaError_t launch_rw_csf(const LaunchCtx& c, int form, const Csf3Dev& B, u64 d0, u64 d1, i64 m, int bits, const RowwiseBufs& b) {
+    return bits <= 32 ? rw_csf_t<unsigned>(c, form, B, d0, d1, m, bits, b) : rw_csf_t<u64>(c, form, B, d0, d1, m, bits, b);
 }
 
 cudaError_t launch_rw_values(const LaunchCtx& c, const void* val, const int* src, i64 n, void* out) {

@@ -1380,7 +1380,7 @@ spws_status_t rw_higher_symbolic(spws_plan_s* plan, const HShapes& H, int64_t P,
     if (H.form == 2)
         CUDA_TRY(launch_rw_fibre_rows(c, false, H.B, H.C, H.D, reinterpret_cast<int*>(x + w.R.fcnt), reinterpret_cast<i64*>(x + w.R.fpos),
                                       reinterpret_cast<int*>(x + w.R.fcrd), nullptr, reinterpret_cast<i64*>(x + w.R.block_sums)));
-    CUDA_TRY(launch_rw_csf(c, H.form, H.B, (u64)(H.order == 3 ? H.odims[1] : 1), w.m, w.bits, rw_bufs(x, w.R)));
+    CUDA_TRY(launch_rw_csf(c, H.form, H.B, (u64)H.odims[0], (u64)(H.order == 3 ? H.odims[1] : 1), w.m, w.bits, rw_bufs(x, w.R)));
     spws_status_t st = rows_symbolic(plan, w.S, w.L, c, scratch_bytes, needed, false, nullptr, nullptr, reinterpret_cast<i64*>(x + w.R.rowptr), sc);
     if (st != SPWS_OK || (st = rows_collect(plan)) != SPWS_OK) return st;
     plan->stats.rows = H.B.nnz;
