@@ -28,13 +28,13 @@ __device__ __forceinline__ int owner_row(const i64* __restrict__ pos, int lo, in
 }
 
 // The same by a whole warp, 32 probes a step: a block looks for the owners of its tile among all rows first (the keys of 1e6 entries
-// in 5e5 fibres 31 us by halves, 27 us like this; of 7e5 in 5e4 rows 23 and 18).
+// in 5e5 fibres 31 us by halves, 27 us like this; of 7e5 in 5e4 rows 23 and 18).  Inside [lo, hi) whatever the offsets, as by halves.
 __device__ __forceinline__ int owner_row_warp(const i64* __restrict__ pos, int lo, int hi, i64 p) {
     const int lane = threadIdx.x & 31;
     while (hi - lo > 1) {
         const int step = (int)(((unsigned)(hi - lo) + 31u) >> 5);
         const i64 at = lo + (i64)lane * step;
-        const int n = __popc(__ballot_sync(0xffffffffu, at < hi && __ldg(pos + at) <= p));       // (one at least)
+        const int n = max(__popc(__ballot_sync(0xffffffffu, at < hi && __ldg(pos + at) <= p)), 1);
         hi = (int)min((i64)hi, lo + (i64)n * step);
         lo += (n - 1) * step;
     }
