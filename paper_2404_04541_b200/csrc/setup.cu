@@ -1053,6 +1053,7 @@ __global__ void __launch_bounds__(FR_THREADS) finish_slices_kernel(int n_i, cons
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tiles = gridDim.x;
     chained_start();
+    not_before(sfp);
     if (tid == 0) s_tile = atomicAdd(&ctl->slices_ticket, 1);
     __syncthreads();
     const int tile = s_tile;

@@ -97,3 +97,22 @@ def test_no_device_is_reported_not_faked(binding):
     from paper_2404_04541_b200 import api
     with pytest.raises(RuntimeError):
         api.Context()
+
+
+def test_chained_kernels_load_nothing_read_only_before_their_wait():
+    """A kernel whose blocks are placed before the kernel ahead of it is done may not load through a read-only pointer at an address
+    that it knows on entry, unless the pointer has passed not_before()."""
+    folder = os.path.join(ROOT, "paper_2404_04541_b200", "csrc")
+    seen = 0
+    for name in sorted(os.listdir(folder)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(folder, name)).read())
+        for m in re.finditer(r"__global__[^;{]*?(\w+_kernel)\(([^{;]*)\)\s*\{(.*?)\n\}", text, flags=re.S):
+            kernel, params, body = m.groups()
+            if "chained_start(" not in body:
+                continue
+            seen += 1
+            known = {re.search(r"(\w+)\s*$", p).group(1) for p in params.split(",")}
+            for pointer in re.findall(r"const \w+\* __restrict__ (\w+)", params):
+                for at in re.findall(r"\b%s(?:\[| \+ )\s*(\w+)" % pointer, body):
+                    assert at not in known and not at.isdigit() or f"not_before({pointer})" in body, (kernel, pointer, at)
+    assert seen >= 12
