@@ -167,9 +167,11 @@ __global__ void __launch_bounds__(THREADS) ism_smem_kernel(const int* __restrict
 // on the stencil (372 since; numeric 370, 309 since), 210 -> 172 us on the rows of 470; 143-product rows (3e4): 44 -> 36
 // and 55 -> 49 us.
 //   Where outputs are at most half of the products and B rows fill a warp, the counting pass leaves the places of the products
-// among the outputs and ism_rank_kernel adds: stencil 41 x 37 x 53, f32, count 374 -> 400 us, numeric 309 -> 147 (of it 11 for
-// the rows at its edges); 40^3, f64, 300 -> 321 and 296 -> 148.  Not with words of 64 bits, whose counting kernel would slow
-// down (60000 rows of 600 products, f64: 881 -> 895 us).  A hash set of the columns before the sort instead: 348 us, and 786 for
+// among the outputs and ism_rank_kernel adds: stencil 41 x 37 x 53, f32, count 374 -> 400 us, numeric 309 -> 135 (of it 11 for
+// the rows at its edges); 40^3, f64, 300 -> 321 and 296 -> 138.  Not with words of 64 bits, whose counting kernel would slow
+// down (60000 rows of 600 products, f64: 881 -> 895 us).  The line at half of the products: 40000 rows of 18 B rows of 32, f32, a call at 2 products an output, where
+// few rows rank, 438 -> 443, at 2.1 436 -> 408, at 3 426 -> 340; of 35 B rows of 17 (a step of the adding kernel fills half a warp) 538 -> 529, 530 -> 477, 519 -> 404; of
+// 10 of 64, f64, at 2 466 -> 473.  A hash set of the columns before the sort instead: 348 us, and 786 for
 // a numeric pass that looks its products up in it.
 // ---------------------------------------------------------------------------------------
 constexpr int IW_WARPS = 4;
@@ -679,7 +681,8 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
 // Numeric pass of the rows whose products' places the counting pass has kept: a warp per row, its lanes across one B row after the
 // other, so that no two lanes add into one output and every output is summed in loop order.  Bound by the chains of loads that lead
 // to a row's B rows: a block for every four rows, four B rows in flight, and shared memory for the outputs alone, so that 40 .. 48
-// warps are on an SM (as a path of ism_warp_kernel, at 28 warps, two B rows in flight 246 us, four 211).
+// warps are on an SM (as a path of ism_warp_kernel, at 28 warps, two B rows in flight 246 us, four 211).  Where few rows of the class
+// have kept places, a warp looks at `step` rows side by side.
 // ---------------------------------------------------------------------------------------
 // start of the B row and its length, place of the entry's first product, A value
 template <typename T> struct __align__(16) RankEntry { u64 row; T a; int at; };
@@ -688,7 +691,7 @@ template <typename T>
 __global__ void __launch_bounds__(IW_WARPS * 32, sizeof(T) == 8 ? 10 : 12) ism_rank_kernel(const int* __restrict__ rows, int n_rows, const DevCtl* __restrict__ ctl, Csr A, Csr B,
                                                                                           const i64* __restrict__ ub, const i64* __restrict__ order_off,
                                                                                           const char* __restrict__ order_arena, const i64* __restrict__ rowptr,
-                                                                                          int* __restrict__ Ccrd, T* __restrict__ Cval, int most) {
+                                                                                          int* __restrict__ Ccrd, T* __restrict__ Cval, int most, int step) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (ctl->status != 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -696,67 +699,75 @@ __global__ void __launch_bounds__(IW_WARPS * 32, sizeof(T) == 8 ? 10 : 12) ism_r
     T* const vals = reinterpret_cast<T*>(smem_raw + sizeof(RankEntry<T>) * 32 * IW_WARPS) + warp * most;
     const T* __restrict__ Aval = (const T*)A.val;
     const T* __restrict__ Bval = (const T*)B.val;
-    const int r = blockIdx.x * IW_WARPS + warp;
-    if (r >= n_rows) return;
-    const int row = __ldg(rows + r);
-    const i64 off = __ldg(order_off + row);
-    const int products = (int)__ldg(ub + row);
-    // (ism_warp_kernel's row; a CTA's, of which nothing has written order_off: at most a class's 4096 products)
-    if (products > ISM_WARP_MAX || off < 0 || !(off & ORDER_RANKS)) return;
-    const i64 ps = __ldg(A.pos + row), pe = __ldg(A.pos + row + 1), out0 = __ldg(rowptr + row);
-    const int n = min((int)(__ldg(rowptr + row + 1) - out0), most);
-    const unsigned* __restrict__ cols = reinterpret_cast<const unsigned*>(order_arena + (off & ~ORDER_RANKS));
-    const unsigned short* __restrict__ place = reinterpret_cast<const unsigned short*>(cols + n);
-    for (int x = lane; x < n; x += 32) {
-        Ccrd[out0 + x] = (int)__ldg(cols + x);
-        vals[x] = (T)-0.0;                              // (the sum of nothing that leaves the sign of a first zero)
+    const i64 r = (i64)(blockIdx.x * IW_WARPS + warp) * step + lane;
+    int my_row = 0, my_products = 0;
+    i64 my_off = -1;
+    if (lane < step && r < n_rows) {
+        my_row = __ldg(rows + r);
+        my_off = __ldg(order_off + my_row);
+        my_products = (int)__ldg(ub + my_row);
     }
-    int total = 0;
-    for (i64 p0 = ps; p0 < pe; p0 += 32) {
-        RankEntry<T> mine;
-        mine.row = 0;
-        mine.a = 0;
-        if (p0 + lane < pe) {
-            const int k = __ldg(A.crd + p0 + lane);
-            mine.a = __ldg(Aval + p0 + lane);
-            if ((unsigned)k < (unsigned)B.nrows) {
-                const i64 qs = __ldg(B.pos + k);
-                mine.row = (u64)qs << 16 | (u64)min(__ldg(B.pos + k + 1) - qs, (i64)products);
-            }
+    // (others are ism_warp_kernel's rows, or a CTA's, of which nothing has written order_off: at most a class's 4096 products)
+    for (unsigned todo = __ballot_sync(0xffffffffu, my_products <= ISM_WARP_MAX && my_off >= 0 && (my_off & ORDER_RANKS)); todo; todo &= todo - 1) {
+        const int src = __ffs(todo) - 1;
+        const int row = __shfl_sync(0xffffffffu, my_row, src), products = __shfl_sync(0xffffffffu, my_products, src);
+        const i64 off = __shfl_sync(0xffffffffu, my_off, src);
+        const i64 ps = __ldg(A.pos + row), pe = __ldg(A.pos + row + 1), out0 = __ldg(rowptr + row);
+        const int n = min((int)(__ldg(rowptr + row + 1) - out0), most);
+        const unsigned* __restrict__ cols = reinterpret_cast<const unsigned*>(order_arena + (off & ~ORDER_RANKS));
+        const unsigned short* __restrict__ place = reinterpret_cast<const unsigned short*>(cols + n);
+        for (int x = lane; x < n; x += 32) {
+            Ccrd[out0 + x] = (int)__ldg(cols + x);
+            vals[x] = (T)-0.0;                              // (the sum of nothing that leaves the sign of a first zero)
         }
-        const int len = (int)(mine.row & 0xffffu), incl = warp_incl_scan(len);
-        mine.at = min(total + incl - len, products - len);          // (the lengths add up to the products)
-        __syncwarp();
-        entry[lane] = mine;
-        __syncwarp();
-        const bool longer = __any_sync(0xffffffffu, len > 32);
-        const int nE = (int)min((i64)32, pe - p0);
-        for (int e = 0; e < nE; e += 4) {               // (length 0 past the last entry)
-            T v[4];
-            int x[4];
-#pragma unroll
-            for (int y = 0; y < 4; ++y) {
-                const RankEntry<T> d = entry[e + y];
-                x[y] = -1;
-                v[y] = 0;
-                if (lane < (int)(d.row & 0xffffu)) { x[y] = __ldg(place + d.at + lane); v[y] = mul_rn(d.a, __ldg(Bval + (d.row >> 16) + lane)); }
-            }
-#pragma unroll
-            for (int y = 0; y < 4; ++y) {
-                if (x[y] >= 0) vals[x[y]] = add_rn(vals[x[y]], v[y]);
-                if (longer) {
-                    const RankEntry<T> d = entry[e + y];
-                    for (int t = 32 + lane; t < (int)(d.row & 0xffffu); t += 32) {
-                        const int z = __ldg(place + d.at + t);
-                        vals[z] = add_rn(vals[z], mul_rn(d.a, __ldg(Bval + (d.row >> 16) + t)));
-                    }
+        int total = 0;
+        for (i64 p0 = ps; p0 < pe; p0 += 32) {
+            RankEntry<T> mine;
+            mine.row = 0;
+            mine.a = 0;
+            if (p0 + lane < pe) {
+                const int k = __ldg(A.crd + p0 + lane);
+                mine.a = __ldg(Aval + p0 + lane);
+                if ((unsigned)k < (unsigned)B.nrows) {
+                    const i64 qs = __ldg(B.pos + k);
+                    mine.row = (u64)qs << 16 | (u64)min(__ldg(B.pos + k + 1) - qs, (i64)products);
                 }
-                __syncwarp();
             }
+            const int len = (int)(mine.row & 0xffffu), incl = warp_incl_scan(len);
+            mine.at = min(total + incl - len, products - len);          // (the lengths add up to the products)
+            __syncwarp();
+            entry[lane] = mine;
+            __syncwarp();
+            const bool longer = __any_sync(0xffffffffu, len > 32);
+            const int nE = (int)min((i64)32, pe - p0);
+            for (int e = 0; e < nE; e += 4) {               // (length 0 past the last entry)
+                T v[4];
+                int x[4];
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                    const RankEntry<T> d = entry[e + y];
+                    x[y] = -1;
+                    v[y] = 0;
+                    if (lane < (int)(d.row & 0xffffu)) { x[y] = __ldg(place + d.at + lane); v[y] = mul_rn(d.a, __ldg(Bval + (d.row >> 16) + lane)); }
+                }
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                    if (x[y] >= 0) vals[x[y]] = add_rn(vals[x[y]], v[y]);
+                    if (longer) {
+                        const RankEntry<T> d = entry[e + y];
+                        for (int t = 32 + lane; t < (int)(d.row & 0xffffu); t += 32) {
+                            const int z = __ldg(place + d.at + t);
+                            vals[z] = add_rn(vals[z], mul_rn(d.a, __ldg(Bval + (d.row >> 16) + t)));
+                        }
+                    }
+                    __syncwarp();
+                }
+            }
+            total += __shfl_sync(0xffffffffu, incl, 31);
         }
-        total += __shfl_sync(0xffffffffu, incl, 31);
+        for (int x = lane; x < n; x += 32) Cval[out0 + x] = vals[x];
+        __syncwarp();
     }
-    for (int x = lane; x < n; x += 32) Cval[out0 + x] = vals[x];
 }
 
 template <typename T, typename P, int CAP, int THREADS>
@@ -853,8 +864,11 @@ static cudaError_t launch_t(const LaunchCtx& c, bool numeric, const IsmLaunch& l
         const size_t smem = IW_WARPS * (sizeof(T) * outputs + 32 * sizeof(RankEntry<T>));
         int per_sm = 0;
         if ((e = resident_blocks((const void*)ism_rank_kernel<T>, IW_WARPS * 32, smem, &per_sm)) != cudaSuccess) return e;
-        ism_rank_kernel<T><<<(l.own + IW_WARPS - 1) / IW_WARPS, IW_WARPS * 32, smem, c.stream>>>(l.rows + (l.n - l.own), l.own, c.ctl, A, B, c.tab.ub, c.tab.bm_off, c.order, rowptr,
-                                                                                                Ccrd, (T*)Cval, outputs);
+        // (two rows a warp: 40000 rows of 576 products of which few, of 595 of which a third rank, f32, a call 443.5 and 534 us with one, 443 and 529
+        // with two, 445 and 538 with four, 457 and 534 with up to 32, a warp's ranked rows one after the other; without places 438 and 538)
+        const int step = 2 * c.n_ranked <= l.own ? 2 : 1, rows = IW_WARPS * step;
+        ism_rank_kernel<T><<<(l.own + rows - 1) / rows, IW_WARPS * 32, smem, c.stream>>>(l.rows + (l.n - l.own), l.own, c.ctl, A, B, c.tab.ub, c.tab.bm_off, c.order, rowptr,
+                                                                                        Ccrd, (T*)Cval, outputs, step);
         ++c.launches;
         rest = c.n_ranked < l.own;
         // the rows of smaller classes that go along with these
