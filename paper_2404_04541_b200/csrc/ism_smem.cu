@@ -257,8 +257,9 @@ constexpr i64 ORDER_RANKS = 1ll << 61;                  // flag above the offset
 
 // Sorts the row's packed words and counts its distinct columns; numeric: leaves the sorted words in `packed`
 // and the places of the run heads in `heads`.  `order` (may be null): numeric: the words as sorted before;
-// else receives them, or (*ranks, when the row is of that kind and may_rank) the columns and places.
-template <typename PK, typename P, int E, bool NUMERIC>
+// else receives them, or (*ranks, when the row is of that kind and may_rank) the columns and places.  (Without RANKS at once: words that
+// live across the count of the heads cost the kernel spills.)
+template <typename PK, typename P, int E, bool NUMERIC, bool RANKS>
 __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int total, P* order, bool may_rank, bool* ranks) {
     const int lane = threadIdx.x & 31;
     P w[E];
@@ -273,6 +274,10 @@ __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int to
             w[x] = i < total ? packed[padded(i)] : PK::sentinel();
         }
         warp_sort<P, E>(w);
+        if (!NUMERIC && !RANKS && order && lane < lanes) {
+#pragma unroll
+            for (int x = 0; x < E; ++x) order[x * lanes + lane] = w[x];
+        }
     }
     const P before = __shfl_up_sync(0xffffffffu, w[E - 1], 1);
     unsigned head = 0;
@@ -282,8 +287,10 @@ __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int to
         if (w[x] != PK::sentinel() && first) head |= 1u << x;
     }
     const int mine = __popc(head);
-    const int incl = warp_incl_scan(mine);
-    const int n = __shfl_sync(0xffffffffu, incl, 31);
+    // (where rows may rank the sum alone, before the words are left: with the scan the kernel spills more)
+    constexpr bool SUM = !NUMERIC && RANKS;
+    const int incl = SUM ? 0 : warp_incl_scan(mine);
+    const int n = SUM ? __reduce_add_sync(0xffffffffu, mine) : __shfl_sync(0xffffffffu, incl, 31);
     if (NUMERIC) {
         __syncwarp();
         int at = incl - mine;
@@ -293,12 +300,12 @@ __device__ __forceinline__ int sort_row(P* packed, unsigned short* heads, int to
             if ((head >> x) & 1u) heads[at++] = (unsigned short)(lane * E + x);
         }
         __syncwarp();
-    } else if (order) {
+    } else if (RANKS && order) {
         if (may_rank && 2 * n <= total) {
             __syncwarp();
             unsigned* const cols = reinterpret_cast<unsigned*>(packed);
             unsigned short* const place = reinterpret_cast<unsigned short*>(cols + n);
-            int at = incl - mine - 1;
+            int at = warp_incl_scan(mine) - mine - 1;
 #pragma unroll
             for (int x = 0; x < E; ++x)
                 if (w[x] != PK::sentinel()) {
@@ -639,22 +646,23 @@ __global__ void __launch_bounds__(IW_WARPS * 32, (iw_blocks<T, P, CAP, NUMERIC>(
         if (total != products) order = nullptr;             // (a malformed B row)
         P* const keep = CAP > 256 ? order : nullptr;
         bool ranks = false;
+        if (!NUMERIC && !RANKS && kept && lane == 0) order_off[row] = order ? (i64)(reinterpret_cast<char*>(order) - order_arena) : -1;
         if constexpr (CAP <= 256) {
             switch (e) {
-                case 4: distinct = sort_row<PK, P, 4, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
-                case 6: distinct = sort_row<PK, P, 6, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
-                default: distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
+                case 4: distinct = sort_row<PK, P, 4, NUMERIC, RANKS>(packed, heads, total, keep, gs == 32, &ranks); break;
+                case 6: distinct = sort_row<PK, P, 6, NUMERIC, RANKS>(packed, heads, total, keep, gs == 32, &ranks); break;
+                default: distinct = sort_row<PK, P, 8, NUMERIC, RANKS>(packed, heads, total, keep, gs == 32, &ranks); break;
             }
         } else {
             switch (e) {
-                case 8: distinct = sort_row<PK, P, 8, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
-                case 12: distinct = sort_row<PK, P, 12, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
-                case 16: distinct = sort_row<PK, P, 16, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
-                case 24: distinct = sort_row<PK, P, 24, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
-                default: distinct = sort_row<PK, P, 32, NUMERIC>(packed, heads, total, keep, RANKS && gs == 32, &ranks); break;
+                case 8: distinct = sort_row<PK, P, 8, NUMERIC, RANKS>(packed, heads, total, keep, gs == 32, &ranks); break;
+                case 12: distinct = sort_row<PK, P, 12, NUMERIC, RANKS>(packed, heads, total, keep, gs == 32, &ranks); break;
+                case 16: distinct = sort_row<PK, P, 16, NUMERIC, RANKS>(packed, heads, total, keep, gs == 32, &ranks); break;
+                case 24: distinct = sort_row<PK, P, 24, NUMERIC, RANKS>(packed, heads, total, keep, gs == 32, &ranks); break;
+                default: distinct = sort_row<PK, P, 32, NUMERIC, RANKS>(packed, heads, total, keep, gs == 32, &ranks); break;
             }
         }
-        if (!NUMERIC && kept && lane == 0) order_off[row] = order ? (i64)(reinterpret_cast<char*>(order) - order_arena) | (ranks ? ORDER_RANKS : 0) : -1;
+        if (!NUMERIC && RANKS && kept && lane == 0) order_off[row] = order ? (i64)(reinterpret_cast<char*>(order) - order_arena) | (ranks ? ORDER_RANKS : 0) : -1;
         if (!NUMERIC && RANKS && ranks && lane == 0) atomicAdd(&ctl->n_ranked, 1);
 
         if (AHEAD) fields();
