@@ -120,8 +120,11 @@ __device__ __forceinline__ int slot_words(int lo, int hi) {
 }
 __device__ __forceinline__ bool dense_cls(int cls) { return cls == CLS_DENSE_WARP || cls == CLS_DENSE_HUB || cls == CLS_DENSE_CTA; }
 
-constexpr int LONG_LIST = 32;
-constexpr int MID_LIST = 64;
+// Long and mid rows that a block lists for its threads and warps to take together; what does not fit is left to lane groups, as serial
+// chains.  With four or five blocks an SM (1e5 rows of 60 entries among 1.9e6 of 2: lists of 32 and 64 rows 121 us, these 119; 2e4 rows of
+// 1100 77 and 75; 5e4 147 and 146, where 16 blocks an SM with lists of 32 took 207).
+constexpr int LONG_LIST = 128;
+constexpr int MID_LIST = 256;
 
 // Products and first / last column of the entries ps + at, ps + at + LANES, ..: four entries per step; the totals of
 // a warp's lanes are returned in every lane.
@@ -224,7 +227,7 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
     __shared__ i64 s_cprod[8][NCLASS];
     __shared__ i64 s_max_ub, s_max_ub_global, s_max_ub_smem, s_bm_words;
     __shared__ int s_max_span_words;
-    __shared__ unsigned s_order_words;              // (at most 1024 a row: no block sees 2^22 rows)
+    __shared__ unsigned s_order_words;              // (at most 1024 a row: of 2^31 rows none of 592 blocks, four an SM, sees 2^22)
     // rows of more than LONG_A_ROW entries, which the block's threads take together at the end: left to
     // its lane group such a row is a serial chain that sets the kernel's time on power-law inputs
     __shared__ int s_long[LONG_LIST], s_nlong;
@@ -260,7 +263,10 @@ __global__ void __launch_bounds__(256, SUMMARY ? 5 : 4) row_bounds_kernel(Csr A,
     // rows and products of the class of this group's last rows: neighbouring rows mostly share a
     // class, so the shared-memory histogram is touched only when the class changes
     int run_cls = -1, run_rows = 0;
-    unsigned my_bm_words = 0;                       // (2^31 rows over the groups of a full grid stay below 2^32 words a group)
+    // (at most 2^14 + 2^9 words a row: 2^32 words are 2.5e5 rows of the widest bitmap in a group.  Groups of 8 lanes and fewer, 18944 of them
+    // at least, do not see as many of 2^31 rows; those of 32, 4736, take rows of more than 32 entries on average when they are so
+    // many, 3.8e10 entries in all, more than memory holds)
+    unsigned my_bm_words = 0;
     i64 run_products = 0;
     auto classify = [&](int row, i64 entries, i64 u, int lo, int hi) {
         if (lo < 0 || hi >= B.ncols) { raise_status(ctl, DEV_NONCANONICAL); u = 0; }

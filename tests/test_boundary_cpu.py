@@ -116,3 +116,12 @@ def test_chained_kernels_load_nothing_read_only_before_their_wait():
                 for at in re.findall(r"\b%s(?:\[| \+ )\s*(\w+)" % pointer, body):
                     assert at not in known and not at.isdigit() or f"not_before({pointer})" in body, (kernel, pointer, at)
     assert seen >= 12
+
+
+def test_bounds_lists_hold_as_many_rows_however_many_blocks_are_resident():
+    """The blocks of the bounds kernel that are resident at once list at least as many long and mid rows together as 16 blocks an SM
+    with lists of 32 and 64."""
+    text = open(os.path.join(ROOT, "paper_2404_04541_b200", "csrc", "setup.cu")).read()
+    blocks = [int(x) for x in re.search(r"__launch_bounds__\(256, SUMMARY \? (\d+) : (\d+)\) row_bounds_kernel", text).groups()]
+    for name, least in (("LONG_LIST", 16 * 32), ("MID_LIST", 16 * 64)):
+        assert min(blocks) * int(re.search(r"constexpr int %s = (\d+);" % name, text).group(1)) >= least
