@@ -623,7 +623,7 @@ public:
         const bool sparse = p->sparse_products >= FORK_PRODUCTS;
         sparse_ = sparse ? 0 : warp ? 1 : 2;
         if ((int)sparse + (int)warp + (int)rest >= 2 && !p->profiling) h_ = p->h->fork_on();
-    on_ = h_ && cudaEventRecord(h_->forked, main_) == cudaSuccess;
+        on_ = h_ && cudaEventRecord(h_->forked, main_) == cudaSuccess;
         if (on_) c_.chain = 0;
     }
     ~Fork() { join(); }
