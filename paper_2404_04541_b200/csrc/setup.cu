@@ -761,7 +761,7 @@ cudaError_t launch_bin_rows(const LaunchCtx& c, int m) {
 // Replaces a three-launch scan, the routing and the per-class count (five launches; seven for the
 // 3-tensor form).
 // Bound by the chain of its steps (2048 rows: 6 us where the five launches took 13 and their gaps; 2e6 fibres: 27 us with five
-// blocks an SM, 21 with seven, which hold all 963 tiles at once).
+// blocks an SM, 21 with seven, which hold all 963 tiles at once, for 24 bytes spilled).
 // ---------------------------------------------------------------------------------------
 constexpr int FR_THREADS = 256;
 constexpr int FR_WARPS = FR_THREADS / 32;
